@@ -38,7 +38,7 @@
  *     multiple of the chunk is completed, inside the library, with tokens that leave the recurrence
  *     untouched (beta = 0, alpha = 1); tensors are never read or written beyond their T rows.
  *     bf16 with dk = dv = 128 runs on the tensor cores (tcgen05); fp32, and bf16 with another head
- *     dimension, run on plain fp32 FMA kernels (qdelta_chunk_path tells which).
+ *     dimension, run on fp32-accurate kernels (qdelta_chunk_path tells which).
  */
 #ifndef QDELTA_H_
 #define QDELTA_H_
@@ -93,7 +93,7 @@ typedef struct {
 typedef struct CUstream_st *qd_stream;   /* a cudaStream_t */
 
 /* Which kernels serve `shape` (the paper has no counterpart; a query for tests and benchmarks):
- * 1 = tensor-core kernels, 0 = fp32 FMA kernels, -1 = invalid or unsupported shape. */
+ * 1 = tensor-core kernels, 0 = fp32-accurate kernels, -1 = invalid or unsupported shape. */
 int qdelta_chunk_path(const qd_shape *shape);
 
 /* Bytes of device workspace the chunkwise calls need for this shape (0 on invalid shape).

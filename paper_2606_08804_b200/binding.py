@@ -136,7 +136,7 @@ def chunk_workspace_bytes(shape: QdShape, for_backward: bool) -> int:
 
 
 def chunk_path(shape: QdShape) -> str:
-    """Which kernels serve this shape: "tensor_core" (tcgen05) or "fp32" (plain FMA)."""
+    """Which kernels serve this shape: "tensor_core" (tcgen05) or "fp32" (fp32-accurate products)."""
     r = load().qdelta_chunk_path(ctypes.byref(shape))
     if r < 0:
         raise QdeltaError("unsupported or invalid shape for the chunkwise kernels")

@@ -9,7 +9,7 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 WsLayout ws_layout(const qd_shape& s) {
     WsLayout L{};
-    const size_t BH = (size_t)s.B * s.H, T = (size_t)simt_padded_T(s), N = T / kChunk;
+    const size_t BH = (size_t)s.B * s.H, T = (size_t)split_padded_T(s), N = T / kChunk;
     const size_t io = s.dtype == QD_BF16 ? 2 : 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
@@ -20,15 +20,14 @@ WsLayout ws_layout(const qd_shape& s) {
     L.U = take(BH * T * s.dv * io);
     L.rqk = take(2 * BH * T * 4);
     L.fwd_end = off;
-    L.nslices = s.dv / kSliceSimt;
-    L.bwd_ctas = 296;
+    L.slice = split_slice(s);
+    L.M = take(BH * N * kChunk * kChunk * 4);
     L.hs = take(BH * N * s.dk * s.dv * 4);
     L.D = take(BH * T * s.dv * io);
     L.dhs = take(BH * N * s.dk * s.dv * 4);
     L.dD = take(BH * T * s.dv * io);
-    L.kdhd = take((size_t)L.nslices * BH * T * 4);
-    L.dhh = take((size_t)L.nslices * BH * N * 4);
-    L.scratch = take((size_t)L.bwd_ctas * 6 * kChunk * s.dk * 4);
+    L.kdhd = take((size_t)(s.dv / L.slice) * BH * T * 4);
+    L.dhh = take((size_t)(s.dv / L.slice) * BH * N * 4);
     L.bwd_end = off;
     return L;
 }
@@ -135,8 +134,8 @@ int qdelta_chunk_fwd(const qd_shape* shape, const void* q, const void* k, const 
         if (timed(ST_CHAIN_FWD, a.stream, [&] { return tc_chain_fwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
         return QD_OK;
     }
-    if (timed(ST_PREP, a.stream, [&] { return simt_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
-    if (timed(ST_CHAIN_FWD, a.stream, [&] { return simt_chain_fwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
+    if (timed(ST_PREP, a.stream, [&] { return split_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
+    if (timed(ST_CHAIN_FWD, a.stream, [&] { return split_chain_fwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
     return QD_OK;
 }
 
@@ -192,11 +191,11 @@ int qdelta_chunk_bwd(const qd_shape* shape, const void* q, const void* k, const 
         if (cudaMemsetAsync(a.ws + a.L.status, 0, 256, a.stream) != cudaSuccess) return QD_ERR_CUDA;
         a.o = a.ws + a.L.dD;
         a.hT = nullptr;
-        if (timed(ST_PREP, a.stream, [&] { return simt_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
-        if (timed(ST_CHAIN_FWD, a.stream, [&] { return simt_chain_fwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
+        if (timed(ST_PREP, a.stream, [&] { return split_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
+        if (timed(ST_CHAIN_FWD, a.stream, [&] { return split_chain_fwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
     }
-    if (timed(ST_CHAIN_BWD, a.stream, [&] { return simt_chain_bwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
-    if (timed(ST_CHUNK_BWD, a.stream, [&] { return simt_chunk_bwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
+    if (timed(ST_CHAIN_BWD, a.stream, [&] { return split_chain_bwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
+    if (timed(ST_CHUNK_BWD, a.stream, [&] { return split_chunk_bwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
     return QD_OK;
 }
 

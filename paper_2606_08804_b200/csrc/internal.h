@@ -10,7 +10,6 @@
 namespace qd {
 
 constexpr int kChunk = 64;        // chunk length C of the chunkwise form
-constexpr int kSliceSimt = 32;    // d_v columns one CTA of the SIMT state chains owns
 
 // Byte offsets of the sections of the caller-provided workspace.  Every section starts on a
 // 256-byte boundary.  "io" sections are stored in the call's dtype.
@@ -28,14 +27,14 @@ struct WsLayout {
     size_t dD;       // io   [BH*T*dv]     gradient w.r.t. Delta
     size_t kdhd;     // fp32 [S][BH*T]     per d_v-slice partial of <(K-> dh)_r, Delta_r>
     size_t dhh;      // fp32 [S][BH*N]     per d_v-slice partial of <dh, h>_F
-    size_t scratch;  // fp32 per-CTA scratch of the SIMT chunk backward
+    size_t M;        // fp32 [BH*N][C][C]  (I+A)^-1 per chunk
     size_t rqk;      // fp32 [2][BH*T]     QD_NORM_QK: 1/|q_t|, then 1/|k_t|
     size_t bwd_end;
-    int nslices;
-    int bwd_ctas;
+    int slice;       // d_v columns one CTA of the state chains owns; S = dv / slice
 };
 
 WsLayout ws_layout(const qd_shape& s);
+int split_slice(const qd_shape& s);
 // QD_OK, or the error code every entry point reports for this shape (host-side validation only).
 int check_shape(const qd_shape* s);
 
@@ -62,7 +61,7 @@ bool tc_supported(const qd_shape& s);
 // Rows per sequence in the tensor-core workspace: T rounded up to a whole number of chunk PAIRS (the preparation kernel
 // takes two chunks at a time).  The rows past T behave as tokens with beta = 0, alpha = 1, q = k = v = 0, which leave the
 // recurrence of Section 3.3.1 untouched; TMA supplies the zeros and drops the stores.
-inline int simt_padded_T(const qd_shape& s) { return (s.T + kChunk - 1) / kChunk * kChunk; }   // fp32 path: whole chunks
+inline int split_padded_T(const qd_shape& s) { return (s.T + kChunk - 1) / kChunk * kChunk; }   // fp32 path: whole chunks
 inline int tc_padded_T(const qd_shape& s) { return (s.T + 2 * kChunk - 1) / (2 * kChunk) * (2 * kChunk); }
 
 // cudaFuncAttributeMaxDynamicSharedMemorySize for `kernel`: set when first needed on a device, and again only if a
@@ -103,11 +102,11 @@ struct ChunkArgs {
     cudaStream_t stream;
 };
 
-// SIMT fp32-arithmetic path (any supported dtype for storage)
-cudaError_t simt_prep(const ChunkArgs& a);        // g, P, W<-, U~
-cudaError_t simt_chain_fwd(const ChunkArgs& a);   // Delta, O, state chain (+ hs, D when a.save)
-cudaError_t simt_chain_bwd(const ChunkArgs& a);   // dDelta, dhs, dh0, scalar partials
-cudaError_t simt_chunk_bwd(const ChunkArgs& a);   // dq, dk, dv, dbeta, dalpha, dlambda
+// fp32-accurate path (any supported dtype for storage)
+cudaError_t split_prep(const ChunkArgs& a);        // g, P, W<-, U~ (+ M when a.save)
+cudaError_t split_chain_fwd(const ChunkArgs& a);   // Delta, O, state chain (+ hs, D when a.save)
+cudaError_t split_chain_bwd(const ChunkArgs& a);   // dDelta, dhs, dh0, scalar partials
+cudaError_t split_chunk_bwd(const ChunkArgs& a);   // dq, dk, dv, dbeta, dalpha, dlambda
 
 // tcgen05 path
 cudaError_t tc_prep(const ChunkArgs& a);
