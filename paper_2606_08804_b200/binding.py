@@ -1,7 +1,8 @@
-"""Thin ctypes binding of ``libqdelta.so`` (declared in ``include/qdelta.h``).
+"""Thin binding of ``libqdelta.so`` (declared in ``include/qdelta.h``).
 
 Argument marshalling only: torch supplies device memory and the current stream; every step of
-the computation runs in the library's CUDA kernels.  There is no fallback: if the library has
+the computation runs in the library's CUDA kernels.  The calls that a program makes per step (forward, backward, decode)
+marshal natively (``host/host.cpp``), the others through ctypes.  There is no fallback: if the library has
 not been built, or a call returns an error code, an exception is raised.
 """
 import ctypes
@@ -32,6 +33,22 @@ class QdeltaError(RuntimeError):
 
 
 _lib = None
+_native = None
+
+
+def _host():
+    """The native marshalling module, which links to libqdelta.so.  Raises if either has not been built."""
+    global _native
+    if _native is None:
+        load()
+        try:
+            from . import _qdelta_host
+        except ImportError as e:
+            raise QdeltaError("_qdelta_host.so is not built: run `python -m paper_2606_08804_b200.build` "
+                              "(or __graft_entry__.build()); there is no fallback path (%s)" % e) from e
+        _qdelta_host.set_error(QdeltaError)
+        _native = _qdelta_host
+    return _native
 
 
 def load():
@@ -159,26 +176,8 @@ def chunk_fwd(q, k, v, beta, alpha=None, lam=None, h0=None, chunk=64, save_for_b
     """Chunkwise forward.  Returns (o, hT, workspace).  All tensors live on the GPU.
     logits=True: beta, alpha, lam hold the logits of sigmoid gates (the kernels apply the sigmoid).
     norm_qk=True: q and k are un-normalised, the kernels L2-normalise them per token and head."""
-    lib = load()
-    s = make_shape(q, v, chunk)
-    B, T, H, dk, dv, dt = s.B, s.T, s.H, s.dk, s.dv, q.dtype
-    if workspace is None:
-        workspace = alloc_workspace(s, save_for_bwd, q.device)
-    if o is None:
-        o = torch.empty((B, T, H, dv), dtype=dt, device=q.device)
-    if hT is None and want_hT:
-        hT = torch.empty((B, H, dk, dv), dtype=torch.float32, device=q.device)
-    rc = lib.qdelta_chunk_fwd(
-        ctypes.byref(s), _ptr(q, dt, (B, T, H, dk), "q"), _ptr(k, dt, (B, T, H, dk), "k"),
-        _ptr(v, dt, (B, T, H, dv), "v"), _ptr(beta, dt, (B, T, H), "beta"),
-        _ptr(alpha, dt, (B, T, H), "alpha"), _ptr(lam, dt, (B, T, H), "lam"),
-        _ptr(h0, torch.float32, (B, H, dk, dv), "h0"), _ptr(o, dt, (B, T, H, dv), "o"),
-        _ptr(hT, torch.float32, (B, H, dk, dv), "hT"),
-        workspace.data_ptr(), workspace.numel(),
-        (QD_FWD_SAVE_FOR_BWD if save_for_bwd else 0) | (QD_COEF_LOGITS if logits else 0) | (QD_NORM_QK if norm_qk else 0),
-        _stream())
-    _check(rc, "qdelta_chunk_fwd")
-    return o, hT, workspace
+    flags = (QD_FWD_SAVE_FOR_BWD if save_for_bwd else 0) | (QD_COEF_LOGITS if logits else 0) | (QD_NORM_QK if norm_qk else 0)
+    return (_native or _host()).chunk_fwd(q, k, v, beta, alpha, lam, h0, int(chunk), workspace, o, hT, bool(want_hT), flags)
 
 
 def chunk_fwd_static(q, k, v, beta, alpha, lam, h0, o, hT=None, status=None, chunk=64):
@@ -212,75 +211,21 @@ def chunk_bwd(q, k, v, beta, alpha, lam, h0, dO, dhT=None, chunk=64, workspace=N
     """Chunkwise backward.  Returns dict(dq, dk, dv, dbeta, dalpha, dlam, dh0) of GPU tensors.
     logits=True: beta, alpha, lam are logits and dbeta, dalpha, dlam are gradients with respect to them.
     norm_qk=True: q, k are un-normalised and dq, dk are gradients with respect to them."""
-    lib = load()
-    s = make_shape(q, v, chunk)
-    B, T, H, dk, dv, dt = s.B, s.T, s.H, s.dk, s.dv, q.dtype
-    dev = q.device
-    if workspace is None:
-        if reuse_fwd:
-            raise QdeltaError("reuse_fwd needs the workspace of the forward call")
-        workspace = alloc_workspace(s, True, dev)
-    g = out if out is not None else {}
-    f32 = torch.float32
-    g.setdefault("dq", torch.empty((B, T, H, dk), dtype=dt, device=dev))
-    g.setdefault("dk", torch.empty((B, T, H, dk), dtype=dt, device=dev))
-    g.setdefault("dv", torch.empty((B, T, H, dv), dtype=dt, device=dev))
-    g.setdefault("dbeta", torch.empty((B, T, H), dtype=f32, device=dev))
-    g.setdefault("dalpha", torch.empty((B, T, H), dtype=f32, device=dev) if alpha is not None else None)
-    g.setdefault("dlam", torch.empty((B, T, H), dtype=f32, device=dev) if lam is not None else None)
-    g.setdefault("dh0", torch.empty((B, H, dk, dv), dtype=f32, device=dev) if want_dh0 else None)
-    rc = lib.qdelta_chunk_bwd(
-        ctypes.byref(s), _ptr(q, dt, (B, T, H, dk), "q"), _ptr(k, dt, (B, T, H, dk), "k"),
-        _ptr(v, dt, (B, T, H, dv), "v"), _ptr(beta, dt, (B, T, H), "beta"),
-        _ptr(alpha, dt, (B, T, H), "alpha"), _ptr(lam, dt, (B, T, H), "lam"),
-        _ptr(h0, f32, (B, H, dk, dv), "h0"), _ptr(dO, dt, (B, T, H, dv), "dO"),
-        _ptr(dhT, f32, (B, H, dk, dv), "dhT"),
-        _ptr(g["dq"], dt, (B, T, H, dk), "dq"), _ptr(g["dk"], dt, (B, T, H, dk), "dk"),
-        _ptr(g["dv"], dt, (B, T, H, dv), "dv"), _ptr(g["dbeta"], f32, (B, T, H), "dbeta"),
-        _ptr(g["dalpha"], f32, (B, T, H), "dalpha"), _ptr(g["dlam"], f32, (B, T, H), "dlam"),
-        _ptr(g["dh0"], f32, (B, H, dk, dv), "dh0"),
-        workspace.data_ptr(), workspace.numel(),
-        (QD_BWD_REUSE_FWD if reuse_fwd else 0) | (QD_COEF_LOGITS if logits else 0) | (QD_NORM_QK if norm_qk else 0),
-        _stream())
-    _check(rc, "qdelta_chunk_bwd")
-    return g
+    if workspace is None and reuse_fwd:
+        raise QdeltaError("reuse_fwd needs the workspace of the forward call")
+    flags = (QD_BWD_REUSE_FWD if reuse_fwd else 0) | (QD_COEF_LOGITS if logits else 0) | (QD_NORM_QK if norm_qk else 0)
+    return (_native or _host()).chunk_bwd(q, k, v, beta, alpha, lam, h0, int(chunk), dO, dhT, workspace,
+                                          out if out is not None else {}, bool(want_dh0), flags)
 
 
 def recurrent_step(q, k, v, beta, alpha, lam, state, o=None):
     """One decode step; `state` [B,H,dk,dv] fp32 is updated in place.  Returns o [B,H,dv]."""
-    lib = load()
-    B, H, dk = q.shape
-    dv = v.shape[-1]
-    dt = q.dtype
-    if o is None:
-        o = torch.empty((B, H, dv), dtype=dt, device=q.device)
-    rc = lib.qdelta_recurrent_step(
-        B, H, dk, dv, _dtype_code(q), _ptr(q, dt, (B, H, dk), "q"), _ptr(k, dt, (B, H, dk), "k"),
-        _ptr(v, dt, (B, H, dv), "v"), _ptr(beta, dt, (B, H), "beta"), _ptr(alpha, dt, (B, H), "alpha"),
-        _ptr(lam, dt, (B, H), "lam"), _ptr(state, torch.float32, (B, H, dk, dv), "state"),
-        _ptr(o, dt, (B, H, dv), "o"), _stream())
-    _check(rc, "qdelta_recurrent_step")
-    return o
+    return (_native or _host()).recurrent_step(q, k, v, beta, alpha, lam, state, o)
 
 
 def recurrent_steps(q, k, v, beta, alpha, lam, state, o=None, logits=False, norm_qk=False):
     """S decode tokens per call: q,k [B,S,H,dk], v [B,S,H,dv], coefficients [B,S,H]; `state` [B,H,dk,dv] fp32 is
     updated in place to the state after the last token.  Returns o [B,S,H,dv].  A bf16 `state` selects the
     reduced-precision state option (QD_STATE_BF16)."""
-    lib = load()
-    B, S, H, dk = q.shape
-    dv = v.shape[-1]
-    dt = q.dtype
-    if state.dtype not in (torch.float32, torch.bfloat16):
-        raise QdeltaError("state must be fp32, or bf16 for the reduced-precision state option")
-    state_bf16 = state.dtype == torch.bfloat16
-    if o is None:
-        o = torch.empty((B, S, H, dv), dtype=dt, device=q.device)
-    rc = lib.qdelta_recurrent_steps(
-        B, S, H, dk, dv, _dtype_code(q), _ptr(q, dt, (B, S, H, dk), "q"), _ptr(k, dt, (B, S, H, dk), "k"),
-        _ptr(v, dt, (B, S, H, dv), "v"), _ptr(beta, dt, (B, S, H), "beta"), _ptr(alpha, dt, (B, S, H), "alpha"),
-        _ptr(lam, dt, (B, S, H), "lam"), _ptr(state, None, (B, H, dk, dv), "state"),
-        _ptr(o, dt, (B, S, H, dv), "o"),
-        (QD_COEF_LOGITS if logits else 0) | (QD_NORM_QK if norm_qk else 0) | (QD_STATE_BF16 if state_bf16 else 0), _stream())
-    _check(rc, "qdelta_recurrent_steps")
-    return o
+    flags = (QD_COEF_LOGITS if logits else 0) | (QD_NORM_QK if norm_qk else 0)
+    return (_native or _host()).recurrent_steps(q, k, v, beta, alpha, lam, state, o, flags)

@@ -1,7 +1,8 @@
-"""Build ``libqdelta.so`` (sm_100a only) in-tree with nvcc.
+"""Build ``libqdelta.so`` (sm_100a only) with nvcc and ``_qdelta_host.so`` with g++, in-tree.
 
 Every ``csrc/*.cu`` is compiled to an object under ``build/`` (in parallel, only when its
-source or a header is newer) and linked into ``paper_2606_08804_b200/libqdelta.so``.
+source or a header is newer) and linked into ``paper_2606_08804_b200/libqdelta.so``.  ``host/host.cpp``
+becomes the extension module ``paper_2606_08804_b200/_qdelta_host.so``, which calls into that library.
 """
 import concurrent.futures as cf
 import glob
@@ -14,6 +15,8 @@ _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 OBJ_DIR = os.path.join(_ROOT, "build", "obj")
 LIB = os.path.join(_HERE, "libqdelta.so")
+HOST_SRC = os.path.join(_HERE, "host", "host.cpp")
+HOST_LIB = os.path.join(_HERE, "_qdelta_host.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -39,6 +42,29 @@ def _compile(src, obj, log):
     return obj
 
 
+def _build_host(force):
+    """The native side of binding.py, against the headers of the installed torch."""
+    header = os.path.join(_ROOT, "include", "qdelta.h")
+    if not force and os.path.exists(HOST_LIB) and \
+            os.path.getmtime(HOST_LIB) >= max(os.path.getmtime(f) for f in (HOST_SRC, header, os.path.abspath(__file__))):
+        return
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    tmp = HOST_LIB + ".tmp.%d" % os.getpid()
+    inc = cpp_extension.include_paths() + [sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
+    libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-w", HOST_SRC, "-o", tmp,
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI] + ["-I" + d for d in inc] + \
+          ["-L" + _HERE, "-lqdelta", "-L" + libdir, "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda",
+           "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed for %s:\n%s" % (HOST_SRC, r.stdout + r.stderr))
+    os.replace(tmp, HOST_LIB)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ_DIR, exist_ok=True)
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
@@ -62,6 +88,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if r.returncode != 0:
             raise RuntimeError("link failed:\n" + r.stdout + r.stderr)
         os.replace(tmp, LIB)
+    _build_host(force)
     if verbose:
         for s, o, log in jobs:
             print(open(log).read())

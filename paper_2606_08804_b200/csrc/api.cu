@@ -127,7 +127,6 @@ int qdelta_chunk_fwd(const qd_shape* shape, const void* q, const void* k, const 
     a.q = q; a.k = k; a.v = v; a.beta = beta; a.alpha = alpha; a.lam = lambda; a.h0 = h0; a.o = o; a.hT = hT;
     a.ws = (char*)workspace;
     a.stream = (cudaStream_t)stream;
-    if (cudaMemsetAsync(a.ws + a.L.status, 0, 256, a.stream) != cudaSuccess) return QD_ERR_CUDA;   // offset 0 in both layouts
     if (tc_supported(*shape)) {
         a.TL = tc_layout(*shape);
         if (timed(ST_PREP, a.stream, [&] { return tc_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
@@ -174,7 +173,6 @@ int qdelta_chunk_bwd(const qd_shape* shape, const void* q, const void* k, const 
         if (!(flags & QD_BWD_REUSE_FWD)) {
             // recompute what a saving forward leaves behind; its o goes to the dDelta section, which
             // the reverse chain overwrites afterwards
-            if (cudaMemsetAsync(a.ws + a.TL.status, 0, 256, a.stream) != cudaSuccess) return QD_ERR_CUDA;
             a.o = a.ws + a.TL.dDt;
             a.hT = nullptr;
             if (timed(ST_PREP, a.stream, [&] { return tc_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
@@ -188,7 +186,6 @@ int qdelta_chunk_bwd(const qd_shape* shape, const void* q, const void* k, const 
     if (!(flags & QD_BWD_REUSE_FWD)) {
         // recompute the forward intermediates (outputs of the forward itself are not rewritten:
         // o goes to the dD section, which the reverse chain overwrites afterwards)
-        if (cudaMemsetAsync(a.ws + a.L.status, 0, 256, a.stream) != cudaSuccess) return QD_ERR_CUDA;
         a.o = a.ws + a.L.dD;
         a.hT = nullptr;
         if (timed(ST_PREP, a.stream, [&] { return split_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;

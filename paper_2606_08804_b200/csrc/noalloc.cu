@@ -12,7 +12,7 @@
 //    different streams, or from different threads) race on it -- callers serialise them, e.g. by
 //    issuing them on one stream;
 //  * nothing in it needs a particular value between calls except the status word (first 256 bytes),
-//    which must start at zero: each call clears it on the caller's stream before its first kernel;
+//    which must start at zero: the first kernel of each call clears it;
 //  * the first call on a device performs the set-up below (it looks up the array's address; the
 //    driver may load this module at that moment), so the first call on each device should be made
 //    before any stream capture begins;

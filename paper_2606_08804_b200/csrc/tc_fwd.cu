@@ -90,6 +90,8 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
     const size_t wtok0 = (size_t)bh * p.Tp + (size_t)t0;             // first row in the workspace's [BH*Tp] view
 
     if (tid == 0) {
+        // the call's status word starts at zero: the first CTA to start clears it, a second before any wait can expire
+        if (blockIdx.x == 0) *p.status = 0;
         mbar_init(&bar_load, 1);
         mbar_init(&bar_mma, 1);
         mbar_init_fence();
