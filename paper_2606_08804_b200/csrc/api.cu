@@ -211,7 +211,7 @@ int qdelta_recurrent_step(int B, int H, int dk, int dv, int dtype, const void* q
     for (const void* p : coef)
         if (p && ((uintptr_t)p & (dtype == QD_BF16 ? 1 : 3))) return QD_ERR_INVALID_ARG;
     if (timed(ST_DECODE, (cudaStream_t)stream, [&] {
-            return decode_step(B * H, dk, dv, dtype, q, k, v, beta, alpha, lambda, state, o, (cudaStream_t)stream);
+            return decode_steps(B, 1, H, dk, dv, dtype, q, k, v, beta, alpha, lambda, state, o, false, false, false, (cudaStream_t)stream);
         }) != cudaSuccess)
         return QD_ERR_CUDA;
     return QD_OK;

@@ -114,10 +114,7 @@ cudaError_t tc_chain_fwd(const ChunkArgs& a);
 cudaError_t tc_chain_bwd(const ChunkArgs& a);
 cudaError_t tc_chunk_bwd(const ChunkArgs& a);
 
-cudaError_t decode_step(int BH, int dk, int dv, int dtype, const void* q, const void* k, const void* v,
-                        const void* beta, const void* alpha, const void* lam, float* state, void* o,
-                        cudaStream_t stream);
-
+// S consecutive tokens of every sequence; qdelta_recurrent_step is S = 1
 cudaError_t decode_steps(int B, int S, int H, int dk, int dv, int dtype, const void* q, const void* k, const void* v,
                          const void* beta, const void* alpha, const void* lam, void* state, void* o,
                          bool logits, bool norm, bool state_bf16, cudaStream_t stream);
