@@ -90,8 +90,6 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
     const size_t wtok0 = (size_t)bh * p.Tp + (size_t)t0;             // first row in the workspace's [BH*Tp] view
 
     if (tid == 0) {
-        // the call's status word starts at zero: the first CTA to start clears it, a second before any wait can expire
-        if (blockIdx.x == 0) *p.status = 0;
         mbar_init(&bar_load, 1);
         mbar_init(&bar_mma, 1);
         mbar_init_fence();
@@ -102,8 +100,11 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
     tc_fence_after();
     const uint32_t tbase = tmem_slot;
 
+    grid_dep_wait();                  // set up while the kernel before drains; nothing is read or written before it has completed
     grid_dep_launch();                // the kernel after this one may set itself up while the last CTAs of this one run
     if (tid == 0) {
+        // the call's status word starts at zero: the first CTA to start clears it, a second before any wait can expire
+        if (blockIdx.x == 0) *p.status = 0;
         mbar_expect_tx(&bar_load, 3 * 32768);
         for (int blk = 0; blk < 2; ++blk) {          // rows at t >= T arrive as zeros
             tma_load_3d(sQ + blk * 16384, &mapQ, hh * D + blk * 64, t0, b, &bar_load);
@@ -730,8 +731,7 @@ cudaError_t tc_prep(const ChunkArgs& a) {
     cudaError_t e = set_smem(kern, kPrepSmem);
     if (e != cudaSuccess) return e;
     const int grid = s.B * s.H * (p.N / 2);
-    kern<<<grid, kPrepThreads, kPrepSmem, a.stream>>>(mQ, mK, mV, mUt, mWt, p);
-    return cudaGetLastError();
+    return launch_overlapped(kern, dim3((unsigned)grid), dim3(kPrepThreads), kPrepSmem, a.stream, mQ, mK, mV, mUt, mWt, p);
 }
 
 cudaError_t tc_chain_fwd(const ChunkArgs& a) {
