@@ -21,6 +21,7 @@
 // operand once.
 #include "internal.h"
 #include "sm100.cuh"
+#include "tf32.cuh"
 
 namespace qd {
 namespace {
@@ -50,15 +51,6 @@ template <typename IO> constexpr int kTerms = 2;                 // tf32 halves 
 template <> constexpr int kTerms<__nv_bfloat16> = 1;
 
 // ---- products -----------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void split(float x, uint32_t& hi, uint32_t& lo) {
-    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;           // 11 significant bits, rounded
-    lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;     // the instruction ignores the low 13 bits
-}
-__device__ __forceinline__ void mma_tf32(float* c, const uint32_t* a, const uint32_t* b) {
-    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
 // acc += A B for the (16 MT) x (8 NTL) tile of this warp at row m0, column n0: contraction extent K, a(m, k) and b(k, n)
 // fetch the operands, TA / TB say how many tf32 halves they need.  Lane (g = lane / 4, t = lane % 4) holds, of every
 // 16 x 8 piece, rows g and g + 8, columns 2t and 2t + 1.
@@ -83,7 +75,7 @@ __device__ __forceinline__ void wmm(float (&acc)[MT][NTL][4], int m0, int n0, in
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float x = a(m0 + 16 * i + g + 8 * (e & 1), k0 + 8 * s + t + 4 * (e >> 1));
-                    if (TA == 2) split(x, ah[s][i][e], al[s][i][e]);
+                    if (TA == 2) tf32_split(x, ah[s][i][e], al[s][i][e]);
                     else ah[s][i][e] = __float_as_uint(x);
                 }
 #pragma unroll
@@ -106,7 +98,7 @@ __device__ __forceinline__ void wmm(float (&acc)[MT][NTL][4], int m0, int n0, in
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const float x = b(k0 + 8 * s + t + 4 * e, n0 + 8 * (jb + j) + g);
-                        if (TB == 2) split(x, bh[j][e], bl[j][e]);
+                        if (TB == 2) tf32_split(x, bh[j][e], bl[j][e]);
                         else bh[j][e] = __float_as_uint(x);
                     }
 #pragma unroll

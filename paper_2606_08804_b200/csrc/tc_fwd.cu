@@ -15,6 +15,7 @@
 // releases its tensor memory and returns.
 #include "internal.h"
 #include "sm100.cuh"
+#include "tf32.cuh"
 
 namespace qd {
 namespace {
@@ -42,44 +43,144 @@ struct PrepParams {
     int T, Tp, H, N, BH;       // T tokens per sequence; the workspace holds Tp = 64 N >= T rows per sequence (N even)
     const bf16 *beta, *alpha, *lam;
     float* g;
-    bf16 *Qg, *P;
+    bf16* Qg;
     bf16* Mt;                  // optional: ((I+A)^-1)^T per chunk, [column i][row r]; kept for the backward
     unsigned* status;
 };
 
-// 96 KB: Q (later X, in place) | K (later A in fp32, then the T tiles) | V; at the end the first and the
+// 96 KB: Q (later X, in place) | K (later A in fp32, then the T tiles, then P) | V; at the end the first and the
 // last 32 KB stage U~^T and W~^T for their TMA stores.  Two CTAs fit on one SM.
 constexpr int kPrepSmem = 3 * 32768 + 1024;
 constexpr int kPrepThreads = 256;
+
+// The 64 x 64 matrices of the inverse are kept transposed, [column i][row r], so that a column is contiguous; groups of
+// four rows are permuted by column so that the fragment loads of a 16 x 8 or 8 x 8 piece, the epilogue's stores (rows
+// across the lanes) and 16-byte accesses along a column all spread over the banks.
+__device__ __forceinline__ int at_off(int i, int r) { return i * C + (r ^ (((i & 3) << 3) | (i & 4))); }
+
+// acc (16 x 16) += X Y over k = 0..15: X(m, k) = a[at_off(am + m, ak + k)], Y(k, n) = b[at_off(bk + k, bn + n)] with am, ak, bk, bn
+// multiples of 8, fp32-accurate (three tf32 products).
+__device__ __forceinline__ void mm16(float (&acc)[2][4], const float* a, int am, int ak, const float* b, int bk, int bn) {
+    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+    const float *a0 = a + (am + g) * C + t + (g & 4), *a1 = a + (am + g) * C + t + (4 - (g & 4));    // columns t, t + 4 of a step
+    const int am8 = (g & 3) << 3;
+    const float *b0 = b + (bk + t) * C + (bn ^ (t << 3)) + g, *b1 = b + (bk + t + 4) * C + (bn ^ (t << 3)) + (g ^ 4);
+    const int b8 = (t & 1) ? -8 : 8;                                                                   // column + 8 of Y
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const int ac = (ak + 8 * s) ^ am8;
+        uint32_t ah[4], al[4], bh[2][2], bl[2][2];
+        tf32_split(a0[ac], ah[0], al[0]); tf32_split(a0[ac + 8 * C], ah[1], al[1]);
+        tf32_split(a1[ac], ah[2], al[2]); tf32_split(a1[ac + 8 * C], ah[3], al[3]);
+        tf32_split(b0[8 * s * C], bh[0][0], bl[0][0]); tf32_split(b1[8 * s * C], bh[0][1], bl[0][1]);
+        tf32_split(b0[8 * s * C + b8], bh[1][0], bl[1][0]); tf32_split(b1[8 * s * C + b8], bh[1][1], bl[1][1]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) mma_tf32(acc[j], al, bh[j]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) mma_tf32(acc[j], ah, bl[j]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) mma_tf32(acc[j], ah, bh[j]);
+    }
+}
+__device__ __forceinline__ void put16(const float (&acc)[2][4], float sign, float* d, int dm, int dn) {
+    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            *reinterpret_cast<float2*>(d + at_off(dm + g + 8 * h, dn + 8 * j + 2 * t)) = make_float2(sign * acc[j][2 * h], sign * acc[j][2 * h + 1]);
+}
+// M_c = (I + A_c)^-1 of two chunks, in place, both transposed (at_off): A^T comes strictly upper triangular in this view,
+// M^T leaves with its zeros and ones.  Block-wise: the 16 x 16 diagonal blocks by right-looking substitution, a column in
+// the registers of a lane, two blocks per warp; then blocks joined twice, M21^T = -M11^T (A21^T M22^T), on the warp-level
+// tensor instruction, zero blocks left out.  A column walked over all 64 rows in registers takes 63 dependent steps whose
+// broadcast loads of A are bound by shared-memory wavefronts: 7300 cycles of a CTA's 28000, against 5500 of 25000 for this.
+__device__ __forceinline__ void invert_pair(float* sA) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp < 4) {
+        const int q = 2 * warp + (lane >> 4), j = lane & 15, o = (q & 3) * 16;
+        float* Ac = sA + (q >> 2) * C * C;
+        float m[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) m[r] = r == j ? 1.f : 0.f;
+#pragma unroll
+        for (int i = 0; i < 15; ++i) {
+#pragma unroll
+            for (int r4 = (i + 1) / 4; r4 < 4; ++r4) {
+                const float4 a = *reinterpret_cast<const float4*>(Ac + at_off(o + i, o + 4 * r4));     // zero at and above row i
+                m[4 * r4] = fmaf(-a.x, m[i], m[4 * r4]); m[4 * r4 + 1] = fmaf(-a.y, m[i], m[4 * r4 + 1]);
+                m[4 * r4 + 2] = fmaf(-a.z, m[i], m[4 * r4 + 2]); m[4 * r4 + 3] = fmaf(-a.w, m[i], m[4 * r4 + 3]);
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r4 = 0; r4 < 4; ++r4)
+            *reinterpret_cast<float4*>(Ac + at_off(o + j, o + 4 * r4)) = make_float4(m[4 * r4], m[4 * r4 + 1], m[4 * r4 + 2], m[4 * r4 + 3]);
+    }
+    __syncthreads();
+    if (warp < 4) {                                              // 16 -> 32: one warp per pair of blocks
+        float* Ac = sA + (warp >> 1) * C * C;
+        const int o = (warp & 1) * 32;
+        float s[2][4] = {}, m[2][4] = {};
+        mm16(s, Ac, o, o + 16, Ac, o + 16, o + 16);
+        __syncwarp();
+        put16(s, 1.f, Ac, o, o + 16);
+        __syncwarp();
+        mm16(m, Ac, o, o, Ac, o, o + 16);
+        __syncwarp();
+        put16(m, -1.f, Ac, o, o + 16);
+    }
+    __syncthreads();
+    {   // 32 -> 64: four warps per chunk, 16 x 16 each; warps w and w + 4 share a scheduler, so the second chunk's pieces
+        // are numbered from the other end: every scheduler gets a long contraction and a short one
+        float* Ac = sA + (warp >> 2) * C * C;
+        const int w = warp < 4 ? warp : 7 - warp, tm = (w & 2) * 8, tn = (w & 1) * 16;
+        float s[2][4] = {}, m[2][4] = {};
+        mm16(s, Ac, tm, 32, Ac, 32, 32 + tn);
+        if (tn) mm16(s, Ac, tm, 48, Ac, 48, 48);                 // M22^T is upper triangular: k <= n
+        __syncthreads();
+        put16(s, 1.f, Ac, tm, 32 + tn);
+        __syncthreads();
+        mm16(m, Ac, tm, 16, Ac, 16, 32 + tn);
+        if (!tm) mm16(m, Ac, 0, 0, Ac, 0, 32 + tn);              // M11^T likewise: k >= m
+        __syncthreads();
+        put16(m, -1.f, Ac, tm, 32 + tn);
+    }
+    __syncthreads();
+}
 
 // One CTA prepares a pair of chunks (128 tokens) of one head.  Thread roles change by phase:
 //   scan / coefficients   thread t < 128 owns token t
 //   row-wise elementwise  16 threads per 256-byte row (coalesced), 16 rows per pass
 //   Gram epilogue         thread (row = t & 127, half = t >> 7) owns 32 columns of its TMEM lane
-//   triangular inverse    lane quad (t >> 2, t < 128) owns columns j0 + 16 k (j0 < 16) of one chunk, quad lane t & 3 the 8-row blocks t & 3 and (t & 3) + 4
+//   triangular inverse    by warps, see invert_pair
 //   final epilogue        thread (d = t & 127, which = t >> 7) owns one row of U~^T resp. W~^T
-// NORM (QD_NORM_QK): L2-normalise the rows of Q and K first.  LOGITS (QD_COEF_LOGITS): the coefficients are logits of
-// sigmoid gates.  Compile-time, because even the untaken sigmoid / log-sigmoid code on the path of the scan, which
-// every later phase of the CTA waits for, cost the kernel 8 %.
+// Both Gram products start as soon as Q and K are there: X K^T = K K^T + diag(lambda) Q K^T is combined in the epilogue, so
+// nothing waits for X, which is formed in registers under the products and takes Q's place when they have read it.
+// NORM (QD_NORM_QK): q and k come un-normalised; 1/|q_t|, 1/|k_t| are factors wherever a row is used.  LOGITS
+// (QD_COEF_LOGITS): the coefficients are logits of sigmoid gates.  Compile-time, because even the untaken sigmoid /
+// log-sigmoid code on the path of the scan, which every later phase of the CTA waits for, cost the kernel 8 %.
 template <bool NORM, bool LOGITS>
 __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_constant__ CUtensorMap mapQ,
                                                              const __grid_constant__ CUtensorMap mapK,
                                                              const __grid_constant__ CUtensorMap mapV,
                                                              const __grid_constant__ CUtensorMap mapUt,
-                                                             const __grid_constant__ CUtensorMap mapWt, PrepParams p) {
+                                                             const __grid_constant__ CUtensorMap mapWt,
+                                                             const __grid_constant__ CUtensorMap mapP, PrepParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *sQ = smem, *sK = smem + 32768, *sV = smem + 65536;
-    // lambda absent (the gated delta rule, Eq. 3): X = K, so nothing is built, both Gram products start at once, and
-    // the scratch that otherwise overwrites K overwrites Q instead
-    const bool has_lam = p.lam != nullptr;
-    unsigned char* sX = has_lam ? sQ : sK;                      // X overwrites Q once Q K^T has been formed
-    unsigned char* sScr = has_lam ? sK : sQ;                    // dead once both Grams are read (and diag(gamma)Q is written)
-    float* sA = reinterpret_cast<float*>(sScr);                 // A^T [2][column i][row r]
+    // lambda absent (the gated delta rule, Eq. 3) and keys given normalised: X = K, nothing is built, and the scratch that
+    // otherwise overwrites K overwrites Q instead
+    const bool build_x = NORM || p.lam != nullptr;
+    unsigned char* sX = build_x ? sQ : sK;
+    unsigned char* sScr = build_x ? sK : sQ;                    // dead once both Grams are formed, diag(gamma)Q and X taken
+    float* sA = reinterpret_cast<float*>(sScr);                 // A^T, then M^T: [2][column][row], at_off
     unsigned char* sT = sScr;                                   // [2] T_c, [2] T_c diag(gamma): 8 KB each, alias A
-    __shared__ uint64_t bar_load, bar_mma;
+    __shared__ uint64_t bar_load, bar_v, bar_mma;
     __shared__ uint32_t tmem_slot;
-    __shared__ float sg[128], sbeta[128], slam[128], swsum[4];
+    __shared__ __align__(16) float sg[128], srk[128];
+    __shared__ float sbeta[128], slam[128], srq[128], swsum[4];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // CTAs are numbered pair-major, last pair first: the forward chain, which starts with chunk 0 of every sequence,
@@ -91,6 +192,7 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
 
     if (tid == 0) {
         mbar_init(&bar_load, 1);
+        mbar_init(&bar_v, 1);
         mbar_init(&bar_mma, 1);
         mbar_init_fence();
     }
@@ -105,12 +207,13 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
     if (tid == 0) {
         // the call's status word starts at zero: the first CTA to start clears it, a second before any wait can expire
         if (blockIdx.x == 0) *p.status = 0;
-        mbar_expect_tx(&bar_load, 3 * 32768);
+        mbar_expect_tx(&bar_load, 2 * 32768);
         for (int blk = 0; blk < 2; ++blk) {          // rows at t >= T arrive as zeros
             tma_load_3d(sQ + blk * 16384, &mapQ, hh * D + blk * 64, t0, b, &bar_load);
             tma_load_3d(sK + blk * 16384, &mapK, hh * D + blk * 64, t0, b, &bar_load);
-            tma_load_3d(sV + blk * 16384, &mapV, hh * D + blk * 64, t0, b, &bar_load);
         }
+        mbar_expect_tx(&bar_v, 32768);               // needed last
+        for (int blk = 0; blk < 2; ++blk) tma_load_3d(sV + blk * 16384, &mapV, hh * D + blk * 64, t0, b, &bar_v);
     }
     // coefficients of token tid; in-chunk cumulative log-decay by a two-warp scan per chunk
     if (tid < 128) {
@@ -132,196 +235,133 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
         p.g[wtok0 + tid] = g;
     }
 
-    bool fail = !mbar_wait(&bar_load, 0);
-    if (__syncthreads_or(fail)) {
+    // all threads leave together when a wait has expired; copies in flight get one more bounded chance to land
+    auto expired = [&](bool fail) {
+        if (!__syncthreads_or(fail)) return false;
         if (tid == 0) *p.status = QD_ERR_TIMEOUT;
-        mbar_wait(&bar_load, 0);           // loads may still be in flight: one more bounded chance
+        mbar_wait(&bar_load, 0);
+        mbar_wait(&bar_v, 0);
         __syncthreads();
         if (warp == 0) tmem_dealloc(tbase, 256);
-        return;
+        return true;
+    };
+    if (expired(!mbar_wait(&bar_load, 0))) return;
+    if (tid == 0) {
+        tc_fence_after();
+        // G1 = K K^T -> columns [0,128), G2 = Q K^T -> columns [128,256)
+        umma_product<false, false>(tbase + 128, smem_u32(sQ), 16384, smem_u32(sK), 16384, 128, 128, false);
+        umma_product<false, false>(tbase, smem_u32(sK), 16384, smem_u32(sK), 16384, 128, 128, false);
+        umma_commit(&bar_mma);
     }
-    // row-wise work: 16 lanes cover one 256-byte row (chunk `ch` of 16 bytes each), 16 rows per pass
+    // meanwhile, row-wise, 16 lanes to a 256-byte row (chunk `ch` of 16 bytes each): Qg = gamma Q to the workspace, and X
+    uint4 xr[8];
     const int ch = tid & 15, rsub = tid >> 4;
     const uint32_t coff = (ch >> 3) * 16384;
-    if (NORM) {
-        // q^ = q / sqrt(|q|^2 + eps), k^ likewise, in place: everything below (and every later kernel, through
-        // diag(gamma) Q^ and the 1/|k| written here) works on the normalised rows
+    {
+        bf16* qg = p.Qg + wtok0 * D + ch * 8;
         const size_t nrows = (size_t)p.BH * p.Tp;
-#pragma unroll 2
+#pragma unroll
         for (int it = 0; it < 8; ++it) {
             const int row = it * 16 + rsub;
             const uint32_t off = coff + sw128_chunk(row, ch & 7);
-            float qv[8], kv[8], sq = 0.f, sk = 0.f;
+            float qv[8], kv[8], rq = 1.f, rk = 1.f;
             load8(sQ + off, qv);
-            load8(sK + off, kv);
+            if (build_x) load8(sK + off, kv);
+            if (NORM) {
+                // 1 / sqrt(|q|^2 + eps), 1 / sqrt(|k|^2 + eps)
+                float sq = 0.f, sk = 0.f;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) { sq = fmaf(qv[e], qv[e], sq); sk = fmaf(kv[e], kv[e], sk); }
+                for (int e = 0; e < 8; ++e) { sq = fmaf(qv[e], qv[e], sq); sk = fmaf(kv[e], kv[e], sk); }
 #pragma unroll
-            for (int o = 1; o < 16; o <<= 1) {
-                sq += __shfl_xor_sync(0xffffffffu, sq, o);
-                sk += __shfl_xor_sync(0xffffffffu, sk, o);
+                for (int o = 1; o < 16; o <<= 1) {
+                    sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                    sk += __shfl_xor_sync(0xffffffffu, sk, o);
+                }
+                rq = rsqrtf(sq + kNormEps);
+                rk = rsqrtf(sk + kNormEps);
+                if (ch == 0) {
+                    srq[row] = rq; srk[row] = rk;
+                    p.rqk[wtok0 + row] = rq; p.rqk[nrows + wtok0 + row] = rk;
+                }
             }
-            const float rq = rsqrtf(sq + kNormEps), rk = rsqrtf(sk + kNormEps);
+            const float gr = __expf(sg[row]) * rq, lm = slam[row] * rq;
+            if (build_x) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) { qv[e] *= rq; kv[e] *= rk; }
-            sts128(sQ + off, pack8(qv));
-            sts128(sK + off, pack8(kv));
-            if (ch == 0) { p.rqk[wtok0 + row] = rq; p.rqk[nrows + wtok0 + row] = rk; }
-        }
-        fence_proxy_async();
-        __syncthreads();
-    }
-    if (tid == 0) {
-        tc_fence_after();
-        // G2 = Q K^T -> columns [128,256);  without lambda also G1 = K K^T -> columns [0,128)
-        umma_product<false, false>(tbase + 128, smem_u32(sQ), 16384, smem_u32(sK), 16384, 128, 128, false);
-        if (!has_lam) umma_product<false, false>(tbase, smem_u32(sK), 16384, smem_u32(sK), 16384, 128, 128, false);
-        umma_commit(&bar_mma);
-    }
-    // meanwhile: Qg = gamma Q to the workspace, a warp writes two full rows per store
-    {
-        bf16* qg = p.Qg + wtok0 * D + ch * 8;
-#pragma unroll 4
-        for (int it = 0; it < 8; ++it) {
-            const int row = it * 16 + rsub;
-            const float gr = __expf(sg[row]);
-            float qv[8];
-            load8(sQ + coff + sw128_chunk(row, ch & 7), qv);
+                for (int e = 0; e < 8; ++e) kv[e] = fmaf(lm, qv[e], NORM ? rk * kv[e] : kv[e]);
+                xr[it] = pack8(kv);
+            }
 #pragma unroll
             for (int e = 0; e < 8; ++e) qv[e] *= gr;
             *reinterpret_cast<uint4*>(qg + (size_t)row * D) = pack8(qv);
         }
     }
-    fail = !mbar_wait(&bar_mma, 0);
-    if (__syncthreads_or(fail)) {
-        if (tid == 0) *p.status = QD_ERR_TIMEOUT;
-        if (warp == 0) tmem_dealloc(tbase, 256);
-        return;
-    }
-    if (has_lam) {
-        // X = K + lambda Q, in place over Q (K-major swizzled layout)
-#pragma unroll 4
-        for (int it = 0; it < 8; ++it) {
-            const int row = it * 16 + rsub;
-            const uint32_t off = coff + sw128_chunk(row, ch & 7);
-            const float lm = slam[row];
-            float qv[8], kv[8];
-            load8(sQ + off, qv);
-            load8(sK + off, kv);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) kv[e] = fmaf(lm, qv[e], kv[e]);
-            sts128(sX + off, pack8(kv));
-        }
-        fence_proxy_async();
-        tc_fence_before();
-        __syncthreads();
-        if (tid == 0) {
-            tc_fence_after();
-            // G1 = X K^T -> columns [0,128)
-            umma_product<false, false>(tbase, smem_u32(sX), 16384, smem_u32(sK), 16384, 128, 128, false);
-            umma_commit(&bar_mma);
-        }
-        fail = !mbar_wait(&bar_mma, 1);
-        if (__syncthreads_or(fail)) {
-            if (tid == 0) *p.status = QD_ERR_TIMEOUT;
-            if (warp == 0) tmem_dealloc(tbase, 256);
-            return;
-        }
-    }
+    if (expired(!mbar_wait(&bar_mma, 0))) return;
     tc_fence_after();
-    // A = strictLower(beta_r Gamma_ri (x_r . k_i)) -> shared fp32, transposed;  P = Gamma_ri (q_r . k_i), i <= r -> workspace
+    // Q, K have been read by everybody: X over Q (K-major swizzled layout), A over K
+    if (build_x) {
+#pragma unroll
+        for (int it = 0; it < 8; ++it) sts128(sX + coff + sw128_chunk(it * 16 + rsub, ch & 7), xr[it]);
+    }
+    // A = strictLower(beta_r Gamma_ri (x_r . k_i)) -> shared fp32, transposed;  P = Gamma_ri (q_r . k_i), i <= r, kept in
+    // registers until its staging tile is free
+    uint4 pk[4];
+    const int row = tid & 127, half = tid >> 7;
     {
-        const int row = tid & 127, half = tid >> 7, c = row >> 6, r = row & 63;
+        const int c = row >> 6, r = row & 63;
         const float g = sg[row], beta = sbeta[row];
-        const float* gc = sg + c * C;
+        const float rq = NORM ? srq[row] : 1.f, rk = NORM ? srk[row] : 1.f, lm = slam[row] * rq;
+        const float *gc = sg + c * C, *rc = srk + c * C;
         float* Ac = sA + c * C * C;
         float v1[32], v2[32];
         tmem_ld32(tmem_addr(tbase, (warp & 3) * 32, c * C + half * 32), v1);
         tmem_ld32(tmem_addr(tbase, (warp & 3) * 32, 128 + c * C + half * 32), v2);
         tmem_ld_wait();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const int col = half * 32 + i;
-            const float dec = (col <= r) ? __expf(g - gc[col]) : 0.f;
-            v1[i] = (col < r) ? beta * dec * v1[i] : 0.f;
-            v2[i] = dec * v2[i];
+        for (int i4 = 0; i4 < 8; ++i4) {
+            const float4 g4 = *reinterpret_cast<const float4*>(gc + half * 32 + i4 * 4);
+            const float4 r4 = NORM ? *reinterpret_cast<const float4*>(rc + half * 32 + i4 * 4) : make_float4(1.f, 1.f, 1.f, 1.f);
+            const float gq[4] = {g4.x, g4.y, g4.z, g4.w}, rq4[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = i4 * 4 + e, col = half * 32 + i;
+                float dec = (col <= r) ? __expf(g - gq[e]) : 0.f;
+                if (NORM) dec *= rq4[e];
+                sts32(Ac + at_off(col, r), (col < r) ? beta * dec * fmaf(lm, v2[i], rk * v1[i]) : 0.f);
+                v2[i] = dec * (rq * v2[i]);
+            }
         }
-        // A^T: entry (column i, row r) at i*64 + r, so that 8 consecutive rows of one column are contiguous
 #pragma unroll
-        for (int i = 0; i < 32; ++i) Ac[(half * 32 + i) * C + r] = v1[i];
-        bf16* prow = p.P + (wtok0 + row) * C + half * 32;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(prow + i * 8) = pack8(v2 + i * 8);
+        for (int i = 0; i < 4; ++i) pk[i] = pack8(v2 + i * 8);
     }
     tc_fence_before();
     __syncthreads();
-    // M_c = (I + A_c)^-1 by right-looking substitution, columns in registers.  A lane quad of the first four warps
-    // owns four columns of one chunk, j0 + 16 k with j0 < 16 (the same loads of A serve all four); lane `ql` of the
-    // quad owns the 8-row blocks ql and ql + 4.  Once m[i] is final its owner hands it to the other three lanes and
-    // every later row gets its update m[r] -= A[r][i] m[i]; rows <= i of a block see A = 0 exactly, so whole blocks
-    // are updated.  Column j0 + 16 k is zero above row 16 k and joins at step 16 k; blocks 0..3 are final after step
-    // 30.  The loads of A are warp-wide broadcasts, and shared-memory wavefronts are what bounds this phase: hence
-    // four columns per load (32 FMAs for two 16-byte loads).
-    const int qd4 = tid >> 2, ql = tid & 3, ic = (qd4 >> 4) & 1, j0 = qd4 & 15;
-    float m[2][4][8];
-    if (tid < 128) {
-        const float* Ac = sA + ic * C * C + ql * 8;
-#pragma unroll
-        for (int sb = 0; sb < 2; ++sb)
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) m[sb][k][e] = ((ql + 4 * sb) * 8 + e == j0 + 16 * k) ? 1.f : 0.f;
-#pragma unroll
-        for (int i = 0; i < C - 1; ++i) {
-            const int bi = i >> 3;                              // block of the pivot row; its owner is quad lane bi & 3
-            const int src = (lane & ~3) | (bi & 3);
-            float mi[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                mi[k] = (i >= 16 * k) ? __shfl_sync(0xffffffffu, m[bi >> 2][k][i & 7], src) : 0.f;
-#pragma unroll
-            for (int sb = (i < 31 ? 0 : 1); sb < 2; ++sb) {
-                const float4 a0 = *reinterpret_cast<const float4*>(Ac + i * C + sb * 32);
-                const float4 a1 = *reinterpret_cast<const float4*>(Ac + i * C + sb * 32 + 4);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (i >= 16 * k) {
-                        float* mm = m[sb][k];
-                        mm[0] = fmaf(-a0.x, mi[k], mm[0]); mm[1] = fmaf(-a0.y, mi[k], mm[1]);
-                        mm[2] = fmaf(-a0.z, mi[k], mm[2]); mm[3] = fmaf(-a0.w, mi[k], mm[3]);
-                        mm[4] = fmaf(-a1.x, mi[k], mm[4]); mm[5] = fmaf(-a1.y, mi[k], mm[5]);
-                        mm[6] = fmaf(-a1.z, mi[k], mm[6]); mm[7] = fmaf(-a1.w, mi[k], mm[7]);
-                    }
-                }
-            }
-        }
-    }
-    __syncthreads();
-    // T_c = M_c diag(beta), T_c diag(gamma): line j of the MN-major tiles holds column j over the rows
-    if (tid < 128) {
-        unsigned char* t0 = sT + ic * 8192;
-        unsigned char* t1 = sT + 16384 + ic * 8192;
-        bf16* mt = p.Mt ? p.Mt + ((size_t)bh * p.N + 2 * pr + ic) * C * C : nullptr;
+    invert_pair(sA);
+    // T_c = M_c diag(beta), T_c diag(gamma): line j of the MN-major tiles holds column j over the rows; thread = (column
+    // j of chunk c, block of eight rows), eight threads to a column.  The tiles take A's place: everything is read first.
+    {
+        float m[4][8];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int j = j0 + 16 * k;
-            const float beta = sbeta[ic * C + j], bg = beta * __expf(sg[ic * C + j]);
+            const int id = k * kPrepThreads + tid, c = id >> 9, j = (id >> 3) & 63, kb = id & 7;
 #pragma unroll
-            for (int sb = 0; sb < 2; ++sb) {
-                const int kb = ql + 4 * sb;
-                float a[8], bq[8];
+            for (int e = 0; e < 8; e += 4)
+                *reinterpret_cast<float4*>(m[k] + e) = *reinterpret_cast<const float4*>(sA + c * C * C + at_off(j, kb * 8 + e));
+        }
+        __syncthreads();
 #pragma unroll
-                for (int e = 0; e < 8; ++e) { a[e] = m[sb][k][e] * beta; bq[e] = m[sb][k][e] * bg; }
-                sts128(t0 + sw128_chunk(j, kb), pack8(a));
-                sts128(t1 + sw128_chunk(j, kb), pack8(bq));
-                if (mt) *reinterpret_cast<uint4*>(mt + (size_t)j * C + kb * 8) = pack8(m[sb][k]);
-            }
+        for (int k = 0; k < 4; ++k) {
+            const int id = k * kPrepThreads + tid, c = id >> 9, j = (id >> 3) & 63, kb = id & 7;
+            const float beta = sbeta[c * C + j], bg = beta * __expf(sg[c * C + j]);
+            float a[8], bq[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) { a[e] = m[k][e] * beta; bq[e] = m[k][e] * bg; }
+            sts128(sT + c * 8192 + sw128_chunk(j, kb), pack8(a));
+            sts128(sT + 16384 + c * 8192 + sw128_chunk(j, kb), pack8(bq));
+            if (p.Mt) *reinterpret_cast<uint4*>(p.Mt + (((size_t)bh * p.N + 2 * pr + c) * C + j) * C + kb * 8) = pack8(m[k]);
         }
     }
     fence_proxy_async();
-    tc_fence_before();
-    __syncthreads();
+    if (expired(!mbar_wait(&bar_v, 0))) return;
     if (tid == 0) {
         tc_fence_after();
         for (int cc = 0; cc < 2; ++cc) {
@@ -333,26 +373,22 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
         }
         umma_commit(&bar_mma);
     }
-    fail = !mbar_wait(&bar_mma, has_lam ? 0 : 1);          // third phase of the barrier with lambda, second without
-    if (__syncthreads_or(fail)) {
-        if (tid == 0) *p.status = QD_ERR_TIMEOUT;
-        if (warp == 0) tmem_dealloc(tbase, 256);
-        return;
-    }
+    if (expired(!mbar_wait(&bar_mma, 1))) return;
     tc_fence_after();
     // row d = tid & 127 of U~^T (threads < 128) resp. W~^T (the others), both chunks: staged as swizzled
-    // [128][64] tiles over the dead Q/X and V regions, then written by TMA
+    // [128][64] tiles over the dead X and V regions; P, [64 tokens][64] per chunk, over the T tiles; all written by TMA
     {
-        const int d = tid & 127, which = tid >> 7;
-        unsigned char* stage = which ? sV : sQ;
+        unsigned char* stage = half ? sV : sX;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sts128(sScr + (row >> 6) * 8192 + sw128_chunk(row & 63, half * 4 + i), pk[i]);
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4) {
             float v[32];
-            tmem_ld32(tmem_addr(tbase, (warp & 3) * 32, which * 128 + q4 * 32), v);
+            tmem_ld32(tmem_addr(tbase, (warp & 3) * 32, half * 128 + q4 * 32), v);
             tmem_ld_wait();
             unsigned char* tile = stage + (q4 >> 1) * 16384;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) sts128(tile + sw128_chunk(d, (q4 & 1) * 4 + i), pack8(v + i * 8));
+            for (int i = 0; i < 4; ++i) sts128(tile + sw128_chunk(row, (q4 & 1) * 4 + i), pack8(v + i * 8));
         }
     }
     fence_proxy_async();
@@ -360,10 +396,12 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
     __syncthreads();
     if (tid == 0) {
         const int y = (int)(((size_t)bh * p.N + 2 * pr) * D);
-        tma_store_2d(&mapUt, sQ, 0, y);
-        tma_store_2d(&mapUt, sQ + 16384, 0, y + D);
+        tma_store_2d(&mapUt, sX, 0, y);
+        tma_store_2d(&mapUt, sX + 16384, 0, y + D);
         tma_store_2d(&mapWt, sV, 0, y);
         tma_store_2d(&mapWt, sV + 16384, 0, y + D);
+        tma_store_2d(&mapP, sScr, 0, (int)wtok0);
+        tma_store_2d(&mapP, sScr + 8192, 0, (int)wtok0 + C);
         tma_store_commit();
         tma_store_wait_read();             // the staging tiles must outlive the reads; the writes complete with the grid
     }
@@ -710,20 +748,21 @@ TcLayout tc_layout(const qd_shape& s) {
 
 cudaError_t tc_prep(const ChunkArgs& a) {
     const qd_shape& s = a.s;
-    CUtensorMap mQ, mK, mV, mUt, mWt;
+    CUtensorMap mQ, mK, mV, mUt, mWt, mP;
     const int Tp = tc_padded_T(s);
     const uint64_t trows = (uint64_t)s.B * s.H * (Tp / kChunk) * D;          // rows of the [chunk][d][64] tiles
     if (!make_tmap_tokens(&mQ, a.q, s.B, s.T, s.H, D, 128) || !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 128) ||
         !make_tmap_tokens(&mV, a.v, s.B, s.T, s.H, D, 128) ||
         !make_tmap_bf16_2d(&mUt, a.ws + a.TL.Ut, 64, trows, 128, 128) ||
-        !make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, trows, 128, 128))
+        !make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, trows, 128, 128) ||
+        !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, (uint64_t)s.B * s.H * Tp, 128, 64))
         return cudaErrorInvalidValue;
     PrepParams p{};
     p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = Tp / kChunk; p.BH = s.B * s.H;
     p.rqk = a.norm ? (float*)(a.ws + a.TL.rqk) : nullptr;
     p.beta = (const bf16*)a.beta; p.alpha = (const bf16*)a.alpha; p.lam = (const bf16*)a.lam;
     p.g = (float*)(a.ws + a.TL.g);
-    p.Qg = (bf16*)(a.ws + a.TL.Qg); p.P = (bf16*)(a.ws + a.TL.P);
+    p.Qg = (bf16*)(a.ws + a.TL.Qg);
     p.Mt = a.save ? (bf16*)(a.ws + a.TL.Mt) : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
     auto kern = a.norm ? (a.logits ? k_tc_prep<true, true> : k_tc_prep<true, false>)
@@ -731,7 +770,7 @@ cudaError_t tc_prep(const ChunkArgs& a) {
     cudaError_t e = set_smem(kern, kPrepSmem);
     if (e != cudaSuccess) return e;
     const int grid = s.B * s.H * (p.N / 2);
-    return launch_overlapped(kern, dim3((unsigned)grid), dim3(kPrepThreads), kPrepSmem, a.stream, mQ, mK, mV, mUt, mWt, p);
+    return launch_overlapped(kern, dim3((unsigned)grid), dim3(kPrepThreads), kPrepSmem, a.stream, mQ, mK, mV, mUt, mWt, mP, p);
 }
 
 cudaError_t tc_chain_fwd(const ChunkArgs& a) {
