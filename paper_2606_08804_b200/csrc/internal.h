@@ -58,6 +58,7 @@ struct TcLayout {
 };
 TcLayout tc_layout(const qd_shape& s);
 bool tc_supported(const qd_shape& s);
+int chain_rows(uint64_t BH);      // d_v rows of a state that one CTA of the state chains owns: 128 or 64
 // Rows per sequence in the tensor-core workspace: T rounded up to a whole number of chunk PAIRS (the preparation kernel
 // takes two chunks at a time).  The rows past T behave as tokens with beta = 0, alpha = 1, q = k = v = 0, which leave the
 // recurrence of Section 3.3.1 untouched; TMA supplies the zeros and drops the stores.

@@ -258,6 +258,56 @@ __device__ __forceinline__ void umma_product_ts(uint32_t d_tmem, uint32_t a_tmem
     }
 }
 
+// ---- the same, issued by a whole converged warp ---------------------------------------------------------------------
+// One lane issues (`issue` is nonzero in one lane only), but the code around it stays warp-uniform, so that descriptors and
+// their increments live in uniform registers.  From a branch that a single lane takes, every instruction's operands are
+// moved there one by one: 80 - 130 cycles per instruction against 20 - 50.  The role of a warp has to come from warp_index().
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ uint32_t elect_lane() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void umma_commit_w(uint64_t* bar, uint32_t issue) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+        ::"r"(smem_u32(bar)), "r"(issue) : "memory");
+}
+template <bool A_MN, bool B_MN>
+__device__ __forceinline__ void umma_product_w(uint32_t d_tmem, uint32_t a_saddr, uint32_t a_blk, uint32_t b_saddr, uint32_t b_blk,
+                                               int N, int K, bool accumulate, uint32_t issue, bool a_neg = false) {
+    const uint32_t idesc = make_idesc(128, N, A_MN, B_MN, a_neg);
+    const uint64_t a0 = A_MN ? desc_mnmajor(a_saddr, a_blk) : desc_kmajor(a_saddr);
+    const uint64_t b0 = B_MN ? desc_mnmajor(b_saddr, b_blk) : desc_kmajor(b_saddr);
+#pragma unroll
+    for (int k = 0; k < K; k += 16) {
+        const uint32_t ao = A_MN ? (uint32_t)k * 128u : (uint32_t)(k >> 6) * a_blk + (uint32_t)(k & 63) * 2u;
+        const uint32_t bo = B_MN ? (uint32_t)k * 128u : (uint32_t)(k >> 6) * b_blk + (uint32_t)(k & 63) * 2u;
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+            "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(a0 + (uint64_t)(ao >> 4)), "l"(b0 + (uint64_t)(bo >> 4)), "r"(idesc),
+              "r"((uint32_t)(accumulate || k > 0)), "r"(issue) : "memory");
+    }
+}
+template <bool B_MN>
+__device__ __forceinline__ void umma_product_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_saddr, uint32_t b_blk, int N, int K,
+                                                  bool accumulate, uint32_t issue, bool a_neg = false) {
+    const uint32_t idesc = make_idesc(128, N, false, B_MN, a_neg);
+    const uint64_t b0 = B_MN ? desc_mnmajor(b_saddr, b_blk) : desc_kmajor(b_saddr);
+#pragma unroll
+    for (int k = 0; k < K; k += 16) {
+        const uint32_t bo = B_MN ? (uint32_t)k * 128u : (uint32_t)(k >> 6) * b_blk + (uint32_t)(k & 63) * 2u;
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+            "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "r"(a_tmem + (uint32_t)(k >> 1)), "l"(b0 + (uint64_t)(bo >> 4)), "r"(idesc),
+              "r"((uint32_t)(accumulate || k > 0)), "r"(issue) : "memory");
+    }
+}
+
 // Byte offset of element (line, e) inside a swizzled [lines][64] bf16 tile (e in 0..63).
 __device__ __forceinline__ uint32_t sw128_off(uint32_t line, uint32_t e) {
     return line * 128u + ((((e >> 3) ^ line) & 7u) << 4) + ((e & 7u) << 1);

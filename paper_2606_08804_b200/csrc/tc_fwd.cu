@@ -417,6 +417,7 @@ struct ChainParams {
     const float* g;
     const float* h0;
     float* hT;
+    int rows;                  // d_v rows of the state per CTA: 128, or 64 (two CTAs per sequence)
     int save;                  // also store, per chunk, the bf16 entry state (mapHs) and Delta^T (mapDt)
     int scaled;                // 0: no forget gate and no key normalisation: every per-token factor on Delta is 1
     const float* rk;           // non-null (QD_NORM_QK): 1/|k_t| per workspace row; the keys are read un-normalised and
@@ -424,15 +425,17 @@ struct ChainParams {
     unsigned* status;
 };
 
-constexpr int kStage = 73728;                                   // Wt 16K | Ut 16K | Qg 16K | K 16K | P 8K
-constexpr int kChainSmem = 2 * kStage + 65536 + 16384 + 1024;   // + h^T 32K, Delta^T 16K, scaled Delta^T 16K, O 16K
+// Tiles of a chunk in shared memory.  Wt 16K | Ut 16K, three deep (Delta^T is staged over Ut and held until it has been
+// read); Qg 16K | K 16K | P 8K, two deep; the exit state 32K; half an output tile 8K.
+constexpr int kDeepA = 3, kStageA = 32768, kStageB = 40960;
+constexpr int kOffB = kDeepA * kStageA, kOffH = kOffB + 2 * kStageB, kOffO = kOffH + 32768;
+constexpr int kChainSmem = kOffO + 8192 + 1024;
 constexpr int kChainCompute = 512;                 // 16 epilogue warps: 4 warpgroups split the accumulator columns
-constexpr int kChainThreads = kChainCompute + 64;  // + 1 MMA-issue warp, 1 TMA warp
-constexpr int kMmaWarp = kChainCompute / 32;
-constexpr int kNb = kChainCompute + 32;            // participants of a named barrier: the epilogue threads and one waiting warp
+constexpr int kChainThreads = kChainCompute + 128 + 64;   // + the output warpgroup, 1 MMA-issue warp, 1 TMA warp
+constexpr int kOutWarp = kChainCompute / 32, kMmaWarp = kOutWarp + 4;
 
-// named barriers: compute threads arrive, the MMA and/or TMA warp wait
-constexpr int kBarH = 1, kBarD = 2, kBarO = 3, kBarHt = 4, kBarDt = 5;   // ..t: the same event, awaited by the TMA warp
+// named barriers: compute threads arrive, the MMA warp waits (they run in lock-step); kBarOut: the output warpgroup among itself
+constexpr int kBarH = 1, kBarD = 2, kBarOut = 3;
 __device__ __forceinline__ void nb_arrive(int id, int count) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory"); }
 __device__ __forceinline__ void nb_sync(int id, int count) {
     __syncwarp();                                   // the lanes of a warp reach the barrier together
@@ -443,8 +446,18 @@ __device__ __forceinline__ void nb_sync(int id, int count) {
 //   h ready -> Delta-accumulator = h^T Wt -> Delta^T -> H-accumulator = (scaled Delta^T) K -> h update;
 // the output products (h^T Qg^T + Delta^T P^T, double-buffered accumulator), the output epilogue and
 // every TMA copy run in its shadow on their own warps.
-// Compute warpgroup w owns tokens [32w, 32w+32) of the 64-column accumulators and d_k columns
-// [64w, 64w+64) of the state; thread l of a warpgroup owns TMEM lane l = d_v index.
+// What bounds a chunk is that sequence, if nothing gets in its way.  Three things did, 3800 cycles per chunk of 64 tokens:
+//  - the shared-memory port: with h^T and Delta^T as shared-memory operands it carried 368 KB per chunk, 2900 cycles.  They
+//    are A operands, so they live in tensor memory (bf16 pairs, written by the epilogues with tcgen05.st): no operand copies,
+//    no re-reading of A by every product;
+//  - the issue of 24 products from a branch taken by one lane, 80 - 130 cycles each: the MMA warp stays converged;
+//  - TMA, whose loads run at 45 and stores at 32 bytes per cycle and SM, one after the other (measured): the 72 KB that a chunk
+//    loads and the 16 KB of its output take 2150 cycles, and the 48 KB of Delta^T and entry state that a forward saves for the
+//    backward 1300 more.  (Ordinary stores, by one or two warps from the tiles or by the epilogue from its registers, were
+//    slower: 4500 - 5000 cycles per chunk.)  So with few heads the d_v rows of a head, which evolve independently, are shared by
+//    two CTAs (`rows` = 64): each loads what both need, but only its half of Ut, and stores its half of everything.
+// Compute warpgroup w owns tokens [16w, 16w+16) of the 64-column accumulators and d_k columns
+// [32w, 32w+32) of the state; thread l of a warpgroup owns TMEM lane l = d_v index.
 __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_constant__ CUtensorMap mapWt,
                                                                 const __grid_constant__ CUtensorMap mapUt,
                                                                 const __grid_constant__ CUtensorMap mapQg,
@@ -456,23 +469,27 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                                                                 ChainParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* sH = smem + 2 * kStage;          // h^T as A operand: K-major, 2 blocks of [128 lines][64]
-    unsigned char* sD = sH + 32768;                 // Delta^T: K-major [128 lines (dv)][64 tokens]
-    unsigned char* sDs = sD + 16384;                // Delta^T scaled by gamma_C/gamma_r per token
-    unsigned char* sO = sDs + 16384;                // output tile [64 tokens][128 dv], 2 blocks of [64 lines][64]
-    __shared__ uint64_t bar_load[2], bar_a, bar_b, bar_o, bar_e;
+    unsigned char* sH = smem + kOffH;               // h^T [128 dv][128 dk] for its store, 2 blocks of [128 lines][64]
+    unsigned char* sO = smem + kOffO;               // half an output tile: [32 tokens][128 dv], 2 blocks of [32 lines][64]
+    // Where one side may run ahead of the other there is a barrier per buffer; it comes round only after the other side has
+    // waited for it.  bar_e: every product of a chunk has finished; bar_dt, bar_ht: Delta^T / exit state staged for their stores
+    // (one arrival per compute warp); bar_hf: the state's tile has been read; bar_o, bar_of: an output accumulator is complete /
+    // has been read.
+    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_ht, bar_hf, bar_a, bar_b, bar_o[2], bar_of[2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
-    // per chunk parity: gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the TMA warp one chunk
-    // ahead and published with its arrival on bar_a, so no epilogue thread waits for a global load
-    __shared__ __align__(16) float sG[2][68];
+    // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the TMA warp before it arrives on the
+    // stage's load barrier, so no epilogue thread waits for a global load
+    __shared__ __align__(16) float sG[kDeepA][68];
 
-    const int tid = threadIdx.x, warp = tid >> 5, wg = tid >> 7, l = tid & 127, wq = warp & 3;
-    const int bh = blockIdx.x, b = bh / p.H, hh = bh % p.H;
+    const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, l = tid & 127, wq = warp & 3;
+    const int rows = p.rows, nwq = rows / 32, nb = 4 * rows + 32;    // d_v rows of this CTA; warps of a warpgroup; barrier participants
+    const int parts = D / rows, bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
 
     if (tid == 0) {
-        mbar_init(&bar_load[0], 1); mbar_init(&bar_load[1], 1);
-        mbar_init(&bar_a, 2); mbar_init(&bar_b, 2); mbar_init(&bar_o, 2); mbar_init(&bar_e, 1);
+        for (int i = 0; i < kDeepA; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_dt[i], 4 * nwq); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar_lb[i], 1); mbar_init(&bar_e[i], 1); mbar_init(&bar_o[i], 1); mbar_init(&bar_of[i], nwq); }
+        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1); mbar_init(&bar_ht, 4 * nwq); mbar_init(&bar_hf, 1);
         mbar_init_fence();
         s_abort = 0;
     }
@@ -480,8 +497,10 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tbase = tmem_slot;
-    const uint32_t tD = tbase, tH = tbase + 128, tO0 = tbase + 256;      // O-accumulators: tO0 + 64 * (n & 1)
+    const uint32_t tbase = uniform(tmem_slot);
+    // accumulators: Delta 64 columns, H 128, O 2 x 64; operands, two bf16 per column: h^T 64, Delta^T 32, scaled Delta^T 32
+    const uint32_t tD = tbase, tH = tbase + 64, tO0 = tbase + 192, aH = tbase + 320, aD = tbase + 384;
+    const uint32_t aDs = p.scaled ? tbase + 416 : aD;               // all factors 1: the scaled copy is Delta itself
     const uint32_t lane_base = (uint32_t)wq * 32;
 
     // bounded wait; once any wait has expired every later wait returns at once (the kernel drains)
@@ -491,11 +510,13 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     };
     const float* gseq = p.g + (size_t)bh * p.Tp;
 
-    if (warp < kMmaWarp) {
+    if (warp < kMmaWarp && wq >= nwq) {
+        // lanes without a row: straight to the end
+    } else if (warp < kOutWarp) {
         // ---------------------------------- compute warps ----------------------------------
         float h[32];      // h^T[j = l][32 wg .. 32 wg + 31], fp32
         if (p.h0) {
-            const float* src = p.h0 + (size_t)bh * D * D + (size_t)(32 * wg) * D + l;
+            const float* src = p.h0 + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
             for (int i = 0; i < 32; ++i) h[i] = src[(size_t)i * D];
         } else {
@@ -504,74 +525,68 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         }
         grid_dep_wait();                  // the loads of h0 (an input) are in flight; everything below depends on the prep kernel
         grid_dep_launch();
-        // my 32 columns of the operand tile: 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
-        unsigned char* myH = sH + (wg >> 1) * 16384;
-        const int hc0 = (wg & 1) * 4;
+        // the state as operand: my 32 columns are 16 packed columns of tensor memory
+        auto put_h = [&]() {
+            uint32_t r[8];
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) sts128(myH + sw128_chunk(l, hc0 + ch), pack8(h + ch * 8));
-        // byte offsets of my (fixed) column inside a staging line, for the 8 possible (token & 7)
-        uint32_t xoff[8];
+            for (int q = 0; q < 2; ++q) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-            xoff[e] = (uint32_t)e * 128u + (((((uint32_t)l & 63u) >> 3) ^ (uint32_t)e) << 4) + ((uint32_t)l & 7u) * 2u;
-        fence_proxy_async();
-        nb_arrive(kBarH, kNb); nb_arrive(kBarHt, kNb);
-
-        auto o_stage = [&](int m) {
-            // output of chunk m: O^T row j = l, my 16 tokens -> staging tile (token-major); stored by the TMA warp
-            unsigned char* stg = sO + (l >> 6) * 8192 + (wg * 16) * 128;
-            float v[16];
-            tmem_ld16(tmem_addr(tO0 + 64 * (m & 1), lane_base, wg * 16), v);
-            tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) sts16(stg + (i >> 3) * 1024 + xoff[i & 7], __float2bfloat16_rn(v[i]));
+                for (int e = 0; e < 8; ++e) r[e] = pack_bf16(h[q * 16 + 2 * e], h[q * 16 + 2 * e + 1]);
+                tmem_st8(tmem_addr(aH, lane_base, wg * 16 + q * 8), r);
+            }
+            tmem_st_wait();
             tc_fence_before();
-            fence_proxy_async();
-            nb_arrive(kBarO, kNb);
+            nb_arrive(kBarH, nb);
         };
-
+        auto staged = [&](uint64_t* bar) {                // my warp's part of a tile is in shared memory, for the TMA warp
+            fence_proxy_async();
+            __syncwarp();
+            if ((tid & 31) == 0) mbar_arrive(bar);
+        };
+        auto save_h = [&]() {             // the state as a tile: 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) sts128(sH + (wg >> 1) * 16384 + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(h + ch * 8));
+            staged(&bar_ht);
+        };
+        put_h();
+        if (p.save) save_h();
+        int s = 0;
         for (int n = 0; n < p.N; ++n) {
-            const unsigned char* st = smem + (n & 1) * kStage;
-            wait(&bar_load[n & 1], (n >> 1) & 1);
+            unsigned char* ut = smem + s * kStageA + 16384;
+            wait(&bar_la[s], (n / kDeepA) & 1);
+            const uint4 u0 = *reinterpret_cast<const uint4*>(ut + sw128_chunk(l, wg * 2));           // before the product is waited for
+            const uint4 u1 = *reinterpret_cast<const uint4*>(ut + sw128_chunk(l, wg * 2 + 1));
+            const float gamC = sG[s][64];
             wait(&bar_a, n & 1);
             tc_fence_after();
-            // decay ratios of my 16 tokens
-            float sc[16];
+            // Delta^T = Ut - acc, my 16 tokens, as operands: plain, and scaled by gamma_C/gamma_r
             {
-                const float4* gp = reinterpret_cast<const float4*>(&sG[n & 1][wg * 16]);
+                float v[16];
+                tmem_ld16(tmem_addr(tD, lane_base, wg * 16), v);
+                const float4* gp = reinterpret_cast<const float4*>(&sG[s][wg * 16]);
+                const uint32_t uw[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+                tmem_ld_wait();
+                uint32_t r[8], rs[8];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const float4 t = gp[q];
-                    sc[q * 4] = t.x; sc[q * 4 + 1] = t.y; sc[q * 4 + 2] = t.z; sc[q * 4 + 3] = t.w;
+                    const float x0 = __uint_as_float(uw[2 * q] << 16) - v[4 * q], x1 = __uint_as_float(uw[2 * q] & 0xffff0000u) - v[4 * q + 1];
+                    const float x2 = __uint_as_float(uw[2 * q + 1] << 16) - v[4 * q + 2], x3 = __uint_as_float(uw[2 * q + 1] & 0xffff0000u) - v[4 * q + 3];
+                    r[2 * q] = pack_bf16(x0, x1); r[2 * q + 1] = pack_bf16(x2, x3);
+                    rs[2 * q] = pack_bf16(x0 * t.x, x1 * t.y); rs[2 * q + 1] = pack_bf16(x2 * t.z, x3 * t.w);
+                }
+                if (p.scaled) tmem_st8(tmem_addr(aDs, lane_base, wg * 8), rs);
+                tmem_st8(tmem_addr(aD, lane_base, wg * 8), r);
+                tmem_st_wait();
+                tc_fence_before();
+                nb_arrive(kBarD, nb);
+                if (p.save) {
+                    sts128(ut + sw128_chunk(l, wg * 2), make_uint4(r[0], r[1], r[2], r[3]));
+                    sts128(ut + sw128_chunk(l, wg * 2 + 1), make_uint4(r[4], r[5], r[6], r[7]));
+                    staged(&bar_dt[s]);
                 }
             }
-            const float gamC = sG[n & 1][64];
-            // Delta^T = Ut - acc, my 16 tokens; two bf16 copies (plain, and scaled by gamma_C/gamma_r) as A operands
-            {
-                const unsigned char* ut = st + 16384;
-                float v[16];
-                tmem_ld16(tmem_addr(tD, lane_base, wg * 16), v);
-                tmem_ld_wait();
-#pragma unroll
-                for (int cc = 0; cc < 2; ++cc) {
-                    float u[8], d1[8];
-                    const uint32_t off = sw128_chunk(l, wg * 2 + cc);
-                    load8(ut + off, u);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        u[e] -= v[cc * 8 + e];
-                        d1[e] = u[e] * sc[cc * 8 + e];
-                    }
-                    sts128(sD + off, pack8(u));
-                    if (p.scaled) sts128(sDs + off, pack8(d1));         // all factors 1: the scaled copy is Delta itself
-                }
-            }
-            tc_fence_before();
-            fence_proxy_async();
-            nb_arrive(kBarD, kNb); nb_arrive(kBarDt, kNb);
-            // in the shadow of the H product: output epilogue of the previous chunk
-            if (n > 0) { wait(&bar_o, (n - 1) & 1); tc_fence_after(); o_stage(n - 1); }
-            // h^T <- gamma_C h^T + acc (my 32 d_k columns), refresh the bf16 operand copy
+            // h^T <- gamma_C h^T + acc (my 32 d_k columns), refresh the operand
             wait(&bar_b, n & 1);
             tc_fence_after();
             {
@@ -580,132 +595,167 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                 tmem_ld_wait();
 #pragma unroll
                 for (int i = 0; i < 32; ++i) h[i] = fmaf(gamC, h[i], v[i]);
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc) sts128(myH + sw128_chunk(l, hc0 + cc), pack8(h + cc * 8));
             }
-            tc_fence_before();
-            fence_proxy_async();
-            nb_arrive(kBarH, kNb); nb_arrive(kBarHt, kNb);
+            put_h();
+            if (p.save && n + 1 < p.N) { wait(&bar_hf, n & 1); save_h(); }
+            if (++s == kDeepA) s = 0;
         }
-        wait(&bar_o, (p.N - 1) & 1);
-        tc_fence_after();
-        o_stage(p.N - 1);
         if (p.hT && !s_abort) {
-            float* dst = p.hT + (size_t)bh * D * D + (size_t)(32 * wg) * D + l;
+            float* dst = p.hT + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
             for (int i = 0; i < 32; ++i) dst[(size_t)i * D] = h[i];
         }
-    } else if (warp == kMmaWarp) {
-        // ---------------------------------- MMA-issue warp ----------------------------------
-        const bool lead = (tid & 31) == 0;
-        grid_dep_wait();
-        grid_dep_launch();
-        const uint32_t aH = smem_u32(sH), aD = smem_u32(sD), aDs = p.scaled ? smem_u32(sDs) : smem_u32(sD);
+    } else if (warp < kMmaWarp) {
+        // ---------------------------------- output warpgroup ----------------------------------
+        // O^T row j = l of a chunk -> token-major half tiles -> TMA; its first thread issues the stores
+        const bool first = tid == kChainCompute;
+        uint32_t xoff[8];                 // byte offsets of my (fixed) column inside a staging line, for the 8 possible (token & 7)
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            xoff[e] = (uint32_t)e * 128u + (((((uint32_t)l & 63u) >> 3) ^ (uint32_t)e) << 4) + ((uint32_t)l & 7u) * 2u;
+        unsigned char* stg = sO + (l >> 6) * 4096;
         for (int n = 0; n < p.N; ++n) {
-            const uint32_t st = smem_u32(smem + (n & 1) * kStage);
-            const uint32_t tO = tO0 + 64 * (n & 1);
-            if (lead) wait(&bar_load[n & 1], (n >> 1) & 1);
-            nb_sync(kBarH, kNb);                          // h^T operand of chunk n is in place
-            if (lead) {
-                tc_fence_after();
-                // Delta-accumulator = h^T Wt (B: MN-major, lines = d_k)
-                umma_product<false, true>(tD, aH, 16384, st, 8192, C, D, false);
-                umma_commit(&bar_a);
-                // O-accumulator = h^T Qg^T (B: K-major); it reads the state tile, so the commit behind the
-                // H product below (which releases that tile) must cover it
-                umma_product<false, false>(tO, aH, 16384, st + 32768, 8192, C, D, false);
-            }
-            nb_sync(kBarD, kNb);                          // Delta^T operands of chunk n are in place
-            if (lead) {
-                tc_fence_after();
-                // H-accumulator = scaled Delta^T K (B: MN-major, lines = tokens)
-                umma_product<false, true>(tH, aDs, 16384, st + 49152, 8192, D, C, false);
-                umma_commit(&bar_b);
-                // O-accumulator += Delta^T P^T (B: K-major [r][s])
-                umma_product<false, false>(tO, aD, 16384, st + 65536, 8192, C, C, true);
-                umma_commit(&bar_o);
-                umma_commit(&bar_e);
+            const int ob = n & 1;
+            wait(&bar_o[ob], (n >> 1) & 1);
+            tc_fence_after();
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                float v[32];
+                tmem_ld32(tmem_addr(tO0 + 64 * ob, lane_base, half * 32), v);
+                tmem_ld_wait();
+                if (half == 1) {                          // the accumulator may be written again
+                    tc_fence_before();
+                    __syncwarp();
+                    if ((tid & 31) == 0) mbar_arrive(&bar_of[ob]);
+                }
+                if (first) tma_store_wait_read_n<0>();    // the half tile before has been read
+                nb_sync(kBarOut, rows);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) sts16(stg + (i >> 3) * 1024 + xoff[i & 7], __float2bfloat16_rn(v[i]));
+                fence_proxy_async();
+                nb_sync(kBarOut, rows);
+                if (first) {                              // rows past the end of the sequence are skipped
+                    tma_store_3d(&mapO, sO, hh * D + v0, n * C + half * 32, b);
+                    if (rows == D) tma_store_3d(&mapO, sO + 4096, hh * D + 64, n * C + half * 32, b);
+                    tma_store_commit();
+                }
             }
         }
-        nb_sync(kBarH, kNb);                              // final arrival of the compute warps
+        if (first) tma_store_wait_all();
+    } else if (warp == kMmaWarp) {
+        // ---------------------------------- MMA-issue warp, converged ----------------------------------
+        const uint32_t issue = elect_lane();
+        grid_dep_wait();
+        grid_dep_launch();
+        int s = 0;
+        for (int n = 0; n < p.N; ++n) {
+            const int ob = n & 1;
+            const uint32_t stA = smem_u32(smem) + s * kStageA, stB = smem_u32(smem) + kOffB + ob * kStageB;
+            const uint32_t tO = tO0 + 64 * ob;
+            wait(&bar_la[s], (n / kDeepA) & 1);
+            nb_sync(kBarH, nb);                          // h^T operand of chunk n is in place
+            tc_fence_after();
+            // Delta-accumulator = h^T Wt (B: MN-major, lines = d_k)
+            umma_product_ts_w<true>(tD, aH, stA, 8192, C, D, false, issue);
+            umma_commit_w(&bar_a, issue);
+            // O-accumulator = h^T Qg^T (B: K-major); it reads the operand that the h update rewrites, so the commit
+            // behind the H product below (which releases that update) must cover it
+            if (n > 1) wait(&bar_of[ob], ((n >> 1) - 1) & 1);
+            wait(&bar_lb[ob], (n >> 1) & 1);
+            tc_fence_after();
+            umma_product_ts_w<false>(tO, aH, stB, 8192, C, D, false, issue);
+            nb_sync(kBarD, nb);                          // Delta^T operands of chunk n are in place
+            tc_fence_after();
+            // H-accumulator = scaled Delta^T K (B: MN-major, lines = tokens)
+            umma_product_ts_w<true>(tH, aDs, stB + 16384, 8192, D, C, false, issue);
+            umma_commit_w(&bar_b, issue);
+            // O-accumulator += Delta^T P^T (B: K-major [r][s])
+            umma_product_ts_w<false>(tO, aD, stB + 32768, 8192, C, C, true, issue);
+            umma_commit_w(&bar_o[ob], issue);
+            umma_commit_w(&bar_e[ob], issue);
+            if (++s == kDeepA) s = 0;
+        }
+        nb_sync(kBarH, nb);                              // final arrival of the compute warps
     } else {
         // ---------------------------------- TMA warp ----------------------------------
         const bool lead = (tid & 31) == 0;
         grid_dep_wait();                  // the tiles and the log-decays read below are written by the prep kernel
         grid_dep_launch();
-        auto issue_load = [&](int n) {
-            unsigned char* st = smem + (n & 1) * kStage;
-            uint64_t* bar = &bar_load[n & 1];
-            mbar_expect_tx(bar, kStage);
-            const int yc = (int)(((size_t)bh * p.N + n) * D);
-            const int yt = (int)((size_t)bh * p.Tp + (size_t)n * C);
-            tma_load_2d(st, &mapWt, 0, yc, bar);
-            tma_load_2d(st + 16384, &mapUt, 0, yc, bar);
-            tma_load_2d(st + 32768, &mapQg, 0, yt, bar);
-            tma_load_2d(st + 32768 + 8192, &mapQg, 64, yt, bar);
-            tma_load_3d(st + 49152, &mapK, hh * D, n * C, b, bar);
-            tma_load_3d(st + 49152 + 8192, &mapK, hh * D + 64, n * C, b, bar);
-            tma_load_2d(st + 65536, &mapP, 0, yt, bar);
-        };
-        if (lead) { issue_load(0); if (p.N > 1) issue_load(1); }
         const int ln = tid & 31;
-        float g0 = gseq[ln], g1 = gseq[32 + ln], gc = gseq[C - 1];     // cumulative log-decays of chunk 0
         const float* rkseq = p.rk ? p.rk + (size_t)bh * p.Tp : nullptr;
-        float r0 = rkseq ? rkseq[ln] : 1.f, r1 = rkseq ? rkseq[32 + ln] : 1.f;
-        for (int n = 0; n < p.N; ++n) {
-            sG[n & 1][ln] = __expf(gc - g0) * r0;
-            sG[n & 1][32 + ln] = __expf(gc - g1) * r1;
-            if (ln == 0) sG[n & 1][64] = __expf(gc);
+        // log-decays (and 1/|k|) of the next chunk to be loaded, fetched ahead
+        float g0, g1, gc, r0 = 1.f, r1 = 1.f;
+        auto fetch_g = [&](int n) {
+            const float* gn = gseq + (size_t)n * C;
+            g0 = gn[ln]; g1 = gn[32 + ln]; gc = gn[C - 1];
+            if (rkseq) { r0 = rkseq[(size_t)n * C + ln]; r1 = rkseq[(size_t)n * C + 32 + ln]; }
+        };
+        auto load_a = [&](int n, int s) {                // by the whole warp
+            sG[s][ln] = __expf(gc - g0) * r0;
+            sG[s][32 + ln] = __expf(gc - g1) * r1;
+            if (ln == 0) sG[s][64] = __expf(gc);
             __syncwarp();
-            if (n + 1 < p.N) {                                  // in flight while this chunk is processed
-                const float* gn = gseq + (size_t)(n + 1) * C;
-                g0 = gn[ln]; g1 = gn[32 + ln]; gc = gn[C - 1];
-                if (rkseq) { r0 = rkseq[(size_t)(n + 1) * C + ln]; r1 = rkseq[(size_t)(n + 1) * C + 32 + ln]; }
-            }
             if (lead) {
-                // every store issued so far (Delta^T of chunk n-1, output of chunk n-2) has read its tile:
-                // the Delta^T tiles may be rewritten (chunk n), the output staging tile too (chunk n-1)
-                tma_store_wait_read_n<0>();
-                mbar_arrive(&bar_a);
-                if (n > 0) mbar_arrive(&bar_o);
+                const int yc = (int)(((size_t)bh * p.N + n) * D);
+                mbar_expect_tx(&bar_la[s], 16384 + rows * 128);
+                tma_load_2d(smem + s * kStageA, &mapWt, 0, yc, &bar_la[s]);
+                tma_load_2d(smem + s * kStageA + 16384, &mapUt, 0, yc + v0, &bar_la[s]);
             }
-            nb_sync(kBarHt, kNb);                          // h^T operand of chunk n is in place
-            if (lead && p.save) {
-                // entry state of chunk n, bf16, exactly the operand tile: rows = d_v index, cols = d_k index
-                const int yh = (int)(((size_t)bh * p.N + n) * D);
-                tma_store_2d(&mapHs, sH, 0, yh);
-                tma_store_2d(&mapHs, sH + 16384, 64, yh);
-            }
-            if (lead) tma_store_commit();                 // group: entry state of chunk n
-            nb_sync(kBarDt, kNb);                          // Delta^T of chunk n is in place
-            if (lead) {
-                if (p.save) tma_store_2d(&mapDt, sD, 0, (int)(((size_t)bh * p.N + n) * D));
-                tma_store_commit();                       // group: Delta^T of chunk n
-                tma_store_wait_read_n<1>();               // the entry-state tile has been read: it may be rewritten
-                mbar_arrive(&bar_b);
-            }
-            if (n > 0) {
-                nb_sync(kBarO, kNb);                      // output tile of chunk n-1 staged
-                if (lead) {
-                    tma_store_3d(&mapO, sO, hh * D, (n - 1) * C, b);      // rows past the end of the sequence are skipped
-                    tma_store_3d(&mapO, sO + 8192, hh * D + 64, (n - 1) * C, b);
-                    tma_store_commit();                   // group: output of chunk n-1
-                }
-            }
-            if (lead) {
-                wait(&bar_e, n & 1);                      // every product of chunk n has finished: refill its stage
-                if (n + 2 < p.N && !s_abort) issue_load(n + 2);
-            }
-        }
-        nb_sync(kBarHt, kNb);                              // final arrival of the compute warps
-        if (lead) { tma_store_wait_read_n<0>(); mbar_arrive(&bar_o); }
-        nb_sync(kBarO, kNb);                              // output tile of the last chunk staged
-        if (lead) {
-            tma_store_3d(&mapO, sO, hh * D, (p.N - 1) * C, b);
-            tma_store_3d(&mapO, sO + 8192, hh * D + 64, (p.N - 1) * C, b);
+            if (n + 1 < p.N) fetch_g(n + 1);
+        };
+        auto load_b = [&](int n) {                       // by the leading lane
+            unsigned char* st = smem + kOffB + (n & 1) * kStageB;
+            uint64_t* bar = &bar_lb[n & 1];
+            const int yt = (int)((size_t)bh * p.Tp + (size_t)n * C);
+            mbar_expect_tx(bar, kStageB);
+            tma_load_2d(st, &mapQg, 0, yt, bar);
+            tma_load_2d(st + 8192, &mapQg, 64, yt, bar);
+            tma_load_3d(st + 16384, &mapK, hh * D, n * C, b, bar);
+            tma_load_3d(st + 16384 + 8192, &mapK, hh * D + 64, n * C, b, bar);
+            tma_load_2d(st + 32768, &mapP, 0, yt, bar);
+        };
+        auto store_h = [&](int n) {       // entry state of chunk n (rows = d_v index, columns = d_k index)
+            const int yh = (int)(((size_t)bh * p.N + n) * D) + v0;
+            tma_store_2d(&mapHs, sH, 0, yh);
+            tma_store_2d(&mapHs, sH + 16384, 64, yh);
             tma_store_commit();
-            tma_store_wait_all();
-            if (s_abort) { mbar_wait(&bar_load[0], 0); mbar_wait(&bar_load[1], 0); }
+        };
+        fetch_g(0);
+        for (int n = 0; n < kDeepA && n < p.N; ++n) {
+            load_a(n, n);
+            if (lead && n < 2) load_b(n);
+        }
+        if (lead && p.save) { wait(&bar_ht, 0); store_h(0); }
+        int s = 0;
+        for (int n = 0; n < p.N; ++n) {
+            bool more = n + kDeepA < p.N;
+            if (lead) {
+                if (p.save) {
+                    wait(&bar_dt[s], (n / kDeepA) & 1);   // Delta^T of chunk n is staged
+                    tma_store_2d(&mapDt, smem + s * kStageA + 16384, 0, (int)(((size_t)bh * p.N + n) * D) + v0);
+                    tma_store_commit();
+                    tma_store_wait_read_n<1>();           // the entry state has been read: its tile may be rewritten
+                    mbar_arrive(&bar_hf);
+                }
+                wait(&bar_e[n & 1], (n >> 1) & 1);        // every product of chunk n has finished: refill its buffers
+                if (n + 2 < p.N && !s_abort) load_b(n + 2);
+                if (more && p.save) tma_store_wait_read_n<0>();
+            }
+            more = __shfl_sync(0xffffffffu, more && !s_abort, 0);     // one answer for the warp
+            if (more) load_a(n + kDeepA, s);
+            if (lead && p.save && n + 1 < p.N) {
+                wait(&bar_ht, (n + 1) & 1);               // exit state of chunk n is staged
+                store_h(n + 1);
+            }
+            __syncwarp();
+            if (++s == kDeepA) s = 0;
+        }
+        if (lead) {
+            if (p.save) tma_store_wait_all();
+            if (s_abort) {                // one more bounded chance for copies in flight
+                for (int i = 0; i < kDeepA; ++i) mbar_wait(&bar_la[i], 0);
+                for (int i = 0; i < 2; ++i) mbar_wait(&bar_lb[i], 0);
+            }
         }
     }
     tc_fence_before();
@@ -722,6 +772,9 @@ bool tc_supported(const qd_shape& s) {
     return s.dtype == QD_BF16 && s.dk == 128 && s.dv == 128 && s.chunk == kChunk &&
            (long long)s.B * s.H * tc_padded_T(s) * 128 < 0x7fffffffLL * 64;
 }
+
+// Two CTAs per sequence while that leaves no SM with two (MEASURED)
+int chain_rows(uint64_t BH) { return BH <= 74 ? 64 : 128; }
 
 TcLayout tc_layout(const qd_shape& s) {
     TcLayout L{};
@@ -777,12 +830,13 @@ cudaError_t tc_chain_fwd(const ChunkArgs& a) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
     const uint64_t BH = (uint64_t)s.B * s.H, N = Tp / kChunk;
+    const int rows = chain_rows(BH);
     CUtensorMap mWt, mUt, mQg, mK, mP, mHs, mDt, mO;
-    if (!make_tmap_bf16_2d(&mHs, a.ws + a.TL.hsT, D, BH * N * D, D * 2, 128) ||
-        !make_tmap_bf16_2d(&mDt, a.ws + a.TL.Dt, 64, BH * N * D, 128, 128) ||
-        !make_tmap_tokens(&mO, a.o, s.B, s.T, s.H, D, 64) ||
+    if (!make_tmap_bf16_2d(&mHs, a.ws + a.TL.hsT, D, BH * N * D, D * 2, rows) ||
+        !make_tmap_bf16_2d(&mDt, a.ws + a.TL.Dt, 64, BH * N * D, 128, rows) ||
+        !make_tmap_tokens(&mO, a.o, s.B, s.T, s.H, D, 32) ||
         !make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, BH * N * D, 128, 128) ||
-        !make_tmap_bf16_2d(&mUt, a.ws + a.TL.Ut, 64, BH * N * D, 128, 128) ||
+        !make_tmap_bf16_2d(&mUt, a.ws + a.TL.Ut, 64, BH * N * D, 128, rows) ||
         !make_tmap_bf16_2d(&mQg, a.ws + a.TL.Qg, D, BH * Tp, D * 2, 64) ||
         !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 64) ||
         !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, BH * Tp, 128, 64))
@@ -792,12 +846,13 @@ cudaError_t tc_chain_fwd(const ChunkArgs& a) {
     p.g = (const float*)(a.ws + a.TL.g);
     p.h0 = a.h0; p.hT = a.hT;
     p.save = a.save ? 1 : 0;
+    p.rows = rows;
     p.scaled = (a.alpha || a.norm) ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
     cudaError_t e = set_smem(k_tc_chain_fwd, kChainSmem);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(k_tc_chain_fwd, dim3((unsigned)BH), dim3(kChainThreads), kChainSmem, a.stream,
+    return launch_overlapped(k_tc_chain_fwd, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream,
                              mWt, mUt, mQg, mK, mP, mHs, mDt, mO, p);
 }
 
