@@ -431,7 +431,7 @@ constexpr int kDeepA = 3, kStageA = 32768, kStageB = 40960;
 constexpr int kOffB = kDeepA * kStageA, kOffH = kOffB + 2 * kStageB, kOffO = kOffH + 32768;
 constexpr int kChainSmem = kOffO + 8192 + 1024;
 constexpr int kChainCompute = 512;                 // 16 epilogue warps: 4 warpgroups split the accumulator columns
-constexpr int kChainThreads = kChainCompute + 128 + 64;   // + the output warpgroup, 1 MMA-issue warp, 1 TMA warp
+constexpr int kChainThreads = kChainCompute + 128 + 96;   // + the output warpgroup, 1 MMA-issue warp, 1 warp each for TMA loads and saves
 constexpr int kOutWarp = kChainCompute / 32, kMmaWarp = kOutWarp + 4;
 
 // named barriers: compute threads arrive, the MMA warp waits (they run in lock-step); kBarOut: the output warpgroup among itself
@@ -473,9 +473,9 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     unsigned char* sO = smem + kOffO;               // half an output tile: [32 tokens][128 dv], 2 blocks of [32 lines][64]
     // Where one side may run ahead of the other there is a barrier per buffer; it comes round only after the other side has
     // waited for it.  bar_e: every product of a chunk has finished; bar_dt, bar_ht: Delta^T / exit state staged for their stores
-    // (one arrival per compute warp); bar_hf: the state's tile has been read; bar_o, bar_of: an output accumulator is complete /
+    // (one arrival per compute warp); bar_df, bar_hf: they have been read; bar_o, bar_of: an output accumulator is complete /
     // has been read.
-    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_ht, bar_hf, bar_a, bar_b, bar_o[2], bar_of[2];
+    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_df[kDeepA], bar_ht, bar_hf, bar_a, bar_b, bar_o[2], bar_of[2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
     // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the TMA warp before it arrives on the
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     const int parts = D / rows, bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
 
     if (tid == 0) {
-        for (int i = 0; i < kDeepA; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_dt[i], 4 * nwq); }
+        for (int i = 0; i < kDeepA; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_dt[i], 4 * nwq); mbar_init(&bar_df[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&bar_lb[i], 1); mbar_init(&bar_e[i], 1); mbar_init(&bar_o[i], 1); mbar_init(&bar_of[i], nwq); }
         mbar_init(&bar_a, 1); mbar_init(&bar_b, 1); mbar_init(&bar_ht, 4 * nwq); mbar_init(&bar_hf, 1);
         mbar_init_fence();
@@ -676,8 +676,33 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             if (++s == kDeepA) s = 0;
         }
         nb_sync(kBarH, nb);                              // final arrival of the compute warps
+    } else if (warp == kMmaWarp + 1) {
+        // ---------------------------------- saving warp ----------------------------------
+        // apart from the loads, which would otherwise wait for what these wait for
+        if ((tid & 31) == 0 && p.save) {
+            grid_dep_wait();
+            int s = 0;
+            for (int n = 0; n < p.N; ++n) {
+                const int y = (int)(((size_t)bh * p.N + n) * D) + v0;
+                wait(&bar_ht, n & 1);                     // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
+                tma_store_2d(&mapHs, sH, 0, y);
+                tma_store_2d(&mapHs, sH + 16384, 64, y);
+                tma_store_commit();
+                if (n > 0) {                              // Delta^T of chunk n - 1 has been read
+                    tma_store_wait_read_n<1>();
+                    mbar_arrive(&bar_df[s == 0 ? kDeepA - 1 : s - 1]);
+                }
+                wait(&bar_dt[s], (n / kDeepA) & 1);       // Delta^T of chunk n is staged
+                tma_store_2d(&mapDt, smem + s * kStageA + 16384, 0, y);
+                tma_store_commit();
+                tma_store_wait_read_n<1>();               // the entry state has been read
+                mbar_arrive(&bar_hf);
+                if (++s == kDeepA) s = 0;
+            }
+            tma_store_wait_all();
+        }
     } else {
-        // ---------------------------------- TMA warp ----------------------------------
+        // ---------------------------------- TMA load warp ----------------------------------
         const bool lead = (tid & 31) == 0;
         grid_dep_wait();                  // the tiles and the log-decays read below are written by the prep kernel
         grid_dep_launch();
@@ -714,48 +739,26 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             tma_load_3d(st + 16384 + 8192, &mapK, hh * D + 64, n * C, b, bar);
             tma_load_2d(st + 32768, &mapP, 0, yt, bar);
         };
-        auto store_h = [&](int n) {       // entry state of chunk n (rows = d_v index, columns = d_k index)
-            const int yh = (int)(((size_t)bh * p.N + n) * D) + v0;
-            tma_store_2d(&mapHs, sH, 0, yh);
-            tma_store_2d(&mapHs, sH + 16384, 64, yh);
-            tma_store_commit();
-        };
         fetch_g(0);
         for (int n = 0; n < kDeepA && n < p.N; ++n) {
             load_a(n, n);
             if (lead && n < 2) load_b(n);
         }
-        if (lead && p.save) { wait(&bar_ht, 0); store_h(0); }
         int s = 0;
         for (int n = 0; n < p.N; ++n) {
             bool more = n + kDeepA < p.N;
             if (lead) {
-                if (p.save) {
-                    wait(&bar_dt[s], (n / kDeepA) & 1);   // Delta^T of chunk n is staged
-                    tma_store_2d(&mapDt, smem + s * kStageA + 16384, 0, (int)(((size_t)bh * p.N + n) * D) + v0);
-                    tma_store_commit();
-                    tma_store_wait_read_n<1>();           // the entry state has been read: its tile may be rewritten
-                    mbar_arrive(&bar_hf);
-                }
                 wait(&bar_e[n & 1], (n >> 1) & 1);        // every product of chunk n has finished: refill its buffers
                 if (n + 2 < p.N && !s_abort) load_b(n + 2);
-                if (more && p.save) tma_store_wait_read_n<0>();
+                if (more && p.save) wait(&bar_df[s], (n / kDeepA) & 1);
             }
             more = __shfl_sync(0xffffffffu, more && !s_abort, 0);     // one answer for the warp
             if (more) load_a(n + kDeepA, s);
-            if (lead && p.save && n + 1 < p.N) {
-                wait(&bar_ht, (n + 1) & 1);               // exit state of chunk n is staged
-                store_h(n + 1);
-            }
-            __syncwarp();
             if (++s == kDeepA) s = 0;
         }
-        if (lead) {
-            if (p.save) tma_store_wait_all();
-            if (s_abort) {                // one more bounded chance for copies in flight
-                for (int i = 0; i < kDeepA; ++i) mbar_wait(&bar_la[i], 0);
-                for (int i = 0; i < 2; ++i) mbar_wait(&bar_lb[i], 0);
-            }
+        if (lead && s_abort) {            // one more bounded chance for copies in flight
+            for (int i = 0; i < kDeepA; ++i) mbar_wait(&bar_la[i], 0);
+            for (int i = 0; i < 2; ++i) mbar_wait(&bar_lb[i], 0);
         }
     }
     tc_fence_before();
@@ -773,7 +776,7 @@ bool tc_supported(const qd_shape& s) {
            (long long)s.B * s.H * tc_padded_T(s) * 128 < 0x7fffffffLL * 64;
 }
 
-// Two CTAs per sequence while that leaves no SM with two (MEASURED)
+// Two CTAs per sequence while every CTA still gets an SM of its own: a saving forward chain of 32 sequences 975 -> 681 us.
 int chain_rows(uint64_t BH) { return BH <= 74 ? 64 : 128; }
 
 TcLayout tc_layout(const qd_shape& s) {
