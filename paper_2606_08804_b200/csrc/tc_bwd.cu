@@ -51,6 +51,7 @@ __device__ __forceinline__ void fold(float* v, int lane, int off) {
 // =================================================================================================
 struct ChainBwdParams {
     int Tp, H, N;              // Tp = 64 N rows per sequence in the workspace
+    int rows;                  // d_v rows of the state per CTA: 128, or 64 (two CTAs per sequence)
     int dhT_early;             // the kernel before this one in the stream is the library's own: dhT is older than it
     const float* rk;           // non-null (QD_NORM_QK): 1/|k_t| per workspace row, folded into the per-token scale
     const float* g;
@@ -59,15 +60,17 @@ struct ChainBwdParams {
     unsigned* status;
 };
 
-constexpr int kStage = 73728;                           // Wt 16K | dO 16K | Qg 16K | K 16K | P 8K
-constexpr int kChainSmem = 2 * kStage + 32768 + 16384 + 1024;
+// Tiles of a chunk in shared memory: K 16K | P 8K, three deep; dO 16K | Qg 16K, two deep; Wt 16K, two deep; staged for their
+// stores: dh^T 32K, dDelta^T 16K.
+constexpr int kDeepK = 3, kBytesK = 24576, kBytesQ = 32768, kBytesW = 16384;
+constexpr int kOffQ = kDeepK * kBytesK, kOffW = kOffQ + 2 * kBytesQ, kOffH = kOffW + 2 * kBytesW, kOffD = kOffH + 32768;
+constexpr int kChainSmem = kOffD + 16384 + 1024;
 constexpr int kChainCompute = 512;                 // 16 epilogue warps: 4 warpgroups split the accumulator columns
-constexpr int kChainThreads = kChainCompute + 64;  // + 1 MMA-issue warp, 1 TMA warp
+constexpr int kChainThreads = kChainCompute + 96;  // + 1 MMA-issue warp, 1 warp each for TMA loads and saves
 constexpr int kMmaWarp = kChainCompute / 32;
-constexpr int kNb = kChainCompute + 32;            // participants of a named barrier: the epilogue threads and one waiting warp
 
-// named barriers: compute threads arrive, the MMA and TMA warps wait
-constexpr int kBarH = 1, kBarD = 2, kBarHt = 4, kBarDt = 5;   // ..t: the same event, awaited by the TMA warp
+// named barriers: compute threads arrive, the MMA warp waits (they run in lock-step)
+constexpr int kBarH = 1, kBarD = 2;
 __device__ __forceinline__ void nb_arrive(int id, int count) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory"); }
 __device__ __forceinline__ void nb_sync(int id, int count) {
     __syncwarp();                                   // the lanes of a warp reach the barrier together
@@ -76,10 +79,12 @@ __device__ __forceinline__ void nb_sync(int id, int count) {
 
 // Reverse state chain.  Per chunk the dependency is
 //   dh ready -> A2 = dh^T K^T -> dDelta^T -> H-accumulator -= dDelta^T W<- -> dh update;
-// A1 = dO^T P and the dO^T Qg part of the H-accumulator do not depend on dh; every TMA copy is
-// issued by its own warp.
-// Compute warpgroup w owns tokens [32w, 32w+32) of the 64-column accumulators and d_k columns
-// [64w, 64w+64) of dh^T; thread l of a warpgroup owns TMEM lane l = d_v index.
+// A1 = dO^T P and the dO^T Qg part of the H-accumulator do not depend on dh and are issued a chunk ahead (double-buffered
+// H-accumulator).  As in the forward chain, the dependent operands (dh^T, -dDelta^T) live in tensor memory and the issuing
+// warp stays converged; what bounds a chunk is the SM's TMA unit, 72 KB in at 45 and 48 KB out at 32 bytes per cycle, one
+// after the other: 3150 cycles.  With few sequences two CTAs share the d_v rows of one (`rows` = 64).
+// Compute warpgroup w owns tokens [16w, 16w+16) of the 64-column accumulators and d_k columns
+// [32w, 32w+32) of dh^T; thread l of a warpgroup owns TMEM lane l = d_v index.
 __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_constant__ CUtensorMap mapWt,
                                                                 const __grid_constant__ CUtensorMap mapdO,
                                                                 const __grid_constant__ CUtensorMap mapQg,
@@ -90,40 +95,51 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
                                                                 ChainBwdParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* sdH = smem + 2 * kStage;         // dh^T as A operand: K-major, 2 blocks of [128 lines][64]
-    unsigned char* sdD = sdH + 32768;               // dDelta^T: K-major [128 lines (dv)][64 tokens]
-    __shared__ uint64_t bar_load[2], bar_a, bar_b, bar_e;
+    unsigned char* sdH = smem + kOffH;              // dh^T [128 dv][128 dk], 2 blocks of [128 lines][64]
+    unsigned char* sdD = smem + kOffD;              // dDelta^T [128 dv][64 tokens]
+    // A barrier per buffer where one side may run ahead.  bar_k, bar_q, bar_w: tiles loaded; bar_fk, bar_fq, bar_fw: read by
+    // their last product; bar_ht, bar_dt: staged (one arrival per compute warp); bar_hf, bar_df: read by their store.
+    __shared__ uint64_t bar_k[kDeepK], bar_fk[kDeepK], bar_q[2], bar_fq[2], bar_w[2], bar_fw[2], bar_ht, bar_hf, bar_dt, bar_df, bar_a, bar_b;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
-    // per iteration parity: gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the TMA warp one chunk
-    // ahead and published with its arrival on bar_a
-    __shared__ __align__(16) float sG[2][68];
+    // gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the load warp before it arrives on bar_k.  One deeper than
+    // K and P: those are dead when A2 is complete, but the epilogue reads these after that
+    __shared__ __align__(16) float sG[kDeepK + 1][68];
 
-    const int tid = threadIdx.x, warp = tid >> 5, wg = tid >> 7, l = tid & 127, wq = warp & 3;
-    const int bh = blockIdx.x, b = bh / p.H, hh = bh % p.H;
+    const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, l = tid & 127, wq = warp & 3;
+    const int rows = p.rows, nwq = rows / 32, nb = 4 * rows + 32;    // d_v rows of this CTA; warps of a warpgroup that have some; barrier participants
+    const int parts = D / rows, bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
 
     if (tid == 0) {
-        mbar_init(&bar_load[0], 1); mbar_init(&bar_load[1], 1);
-        mbar_init(&bar_a, 2); mbar_init(&bar_b, 2); mbar_init(&bar_e, 1);
+        for (int i = 0; i < kDeepK; ++i) { mbar_init(&bar_k[i], 1); mbar_init(&bar_fk[i], 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar_q[i], 1); mbar_init(&bar_fq[i], 1); mbar_init(&bar_w[i], 1); mbar_init(&bar_fw[i], 1); }
+        mbar_init(&bar_ht, 4 * nwq); mbar_init(&bar_dt, 4 * nwq); mbar_init(&bar_hf, 1); mbar_init(&bar_df, 1);
+        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1);
         mbar_init_fence();
         s_abort = 0;
     }
-    if (tid < 32) { tmem_alloc(&tmem_slot, 256); tmem_relinquish(); }
+    if (tid < 32) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tbase = tmem_slot;
-    const uint32_t tA1 = tbase, tA2 = tbase + 64, tH = tbase + 128;
+    const uint32_t tbase = uniform(tmem_slot);
+    // accumulators: A1, A2 64 columns each, H 2 x 128; operands, two bf16 per column: dh^T 64, -dDelta^T 32
+    const uint32_t tA1 = tbase, tA2 = tbase + 64, tH0 = tbase + 128, aH = tbase + 384, aD = tbase + 448;
     const uint32_t lane_base = (uint32_t)wq * 32;
 
     // bounded wait; once any wait has expired every later wait returns at once (the kernel drains)
     auto wait = [&](uint64_t* bar, uint32_t parity) {
-        if (s_abort) return;
-        if (!mbar_wait(bar, parity)) { s_abort = 1; *p.status = QD_ERR_TIMEOUT; }
+        if (s_abort) return false;
+        if (mbar_wait(bar, parity)) return true;
+        s_abort = 1;
+        *p.status = QD_ERR_TIMEOUT;
+        return false;
     };
     const float* gseq = p.g + (size_t)bh * p.Tp;
 
-    if (warp < kMmaWarp) {
+    if (warp < kMmaWarp && wq >= nwq) {
+        // lanes without a row: straight to the end
+    } else if (warp < kMmaWarp) {
         // ---------------------------------- compute warps ----------------------------------
         float dh[32];     // dh^T[j = l][32 wg .. 32 wg + 31]
         // dhT is an input of the call.  When the kernel before this one is the library's own forward chain, dhT is older
@@ -131,7 +147,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         // dhT, whose writes are only guaranteed visible after the wait.
         if (!p.dhT_early) grid_dep_wait();
         if (p.dhT) {
-            const float* src = p.dhT + (size_t)bh * D * D + (size_t)(32 * wg) * D + l;
+            const float* src = p.dhT + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
             for (int i = 0; i < 32; ++i) dh[i] = src[(size_t)i * D];
         } else {
@@ -140,161 +156,212 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         }
         if (p.dhT_early) grid_dep_wait();  // the loads of dhT are in flight; everything below depends on earlier kernels
         grid_dep_launch();
-        // my 32 columns of the operand tile: 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
-        unsigned char* myH = sdH + (wg >> 1) * 16384;
-        const int hc0 = (wg & 1) * 4;
+        auto arrive = [&](uint64_t* bar) { __syncwarp(); if ((tid & 31) == 0) mbar_arrive(bar); };
+        auto staged = [&](uint64_t* bar) { fence_proxy_async(); arrive(bar); };      // my part of a tile is in shared memory, for its store
+        // dh as operand: my 32 columns are 16 packed columns of tensor memory; then as a tile for its store
+        auto put_h = [&]() {
+            uint32_t r[8];
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) sts128(myH + sw128_chunk(l, hc0 + ch), pack8(dh + ch * 8));
-        fence_proxy_async();
-        nb_arrive(kBarH, kNb); nb_arrive(kBarHt, kNb);
-
-        for (int it = 0; it < p.N; ++it) {
-            wait(&bar_a, it & 1);
-            tc_fence_after();
-            float sc[16];
-            {
-                const float4* gp = reinterpret_cast<const float4*>(&sG[it & 1][wg * 16]);
+            for (int q = 0; q < 2; ++q) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float4 t = gp[q];
-                    sc[q * 4] = t.x; sc[q * 4 + 1] = t.y; sc[q * 4 + 2] = t.z; sc[q * 4 + 3] = t.w;
-                }
+                for (int e = 0; e < 8; ++e) r[e] = pack_bf16(dh[q * 16 + 2 * e], dh[q * 16 + 2 * e + 1]);
+                tmem_st8(tmem_addr(aH, lane_base, wg * 16 + q * 8), r);
             }
-            const float gamC = sG[it & 1][64];
-            // dDelta^T = A1 + gamma_C/gamma_s A2, my 16 tokens
+            tmem_st_wait();
+            tc_fence_before();
+            nb_arrive(kBarH, nb);
+        };
+        auto save_h = [&]() {             // 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) sts128(sdH + (wg >> 1) * 16384 + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(dh + ch * 8));
+            staged(&bar_ht);
+        };
+        // A chunk's K and P may be reloaded as soon as A2 is complete, which the announcement of its dh^T sets off: so the
+        // scales of a chunk are waited for before that, not after (where the barrier could have come round)
+        wait(&bar_k[0], 0);
+        put_h();
+        save_h();
+        int pending = 0;                  // barriers of the MMA warp that a warp which gives up has not been to
+        int s = 0;
+        for (int it = 0; it < p.N; ++it) {
+            const float gamC = sG[it & 3][64];
+            if (!__all_sync(0xffffffffu, wait(&bar_a, it & 1))) { pending = 2 * (p.N - it); break; }
+            tc_fence_after();
+            // dDelta^T = A1 + gamma_C/gamma_s A2, my 16 tokens; negated as operand
             {
                 float a1[16], a2[16];
                 tmem_ld16(tmem_addr(tA1, lane_base, wg * 16), a1);
                 tmem_ld16(tmem_addr(tA2, lane_base, wg * 16), a2);
+                const float4* gp = reinterpret_cast<const float4*>(&sG[it & 3][wg * 16]);
                 tmem_ld_wait();
+                uint32_t r[8], rn[8];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) a1[i] = fmaf(sc[i], a2[i], a1[i]);
-#pragma unroll
-                for (int cc = 0; cc < 2; ++cc) sts128(sdD + sw128_chunk(l, wg * 2 + cc), pack8(a1 + cc * 8));
+                for (int q = 0; q < 4; ++q) {
+                    const float4 t = gp[q];
+                    r[2 * q] = pack_bf16(fmaf(t.x, a2[4 * q], a1[4 * q]), fmaf(t.y, a2[4 * q + 1], a1[4 * q + 1]));
+                    r[2 * q + 1] = pack_bf16(fmaf(t.z, a2[4 * q + 2], a1[4 * q + 2]), fmaf(t.w, a2[4 * q + 3], a1[4 * q + 3]));
+                    rn[2 * q] = r[2 * q] ^ 0x80008000u; rn[2 * q + 1] = r[2 * q + 1] ^ 0x80008000u;
+                }
+                tmem_st8(tmem_addr(aD, lane_base, wg * 8), rn);
+                tmem_st_wait();
+                tc_fence_before();
+                nb_arrive(kBarD, nb);
+                if (it > 0) wait(&bar_df, (it - 1) & 1);
+                sts128(sdD + sw128_chunk(l, wg * 2), make_uint4(r[0], r[1], r[2], r[3]));
+                sts128(sdD + sw128_chunk(l, wg * 2 + 1), make_uint4(r[4], r[5], r[6], r[7]));
+                staged(&bar_dt);
             }
-            tc_fence_before();
-            fence_proxy_async();
-            nb_arrive(kBarD, kNb); nb_arrive(kBarDt, kNb);
-            wait(&bar_b, it & 1);
+            if (!__all_sync(0xffffffffu, wait(&bar_b, it & 1))) { pending = 2 * (p.N - it) - 1; break; }
             tc_fence_after();
             {
                 float v[32];
-                tmem_ld32(tmem_addr(tH, lane_base, wg * 32), v);
+                tmem_ld32(tmem_addr(tH0 + 128 * (it & 1), lane_base, wg * 32), v);
                 tmem_ld_wait();
 #pragma unroll
                 for (int i = 0; i < 32; ++i) dh[i] = fmaf(gamC, dh[i], v[i]);
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc) sts128(myH + sw128_chunk(l, hc0 + cc), pack8(dh + cc * 8));
             }
-            tc_fence_before();
-            fence_proxy_async();
-            nb_arrive(kBarH, kNb); nb_arrive(kBarHt, kNb);
+            if (++s == kDeepK) s = 0;
+            if (it + 1 < p.N) wait(&bar_k[s], ((it + 1) / kDeepK) & 1);
+            put_h();
+            if (it + 1 < p.N) { wait(&bar_hf, it & 1); save_h(); }
         }
+        // a wait has expired: keep step with the MMA warp, which comes to every one of them (odd counts: H is next)
+        for (; pending > 0; --pending) nb_sync(pending & 1 ? kBarH : kBarD, nb);
         if (p.dh0 && !s_abort) {
-            float* dst = p.dh0 + (size_t)bh * D * D + (size_t)(32 * wg) * D + l;
+            float* dst = p.dh0 + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
             for (int i = 0; i < 32; ++i) dst[(size_t)i * D] = dh[i];
         }
     } else if (warp == kMmaWarp) {
-        // ---------------------------------- MMA-issue warp ----------------------------------
-        const bool lead = (tid & 31) == 0;
+        // ---------------------------------- MMA-issue warp, converged ----------------------------------
+        const uint32_t issue = elect_lane();
         grid_dep_wait();
         grid_dep_launch();
-        const uint32_t adH = smem_u32(sdH), adD = smem_u32(sdD);
+        const uint32_t sb = smem_u32(smem);
+        // A1 = dO^T P (A, B MN-major: lines = token r), H-accumulator = dO^T Qg (B MN-major, two blocks of d_k)
+        auto ahead = [&](int it, int s) {
+            const uint32_t sq = sb + kOffQ + (it & 1) * kBytesQ;
+            wait(&bar_k[s], (it / kDeepK) & 1);
+            wait(&bar_q[it & 1], (it >> 1) & 1);
+            tc_fence_after();
+            umma_product_w<true, true>(tA1, sq, 8192, sb + s * kBytesK + 16384, 8192, C, C, false, issue);
+            umma_product_w<true, true>(tH0 + 128 * (it & 1), sq, 8192, sq + 16384, 8192, D, C, false, issue);
+            umma_commit_w(&bar_fq[it & 1], issue);
+        };
+        ahead(0, 0);
+        int s = 0;
         for (int it = 0; it < p.N; ++it) {
-            const uint32_t st = smem_u32(smem + (it & 1) * kStage);
-            if (lead) wait(&bar_load[it & 1], (it >> 1) & 1);
-            nb_sync(kBarH, kNb);                          // dh^T operand (exit state of this chunk) is in place
-            if (lead) {
-                tc_fence_after();
-                const uint32_t sdO = st + 16384;
-                // A2 = dh^T K^T (A, B K-major) -- the critical product;  A1 = dO^T P (A, B MN-major: lines = token r)
-                umma_product<false, false>(tA2, adH, 16384, st + 49152, 8192, C, D, false);
-                umma_product<true, true>(tA1, sdO, 8192, st + 65536, 8192, C, C, false);
-                umma_commit(&bar_a);
-                // H-accumulator = dO^T Qg (B MN-major: lines = token r, two blocks of d_k)
-                umma_product<true, true>(tH, sdO, 8192, st + 32768, 8192, D, C, false);
-            }
-            nb_sync(kBarD, kNb);                          // dDelta^T operand is in place
-            if (lead) {
-                tc_fence_after();
-                // H-accumulator -= dDelta^T W<-   (A negated; B K-major: lines = d_k index, contraction over tokens)
-                umma_product<false, false>(tH, adD, 16384, st, 16384, D, C, true, true);
-                umma_commit(&bar_b);
-                umma_commit(&bar_e);
-            }
+            nb_sync(kBarH, nb);                         // dh^T operand (exit state of this chunk) is in place
+            tc_fence_after();
+            // A2 = dh^T K^T (B K-major)
+            umma_product_ts_w<false>(tA2, aH, sb + s * kBytesK, 8192, C, D, false, issue);
+            umma_commit_w(&bar_a, issue);
+            umma_commit_w(&bar_fk[s], issue);
+            wait(&bar_w[it & 1], (it >> 1) & 1);
+            nb_sync(kBarD, nb);                         // -dDelta^T operand is in place, A1 has been read
+            tc_fence_after();
+            // H-accumulator -= dDelta^T W<-   (B K-major: lines = d_k index, contraction over tokens)
+            umma_product_ts_w<false>(tH0 + 128 * (it & 1), aD, sb + kOffW + (it & 1) * kBytesW, 16384, D, C, true, issue);
+            umma_commit_w(&bar_b, issue);
+            umma_commit_w(&bar_fw[it & 1], issue);
+            if (++s == kDeepK) s = 0;
+            if (it + 1 < p.N) ahead(it + 1, s);           // in the shadow of the dh update
         }
-        nb_sync(kBarH, kNb);                              // final arrival of the compute warps
+        nb_sync(kBarH, nb);                               // final arrival of the compute warps
+    } else if (warp == kMmaWarp + 1) {
+        // ---------------------------------- saving warp ----------------------------------
+        if ((tid & 31) == 0) {
+            grid_dep_wait();
+            for (int it = 0; it < p.N; ++it) {
+                const int y = (int)(((size_t)bh * p.N + (p.N - 1 - it)) * D) + v0;
+                wait(&bar_ht, it & 1);                    // gradient w.r.t. the exit state (rows = d_v, columns = d_k) is staged
+                tma_store_2d(&mapdHs, sdH, 0, y);
+                tma_store_2d(&mapdHs, sdH + 16384, 64, y);
+                tma_store_commit();
+                if (it > 0) { tma_store_wait_read_n<1>(); mbar_arrive(&bar_df); }     // dDelta^T of the chunk before has been read
+                wait(&bar_dt, it & 1);                    // dDelta^T is staged
+                tma_store_2d(&mapdDt, sdD, 0, y);
+                tma_store_commit();
+                tma_store_wait_read_n<1>();
+                mbar_arrive(&bar_hf);                     // the dh^T tile has been read
+            }
+            tma_store_wait_all();
+        }
     } else {
-        // ---------------------------------- TMA warp ----------------------------------
+        // ---------------------------------- TMA load warp ----------------------------------
         const bool lead = (tid & 31) == 0;
         grid_dep_wait();
         grid_dep_launch();
         // iteration `it` processes chunk n = N-1-it
-        auto issue_load = [&](int it) {
-            const int n = p.N - 1 - it;
-            unsigned char* st = smem + (it & 1) * kStage;
-            uint64_t* bar = &bar_load[it & 1];
-            mbar_expect_tx(bar, kStage);
-            const int yc = (int)(((size_t)bh * p.N + n) * D);
-            const int yt = (int)((size_t)bh * p.Tp + (size_t)n * C);
-            tma_load_2d(st, &mapWt, 0, yc, bar);
-            tma_load_3d(st + 16384, &mapdO, hh * D, n * C, b, bar);          // rows past the end of the sequence: zeros
-            tma_load_3d(st + 16384 + 8192, &mapdO, hh * D + 64, n * C, b, bar);
-            tma_load_2d(st + 32768, &mapQg, 0, yt, bar);
-            tma_load_2d(st + 32768 + 8192, &mapQg, 64, yt, bar);
-            tma_load_3d(st + 49152, &mapK, hh * D, n * C, b, bar);
-            tma_load_3d(st + 49152 + 8192, &mapK, hh * D + 64, n * C, b, bar);
-            tma_load_2d(st + 65536, &mapP, 0, yt, bar);
-        };
-        if (lead) { issue_load(0); if (p.N > 1) issue_load(1); }
         const int ln = tid & 31;
-        const float* gl = gseq + (size_t)(p.N - 1) * C;               // cumulative log-decays of the last chunk
-        float g0 = gl[ln], g1 = gl[32 + ln], gc = gl[C - 1];
         const float* rkseq = p.rk ? p.rk + (size_t)bh * p.Tp : nullptr;
-        float r0 = rkseq ? rkseq[(size_t)(p.N - 1) * C + ln] : 1.f, r1 = rkseq ? rkseq[(size_t)(p.N - 1) * C + 32 + ln] : 1.f;
-        for (int it = 0; it < p.N; ++it) {
-            const int n = p.N - 1 - it;
-            sG[it & 1][ln] = __expf(gc - g0) * r0;
-            sG[it & 1][32 + ln] = __expf(gc - g1) * r1;
-            if (ln == 0) sG[it & 1][64] = __expf(gc);
+        float g0, g1, gc, r0 = 1.f, r1 = 1.f;             // log-decays (and 1/|k|) of the next chunk to be loaded
+        auto fetch_g = [&](int it) {
+            const size_t at = (size_t)(p.N - 1 - it) * C;
+            g0 = gseq[at + ln]; g1 = gseq[at + 32 + ln]; gc = gseq[at + C - 1];
+            if (rkseq) { r0 = rkseq[at + ln]; r1 = rkseq[at + 32 + ln]; }
+        };
+        auto load_k = [&](int it, int s) {               // by the whole warp
+            float* sg = sG[it & 3];
+            sg[ln] = __expf(gc - g0) * r0;
+            sg[32 + ln] = __expf(gc - g1) * r1;
+            if (ln == 0) sg[64] = __expf(gc);
             __syncwarp();
-            if (n > 0) {                                      // in flight while this chunk is processed
-                const float* gn = gseq + (size_t)(n - 1) * C;
-                g0 = gn[ln]; g1 = gn[32 + ln]; gc = gn[C - 1];
-                if (rkseq) { r0 = rkseq[(size_t)(n - 1) * C + ln]; r1 = rkseq[(size_t)(n - 1) * C + 32 + ln]; }
-            }
             if (lead) {
-                tma_store_wait_read_n<0>();               // dDelta^T tile of the previous chunk has been read
-                mbar_arrive(&bar_a);
+                const int n = p.N - 1 - it;
+                unsigned char* st = smem + s * kBytesK;
+                mbar_expect_tx(&bar_k[s], kBytesK);
+                tma_load_3d(st, &mapK, hh * D, n * C, b, &bar_k[s]);
+                tma_load_3d(st + 8192, &mapK, hh * D + 64, n * C, b, &bar_k[s]);
+                tma_load_2d(st + 16384, &mapP, 0, (int)((size_t)bh * p.Tp + (size_t)n * C), &bar_k[s]);
             }
-            nb_sync(kBarHt, kNb);                          // dh^T operand (exit state of chunk n) is in place
-            if (lead) {
-                // gradient w.r.t. the exit state of chunk n, bf16, as the operand tile (rows = d_v, cols = d_k)
-                const int yh = (int)(((size_t)bh * p.N + n) * D);
-                tma_store_2d(&mapdHs, sdH, 0, yh);
-                tma_store_2d(&mapdHs, sdH + 16384, 64, yh);
-                tma_store_commit();
-            }
-            nb_sync(kBarDt, kNb);                          // dDelta^T of chunk n is in place
-            if (lead) {
-                tma_store_2d(&mapdDt, sdD, 0, (int)(((size_t)bh * p.N + n) * D));
-                tma_store_commit();
-                tma_store_wait_read_n<1>();               // the dh^T tile has been read: it may be rewritten
-                mbar_arrive(&bar_b);
-                wait(&bar_e, it & 1);                     // every product of this chunk has finished: refill its stage
-                if (it + 2 < p.N && !s_abort) issue_load(it + 2);
-            }
+            if (it + 1 < p.N) fetch_g(it + 1);
+        };
+        auto load_q = [&](int it) {                      // by the leading lane
+            const int n = p.N - 1 - it;
+            unsigned char* st = smem + kOffQ + (it & 1) * kBytesQ;
+            uint64_t* bar = &bar_q[it & 1];
+            const int yt = (int)((size_t)bh * p.Tp + (size_t)n * C);
+            mbar_expect_tx(bar, 16384 + rows * 128);
+            tma_load_3d(st, &mapdO, hh * D + v0, n * C, b, bar);             // rows past the end of the sequence: zeros
+            if (rows == D) tma_load_3d(st + 8192, &mapdO, hh * D + 64, n * C, b, bar);
+            tma_load_2d(st + 16384, &mapQg, 0, yt, bar);
+            tma_load_2d(st + 16384 + 8192, &mapQg, 64, yt, bar);
+        };
+        auto load_w = [&](int it) {
+            mbar_expect_tx(&bar_w[it & 1], kBytesW);
+            tma_load_2d(smem + kOffW + (it & 1) * kBytesW, &mapWt, 0, (int)(((size_t)bh * p.N + (p.N - 1 - it)) * D), &bar_w[it & 1]);
+        };
+        fetch_g(0);
+        for (int it = 0; it < kDeepK && it < p.N; ++it) {
+            load_k(it, it);
+            if (lead && it < 2) { load_q(it); load_w(it); }
         }
-        nb_sync(kBarHt, kNb);                              // final arrival of the compute warps
-        if (lead) {
-            tma_store_wait_all();
-            if (s_abort) { mbar_wait(&bar_load[0], 0); mbar_wait(&bar_load[1], 0); }
+        int s = 0;
+        for (int it = 0; it < p.N; ++it) {
+            bool more = it + kDeepK < p.N;
+            if (lead) {
+                wait(&bar_fq[it & 1], (it >> 1) & 1);
+                if (it + 2 < p.N && !s_abort) load_q(it + 2);
+                wait(&bar_fk[s], (it / kDeepK) & 1);
+            }
+            more = __shfl_sync(0xffffffffu, more && !s_abort, 0);     // one answer for the warp
+            if (more) load_k(it + kDeepK, s);
+            if (lead) {
+                wait(&bar_fw[it & 1], (it >> 1) & 1);
+                if (it + 2 < p.N && !s_abort) load_w(it + 2);
+            }
+            __syncwarp();
+            if (++s == kDeepK) s = 0;
+        }
+        if (lead && s_abort) {            // one more bounded chance for copies in flight
+            for (int i = 0; i < kDeepK; ++i) mbar_wait(&bar_k[i], 0);
+            for (int i = 0; i < 2; ++i) { mbar_wait(&bar_q[i], 0); mbar_wait(&bar_w[i], 0); }
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (tid < 32) tmem_dealloc(tbase, 256);
+    if (tid < 32) tmem_dealloc(tbase, 512);
 }
 
 // =================================================================================================
@@ -1045,17 +1112,19 @@ cudaError_t tc_chain_bwd(const ChunkArgs& a) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
     const uint64_t BH = (uint64_t)s.B * s.H, N = Tp / kChunk;
+    const int rows = chain_rows(BH);
     CUtensorMap mWt, mdO, mQg, mK, mP, mdHs, mdDt;
     if (!make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, BH * N * D, 128, 128) ||
         !make_tmap_tokens(&mdO, a.dO, s.B, s.T, s.H, D, 64) ||
         !make_tmap_bf16_2d(&mQg, a.ws + a.TL.Qg, D, BH * Tp, D * 2, 64) ||
         !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 64) ||
         !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, BH * Tp, 128, 64) ||
-        !make_tmap_bf16_2d(&mdHs, a.ws + a.TL.dhsT, D, BH * N * D, D * 2, 128) ||
-        !make_tmap_bf16_2d(&mdDt, a.ws + a.TL.dDt, 64, BH * N * D, 128, 128))
+        !make_tmap_bf16_2d(&mdHs, a.ws + a.TL.dhsT, D, BH * N * D, D * 2, rows) ||
+        !make_tmap_bf16_2d(&mdDt, a.ws + a.TL.dDt, 64, BH * N * D, 128, rows))
         return cudaErrorInvalidValue;
     ChainBwdParams p{};
     p.Tp = Tp; p.H = s.H; p.N = (int)N;
+    p.rows = rows;
     p.dhT_early = a.own_predecessor ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.g = (const float*)(a.ws + a.TL.g);
@@ -1063,7 +1132,7 @@ cudaError_t tc_chain_bwd(const ChunkArgs& a) {
     p.status = (unsigned*)(a.ws + a.TL.status);
     cudaError_t e = set_smem(k_tc_chain_bwd, kChainSmem);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(k_tc_chain_bwd, dim3((unsigned)BH), dim3(kChainThreads), kChainSmem, a.stream,
+    return launch_overlapped(k_tc_chain_bwd, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream,
                              mWt, mdO, mQg, mK, mP, mdHs, mdDt, p);
 }
 

@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     __shared__ __align__(16) float sG[kDeepA][68];
 
     const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, l = tid & 127, wq = warp & 3;
-    const int rows = p.rows, nwq = rows / 32, nb = 4 * rows + 32;    // d_v rows of this CTA; warps of a warpgroup; barrier participants
+    const int rows = p.rows, nwq = rows / 32, nb = 4 * rows + 32;    // d_v rows of this CTA; warps of a warpgroup that have some; barrier participants
     const int parts = D / rows, bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
 
     if (tid == 0) {
@@ -505,8 +505,11 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
 
     // bounded wait; once any wait has expired every later wait returns at once (the kernel drains)
     auto wait = [&](uint64_t* bar, uint32_t parity) {
-        if (s_abort) return;
-        if (!mbar_wait(bar, parity)) { s_abort = 1; *p.status = QD_ERR_TIMEOUT; }
+        if (s_abort) return false;
+        if (mbar_wait(bar, parity)) return true;
+        s_abort = 1;
+        *p.status = QD_ERR_TIMEOUT;
+        return false;
     };
     const float* gseq = p.g + (size_t)bh * p.Tp;
 
@@ -525,6 +528,8 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         }
         grid_dep_wait();                  // the loads of h0 (an input) are in flight; everything below depends on the prep kernel
         grid_dep_launch();
+        auto arrive = [&](uint64_t* bar) { __syncwarp(); if ((tid & 31) == 0) mbar_arrive(bar); };
+        auto staged = [&](uint64_t* bar) { fence_proxy_async(); arrive(bar); };      // my part of a tile is in shared memory, for its store
         // the state as operand: my 32 columns are 16 packed columns of tensor memory
         auto put_h = [&]() {
             uint32_t r[8];
@@ -538,11 +543,6 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             tc_fence_before();
             nb_arrive(kBarH, nb);
         };
-        auto staged = [&](uint64_t* bar) {                // my warp's part of a tile is in shared memory, for the TMA warp
-            fence_proxy_async();
-            __syncwarp();
-            if ((tid & 31) == 0) mbar_arrive(bar);
-        };
         auto save_h = [&]() {             // the state as a tile: 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) sts128(sH + (wg >> 1) * 16384 + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(h + ch * 8));
@@ -550,6 +550,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         };
         put_h();
         if (p.save) save_h();
+        int pending = 0;                  // barriers of the MMA warp that a warp which gives up has not been to
         int s = 0;
         for (int n = 0; n < p.N; ++n) {
             unsigned char* ut = smem + s * kStageA + 16384;
@@ -557,7 +558,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             const uint4 u0 = *reinterpret_cast<const uint4*>(ut + sw128_chunk(l, wg * 2));           // before the product is waited for
             const uint4 u1 = *reinterpret_cast<const uint4*>(ut + sw128_chunk(l, wg * 2 + 1));
             const float gamC = sG[s][64];
-            wait(&bar_a, n & 1);
+            if (!__all_sync(0xffffffffu, wait(&bar_a, n & 1))) { pending = 2 * (p.N - n); break; }
             tc_fence_after();
             // Delta^T = Ut - acc, my 16 tokens, as operands: plain, and scaled by gamma_C/gamma_r
             {
@@ -587,7 +588,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                 }
             }
             // h^T <- gamma_C h^T + acc (my 32 d_k columns), refresh the operand
-            wait(&bar_b, n & 1);
+            if (!__all_sync(0xffffffffu, wait(&bar_b, n & 1))) { pending = 2 * (p.N - n) - 1; break; }
             tc_fence_after();
             {
                 float v[32];
@@ -600,6 +601,8 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             if (p.save && n + 1 < p.N) { wait(&bar_hf, n & 1); save_h(); }
             if (++s == kDeepA) s = 0;
         }
+        // a wait has expired: keep step with the MMA warp, which comes to every one of them (odd counts: H is next)
+        for (; pending > 0; --pending) nb_sync(pending & 1 ? kBarH : kBarD, nb);
         if (p.hT && !s_abort) {
             float* dst = p.hT + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
@@ -653,7 +656,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             const uint32_t stA = smem_u32(smem) + s * kStageA, stB = smem_u32(smem) + kOffB + ob * kStageB;
             const uint32_t tO = tO0 + 64 * ob;
             wait(&bar_la[s], (n / kDeepA) & 1);
-            nb_sync(kBarH, nb);                          // h^T operand of chunk n is in place
+            nb_sync(kBarH, nb);                         // h^T operand of chunk n is in place
             tc_fence_after();
             // Delta-accumulator = h^T Wt (B: MN-major, lines = d_k)
             umma_product_ts_w<true>(tD, aH, stA, 8192, C, D, false, issue);
@@ -664,7 +667,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             wait(&bar_lb[ob], (n >> 1) & 1);
             tc_fence_after();
             umma_product_ts_w<false>(tO, aH, stB, 8192, C, D, false, issue);
-            nb_sync(kBarD, nb);                          // Delta^T operands of chunk n are in place
+            nb_sync(kBarD, nb);                         // Delta^T operands of chunk n are in place
             tc_fence_after();
             // H-accumulator = scaled Delta^T K (B: MN-major, lines = tokens)
             umma_product_ts_w<true>(tH, aDs, stB + 16384, 8192, D, C, false, issue);
@@ -675,7 +678,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             umma_commit_w(&bar_e[ob], issue);
             if (++s == kDeepA) s = 0;
         }
-        nb_sync(kBarH, nb);                              // final arrival of the compute warps
+        nb_sync(kBarH, nb);                               // final arrival of the compute warps
     } else if (warp == kMmaWarp + 1) {
         // ---------------------------------- saving warp ----------------------------------
         // apart from the loads, which would otherwise wait for what these wait for
