@@ -166,6 +166,30 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
                  : "r"(taddr)
                  : "memory");
 }
+// 16 lanes x 8 N columns in fragment layout: thread t of the warp holds, of every 8 columns, row t / 4 (v[0], v[1]) and row
+// t / 4 + 8 (v[2], v[3]), columns 2 (t % 4) and 2 (t % 4) + 1 -- the layout of ldmatrix / stmatrix, so that tiles are read and
+// written transposed or not in 16-byte rows instead of single elements
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float* v) {
+    uint32_t* r = reinterpret_cast<uint32_t*>(v);
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
+// Four 8 x 8 bf16 matrices; lane l passes the address of row l % 8 of matrix l / 8.  T: transposed, register m of thread t
+// holds elements (row 2 (t % 4) + {0, 1}, column t / 4) of matrix m instead of (row t / 4, columns 2 (t % 4) + {0, 1})
+template <bool T>
+__device__ __forceinline__ void ldsm4(const void* p, uint32_t* r) {
+    if (T) asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
+    else asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
+}
+template <bool T>
+__device__ __forceinline__ void stsm4(void* p, const uint32_t* r) {
+    if (T) asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};"
+                        ::"r"(smem_u32(p)), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+    else asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};"
+                      ::"r"(smem_u32(p)), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
 // store 8 consecutive 32-bit columns of this thread's lane
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"

@@ -379,30 +379,24 @@ struct ChunkBwdParams {
 // shared-memory map of k_tc_chunk_bwd (bytes from the 1024-aligned base)
 constexpr int oQ = 0, oK = 16384, oV = 32768, odO = 49152, oX = 65536, oMt = 81920, oP = 90112, oDt = 98304,
               odDt = 114688, oH = 131072, odH = 163840;                            // TMA-loaded tiles (X is built)
-constexpr int kBwdEarlyBytes = 2 * 16384 + 2 * 8192;
+constexpr int kBwdEarlyBytes = 4 * 16384 + 2 * 8192;
 // tiles built later reuse regions whose contents are dead by then
-constexpr int odPG = oV, odTb = oV + 8192, odW = 196608, oN = oH, odXK = oH + 8192, oPP = oH + 16384,
-              oAA = odH + 1024, oStDv = odDt, oStDk = oDt, oStDq = odDt;
+constexpr int odPG = oV, odTb = oV + 8192, odW = 196608, oN = oDt, odXK = oDt + 8192, oStDv = odDt, oStDk = oX, oStDq = odW;
 constexpr int kBwdSmem = 196608 + 16384 + 1024;      // + the dW<-^T tile, written while dO is still an operand
-constexpr int LDAA = C + 1;
 constexpr int kNWG = 4;                       // warpgroups; each owns 64/kNWG columns of every 64-column accumulator
 constexpr int kCW = C / kNWG, kG8 = kCW / 8;    // columns per warpgroup, groups of 8 columns
 constexpr int kBwdCompute = 128 * kNWG;                 // epilogue threads
-constexpr int kBwdThreads = kBwdCompute + 32;            // + one warp that issues every TMA copy and every MMA
+// + a warp that issues every MMA, a warp that issues every TMA copy, and two whose threads own a token each: coefficients
+// and the sums over rows and columns that become d beta, d lambda and d alpha
+constexpr int kBwdTail = kBwdCompute + 64, kBwdThreads = kBwdTail + C;
+constexpr int kBwdNb = kBwdCompute + 32;                 // participants of a named barrier: the epilogue threads and a waiting warp
 // named barriers of k_tc_chunk_bwd: 1 = the epilogue threads among themselves; the others are raised by the
-// epilogue threads (bar.arrive) when an operand tile is complete and awaited by the issuing warp (bar.sync)
-constexpr int kNbC = 1, kNbX = 2, kNbDW = 3, kNbDTb = 4, kNbN = 5, kNbDXK = 6, kNbOut = 7, kNbDV = 8, kNbScr = 9;
+// epilogue threads (bar.arrive) when a tile is complete and awaited by the MMA warp or the TMA warp (bar.sync); Sum: row
+// and column sums complete, awaited by the token threads; Tok: among themselves; End: everybody, the
+// TMA warp only arrives
+constexpr int kNbC = 1, kNbX = 2, kNbDW = 3, kNbDTb = 4, kNbN = 5, kNbDXK = 6, kNbOut = 7, kNbDV = 8, kNbDVt = 10, kNbSum = 11, kNbTok = 12, kNbEnd = 13;
+constexpr int kNbSumN = kBwdCompute + C;
 
-// Column sums across the 32 lanes of a warp for 8 columns: returns, in every lane, the warp-wide sum of
-// column col8_of_lane(lane) (four lanes hold each column).
-__device__ __forceinline__ float col_reduce8(float* v, int lane) {
-    fold<8>(v, lane, 16); fold<4>(v, lane, 8); fold<2>(v, lane, 4);
-    float x = v[0];
-    x += __shfl_xor_sync(0xffffffffu, x, 2);
-    x += __shfl_xor_sync(0xffffffffu, x, 1);
-    return x;
-}
-__device__ __forceinline__ int col8_of_lane(int lane) { return ((lane & 16) ? 4 : 0) + ((lane & 8) ? 2 : 0) + ((lane & 4) ? 1 : 0); }
 // 8 TMEM columns of this thread's lane (no wait)
 __device__ __forceinline__ void ld8(uint32_t taddr, float* v) { tmem_ld8(taddr, v); }
 
@@ -433,25 +427,28 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
                                                               ChunkBwdParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t bar_load, bar_late, bm_a, bm_b, bm_c, bm_2, bm_3, bm_4, bm_5;
+    // bar_load: V, dO, M^T, P, Delta^T, dDelta^T; bar_h: h^T, dh^T; bar_qk: Q, K; bar_st: the staged dk, dq have been read
+    __shared__ uint64_t bar_load, bar_h, bar_qk, bar_st, bm_a, bm_b, bm_c, bm_2, bm_3, bm_4, bm_5;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort, s_latch;
-    __shared__ float sbeta[C], slam[C], salpha[C], sg[C], sgam[C];
-    __shared__ float4 scf[C];         // per token: {gamma beta, gamma_C / gamma, gamma, lambda}, one load in the last epilogue
-    __shared__ float sred[3][4][C];   // per-warp column sums: [0] <(K-> dh)_r, Delta_r>, [1] d lambda, [2] rowsum(dQ1 o Q)
-    __shared__ float2 srn[C];          // NORM: {1/|k_t|, 1/|q_t|}
+    // by parity of the chunk, so that the token threads can publish a chunk ahead and take their sums a chunk late
+    __shared__ __align__(16) float sbeta_[2][C], sg_[2][C], slam_[2][C], sgam_[2][C];
+    __shared__ float4 scf_[2][C];     // per token: {gamma beta, gamma_C / gamma, gamma, lambda}, one load in the last epilogue
+    __shared__ float2 srn_[2][C];     // NORM: {1/|k_t|, 1/|q_t|}
+    __shared__ float sred_[2][2][4][C];   // per-warp column sums: [0] rowsum(dQ1 o Q) - <(K-> dh)_r, Delta_r>, [1] d lambda
+    __shared__ float swk_[2][kBwdCompute / 32];        // per-warp sums of <(K-> dh)_r, Delta_r>
+    __shared__ float scol[2][2][C];   // column sums of dP o P, dA o A by halves of the rows
     __shared__ __align__(16) float srow[6][kNWG][C];   // per-row partial sums over each warpgroup's columns: rPP, d beta, t2, rAA; [4], [5]: d beta and
                                          // rAA of the column groups that the upper lanes take
-    __shared__ float sdg[C], skd[C], swp[kBwdCompute / 32], scol[2][kBwdCompute / 64][C];
+    __shared__ float swp[kBwdCompute / 32], stot[2];
 
     const int tid = threadIdx.x, wg = tid >> 7, l = tid & 127, lane = tid & 31, wq = (tid >> 5) & 3;
     const int c0 = wg * kCW;                                      // my columns of a 64-column accumulator
 
     if (tid == 0) {
-        mbar_init(&bar_load, 1);
-        mbar_init(&bar_late, 1);
+        mbar_init(&bar_load, 1); mbar_init(&bar_h, 1); mbar_init(&bar_qk, 1); mbar_init(&bar_st, 1);
         mbar_init(&bm_a, 1); mbar_init(&bm_b, 1); mbar_init(&bm_c, 1); mbar_init(&bm_2, 1); mbar_init(&bm_3, 1); mbar_init(&bm_4, 1);
-        mbar_init(&bm_5, 2);              // the products' completion and "the dv staging tile has been read"
+        mbar_init(&bm_5, 1);
         mbar_init_fence();
         s_abort = 0;
         s_latch = 0;
@@ -466,9 +463,9 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     const uint32_t lane_base = (uint32_t)wq * 32;
     auto my = [&](uint32_t t) { return tmem_addr(t, lane_base, (uint32_t)c0); };
 
-    // The tiles of a chunk arrive in two groups.  "early": V, dO, M^T, P -- their regions are dead once the
-    // last products of the previous chunk have finished; "late": Q, Delta^T, dDelta^T, h^T, dh^T -- regions
-    // that the previous chunk uses up to its end (staging tiles of the stores, scratch of the reductions).
+    // The tiles of a chunk arrive in three groups, as their regions fall free in the chunk before: V, dO, M^T, P, Delta^T,
+    // dDelta^T after its last products; h^T, dh^T in the middle; Q, K, which the last epilogue
+    // reads, at its end.  The first products need only the first two.
     // Work item `ch` is chunk n_ of sequence bh_.  GROUPED = false: sequence-major numbering.  GROUPED = true: items are
     // numbered in groups of p.group sequences, chunk-major inside a group, so that at any time the CTAs of the grid work
     // on a few chunk indices of p.group sequences instead of on ~148 consecutive chunks of one long sequence.  Measured,
@@ -492,40 +489,35 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
         const int yt = (int)((size_t)bh_ * p.Tp + (size_t)n_ * C);
         mbar_expect_tx(&bar_load, kBwdEarlyBytes);
-        for (int blk = 0; blk < 2; ++blk) {       // token rows past the end of the sequence arrive as zeros
-            tma_load_3d(sm + oV + blk * 8192, &mapV, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
-            tma_load_3d(sm + odO + blk * 8192, &mapdO, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
-        }
+        const int yc = (int)(((size_t)bh_ * p.N + n_) * D);
+        tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_load);
         tma_load_2d(sm + oMt, &mapMt, 0, yt, &bar_load);
+        for (int blk = 0; blk < 2; ++blk)         // token rows past the end of the sequence arrive as zeros
+            tma_load_3d(sm + oV + blk * 8192, &mapV, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
+        tma_load_2d(sm + oDt, &mapDt, 0, yc, &bar_load);
+        for (int blk = 0; blk < 2; ++blk)
+            tma_load_3d(sm + odO + blk * 8192, &mapdO, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
         tma_load_2d(sm + oP, &mapP, 0, yt, &bar_load);
     };
-    // The late group goes in three batches as its regions fall free: part 0 = Q, K (after the last epilogue),
-    // part 1 = h^T, dh^T (after the last products and the column sums have read the scratch that aliases them), part 2 = Delta^T,
-    // dDelta^T (after the stores have read the staging tiles).  Only the last batch arrives on the barrier.
-    auto issue_late = [&](int ch, int part) {
+    auto issue_h = [&](int ch) {
         int n_, bh_; item(ch, n_, bh_);
-        const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
         const int yc = (int)(((size_t)bh_ * p.N + n_) * D);
-        if (part == 0) {
-            mbar_expect_tx_only(&bar_late, 2 * 16384);
-            for (int blk = 0; blk < 2; ++blk) {
-                tma_load_3d(sm + oQ + blk * 8192, &mapQ, hh_ * D + blk * 64, n_ * C, b_, &bar_late);
-                tma_load_3d(sm + oK + blk * 8192, &mapK, hh_ * D + blk * 64, n_ * C, b_, &bar_late);
-            }
-        } else if (part == 1) {
-            mbar_expect_tx_only(&bar_late, 2 * 32768);
-            for (int blk = 0; blk < 2; ++blk) {
-                tma_load_2d(sm + oH + blk * 16384, &mapHs, blk * 64, yc, &bar_late);
-                tma_load_2d(sm + odH + blk * 16384, &mapdHs, blk * 64, yc, &bar_late);
-            }
-        } else {
-            mbar_expect_tx(&bar_late, 2 * 16384);
-            tma_load_2d(sm + oDt, &mapDt, 0, yc, &bar_late);
-            tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_late);
+        mbar_expect_tx(&bar_h, 2 * 32768);
+        for (int blk = 0; blk < 2; ++blk) {
+            tma_load_2d(sm + oH + blk * 16384, &mapHs, blk * 64, yc, &bar_h);
+            tma_load_2d(sm + odH + blk * 16384, &mapdHs, blk * 64, yc, &bar_h);
         }
     };
-    // the late group of a chunk into L2 only, issued a chunk time before its load: the load, which can only be
-    // issued at the very end of the previous chunk and is waited for at once, then finds the tiles in L2
+    auto issue_qk = [&](int ch) {
+        int n_, bh_; item(ch, n_, bh_);
+        const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
+        mbar_expect_tx(&bar_qk, 2 * 16384);
+        for (int blk = 0; blk < 2; ++blk) {
+            tma_load_3d(sm + oQ + blk * 8192, &mapQ, hh_ * D + blk * 64, n_ * C, b_, &bar_qk);
+            tma_load_3d(sm + oK + blk * 8192, &mapK, hh_ * D + blk * 64, n_ * C, b_, &bar_qk);
+        }
+    };
+    // what is loaded late of a chunk into L2 only, a chunk time ahead
     auto prefetch_late = [&](int ch) {
         int n_, bh_; item(ch, n_, bh_);
         const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
@@ -538,24 +530,6 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         }
         tma_prefetch_2d(&mapDt, 0, yc);
         tma_prefetch_2d(&mapdDt, 0, yc);
-    };
-    // coefficients of token tid (< C) of a chunk, fetched one chunk ahead into registers
-    float cf_beta = 0.f, cf_lam = 0.f, cf_alpha = 1.f, cf_g = 0.f, cf_rq = 1.f, cf_rk = 1.f;
-    auto fetch_coef = [&](int ch) {
-        if (tid < C) {
-            int n_, bh_; item(ch, n_, bh_);
-            const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
-            const bool live = n_ * C + tid < p.T;             // tokens past the end of the sequence: beta = 0, alpha = 1
-            const size_t cr = ((size_t)b_ * p.T + (size_t)n_ * C + tid) * p.H + hh_;
-            cf_beta = live ? gate(__bfloat162float(p.beta[cr]), p.logits) : 0.f;
-            cf_lam = (live && p.lam) ? gate(__bfloat162float(p.lam[cr]), p.logits) : 0.f;
-            cf_alpha = (live && p.alpha) ? gate(__bfloat162float(p.alpha[cr]), p.logits) : 1.f;
-            cf_g = p.g[(size_t)bh_ * p.Tp + (size_t)n_ * C + tid];
-            if (NORM) {
-                cf_rq = p.rqk[(size_t)bh_ * p.Tp + (size_t)n_ * C + tid];
-                cf_rk = p.rqk[(size_t)p.BH * p.Tp + (size_t)bh_ * p.Tp + (size_t)n_ * C + tid];
-            }
-        }
     };
     // bounded wait; once any wait has expired every later wait returns at once and the kernel drains: all
     // threads still pass every barrier, results are garbage, the status word says so
@@ -571,148 +545,292 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     constexpr bool has_lam = HAS_LAM, has_alpha = HAS_ALPHA, want_dl = HAS_LAM, want_da = HAS_ALPHA;
     const uint32_t aXe = has_lam ? aX : aK;
 
-    if (tid >= kBwdCompute) {
-        // =============================== issuing warp: TMA copies and MMAs ===============================
+    if (tid >= kBwdCompute && tid < kBwdNb) {
+        // =============================== MMA warp ===============================
+        // Nothing here is done by one lane alone but the issue itself, so that descriptors and their increments stay in
+        // uniform registers (see umma_product_w); copies have a warp of their own.
+        const uint32_t issue = elect_lane();
+        const uint32_t tbu = uniform(tb);
+        const uint32_t T0 = tbu, T1 = tbu + 64, T2 = tbu + 128, T3 = tbu + 192, T4 = tbu + 256, T5 = tbu + 320, T6 = tbu + 384, T7 = tbu + 448;
+        grid_dep_wait();
+        __syncthreads();                                                 // the first chunk's coefficients have been published
+        for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
+            const uint32_t ph = it & 1;
+            if (__any_sync(0xffffffffu, s_latch)) break;
+            wait(&bar_load, ph);
+            wait(&bar_h, ph);
+            __syncwarp();
+            tc_fence_after();
+            umma_product_w<true, true>(T3, aH, 16384, adDt, 8192, C, D, false, issue, true);     // -h dDelta^T      [i][r] = dW<-^T
+            umma_commit_w(&bm_a, issue);
+            umma_product_w<false, false>(T6, adDt, 16384, aMt, 8192, C, C, false, issue);        // dDelta^T M       [j][s]
+            umma_product_w<false, true>(T2, aV, 8192, adDt, 8192, C, D, false, issue);           // V dDelta^T       [s][r]
+            umma_commit_w(&bm_b, issue);                // from here on no product reads V or dDelta^T any more
+            umma_product_w<false, true>(T1, adO - 8192, 8192, aDt, 8192, C, D, false, issue);    // dO Delta^T [r][s], rows r on lanes 64 + r
+            umma_product_w<true, false>(T4, aH, 16384, adO, 8192, C, D, false, issue);           // h dO^T           [i][r]
+            umma_commit_w(&bm_c, issue);                // from here on no product reads dO or h any more
+            wait(&bar_qk, ph);
+            nb_sync(kNbDW, kBwdNb);                                      // the dW<-^T tile is complete
+            nb_sync(kNbX, kBwdNb);                                       // X has been built
+            tc_fence_after();
+            // the product that the dependent chain waits for goes first, the two that are needed late after it
+            umma_product_w<false, true>(T3, aXe, 8192, adW, 8192, C, D, false, issue);           // X dW<-^T         [s][r]
+            umma_commit_w(&bm_2, issue);
+            umma_product_w<true, true>(T5, adH, 16384, aDt, 8192, C, D, false, issue);           // dh Delta^T       [i][s]
+            umma_product_w<false, false>(T0, aXe, 8192, aK, 8192, C, D, false, issue);           // X K^T            [r][i]
+            umma_product_w<false, false>(T7, aXe - 8192, 8192, aK, 8192, C, D, false, issue);    // once more, rows r on lanes 64 + r
+            nb_sync(kNbDV, kBwdNb);                                      // T6 has been read
+            tc_fence_after();
+            umma_product_w<false, false>(T6, adW, 16384, aMt, 8192, C, C, false, issue);         // dW<-^T M         [i][s]
+            nb_sync(kNbDTb, kBwdNb);
+            tc_fence_after();
+            umma_product_w<true, true>(T3, adTb, 8192, aMt, 8192, C, C, false, issue);           // N~ = dT diag(beta) M^T   [r][u]
+            umma_commit_w(&bm_3, issue);
+            nb_sync(kNbN, kBwdNb);
+            tc_fence_after();
+            umma_product_w<false, true>(T2, aMt, 8192, aN, 8192, C, C, false, issue, true);      // dA = -M^T N~     [r][s]
+            umma_product_w<false, true>(T3, aMt - 8192, 8192, aN, 8192, C, C, false, issue, true);   // once more, rows r on lanes 64 + r
+            umma_commit_w(&bm_4, issue);
+            nb_sync(kNbDXK, kBwdNb);
+            tc_fence_after();
+            umma_product_w<true, false>(T7, aK, 8192, adXK, 8192, C, C, false, issue);           // (dXK K)^T        [i][r]
+            umma_product_w<true, true>(T1, aXe, 8192, adXK, 8192, C, C, false, issue);           // (dXK^T X)^T      [i][s]
+            umma_product_w<true, true>(T1, aQ, 8192, adPG, 8192, C, C, true, issue);             // + (dPG^T Q)^T
+            umma_product_w<true, false>(T2, aK, 8192, adPG, 8192, C, C, false, issue);           // (dPG K)^T        [i][r]
+            umma_commit_w(&bm_5, issue);
+            nb_sync(kNbEnd, kBwdThreads);                                // every read of this chunk's tiles and accumulators is done
+        }
+    } else if (tid >= kBwdNb && tid < kBwdTail) {
+        // =============================== TMA warp ===============================
         const bool lead = lane == 0;
         if (lead && (int)blockIdx.x < p.total) {
             // first chunk: everything that the reverse chain (the kernel before this one) does not write is fetched
             // before waiting for it -- inputs, and tiles of kernels that had finished before the reverse chain began
             const int ch = blockIdx.x;
             int n_, bh_; item(ch, n_, bh_);
-            const int yc = (int)(((size_t)bh_ * p.N + n_) * D);
-            issue_early(ch);
-            issue_late(ch, 0);
-            mbar_expect_tx_only(&bar_late, 32768 + 16384);
-            for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + oH + blk * 16384, &mapHs, blk * 64, yc, &bar_late);
-            tma_load_2d(sm + oDt, &mapDt, 0, yc, &bar_late);
+            const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
+            const int yc = (int)(((size_t)bh_ * p.N + n_) * D), yt = (int)((size_t)bh_ * p.Tp + (size_t)n_ * C);
+            issue_qk(ch);
+            mbar_expect_tx_only(&bar_load, kBwdEarlyBytes - 16384);
+            for (int blk = 0; blk < 2; ++blk) {
+                tma_load_3d(sm + oV + blk * 8192, &mapV, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
+                tma_load_3d(sm + odO + blk * 8192, &mapdO, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
+            }
+            tma_load_2d(sm + oMt, &mapMt, 0, yt, &bar_load);
+            tma_load_2d(sm + oP, &mapP, 0, yt, &bar_load);
+            tma_load_2d(sm + oDt, &mapDt, 0, yc, &bar_load);
+            mbar_expect_tx_only(&bar_h, 32768);
+            for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + oH + blk * 16384, &mapHs, blk * 64, yc, &bar_h);
             grid_dep_wait();
-            mbar_expect_tx(&bar_late, 32768 + 16384);
-            for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + odH + blk * 16384, &mapdHs, blk * 64, yc, &bar_late);
-            tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_late);
+            mbar_expect_tx(&bar_h, 32768);
+            for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + odH + blk * 16384, &mapdHs, blk * 64, yc, &bar_h);
+            mbar_expect_tx(&bar_load, 16384);
+            tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_load);
+            mbar_arrive(&bar_st);                                        // nothing is staged yet
         }
         grid_dep_wait();
+        __syncthreads();                                                 // the first chunk's coefficients have been published
         for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
             int n, bh; item(ch_id, n, bh);
             const int b = bh / p.H, hh = bh % p.H;
             const int next_id = ch_id + gridDim.x;
+            const bool more = next_id < p.total;
             const uint32_t ph = it & 1;
-            if (s_latch) break;
-            if (lead) {
-                wait(&bar_load, ph);
-                wait(&bar_late, ph);
-                tc_fence_after();
-                umma_product<true, true>(T3, aH, 16384, adDt, 8192, C, D, false, true);     // -h dDelta^T      [i][r] = dW<-^T
-                umma_commit(&bm_a);
-                umma_product<false, false>(T6, adDt, 16384, aMt, 8192, C, C, false);        // dDelta^T M       [j][s]
-                umma_product<false, true>(T2, aV, 8192, adDt, 8192, C, D, false);           // V dDelta^T       [s][r]
-                umma_commit(&bm_b);                 // from here on no product reads V or dDelta^T any more
-                umma_product<false, true>(T1, adO - 8192, 8192, aDt, 8192, C, D, false);    // dO Delta^T [r][s], rows r on lanes 64 + r
-                umma_product<true, false>(T4, aH, 16384, adO, 8192, C, D, false);           // h dO^T           [i][r]
-                umma_commit(&bm_c);                 // from here on no product reads dO or h any more
-                if (next_id < p.total) prefetch_late(next_id);
-            }
-            nb_sync(kNbX, kBwdThreads);                                  // X has been built
-            nb_sync(kNbDW, kBwdThreads);                                 // the dW<-^T tile is complete
-            if (lead) {
-                tc_fence_after();
-                // the product that the dependent chain waits for goes first, the two that are needed late after it
-                umma_product<false, true>(T3, aXe, 8192, adW, 8192, C, D, false);           // X dW<-^T         [s][r]
-                umma_commit(&bm_2);
-                umma_product<true, true>(T5, adH, 16384, aDt, 8192, C, D, false);           // dh Delta^T       [i][s]
-                umma_product<false, false>(T0, aXe, 8192, aK, 8192, C, D, false);           // X K^T            [r][i]
-                umma_product<false, false>(T7, aXe - 8192, 8192, aK, 8192, C, D, false);    // once more, rows r on lanes 64 + r
-            }
-            nb_sync(kNbDV, kBwdThreads);                                 // the dv staging tile is complete, T6 has been read
+            if (__any_sync(0xffffffffu, s_latch)) break;
+            if (lead && more) prefetch_late(next_id);
+            nb_sync(kNbDVt, kBwdNb);                                     // the dv staging tile is complete
             if (lead) {
                 tma_store_3d(&mapdV, sm + oStDv, hh * D, n * C, b);          // rows past the end of the sequence are skipped
                 tma_store_3d(&mapdV, sm + oStDv + 8192, hh * D + 64, n * C, b);
                 tma_store_commit();
-                tc_fence_after();
-                umma_product<false, false>(T6, adW, 16384, aMt, 8192, C, C, false);         // dW<-^T M         [i][s]
             }
-            nb_sync(kNbDTb, kBwdThreads);
             if (lead) {
-                tc_fence_after();
-                umma_product<true, true>(T3, adTb, 8192, aMt, 8192, C, C, false);           // N~ = dT diag(beta) M^T   [r][u]
-                umma_commit(&bm_3);
-            }
-            nb_sync(kNbN, kBwdThreads);
-            if (lead) {
-                tc_fence_after();
-                umma_product<false, true>(T2, aMt, 8192, aN, 8192, C, C, false, true);      // dA = -M^T N~     [r][s]
-                umma_product<false, true>(T3, aMt - 8192, 8192, aN, 8192, C, C, false, true);   // once more, rows r on lanes 64 + r
-                umma_commit(&bm_4);
-            }
-            nb_sync(kNbDXK, kBwdThreads);
-            if (lead) {
-                tc_fence_after();
-                umma_product<true, false>(T7, aK, 8192, adXK, 8192, C, C, false);           // (dXK K)^T        [i][r]
-                umma_product<true, true>(T1, aXe, 8192, adXK, 8192, C, C, false);           // (dXK^T X)^T      [i][s]
-                umma_product<true, true>(T1, aQ, 8192, adPG, 8192, C, C, true);             // + (dPG^T Q)^T
-                umma_product<true, false>(T2, aK, 8192, adPG, 8192, C, C, false);           // (dPG K)^T        [i][r]
-                umma_commit(&bm_5);
-                tma_store_wait_read();                                   // the dv staging tile may be reused now
-                mbar_arrive(&bm_5);
-                wait(&bm_5, ph);
-                // V, dO, M^T, P of this chunk are dead: fetch the next chunk's
-                if (next_id < p.total && !s_abort) issue_early(next_id);
-            }
-            nb_sync(kNbScr, kBwdThreads);                                // the column sums have read the scratch over h^T, dh^T
-            if (lead) {
+                wait(&bm_3, ph);                                         // from here on nobody reads h or dh
+                if (more && !s_abort) issue_h(next_id);
+                wait(&bm_5, ph);                                         // nor anything but Q, K
+                tma_store_wait_read();                                   // dv's staging tile
                 fence_proxy_async();
-                if (next_id < p.total && !s_abort) issue_late(next_id, 1);
+                if (more && !s_abort) issue_early(next_id);
             }
-            nb_sync(kNbOut, kBwdThreads);                                // the dk and dq staging tiles are complete
+            nb_sync(kNbOut, kBwdNb);                                     // the dk and dq staging tiles are complete
+            // s_latch is read by everyone right after the barrier and not written again before the next one;
+            // an expiry that this read misses is seen one chunk later (waits return at once meanwhile)
+            if (lead) s_latch = s_abort;
+            __syncwarp();
+            nb_arrive(kNbEnd, kBwdThreads);                              // nobody waits for the copies to be issued
             if (lead) {
+                fence_proxy_async();                                     // the epilogue's reads of Q precede the copy into its region
+                if (more && !s_abort) issue_qk(next_id);
                 tma_store_3d(&mapdK, sm + oStDk, hh * D, n * C, b);
                 tma_store_3d(&mapdK, sm + oStDk + 8192, hh * D + 64, n * C, b);
                 tma_store_3d(&mapdQ, sm + oStDq, hh * D, n * C, b);
                 tma_store_3d(&mapdQ, sm + oStDq + 8192, hh * D + 64, n * C, b);
                 tma_store_commit();
-                fence_proxy_async();                                     // the epilogue's reads of Q precede the copy into its region
-                if (next_id < p.total && !s_abort) issue_late(next_id, 0);
             }
-            // s_latch is read by everyone right after the barrier and not written again before the next one;
-            // an expiry that this read misses is seen one chunk later (waits return at once meanwhile)
-            if (lead) s_latch = s_abort;
-            __syncthreads();                                             // every read of this chunk's tiles and scratch is done
             if (lead) {
                 tma_store_wait_read();                                   // the staging tiles have been read by the stores
-                fence_proxy_async();
-                if (next_id < p.total && !s_abort) issue_late(next_id, 2);
+                mbar_arrive(&bar_st);
             }
+            __syncwarp();
         }
         if (lead) tma_store_wait_all();
+    } else if (tid >= kBwdTail) {
+        // =============================== token threads ===============================
+        // thread r owns token r of the chunk
+        const int r = tid - kBwdTail;
+        bf16 zb = __float2bfloat16_rn(0.f), zl = zb, za = zb;                // as stored, converted a chunk later: nothing waits for the loads
+        float cg = 0.f, cgC = 0.f, rq = 1.f, rk = 1.f;
+        bool tok = false;
+        auto fetch = [&](int ch) {
+            int n_, bh_; item(ch, n_, bh_);
+            const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
+            tok = n_ * C + r < p.T;                               // tokens past the end of the sequence: beta = 0, alpha = 1
+            const size_t cr = ((size_t)b_ * p.T + (size_t)n_ * C + r) * p.H + hh_, wr = (size_t)bh_ * p.Tp + (size_t)n_ * C;
+            if (tok) {
+                zb = p.beta[cr];
+                if (p.lam) zl = p.lam[cr];
+                if (p.alpha) za = p.alpha[cr];
+            }
+            cg = p.g[wr + r];
+            cgC = p.g[wr + C - 1];
+            if (NORM) { rq = p.rqk[wr + r]; rk = p.rqk[(size_t)p.BH * p.Tp + wr + r]; }
+        };
+        float be = 0.f, lm = 0.f, al = 1.f;
+        auto publish = [&](int par) {
+            be = tok ? gate(__bfloat162float(zb), p.logits) : 0.f;
+            lm = (tok && p.lam) ? gate(__bfloat162float(zl), p.logits) : 0.f;
+            al = (tok && p.alpha) ? gate(__bfloat162float(za), p.logits) : 1.f;
+            const float gm = __expf(cg);
+            sbeta_[par][r] = be; slam_[par][r] = lm; sg_[par][r] = cg; sgam_[par][r] = gm;
+            scf_[par][r] = make_float4(gm * be, __expf(cgC - cg), gm, lm);
+            if (NORM) srn_[par][r] = make_float2(rk, rq);
+        };
+        if ((int)blockIdx.x < p.total) { fetch(blockIdx.x); publish(0); }
+        grid_dep_wait();                    // coefficients and log-decays are older than the reverse chain; the results below are not
+        __syncthreads();
+        // what the sums at the end of a chunk need of it, taken up a chunk later
+        float dg_pre = 0.f, dhh = 0.f, be0 = 0.f, lm0 = 0.f, al0 = 1.f, gmC = 1.f;
+        auto finish = [&](int ch, int par) {
+            int n, bh; item(ch, n, bh);
+            const size_t at = ((size_t)(bh / p.H) * p.T + (size_t)n * C + r) * p.H + bh % p.H;
+            const bool in = n * C + r < p.T;
+            float dg = dg_pre, dl = 0.f;
+#pragma unroll
+            for (int w4 = 0; w4 < 4; ++w4) {
+                if (want_da) dg += sred_[par][0][w4][r];
+                if (want_dl) dl += sred_[par][1][w4][r];
+            }
+            if (want_dl && in) p.dlam[at] = p.logits ? dl * lm0 * (1.f - lm0) : dl;
+            if (want_da) {
+                if (r == C - 1) {
+                    float kds = 0.f;
+#pragma unroll
+                    for (int w = 0; w < kBwdCompute / 32; ++w) kds += swk_[par][w];
+                    dg += gmC * dhh + kds;
+                }
+                // d log alpha_i = sum_{r >= i} dg_r (suffix sums over 64 tokens, two warps)
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const float t = __shfl_down_sync(0xffffffffu, dg, o);
+                    if (lane + o < 32) dg += t;
+                }
+                if (lane == 0) stot[r >> 5] = dg;
+                nb_sync(kNbTok, C);
+                if (r < 32) dg += stot[1];
+                // d log alpha -> d alpha = d log alpha / alpha;  with logit inputs d/dz log sigmoid(z) = 1 - sigmoid(z)
+                if (in && p.dalpha) p.dalpha[at] = p.logits ? dg * (1.f - al0) : dg / al0;
+            }
+        };
+        int prev = -1;
+        uint32_t last_ph = 0;
+        for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
+            int n, bh; item(ch_id, n, bh);
+            const int next_id = ch_id + gridDim.x;
+            const uint32_t ph = it & 1;
+            if (__any_sync(0xffffffffu, s_latch)) { prev = -1; break; }
+            if (prev >= 0) finish(prev, ph ^ 1);
+            const float gm = sgam_[ph][C - 1];
+            be0 = be; lm0 = lm; al0 = al; gmC = gm;
+            if (next_id < p.total) fetch(next_id);
+            nb_sync(kNbSum, kNbSumN);                                    // row sums and scratch are complete
+            float rPP = 0.f, t2 = 0.f, rAA = 0.f, dbt = 0.f;
+#pragma unroll
+            for (int w4 = 0; w4 < kNWG; ++w4) {
+                rPP += srow[0][w4][r]; dbt += srow[1][w4][r] + srow[4][w4][r]; t2 += srow[2][w4][r]; rAA += srow[3][w4][r] + srow[5][w4][r];
+            }
+            dg_pre = rPP + t2 + rAA;
+            if (want_da) dg_pre -= scol[0][0][r] + scol[0][1][r] + scol[1][0][r] + scol[1][1][r];
+            // with logit inputs: d/dz of sigmoid(z) is sigmoid(z) (1 - sigmoid(z))
+            if (n * C + r < p.T) p.dbeta[((size_t)(bh / p.H) * p.T + (size_t)n * C + r) * p.H + bh % p.H] = p.logits ? dbt * be0 * (1.f - be0) : dbt;
+            if (want_da) {
+                dhh = 0.f;
+#pragma unroll
+                for (int w = 0; w < kBwdCompute / 32; ++w) dhh += swp[w];
+            }
+            if (next_id < p.total) publish(ph ^ 1);
+            nb_sync(kNbEnd, kBwdThreads);                                // every read of this chunk's tiles and accumulators is done
+            prev = ch_id;
+            last_ph = ph;
+        }
+        if (prev >= 0) finish(prev, last_ph);
     } else {
     // ======================================== epilogue threads ========================================
     auto csync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(kNbC), "r"(kBwdCompute) : "memory"); };   // warps arrive converged
-    if ((int)blockIdx.x < p.total) fetch_coef(blockIdx.x);
-    grid_dep_wait();                    // coefficients and log-decays are older than the reverse chain; the results below are not
+    // fragment layout (tmem_ld_frag): columns c0 + 8 g + ft + {0, 1} of 16-row halves hf; the matching rows of a token-major
+    // tile, transposed: lane l addresses token c0 + 8 g + l % 8, rows 32 wq + 8 (l / 8) ..
+    const int ft = 2 * (lane & 3);
+    auto frag = [&](uint32_t t, int g, int hf) { return tmem_addr(t, lane_base + 16 * hf, (uint32_t)c0 + 8 * g); };
+    uint32_t foff[2];
+#pragma unroll
+    for (int g = 0; g < 2; ++g) foff[g] = (wq >> 1) * 8192 + sw128_chunk(c0 + 8 * g + (lane & 7), (wq & 1) * 4 + (lane >> 3));
+    grid_dep_wait();
+    __syncthreads();                    // the first chunk's coefficients have been published
 
     for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
-    int n, bh; item(ch_id, n, bh);
-    const int b = bh / p.H, hh = bh % p.H;
-    const size_t row0 = (size_t)b * p.T + (size_t)n * C;          // token row in the [B*T] view
-    const int live = min(C, p.T - n * C);                          // tokens of this chunk inside the sequence (may be <= 0)
-    const int next_id = ch_id + gridDim.x;
     const uint32_t ph = it & 1;
     if (s_latch) break;
-    if (tid < C) {
-        sbeta[tid] = cf_beta;
-        slam[tid] = cf_lam;
-        salpha[tid] = cf_alpha;
-        sg[tid] = cf_g;
-        sgam[tid] = __expf(cf_g);
-        if (NORM) srn[tid] = make_float2(cf_rk, cf_rq);
-    }
-    csync();
-    if (tid < C) {
-        const float ec = __expf(sg[C - 1] - sg[tid]);
-        scf[tid] = make_float4(sgam[tid] * sbeta[tid], ec, sgam[tid], slam[tid]);
-    }
+    const float *sbeta = sbeta_[ph], *slam = slam_[ph], *sg = sg_[ph], *sgam = sgam_[ph];
+    const float4* scf = scf_[ph];
+    const float2* srn = srn_[ph];
+    // ---- partial <dh,h>_F, under the first products ---------------------------------------------------
     wait(&bar_load, ph);
-    wait(&bar_late, ph);
-    // ---- X = K + lambda Q (the products that do not read X are already running); partial <dh,h>_F -------
+    wait(&bar_h, ph);
+    float dhh_part = 0.f;
+    if (want_da)
+#pragma unroll
+    for (int cc = 0; cc < 16 / kNWG; ++cc) {
+        const int ci = wg * (16 / kNWG) + cc;                // chunk 0..15 of line l
+        const uint32_t off = (ci >> 3) * 16384 + sw128_chunk(l, ci & 7);
+        float a[8], c8[8];
+        load8(sm + oH + off, a);
+        load8(sm + odH + off, c8);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) dhh_part = fmaf(a[e], c8[e], dhh_part);
+    }
+    if (want_da) {
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 16);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 8);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 4);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 2);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 1);
+        if (lane == 0) swp[tid >> 5] = dhh_part;
+    }
+    // ---- dW<-^T = -h dDelta^T: row i = l as an operand tile (region of its own: dO is still being read) -----
+    wait(&bar_st, ph);                                    // the staged dk, dq of the chunk before lie over X and this tile
+    wait(&bm_a, ph);
+    tc_fence_after();
+#pragma unroll
+    for (int g8 = 0; g8 < kG8; ++g8) {
+        float dw[8];
+        ld8(my(T3) + g8 * 8, dw);
+        tmem_ld_wait();
+        sts128(sm + odW + sw128_chunk(l, wg * kG8 + g8), pack8(dw));
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    nb_arrive(kNbDW, kBwdNb);
+    wait(&bar_qk, ph);
+    // ---- X = K + lambda Q (the products that do not read X are already running) ------------------------
     if (has_lam || NORM) {
         constexpr int kPer = 16 / (kBwdCompute / 64);     // 16-byte chunks of a row per thread
         const int r = tid & 63, part = tid >> 6;
@@ -739,367 +857,307 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         }
     }
     fence_proxy_async();
-    tc_fence_before();                                    // also orders the previous chunk's TMEM reads before the new products
-    nb_arrive(kNbX, kBwdThreads);
-    float dhh_part = 0.f;
-    if (want_da)
-#pragma unroll
-    for (int cc = 0; cc < 16 / kNWG; ++cc) {
-        const int ci = wg * (16 / kNWG) + cc;                // chunk 0..15 of line l
-        const uint32_t off = (ci >> 3) * 16384 + sw128_chunk(l, ci & 7);
-        float a[8], c8[8];
-        load8(sm + oH + off, a);
-        load8(sm + odH + off, c8);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) dhh_part = fmaf(a[e], c8[e], dhh_part);
-    }
-    // ---- dW<-^T = -h dDelta^T: row i = l as an operand tile (region of its own: dO is still being read) -----
-    wait(&bm_a, ph);
-    tc_fence_after();
-#pragma unroll
-    for (int g8 = 0; g8 < kG8; ++g8) {
-        float dw[8];
-        ld8(my(T3) + g8 * 8, dw);
-        tmem_ld_wait();
-        sts128(sm + odW + sw128_chunk(l, wg * kG8 + g8), pack8(dw));
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    nb_arrive(kNbDW, kBwdThreads);
+    nb_arrive(kNbX, kBwdNb);
     wait(&bm_b, ph);
     tc_fence_after();
-    float* sPP = reinterpret_cast<float*>(sm + oPP);
     {
-        // my columns in groups of 8 (one 16-byte bf16 chunk each)
-        unsigned char* stg = sm + oStDv + (l >> 6) * 8192;
+        // dV^T [j][s], scaled by beta_s, transposed into the staging tile
+        float dvv[2][2][4];                               // [8 columns][16 rows]
 #pragma unroll
-        for (int g8 = 0; g8 < kG8; ++g8) {
-            const int cb = c0 + g8 * 8;
-            float dvv[8];
-            ld8(my(T6) + g8 * 8, dvv);
-            tmem_ld_wait();
-            // dV^T row j = l scaled by beta_s into the staging tile
+        for (int g = 0; g < 2; ++g)
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                sts16(stg + sw128_off(cb + e, l & 63), __float2bfloat16_rn(sbeta[cb + e] * dvv[e]));
+            for (int hf = 0; hf < 2; ++hf) tmem_ld_frag(frag(T6, g, hf), dvv[g][hf]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const float2 be = *reinterpret_cast<const float2*>(sbeta + c0 + 8 * g + ft);
+            uint32_t r[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) r[m] = pack_bf16(be.x * dvv[g][m >> 1][2 * (m & 1)], be.y * dvv[g][m >> 1][2 * (m & 1) + 1]);
+            stsm4<true>(sm + oStDv + foff[g], r);
         }
     }
     fence_proxy_async();
     tc_fence_before();
-    nb_arrive(kNbDV, kBwdThreads);
-    float* sAA = reinterpret_cast<float*>(sm + oAA);
-    // One group of 8 columns of the dA epilogue for row r; tA = dA, tX = X K^T, both with row r on this thread's lane.
-    auto dA_group = [&](uint32_t tA, uint32_t tX, int g8, int r, float& db, float& rAA) {
-        const float gr = sg[r], br = sbeta[r];
-        const int cb = c0 + g8 * 8;
-        float da[8], xk[8];
-        ld8(my(tA) + g8 * 8, da);
-        ld8(my(tX) + g8 * 8, xk);
-        tmem_ld_wait();
+    nb_arrive(kNbDV, kBwdNb);
+    nb_arrive(kNbDVt, kBwdNb);
+    // The 64-row accumulators, in fragments: this thread's rows are rw + 16 hf + 8 j + lane / 4; of a sum over columns, the
+    // lane ends up with that of row `mine` (quad_sum), of a sum over a warp's 32 rows with that of a column (see below).
+    const int rw = 32 * (wq & 1), mine = rw + 8 * (lane & 3) + (lane >> 2);
+    auto quad_sum = [&](float* v) { fold<4>(v, lane, 2); fold<2>(v, lane, 1); return v[0]; };
+    auto row_of = [&](int m) { return rw + 8 * m + (lane >> 2); };                     // m = 2 hf + j
+    auto at = [&](int g) { return sw128_chunk(rw + 8 * (lane >> 3) + (lane & 7), wg * 2 + g); };   // of a [64 rows][64] tile
+    // 8 columns of the dA epilogue; tA = dA, tX = X K^T, both with their rows on this warp's lanes
+    auto dA_group = [&](uint32_t tA, uint32_t tX, int g, float& db, float& rAA) {
+        float da[2][4], xk[2][4], dbr[4] = {}, cA[2] = {};
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int s = cb + e;
-            const bool on = s < r;
-            const float gm = on ? (has_alpha ? __expf(gr - sg[s]) : 1.f) : 0.f;
-            const float d = on ? da[e] : 0.f;
-            const float dgx = d * gm * xk[e];
-            db += dgx;
-            const float aa = br * dgx;
-            rAA += aa;
-            if (want_da) sts32(&sAA[r * LDAA + s], aa);
-            da[e] = d * br * gm;                               // dXK
+        for (int hf = 0; hf < 2; ++hf) { tmem_ld_frag(frag(tA, g, hf), da[hf]); tmem_ld_frag(frag(tX, g, hf), xk[hf]); }
+        const int s = c0 + 8 * g + ft;
+        const float2 gs = *reinterpret_cast<const float2*>(sg + s);
+        tmem_ld_wait();
+        uint32_t o[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int r = row_of(m);
+            const float gr = sg[r], br = sbeta[r];
+            float out[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool on = s + e < r;
+                const float gm = on ? (has_alpha ? __expf(gr - (e ? gs.y : gs.x)) : 1.f) : 0.f;
+                const float d = on ? da[m >> 1][2 * (m & 1) + e] * gm : 0.f;
+                const float dgx = d * xk[m >> 1][2 * (m & 1) + e];
+                dbr[m] += dgx;
+                cA[e] = fmaf(br, dgx, cA[e]);
+                out[e] = br * d;                               // dXK
+            }
+            o[m] = pack_bf16(out[0], out[1]);
         }
-        sts128(sm + odXK + sw128_chunk(r, wg * kG8 + g8), pack8(da));
+        stsm4<false>(sm + odXK + at(g), o);
+        db = quad_sum(dbr);
+        rAA = sbeta[mine] * db;
+        if (want_da) {
+            fold<2>(cA, lane, 16);
+            float x = cA[0];
+            x += __shfl_xor_sync(0xffffffffu, x, 8);
+            x += __shfl_xor_sync(0xffffffffu, x, 4);
+            if (!(lane & 12)) scol[1][wq & 1][s + (lane >> 4)] = x;
+        }
     };
     static_assert(kG8 == 2, "the dA epilogue gives one column group to each half of a warpgroup");
-    // From here to the column sums the two halves of every warpgroup go separate ways.  Lanes 64..127 (whose rows
+    // From here to the last products the two halves of every warpgroup go separate ways.  Lanes 64..127 (whose rows
     // of the 64-row accumulators are padding) take dP, whose product was issued with its rows on their lanes; lanes
     // 0..63 walk the dependent chain dT -> N~ -> dA -> dXK.  Both raise every barrier of the chain exactly once.
-    if (l >= C) {
-        nb_arrive(kNbDTb, kBwdThreads);
-        nb_arrive(kNbN, kBwdThreads);
-        wait(&bm_c, ph);                  // dP's product; its scratch lies over h^T, which that group has read
+    if (wq >= 2) {
+        nb_arrive(kNbDTb, kBwdNb);
+        nb_arrive(kNbN, kBwdNb);
+        wait(&bm_c, ph);                  // dP's product
+        wait(&bm_2, ph);                  // of the tile over V that is written here nobody reads any more
         tc_fence_after();
-        // dP row r = l - 64: causal mask, dP o P (row and column sums), dP o Gamma as an operand tile
-        const int r = l - C;
-        const float gr = sg[r];
-        float rPP = 0.f;
+        // dP: causal mask, dP o P (row and column sums), dP o Gamma as an operand tile
+        float v[2][2][4], rPP[4] = {}, cP[4];
+        uint32_t pr[2][4];
 #pragma unroll
-        for (int g8 = 0; g8 < kG8; ++g8) {
-            const int cb = c0 + g8 * 8, ck = wg * kG8 + g8;
-            float v[8], pv[8], pg[8];
-            ld8(my(T1) + g8 * 8, v);
-            tmem_ld_wait();
-            load8(sm + oP + sw128_chunk(r, ck), pv);
+        for (int g = 0; g < 2; ++g) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int s = cb + e;
-                const float dp = (s <= r) ? v[e] : 0.f;
-                const float pp = dp * pv[e];
-                rPP += pp;
-                if (want_da) sts32(&sPP[r * C + ((s + r) & (C - 1))], pp);   // rotated rows: 64 x 64 floats fit the h^T half exactly
-                pg[e] = (s <= r) ? (has_alpha ? dp * __expf(gr - sg[s]) : dp) : 0.f;
-            }
-            sts128(sm + odPG + sw128_chunk(r, ck), pack8(pg));
+            for (int hf = 0; hf < 2; ++hf) tmem_ld_frag(frag(T1, g, hf), v[g][hf]);
+            ldsm4<false>(sm + oP + at(g), pr[g]);
         }
-        srow[0][wg][r] = rPP;
+        tmem_ld_wait();
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const int s = c0 + 8 * g + ft;
+            const float2 gs = *reinterpret_cast<const float2*>(sg + s);
+            float c[2] = {};
+            uint32_t o[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int r = row_of(m);
+                const float gr = sg[r];
+                float pg[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const bool on = s + e <= r;
+                    const float dp = on ? v[g][m >> 1][2 * (m & 1) + e] : 0.f;
+                    const float pp = dp * __uint_as_float(e ? pr[g][m] & 0xffff0000u : pr[g][m] << 16);
+                    rPP[m] += pp;
+                    c[e] += pp;
+                    pg[e] = on ? (has_alpha ? dp * __expf(gr - (e ? gs.y : gs.x)) : dp) : 0.f;
+                }
+                o[m] = pack_bf16(pg[0], pg[1]);
+            }
+            stsm4<false>(sm + odPG + at(g), o);
+            cP[2 * g] = c[0]; cP[2 * g + 1] = c[1];
+        }
+        srow[0][wg][mine] = quad_sum(rPP);
+        if (want_da) {
+            fold<4>(cP, lane, 16); fold<2>(cP, lane, 8);
+            const float x = cP[0] + __shfl_xor_sync(0xffffffffu, cP[0], 4);
+            if (!(lane & 4)) scol[0][wq & 1][c0 + ((lane & 16) ? 8 : 0) + ft + ((lane & 8) ? 1 : 0)] = x;
+        }
         // second column group of the dA epilogue, from the copies of dA and X K^T whose rows lie on these lanes
         wait(&bm_4, ph);
         tc_fence_after();
-        float db = 0.f, rAA = 0.f;
-        dA_group(T3, T7, 1, r, db, rAA);
-        srow[4][wg][r] = db;
-        srow[5][wg][r] = rAA;
+        float db, rAA;
+        dA_group(T3, T7, 1, db, rAA);
+        srow[4][wg][mine] = db;
+        srow[5][wg][mine] = rAA;
     } else {
-    wait(&bm_2, ph);
-    tc_fence_after();
-    if (l < C) {
-        // dT^T row s = l, my 32 values of r;  M[r][s] = line s of Mt
-        const int s = l;
-        const float gs = sgam[s], bs = sbeta[s];
-        float mb = 0.f, db = 0.f;
+        wait(&bm_2, ph);
+        tc_fence_after();
+        {
+            // dT^T row s, my columns r;  M[r][s] = line s of Mt
+            float a[2][2][4], bq[2][2][4], db[4] = {}, mb[4] = {};
+            uint32_t mr[2][4];
 #pragma unroll
-        for (int g8 = 0; g8 < kG8; ++g8) {
-            const int ck = wg * kG8 + g8;
-            float a[8], bq[8], m[8], tb8[8];
-            ld8(my(T2) + g8 * 8, a);
-            ld8(my(T3) + g8 * 8, bq);
-            tmem_ld_wait();
-            load8(sm + oMt + sw128_chunk(s, ck), m);
+            for (int g = 0; g < 2; ++g) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float dt = fmaf(gs, bq[e], a[e]);
-                db = fmaf(dt, m[e], db);
-                mb = fmaf(m[e], bq[e], mb);
-                tb8[e] = bs * dt;
+                for (int hf = 0; hf < 2; ++hf) { tmem_ld_frag(frag(T2, g, hf), a[g][hf]); tmem_ld_frag(frag(T3, g, hf), bq[g][hf]); }
+                ldsm4<false>(sm + oMt + at(g), mr[g]);
             }
-            sts128(sm + odTb + sw128_chunk(s, ck), pack8(tb8));
-        }
-        srow[1][wg][s] = db;
-        srow[2][wg][s] = gs * bs * mb;
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    nb_arrive(kNbDTb, kBwdThreads);
-    // ---- N~ = dT diag(beta) M^T, copied out as an operand tile --------------------------------------
-    wait(&bm_3, ph);
-    tc_fence_after();
-    if (l < C) {
-#pragma unroll
-        for (int g8 = 0; g8 < kG8; ++g8) {
-            float v[8];
-            ld8(my(T3) + g8 * 8, v);
             tmem_ld_wait();
-            sts128(sm + oN + sw128_chunk(l, wg * kG8 + g8), pack8(v));
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                uint32_t o[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float gs = sgam[row_of(m)], bs = sbeta[row_of(m)];
+                    float tb8[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float x = bq[g][m >> 1][2 * (m & 1) + e], mv = __uint_as_float(e ? mr[g][m] & 0xffff0000u : mr[g][m] << 16);
+                        const float dt = fmaf(gs, x, a[g][m >> 1][2 * (m & 1) + e]);
+                        db[m] = fmaf(dt, mv, db[m]);
+                        mb[m] = fmaf(mv, x, mb[m]);
+                        tb8[e] = bs * dt;
+                    }
+                    o[m] = pack_bf16(tb8[0], tb8[1]);
+                }
+                stsm4<false>(sm + odTb + at(g), o);
+            }
+            fence_proxy_async();
+            tc_fence_before();
+            nb_arrive(kNbDTb, kBwdNb);
+            srow[1][wg][mine] = quad_sum(db);
+            srow[2][wg][mine] = sgam[mine] * sbeta[mine] * quad_sum(mb);
         }
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    nb_arrive(kNbN, kBwdThreads);
-    // ---- dA = -M^T N~ -----------------------------------------------------------------------------
-    wait(&bm_4, ph);
-    tc_fence_after();
-    {
-        const int r = l;
-        float rAA = 0.f, db = 0.f;
-        dA_group(T2, T0, 0, r, db, rAA);
-        srow[1][wg][r] += db;
-        srow[3][wg][r] = rAA;
-    }
+        // ---- N~ = dT diag(beta) M^T, copied out as an operand tile --------------------------------------
+        wait(&bm_3, ph);
+        tc_fence_after();
+        {
+            float v[2][2][4];
+#pragma unroll
+            for (int g = 0; g < 2; ++g)
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) tmem_ld_frag(frag(T3, g, hf), v[g][hf]);
+            tmem_ld_wait();
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                uint32_t o[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) o[m] = pack_bf16(v[g][m >> 1][2 * (m & 1)], v[g][m >> 1][2 * (m & 1) + 1]);
+                stsm4<false>(sm + oN + at(g), o);
+            }
+        }
+        fence_proxy_async();
+        tc_fence_before();
+        nb_arrive(kNbN, kBwdNb);
+        // ---- dA = -M^T N~ -----------------------------------------------------------------------------
+        wait(&bm_4, ph);
+        tc_fence_after();
+        float db, rAA;
+        dA_group(T2, T0, 0, db, rAA);
+        srow[1][wg][mine] += db;
+        srow[3][wg][mine] = rAA;
     }  // lanes 0..63: the dependent chain
     fence_proxy_async();
     tc_fence_before();
-    nb_arrive(kNbDXK, kBwdThreads);
-    // ---- the last products; meanwhile the column sums of dA o A and dP o P (kBwdCompute/64 threads per column)
-    // and the coefficients of the next chunk -------------------------------------------------------------------
-    csync();
-    if (want_da) {
-        const float* sAAc = reinterpret_cast<const float*>(sm + oAA);
-        const int r = tid & 63, part = tid >> 6;
-        float cA = 0.f, cP = 0.f;
-        constexpr int kRows = C / (kBwdCompute / 64);
-#pragma unroll
-        for (int k = 0; k < kRows; ++k) {
-            cA += sAAc[(part * kRows + k) * LDAA + r];
-            cP += sPP[(part * kRows + k) * C + ((r + part * kRows + k) & (C - 1))];
-        }
-        scol[0][part][r] = cA;
-        scol[1][part][r] = cP;
-    }
-    nb_arrive(kNbScr, kBwdThreads);      // the scratch tiles over h^T and dh^T are dead from here on
-    if (want_da) {
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 16);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 8);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 4);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 2);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 1);
-        if (lane == 0) swp[tid >> 5] = dhh_part;
-    }
-    csync();
-    // everything of the decay gradient that does not wait for the last epilogue
-    float dg_pre = 0.f;
-    if (tid < C) {
-        const int r = tid;
-        float cAA = 0.f, cPP = 0.f;
-#pragma unroll
-        for (int w4 = 0; w4 < kBwdCompute / 64; ++w4) { cAA += scol[0][w4][r]; cPP += scol[1][w4][r]; }
-        float rPP = 0.f, t2 = 0.f, rAA = 0.f, dbt = 0.f;
-#pragma unroll
-        for (int w4 = 0; w4 < kNWG; ++w4) {
-            rPP += srow[0][w4][r]; dbt += srow[1][w4][r] + srow[4][w4][r]; t2 += srow[2][w4][r]; rAA += srow[3][w4][r] + srow[5][w4][r];
-        }
-        dg_pre = rPP - cPP + t2 + rAA - cAA;
-        // with logit inputs: d/dz of sigmoid(z) is sigmoid(z) (1 - sigmoid(z))
-        if (r < live) p.dbeta[(row0 + r) * p.H + hh] = p.logits ? dbt * sbeta[r] * (1.f - sbeta[r]) : dbt;
-    }
-    if (next_id < p.total) fetch_coef(next_id);
+    nb_arrive(kNbDXK, kBwdNb);
+    nb_arrive(kNbSum, kNbSumN);
     wait(&bm_5, ph);
     tc_fence_after();
-    // The last epilogue: thread = d_k index i, its 16 tokens in groups of 8: dk and dq, transposed, into their staging
-    // tiles, and the column sums (over i, i.e. across the lanes) that d lambda and the decay gradient need.
+    // The last epilogue: dk and dq, transposed, into their staging tiles, and the column sums (over the d_k index i, i.e.
+    // down the fragments and across eight lanes) that d lambda and the decay gradient need.
     {
-        const int i = l;
-        unsigned char* stk = sm + oStDk + (i >> 6) * 8192;
-        unsigned char* stq = sm + oStDq + (i >> 6) * 8192;
-        const unsigned char* qcol = sm + oQ + (i >> 6) * 8192;
-        const unsigned char* kcol = sm + oK + (i >> 6) * 8192;
+        float ksum = 0.f, t1[4], dl[4];                   // [2 (8 columns) + column of the pair]
 #pragma unroll
-        for (int g8 = 0; g8 < kG8; ++g8) {
-            const int cb = c0 + g8 * 8;
-            float dx[8], v[8], w[8], u[8], z[8], y[8];
-            ld8(my(T6) + g8 * 8, dx);
-            ld8(my(T7) + g8 * 8, v);
-            ld8(my(T1) + g8 * 8, w);
-            ld8(my(T5) + g8 * 8, u);
-            ld8(my(T4) + g8 * 8, z);
-            ld8(my(T2) + g8 * 8, y);
+        for (int g = 0; g < 2; ++g) {
+            const int t = c0 + 8 * g + ft;
+            float dx[2][4], v[2][4], w[2][4], u[2][4], z[2][4], y[2][4];
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                tmem_ld_frag(frag(T6, g, hf), dx[hf]); tmem_ld_frag(frag(T7, g, hf), v[hf]); tmem_ld_frag(frag(T1, g, hf), w[hf]);
+                tmem_ld_frag(frag(T5, g, hf), u[hf]); tmem_ld_frag(frag(T4, g, hf), z[hf]); tmem_ld_frag(frag(T2, g, hf), y[hf]);
+            }
+            uint32_t qr[4], kr[4], dkr[4], dqr[4];
+            ldsm4<true>(sm + oQ + foff[g], qr);
+            ldsm4<true>(sm + oK + foff[g], kr);
+            const float4 cf[2] = {scf[t], scf[t + 1]};
             tmem_ld_wait();
+            float s1[2] = {}, s2[2] = {};
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int t = cb + e;
-                const float4 cf = scf[t];
-                const float dxe = fmaf(cf.x, dx[e], v[e]);                                  // dX^T[i][t]
-                const float kh = cf.y * u[e];                                               // (K-> ^T applied to dh Delta^T)[i][t]
-                sts16(stk + sw128_off(t, i & 63), __float2bfloat16_rn(w[e] + kh + dxe));    // d k  (d k^ with NORM)
-                // <(K-> dh)_t, Delta_t> = gamma_C/gamma_t sum_i K[t][i] (dh Delta^T)[i][t], all of it in fp32
-                u[e] = kh * __bfloat162float(*reinterpret_cast<const bf16*>(kcol + sw128_off(t, i & 63)));
-                const float q1 = cf.z * z[e];
-                sts16(stq + sw128_off(t, i & 63), __float2bfloat16_rn(q1 + y[e] + cf.w * dxe));   // d q  (d q^ with NORM)
-                const float qv = __bfloat162float(*reinterpret_cast<const bf16*>(qcol + sw128_off(t, i & 63)));
-                z[e] = q1 * qv;
-                dx[e] = dxe * qv;
-            }
-            // column sums over the d_k index (across the lanes): d lambda, and the two that only the decay gradient needs
-            if (want_dl) {
-                const float dls = col_reduce8(dx, lane);
-                if ((lane & 3) == 0) sred[1][wq][cb + col8_of_lane(lane)] = dls;
-            }
-            if (want_da) {
-                const float t1s = col_reduce8(z, lane), kds = col_reduce8(u, lane);
-                if ((lane & 3) == 0) {
-                    const int col = cb + col8_of_lane(lane);
-                    sred[0][wq][col] = kds;
-                    sred[2][wq][col] = t1s;
+            for (int m = 0; m < 4; ++m) {
+                float dkv[2], dqv[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int hf = m >> 1, x = 2 * (m & 1) + e;
+                    const float qv = __uint_as_float(e ? qr[m] & 0xffff0000u : qr[m] << 16), kv = __uint_as_float(e ? kr[m] & 0xffff0000u : kr[m] << 16);
+                    const float dxe = fmaf(cf[e].x, dx[hf][x], v[hf][x]);                       // dX^T[i][t]
+                    const float kh = cf[e].y * u[hf][x];                                        // (K-> ^T applied to dh Delta^T)[i][t]
+                    const float q1 = cf[e].z * z[hf][x];
+                    dkv[e] = w[hf][x] + kh + dxe;                                               // d k  (d k^ with NORM)
+                    dqv[e] = q1 + y[hf][x] + cf[e].w * dxe;                                     // d q  (d q^ with NORM)
+                    // <(K-> dh)_t, Delta_t> = gamma_C/gamma_t sum_i K[t][i] (dh Delta^T)[i][t], all of it in fp32
+                    const float kd = kh * kv;
+                    ksum += kd;
+                    s1[e] += fmaf(q1, qv, -kd);
+                    s2[e] = fmaf(dxe, qv, s2[e]);
                 }
+                dkr[m] = pack_bf16(dkv[0], dkv[1]);
+                dqr[m] = pack_bf16(dqv[0], dqv[1]);
             }
+            stsm4<true>(sm + oStDk + foff[g], dkr);
+            stsm4<true>(sm + oStDq + foff[g], dqr);
+            t1[2 * g] = s1[0]; t1[2 * g + 1] = s1[1];
+            dl[2 * g] = s2[0]; dl[2 * g + 1] = s2[1];
+        }
+        // lane: column 8 (bit 4) + 2 (lane % 4) + (bit 3)
+        const int col = c0 + ((lane & 16) ? 8 : 0) + ft + ((lane & 8) ? 1 : 0);
+        if (want_dl) {
+            fold<4>(dl, lane, 16); fold<2>(dl, lane, 8);
+            const float x = dl[0] + __shfl_xor_sync(0xffffffffu, dl[0], 4);
+            if (!(lane & 4)) sred_[ph][1][wq][col] = x;
+        }
+        if (want_da) {
+            fold<4>(t1, lane, 16); fold<2>(t1, lane, 8);
+            const float x = t1[0] + __shfl_xor_sync(0xffffffffu, t1[0], 4);
+            if (!(lane & 4)) sred_[ph][0][wq][col] = x;
+        }
+        if (want_da) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) ksum += __shfl_xor_sync(0xffffffffu, ksum, o);
+            if (lane == 0) swk_[ph][tid >> 5] = ksum;
         }
     }
     if (NORM) {
         // Through the normalisation: dx = r (dx^ - x^ <x^, dx^>).  The staged tiles hold dk^ and dq^ token-major, like the
-        // K^ and Q^ tiles, so both steps are row-wise passes with 16-byte accesses: thread (row r, part) takes two
-        // 16-byte chunks of its row; first the partial row dot products (eight parts per row, summed through scratch
-        // over the dead row sums), then the corrected rows.
-        float (*part_k)[C] = reinterpret_cast<float (*)[C]>(&srow[0][0][0]);     // [8][C]
-        float (*part_q)[C] = reinterpret_cast<float (*)[C]>(&srow[2][0][0]);     // [8][C]
-        constexpr int kPer = 16 / (kBwdCompute / 64);
-        static_assert(kBwdCompute / 64 == 8 && kNWG == 4, "scratch of the row dot products: 8 parts of 64 rows, twice");
-        const int r = tid & 63, part = tid >> 6;
-        csync();                             // the staged tiles are complete; the row sums have been consumed
-        float ck = 0.f, cq = 0.f;
+        // K^ and Q^ tiles: 16 lanes to a row, one 16-byte chunk each, the row's dot product by shuffles.
+        csync();                             // the staged tiles are complete
+        const int ci = tid & 15;
 #pragma unroll
-        for (int cc = 0; cc < kPer; ++cc) {
-            const int ci = part * kPer + cc;
+        for (int r = tid >> 4; r < C; r += kBwdCompute / 16) {
             const uint32_t off = (ci >> 3) * 8192 + sw128_chunk(r, ci & 7);
-            float a8[8], x8[8];
+            float a8[8], x8[8], b8[8], y8[8], ck = 0.f, cq = 0.f;
             load8(sm + oStDk + off, a8);
             load8(sm + oK + off, x8);
+            load8(sm + oStDq + off, b8);
+            load8(sm + oQ + off, y8);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) ck = fmaf(a8[e], x8[e], ck);
-            load8(sm + oStDq + off, a8);
-            load8(sm + oQ + off, x8);
+            for (int e = 0; e < 8; ++e) { ck = fmaf(a8[e], x8[e], ck); cq = fmaf(b8[e], y8[e], cq); }
 #pragma unroll
-            for (int e = 0; e < 8; ++e) cq = fmaf(a8[e], x8[e], cq);
-        }
-        part_k[part][r] = ck;
-        part_q[part][r] = cq;
-        csync();
-        ck = 0.f; cq = 0.f;
+            for (int o = 1; o < 16; o <<= 1) {
+                ck += __shfl_xor_sync(0xffffffffu, ck, o);
+                cq += __shfl_xor_sync(0xffffffffu, cq, o);
+            }
+            const float2 rn = srn[r];        // {1/|k|, 1/|q|}
 #pragma unroll
-        for (int pp = 0; pp < 8; ++pp) { ck += part_k[pp][r]; cq += part_q[pp][r]; }
-        const float2 rn = srn[r];            // {1/|k|, 1/|q|}
-#pragma unroll
-        for (int cc = 0; cc < kPer; ++cc) {
-            const int ci = part * kPer + cc;
-            const uint32_t off = (ci >> 3) * 8192 + sw128_chunk(r, ci & 7);
-            float a8[8], x8[8];
-            load8(sm + oStDk + off, a8);
-            load8(sm + oK + off, x8);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) a8[e] = rn.x * fmaf(-ck, x8[e], a8[e]);
+            for (int e = 0; e < 8; ++e) {
+                a8[e] = rn.x * fmaf(-ck, x8[e], a8[e]);
+                b8[e] = rn.y * fmaf(-cq, y8[e], b8[e]);
+            }
             sts128(sm + oStDk + off, pack8(a8));
-            load8(sm + oStDq + off, a8);
-            load8(sm + oQ + off, x8);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) a8[e] = rn.y * fmaf(-cq, x8[e], a8[e]);
-            sts128(sm + oStDq + off, pack8(a8));
+            sts128(sm + oStDq + off, pack8(b8));
         }
     }
     fence_proxy_async();
     tc_fence_before();
-    nb_arrive(kNbOut, kBwdThreads);
-    csync();
-    // ---- decay gradient ----------------------------------------------------------------------------
-    if (tid < C && (want_dl || want_da)) {
-        const int r = tid;
-        float kd = 0.f, dl = 0.f, t1 = 0.f;
-#pragma unroll
-        for (int w4 = 0; w4 < 4; ++w4) { kd += sred[0][w4][r]; dl += sred[1][w4][r]; t1 += sred[2][w4][r]; }
-        sdg[r] = t1 + dg_pre - kd;
-        skd[r] = kd;                            // summed below into dg of the last token
-        if (want_dl && r < live) p.dlam[(row0 + r) * p.H + hh] = p.logits ? dl * slam[r] * (1.f - slam[r]) : dl;
-    }
-    csync();
-    if (tid < 32 && want_da) {
-        // warp 0: lane owns tokens 2*lane, 2*lane+1; d log alpha_i = sum_{r >= i} dg_r (suffix sums)
-        const float a = sdg[2 * lane];
-        float b2 = sdg[2 * lane + 1];
-        float kds = skd[2 * lane] + skd[2 * lane + 1];
-        float dhh = lane < kBwdCompute / 32 ? swp[lane] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            kds += __shfl_xor_sync(0xffffffffu, kds, o);
-            dhh += __shfl_xor_sync(0xffffffffu, dhh, o);
-        }
-        if (lane == 31) b2 += sgam[C - 1] * dhh + kds;
-        float sfx = a + b2;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float t = __shfl_down_sync(0xffffffffu, sfx, o);
-            if (lane + o < 32) sfx += t;
-        }
-        if (p.dalpha) {
-            // d log alpha -> d alpha = d log alpha / alpha;  with logit inputs d/dz log sigmoid(z) = 1 - sigmoid(z)
-            const float a0 = salpha[2 * lane], a1 = salpha[2 * lane + 1];
-            if (2 * lane < live) p.dalpha[(row0 + 2 * lane) * p.H + hh] = p.logits ? sfx * (1.f - a0) : sfx / a0;
-            if (2 * lane + 1 < live) p.dalpha[(row0 + 2 * lane + 1) * p.H + hh] = p.logits ? (sfx - a) * (1.f - a1) : (sfx - a) / a1;
-        }
-    }
-    __syncthreads();                     // every read of this chunk's tiles and scratch is done
+    nb_arrive(kNbOut, kBwdNb);
+    nb_sync(kNbEnd, kBwdThreads);        // every read of this chunk's tiles and accumulators is done
     }  // chunk loop
     }  // epilogue threads
     tc_fence_before();
     __syncthreads();
-    if (tid == kBwdCompute && s_abort) { mbar_wait(&bar_load, 0); mbar_wait(&bar_late, 0); }   // one more bounded chance for copies in flight
+    if (tid == kBwdCompute && s_abort) { mbar_wait(&bar_load, 0); mbar_wait(&bar_h, 0); mbar_wait(&bar_qk, 0); }   // one more bounded chance for copies in flight
     if (tid < 32) tmem_dealloc(tb, 512);
 }
 
