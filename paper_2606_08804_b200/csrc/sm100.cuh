@@ -174,6 +174,11 @@ __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float* v) {
     asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld_frag2(uint32_t taddr, float* v) {            // 16 columns: v[4 (8 columns) + ..]
+    uint32_t* r = reinterpret_cast<uint32_t*>(v);
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
 // Four 8 x 8 bf16 matrices; lane l passes the address of row l % 8 of matrix l / 8.  T: transposed, register m of thread t
 // holds elements (row 2 (t % 4) + {0, 1}, column t / 4) of matrix m instead of (row t / 4, columns 2 (t % 4) + {0, 1})
 template <bool T>
@@ -299,10 +304,11 @@ __device__ __forceinline__ void umma_commit_w(uint64_t* bar, uint32_t issue) {
         "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
         ::"r"(smem_u32(bar)), "r"(issue) : "memory");
 }
-template <bool A_MN, bool B_MN>
+// M = 64: row r of the product lands on TMEM lane 32 (r / 16) + r % 16, i.e. every warp of a warpgroup gets 16 rows.
+template <bool A_MN, bool B_MN, int M = 128>
 __device__ __forceinline__ void umma_product_w(uint32_t d_tmem, uint32_t a_saddr, uint32_t a_blk, uint32_t b_saddr, uint32_t b_blk,
                                                int N, int K, bool accumulate, uint32_t issue, bool a_neg = false) {
-    const uint32_t idesc = make_idesc(128, N, A_MN, B_MN, a_neg);
+    const uint32_t idesc = make_idesc(M, N, A_MN, B_MN, a_neg);
     const uint64_t a0 = A_MN ? desc_mnmajor(a_saddr, a_blk) : desc_kmajor(a_saddr);
     const uint64_t b0 = B_MN ? desc_mnmajor(b_saddr, b_blk) : desc_kmajor(b_saddr);
 #pragma unroll

@@ -437,9 +437,9 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     __shared__ float2 srn_[2][C];     // NORM: {1/|k_t|, 1/|q_t|}
     __shared__ float sred_[2][2][4][C];   // per-warp column sums: [0] rowsum(dQ1 o Q) - <(K-> dh)_r, Delta_r>, [1] d lambda
     __shared__ float swk_[2][kBwdCompute / 32];        // per-warp sums of <(K-> dh)_r, Delta_r>
-    __shared__ float scol[2][2][C];   // column sums of dP o P, dA o A by halves of the rows
-    __shared__ __align__(16) float srow[6][kNWG][C];   // per-row partial sums over each warpgroup's columns: rPP, d beta, t2, rAA; [4], [5]: d beta and
-                                         // rAA of the column groups that the upper lanes take
+    __shared__ float scol[2][4][C];   // column sums of dP o P, dA o A by quarters of the rows
+    __shared__ float srow[4][kNWG][C];   // per-row partial sums over each warpgroup's columns: rPP, d beta, t2, rAA
+
     __shared__ float swp[kBwdCompute / 32], stot[2];
 
     const int tid = threadIdx.x, wg = tid >> 7, l = tid & 127, lane = tid & 31, wq = (tid >> 5) & 3;
@@ -565,39 +565,37 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             umma_product_w<true, true>(T3, aH, 16384, adDt, 8192, C, D, false, issue, true);     // -h dDelta^T      [i][r] = dW<-^T
             umma_commit_w(&bm_a, issue);
             umma_product_w<false, false>(T6, adDt, 16384, aMt, 8192, C, C, false, issue);        // dDelta^T M       [j][s]
-            umma_product_w<false, true>(T2, aV, 8192, adDt, 8192, C, D, false, issue);           // V dDelta^T       [s][r]
+            umma_product_w<false, true, 64>(T2, aV, 8192, adDt, 8192, C, D, false, issue);       // V dDelta^T       [s][r]
             umma_commit_w(&bm_b, issue);                // from here on no product reads V or dDelta^T any more
-            umma_product_w<false, true>(T1, adO - 8192, 8192, aDt, 8192, C, D, false, issue);    // dO Delta^T [r][s], rows r on lanes 64 + r
+            umma_product_w<false, true, 64>(T1, adO, 8192, aDt, 8192, C, D, false, issue);       // dO Delta^T       [r][s]
+            umma_commit_w(&bm_c, issue);
             umma_product_w<true, false>(T4, aH, 16384, adO, 8192, C, D, false, issue);           // h dO^T           [i][r]
-            umma_commit_w(&bm_c, issue);                // from here on no product reads dO or h any more
             wait(&bar_qk, ph);
             nb_sync(kNbDW, kBwdNb);                                      // the dW<-^T tile is complete
             nb_sync(kNbX, kBwdNb);                                       // X has been built
             tc_fence_after();
-            // the product that the dependent chain waits for goes first, the two that are needed late after it
-            umma_product_w<false, true>(T3, aXe, 8192, adW, 8192, C, D, false, issue);           // X dW<-^T         [s][r]
+            // the product that the dependent chain waits for goes first, those that are needed late after it
+            umma_product_w<false, true, 64>(T3, aXe, 8192, adW, 8192, C, D, false, issue);       // X dW<-^T         [s][r]
             umma_commit_w(&bm_2, issue);
+            umma_product_w<false, false, 64>(T0, aXe, 8192, aK, 8192, C, D, false, issue);       // X K^T            [r][i]
             umma_product_w<true, true>(T5, adH, 16384, aDt, 8192, C, D, false, issue);           // dh Delta^T       [i][s]
-            umma_product_w<false, false>(T0, aXe, 8192, aK, 8192, C, D, false, issue);           // X K^T            [r][i]
-            umma_product_w<false, false>(T7, aXe - 8192, 8192, aK, 8192, C, D, false, issue);    // once more, rows r on lanes 64 + r
+            nb_sync(kNbDTb, kBwdNb);
+            tc_fence_after();
+            umma_product_w<true, true, 64>(T3, adTb, 8192, aMt, 8192, C, C, false, issue);       // N~ = dT diag(beta) M^T   [r][u]
+            umma_commit_w(&bm_3, issue);                // from here on nobody reads h, dh or Delta^T
+            nb_sync(kNbN, kBwdNb);                                       // N~ is a tile, and so is dP o Gamma
+            tc_fence_after();
+            umma_product_w<false, true, 64>(T2, aMt, 8192, aN, 8192, C, C, false, issue, true);  // dA = -M^T N~     [r][s]
+            umma_commit_w(&bm_4, issue);
+            umma_product_w<true, true>(T1, aQ, 8192, adPG, 8192, C, C, false, issue);            // (dPG^T Q)^T      [i][s]
+            umma_product_w<true, false>(T3, aK, 8192, adPG, 8192, C, C, false, issue);           // (dPG K)^T        [i][r]
             nb_sync(kNbDV, kBwdNb);                                      // T6 has been read
             tc_fence_after();
             umma_product_w<false, false>(T6, adW, 16384, aMt, 8192, C, C, false, issue);         // dW<-^T M         [i][s]
-            nb_sync(kNbDTb, kBwdNb);
-            tc_fence_after();
-            umma_product_w<true, true>(T3, adTb, 8192, aMt, 8192, C, C, false, issue);           // N~ = dT diag(beta) M^T   [r][u]
-            umma_commit_w(&bm_3, issue);
-            nb_sync(kNbN, kBwdNb);
-            tc_fence_after();
-            umma_product_w<false, true>(T2, aMt, 8192, aN, 8192, C, C, false, issue, true);      // dA = -M^T N~     [r][s]
-            umma_product_w<false, true>(T3, aMt - 8192, 8192, aN, 8192, C, C, false, issue, true);   // once more, rows r on lanes 64 + r
-            umma_commit_w(&bm_4, issue);
             nb_sync(kNbDXK, kBwdNb);
             tc_fence_after();
             umma_product_w<true, false>(T7, aK, 8192, adXK, 8192, C, C, false, issue);           // (dXK K)^T        [i][r]
-            umma_product_w<true, true>(T1, aXe, 8192, adXK, 8192, C, C, false, issue);           // (dXK^T X)^T      [i][s]
-            umma_product_w<true, true>(T1, aQ, 8192, adPG, 8192, C, C, true, issue);             // + (dPG^T Q)^T
-            umma_product_w<true, false>(T2, aK, 8192, adPG, 8192, C, C, false, issue);           // (dPG K)^T        [i][r]
+            umma_product_w<true, true>(T1, aXe, 8192, adXK, 8192, C, C, true, issue);            // + (dXK^T X)^T    [i][s]
             umma_commit_w(&bm_5, issue);
             nb_sync(kNbEnd, kBwdThreads);                                // every read of this chunk's tiles and accumulators is done
         }
@@ -639,17 +637,17 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             const uint32_t ph = it & 1;
             if (__any_sync(0xffffffffu, s_latch)) break;
             if (lead && more) prefetch_late(next_id);
+            if (lead) {
+                wait(&bm_3, ph);                                         // from here on nobody reads h or dh
+                if (more && !s_abort) issue_h(next_id);
+            }
             nb_sync(kNbDVt, kBwdNb);                                     // the dv staging tile is complete
             if (lead) {
                 tma_store_3d(&mapdV, sm + oStDv, hh * D, n * C, b);          // rows past the end of the sequence are skipped
                 tma_store_3d(&mapdV, sm + oStDv + 8192, hh * D + 64, n * C, b);
                 tma_store_commit();
-            }
-            if (lead) {
-                wait(&bm_3, ph);                                         // from here on nobody reads h or dh
-                if (more && !s_abort) issue_h(next_id);
-                wait(&bm_5, ph);                                         // nor anything but Q, K
-                tma_store_wait_read();                                   // dv's staging tile
+                tma_store_wait_read();
+                wait(&bm_5, ph);                                         // from here on nobody reads anything but Q, K
                 fence_proxy_async();
                 if (more && !s_abort) issue_early(next_id);
             }
@@ -757,10 +755,13 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             float rPP = 0.f, t2 = 0.f, rAA = 0.f, dbt = 0.f;
 #pragma unroll
             for (int w4 = 0; w4 < kNWG; ++w4) {
-                rPP += srow[0][w4][r]; dbt += srow[1][w4][r] + srow[4][w4][r]; t2 += srow[2][w4][r]; rAA += srow[3][w4][r] + srow[5][w4][r];
+                rPP += srow[0][w4][r]; dbt += srow[1][w4][r]; t2 += srow[2][w4][r]; rAA += srow[3][w4][r];
             }
             dg_pre = rPP + t2 + rAA;
-            if (want_da) dg_pre -= scol[0][0][r] + scol[0][1][r] + scol[1][0][r] + scol[1][1][r];
+            if (want_da) {
+#pragma unroll
+                for (int w4 = 0; w4 < 4; ++w4) dg_pre -= scol[0][w4][r] + scol[1][w4][r];
+            }
             // with logit inputs: d/dz of sigmoid(z) is sigmoid(z) (1 - sigmoid(z))
             if (n * C + r < p.T) p.dbeta[((size_t)(bh / p.H) * p.T + (size_t)n * C + r) * p.H + bh % p.H] = p.logits ? dbt * be0 * (1.f - be0) : dbt;
             if (want_da) {
@@ -793,28 +794,6 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     const float *sbeta = sbeta_[ph], *slam = slam_[ph], *sg = sg_[ph], *sgam = sgam_[ph];
     const float4* scf = scf_[ph];
     const float2* srn = srn_[ph];
-    // ---- partial <dh,h>_F, under the first products ---------------------------------------------------
-    wait(&bar_h, ph);
-    float dhh_part = 0.f;
-    if (want_da)
-#pragma unroll
-    for (int cc = 0; cc < 16 / kNWG; ++cc) {
-        const int ci = wg * (16 / kNWG) + cc;                // chunk 0..15 of line l
-        const uint32_t off = (ci >> 3) * 16384 + sw128_chunk(l, ci & 7);
-        float a[8], c8[8];
-        load8(sm + oH + off, a);
-        load8(sm + odH + off, c8);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) dhh_part = fmaf(a[e], c8[e], dhh_part);
-    }
-    if (want_da) {
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 16);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 8);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 4);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 2);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 1);
-        if (lane == 0) swp[tid >> 5] = dhh_part;
-    }
     // ---- dW<-^T = -h dDelta^T: row i = l as an operand tile (region of its own: dO is still being read) -----
     wait(&bar_st, ph);                                    // the staged dk, dq of the chunk before lie over X and this tile
     wait(&bm_a, ph);
@@ -859,8 +838,132 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     }
     fence_proxy_async();
     nb_arrive(kNbX, kBwdNb);
+    // ---- partial <dh,h>_F, under X dW<-^T -------------------------------------------------------------
+    wait(&bar_h, ph);                                     // (long there: for what TMA wrote to be visible to this thread)
+    float dhh_part = 0.f;
+    if (want_da)
+#pragma unroll
+    for (int cc = 0; cc < 16 / kNWG; ++cc) {
+        const int ci = wg * (16 / kNWG) + cc;                // chunk 0..15 of line l
+        const uint32_t off = (ci >> 3) * 16384 + sw128_chunk(l, ci & 7);
+        float a[8], c8[8];
+        load8(sm + oH + off, a);
+        load8(sm + odH + off, c8);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) dhh_part = fmaf(a[e], c8[e], dhh_part);
+    }
+    if (want_da) {
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 16);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 8);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 4);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 2);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 1);
+        if (lane == 0) swp[tid >> 5] = dhh_part;
+    }
+    // The 64-row accumulators: this thread's rows are rw + 8 j + lane / 4, j = 0, 1, its columns c0 + 8 g + ft + {0, 1}.  Of a
+    // sum over columns, the lane ends up with that of row `mine`, of a sum over the warp's 16 rows with that of column `ours`.
+    const int rw = 16 * wq, mine = rw + 4 * (lane & 2) + (lane >> 2), ours = c0 + ((lane & 16) ? 8 : 0) + ft + ((lane & 8) ? 1 : 0);
+    const bool my_row = !(lane & 1), our_col = !(lane & 4);
+    auto row_sum = [&](float* v) { fold<2>(v, lane, 2); return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1); };
+    auto col_sum = [&](float* v) { fold<4>(v, lane, 16); fold<2>(v, lane, 8); return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 4); };
+    const int r0 = rw + (lane >> 2);                       // rows r0, r0 + 8
+    // of a [64 rows][64] tile: matrix m = 2 g + j, rows rw + 8 j .., columns c0 + 8 g ..
+    const uint32_t at = sw128_chunk(rw + (lane & 15), wg * 2 + (lane >> 4));
+    // ---- dT^T row s, columns r;  M[r][s] = line s of Mt ------------------------------------------------
     wait(&bm_b, ph);
+    wait(&bm_2, ph);
     tc_fence_after();
+    {
+        float a[8], bq[8], db[2] = {}, mb[2] = {};
+        uint32_t mr[4], o[4];
+        tmem_ld_frag2(frag(T2, 0, 0), a);
+        tmem_ld_frag2(frag(T3, 0, 0), bq);
+        ldsm4<false>(sm + oMt + at, mr);
+        const float gs[2] = {sgam[r0], sgam[r0 + 8]}, bs[2] = {sbeta[r0], sbeta[r0 + 8]};
+        tmem_ld_wait();
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int j = m & 1;
+            float tb8[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int x = 4 * (m >> 1) + 2 * j + e;
+                const float mv = __uint_as_float(e ? mr[m] & 0xffff0000u : mr[m] << 16), dt = fmaf(gs[j], bq[x], a[x]);
+                db[j] = fmaf(dt, mv, db[j]);
+                mb[j] = fmaf(mv, bq[x], mb[j]);
+                tb8[e] = bs[j] * dt;
+            }
+            o[m] = pack_bf16(tb8[0], tb8[1]);
+        }
+        stsm4<false>(sm + odTb + at, o);
+        fence_proxy_async();
+        tc_fence_before();
+        nb_arrive(kNbDTb, kBwdNb);
+        const float d = row_sum(db), t2 = sgam[mine] * sbeta[mine] * row_sum(mb);
+        if (my_row) { srow[1][wg][mine] = d; srow[2][wg][mine] = t2; }
+    }
+    const float gr[2] = {sg[r0], sg[r0 + 8]};
+    float gm[8];                                           // Gamma_rs, s <= r
+    {
+        float gs[4];
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const float2 t = *reinterpret_cast<const float2*>(sg + c0 + 8 * g + ft);
+            gs[2 * g] = t.x; gs[2 * g + 1] = t.y;
+        }
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            const int s = c0 + 8 * (x >> 2) + ft + (x & 1), r = r0 + 8 * ((x >> 1) & 1);
+            gm[x] = s <= r ? (has_alpha ? __expf(gr[(x >> 1) & 1] - gs[2 * (x >> 2) + (x & 1)]) : 1.f) : 0.f;
+        }
+    }
+    // ---- dP, under N~: causal mask, dP o P (row and column sums), dP o Gamma as an operand tile ----------
+    wait(&bm_c, ph);
+    tc_fence_after();
+    {
+        float v[8], rPP[2] = {}, cP[4] = {};
+        uint32_t pr[4], o[4];
+        tmem_ld_frag2(frag(T1, 0, 0), v);
+        ldsm4<false>(sm + oP + at, pr);                    // causal: zero above the diagonal
+        tmem_ld_wait();
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int j = m & 1;
+            float pg[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int x = 4 * (m >> 1) + 2 * j + e;
+                const float pp = v[x] * __uint_as_float(e ? pr[m] & 0xffff0000u : pr[m] << 16);
+                rPP[j] += pp;
+                cP[2 * (m >> 1) + e] += pp;
+                pg[e] = gm[x] * v[x];
+            }
+            o[m] = pack_bf16(pg[0], pg[1]);
+        }
+        stsm4<false>(sm + odPG + at, o);
+        const float d = row_sum(rPP);
+        if (my_row) srow[0][wg][mine] = d;
+        if (want_da) {
+            const float x = col_sum(cP);
+            if (our_col) scol[0][wq][ours] = x;
+        }
+    }
+    // ---- N~ = dT diag(beta) M^T, copied out as an operand tile --------------------------------------
+    wait(&bm_3, ph);
+    tc_fence_after();
+    {
+        float v[8];
+        uint32_t o[4];
+        tmem_ld_frag2(frag(T3, 0, 0), v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int m = 0; m < 4; ++m) o[m] = pack_bf16(v[4 * (m >> 1) + 2 * (m & 1)], v[4 * (m >> 1) + 2 * (m & 1) + 1]);
+        stsm4<false>(sm + oN + at, o);
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    nb_arrive(kNbN, kBwdNb);
+    // ---- dV, under dA ---------------------------------------------------------------------------------
     {
         // dV^T [j][s], scaled by beta_s, transposed into the staging tile
         float dvv[2][2][4];                               // [8 columns][16 rows]
@@ -882,178 +985,41 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     tc_fence_before();
     nb_arrive(kNbDV, kBwdNb);
     nb_arrive(kNbDVt, kBwdNb);
-    // The 64-row accumulators, in fragments: this thread's rows are rw + 16 hf + 8 j + lane / 4; of a sum over columns, the
-    // lane ends up with that of row `mine` (quad_sum), of a sum over a warp's 32 rows with that of a column (see below).
-    const int rw = 32 * (wq & 1), mine = rw + 8 * (lane & 3) + (lane >> 2);
-    auto quad_sum = [&](float* v) { fold<4>(v, lane, 2); fold<2>(v, lane, 1); return v[0]; };
-    auto row_of = [&](int m) { return rw + 8 * m + (lane >> 2); };                     // m = 2 hf + j
-    auto at = [&](int g) { return sw128_chunk(rw + 8 * (lane >> 3) + (lane & 7), wg * 2 + g); };   // of a [64 rows][64] tile
-    // 8 columns of the dA epilogue; tA = dA, tX = X K^T, both with their rows on this warp's lanes
-    auto dA_group = [&](uint32_t tA, uint32_t tX, int g, float& db, float& rAA) {
-        float da[2][4], xk[2][4], dbr[4] = {}, cA[2] = {};
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) { tmem_ld_frag(frag(tA, g, hf), da[hf]); tmem_ld_frag(frag(tX, g, hf), xk[hf]); }
-        const int s = c0 + 8 * g + ft;
-        const float2 gs = *reinterpret_cast<const float2*>(sg + s);
-        tmem_ld_wait();
+    // ---- dA = -M^T N~ -----------------------------------------------------------------------------
+    wait(&bm_4, ph);
+    tc_fence_after();
+    {
+        float da[8], xk[8], dbr[2] = {}, cA[4] = {};
         uint32_t o[4];
+        tmem_ld_frag2(frag(T2, 0, 0), da);
+        tmem_ld_frag2(frag(T0, 0, 0), xk);
+        const float br[2] = {sbeta[r0], sbeta[r0 + 8]};
+        tmem_ld_wait();
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            const int r = row_of(m);
-            const float gr = sg[r], br = sbeta[r];
+            const int j = m & 1;
             float out[2];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const bool on = s + e < r;
-                const float gm = on ? (has_alpha ? __expf(gr - (e ? gs.y : gs.x)) : 1.f) : 0.f;
-                const float d = on ? da[m >> 1][2 * (m & 1) + e] * gm : 0.f;
-                const float dgx = d * xk[m >> 1][2 * (m & 1) + e];
-                dbr[m] += dgx;
-                cA[e] = fmaf(br, dgx, cA[e]);
-                out[e] = br * d;                               // dXK
+                const int x = 4 * (m >> 1) + 2 * j + e;
+                const float d = c0 + 8 * (m >> 1) + ft + e < r0 + 8 * j ? da[x] * gm[x] : 0.f, dgx = d * xk[x];
+                dbr[j] += dgx;
+                cA[2 * (m >> 1) + e] = fmaf(br[j], dgx, cA[2 * (m >> 1) + e]);
+                out[e] = br[j] * d;                        // dXK
             }
             o[m] = pack_bf16(out[0], out[1]);
         }
-        stsm4<false>(sm + odXK + at(g), o);
-        db = quad_sum(dbr);
-        rAA = sbeta[mine] * db;
-        if (want_da) {
-            fold<2>(cA, lane, 16);
-            float x = cA[0];
-            x += __shfl_xor_sync(0xffffffffu, x, 8);
-            x += __shfl_xor_sync(0xffffffffu, x, 4);
-            if (!(lane & 12)) scol[1][wq & 1][s + (lane >> 4)] = x;
-        }
-    };
-    static_assert(kG8 == 2, "the dA epilogue gives one column group to each half of a warpgroup");
-    // From here to the last products the two halves of every warpgroup go separate ways.  Lanes 64..127 (whose rows
-    // of the 64-row accumulators are padding) take dP, whose product was issued with its rows on their lanes; lanes
-    // 0..63 walk the dependent chain dT -> N~ -> dA -> dXK.  Both raise every barrier of the chain exactly once.
-    if (wq >= 2) {
-        nb_arrive(kNbDTb, kBwdNb);
-        nb_arrive(kNbN, kBwdNb);
-        wait(&bm_c, ph);                  // dP's product
-        wait(&bm_2, ph);                  // of the tile over V that is written here nobody reads any more
-        tc_fence_after();
-        // dP: causal mask, dP o P (row and column sums), dP o Gamma as an operand tile
-        float v[2][2][4], rPP[4] = {}, cP[4];
-        uint32_t pr[2][4];
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) tmem_ld_frag(frag(T1, g, hf), v[g][hf]);
-            ldsm4<false>(sm + oP + at(g), pr[g]);
-        }
-        tmem_ld_wait();
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            const int s = c0 + 8 * g + ft;
-            const float2 gs = *reinterpret_cast<const float2*>(sg + s);
-            float c[2] = {};
-            uint32_t o[4];
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const int r = row_of(m);
-                const float gr = sg[r];
-                float pg[2];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const bool on = s + e <= r;
-                    const float dp = on ? v[g][m >> 1][2 * (m & 1) + e] : 0.f;
-                    const float pp = dp * __uint_as_float(e ? pr[g][m] & 0xffff0000u : pr[g][m] << 16);
-                    rPP[m] += pp;
-                    c[e] += pp;
-                    pg[e] = on ? (has_alpha ? dp * __expf(gr - (e ? gs.y : gs.x)) : dp) : 0.f;
-                }
-                o[m] = pack_bf16(pg[0], pg[1]);
-            }
-            stsm4<false>(sm + odPG + at(g), o);
-            cP[2 * g] = c[0]; cP[2 * g + 1] = c[1];
-        }
-        srow[0][wg][mine] = quad_sum(rPP);
-        if (want_da) {
-            fold<4>(cP, lane, 16); fold<2>(cP, lane, 8);
-            const float x = cP[0] + __shfl_xor_sync(0xffffffffu, cP[0], 4);
-            if (!(lane & 4)) scol[0][wq & 1][c0 + ((lane & 16) ? 8 : 0) + ft + ((lane & 8) ? 1 : 0)] = x;
-        }
-        // second column group of the dA epilogue, from the copies of dA and X K^T whose rows lie on these lanes
-        wait(&bm_4, ph);
-        tc_fence_after();
-        float db, rAA;
-        dA_group(T3, T7, 1, db, rAA);
-        srow[4][wg][mine] = db;
-        srow[5][wg][mine] = rAA;
-    } else {
-        wait(&bm_2, ph);
-        tc_fence_after();
-        {
-            // dT^T row s, my columns r;  M[r][s] = line s of Mt
-            float a[2][2][4], bq[2][2][4], db[4] = {}, mb[4] = {};
-            uint32_t mr[2][4];
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) { tmem_ld_frag(frag(T2, g, hf), a[g][hf]); tmem_ld_frag(frag(T3, g, hf), bq[g][hf]); }
-                ldsm4<false>(sm + oMt + at(g), mr[g]);
-            }
-            tmem_ld_wait();
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                uint32_t o[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const float gs = sgam[row_of(m)], bs = sbeta[row_of(m)];
-                    float tb8[2];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const float x = bq[g][m >> 1][2 * (m & 1) + e], mv = __uint_as_float(e ? mr[g][m] & 0xffff0000u : mr[g][m] << 16);
-                        const float dt = fmaf(gs, x, a[g][m >> 1][2 * (m & 1) + e]);
-                        db[m] = fmaf(dt, mv, db[m]);
-                        mb[m] = fmaf(mv, x, mb[m]);
-                        tb8[e] = bs * dt;
-                    }
-                    o[m] = pack_bf16(tb8[0], tb8[1]);
-                }
-                stsm4<false>(sm + odTb + at(g), o);
-            }
-            fence_proxy_async();
-            tc_fence_before();
-            nb_arrive(kNbDTb, kBwdNb);
-            srow[1][wg][mine] = quad_sum(db);
-            srow[2][wg][mine] = sgam[mine] * sbeta[mine] * quad_sum(mb);
-        }
-        // ---- N~ = dT diag(beta) M^T, copied out as an operand tile --------------------------------------
-        wait(&bm_3, ph);
-        tc_fence_after();
-        {
-            float v[2][2][4];
-#pragma unroll
-            for (int g = 0; g < 2; ++g)
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) tmem_ld_frag(frag(T3, g, hf), v[g][hf]);
-            tmem_ld_wait();
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                uint32_t o[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) o[m] = pack_bf16(v[g][m >> 1][2 * (m & 1)], v[g][m >> 1][2 * (m & 1) + 1]);
-                stsm4<false>(sm + oN + at(g), o);
-            }
-        }
+        stsm4<false>(sm + odXK + at, o);
         fence_proxy_async();
         tc_fence_before();
-        nb_arrive(kNbN, kBwdNb);
-        // ---- dA = -M^T N~ -----------------------------------------------------------------------------
-        wait(&bm_4, ph);
-        tc_fence_after();
-        float db, rAA;
-        dA_group(T2, T0, 0, db, rAA);
-        srow[1][wg][mine] += db;
-        srow[3][wg][mine] = rAA;
-    }  // lanes 0..63: the dependent chain
-    fence_proxy_async();
-    tc_fence_before();
-    nb_arrive(kNbDXK, kBwdNb);
+        nb_arrive(kNbDXK, kBwdNb);
+        const float d = row_sum(dbr);
+        if (my_row) { srow[1][wg][mine] += d; srow[3][wg][mine] = sbeta[mine] * d; }
+        if (want_da) {
+            const float x = col_sum(cA);
+            if (our_col) scol[1][wq][ours] = x;
+        }
+    }
     nb_arrive(kNbSum, kNbSumN);
     wait(&bm_5, ph);
     tc_fence_after();
@@ -1068,7 +1034,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
                 tmem_ld_frag(frag(T6, g, hf), dx[hf]); tmem_ld_frag(frag(T7, g, hf), v[hf]); tmem_ld_frag(frag(T1, g, hf), w[hf]);
-                tmem_ld_frag(frag(T5, g, hf), u[hf]); tmem_ld_frag(frag(T4, g, hf), z[hf]); tmem_ld_frag(frag(T2, g, hf), y[hf]);
+                tmem_ld_frag(frag(T5, g, hf), u[hf]); tmem_ld_frag(frag(T4, g, hf), z[hf]); tmem_ld_frag(frag(T3, g, hf), y[hf]);
             }
             uint32_t qr[4], kr[4], dkr[4], dqr[4];
             ldsm4<true>(sm + oQ + foff[g], qr);
