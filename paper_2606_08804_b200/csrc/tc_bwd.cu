@@ -658,13 +658,13 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             __syncwarp();
             nb_arrive(kNbEnd, kBwdThreads);                              // nobody waits for the copies to be issued
             if (lead) {
-                fence_proxy_async();                                     // the epilogue's reads of Q precede the copy into its region
-                if (more && !s_abort) issue_qk(next_id);
                 tma_store_3d(&mapdK, sm + oStDk, hh * D, n * C, b);
                 tma_store_3d(&mapdK, sm + oStDk + 8192, hh * D + 64, n * C, b);
                 tma_store_3d(&mapdQ, sm + oStDq, hh * D, n * C, b);
                 tma_store_3d(&mapdQ, sm + oStDq + 8192, hh * D + 64, n * C, b);
                 tma_store_commit();
+                fence_proxy_async();                                     // the epilogue's reads of Q precede the copy into its region
+                if (more && !s_abort) issue_qk(next_id);
             }
             if (lead) {
                 tma_store_wait_read();                                   // the staging tiles have been read by the stores
@@ -794,6 +794,28 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     const float *sbeta = sbeta_[ph], *slam = slam_[ph], *sg = sg_[ph], *sgam = sgam_[ph];
     const float4* scf = scf_[ph];
     const float2* srn = srn_[ph];
+    // ---- partial <dh,h>_F, under the first products ---------------------------------------------------
+    wait(&bar_h, ph);
+    float dhh_part = 0.f;
+    if (want_da)
+#pragma unroll
+    for (int cc = 0; cc < 16 / kNWG; ++cc) {
+        const int ci = wg * (16 / kNWG) + cc;                // chunk 0..15 of line l
+        const uint32_t off = (ci >> 3) * 16384 + sw128_chunk(l, ci & 7);
+        float a[8], c8[8];
+        load8(sm + oH + off, a);
+        load8(sm + odH + off, c8);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) dhh_part = fmaf(a[e], c8[e], dhh_part);
+    }
+    if (want_da) {
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 16);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 8);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 4);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 2);
+        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 1);
+        if (lane == 0) swp[tid >> 5] = dhh_part;
+    }
     // ---- dW<-^T = -h dDelta^T: row i = l as an operand tile (region of its own: dO is still being read) -----
     wait(&bar_st, ph);                                    // the staged dk, dq of the chunk before lie over X and this tile
     wait(&bm_a, ph);
@@ -838,28 +860,6 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     }
     fence_proxy_async();
     nb_arrive(kNbX, kBwdNb);
-    // ---- partial <dh,h>_F, under X dW<-^T -------------------------------------------------------------
-    wait(&bar_h, ph);                                     // (long there: for what TMA wrote to be visible to this thread)
-    float dhh_part = 0.f;
-    if (want_da)
-#pragma unroll
-    for (int cc = 0; cc < 16 / kNWG; ++cc) {
-        const int ci = wg * (16 / kNWG) + cc;                // chunk 0..15 of line l
-        const uint32_t off = (ci >> 3) * 16384 + sw128_chunk(l, ci & 7);
-        float a[8], c8[8];
-        load8(sm + oH + off, a);
-        load8(sm + odH + off, c8);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) dhh_part = fmaf(a[e], c8[e], dhh_part);
-    }
-    if (want_da) {
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 16);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 8);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 4);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 2);
-        dhh_part += __shfl_xor_sync(0xffffffffu, dhh_part, 1);
-        if (lane == 0) swp[tid >> 5] = dhh_part;
-    }
     // The 64-row accumulators: this thread's rows are rw + 8 j + lane / 4, j = 0, 1, its columns c0 + 8 g + ft + {0, 1}.  Of a
     // sum over columns, the lane ends up with that of row `mine`, of a sum over the warp's 16 rows with that of column `ours`.
     const int rw = 16 * wq, mine = rw + 4 * (lane & 2) + (lane >> 2), ours = c0 + ((lane & 16) ? 8 : 0) + ft + ((lane & 8) ? 1 : 0);
@@ -1041,7 +1041,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             ldsm4<true>(sm + oK + foff[g], kr);
             const float4 cf[2] = {scf[t], scf[t + 1]};
             tmem_ld_wait();
-            float s1[2] = {}, s2[2] = {};
+            float s0[2] = {}, s1[2] = {}, s2[2] = {};      // sums of U k, Z q, dX q
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 float dkv[2], dqv[2];
@@ -1050,23 +1050,25 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
                     const int hf = m >> 1, x = 2 * (m & 1) + e;
                     const float qv = __uint_as_float(e ? qr[m] & 0xffff0000u : qr[m] << 16), kv = __uint_as_float(e ? kr[m] & 0xffff0000u : kr[m] << 16);
                     const float dxe = fmaf(cf[e].x, dx[hf][x], v[hf][x]);                       // dX^T[i][t]
-                    const float kh = cf[e].y * u[hf][x];                                        // (K-> ^T applied to dh Delta^T)[i][t]
-                    const float q1 = cf[e].z * z[hf][x];
-                    dkv[e] = w[hf][x] + kh + dxe;                                               // d k  (d k^ with NORM)
-                    dqv[e] = q1 + y[hf][x] + cf[e].w * dxe;                                     // d q  (d q^ with NORM)
-                    // <(K-> dh)_t, Delta_t> = gamma_C/gamma_t sum_i K[t][i] (dh Delta^T)[i][t], all of it in fp32
-                    const float kd = kh * kv;
-                    ksum += kd;
-                    s1[e] += fmaf(q1, qv, -kd);
+                    dkv[e] = fmaf(cf[e].y, u[hf][x], w[hf][x] + dxe);                           // d k  (d k^ with NORM)
+                    dqv[e] = fmaf(cf[e].w, dxe, fmaf(cf[e].z, z[hf][x], y[hf][x]));             // d q  (d q^ with NORM)
+                    s0[e] = fmaf(u[hf][x], kv, s0[e]);
+                    s1[e] = fmaf(z[hf][x], qv, s1[e]);
                     s2[e] = fmaf(dxe, qv, s2[e]);
                 }
                 dkr[m] = pack_bf16(dkv[0], dkv[1]);
                 dqr[m] = pack_bf16(dqv[0], dqv[1]);
             }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                // <(K-> dh)_t, Delta_t> = gamma_C/gamma_t sum_i K[t][i] (dh Delta^T)[i][t], all of it in fp32
+                const float kd = cf[e].y * s0[e];
+                ksum += kd;
+                t1[2 * g + e] = fmaf(cf[e].z, s1[e], -kd);
+                dl[2 * g + e] = s2[e];
+            }
             stsm4<true>(sm + oStDk + foff[g], dkr);
             stsm4<true>(sm + oStDq + foff[g], dqr);
-            t1[2 * g] = s1[0]; t1[2 * g + 1] = s1[1];
-            dl[2 * g] = s2[0]; dl[2 * g + 1] = s2[1];
         }
         // lane: column 8 (bit 4) + 2 (lane % 4) + (bit 3)
         const int col = c0 + ((lane & 16) ? 8 : 0) + ft + ((lane & 8) ? 1 : 0);
