@@ -379,7 +379,7 @@ struct ChunkBwdParams {
 // shared-memory map of k_tc_chunk_bwd (bytes from the 1024-aligned base)
 constexpr int oQ = 0, oK = 16384, oV = 32768, odO = 49152, oX = 65536, oMt = 81920, oP = 90112, oDt = 98304,
               odDt = 114688, oH = 131072, odH = 163840;                            // TMA-loaded tiles (X is built)
-constexpr int kBwdEarlyBytes = 4 * 16384 + 2 * 8192;
+constexpr int kBwdEarlyBytes = 3 * 16384 + 2 * 8192;
 // tiles built later reuse regions whose contents are dead by then
 constexpr int odPG = oV, odTb = oV + 8192, odW = 196608, oN = oDt, odXK = oDt + 8192, oStDv = odDt, oStDk = oX, oStDq = odW;
 constexpr int kBwdSmem = 196608 + 16384 + 1024;      // + the dW<-^T tile, written while dO is still an operand
@@ -427,8 +427,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
                                                               ChunkBwdParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    // bar_load: V, dO, M^T, P, Delta^T, dDelta^T; bar_h: h^T, dh^T; bar_qk: Q, K; bar_st: the staged dk, dq have been read
-    __shared__ uint64_t bar_load, bar_h, bar_qk, bar_st, bm_a, bm_b, bm_c, bm_2, bm_3, bm_4, bm_5;
+    // bar_load: V, dO, M^T, P, Delta^T; bar_d: dDelta^T; bar_h: h^T, dh^T; bar_qk: Q, K; bar_st: the staged dk, dq have been read
+    __shared__ uint64_t bar_load, bar_d, bar_h, bar_qk, bar_st, bm_a, bm_b, bm_c, bm_2, bm_3, bm_4, bm_5;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort, s_latch;
     // by parity of the chunk, so that the token threads can publish a chunk ahead and take their sums a chunk late
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     const int c0 = wg * kCW;                                      // my columns of a 64-column accumulator
 
     if (tid == 0) {
-        mbar_init(&bar_load, 1); mbar_init(&bar_h, 1); mbar_init(&bar_qk, 1); mbar_init(&bar_st, 1);
+        mbar_init(&bar_load, 1); mbar_init(&bar_d, 1); mbar_init(&bar_h, 1); mbar_init(&bar_qk, 1); mbar_init(&bar_st, 1);
         mbar_init(&bm_a, 1); mbar_init(&bm_b, 1); mbar_init(&bm_c, 1); mbar_init(&bm_2, 1); mbar_init(&bm_3, 1); mbar_init(&bm_4, 1);
         mbar_init(&bm_5, 1);
         mbar_init_fence();
@@ -488,9 +488,10 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         int n_, bh_; item(ch, n_, bh_);
         const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
         const int yt = (int)((size_t)bh_ * p.Tp + (size_t)n_ * C);
-        mbar_expect_tx(&bar_load, kBwdEarlyBytes);
         const int yc = (int)(((size_t)bh_ * p.N + n_) * D);
-        tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_load);
+        mbar_expect_tx(&bar_d, 16384);            // on its own: the first product waits for it
+        tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_d);
+        mbar_expect_tx(&bar_load, kBwdEarlyBytes);
         tma_load_2d(sm + oMt, &mapMt, 0, yt, &bar_load);
         for (int blk = 0; blk < 2; ++blk)         // token rows past the end of the sequence arrive as zeros
             tma_load_3d(sm + oV + blk * 8192, &mapV, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
@@ -558,12 +559,13 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
             const uint32_t ph = it & 1;
             if (__any_sync(0xffffffffu, s_latch)) break;
-            wait(&bar_load, ph);
+            wait(&bar_d, ph);
             wait(&bar_h, ph);
             __syncwarp();
             tc_fence_after();
             umma_product_w<true, true>(T3, aH, 16384, adDt, 8192, C, D, false, issue, true);     // -h dDelta^T      [i][r] = dW<-^T
             umma_commit_w(&bm_a, issue);
+            wait(&bar_load, ph);
             umma_product_w<false, false>(T6, adDt, 16384, aMt, 8192, C, C, false, issue);        // dDelta^T M       [j][s]
             umma_product_w<false, true, 64>(T2, aV, 8192, adDt, 8192, C, D, false, issue);       // V dDelta^T       [s][r]
             umma_commit_w(&bm_b, issue);                // from here on no product reads V or dDelta^T any more
@@ -610,7 +612,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
             const int yc = (int)(((size_t)bh_ * p.N + n_) * D), yt = (int)((size_t)bh_ * p.Tp + (size_t)n_ * C);
             issue_qk(ch);
-            mbar_expect_tx_only(&bar_load, kBwdEarlyBytes - 16384);
+            mbar_expect_tx(&bar_load, kBwdEarlyBytes);
             for (int blk = 0; blk < 2; ++blk) {
                 tma_load_3d(sm + oV + blk * 8192, &mapV, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
                 tma_load_3d(sm + odO + blk * 8192, &mapdO, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
@@ -623,8 +625,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             grid_dep_wait();
             mbar_expect_tx(&bar_h, 32768);
             for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + odH + blk * 16384, &mapdHs, blk * 64, yc, &bar_h);
-            mbar_expect_tx(&bar_load, 16384);
-            tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_load);
+            mbar_expect_tx(&bar_d, 16384);
+            tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_d);
             mbar_arrive(&bar_st);                                        // nothing is staged yet
         }
         grid_dep_wait();
@@ -869,6 +871,21 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     const int r0 = rw + (lane >> 2);                       // rows r0, r0 + 8
     // of a [64 rows][64] tile: matrix m = 2 g + j, rows rw + 8 j .., columns c0 + 8 g ..
     const uint32_t at = sw128_chunk(rw + (lane & 15), wg * 2 + (lane >> 4));
+    const float gr[2] = {sg[r0], sg[r0 + 8]};
+    float gm[8];                                           // Gamma_rs, s <= r
+    {
+        float gs[4];
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const float2 t = *reinterpret_cast<const float2*>(sg + c0 + 8 * g + ft);
+            gs[2 * g] = t.x; gs[2 * g + 1] = t.y;
+        }
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            const int s = c0 + 8 * (x >> 2) + ft + (x & 1), r = r0 + 8 * ((x >> 1) & 1);
+            gm[x] = s <= r ? (has_alpha ? __expf(gr[(x >> 1) & 1] - gs[2 * (x >> 2) + (x & 1)]) : 1.f) : 0.f;
+        }
+    }
     // ---- dT^T row s, columns r;  M[r][s] = line s of Mt ------------------------------------------------
     wait(&bm_b, ph);
     wait(&bm_2, ph);
@@ -901,21 +918,6 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         nb_arrive(kNbDTb, kBwdNb);
         const float d = row_sum(db), t2 = sgam[mine] * sbeta[mine] * row_sum(mb);
         if (my_row) { srow[1][wg][mine] = d; srow[2][wg][mine] = t2; }
-    }
-    const float gr[2] = {sg[r0], sg[r0 + 8]};
-    float gm[8];                                           // Gamma_rs, s <= r
-    {
-        float gs[4];
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            const float2 t = *reinterpret_cast<const float2*>(sg + c0 + 8 * g + ft);
-            gs[2 * g] = t.x; gs[2 * g + 1] = t.y;
-        }
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const int s = c0 + 8 * (x >> 2) + ft + (x & 1), r = r0 + 8 * ((x >> 1) & 1);
-            gm[x] = s <= r ? (has_alpha ? __expf(gr[(x >> 1) & 1] - gs[2 * (x >> 2) + (x & 1)]) : 1.f) : 0.f;
-        }
     }
     // ---- dP, under N~: causal mask, dP o P (row and column sums), dP o Gamma as an operand tile ----------
     wait(&bm_c, ph);
@@ -1126,7 +1128,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     }  // epilogue threads
     tc_fence_before();
     __syncthreads();
-    if (tid == kBwdCompute && s_abort) { mbar_wait(&bar_load, 0); mbar_wait(&bar_h, 0); mbar_wait(&bar_qk, 0); }   // one more bounded chance for copies in flight
+    if (tid == kBwdCompute && s_abort) { mbar_wait(&bar_load, 0); mbar_wait(&bar_d, 0); mbar_wait(&bar_h, 0); mbar_wait(&bar_qk, 0); }   // one more bounded chance for copies in flight
     if (tid < 32) tmem_dealloc(tb, 512);
 }
 
