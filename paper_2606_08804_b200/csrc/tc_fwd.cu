@@ -94,7 +94,7 @@ __device__ __forceinline__ void put16(const float (&acc)[2][4], float sign, floa
 // M^T leaves with its zeros and ones.  Block-wise: the 16 x 16 diagonal blocks by right-looking substitution, a column in
 // the registers of a lane, two blocks per warp; then blocks joined twice, M21^T = -M11^T (A21^T M22^T), on the warp-level
 // tensor instruction, zero blocks left out.  A column walked over all 64 rows in registers takes 63 dependent steps whose
-// broadcast loads of A are bound by shared-memory wavefronts: 7300 cycles of a CTA's 28000, against 5500 of 25000 for this.
+// broadcast loads of A are bound by shared-memory wavefronts: 7300 cycles of a CTA's 28000, against 4600 - 5300 of 24400 for this.
 __device__ __forceinline__ void invert_pair(float* sA) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp < 4) {
@@ -204,7 +204,9 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
 
     grid_dep_wait();                  // set up while the kernel before drains; nothing is read or written before it has completed
     grid_dep_launch();                // the kernel after this one may set itself up while the last CTAs of this one run
-    if (tid == 0) {
+    // copies, products and coefficients start from different warps: none of them waits for another (a thread that issues
+    // copies is held up while the other CTA's stores are in the queue)
+    if (tid == 128) {
         // the call's status word starts at zero: the first CTA to start clears it, a second before any wait can expire
         if (blockIdx.x == 0) *p.status = 0;
         mbar_expect_tx(&bar_load, 2 * 32768);
@@ -218,11 +220,13 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
     // coefficients of token tid; in-chunk cumulative log-decay by a two-warp scan per chunk
     if (tid < 128) {
         // a token past the end of the sequence is an exact no-op of the recurrence: beta = 0, alpha = 1 (and q = k = v = 0)
-        const bool live = t0 + tid < p.T;
+        const bool live = t0 + tid < p.T, has_a = live && p.alpha, has_l = live && p.lam;
         const size_t crow = ((size_t)b * p.T + t0 + tid) * p.H + hh;
-        sbeta[tid] = live ? gate(__bfloat162float(p.beta[crow]), LOGITS) : 0.f;
-        slam[tid] = (live && p.lam) ? gate(__bfloat162float(p.lam[crow]), LOGITS) : 0.f;
-        float g = (live && p.alpha) ? log_gate(__bfloat162float(p.alpha[crow]), LOGITS) : 0.f;
+        const bf16 zero = __ushort_as_bfloat16(0);
+        const bf16 za = has_a ? p.alpha[crow] : zero, zb = live ? p.beta[crow] : zero, zl = has_l ? p.lam[crow] : zero;   // all in flight
+        float g = has_a ? log_gate(__bfloat162float(za), LOGITS) : 0.f;
+        sbeta[tid] = live ? gate(__bfloat162float(zb), LOGITS) : 0.f;
+        slam[tid] = has_l ? gate(__bfloat162float(zl), LOGITS) : 0.f;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const float t = __shfl_up_sync(0xffffffffu, g, o);
@@ -245,14 +249,14 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
         if (warp == 0) tmem_dealloc(tbase, 256);
         return true;
     };
-    if (expired(!mbar_wait(&bar_load, 0))) return;
-    if (tid == 0) {
+    if (tid == 160 && mbar_wait(&bar_load, 0)) {
         tc_fence_after();
         // G1 = K K^T -> columns [0,128), G2 = Q K^T -> columns [128,256)
         umma_product<false, false>(tbase + 128, smem_u32(sQ), 16384, smem_u32(sK), 16384, 128, 128, false);
         umma_product<false, false>(tbase, smem_u32(sK), 16384, smem_u32(sK), 16384, 128, 128, false);
         umma_commit(&bar_mma);
     }
+    if (expired(!mbar_wait(&bar_load, 0))) return;
     // meanwhile, row-wise, 16 lanes to a 256-byte row (chunk `ch` of 16 bytes each): Qg = gamma Q to the workspace, and X
     uint4 xr[8];
     const int ch = tid & 15, rsub = tid >> 4;
