@@ -27,7 +27,7 @@ namespace qd {
 namespace {
 
 constexpr int C = kChunk;
-constexpr int NT = 256;            // threads of every kernel here: 8 warps
+constexpr int NT = 256;            // threads of the kernels that take a chunk each: 8 warps
 constexpr int LDC = C + 4;         // leading dimension of the C x C matrices in shared memory
 constexpr int kPad = 4;            // of a d-wide tile: rows g, columns t of a fragment fall on banks 4 g + t
 
@@ -174,25 +174,25 @@ __device__ __forceinline__ float2 ld2(const __nv_bfloat16* p) {
 // A ROWS x W tile on its way from global memory (rows `stride` elements apart, rows >= live read as zeros) through
 // registers into shared memory as fp32 with leading dimension LD.  All loads of a tile are in flight together, and a
 // caller may put work between get() and put().
-template <typename IO, int ROWS, int W, int LD>
+template <typename IO, int ROWS, int W, int LD, int TH = NT>
 struct Tile {
     static constexpr int kPer = 16 / (int)sizeof(IO), kChunks = W / kPer, kTotal = ROWS * kChunks;
-    static constexpr int kN = (kTotal + NT - 1) / NT;
+    static constexpr int kN = (kTotal + TH - 1) / TH;
     uint4 r[kN];
     __device__ __forceinline__ void get(const IO* src, size_t stride, int live) {
 #pragma unroll
         for (int i = 0; i < kN; ++i) {
-            const int id = i * NT + threadIdx.x, row = id / kChunks, c = id % kChunks;
+            const int id = i * TH + threadIdx.x, row = id / kChunks, c = id % kChunks;
             r[i] = make_uint4(0, 0, 0, 0);
-            if ((kTotal % NT == 0 || id < kTotal) && row < live)
+            if ((kTotal % TH == 0 || id < kTotal) && row < live)
                 r[i] = *reinterpret_cast<const uint4*>(src + (size_t)row * stride + c * kPer);
         }
     }
     __device__ __forceinline__ void put(float* dst) const {
 #pragma unroll
         for (int i = 0; i < kN; ++i) {
-            const int id = i * NT + threadIdx.x, row = id / kChunks, c = id % kChunks;
-            if (kTotal % NT != 0 && id >= kTotal) continue;
+            const int id = i * TH + threadIdx.x, row = id / kChunks, c = id % kChunks;
+            if (kTotal % TH != 0 && id >= kTotal) continue;
             float4* d = reinterpret_cast<float4*>(dst + row * LD + c * kPer);
             if (sizeof(IO) == 4) {
                 d[0] = make_float4(__uint_as_float(r[i].x), __uint_as_float(r[i].y), __uint_as_float(r[i].z), __uint_as_float(r[i].w));
@@ -401,10 +401,12 @@ __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
 // K2: forward state chain.  One CTA per (sequence, DS-column slice of d_v); columns of the state evolve independently,
 // the chunks of a sequence are walked in order.  The next chunk's tiles are fetched into registers while the present
 // chunk is worked on: a chunk costs its two dependent products and three barriers, not its loads.
-template <typename IO, int DK, int DS>
-__global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
+template <typename IO, int DK, int DS, int TH>
+__global__ void __launch_bounds__(TH) k_chain_fwd(Ptrs p, int DV) {
     extern __shared__ float sm[];
     constexpr int LA = DK + 4, LB = DK + 8, LS = DS + 8, TI = kTerms<IO>, NS = DS / 8;
+    // the two products of a phase take half of the warps each: 64 tokens x DS columns in 16 x 8 NH, DK x DS in 16 MU x 8 NU
+    constexpr int HW = TH / 64, NH = NS / (HW / 4), MU = DK / 16 > HW ? DK / 16 / HW : 1, RU = DK / 16 / MU, NU = NS / (HW / RU);
     constexpr bool EX = TI == 2;
     float *sW = sm, *sQ = sW + C * LA, *sK = sQ + C * LA, *sP = sK + C * LB, *sU = sP + C * LDC, *sD = sU + C * LS,
           *sDs = sD + C * LS, *sh = sDs + C * LS;                     // sh: the state slice [DK][DS]
@@ -413,12 +415,12 @@ __global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
     const int tid = threadIdx.x, warp = tid >> 5;
     sm100::grid_dep_wait();            // launched while the kernel before it drains
     sm100::grid_dep_launch();
-    for (int e = tid; e < DK * DS; e += NT)
+    for (int e = tid; e < DK * DS; e += TH)
         sh[(e / DS) * LS + e % DS] = p.h0 ? p.h0[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] : 0.f;
-    Tile<IO, C, DK, LA> tw, tq;
-    Tile<IO, C, DK, LB> tk;
-    Tile<IO, C, C, LDC> tp;
-    Tile<IO, C, DS, LS> tu;
+    Tile<IO, C, DK, LA, TH> tw, tq;
+    Tile<IO, C, DK, LB, TH> tk;
+    Tile<IO, C, C, LDC, TH> tp;
+    Tile<IO, C, DS, LS, TH> tu;
     float g = 0.f, gC = 0.f, rq = 1.f, rk = 1.f;
     const size_t nrows = (size_t)p.B * H * p.Tp;
     auto fetch = [&](int n) {
@@ -444,46 +446,46 @@ __global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
         if (n + 1 < p.N) fetch(n + 1);
         if (p.save) {
             float* dst = p.hs + ((size_t)bh * p.N + n) * DK * DV + j0;
-            for (int e = tid * 4; e < DK * DS; e += NT * 4)
+            for (int e = tid * 4; e < DK * DS; e += TH * 4)
                 *reinterpret_cast<float4*>(dst + (size_t)(e / DS) * DV + e % DS) =
                     *reinterpret_cast<const float4*>(sh + (e / DS) * LS + e % DS);
         }
-        // warps 0..3: Delta = U~ - W<- h;  warps 4..7: Q h, the inter-chunk part of the output, kept in registers
-        float acc[1][NS][4];
+        // first half of the warps: Delta = U~ - W<- h;  second: Q h, the inter-chunk part of the output, kept in registers
+        float acc[1][NH][4];
         zero(acc);
-        const int m0 = (warp & 3) * 16;
+        const int m0 = (warp & 3) * 16, n0 = (warp % HW / 4) * 8 * NH;
         auto hf = [&](int i, int j) { return sh[i * LS + j]; };
-        if (warp < 4) {
-            wmm<1, NS, TI, 2, EX>(acc, m0, 0, DK, [&](int r, int i) { return sW[r * LA + i]; }, hf);
-            each(acc, m0, 0, [&](int r, int j, float x, float y) {
+        if (warp < HW) {
+            wmm<1, NH, TI, 2, EX>(acc, m0, n0, DK, [&](int r, int i) { return sW[r * LA + i]; }, hf);
+            each(acc, m0, n0, [&](int r, int j, float x, float y) {
                 x = sU[r * LS + j] - x; y = sU[r * LS + j + 1] - y;
                 st2(sD + r * LS + j, x, y);
                 st2(sDs + r * LS + j, x * sgk[r], y * sgk[r]);
                 if (p.save) st2((IO*)p.D + (wrow0 + r) * DV + j0 + j, x, y);
             });
         } else {
-            wmm<1, NS, TI, 2, EX>(acc, m0, 0, DK, [&](int r, int i) { return sQ[r * LA + i]; }, hf);
+            wmm<1, NH, TI, 2, EX>(acc, m0, n0, DK, [&](int r, int i) { return sQ[r * LA + i]; }, hf);
         }
         __syncthreads();
-        if (warp >= 4) {
+        if (warp >= HW) {
             // + P Delta, the intra-chunk part
             const int gq = (tid & 31) >> 2;
             const float s0 = sgq[m0 + gq], s1 = sgq[m0 + 8 + gq];
 #pragma unroll
-            for (int j = 0; j < NS; ++j) { acc[0][j][0] *= s0; acc[0][j][1] *= s0; acc[0][j][2] *= s1; acc[0][j][3] *= s1; }
-            wmm<1, NS, TI, 2, EX>(acc, m0, 0, C, [&](int r, int s) { return sP[r * LDC + s]; },
-                              [&](int s, int j) { return sD[s * LS + j]; });
-            each(acc, m0, 0, [&](int r, int j, float x, float y) {
+            for (int j = 0; j < NH; ++j) { acc[0][j][0] *= s0; acc[0][j][1] *= s0; acc[0][j][2] *= s1; acc[0][j][3] *= s1; }
+            wmm<1, NH, TI, 2, EX>(acc, m0, n0, C, [&](int r, int s) { return sP[r * LDC + s]; },
+                                  [&](int s, int j) { return sD[s * LS + j]; });
+            each(acc, m0, n0, [&](int r, int j, float x, float y) {
                 if (r < live) st2((IO*)p.o + (row0 + (size_t)r * H) * DV + j0 + j, x, y);
             });
         } else {
             // h <- gamma_C h + K^T (diag(gamma_C/gamma) Delta)
-            float ha[DK / 64][NS][4];
+            float ha[MU][NU][4];
             zero(ha);
-            const int i0 = warp * (DK / 4);
-            wmm<DK / 64, NS, TI, 2, EX>(ha, i0, 0, C, [&](int i, int r) { return sK[r * LB + i]; },
-                                    [&](int r, int j) { return sDs[r * LS + j]; });
-            each(ha, i0, 0, [&](int i, int j, float x, float y) {
+            const int i0 = (warp % RU) * 16 * MU, u0 = (warp / RU) * 8 * NU;
+            wmm<MU, NU, TI, 2, EX>(ha, i0, u0, C, [&](int i, int r) { return sK[r * LB + i]; },
+                                   [&](int r, int j) { return sDs[r * LS + j]; });
+            each(ha, i0, u0, [&](int i, int j, float x, float y) {
                 float* d = sh + i * LS + j;
                 st2(d, fmaf(sgC, d[0], x), fmaf(sgC, d[1], y));
             });
@@ -491,7 +493,7 @@ __global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
         __syncthreads();
     }
     if (p.hT)
-        for (int e = tid; e < DK * DS; e += NT)
+        for (int e = tid; e < DK * DS; e += TH)
             p.hT[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] = sh[(e / DS) * LS + e % DS];
 }
 
@@ -499,25 +501,27 @@ __global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
 // K3: reverse state chain.  Carries dh (gradient w.r.t. the chunk's exit state) backwards:
 //   dDelta = P^T dO + K-> dh ;   dh_in = gamma_C dh + (diag(gamma) Q)^T dO - W<-^T dDelta
 // and leaves per chunk: dh (exit), dDelta, and two scalar partial sums the decay gradient needs.
-template <typename IO, int DK, int DS>
-__global__ void __launch_bounds__(NT) k_chain_bwd(Ptrs p, int DV) {
+template <typename IO, int DK, int DS, int TH>
+__global__ void __launch_bounds__(TH) k_chain_bwd(Ptrs p, int DV) {
     extern __shared__ float sm[];
     constexpr int LA = DK + 4, LB = DK + 8, LP = C + 8, LS = DS + 8, TI = kTerms<IO>, NS = DS / 8;
+    // the two products of a phase take half of the warps each: 64 tokens x DS columns in 16 x 8 NH, DK x DS in 16 MU x 8 NU
+    constexpr int HW = TH / 64, NH = NS / (HW / 4), MU = DK / 16 > HW ? DK / 16 / HW : 1, RU = DK / 16 / MU, NU = NS / (HW / RU);
     constexpr bool EX = TI == 2;
     float *sK = sm, *sQ = sK + C * LA, *sW = sQ + C * LB, *sP = sW + C * LB, *sO = sP + C * LP, *sOs = sO + C * LS,
           *sD = sOs + C * LS, *sdD = sD + C * LS, *sdh = sdD + C * LS;
-    __shared__ float sgq[C], sgk[C], sgC, sred[NT / 32];
+    __shared__ float sgq[C], sgk[C], sgC, sred[TH / 32], skd[HW / 4][C];
     const int H = p.H, nsl = DV / DS, sl = blockIdx.x % nsl, j0 = sl * DS, bh = blockIdx.x / nsl, b = bh / H, hh = bh % H;
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t nrows = (size_t)p.B * H * p.Tp, BHN = (size_t)p.B * H * p.N;
     sm100::grid_dep_wait();            // launched while the kernel before it drains
     sm100::grid_dep_launch();
-    for (int e = tid; e < DK * DS; e += NT)
+    for (int e = tid; e < DK * DS; e += TH)
         sdh[(e / DS) * LS + e % DS] = p.dhT ? p.dhT[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] : 0.f;
-    Tile<IO, C, DK, LA> tk;
-    Tile<IO, C, DK, LB> tq, tw;
-    Tile<IO, C, C, LP> tp;
-    Tile<IO, C, DS, LS> to, td;
+    Tile<IO, C, DK, LA, TH> tk;
+    Tile<IO, C, DK, LB, TH> tq, tw;
+    Tile<IO, C, C, LP, TH> tp;
+    Tile<IO, C, DS, LS, TH> to, td;
     float g = 0.f, gC = 0.f, rq = 1.f, rk = 1.f;
     auto fetch = [&](int n) {
         const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
@@ -546,7 +550,7 @@ __global__ void __launch_bounds__(NT) k_chain_bwd(Ptrs p, int DV) {
             const float* hsrc = p.hs + ((size_t)bh * p.N + n) * DK * DV + j0;
             float part = 0.f;
 #pragma unroll 2
-            for (int e = tid * 4; e < DK * DS; e += NT * 4) {
+            for (int e = tid * 4; e < DK * DS; e += TH * 4) {
                 const size_t off = (size_t)(e / DS) * DV + e % DS;
                 const float4 x = *reinterpret_cast<const float4*>(sdh + (e / DS) * LS + e % DS);
                 const float4 y = *reinterpret_cast<const float4*>(hsrc + off);
@@ -555,7 +559,7 @@ __global__ void __launch_bounds__(NT) k_chain_bwd(Ptrs p, int DV) {
             }
             part = warp_sum(part);
             if ((tid & 31) == 0) sred[warp] = part;
-            for (int e = tid; e < C * DS; e += NT) {             // diag(gamma / |q|) dO, the operand of Q^T
+            for (int e = tid; e < C * DS; e += TH) {             // diag(gamma / |q|) dO, the operand of Q^T
                 const int r = e / DS, j = e % DS;
                 sOs[r * LS + j] = sO[r * LS + j] * sgq[r];
             }
@@ -563,48 +567,52 @@ __global__ void __launch_bounds__(NT) k_chain_bwd(Ptrs p, int DV) {
         __syncthreads();
         if (tid == 0) {
             float tot = 0.f;
-            for (int w = 0; w < NT / 32; ++w) tot += sred[w];
+            for (int w = 0; w < TH / 32; ++w) tot += sred[w];
             p.dhh[(size_t)sl * BHN + (size_t)bh * p.N + n] = tot;
         }
-        float ha[DK / 64][NS][4];
+        float ha[MU][NU][4];
         zero(ha);
-        const int i0 = (warp & 3) * (DK / 4);
-        if (warp < 4) {
+        const int hw = warp % HW, i0 = (hw % RU) * 16 * MU, u0 = (hw / RU) * 8 * NU;
+        if (warp < HW) {
             // dDelta = diag(gamma_C/gamma) K dh + P^T dO, 16 tokens per warp; row sums of the first term times Delta
-            float acc[1][NS][4];
+            float acc[1][NH][4];
             zero(acc);
-            const int m0 = warp * 16;
-            wmm<1, NS, TI, 2, EX>(acc, m0, 0, DK, [&](int s, int i) { return sK[s * LA + i]; },
-                              [&](int i, int j) { return sdh[i * LS + j]; });
+            const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 8 * NH;
+            wmm<1, NH, TI, 2, EX>(acc, m0, n0, DK, [&](int s, int i) { return sK[s * LA + i]; },
+                                  [&](int i, int j) { return sdh[i * LS + j]; });
             const int gq = (tid & 31) >> 2;
             const float s0 = sgk[m0 + gq], s1 = sgk[m0 + 8 + gq];
 #pragma unroll
-            for (int j = 0; j < NS; ++j) { acc[0][j][0] *= s0; acc[0][j][1] *= s0; acc[0][j][2] *= s1; acc[0][j][3] *= s1; }
-            row_sums(acc, m0, 0, p.kdhd + (size_t)sl * nrows + wrow0,
+            for (int j = 0; j < NH; ++j) { acc[0][j][0] *= s0; acc[0][j][1] *= s0; acc[0][j][2] *= s1; acc[0][j][3] *= s1; }
+            row_sums(acc, m0, n0, skd[warp >> 2],
                      [&](int s, int j, float x, float y) { return fmaf(x, sD[s * LS + j], y * sD[s * LS + j + 1]); });
-            wmm<1, NS, TI, TI, EX>(acc, m0, 0, C, [&](int s, int r) { return sP[r * LP + s]; },
-                               [&](int r, int j) { return sO[r * LS + j]; });
-            each(acc, m0, 0, [&](int s, int j, float x, float y) {
+            wmm<1, NH, TI, TI, EX>(acc, m0, n0, C, [&](int s, int r) { return sP[r * LP + s]; },
+                                   [&](int r, int j) { return sO[r * LS + j]; });
+            each(acc, m0, n0, [&](int s, int j, float x, float y) {
                 st2(sdD + s * LS + j, -x, -y);
                 st2((IO*)p.dD + (wrow0 + s) * DV + j0 + j, x, y);
             });
         } else {
-            wmm<DK / 64, NS, TI, 2, EX>(ha, i0, 0, C, [&](int i, int r) { return sQ[r * LB + i]; },
-                                    [&](int r, int j) { return sOs[r * LS + j]; });
+            wmm<MU, NU, TI, 2, EX>(ha, i0, u0, C, [&](int i, int r) { return sQ[r * LB + i]; },
+                                   [&](int r, int j) { return sOs[r * LS + j]; });
         }
         __syncthreads();
-        if (warp >= 4) {
-            wmm<DK / 64, NS, TI, 2, EX>(ha, i0, 0, C, [&](int i, int r) { return sW[r * LB + i]; },
-                                    [&](int r, int j) { return sdD[r * LS + j]; });
-            each(ha, i0, 0, [&](int i, int j, float x, float y) {
+        if (warp >= HW) {
+            wmm<MU, NU, TI, 2, EX>(ha, i0, u0, C, [&](int i, int r) { return sW[r * LB + i]; },
+                                   [&](int r, int j) { return sdD[r * LS + j]; });
+            each(ha, i0, u0, [&](int i, int j, float x, float y) {
                 float* d = sdh + i * LS + j;
                 st2(d, fmaf(sgC, d[0], x), fmaf(sgC, d[1], y));
             });
+        } else if (tid < C) {
+            float kd = skd[0][tid];
+            if (HW > 4) kd += skd[HW / 4 - 1][tid];
+            p.kdhd[(size_t)sl * nrows + wrow0 + tid] = kd;
         }
         __syncthreads();
     }
     if (p.dh0)
-        for (int e = tid; e < DK * DS; e += NT)
+        for (int e = tid; e < DK * DS; e += TH)
             p.dh0[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] = sdh[(e / DS) * LS + e % DS];
 }
 
@@ -899,32 +907,37 @@ Ptrs make_ptrs(const ChunkArgs& a) {
 // launched while the kernel before them drains.  Larger ones are not: CTAs that come early take the SMs that are free first
 // instead of one each, which cost 15 us on 128 chunks of 128 x 128 and 40 where two chains fit an SM.
 template <class K, class... Args>
-cudaError_t launch(K kern, int grid, size_t smem, cudaStream_t stream, Args... args) {
+cudaError_t launch(K kern, int grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
     cudaError_t e = set_max_smem_once(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
-    if (grid <= 64) return launch_overlapped(kern, dim3((unsigned)grid), dim3(NT), smem, stream, args...);
-    kern<<<grid, NT, smem, stream>>>(args...);
+    if (grid <= 64) return launch_overlapped(kern, dim3((unsigned)grid), dim3(threads), smem, stream, args...);
+    kern<<<grid, threads, smem, stream>>>(args...);
     return cudaGetLastError();
 }
 
 template <typename IO, int DK, int DV>
 cudaError_t prep_for(const ChunkArgs& a, const Ptrs& p) {
     constexpr size_t smem = sizeof(float) * (2 * C * (DK + kPad) + C * (DV + kPad) + 3 * C * LDC);
-    return launch(k_prep<IO, DK, DV>, a.s.B * a.s.H * p.N, smem, a.stream, p);
+    return launch(k_prep<IO, DK, DV>, a.s.B * a.s.H * p.N, NT, smem, a.stream, p);
 }
+// 16 warps where a chunk's products are small and its operands need little splitting: bf16, d_k = 64 (82 -> 72 and 97 -> 85 us
+// on 64 sequences of 16 chunks).  fp32 operands are split by every warp that reads them, so that 8 warps with larger tiles win
+// (52 against 48 us at d_k = 128 on 16 sequences of 8 chunks; one short call of d_k = 64, 28.7 against 27.2).
+template <typename IO, int DK> constexpr int chain_threads = sizeof(IO) == 2 && DK == 64 ? 512 : 256;
+
 template <typename IO, int DK, int DS>
 cudaError_t chain_fwd_for(const ChunkArgs& a, const Ptrs& p) {
     constexpr size_t smem = sizeof(float) * (2 * C * (DK + 4) + C * (DK + 8) + C * LDC + (3 * C + DK) * (DS + 8));
-    return launch(k_chain_fwd<IO, DK, DS>, a.s.B * a.s.H * (a.s.dv / DS), smem, a.stream, p, a.s.dv);
+    return launch(k_chain_fwd<IO, DK, DS, chain_threads<IO, DK>>, a.s.B * a.s.H * (a.s.dv / DS), chain_threads<IO, DK>, smem, a.stream, p, a.s.dv);
 }
 template <typename IO, int DK, int DS>
 cudaError_t chain_bwd_for(const ChunkArgs& a, const Ptrs& p) {
     constexpr size_t smem = sizeof(float) * (C * (DK + 4) + 2 * C * (DK + 8) + C * (C + 8) + (4 * C + DK) * (DS + 8));
-    return launch(k_chain_bwd<IO, DK, DS>, a.s.B * a.s.H * (a.s.dv / DS), smem, a.stream, p, a.s.dv);
+    return launch(k_chain_bwd<IO, DK, DS, chain_threads<IO, DK>>, a.s.B * a.s.H * (a.s.dv / DS), chain_threads<IO, DK>, smem, a.stream, p, a.s.dv);
 }
 template <typename IO, int DK, int DV>
 cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {
-    return launch(k_chunk_bwd<IO, DK, DV>, a.s.B * a.s.H * p.N, BwdSmem<DK, DV>::bytes, a.stream, p);
+    return launch(k_chunk_bwd<IO, DK, DV>, a.s.B * a.s.H * p.N, NT, BwdSmem<DK, DV>::bytes, a.stream, p);
 }
 
 typedef __nv_bfloat16 bf16;
