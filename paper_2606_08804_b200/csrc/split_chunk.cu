@@ -22,6 +22,7 @@
 #include "internal.h"
 #include "sm100.cuh"
 #include "tf32.cuh"
+#include "planes.cuh"
 
 namespace qd {
 namespace {
@@ -616,6 +617,56 @@ __global__ void __launch_bounds__(TH) k_chain_bwd(Ptrs p, int DV) {
             p.dh0[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] = sdh[(e / DS) * LS + e % DS];
 }
 
+// Per token, from the row sums (prow: dP o P, t1, t2, d beta, d lambda) and the column sums (cP: dP o P, cA: dA o A; db1: dT o M,
+// of token threadIdx.x): d beta, d lambda, and the decay gradient: dg, its reverse in-chunk cumulative sum,
+// d alpha = d log alpha / alpha.  sdg and skd are scratch.
+template <typename IO>
+__device__ __forceinline__ void token_gradients(const Ptrs& p, const float (&prow)[5][4][C], const float (&cP)[4][C],
+                                                const float (&cA)[4][C], float db1, const float* sbeta, const float* slam,
+                                                const float* salpha, const float* sgam, float* sdg, float* skd, size_t row0,
+                                                size_t wrow0, int bh, int n, int live) {
+    const int tid = threadIdx.x, H = p.H;
+    const size_t nrows = (size_t)p.B * H * p.Tp, BHN = (size_t)p.B * H * p.N;
+    if (tid < C) {
+        auto rows = [&](int w) { return prow[w][0][tid] + prow[w][1][tid] + prow[w][2][tid] + prow[w][3][tid]; };
+        const float be = sbeta[tid], la = slam[tid], db2 = rows(3), dl = rows(4);
+        float kd = 0.f;
+        for (int s = 0; s < p.nslices; ++s) kd += p.kdhd[(size_t)s * nrows + wrow0 + tid];
+        const float sP = cP[0][tid] + cP[1][tid] + cP[2][tid] + cP[3][tid];
+        const float sA = cA[0][tid] + cA[1][tid] + cA[2][tid] + cA[3][tid];
+        sdg[tid] = rows(0) - sP + be * db2 - sA + rows(1) + rows(2) - kd;
+        skd[tid] = kd;
+        if (tid < live) {
+            const size_t r = row0 + (size_t)tid * H;
+            // with logit inputs the gradients are taken w.r.t. the logits: sigmoid' = s (1 - s), (log sigmoid)' = 1 - s
+            const float db = db1 + db2;
+            p.dbeta[r] = p.logits ? db * be * (1.f - be) : db;
+            if (p.dlam) p.dlam[r] = p.logits ? dl * la * (1.f - la) : dl;
+        }
+    }
+    __syncthreads();
+    if (tid < 32 && p.dalpha) {
+        // lane owns tokens 2 lane, 2 lane + 1; d log alpha_i = sum_{r >= i} dg_r (suffix sums)
+        float dhh = 0.f, kds = skd[2 * tid] + skd[2 * tid + 1];
+        if (tid < p.nslices) dhh = p.dhh[(size_t)tid * BHN + (size_t)bh * p.N + n];
+        dhh = warp_sum(dhh);
+        kds = warp_sum(kds);
+        const float a = sdg[2 * tid];
+        float b2 = sdg[2 * tid + 1];
+        if (tid == 31) b2 += sgam[C - 1] * dhh + kds;
+        float sfx = a + b2;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float t = __shfl_down_sync(0xffffffffu, sfx, o);
+            if (tid + o < 32) sfx += t;
+        }
+        const size_t r = row0 + (size_t)(2 * tid) * H;
+        const float a0 = salpha[2 * tid], a1 = salpha[2 * tid + 1];
+        if (2 * tid < live) p.dalpha[r] = p.logits ? sfx * (1.f - a0) : sfx / a0;
+        if (2 * tid + 1 < live) p.dalpha[r + H] = p.logits ? (sfx - a) * (1.f - a1) : (sfx - a) / a1;
+    }
+}
+
 // ---------------------------------------------------------------------------------------------
 // K4: chunk-parallel part of the backward: dq, dk, dv, dbeta, dlambda, dalpha.  The 64 x d_k results dX, dq and dk stay in
 // registers from their first product to their store (each warp owns the same 32 x d_k/4 tile of all three); four tile
@@ -626,8 +677,9 @@ struct BwdSmem {
     static constexpr int kSlot = C * LT;
     static constexpr size_t bytes = sizeof(float) * (4 * kSlot + 5 * C * LDC);
 };
-template <typename IO, int DK, int DV>
+template <int DK, int DV>
 __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
+    typedef float IO;
     extern __shared__ float sm[];
     constexpr int LT = BwdSmem<DK, DV>::LT, LH = DV + kPad, TI = kTerms<IO>, kSlot = BwdSmem<DK, DV>::kSlot, NK = DK / 32;
     constexpr bool EX = TI == 2;
@@ -644,7 +696,7 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     const int H = p.H, ch = blockIdx.x, n = ch % p.N, bh = ch / p.N, b = bh / H, hh = bh % H;
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
-    const size_t nrows = (size_t)p.B * H * p.Tp, BHN = (size_t)p.B * H * p.N;
+    const size_t nrows = (size_t)p.B * H * p.Tp;
     const int live = min(C, p.T - n * C);
     const float* hs = p.hs + ((size_t)bh * p.N + n) * DK * DV;
     const float* dhs = p.dhs + ((size_t)bh * p.N + n) * DK * DV;
@@ -835,7 +887,6 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     }
     each(aK, wm, nk, [&](int r, int i, float x, float y) { if (r < live) st2((IO*)p.dk_ + (row0 + (size_t)r * H) * DK + i, x, y); });
     each(aQ, wm, nk, [&](int r, int i, float x, float y) { if (r < live) st2((IO*)p.dq + (row0 + (size_t)r * H) * DK + i, x, y); });
-    // ---- decay gradient: dg, reverse in-chunk cumulative sum, d alpha = d log alpha / alpha -------------
     __syncthreads();
     {
         const int col = tid & 63, q4 = tid >> 6;
@@ -845,44 +896,246 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
         part[q4][col] = s;
     }
     __syncthreads();
-    if (tid < C) {
-        auto rows = [&](int w) { return prow[w][0][tid] + prow[w][1][tid] + prow[w][2][tid] + prow[w][3][tid]; };
-        const float be = sbeta[tid], la = slam[tid], db2 = rows(3), dl = rows(4);
-        float kd = 0.f;
-        for (int s = 0; s < p.nslices; ++s) kd += p.kdhd[(size_t)s * nrows + wrow0 + tid];
-        const float cP = pcol[0][tid] + pcol[1][tid] + pcol[2][tid] + pcol[3][tid];
-        const float cA = part[0][tid] + part[1][tid] + part[2][tid] + part[3][tid];
-        sdg[tid] = rows(0) - cP + be * db2 - cA + rows(1) + rows(2) - kd;
-        skd[tid] = kd;
-        if (tid < live) {
-            const size_t r = row0 + (size_t)tid * H;
-            // with logit inputs the gradients are taken w.r.t. the logits: sigmoid' = s (1 - s), (log sigmoid)' = 1 - s
-            const float db = db1 + db2;
-            p.dbeta[r] = p.logits ? db * be * (1.f - be) : db;
-            if (p.dlam) p.dlam[r] = p.logits ? dl * la * (1.f - la) : dl;
-        }
-    }
-    __syncthreads();
-    if (tid < 32 && p.dalpha) {
-        // lane owns tokens 2 lane, 2 lane + 1; d log alpha_i = sum_{r >= i} dg_r (suffix sums)
-        float dhh = 0.f, kds = skd[2 * tid] + skd[2 * tid + 1];
-        if (tid < p.nslices) dhh = p.dhh[(size_t)tid * BHN + (size_t)bh * p.N + n];
-        dhh = warp_sum(dhh);
-        kds = warp_sum(kds);
-        const float a = sdg[2 * tid];
-        float b2 = sdg[2 * tid + 1];
-        if (tid == 31) b2 += sgam[C - 1] * dhh + kds;
-        float sfx = a + b2;
+    token_gradients<IO>(p, prow, pcol, part, db1, sbeta, slam, salpha, sgam, sdg, skd, row0, wrow0, bh, n, live);
+}
+
+// The same for bf16 storage, on bf16 planes: 16 warps, each a 16 x d/4 tile of every product.  X is never formed: a product
+// with it is one with K and one with Q, which are exact in one plane, their coefficients applied to the result or to the
+// other operand.  One slot of shared memory holds dh, h and dW<- in turn; Delta's, V's and dO's room is used again for the
+// smaller matrices.  B4 T1024 H16 d_k = d_v = 64: 208 us with tf32 halves, @@ so, bound by latency between its barriers.
+template <int DK, int DV>
+struct BwdPlanes {
+    typedef Planes<C, DK, 1> TQ;
+    typedef Planes<C, DV, 1> TV;
+    typedef Planes<DK, DV, 3> TS;
+    typedef Planes<C, DK, 3> TW;
+    typedef Planes<C, C, 3> TC;
+    static constexpr int kV = 2 * TQ::kBytes, kS = kV + 4 * TV::kBytes, kM = kS + (TS::kBytes > TW::kBytes ? TS::kBytes : TW::kBytes),
+                         kT = kM + TC::kBytes, kBytes = kT + TC::kBytes, kE = kBytes - 4 * TC::kBytes;
+    static_assert(TC::kBytes <= 3 * TV::kBytes && kE >= kV, "reused room");
+};
+template <int DK, int DV>
+__global__ void __launch_bounds__(512) k_chunk_bwd_planes(Ptrs p) {
+    extern __shared__ __align__(16) unsigned char smb[];
+    typedef BwdPlanes<DK, DV> L;
+    typedef __nv_bfloat16 IO;
+    constexpr int TH = 512, NK = DK / 32, NV = DV / 32;
+    const typename L::TQ mQ(smb), mK(smb + L::TQ::kBytes);
+    const typename L::TV mO(smb + L::kV), mD(smb + L::kV + L::TV::kBytes), mdD(smb + L::kV + 2 * L::TV::kBytes), mV(smb + L::kV + 3 * L::TV::kBytes);
+    const typename L::TS mS(smb + L::kS);
+    const typename L::TW mW(smb + L::kS);
+    const typename L::TC mM(smb + L::kM), mT(smb + L::kT), m4(smb + L::kV);
+    __shared__ float sbeta[C], slam[C], salpha[C], sg[C], sgam[C], segc[C], srq[C], srk[C], scq[C];
+    __shared__ float sdg[C], skd[C], part[4][C], prow[5][4][C];   // prow: row sums by warp column: dP o P, t1, t2, d beta, d lambda
+    __shared__ float pcol[3][4][C];                               // column sums by warp row: dP o P, dT o M, dA o A
+    const int H = p.H, ch = blockIdx.x, n = ch % p.N, bh = ch / p.N, b = bh / H, hh = bh % H;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
+    const size_t nrows = (size_t)p.B * H * p.Tp;
+    const int live = min(C, p.T - n * C);
+    const int wr = warp & 3, wm = wr * 16, wn = warp >> 2, nc = wn * 16, nk = wn * (DK / 4), nv = wn * (DV / 4);
+    // sums over this warp's 16 rows of each of its 16 columns, to dst[column]
+    auto col_sums = [&](float (&a)[1][2][4], float* dst) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float t = __shfl_down_sync(0xffffffffu, sfx, o);
-            if (tid + o < 32) sfx += t;
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float s = a[0][j][e] + a[0][j][e + 2];
+                s += __shfl_xor_sync(0xffffffffu, s, 4);
+                s += __shfl_xor_sync(0xffffffffu, s, 8);
+                s += __shfl_xor_sync(0xffffffffu, s, 16);
+                if (lane < 4) dst[nc + 8 * j + 2 * lane + e] = s;
+            }
+    };
+    sm100::grid_dep_wait();            // launched while the kernel before it drains
+    sm100::grid_dep_launch();
+    // ---- everything that the chunk reads, but the entry state, in flight together ----------------
+    mQ.template fetch<TH>((const IO*)p.q + row0 * DK, (size_t)H * DK, live);
+    mK.template fetch<TH>((const IO*)p.k + row0 * DK, (size_t)H * DK, live);
+    mO.template fetch<TH>((const IO*)p.dO + row0 * DV, (size_t)H * DV, live);
+    mD.template fetch<TH>((const IO*)p.D + wrow0 * DV, DV, C);
+    mdD.template fetch<TH>((const IO*)p.dD + wrow0 * DV, DV, C);
+    mV.template fetch<TH>((const IO*)p.v + row0 * DV, (size_t)H * DV, live);
+    float2 pv[2][2];                                              // P at this thread's elements
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) pv[h][j] = ld2((const IO*)p.P + (wrow0 + wm + 8 * h + (lane >> 2)) * C + nc + 8 * j + 2 * (lane & 3));
+    FloatTile<DK, DV, TH> th;
+    {
+        FloatTile<C, C, TH> tm;
+        th.get(p.dhs + ((size_t)bh * p.N + n) * DK * DV);
+        tm.get(p.M + wrow0 * C);
+        if (tid < C) {
+            const size_t r = row0 + (size_t)tid * H;
+            const bool in = tid < live;
+            const float g = p.g[wrow0 + tid], gC = p.g[wrow0 + C - 1];
+            sbeta[tid] = in ? gate(ld((const IO*)p.beta, r), p.logits) : 0.f;
+            const float lm = (in && p.lam) ? gate(ld((const IO*)p.lam, r), p.logits) : 0.f;
+            salpha[tid] = (in && p.alpha) ? gate(ld((const IO*)p.alpha, r), p.logits) : 1.f;
+            const float rq = p.rqk ? p.rqk[wrow0 + tid] : 1.f, rk = p.rqk ? p.rqk[nrows + wrow0 + tid] : 1.f;
+            slam[tid] = lm; sg[tid] = g; sgam[tid] = expf(g); segc[tid] = expf(gC - g);
+            srq[tid] = rq; srk[tid] = rk; scq[tid] = lm * rq;
         }
-        const size_t r = row0 + (size_t)(2 * tid) * H;
-        const float a0 = salpha[2 * tid], a1 = salpha[2 * tid + 1];
-        if (2 * tid < live) p.dalpha[r] = p.logits ? sfx * (1.f - a0) : sfx / a0;
-        if (2 * tid + 1 < live) p.dalpha[r + H] = p.logits ? (sfx - a) * (1.f - a1) : (sfx - a) / a1;
+        th.put(mS);
+        tm.put(mM);
     }
+    th.get(p.hs + ((size_t)bh * p.N + n) * DK * DV);
+    fetch_wait();
+    __syncthreads();
+    // ---- dP with its uses: dP o P (row and column sums), dP o Gamma;  dk <- diag(gamma_C/gamma) Delta dh^T ----
+    float a3[1][2][4], aK[1][NK][4], aQ[1][NK][4], aX[1][NK][4];
+    zero(a3); zero(aK); zero(aQ); zero(aX);
+    pmm<false, false>(a3, mO, mD, wm, nc, DV);
+    {
+        float a[1][2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int r = wm + 8 * h + (lane >> 2), s = nc + 8 * j + 2 * (lane & 3);
+                const float d0 = s <= r ? a3[0][j][2 * h] : 0.f, d1 = s + 1 <= r ? a3[0][j][2 * h + 1] : 0.f;
+                a[0][j][2 * h] = d0 * pv[h][j].x; a[0][j][2 * h + 1] = d1 * pv[h][j].y;
+                a3[0][j][2 * h] = s <= r ? d0 * expf(sg[r] - sg[s]) : 0.f;
+                a3[0][j][2 * h + 1] = s + 1 <= r ? d1 * expf(sg[r] - sg[s + 1]) : 0.f;
+            }
+        col_sums(a, pcol[0][wr]);
+        row_sums(a, wm, nc, prow[0][wn], [&](int, int, float x, float y) { return x + y; });
+    }
+    pmm<false, false>(aK, mD, mS, wm, nk, DV);
+    each(aK, wm, nk, [&](int r, int, float& x, float& y) { x *= segc[r]; y *= segc[r]; });
+    __syncthreads();                                            // dh has been read
+    th.put(mS);
+    __syncthreads();
+    // ---- dq <- diag(gamma) dO h^T;  dW<- = -dDelta h^T;  dT = dDelta V^T + ...;  dV = T^T dDelta ------------
+    float aT[1][2][4];
+    zero(aT);
+    pmm<false, false>(aQ, mO, mS, wm, nk, DV);
+    pmm<false, false>(aX, mdD, mS, wm, nk, DV);
+    pmm<false, false>(aT, mdD, mV, wm, nc, DV);
+    {
+        float a[1][NV][4];
+        zero(a);
+        pmm<true, true>(a, mM, mdD, wm, nv, C);
+        each(a, wm, nv, [&](int s, int j, float x, float y) {
+            if (s < live) st2((IO*)p.dv_ + (row0 + (size_t)s * H) * DV + j, sbeta[s] * x, sbeta[s] * y);
+        });
+    }
+    each(aQ, wm, nk, [&](int r, int, float& x, float& y) { x *= sgam[r]; y *= sgam[r]; });
+    auto qsum = [&](int r, int i, float x, float y) { const float2 q = mQ.ld2(r, i); return srq[r] * fmaf(x, q.x, y * q.y); };
+    auto ksum = [&](int r, int i, float x, float y) { const float2 k = mK.ld2(r, i); return srk[r] * fmaf(x, k.x, y * k.y); };
+    row_sums(aQ, wm, nk, prow[1][wn], qsum);                    // t1 = <dQ1, Q>
+    __syncthreads();                                            // h has been read
+    each(aX, wm, nk, [&](int r, int i, float x, float y) { mW.st2(r, i, -x, -y); });
+    __syncthreads();
+    // ---- ... + dW<- (gamma X)^T;  d beta from T;  dX <- diag(gamma) T^T dW<-;  t2 = <dXg, gamma X> ----------
+    {
+        float a1[1][2][4], a2[1][2][4];
+        zero(a1); zero(a2);
+        pmm<false, false>(a1, mW, mK, wm, nc, DK);
+        pmm<false, false>(a2, mW, mQ, wm, nc, DK);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int s = nc + 8 * j + 2 * (lane & 3) + (e & 1);
+                aT[0][j][e] = fmaf(sgam[s], fmaf(srk[s], a1[0][j][e], scq[s] * a2[0][j][e]), aT[0][j][e]);
+            }
+        each(aT, wm, nc, [&](int r, int s, float& x, float& y) {
+            const float2 m = mM.ld2(r, s);
+            mT.st2(r, s, x * sbeta[s], y * sbeta[s + 1]);
+            x *= m.x; y *= m.y;
+        });
+        col_sums(aT, pcol[1][wr]);
+    }
+    zero(aX);
+    pmm<true, true>(aX, mM, mW, wm, nk, C);
+    each(aX, wm, nk, [&](int s, int, float& x, float& y) { const float f = sbeta[s] * sgam[s]; x *= f; y *= f; });
+    row_sums(aX, wm, nk, prow[2][wn], [&](int r, int i, float x, float y) {
+        const float2 k = mK.ld2(r, i), q = mQ.ld2(r, i);
+        return fmaf(x, fmaf(scq[r], q.x, srk[r] * k.x), y * fmaf(scq[r], q.y, srk[r] * k.y));
+    });
+    __syncthreads();                                            // dT diag(beta) is complete
+    // ---- dA = -strictLower(M^T (dT diag(beta) M^T)) -------------------------------------------------
+    {
+        float a[1][2][4];
+        zero(a);
+        pmm<false, false>(a, mT, mM, wm, nc, C);
+        each(a, wm, nc, [&](int r, int s, float x, float y) { m4.st2(r, s, x, y); });
+    }
+    float kk[1][2][4], qk[1][2][4];
+    zero(kk); zero(qk);
+    pmm<false, false>(kk, mK, mK, wm, nc, DK);
+    pmm<false, false>(qk, mQ, mK, wm, nc, DK);
+    __syncthreads();
+    {
+        float a[1][2][4];
+        zero(a);
+        pmm<true, true>(a, mM, m4, wm, nc, C);
+        __syncthreads();                                        // M and dT M^T have been read: dX K^T and dP o Gamma over them
+        // the uses of dA: d beta (row sums), dA o A (column sums), d(X K^T)
+        const typename L::TC e1(smb + L::kE), e2(smb + L::kE + L::TC::kBytes), e3(smb + L::kE + 2 * L::TC::kBytes), e4(smb + L::kE + 3 * L::TC::kBytes);
+        float ca[1][2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int r = wm + 8 * h + (lane >> 2), s = nc + 8 * j + 2 * (lane & 3);
+                const float be = sbeta[r], cq = scq[r], ck = srk[r], rq = srq[r];
+                float d[2], f[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float x = s + e < r ? -a[0][j][2 * h + e] * expf(sg[r] - sg[s + e]) : 0.f;
+                    const float xk = srk[s + e] * fmaf(ck, kk[0][j][2 * h + e], cq * qk[0][j][2 * h + e]);
+                    a[0][j][2 * h + e] = x * xk;
+                    ca[0][j][2 * h + e] = be * x * xk;
+                    d[e] = be * x; f[e] = a3[0][j][2 * h + e];
+                }
+                e1.st2(r, s, d[0] * srk[s], d[1] * srk[s + 1]);
+                e2.st2(r, s, f[0] * srk[s], f[1] * srk[s + 1]);
+                e3.st2(r, s, fmaf(cq, d[0], rq * f[0]), fmaf(cq, d[1], rq * f[1]));
+                if (p.rqk) e4.st2(r, s, d[0] * ck, d[1] * ck);
+            }
+        row_sums(a, wm, nc, prow[3][wn], [&](int, int, float x, float y) { return x + y; });
+        col_sums(ca, pcol[2][wr]);
+        __syncthreads();
+        // ---- dX += dXK K;  dk += dXK^T X + dPG^T Q + dX;  dq += dPG K + lambda dX ----------------------
+        pmm<false, true>(aX, e1, mK, wm, nk, C);
+        row_sums(aX, wm, nk, prow[4][wn], qsum);
+        pmm<false, true>(aQ, e2, mK, wm, nk, C);
+        pmm<true, true>(aK, e3, mQ, wm, nk, C);
+        pmm<true, true>(aK, p.rqk ? e4 : e1, mK, wm, nk, C);
+    }
+#pragma unroll
+    for (int j = 0; j < NK; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            aK[0][j][e] += aX[0][j][e];
+            aQ[0][j][e] = fmaf(slam[wm + 8 * (e >> 1) + (lane >> 2)], aX[0][j][e], aQ[0][j][e]);
+        }
+    if (p.rqk) {
+        // through the normalisation: dx = r (dx^ - x^ <x^, dx^>)
+        row_sums(aQ, wm, nk, part[wn], qsum);
+        __syncthreads();
+        each(aQ, wm, nk, [&](int r, int i, float& x, float& y) {
+            const float c = part[0][r] + part[1][r] + part[2][r] + part[3][r], f = srq[r];
+            const float2 q = mQ.ld2(r, i);
+            x = f * fmaf(-c * f, q.x, x); y = f * fmaf(-c * f, q.y, y);
+        });
+        __syncthreads();
+        row_sums(aK, wm, nk, part[wn], ksum);
+        __syncthreads();
+        each(aK, wm, nk, [&](int r, int i, float& x, float& y) {
+            const float c = part[0][r] + part[1][r] + part[2][r] + part[3][r], f = srk[r];
+            const float2 k = mK.ld2(r, i);
+            x = f * fmaf(-c * f, k.x, x); y = f * fmaf(-c * f, k.y, y);
+        });
+    }
+    each(aK, wm, nk, [&](int r, int i, float x, float y) { if (r < live) st2((IO*)p.dk_ + (row0 + (size_t)r * H) * DK + i, x, y); });
+    each(aQ, wm, nk, [&](int r, int i, float x, float y) { if (r < live) st2((IO*)p.dq + (row0 + (size_t)r * H) * DK + i, x, y); });
+    __syncthreads();
+    const float db1 = tid < C ? pcol[1][0][tid] + pcol[1][1][tid] + pcol[1][2][tid] + pcol[1][3][tid] : 0.f;
+    token_gradients<IO>(p, prow, pcol[0], pcol[2], db1, sbeta, slam, salpha, sgam, sdg, skd, row0, wrow0, bh, n, live);
 }
 
 Ptrs make_ptrs(const ChunkArgs& a) {
@@ -937,7 +1190,11 @@ cudaError_t chain_bwd_for(const ChunkArgs& a, const Ptrs& p) {
 }
 template <typename IO, int DK, int DV>
 cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {
-    return launch(k_chunk_bwd<IO, DK, DV>, a.s.B * a.s.H * p.N, NT, BwdSmem<DK, DV>::bytes, a.stream, p);
+    if constexpr (sizeof(IO) == 2) {
+        return launch(k_chunk_bwd_planes<DK, DV>, a.s.B * a.s.H * p.N, 512, BwdPlanes<DK, DV>::kBytes, a.stream, p);
+    } else {
+        return launch(k_chunk_bwd<DK, DV>, a.s.B * a.s.H * p.N, NT, BwdSmem<DK, DV>::bytes, a.stream, p);
+    }
 }
 
 typedef __nv_bfloat16 bf16;
