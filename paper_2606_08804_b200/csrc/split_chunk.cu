@@ -144,6 +144,18 @@ __device__ __forceinline__ void each(float (&acc)[MT][NTL][4], int m0, int n0, F
 #pragma unroll
             for (int j = 0; j < NTL; ++j) f(m0 + 16 * i + 8 * h + g, n0 + 8 * j + 2 * t, acc[i][j][2 * h], acc[i][j][2 * h + 1]);
 }
+// f(row, column, value pair of a, value pair of b) over two accumulators of the same tile
+template <int MT, int NTL, class F>
+__device__ __forceinline__ void each2(float (&a)[MT][NTL][4], float (&b)[MT][NTL][4], int m0, int n0, F f) {
+    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < NTL; ++j)
+                f(m0 + 16 * i + 8 * h + g, n0 + 8 * j + 2 * t, a[i][j][2 * h], a[i][j][2 * h + 1], b[i][j][2 * h], b[i][j][2 * h + 1]);
+}
 // Row sums over a warp's tile: f(row, column, x0, x1) gives what the pair adds; the sum over the warp's columns of row r
 // goes to dst[r] (one lane of four writes).
 template <int MT, int NTL, class F>
@@ -620,9 +632,9 @@ __global__ void __launch_bounds__(TH) k_chain_bwd(Ptrs p, int DV) {
 // Per token, from the row sums (prow: dP o P, t1, t2, d beta, d lambda) and the column sums (cP: dP o P, cA: dA o A; db1: dT o M,
 // of token threadIdx.x): d beta, d lambda, and the decay gradient: dg, its reverse in-chunk cumulative sum,
 // d alpha = d log alpha / alpha.  sdg and skd are scratch.
-template <typename IO>
-__device__ __forceinline__ void token_gradients(const Ptrs& p, const float (&prow)[5][4][C], const float (&cP)[4][C],
-                                                const float (&cA)[4][C], float db1, const float* sbeta, const float* slam,
+template <typename IO, int NC>
+__device__ __forceinline__ void token_gradients(const Ptrs& p, const float (&prow)[5][4][C], const float (&cP)[NC][C],
+                                                const float (&cA)[NC][C], float db1, const float* sbeta, const float* slam,
                                                 const float* salpha, const float* sgam, float* sdg, float* skd, size_t row0,
                                                 size_t wrow0, int bh, int n, int live) {
     const int tid = threadIdx.x, H = p.H;
@@ -632,8 +644,9 @@ __device__ __forceinline__ void token_gradients(const Ptrs& p, const float (&pro
         const float be = sbeta[tid], la = slam[tid], db2 = rows(3), dl = rows(4);
         float kd = 0.f;
         for (int s = 0; s < p.nslices; ++s) kd += p.kdhd[(size_t)s * nrows + wrow0 + tid];
-        const float sP = cP[0][tid] + cP[1][tid] + cP[2][tid] + cP[3][tid];
-        const float sA = cA[0][tid] + cA[1][tid] + cA[2][tid] + cA[3][tid];
+        float sP = 0.f, sA = 0.f;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) { sP += cP[c][tid]; sA += cA[c][tid]; }
         sdg[tid] = rows(0) - sP + be * db2 - sA + rows(1) + rows(2) - kd;
         skd[tid] = kd;
         if (tid < live) {
@@ -899,10 +912,12 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     token_gradients<IO>(p, prow, pcol, part, db1, sbeta, slam, salpha, sgam, sdg, skd, row0, wrow0, bh, n, live);
 }
 
-// The same for bf16 storage, on bf16 planes: 16 warps, each a 16 x d/4 tile of every product.  X is never formed: a product
-// with it is one with K and one with Q, which are exact in one plane, their coefficients applied to the result or to the
-// other operand.  One slot of shared memory holds dh, h and dW<- in turn; Delta's, V's and dO's room is used again for the
-// smaller matrices.  B4 T1024 H16 d_k = d_v = 64: 208 us with tf32 halves, @@ so, bound by latency between its barriers.
+// The same for bf16 storage, on bf16 planes.  X is never formed: a product with it is one with K and one with Q, which are
+// exact in one plane, their coefficients applied to the result or to the other operand.  One slot of shared memory holds dh,
+// h, dW<- and dT M^T in turn; M takes Delta's place, dT that of dO, dDelta and V.  So two CTAs fit an SM at d_k = d_v = 64: one
+// computes while the other loads or waits at a barrier, and a warp's 32 x 16 tile reads 1.5 operand pieces per 16 x 16 x 16
+// product, half of what 16 x 16 tiles of 16 warps would.  B4 T1024 H16 d_k = d_v = 64: 208 us with tf32 halves, 150 with 16
+// warps and one CTA, 122 so.
 template <int DK, int DV>
 struct BwdPlanes {
     typedef Planes<C, DK, 1> TQ;
@@ -910,37 +925,41 @@ struct BwdPlanes {
     typedef Planes<DK, DV, 3> TS;
     typedef Planes<C, DK, 3> TW;
     typedef Planes<C, C, 3> TC;
-    static constexpr int kV = 2 * TQ::kBytes, kS = kV + 4 * TV::kBytes, kM = kS + (TS::kBytes > TW::kBytes ? TS::kBytes : TW::kBytes),
-                         kT = kM + TC::kBytes, kBytes = kT + TC::kBytes, kE = kBytes - 4 * TC::kBytes;
-    static_assert(TC::kBytes <= 3 * TV::kBytes && kE >= kV, "reused room");
+    static constexpr int kV = 2 * TQ::kBytes, kS = kV + 3 * TV::kBytes, kM = kS + (TS::kBytes > TW::kBytes ? TS::kBytes : TW::kBytes),
+                         kBytes = kM + TC::kBytes;
+    static_assert(TV::kBytes <= TC::kBytes && TC::kBytes <= 3 * TV::kBytes && TC::kBytes <= kM - kS && kV + 3 * TC::kBytes <= kBytes, "reused room");
+    // where two CTAs fit: 32 x 16 tiles of 8 warps; one CTA: 16 warps hide more (d 128 and 64: 202 against 207 us, normalised 217, 233)
+    static constexpr int kCtas = kBytes <= 100 * 1024 ? 2 : 1, kThreads = kCtas == 2 ? 256 : 512;
 };
 template <int DK, int DV>
-__global__ void __launch_bounds__(512) k_chunk_bwd_planes(Ptrs p) {
+__global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>::kCtas) k_chunk_bwd_planes(Ptrs p) {
     extern __shared__ __align__(16) unsigned char smb[];
     typedef BwdPlanes<DK, DV> L;
     typedef __nv_bfloat16 IO;
-    constexpr int TH = 512, NK = DK / 32, NV = DV / 32;
+    constexpr int TH = L::kThreads, MT = 512 / TH, NK = DK / 32, NV = DV / 32, WR = 4 / MT;      // WR x 4 warps of 16 MT rows
     const typename L::TQ mQ(smb), mK(smb + L::TQ::kBytes);
-    const typename L::TV mO(smb + L::kV), mD(smb + L::kV + L::TV::kBytes), mdD(smb + L::kV + 2 * L::TV::kBytes), mV(smb + L::kV + 3 * L::TV::kBytes);
+    const typename L::TV mO(smb + L::kV), mdD(smb + L::kV + L::TV::kBytes), mV(smb + L::kV + 2 * L::TV::kBytes), mD(smb + L::kM);
     const typename L::TS mS(smb + L::kS);
     const typename L::TW mW(smb + L::kS);
-    const typename L::TC mM(smb + L::kM), mT(smb + L::kT), m4(smb + L::kV);
+    const typename L::TC mM(smb + L::kM), mT(smb + L::kV), m4(smb + L::kS);
     __shared__ float sbeta[C], slam[C], salpha[C], sg[C], sgam[C], segc[C], srq[C], srk[C], scq[C];
     __shared__ float sdg[C], skd[C], part[4][C], prow[5][4][C];   // prow: row sums by warp column: dP o P, t1, t2, d beta, d lambda
-    __shared__ float pcol[3][4][C];                               // column sums by warp row: dP o P, dT o M, dA o A
+    __shared__ float pcol[3][WR][C];                              // column sums by warp row: dP o P, dT o M, dA o A
     const int H = p.H, ch = blockIdx.x, n = ch % p.N, bh = ch / p.N, b = bh / H, hh = bh % H;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
     const size_t nrows = (size_t)p.B * H * p.Tp;
     const int live = min(C, p.T - n * C);
-    const int wr = warp & 3, wm = wr * 16, wn = warp >> 2, nc = wn * 16, nk = wn * (DK / 4), nv = wn * (DV / 4);
-    // sums over this warp's 16 rows of each of its 16 columns, to dst[column]
-    auto col_sums = [&](float (&a)[1][2][4], float* dst) {
+    const int wr = warp % WR, wm = wr * 16 * MT, wn = warp / WR, nc = wn * 16, nk = wn * (DK / 4), nv = wn * (DV / 4);
+    // sums over this warp's rows of each of its 16 columns, to dst[column]
+    auto col_sums = [&](float (&a)[MT][2][4], float* dst) {
 #pragma unroll
         for (int j = 0; j < 2; ++j)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                float s = a[0][j][e] + a[0][j][e + 2];
+                float s = 0.f;
+#pragma unroll
+                for (int i = 0; i < MT; ++i) s += a[i][j][e] + a[i][j][e + 2];
                 s += __shfl_xor_sync(0xffffffffu, s, 4);
                 s += __shfl_xor_sync(0xffffffffu, s, 8);
                 s += __shfl_xor_sync(0xffffffffu, s, 16);
@@ -956,16 +975,10 @@ __global__ void __launch_bounds__(512) k_chunk_bwd_planes(Ptrs p) {
     mD.template fetch<TH>((const IO*)p.D + wrow0 * DV, DV, C);
     mdD.template fetch<TH>((const IO*)p.dD + wrow0 * DV, DV, C);
     mV.template fetch<TH>((const IO*)p.v + row0 * DV, (size_t)H * DV, live);
-    float2 pv[2][2];                                              // P at this thread's elements
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) pv[h][j] = ld2((const IO*)p.P + (wrow0 + wm + 8 * h + (lane >> 2)) * C + nc + 8 * j + 2 * (lane & 3));
     FloatTile<DK, DV, TH> th;
+    FloatTile<C, C, TH> tm;
+    th.get(p.dhs + ((size_t)bh * p.N + n) * DK * DV);
     {
-        FloatTile<C, C, TH> tm;
-        th.get(p.dhs + ((size_t)bh * p.N + n) * DK * DV);
-        tm.get(p.M + wrow0 * C);
         if (tid < C) {
             const size_t r = row0 + (size_t)tid * H;
             const bool in = tid < live;
@@ -977,44 +990,49 @@ __global__ void __launch_bounds__(512) k_chunk_bwd_planes(Ptrs p) {
             slam[tid] = lm; sg[tid] = g; sgam[tid] = expf(g); segc[tid] = expf(gC - g);
             srq[tid] = rq; srk[tid] = rk; scq[tid] = lm * rq;
         }
-        th.put(mS);
-        tm.put(mM);
     }
+    th.put(mS);
     th.get(p.hs + ((size_t)bh * p.N + n) * DK * DV);
+    tm.get(p.M + wrow0 * C);
     fetch_wait();
     __syncthreads();
     // ---- dP with its uses: dP o P (row and column sums), dP o Gamma;  dk <- diag(gamma_C/gamma) Delta dh^T ----
-    float a3[1][2][4], aK[1][NK][4], aQ[1][NK][4], aX[1][NK][4];
+    float a3[MT][2][4], aK[MT][NK][4], aQ[MT][NK][4], aX[MT][NK][4];
     zero(a3); zero(aK); zero(aQ); zero(aX);
     pmm<false, false>(a3, mO, mD, wm, nc, DV);
     {
-        float a[1][2][4];
+        float a[MT][2][4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int i = 0; i < MT; ++i)
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int r = wm + 8 * h + (lane >> 2), s = nc + 8 * j + 2 * (lane & 3);
-                const float d0 = s <= r ? a3[0][j][2 * h] : 0.f, d1 = s + 1 <= r ? a3[0][j][2 * h + 1] : 0.f;
-                a[0][j][2 * h] = d0 * pv[h][j].x; a[0][j][2 * h + 1] = d1 * pv[h][j].y;
-                a3[0][j][2 * h] = s <= r ? d0 * expf(sg[r] - sg[s]) : 0.f;
-                a3[0][j][2 * h + 1] = s + 1 <= r ? d1 * expf(sg[r] - sg[s + 1]) : 0.f;
-            }
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int r = wm + 16 * i + 8 * h + (lane >> 2), s = nc + 8 * j + 2 * (lane & 3);
+                    float *d = a3[i][j] + 2 * h, *o = a[i][j] + 2 * h;
+                    const float2 pv = ld2((const IO*)p.P + (wrow0 + r) * C + s);
+                    const float d0 = s <= r ? d[0] : 0.f, d1 = s + 1 <= r ? d[1] : 0.f;
+                    o[0] = d0 * pv.x; o[1] = d1 * pv.y;
+                    d[0] = s <= r ? d0 * expf(sg[r] - sg[s]) : 0.f;
+                    d[1] = s + 1 <= r ? d1 * expf(sg[r] - sg[s + 1]) : 0.f;
+                }
         col_sums(a, pcol[0][wr]);
         row_sums(a, wm, nc, prow[0][wn], [&](int, int, float x, float y) { return x + y; });
     }
     pmm<false, false>(aK, mD, mS, wm, nk, DV);
     each(aK, wm, nk, [&](int r, int, float& x, float& y) { x *= segc[r]; y *= segc[r]; });
-    __syncthreads();                                            // dh has been read
+    __syncthreads();                                            // dh and Delta have been read
     th.put(mS);
+    tm.put(mM);
     __syncthreads();
     // ---- dq <- diag(gamma) dO h^T;  dW<- = -dDelta h^T;  dT = dDelta V^T + ...;  dV = T^T dDelta ------------
-    float aT[1][2][4];
+    float aT[MT][2][4];
     zero(aT);
     pmm<false, false>(aQ, mO, mS, wm, nk, DV);
     pmm<false, false>(aX, mdD, mS, wm, nk, DV);
     pmm<false, false>(aT, mdD, mV, wm, nc, DV);
     {
-        float a[1][NV][4];
+        float a[MT][NV][4];
         zero(a);
         pmm<true, true>(a, mM, mdD, wm, nv, C);
         each(a, wm, nv, [&](int s, int j, float x, float y) {
@@ -1025,22 +1043,22 @@ __global__ void __launch_bounds__(512) k_chunk_bwd_planes(Ptrs p) {
     auto qsum = [&](int r, int i, float x, float y) { const float2 q = mQ.ld2(r, i); return srq[r] * fmaf(x, q.x, y * q.y); };
     auto ksum = [&](int r, int i, float x, float y) { const float2 k = mK.ld2(r, i); return srk[r] * fmaf(x, k.x, y * k.y); };
     row_sums(aQ, wm, nk, prow[1][wn], qsum);                    // t1 = <dQ1, Q>
-    __syncthreads();                                            // h has been read
+    __syncthreads();                                            // h, dO, dDelta and V have been read
     each(aX, wm, nk, [&](int r, int i, float x, float y) { mW.st2(r, i, -x, -y); });
     __syncthreads();
     // ---- ... + dW<- (gamma X)^T;  d beta from T;  dX <- diag(gamma) T^T dW<-;  t2 = <dXg, gamma X> ----------
     {
-        float a1[1][2][4], a2[1][2][4];
-        zero(a1); zero(a2);
-        pmm<false, false>(a1, mW, mK, wm, nc, DK);
-        pmm<false, false>(a2, mW, mQ, wm, nc, DK);
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int s = nc + 8 * j + 2 * (lane & 3) + (e & 1);
-                aT[0][j][e] = fmaf(sgam[s], fmaf(srk[s], a1[0][j][e], scq[s] * a2[0][j][e]), aT[0][j][e]);
-            }
+        float a[MT][2][4];
+        zero(a);
+        pmm<false, false>(a, mW, mK, wm, nc, DK);
+        each2(aT, a, wm, nc, [&](int, int s, float& x, float& y, float u, float v) {
+            x = fmaf(sgam[s] * srk[s], u, x); y = fmaf(sgam[s + 1] * srk[s + 1], v, y);
+        });
+        zero(a);
+        pmm<false, false>(a, mW, mQ, wm, nc, DK);
+        each2(aT, a, wm, nc, [&](int, int s, float& x, float& y, float u, float v) {
+            x = fmaf(sgam[s] * scq[s], u, x); y = fmaf(sgam[s + 1] * scq[s + 1], v, y);
+        });
         each(aT, wm, nc, [&](int r, int s, float& x, float& y) {
             const float2 m = mM.ld2(r, s);
             mT.st2(r, s, x * sbeta[s], y * sbeta[s + 1]);
@@ -1058,61 +1076,71 @@ __global__ void __launch_bounds__(512) k_chunk_bwd_planes(Ptrs p) {
     __syncthreads();                                            // dT diag(beta) is complete
     // ---- dA = -strictLower(M^T (dT diag(beta) M^T)) -------------------------------------------------
     {
-        float a[1][2][4];
+        float a[MT][2][4];
         zero(a);
         pmm<false, false>(a, mT, mM, wm, nc, C);
         each(a, wm, nc, [&](int r, int s, float x, float y) { m4.st2(r, s, x, y); });
     }
-    float kk[1][2][4], qk[1][2][4];
-    zero(kk); zero(qk);
-    pmm<false, false>(kk, mK, mK, wm, nc, DK);
-    pmm<false, false>(qk, mQ, mK, wm, nc, DK);
     __syncthreads();
     {
-        float a[1][2][4];
-        zero(a);
+        float a[MT][2][4], x[MT][2][4];
+        zero(a); zero(x);
         pmm<true, true>(a, mM, m4, wm, nc, C);
+        pmm<false, false>(x, mQ, mK, wm, nc, DK);               // X K^T
+        each(x, wm, nc, [&](int r, int, float& u, float& v) { u *= scq[r]; v *= scq[r]; });
+        {
+            float y[MT][2][4];
+            zero(y);
+            pmm<false, false>(y, mK, mK, wm, nc, DK);
+            each2(x, y, wm, nc, [&](int r, int s, float& u, float& v, float k0, float k1) {
+                u = srk[s] * fmaf(srk[r], k0, u); v = srk[s + 1] * fmaf(srk[r], k1, v);
+            });
+        }
         __syncthreads();                                        // M and dT M^T have been read: dX K^T and dP o Gamma over them
         // the uses of dA: d beta (row sums), dA o A (column sums), d(X K^T)
-        const typename L::TC e1(smb + L::kE), e2(smb + L::kE + L::TC::kBytes), e3(smb + L::kE + 2 * L::TC::kBytes), e4(smb + L::kE + 3 * L::TC::kBytes);
-        float ca[1][2][4];
+        const typename L::TC e1(smb + L::kV), e2(smb + L::kV + L::TC::kBytes), e3(smb + L::kV + 2 * L::TC::kBytes);
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int i = 0; i < MT; ++i)
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int r = wm + 8 * h + (lane >> 2), s = nc + 8 * j + 2 * (lane & 3);
-                const float be = sbeta[r], cq = scq[r], ck = srk[r], rq = srq[r];
-                float d[2], f[2];
+            for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const float x = s + e < r ? -a[0][j][2 * h + e] * expf(sg[r] - sg[s + e]) : 0.f;
-                    const float xk = srk[s + e] * fmaf(ck, kk[0][j][2 * h + e], cq * qk[0][j][2 * h + e]);
-                    a[0][j][2 * h + e] = x * xk;
-                    ca[0][j][2 * h + e] = be * x * xk;
-                    d[e] = be * x; f[e] = a3[0][j][2 * h + e];
+                for (int j = 0; j < 2; ++j) {
+                    const int r = wm + 16 * i + 8 * h + (lane >> 2), s = nc + 8 * j + 2 * (lane & 3);
+                    const float be = sbeta[r], cq = scq[r], rq = srq[r];
+                    float d[2], *f = a3[i][j] + 2 * h;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        float& v = a[i][j][2 * h + e];
+                        float& w = x[i][j][2 * h + e];
+                        const float u = s + e < r ? -v * expf(sg[r] - sg[s + e]) : 0.f;
+                        v = u * w;
+                        w = be * v;
+                        d[e] = be * u;
+                    }
+                    e1.st2(r, s, d[0] * srk[s], d[1] * srk[s + 1]);
+                    e2.st2(r, s, f[0] * srk[s], f[1] * srk[s + 1]);
+                    e3.st2(r, s, fmaf(cq, d[0], rq * f[0]), fmaf(cq, d[1], rq * f[1]));
                 }
-                e1.st2(r, s, d[0] * srk[s], d[1] * srk[s + 1]);
-                e2.st2(r, s, f[0] * srk[s], f[1] * srk[s + 1]);
-                e3.st2(r, s, fmaf(cq, d[0], rq * f[0]), fmaf(cq, d[1], rq * f[1]));
-                if (p.rqk) e4.st2(r, s, d[0] * ck, d[1] * ck);
-            }
-        row_sums(a, wm, nc, prow[3][wn], [&](int, int, float x, float y) { return x + y; });
-        col_sums(ca, pcol[2][wr]);
+        row_sums(a, wm, nc, prow[3][wn], [&](int, int, float u, float v) { return u + v; });
+        col_sums(x, pcol[2][wr]);
         __syncthreads();
         // ---- dX += dXK K;  dk += dXK^T X + dPG^T Q + dX;  dq += dPG K + lambda dX ----------------------
         pmm<false, true>(aX, e1, mK, wm, nk, C);
         row_sums(aX, wm, nk, prow[4][wn], qsum);
         pmm<false, true>(aQ, e2, mK, wm, nk, C);
         pmm<true, true>(aK, e3, mQ, wm, nk, C);
-        pmm<true, true>(aK, p.rqk ? e4 : e1, mK, wm, nk, C);
-    }
-#pragma unroll
-    for (int j = 0; j < NK; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            aK[0][j][e] += aX[0][j][e];
-            aQ[0][j][e] = fmaf(slam[wm + 8 * (e >> 1) + (lane >> 2)], aX[0][j][e], aQ[0][j][e]);
+        if (p.rqk) {                                            // dXK scaled by row instead of by column
+            __syncthreads();
+            each(a, wm, nc, [&](int r, int s, float, float) {
+                const float2 d = e1.ld2(r, s);
+                e1.st2(r, s, d.x * (srk[r] / srk[s]), d.y * (srk[r] / srk[s + 1]));
+            });
+            __syncthreads();
         }
+        pmm<true, true>(aK, e1, mK, wm, nk, C);
+    }
+    each2(aQ, aX, wm, nk, [&](int r, int, float& x, float& y, float u, float v) { x = fmaf(slam[r], u, x); y = fmaf(slam[r], v, y); });
+    each2(aK, aX, wm, nk, [&](int, int, float& x, float& y, float u, float v) { x += u; y += v; });
     if (p.rqk) {
         // through the normalisation: dx = r (dx^ - x^ <x^, dx^>)
         row_sums(aQ, wm, nk, part[wn], qsum);
@@ -1134,7 +1162,11 @@ __global__ void __launch_bounds__(512) k_chunk_bwd_planes(Ptrs p) {
     each(aK, wm, nk, [&](int r, int i, float x, float y) { if (r < live) st2((IO*)p.dk_ + (row0 + (size_t)r * H) * DK + i, x, y); });
     each(aQ, wm, nk, [&](int r, int i, float x, float y) { if (r < live) st2((IO*)p.dq + (row0 + (size_t)r * H) * DK + i, x, y); });
     __syncthreads();
-    const float db1 = tid < C ? pcol[1][0][tid] + pcol[1][1][tid] + pcol[1][2][tid] + pcol[1][3][tid] : 0.f;
+    float db1 = 0.f;
+    if (tid < C) {
+#pragma unroll
+        for (int c = 0; c < WR; ++c) db1 += pcol[1][c][tid];
+    }
     token_gradients<IO>(p, prow, pcol[0], pcol[2], db1, sbeta, slam, salpha, sgam, sdg, skd, row0, wrow0, bh, n, live);
 }
 
@@ -1191,7 +1223,7 @@ cudaError_t chain_bwd_for(const ChunkArgs& a, const Ptrs& p) {
 template <typename IO, int DK, int DV>
 cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {
     if constexpr (sizeof(IO) == 2) {
-        return launch(k_chunk_bwd_planes<DK, DV>, a.s.B * a.s.H * p.N, 512, BwdPlanes<DK, DV>::kBytes, a.stream, p);
+        return launch(k_chunk_bwd_planes<DK, DV>, a.s.B * a.s.H * p.N, BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>::kBytes, a.stream, p);
     } else {
         return launch(k_chunk_bwd<DK, DV>, a.s.B * a.s.H * p.N, NT, BwdSmem<DK, DV>::bytes, a.stream, p);
     }
