@@ -85,9 +85,9 @@ __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-// acc += A B for the (16 MT) x (8 NTL) tile of this warp at row m0, column n0, contraction extent K.  A is stored as [m][k], or
+// acc += A B for the (16 MT) x (8 NTL) tile of this warp at row m0 (pieces of 16 rows MS apart), column n0, contraction extent K.  A is stored as [m][k], or
 // as [k][m] with AT; B as [n][k], or as [k][n] with BT.  Fragments of acc: rows g and g + 8, columns 2t and 2t + 1.
-template <bool AT, bool BT, int MT, int NTL, class MA, class MB>
+template <bool AT, bool BT, int MT, int NTL, class MA, class MB, int MS = 16>
 __device__ __forceinline__ void pmm(float (&acc)[MT][NTL][4], const MA& A, const MB& B, int m0, int n0, int K) {
     static_assert(NTL % 2 == 0, "columns come in pairs of 8");
     constexpr int PA = MA::NP, PB = MB::NP;
@@ -103,7 +103,7 @@ __device__ __forceinline__ void pmm(float (&acc)[MT][NTL][4], const MA& A, const
         for (int i = 0; i < MT; ++i)
 #pragma unroll
             for (int x = 0; x < PA; ++x)
-                sm100::ldsm4<AT>(pa + x * MA::PS + (AT ? k0 * MA::LD + 16 * i : 16 * i * MA::LD + k0), a[i][x]);
+                sm100::ldsm4<AT>(pa + x * MA::PS + (AT ? k0 * MA::LD + MS * i : MS * i * MA::LD + k0), a[i][x]);
 #pragma unroll
         for (int j = 0; j < NTL; j += 2) {
             uint32_t b[PB][4];

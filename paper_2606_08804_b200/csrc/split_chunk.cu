@@ -414,8 +414,10 @@ __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
 // K2: forward state chain.  One CTA per (sequence, DS-column slice of d_v); columns of the state evolve independently,
 // the chunks of a sequence are walked in order.  The next chunk's tiles are fetched into registers while the present
 // chunk is worked on: a chunk costs its two dependent products and three barriers, not its loads.
-template <typename IO, int DK, int DS, int TH>
-__global__ void __launch_bounds__(TH) k_chain_fwd(Ptrs p, int DV) {
+template <int DK, int DS>
+__global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
+    typedef float IO;
+    constexpr int TH = NT;
     extern __shared__ float sm[];
     constexpr int LA = DK + 4, LB = DK + 8, LS = DS + 8, TI = kTerms<IO>, NS = DS / 8;
     // the two products of a phase take half of the warps each: 64 tokens x DS columns in 16 x 8 NH, DK x DS in 16 MU x 8 NU
@@ -514,8 +516,10 @@ __global__ void __launch_bounds__(TH) k_chain_fwd(Ptrs p, int DV) {
 // K3: reverse state chain.  Carries dh (gradient w.r.t. the chunk's exit state) backwards:
 //   dDelta = P^T dO + K-> dh ;   dh_in = gamma_C dh + (diag(gamma) Q)^T dO - W<-^T dDelta
 // and leaves per chunk: dh (exit), dDelta, and two scalar partial sums the decay gradient needs.
-template <typename IO, int DK, int DS, int TH>
-__global__ void __launch_bounds__(TH) k_chain_bwd(Ptrs p, int DV) {
+template <int DK, int DS>
+__global__ void __launch_bounds__(NT) k_chain_bwd(Ptrs p, int DV) {
+    typedef float IO;
+    constexpr int TH = NT;
     extern __shared__ float sm[];
     constexpr int LA = DK + 4, LB = DK + 8, LP = C + 8, LS = DS + 8, TI = kTerms<IO>, NS = DS / 8;
     // the two products of a phase take half of the warps each: 64 tokens x DS columns in 16 x 8 NH, DK x DS in 16 MU x 8 NU
@@ -629,6 +633,283 @@ __global__ void __launch_bounds__(TH) k_chain_bwd(Ptrs p, int DV) {
             p.dh0[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] = sdh[(e / DS) * LS + e % DS];
 }
 
+// The state chains for bf16 storage, on bf16 planes.  Every warp takes a 16 x 16 tile of the 64 x DS products and DK/4 x 16 of
+// the state, which it keeps in fp32 in its registers (planes of it are what the others read).  A chunk is two phases and two
+// barriers; the tiles of one phase arrive while the other is worked on, those of the first two phases ahead.  Slices of 32
+// columns and d_k = 64 let two CTAs share an SM.  B4 T1024 H16 d_k = d_v = 64: 73 and 85 us with tf32 halves, 50 and 56 so (3 us a
+// chunk, of which the tensor unit works a quarter: the rest is the latency of two dependent products and two barriers).
+template <int DK, int DS>
+struct ChainPlanes {
+    typedef Planes<C, DK, 1> TA;
+    typedef Planes<2 * C, DK, 1> TA2;      // W<- above Q
+    typedef Planes<C, C, 1> TP;
+    typedef Planes<C, DS, 1> TO;
+    typedef Planes<C, DS, 3> TD;
+    typedef Planes<DK, DS, 3> TS;
+    static constexpr int kThreads = 8 * DS, kFwd = 2 * TA2::kBytes + TA::kBytes + TP::kBytes + TS::kBytes + 2 * TD::kBytes,
+                         kBwd = 2 * (TA::kBytes + TP::kBytes + TO::kBytes) + 2 * TA::kBytes + TS::kBytes + 2 * TD::kBytes;
+};
+template <int N> __device__ __forceinline__ void fetch_wait_but() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// decay factors of a chunk's tokens, thread t < 64 token t: fetched a chunk ahead, written before the barrier that ends the present one
+struct ChainCoef {
+    float g = 0.f, gC = 0.f, rq = 1.f, rk = 1.f;
+    __device__ __forceinline__ void get(const Ptrs& p, size_t wrow0, size_t nrows) {
+        if (threadIdx.x >= C) return;
+        g = p.g[wrow0 + threadIdx.x]; gC = p.g[wrow0 + C - 1];
+        if (p.rqk) { rq = p.rqk[wrow0 + threadIdx.x]; rk = p.rqk[nrows + wrow0 + threadIdx.x]; }
+    }
+    __device__ __forceinline__ void put(float* gq, float* gk, float* gc) const {
+        if (threadIdx.x >= C) return;
+        gq[threadIdx.x] = expf(g) * rq; gk[threadIdx.x] = expf(gC - g) * rk;
+        if (threadIdx.x == 0) *gc = expf(gC);
+    }
+};
+template <int DK, int DS>
+__global__ void __launch_bounds__(8 * DS) k_chain_fwd_planes(Ptrs p, int DV) {
+    extern __shared__ __align__(16) unsigned char smb[];
+    typedef ChainPlanes<DK, DS> L;
+    typedef __nv_bfloat16 IO;
+    constexpr int TH = L::kThreads, MU = DK / 64;
+    typename L::TA2 mWQ(smb);
+    const typename L::TA mK(smb + 2 * L::TA2::kBytes);
+    const typename L::TP mP(smb + 2 * L::TA2::kBytes + L::TA::kBytes);
+    const typename L::TS mS(smb + 2 * L::TA2::kBytes + L::TA::kBytes + L::TP::kBytes);
+    const typename L::TD mD(smb + L::kFwd - 2 * L::TD::kBytes), mDs(smb + L::kFwd - L::TD::kBytes);
+    __shared__ float sgq[2][C], sgk[2][C], sgC[2];
+    const int H = p.H, nsl = DV / DS, j0 = (blockIdx.x % nsl) * DS, bh = blockIdx.x / nsl, b = bh / H, hh = bh % H;
+    const int tid = threadIdx.x, warp = tid >> 5, g = (tid & 31) >> 2, t = tid & 3;
+    const int wm = (warp & 3) * 16, wn = (warp >> 2) * 16, si = (warp & 3) * 16 * MU;
+    const size_t nrows = (size_t)p.B * H * p.Tp, row0 = (size_t)b * p.T * H + hh, wrow0 = (size_t)bh * p.Tp;
+    sm100::grid_dep_wait();            // launched while the kernel before it drains
+    sm100::grid_dep_launch();
+    auto fetch1 = [&](int n) {         // W<- and Q, read in the first phase of chunk n
+        const typename L::TA w(smb + (n & 1) * L::TA2::kBytes), q(smb + (n & 1) * L::TA2::kBytes + L::TA::kBytes);
+        w.template fetch<TH>((const IO*)p.W + (wrow0 + (size_t)n * C) * DK, DK, C);
+        q.template fetch<TH>((const IO*)p.q + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C));
+    };
+    auto fetch2 = [&](int n) {         // K and P, read in the second
+        mK.template fetch<TH>((const IO*)p.k + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C));
+        mP.template fetch<TH>((const IO*)p.P + (wrow0 + (size_t)n * C) * C, C, C);
+    };
+    uint32_t u[2][2];                  // U~ at this thread's elements
+    auto fetch_u = [&](int n) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                u[h][j] = *reinterpret_cast<const uint32_t*>((const IO*)p.U + (wrow0 + (size_t)n * C + wm + 8 * h + g) * DV + j0 + wn + 8 * j + 2 * t);
+    };
+    ChainCoef cf;
+    fetch1(0);
+    fetch_commit();
+    cf.get(p, wrow0, nrows);
+    fetch_u(0);
+    float hst[MU][2][4];
+    zero(hst);
+    auto state_at = [&](float* base, int i, int j) { return reinterpret_cast<float2*>(base + (size_t)i * DV + j0 + j); };
+    if (p.h0) each(hst, si, wn, [&](int i, int j, float& x, float& y) {
+        const float2 v = *state_at(const_cast<float*>(p.h0) + (size_t)bh * DK * DV, i, j);
+        x = v.x; y = v.y;
+    });
+    each(hst, si, wn, [&](int i, int j, float x, float y) {
+        mS.st2(i, j, x, y);
+        if (p.save) *state_at(p.hs + (size_t)bh * p.N * DK * DV, i, j) = make_float2(x, y);
+    });
+    cf.put(sgq[0], sgk[0], sgC);
+    for (int n = 0; n < p.N; ++n) {
+        const int bf = n & 1, live = min(C, p.T - n * C);
+        const bool more = n + 1 < p.N;
+        fetch_wait();
+        __syncthreads();
+        fetch2(n);
+        fetch_commit();
+        if (more) { fetch1(n + 1); cf.get(p, wrow0 + (size_t)(n + 1) * C, nrows); }
+        fetch_commit();
+        // Delta = U~ - W<- h, and Q h, the inter-chunk part of the output
+        float a[2][2][4], o[1][2][4];
+        zero(a); zero(o);
+        mWQ.p = reinterpret_cast<IO*>(smb + bf * L::TA2::kBytes);
+        pmm<false, true, 2, 2, typename L::TA2, typename L::TS, C>(a, mWQ, mS, wm, wn, DK);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int r = wm + 8 * h + g, c = wn + 8 * j + 2 * t;
+                const float x = __uint_as_float(u[h][j] << 16) - a[0][j][2 * h], y = __uint_as_float(u[h][j] & 0xffff0000u) - a[0][j][2 * h + 1];
+                mD.st2(r, c, x, y);
+                mDs.st2(r, c, x * sgk[bf][r], y * sgk[bf][r]);
+                if (p.save) st2((IO*)p.D + (wrow0 + (size_t)n * C + r) * DV + j0 + c, x, y);
+            }
+        if (more) fetch_u(n + 1);
+        fetch_wait_but<1>();
+        __syncthreads();
+        // h <- gamma_C h + K^T (diag(gamma_C/gamma) Delta)
+        {
+            float s[MU][2][4];
+            zero(s);
+            pmm<true, true>(s, mK, mDs, si, wn, C);
+            const float gc = sgC[bf];
+            each2(hst, s, si, wn, [&](int i, int j, float& x, float& y, float dx, float dy) {
+                x = fmaf(gc, x, dx); y = fmaf(gc, y, dy);
+                mS.st2(i, j, x, y);
+                if (p.save && more) *state_at(p.hs + ((size_t)bh * p.N + n + 1) * DK * DV, i, j) = make_float2(x, y);
+            });
+        }
+        // o = diag(gamma) Q h + P Delta
+        pmm<false, true>(o, mP, mD, wm, wn, C);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int r = wm + 8 * h + g;
+                const float f = sgq[bf][r];
+                if (r < live) st2((IO*)p.o + (row0 + (size_t)(n * C + r) * H) * DV + j0 + wn + 8 * j + 2 * t,
+                                  fmaf(f, a[1][j][2 * h], o[0][j][2 * h]), fmaf(f, a[1][j][2 * h + 1], o[0][j][2 * h + 1]));
+            }
+        if (more) cf.put(sgq[bf ^ 1], sgk[bf ^ 1], sgC + (bf ^ 1));
+    }
+    if (p.hT) each(hst, si, wn, [&](int i, int j, float x, float y) { *state_at(p.hT + (size_t)bh * DK * DV, i, j) = make_float2(x, y); });
+}
+
+template <int DK, int DS>
+__global__ void __launch_bounds__(8 * DS) k_chain_bwd_planes(Ptrs p, int DV) {
+    extern __shared__ __align__(16) unsigned char smb[];
+    typedef ChainPlanes<DK, DS> L;
+    typedef __nv_bfloat16 IO;
+    constexpr int TH = L::kThreads, MU = DK / 64, kSet = L::TA::kBytes + L::TP::kBytes + L::TO::kBytes;
+    const typename L::TA mQ(smb + 2 * kSet), mW(smb + 2 * kSet + L::TA::kBytes);
+    const typename L::TS mS(smb + 2 * kSet + 2 * L::TA::kBytes);
+    const typename L::TD mdD(smb + L::kBwd - 2 * L::TD::kBytes), mOs(smb + L::kBwd - L::TD::kBytes);
+    __shared__ float sgq[2][C], sgk[2][C], sgC[2], sred[TH / 32], skd[DS / 16][C];
+    const int H = p.H, nsl = DV / DS, sl = blockIdx.x % nsl, j0 = sl * DS, bh = blockIdx.x / nsl, b = bh / H, hh = bh % H;
+    const int tid = threadIdx.x, warp = tid >> 5, g = (tid & 31) >> 2, t = tid & 3;
+    const int wm = (warp & 3) * 16, wn = (warp >> 2) * 16, si = (warp & 3) * 16 * MU;
+    const size_t nrows = (size_t)p.B * H * p.Tp, BHN = (size_t)p.B * H * p.N, row0 = (size_t)b * p.T * H + hh, wrow0 = (size_t)bh * p.Tp;
+    sm100::grid_dep_wait();            // launched while the kernel before it drains
+    sm100::grid_dep_launch();
+    auto fetch1 = [&](int n) {         // K, P and dO, read in the first phase of chunk n
+        unsigned char* s = smb + (n & 1) * kSet;
+        const typename L::TA k(s);
+        const typename L::TP pm(s + L::TA::kBytes);
+        const typename L::TO o(s + L::TA::kBytes + L::TP::kBytes);
+        const int live = min(C, p.T - n * C);
+        k.template fetch<TH>((const IO*)p.k + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, live);
+        pm.template fetch<TH>((const IO*)p.P + (wrow0 + (size_t)n * C) * C, C, C);
+        o.template fetch<TH>((const IO*)p.dO + (row0 + (size_t)n * C * H) * DV + j0, (size_t)H * DV, live);
+    };
+    auto fetch2 = [&](int n) {         // Q and W<-, read in the second
+        mQ.template fetch<TH>((const IO*)p.q + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C));
+        mW.template fetch<TH>((const IO*)p.W + (wrow0 + (size_t)n * C) * DK, DK, C);
+    };
+    uint32_t d[2][2];                  // Delta and the entry state at this thread's elements
+    float2 hin[MU][2][2];
+    auto state_at = [&](float* base, int i, int j) { return reinterpret_cast<float2*>(base + (size_t)i * DV + j0 + j); };
+    auto fetch_d = [&](int n) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                d[h][j] = *reinterpret_cast<const uint32_t*>((const IO*)p.D + (wrow0 + (size_t)n * C + wm + 8 * h + g) * DV + j0 + wn + 8 * j + 2 * t);
+#pragma unroll
+                for (int m = 0; m < MU; ++m) hin[m][h][j] = *state_at(p.hs + ((size_t)bh * p.N + n) * DK * DV, si + 16 * m + 8 * h + g, wn + 8 * j + 2 * t);
+            }
+    };
+    ChainCoef cf;
+    fetch1(p.N - 1);
+    fetch_commit();
+    cf.get(p, wrow0 + (size_t)(p.N - 1) * C, nrows);
+    fetch_d(p.N - 1);
+    float dst[MU][2][4];
+    zero(dst);
+    if (p.dhT) each(dst, si, wn, [&](int i, int j, float& x, float& y) {
+        const float2 v = *state_at(const_cast<float*>(p.dhT) + (size_t)bh * DK * DV, i, j);
+        x = v.x; y = v.y;
+    });
+    each(dst, si, wn, [&](int i, int j, float x, float y) { mS.st2(i, j, x, y); });
+    cf.put(sgq[(p.N - 1) & 1], sgk[(p.N - 1) & 1], sgC + ((p.N - 1) & 1));
+    for (int n = p.N - 1; n >= 0; --n) {
+        const int bf = n & 1;
+        fetch_wait();
+        __syncthreads();
+        fetch2(n);
+        fetch_commit();
+        if (n > 0) { fetch1(n - 1); cf.get(p, wrow0 + (size_t)(n - 1) * C, nrows); }
+        fetch_commit();
+        const typename L::TA mK(smb + bf * kSet);
+        const typename L::TP mP(smb + bf * kSet + L::TA::kBytes);
+        const typename L::TO mO(smb + bf * kSet + L::TA::kBytes + L::TP::kBytes);
+        // dDelta = diag(gamma_C/gamma) K dh + P^T dO; row sums of the first term times Delta
+        {
+            float a[1][2][4], c[1][2][4];
+            zero(a); zero(c);
+            pmm<false, true>(a, mK, mS, wm, wn, DK);
+            each(a, wm, wn, [&](int r, int, float& x, float& y) { x *= sgk[bf][r]; y *= sgk[bf][r]; });
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float s = 0.f;
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    s += fmaf(a[0][j][2 * h], __uint_as_float(d[h][j] << 16), a[0][j][2 * h + 1] * __uint_as_float(d[h][j] & 0xffff0000u));
+                s += __shfl_xor_sync(0xffffffffu, s, 1);
+                s += __shfl_xor_sync(0xffffffffu, s, 2);
+                if (t == 0) skd[warp >> 2][wm + 8 * h + g] = s;
+            }
+            pmm<true, true>(c, mP, mO, wm, wn, C);
+            each2(a, c, wm, wn, [&](int s, int j, float x, float y, float u, float v) {
+                x += u; y += v;
+                mdD.st2(s, j, -x, -y);
+                st2((IO*)p.dD + (wrow0 + (size_t)n * C + s) * DV + j0 + j, x, y);
+                const float2 o = mO.ld2(s, j);                   // diag(gamma / |q|) dO, the operand of Q^T
+                mOs.st2(s, j, o.x * sgq[bf][s], o.y * sgq[bf][s]);
+            });
+        }
+        // keep dh of this chunk's exit state; partial <dh, h_entry>_F over this slice
+        float part = 0.f;
+#pragma unroll
+        for (int m = 0; m < MU; ++m)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const float2 v = make_float2(dst[m][j][2 * h], dst[m][j][2 * h + 1]);
+                    *state_at(p.dhs + ((size_t)bh * p.N + n) * DK * DV, si + 16 * m + 8 * h + g, wn + 8 * j + 2 * t) = v;
+                    part = fmaf(v.x, hin[m][h][j].x, fmaf(v.y, hin[m][h][j].y, part));
+                }
+        part = warp_sum(part);
+        if ((tid & 31) == 0) sred[warp] = part;
+        if (n > 0) fetch_d(n - 1);
+        fetch_wait_but<1>();
+        __syncthreads();
+        if (tid < C) {
+            float kd = 0.f;
+#pragma unroll
+            for (int w = 0; w < DS / 16; ++w) kd += skd[w][tid];
+            p.kdhd[(size_t)sl * nrows + wrow0 + (size_t)n * C + tid] = kd;
+        }
+        if (tid == TH - 1) {
+            float tot = 0.f;
+            for (int w = 0; w < TH / 32; ++w) tot += sred[w];
+            p.dhh[(size_t)sl * BHN + (size_t)bh * p.N + n] = tot;
+        }
+        // dh <- gamma_C dh + (diag(gamma) Q)^T dO - W<-^T dDelta
+        {
+            float s[MU][2][4];
+            zero(s);
+            pmm<true, true>(s, mQ, mOs, si, wn, C);
+            pmm<true, true>(s, mW, mdD, si, wn, C);
+            const float gc = sgC[bf];
+            each2(dst, s, si, wn, [&](int i, int j, float& x, float& y, float dx, float dy) {
+                x = fmaf(gc, x, dx); y = fmaf(gc, y, dy);
+                mS.st2(i, j, x, y);
+            });
+        }
+        if (n > 0) cf.put(sgq[bf ^ 1], sgk[bf ^ 1], sgC + (bf ^ 1));
+    }
+    if (p.dh0) each(dst, si, wn, [&](int i, int j, float x, float y) { *state_at(p.dh0 + (size_t)bh * DK * DV, i, j) = make_float2(x, y); });
+}
+
+// ---------------------------------------------------------------------------------------------
 // Per token, from the row sums (prow: dP o P, t1, t2, d beta, d lambda) and the column sums (cP: dP o P, cA: dA o A; db1: dT o M,
 // of token threadIdx.x): d beta, d lambda, and the decay gradient: dg, its reverse in-chunk cumulative sum,
 // d alpha = d log alpha / alpha.  sdg and skd are scratch.
@@ -1205,20 +1486,27 @@ cudaError_t prep_for(const ChunkArgs& a, const Ptrs& p) {
     constexpr size_t smem = sizeof(float) * (2 * C * (DK + kPad) + C * (DV + kPad) + 3 * C * LDC);
     return launch(k_prep<IO, DK, DV>, a.s.B * a.s.H * p.N, NT, smem, a.stream, p);
 }
-// 16 warps where a chunk's products are small and its operands need little splitting: bf16, d_k = 64 (82 -> 72 and 97 -> 85 us
-// on 64 sequences of 16 chunks).  fp32 operands are split by every warp that reads them, so that 8 warps with larger tiles win
-// (52 against 48 us at d_k = 128 on 16 sequences of 8 chunks; one short call of d_k = 64, 28.7 against 27.2).
-template <typename IO, int DK> constexpr int chain_threads = sizeof(IO) == 2 && DK == 64 ? 512 : 256;
-
 template <typename IO, int DK, int DS>
 cudaError_t chain_fwd_for(const ChunkArgs& a, const Ptrs& p) {
-    constexpr size_t smem = sizeof(float) * (2 * C * (DK + 4) + C * (DK + 8) + C * LDC + (3 * C + DK) * (DS + 8));
-    return launch(k_chain_fwd<IO, DK, DS, chain_threads<IO, DK>>, a.s.B * a.s.H * (a.s.dv / DS), chain_threads<IO, DK>, smem, a.stream, p, a.s.dv);
+    const int grid = a.s.B * a.s.H * (a.s.dv / DS);
+    if constexpr (sizeof(IO) == 2) {
+        typedef ChainPlanes<DK, DS> L;
+        return launch(k_chain_fwd_planes<DK, DS>, grid, L::kThreads, L::kFwd, a.stream, p, a.s.dv);
+    } else {
+        constexpr size_t smem = sizeof(float) * (2 * C * (DK + 4) + C * (DK + 8) + C * LDC + (3 * C + DK) * (DS + 8));
+        return launch(k_chain_fwd<DK, DS>, grid, NT, smem, a.stream, p, a.s.dv);
+    }
 }
 template <typename IO, int DK, int DS>
 cudaError_t chain_bwd_for(const ChunkArgs& a, const Ptrs& p) {
-    constexpr size_t smem = sizeof(float) * (C * (DK + 4) + 2 * C * (DK + 8) + C * (C + 8) + (4 * C + DK) * (DS + 8));
-    return launch(k_chain_bwd<IO, DK, DS, chain_threads<IO, DK>>, a.s.B * a.s.H * (a.s.dv / DS), chain_threads<IO, DK>, smem, a.stream, p, a.s.dv);
+    const int grid = a.s.B * a.s.H * (a.s.dv / DS);
+    if constexpr (sizeof(IO) == 2) {
+        typedef ChainPlanes<DK, DS> L;
+        return launch(k_chain_bwd_planes<DK, DS>, grid, L::kThreads, L::kBwd, a.stream, p, a.s.dv);
+    } else {
+        constexpr size_t smem = sizeof(float) * (C * (DK + 4) + 2 * C * (DK + 8) + C * (C + 8) + (4 * C + DK) * (DS + 8));
+        return launch(k_chain_bwd<DK, DS>, grid, NT, smem, a.stream, p, a.s.dv);
+    }
 }
 template <typename IO, int DK, int DV>
 cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {
