@@ -30,6 +30,7 @@ namespace {
 constexpr int C = kChunk;
 constexpr int NT = 256;            // threads of the kernels that take a chunk each: 8 warps
 constexpr int LDC = C + 4;         // leading dimension of the C x C matrices in shared memory
+constexpr int LDI = C / 2 + 4;    // of the inverse's scratch
 constexpr int kPad = 4;            // of a d-wide tile: rows g, columns t of a fragment fall on banks 4 g + t
 
 struct Ptrs {
@@ -268,7 +269,7 @@ __device__ __forceinline__ void invert_unit_lower(const float* sA, float* sM, fl
                 const float4 b = *reinterpret_cast<const float4*>(sM + (o + k) * LDC + o + c);
                 x.x = fmaf(av, b.x, x.x); x.y = fmaf(av, b.y, x.y); x.z = fmaf(av, b.z, x.z); x.w = fmaf(av, b.w, x.w);
             }
-            *reinterpret_cast<float4*>(sS + (o + r) * LDC + c) = x;
+            *reinterpret_cast<float4*>(sS + (o + r) * LDI + c) = x;
         }
         __syncthreads();
         for (int e = tid; e < pairs * quads; e += NT) {
@@ -277,7 +278,7 @@ __device__ __forceinline__ void invert_unit_lower(const float* sA, float* sM, fl
 #pragma unroll 8
             for (int k = 0; k < S; ++k) {
                 const float av = -sM[(o + S + r) * LDC + o + S + k];
-                const float4 b = *reinterpret_cast<const float4*>(sS + (o + k) * LDC + c);
+                const float4 b = *reinterpret_cast<const float4*>(sS + (o + k) * LDI + c);
                 x.x = fmaf(av, b.x, x.x); x.y = fmaf(av, b.y, x.y); x.z = fmaf(av, b.z, x.z); x.w = fmaf(av, b.w, x.w);
             }
             *reinterpret_cast<float4*>(sM + (o + S + r) * LDC + o + c) = x;
@@ -306,8 +307,9 @@ __device__ __forceinline__ void scan64(float x, float* sg) {
 
 // ---------------------------------------------------------------------------------------------
 // K1: per chunk-head, state-independent part: g, P, W<-, U~ (and M for the backward).
-template <typename IO, int DK, int DV>
+template <int DK, int DV>
 __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
+    typedef float IO;
     extern __shared__ float sm[];
     constexpr int LK = DK + kPad, LV = DV + kPad, TI = kTerms<IO>;
     constexpr bool EX = TI == 2;
@@ -408,6 +410,123 @@ __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
         wmm<2, DK / 32, 2, 2, EX>(w, wm, wn * (DK / 4), C, Tf, Xf);
         each(w, wm, wn * (DK / 4), [&](int r, int d, float x, float y) { st2((IO*)p.W + (wrow0 + r) * DK + d, x, y); });
     }
+}
+
+// The same for bf16 storage, on bf16 planes: X is never formed, X K^T and T diag(gamma) X are each a product with K and one
+// with Q, their coefficients applied to the result or to T.  One set of planes holds T, T diag(gamma / |k|) and
+// T diag(lambda gamma / |q|) in turn, over what the inverse needed; at d_k = d_v = 64 three CTAs fit an SM.
+// 1024 chunks of 64 x 64: 72 us with tf32 halves and two CTAs, 56 so (d_k 128, d_v 64: 119 and 70), bound by the latency of its
+// chain of small steps.
+template <int DK, int DV>
+struct PrepPlanes {
+    typedef Planes<C, DK, 1> TQ;
+    typedef Planes<C, DV, 1> TV;
+    typedef Planes<C, C, 3> TC;
+    static constexpr int kT = 2 * TQ::kBytes + TV::kBytes, kM = kT + TC::kBytes, kBytes = kM + C * LDC * 4, kCtas = kBytes <= 74 * 1024 ? 3 : 2;
+    static_assert(C * (LDC + LDI) * 4 <= TC::kBytes, "A and the inverse's scratch");
+};
+template <int DK, int DV>
+__global__ void __launch_bounds__(NT, PrepPlanes<DK, DV>::kCtas) k_prep_planes(Ptrs p) {
+    extern __shared__ __align__(16) unsigned char smb[];
+    typedef PrepPlanes<DK, DV> L;
+    typedef __nv_bfloat16 IO;
+    const typename L::TQ mQ(smb), mK(smb + L::TQ::kBytes);
+    const typename L::TV mV(smb + 2 * L::TQ::kBytes);
+    const typename L::TC mT(smb + L::kT);
+    float *sA = reinterpret_cast<float*>(smb + L::kT), *sS = sA + C * LDC, *sM = reinterpret_cast<float*>(smb + L::kM);
+    __shared__ __align__(16) float sg[C], sbeta[C], scq[C], sck[C], srq[C], srk[C];
+    const int ch = blockIdx.x, n = ch % p.N, bh = ch / p.N, b = bh / p.H, hh = bh % p.H, H = p.H, tid = threadIdx.x;
+    const int warp = tid >> 5, lane = tid & 31;
+    const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh;
+    const size_t wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
+    const int live = min(C, p.T - n * C);
+    sm100::grid_dep_wait();            // launched while the kernel before it drains
+    sm100::grid_dep_launch();
+    if (ch == 0 && tid == 0) *p.status = 0;
+    mQ.template fetch<NT>((const IO*)p.q + row0 * DK, (size_t)H * DK, live);
+    mK.template fetch<NT>((const IO*)p.k + row0 * DK, (size_t)H * DK, live);
+    mV.template fetch<NT>((const IO*)p.v + row0 * DV, (size_t)H * DV, live);
+    if (tid < C) {
+        const size_t r = row0 + (size_t)tid * H;
+        const bool in = tid < live;
+        const float la = (in && p.alpha) ? log_gate(ld((const IO*)p.alpha, r), p.logits) : 0.f;
+        const float be = in ? gate(ld((const IO*)p.beta, r), p.logits) : 0.f;
+        const float lm = (in && p.lam) ? gate(ld((const IO*)p.lam, r), p.logits) : 0.f;
+        scan64(la, sg);
+        p.g[wrow0 + tid] = sg[tid];
+        sbeta[tid] = be;
+        scq[tid] = lm; sck[tid] = 1.f; srq[tid] = 1.f; srk[tid] = 1.f;
+    }
+    fetch_wait();
+    __syncthreads();
+    if (p.rqk) {
+        const size_t nrows = (size_t)p.B * H * p.Tp;
+        for (int r = warp; r < C; r += NT / 32) {
+            float sq = 0.f, sk = 0.f;
+#pragma unroll
+            for (int d = 2 * lane; d < DK; d += 64) {
+                const float2 q = mQ.ld2(r, d), k = mK.ld2(r, d);
+                sq = fmaf(q.x, q.x, fmaf(q.y, q.y, sq));
+                sk = fmaf(k.x, k.x, fmaf(k.y, k.y, sk));
+            }
+            sq = warp_sum(sq); sk = warp_sum(sk);
+            if (lane == 0) {
+                const float rq = 1.f / sqrtf(sq + kNormEps), rk = 1.f / sqrtf(sk + kNormEps);
+                srq[r] = rq; srk[r] = rk;
+                scq[r] *= rq; sck[r] = rk;
+                p.rqk[wrow0 + r] = rq; p.rqk[nrows + wrow0 + r] = rk;
+            }
+        }
+        __syncthreads();
+    }
+    const int wm = (warp & 1) * 32, wn = warp >> 1;
+    {
+        float kk[2][2][4], qk[2][2][4];
+        zero(kk); zero(qk);
+        pmm<false, false>(kk, mK, mK, wm, wn * 16, DK);
+        pmm<false, false>(qk, mQ, mK, wm, wn * 16, DK);
+        // A = strictLower(beta_r Gamma_ri (x_r . k_i)),  P = Gamma o (Q K^T), causal including the diagonal
+        each2(kk, qk, wm, wn * 16, [&](int r, int i, float k0, float k1, float q0, float q1) {
+            const float e0 = i <= r ? expf(sg[r] - sg[i]) * srk[i] : 0.f, e1 = i + 1 <= r ? expf(sg[r] - sg[i + 1]) * srk[i + 1] : 0.f;
+            const float f = sbeta[r], cq = scq[r], ck = sck[r], rq = srq[r];
+            st2(sA + r * LDC + i, i < r ? f * e0 * fmaf(ck, k0, cq * q0) : 0.f, i + 1 < r ? f * e1 * fmaf(ck, k1, cq * q1) : 0.f);
+            st2((IO*)p.P + (wrow0 + r) * C + i, rq * e0 * q0, rq * e1 * q1);
+        });
+    }
+    __syncthreads();
+    invert_unit_lower(sA, sM, sS);
+    // T diag(f) into the planes
+    auto put_T = [&](auto f) {
+#pragma unroll
+        for (int e = tid * 4; e < C * C; e += NT * 4) {
+            const int r = e / C, i = e % C;
+            float4 m = *reinterpret_cast<const float4*>(sM + r * LDC + i);
+            m.x *= f(i); m.y *= f(i + 1); m.z *= f(i + 2); m.w *= f(i + 3);
+            mT.st4(r, i, m);
+        }
+        __syncthreads();
+    };
+    if (p.save)
+#pragma unroll
+        for (int e = tid * 4; e < C * C; e += NT * 4)
+            *reinterpret_cast<float4*>(p.M + wrow0 * C + e) = *reinterpret_cast<const float4*>(sM + (e / C) * LDC + e % C);
+    if (tid < C) { const float gm = expf(sg[tid]) * sbeta[tid]; scq[tid] *= gm; sck[tid] *= gm; }
+    put_T([&](int i) { return sbeta[i]; });
+    {
+        float u[2][DV / 32][4];
+        zero(u);
+        pmm<false, true>(u, mT, mV, wm, wn * (DV / 4), C);
+        each(u, wm, wn * (DV / 4), [&](int r, int j, float x, float y) { st2((IO*)p.U + (wrow0 + r) * DV + j, x, y); });
+    }
+    __syncthreads();
+    float w[2][DK / 32][4];
+    zero(w);
+    put_T([&](int i) { return sck[i]; });
+    pmm<false, true>(w, mT, mK, wm, wn * (DK / 4), C);
+    __syncthreads();
+    put_T([&](int i) { return scq[i]; });
+    pmm<false, true>(w, mT, mQ, wm, wn * (DK / 4), C);
+    each(w, wm, wn * (DK / 4), [&](int r, int d, float x, float y) { st2((IO*)p.W + (wrow0 + r) * DK + d, x, y); });
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1483,8 +1602,13 @@ cudaError_t launch(K kern, int grid, int threads, size_t smem, cudaStream_t stre
 
 template <typename IO, int DK, int DV>
 cudaError_t prep_for(const ChunkArgs& a, const Ptrs& p) {
-    constexpr size_t smem = sizeof(float) * (2 * C * (DK + kPad) + C * (DV + kPad) + 3 * C * LDC);
-    return launch(k_prep<IO, DK, DV>, a.s.B * a.s.H * p.N, NT, smem, a.stream, p);
+    const int grid = a.s.B * a.s.H * p.N;
+    if constexpr (sizeof(IO) == 2) {
+        return launch(k_prep_planes<DK, DV>, grid, NT, PrepPlanes<DK, DV>::kBytes, a.stream, p);
+    } else {
+        constexpr size_t smem = sizeof(float) * (2 * C * (DK + kPad) + C * (DV + kPad) + 2 * C * LDC + C * LDI);
+        return launch(k_prep<DK, DV>, grid, NT, smem, a.stream, p);
+    }
 }
 template <typename IO, int DK, int DS>
 cudaError_t chain_fwd_for(const ChunkArgs& a, const Ptrs& p) {
