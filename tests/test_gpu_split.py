@@ -2,8 +2,10 @@
 pair, ragged last chunks, against the oracle."""
 from dataclasses import replace
 
+import numpy as np
 import pytest
 
+import gpu_util as gu
 from paper_2606_08804_b200 import inputs as gen
 from test_gpu_chunk import _bwd_check, _fwd_check
 
@@ -27,3 +29,30 @@ def test_split_kernels(dtype, B, H, T, dk, dv):
     _fwd_check(cfg, d)
     _bwd_check(cfg, d)
     _bwd_check(cfg, d, reuse=True)
+
+
+@pytest.mark.parametrize("T,dk,dv,logits", [(97, 64, 64, False), (64, 128, 64, True), (65, 64, 128, False)])
+def test_split_kernels_normalise(T, dk, dv, logits):
+    # bf16 with d_k or d_v = 64, q and k normalised in the kernels (their own branch of the chunk backward)
+    from oracle import recurrence as orc
+    from paper_2606_08804_b200 import binding as qd
+    cfg = replace(gen.CONFIGS["cfg2"], B=2, H=3, T=T, dk=dk, dv=dv, regime="alpha_slow", seed=223)
+    d = gen.make_chunk_inputs(cfg)
+    r = np.random.default_rng(13)
+    rnd = lambda x: gen.round_bf16(x.astype(np.float32))
+    for n in ("q", "k"):
+        d[n] = rnd(d[n] * np.exp(r.normal(0.0, 1.0, d[n].shape[:-1] + (1,))))
+    if logits:
+        shp = (cfg.B, cfg.T, cfg.H)
+        d["beta"], d["alpha"], d["lam"] = rnd(r.normal(0.0, 1.5, shp)), rnd(r.normal(3.0, 1.5, shp)), rnd(r.normal(-0.8, 1.0, shp))
+    t = gu.dev_inputs(d, cfg.dtype)
+    args = (d["q"], d["k"], d["v"], d["beta"], d["alpha"], d["lam"], d["h0"])
+    ro, rh = orc.forward_fused(*args, logits=logits, norm_qk=True)
+    ref = orc.backward_fused(*args, d["dO"], d["dhT"], logits=logits, norm_qk=True)
+    dev = [t[n] for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")]
+    o, hT, ws = qd.chunk_fwd(*dev, save_for_bwd=True, logits=logits, norm_qk=True)
+    g = qd.chunk_bwd(*dev, t["dO"], t["dhT"], workspace=ws, reuse_fwd=True, logits=logits, norm_qk=True)
+    gu.check("split norm", "o", o, ro, cfg.dtype)
+    gu.check("split norm", "hT", hT, rh, cfg.dtype, state=True)
+    for n in ("dq", "dk", "dv", "dbeta", "dalpha", "dlam", "dh0"):
+        gu.check("split norm", n, g[n], ref[n], cfg.dtype, state=(n == "dh0"))
