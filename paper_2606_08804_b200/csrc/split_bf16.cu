@@ -11,7 +11,7 @@ namespace {
 // K1: per chunk-head, state-independent part: g, P, W<-, U~ (and M for the backward).  X is never formed, X K^T and T diag(gamma) X are each a product with K and one
 // with Q, their coefficients applied to the result or to T.  One set of planes holds T, T diag(gamma / |k|) and
 // T diag(lambda gamma / |q|) in turn, over what the inverse needed; at d_k = d_v = 64 three CTAs fit an SM.
-// 1024 chunks of 64 x 64: 72 us with tf32 halves and two CTAs, 56 so (d_k 128, d_v 64: 119 and 70), bound by the latency of its
+// 1024 chunks of 64 x 64: 72 us with tf32 halves and two CTAs, 50 so (d_k 128, d_v 64: 119 and 64), bound by the latency of its
 // chain of small steps.
 template <int DK, int DV>
 struct PrepPlanes {

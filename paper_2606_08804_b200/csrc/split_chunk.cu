@@ -7,7 +7,6 @@
 // multiply-adds here.  Operands live in shared memory as fp32 tiles with padded rows; each kernel reads every global
 // operand once.
 #include "split_common.cuh"
-#include "tf32.cuh"
 
 namespace qd {
 
@@ -21,70 +20,6 @@ namespace {
 
 constexpr int kPad = 4;            // of a d-wide tile: rows g, columns t of a fragment fall on banks 4 g + t
 
-// ---- products -----------------------------------------------------------------------------------------------------
-// acc += A B for the (16 MT) x (8 NTL) tile of this warp at row m0, column n0: contraction extent K, a(m, k) and b(k, n)
-// fetch the operands.  Lane (g = lane / 4, t = lane % 4) holds, of every
-// 16 x 8 piece, rows g and g + 8, columns 2t and 2t + 1.
-// The tensor instruction truncates as it accumulates, which over a long contraction biases the sum by 1e-6 of itself; so it
-// only sums 16 terms at a time, from zero, and those sums are added with rounded fp32 additions.
-// Measured against fp64 on 1024 tokens: slowly forgetting gates, rms error of the outputs 1.2e-6 without, 2.9e-7 with, 2.6e-7 for plain fp32 FMAs.
-__device__ __forceinline__ void add2(float& x, float& y, float a, float b) {
-    asm("{\n\t.reg .b64 u, v;\n\tmov.b64 u, {%0, %1};\n\tmov.b64 v, {%2, %3};\n\tadd.rn.f32x2 u, u, v;\n\tmov.b64 {%0, %1}, u;\n\t}"
-        : "+f"(x), "+f"(y) : "f"(a), "f"(b));
-}
-template <int MT, int NTL, class FA, class FB>
-__device__ __forceinline__ void wmm(float (&acc)[MT][NTL][4], int m0, int n0, int K, FA a, FB b) {
-    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
-    constexpr int KS = 2, JN = NTL > 2 ? 2 : NTL;      // k steps per group; columns whose sums are open at a time
-#pragma unroll 1
-    for (int k0 = 0; k0 < K; k0 += 8 * KS) {
-        uint32_t ah[KS][MT][4], al[KS][MT][4];
-#pragma unroll
-        for (int s = 0; s < KS; ++s)
-#pragma unroll
-            for (int i = 0; i < MT; ++i)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float x = a(m0 + 16 * i + g + 8 * (e & 1), k0 + 8 * s + t + 4 * (e >> 1));
-                    tf32_split(x, ah[s][i][e], al[s][i][e]);
-                }
-#pragma unroll
-        for (int jb = 0; jb < NTL; jb += JN) {
-            float part[MT][JN][4];
-#pragma unroll
-            for (int i = 0; i < MT; ++i)
-#pragma unroll
-                for (int j = 0; j < JN; ++j)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) part[i][j][e] = 0.f;
-#pragma unroll
-            for (int s = 0; s < KS; ++s) {
-                uint32_t bh[JN][2], bl[JN][2];
-#pragma unroll
-                for (int j = 0; j < JN; ++j)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const float x = b(k0 + 8 * s + t + 4 * e, n0 + 8 * (jb + j) + g);
-                        tf32_split(x, bh[j][e], bl[j][e]);
-                    }
-#pragma unroll
-                for (int term = 0; term < 3; ++term)                         // lo hi, hi lo, hi hi
-#pragma unroll
-                    for (int i = 0; i < MT; ++i)
-#pragma unroll
-                        for (int j = 0; j < JN; ++j)
-                            mma_tf32(part[i][j], term == 0 ? al[s][i] : ah[s][i], term == 1 ? bl[j] : bh[j]);
-            }
-#pragma unroll
-            for (int i = 0; i < MT; ++i)
-#pragma unroll
-                for (int j = 0; j < JN; ++j) {
-                    add2(acc[i][jb + j][0], acc[i][jb + j][1], part[i][j][0], part[i][j][1]);
-                    add2(acc[i][jb + j][2], acc[i][jb + j][3], part[i][j][2], part[i][j][3]);
-                }
-        }
-    }
-}
 // ---- tiles --------------------------------------------------------------------------------------------------------
 // A ROWS x W tile on its way from global memory (rows `stride` elements apart, rows >= live read as zeros) through
 // registers into shared memory with leading dimension LD.  All loads of a tile are in flight together, and a
