@@ -85,10 +85,11 @@ __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-// acc += A B for the (16 MT) x (8 NTL) tile of this warp at row m0 (pieces of 16 rows MS apart), column n0, contraction extent K.  A is stored as [m][k], or
+// acc += A B for the (16 MT) x (8 NTL) tile of this warp at row m0 (pieces of 16 rows MS apart), column n0, contraction over [kb, k1):
+// a triangular operand is read from or up to its diagonal only.  A is stored as [m][k], or
 // as [k][m] with AT; B as [n][k], or as [k][n] with BT.  Fragments of acc: rows g and g + 8, columns 2t and 2t + 1.
 template <bool AT, bool BT, int MT, int NTL, class MA, class MB, int MS = 16>
-__device__ __forceinline__ void pmm(float (&acc)[MT][NTL][4], const MA& A, const MB& B, int m0, int n0, int K) {
+__device__ __forceinline__ void pmm(float (&acc)[MT][NTL][4], const MA& A, const MB& B, int m0, int n0, int k1, int kb = 0) {
     static_assert(NTL % 2 == 0, "columns come in pairs of 8");
     constexpr int PA = MA::NP, PB = MB::NP;
     const int lane = threadIdx.x & 31;
@@ -97,7 +98,7 @@ __device__ __forceinline__ void pmm(float (&acc)[MT][NTL][4], const MA& A, const
     const __nv_bfloat16* pb = B.p + (BT ? (lane & 15) * MB::LD + n0 + (lane >> 4) * 8
                                         : (n0 + (lane & 7) + (lane >> 4) * 8) * MB::LD + ((lane >> 3) & 1) * 8);
 #pragma unroll 2
-    for (int k0 = 0; k0 < K; k0 += 16) {
+    for (int k0 = kb; k0 < k1; k0 += 16) {
         uint32_t a[MT][PA][4];
 #pragma unroll
         for (int i = 0; i < MT; ++i)

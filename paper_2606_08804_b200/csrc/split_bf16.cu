@@ -79,8 +79,10 @@ __global__ void __launch_bounds__(NT, PrepPlanes<DK, DV>::kCtas) k_prep(Ptrs p) 
     {
         float kk[2][2][4], qk[2][2][4];
         zero(kk); zero(qk);
-        pmm<false, false>(kk, mK, mK, wm, wn * 16, DK);
-        pmm<false, false>(qk, mQ, mK, wm, wn * 16, DK);
+        if (wn * 16 < wm + 32) {                                // not above the diagonal
+            pmm<false, false>(kk, mK, mK, wm, wn * 16, DK);
+            pmm<false, false>(qk, mQ, mK, wm, wn * 16, DK);
+        }
         // A = strictLower(beta_r Gamma_ri (x_r . k_i)),  P = Gamma o (Q K^T), causal including the diagonal
         each2(kk, qk, wm, wn * 16, [&](int r, int i, float k0, float k1, float q0, float q1) {
             const float e0 = i <= r ? expf(sg[r] - sg[i]) * srk[i] : 0.f, e1 = i + 1 <= r ? expf(sg[r] - sg[i + 1]) * srk[i + 1] : 0.f;
@@ -111,17 +113,17 @@ __global__ void __launch_bounds__(NT, PrepPlanes<DK, DV>::kCtas) k_prep(Ptrs p) 
     {
         float u[2][DV / 32][4];
         zero(u);
-        pmm<false, true>(u, mT, mV, wm, wn * (DV / 4), C);
+        pmm<false, true>(u, mT, mV, wm, wn * (DV / 4), wm + 32);
         each(u, wm, wn * (DV / 4), [&](int r, int j, float x, float y) { st2((IO*)p.U + (wrow0 + r) * DV + j, x, y); });
     }
     __syncthreads();
     float w[2][DK / 32][4];
     zero(w);
     put_T([&](int i) { return sck[i]; });
-    pmm<false, true>(w, mT, mK, wm, wn * (DK / 4), C);
+    pmm<false, true>(w, mT, mK, wm, wn * (DK / 4), wm + 32);
     __syncthreads();
     put_T([&](int i) { return scq[i]; });
-    pmm<false, true>(w, mT, mQ, wm, wn * (DK / 4), C);
+    pmm<false, true>(w, mT, mQ, wm, wn * (DK / 4), wm + 32);
     each(w, wm, wn * (DK / 4), [&](int r, int d, float x, float y) { st2((IO*)p.W + (wrow0 + r) * DK + d, x, y); });
 }
 
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
             });
         }
         // o = diag(gamma) Q h + P Delta
-        pmm<false, true>(o, mP, mD, wm, wn, C);
+        pmm<false, true>(o, mP, mD, wm, wn, wm + 16);
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
                 s += __shfl_xor_sync(0xffffffffu, s, 2);
                 if (t == 0) skd[warp >> 2][wm + 8 * h + g] = s;
             }
-            pmm<true, true>(c, mP, mO, wm, wn, C);
+            pmm<true, true>(c, mP, mO, wm, wn, C, wm);
             each2(a, c, wm, wn, [&](int s, int j, float x, float y, float u, float v) {
                 x += u; y += v;
                 mdD.st2(s, j, -x, -y);
@@ -428,6 +430,8 @@ __global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>
     const size_t nrows = (size_t)p.B * H * p.Tp;
     const int live = min(C, p.T - n * C);
     const int wr = warp % WR, wm = wr * 16 * MT, wn = warp / WR, nc = wn * 16, nk = wn * (DK / 4), nv = wn * (DV / 4);
+    const int re = wm + 16 * MT;                                // a 64 x 64 tile of this warp matters only if it
+    const bool low = nc < re;                                   // reaches below the diagonal
     // sums over this warp's rows of each of its 16 columns, to dst[column]
     auto col_sums = [&](float (&a)[MT][2][4], float* dst) {
 #pragma unroll
@@ -476,7 +480,7 @@ __global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>
     // ---- dP with its uses: dP o P (row and column sums), dP o Gamma;  dk <- diag(gamma_C/gamma) Delta dh^T ----
     float a3[MT][2][4], aK[MT][NK][4], aQ[MT][NK][4], aX[MT][NK][4];
     zero(a3); zero(aK); zero(aQ); zero(aX);
-    pmm<false, false>(a3, mO, mD, wm, nc, DV);
+    if (low) pmm<false, false>(a3, mO, mD, wm, nc, DV);
     {
         float a[MT][2][4];
 #pragma unroll
@@ -507,11 +511,11 @@ __global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>
     zero(aT);
     pmm<false, false>(aQ, mO, mS, wm, nk, DV);
     pmm<false, false>(aX, mdD, mS, wm, nk, DV);
-    pmm<false, false>(aT, mdD, mV, wm, nc, DV);
+    if (low) pmm<false, false>(aT, mdD, mV, wm, nc, DV);
     {
         float a[MT][NV][4];
         zero(a);
-        pmm<true, true>(a, mM, mdD, wm, nv, C);
+        pmm<true, true>(a, mM, mdD, wm, nv, C, wm);
         each(a, wm, nv, [&](int s, int j, float x, float y) {
             if (s < live) st2((IO*)p.dv_ + (row0 + (size_t)s * H) * DV + j, sbeta[s] * x, sbeta[s] * y);
         });
@@ -527,12 +531,12 @@ __global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>
     {
         float a[MT][2][4];
         zero(a);
-        pmm<false, false>(a, mW, mK, wm, nc, DK);
+        if (low) pmm<false, false>(a, mW, mK, wm, nc, DK);
         each2(aT, a, wm, nc, [&](int, int s, float& x, float& y, float u, float v) {
             x = fmaf(sgam[s] * srk[s], u, x); y = fmaf(sgam[s + 1] * srk[s + 1], v, y);
         });
         zero(a);
-        pmm<false, false>(a, mW, mQ, wm, nc, DK);
+        if (low) pmm<false, false>(a, mW, mQ, wm, nc, DK);
         each2(aT, a, wm, nc, [&](int, int s, float& x, float& y, float u, float v) {
             x = fmaf(sgam[s] * scq[s], u, x); y = fmaf(sgam[s + 1] * scq[s + 1], v, y);
         });
@@ -544,7 +548,7 @@ __global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>
         col_sums(aT, pcol[1][wr]);
     }
     zero(aX);
-    pmm<true, true>(aX, mM, mW, wm, nk, C);
+    pmm<true, true>(aX, mM, mW, wm, nk, C, wm);
     each(aX, wm, nk, [&](int s, int, float& x, float& y) { const float f = sbeta[s] * sgam[s]; x *= f; y *= f; });
     row_sums(aX, wm, nk, prow[2][wn], [&](int r, int i, float x, float y) {
         const float2 k = mK.ld2(r, i), q = mQ.ld2(r, i);
@@ -555,20 +559,22 @@ __global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>
     {
         float a[MT][2][4];
         zero(a);
-        pmm<false, false>(a, mT, mM, wm, nc, C);
+        if (low) pmm<false, false>(a, mT, mM, wm, nc, nc + 16);
         each(a, wm, nc, [&](int r, int s, float x, float y) { m4.st2(r, s, x, y); });
     }
     __syncthreads();
     {
         float a[MT][2][4], x[MT][2][4];
         zero(a); zero(x);
-        pmm<true, true>(a, mM, m4, wm, nc, C);
-        pmm<false, false>(x, mQ, mK, wm, nc, DK);               // X K^T
+        if (low) {
+            pmm<true, true>(a, mM, m4, wm, nc, C, wm);
+            pmm<false, false>(x, mQ, mK, wm, nc, DK);           // X K^T
+        }
         each(x, wm, nc, [&](int r, int, float& u, float& v) { u *= scq[r]; v *= scq[r]; });
         {
             float y[MT][2][4];
             zero(y);
-            pmm<false, false>(y, mK, mK, wm, nc, DK);
+            if (low) pmm<false, false>(y, mK, mK, wm, nc, DK);
             each2(x, y, wm, nc, [&](int r, int s, float& u, float& v, float k0, float k1) {
                 u = srk[s] * fmaf(srk[r], k0, u); v = srk[s + 1] * fmaf(srk[r], k1, v);
             });
@@ -602,10 +608,10 @@ __global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>
         col_sums(x, pcol[2][wr]);
         __syncthreads();
         // ---- dX += dXK K;  dk += dXK^T X + dPG^T Q + dX;  dq += dPG K + lambda dX ----------------------
-        pmm<false, true>(aX, e1, mK, wm, nk, C);
+        pmm<false, true>(aX, e1, mK, wm, nk, re);
         row_sums(aX, wm, nk, prow[4][wn], qsum);
-        pmm<false, true>(aQ, e2, mK, wm, nk, C);
-        pmm<true, true>(aK, e3, mQ, wm, nk, C);
+        pmm<false, true>(aQ, e2, mK, wm, nk, re);
+        pmm<true, true>(aK, e3, mQ, wm, nk, C, wm);
         if (p.rqk) {                                            // dXK scaled by row instead of by column
             __syncthreads();
             each(a, wm, nc, [&](int r, int s, float, float) {
@@ -614,7 +620,7 @@ __global__ void __launch_bounds__(BwdPlanes<DK, DV>::kThreads, BwdPlanes<DK, DV>
             });
             __syncthreads();
         }
-        pmm<true, true>(aK, e1, mK, wm, nk, C);
+        pmm<true, true>(aK, e1, mK, wm, nk, C, wm);
     }
     each2(aQ, aX, wm, nk, [&](int r, int, float& x, float& y, float u, float v) { x = fmaf(slam[r], u, x); y = fmaf(slam[r], v, y); });
     each2(aK, aX, wm, nk, [&](int, int, float& x, float& y, float u, float v) { x += u; y += v; });
