@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(NT, PrepPlanes<DK, DV>::kCtas) k_prep(Ptrs p) 
         }
         __syncthreads();
     }
-    const int wm = (warp & 1) * 32, wn = warp >> 1;
+    const int wm = ((warp ^ (warp >> 2)) & 1) * 32, wn = warp >> 1;      // both halves of the rows on every scheduler
     {
         float kk[2][2][4], qk[2][2][4];
         zero(kk); zero(qk);
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
     __shared__ float sgq[2][C], sgk[2][C], sgC[2];
     const int H = p.H, nsl = DV / DS, j0 = (blockIdx.x % nsl) * DS, bh = blockIdx.x / nsl, b = bh / H, hh = bh % H;
     const int tid = threadIdx.x, warp = tid >> 5, g = (tid & 31) >> 2, t = tid & 3;
-    const int wm = (warp & 3) * 16, wn = (warp >> 2) * 16, si = (warp & 3) * 16 * MU;
+    const int wm = (warp & 4 ? 3 - (warp & 3) : warp & 3) * 16, wn = (warp >> 2) * 16, si = (warp & 3) * 16 * MU;
     const size_t nrows = (size_t)p.B * H * p.Tp, row0 = (size_t)b * p.T * H + hh, wrow0 = (size_t)bh * p.Tp;
     sm100::grid_dep_wait();            // launched while the kernel before it drains
     sm100::grid_dep_launch();
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
     __shared__ float sgq[2][C], sgk[2][C], sgC[2], sred[TH / 32], skd[DS / 16][C];
     const int H = p.H, nsl = DV / DS, sl = blockIdx.x % nsl, j0 = sl * DS, bh = blockIdx.x / nsl, b = bh / H, hh = bh % H;
     const int tid = threadIdx.x, warp = tid >> 5, g = (tid & 31) >> 2, t = tid & 3;
-    const int wm = (warp & 3) * 16, wn = (warp >> 2) * 16, si = (warp & 3) * 16 * MU;
+    const int wm = (warp & 4 ? 3 - (warp & 3) : warp & 3) * 16, wn = (warp >> 2) * 16, si = (warp & 3) * 16 * MU;
     const size_t nrows = (size_t)p.B * H * p.Tp, BHN = (size_t)p.B * H * p.N, row0 = (size_t)b * p.T * H + hh, wrow0 = (size_t)bh * p.Tp;
     sm100::grid_dep_wait();            // launched while the kernel before it drains
     sm100::grid_dep_launch();

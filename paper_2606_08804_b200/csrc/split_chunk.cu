@@ -112,13 +112,15 @@ __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
     }
     // x_r = (1/|k_r|) k_r + (lambda_r / |q_r|) q_r; the stored rows stay as they are, exact in their storage type
     auto Xf = [&](int r, int d) { return fmaf(scq[r], sQ[r * LK + d], sck[r] * sK[r * LK + d]); };
-    const int wm = (warp & 1) * 32, wn = warp >> 1;
+    const int wm = ((warp ^ (warp >> 2)) & 1) * 32, wn = warp >> 1;      // both halves of the rows on every scheduler
     {
         float a1[2][2][4], a2[2][2][4];
         zero(a1); zero(a2);
         auto Kt = [&](int d, int i) { return sK[i * LK + d]; };
-        wmm<2, 2>(a1, wm, wn * 16, DK, Xf, Kt);
-        wmm<2, 2>(a2, wm, wn * 16, DK, [&](int r, int d) { return sQ[r * LK + d]; }, Kt);
+        if (wn * 16 < wm + 32) {                                // not above the diagonal
+            wmm<2, 2>(a1, wm, wn * 16, DK, Xf, Kt);
+            wmm<2, 2>(a2, wm, wn * 16, DK, [&](int r, int d) { return sQ[r * LK + d]; }, Kt);
+        }
         // A = strictLower(beta_r Gamma_ri (x_r . k_i)),  P = Gamma o (Q K^T), causal including the diagonal
         each(a1, wm, wn * 16, [&](int r, int i, float x, float y) {
             const float f = sbeta[r];
@@ -148,13 +150,13 @@ __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
     {
         float u[2][DV / 32][4];
         zero(u);
-        wmm<2, DV / 32>(u, wm, wn * (DV / 4), C, Tf, [&](int i, int j) { return sV[i * LV + j]; });
+        wmm<2, DV / 32>(u, wm, wn * (DV / 4), wm + 32, Tf, [&](int i, int j) { return sV[i * LV + j]; });
         each(u, wm, wn * (DV / 4), [&](int r, int j, float x, float y) { st2((float*)p.U + (wrow0 + r) * DV + j, x, y); });
     }
     {
         float w[2][DK / 32][4];
         zero(w);
-        wmm<2, DK / 32>(w, wm, wn * (DK / 4), C, Tf, Xf);
+        wmm<2, DK / 32>(w, wm, wn * (DK / 4), wm + 32, Tf, Xf);
         each(w, wm, wn * (DK / 4), [&](int r, int d, float x, float y) { st2((float*)p.W + (wrow0 + r) * DK + d, x, y); });
     }
 }
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
             const float s0 = sgq[m0 + gq], s1 = sgq[m0 + 8 + gq];
 #pragma unroll
             for (int j = 0; j < NS; ++j) { acc[0][j][0] *= s0; acc[0][j][1] *= s0; acc[0][j][2] *= s1; acc[0][j][3] *= s1; }
-            wmm<1, NS>(acc, m0, 0, C, [&](int r, int s) { return sP[r * LDC + s]; },
+            wmm<1, NS>(acc, m0, 0, m0 + 16, [&](int r, int s) { return sP[r * LDC + s]; },
                                   [&](int s, int j) { return sD[s * LS + j]; });
             each(acc, m0, 0, [&](int r, int j, float x, float y) {
                 if (r < live) st2((float*)p.o + (row0 + (size_t)r * H) * DV + j0 + j, x, y);
@@ -402,6 +404,7 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     const float* hs = p.hs + ((size_t)bh * p.N + n) * DK * DV;
     const float* dhs = p.dhs + ((size_t)bh * p.N + n) * DK * DV;
     const int wm = (warp & 1) * 32, wn = warp >> 1, nc = wn * 16, nk = wn * (DK / 4);
+    const bool low = nc < wm + 32;                              // a 64 x 64 tile of this warp matters only if it reaches below the diagonal
 
     Tile<C, DK, LT> tq, tk;
     Tile<C, DV, LT> tv;
@@ -435,10 +438,10 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     {
         float a[2][2][4];
         zero(a);
-        wmm<2, 2>(a, wm, nc, DK, Xf, [&](int d, int i) { return s1[i * LT + d]; });
+        if (low) wmm<2, 2>(a, wm, nc, DK, Xf, [&](int d, int i) { return s1[i * LT + d]; });
         each(a, wm, nc, [&](int r, int i, float x, float y) { st2(m0 + r * LDC + i, x * srk[i], y * srk[i + 1]); });
         zero(a);
-        wmm<2, 2>(a, wm, nc, DV, [&](int r, int j) { return s2[r * LT + j]; }, [&](int j, int s) { return s3[s * LT + j]; });
+        if (low) wmm<2, 2>(a, wm, nc, DV, [&](int r, int j) { return s2[r * LT + j]; }, [&](int j, int s) { return s3[s * LT + j]; });
         each(a, wm, nc, [&](int r, int s, float& x, float& y) {
             const float2 pv = ld2((const float*)p.P + (wrow0 + r) * C + s);
             const float d0 = s <= r ? x : 0.f, d1 = s + 1 <= r ? y : 0.f;
@@ -483,12 +486,12 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     // ---- dT = dDelta V^T + dW<- (gamma X)^T;  dV = T^T dDelta -------------------------------------
     float aT[2][2][4];
     zero(aT);
-    wmm<2, 2>(aT, wm, nc, DV, [&](int r, int j) { return s3[r * LT + j]; }, [&](int j, int s) { return s0[s * LT + j]; });
+    if (low) wmm<2, 2>(aT, wm, nc, DV, [&](int r, int j) { return s3[r * LT + j]; }, [&](int j, int s) { return s0[s * LT + j]; });
     {
         float a[2][DV / 32][4];
         zero(a);
         wmm<2, DV / 32>(a, wm, wn * (DV / 4), C, [&](int s, int r) { return m1[r * LDC + s]; },
-                               [&](int r, int j) { return s3[r * LT + j]; });
+                               [&](int r, int j) { return s3[r * LT + j]; }, wm);
         each(a, wm, wn * (DV / 4), [&](int s, int j, float x, float y) {
             if (s < live) st2((float*)p.dv_ + (row0 + (size_t)s * H) * DV + j, sbeta[s] * x, sbeta[s] * y);
         });
@@ -499,7 +502,7 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     {
         float a[2][2][4];
         zero(a);
-        wmm<2, 2>(a, wm, nc, DK, [&](int r, int i) { return s2[r * LT + i]; }, [&](int i, int s) { return Xf(s, i); });
+        if (low) wmm<2, 2>(a, wm, nc, DK, [&](int r, int i) { return s2[r * LT + i]; }, [&](int i, int s) { return Xf(s, i); });
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -513,7 +516,7 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     }
     // ---- dX <- diag(gamma) T^T dW<-; the row sums t1 = <dQ1, Q>, t2 = <dXg, gamma X> -----------------
     zero(aX);
-    wmm<2, NK>(aX, wm, nk, C, [&](int s, int r) { return m1[r * LDC + s]; }, [&](int r, int i) { return s2[r * LT + i]; });
+    wmm<2, NK>(aX, wm, nk, C, [&](int s, int r) { return m1[r * LDC + s]; }, [&](int r, int i) { return s2[r * LT + i]; }, wm);
     each(aX, wm, nk, [&](int s, int, float& x, float& y) { const float f = sbeta[s] * sgam[s]; x *= f; y *= f; });
     row_sums(aX, wm, nk, prow[2][wn], [&](int r, int i, float x, float y) { return fmaf(x, Xf(r, i), y * Xf(r, i + 1)); });
     row_sums(aQ, wm, nk, prow[1][wn],
@@ -528,14 +531,14 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
         part[q4][col] = s;
         float a[2][2][4];
         zero(a);
-        wmm<2, 2>(a, wm, nc, C, [&](int r, int u) { return m2[r * LDC + u] * sbeta[u]; }, [&](int u, int s2_) { return m1[s2_ * LDC + u]; });
+        if (low) wmm<2, 2>(a, wm, nc, nc + 16, [&](int r, int u) { return m2[r * LDC + u] * sbeta[u]; }, [&](int u, int s2_) { return m1[s2_ * LDC + u]; });
         each(a, wm, nc, [&](int r, int s_, float x, float y) { st2(m4 + r * LDC + s_, x, y); });
     }
     __syncthreads();
     {
         float a[2][2][4];
         zero(a);
-        wmm<2, 2>(a, wm, nc, C, [&](int r, int u) { return m1[u * LDC + r]; }, [&](int u, int s) { return m4[u * LDC + s]; });
+        if (low) wmm<2, 2>(a, wm, nc, C, [&](int r, int u) { return m1[u * LDC + r]; }, [&](int u, int s) { return m4[u * LDC + s]; }, wm);
         // its uses: d beta (row sums), dA o A (column sums), d(X K^T)
         each(a, wm, nc, [&](int r, int s, float& x, float& y) {
             const float e0 = s < r ? -x * expf(sg[r] - sg[s]) : 0.f, e1 = s + 1 < r ? -y * expf(sg[r] - sg[s + 1]) : 0.f;
@@ -549,12 +552,12 @@ __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
     }
     __syncthreads();
     // ---- dX += dXK K;  dk += dXK^T X + dPG^T Q + dX;  dq += dPG K + lambda dX ----------------------
-    wmm<2, NK>(aX, wm, nk, C, [&](int r, int s) { return m2[r * LDC + s]; }, [&](int s, int d) { return srk[s] * Kf(s, d); });
+    wmm<2, NK>(aX, wm, nk, wm + 32, [&](int r, int s) { return m2[r * LDC + s]; }, [&](int s, int d) { return srk[s] * Kf(s, d); });
     row_sums(aX, wm, nk, prow[4][wn],
              [&](int r, int i, float x, float y) { return srq[r] * fmaf(x, Qf(r, i), y * Qf(r, i + 1)); });
-    wmm<2, NK>(aK, wm, nk, C, [&](int i, int r) { return m2[r * LDC + i]; }, Xf);
-    wmm<2, NK>(aK, wm, nk, C, [&](int i, int r) { return m3[r * LDC + i]; }, [&](int r, int d) { return srq[r] * Qf(r, d); });
-    wmm<2, NK>(aQ, wm, nk, C, [&](int r, int s) { return m3[r * LDC + s]; }, [&](int s, int d) { return srk[s] * Kf(s, d); });
+    wmm<2, NK>(aK, wm, nk, C, [&](int i, int r) { return m2[r * LDC + i]; }, Xf, wm);
+    wmm<2, NK>(aK, wm, nk, C, [&](int i, int r) { return m3[r * LDC + i]; }, [&](int r, int d) { return srq[r] * Qf(r, d); }, wm);
+    wmm<2, NK>(aQ, wm, nk, wm + 32, [&](int r, int s) { return m3[r * LDC + s]; }, [&](int s, int d) { return srk[s] * Kf(s, d); });
     {
         const int g = (tid & 31) >> 2;
 #pragma unroll

@@ -40,7 +40,7 @@ struct Ptrs {
 };
 
 // ---- products -----------------------------------------------------------------------------------------------------
-// acc += A B for the (16 MT) x (8 NTL) tile of this warp at row m0, column n0: contraction extent K, a(m, k) and b(k, n)
+// acc += A B for the (16 MT) x (8 NTL) tile of this warp at row m0, column n0: contraction over [kb, k1), a(m, k) and b(k, n)
 // fetch the operands.  Lane (g = lane / 4, t = lane % 4) holds, of every
 // 16 x 8 piece, rows g and g + 8, columns 2t and 2t + 1.
 // The tensor instruction truncates as it accumulates, which over a long contraction biases the sum by 1e-6 of itself; so it
@@ -51,11 +51,11 @@ __device__ __forceinline__ void add2(float& x, float& y, float a, float b) {
         : "+f"(x), "+f"(y) : "f"(a), "f"(b));
 }
 template <int MT, int NTL, class FA, class FB>
-__device__ __forceinline__ void wmm(float (&acc)[MT][NTL][4], int m0, int n0, int K, FA a, FB b) {
+__device__ __forceinline__ void wmm(float (&acc)[MT][NTL][4], int m0, int n0, int k1, FA a, FB b, int kb = 0) {
     const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
     constexpr int KS = 2, JN = NTL > 2 ? 2 : NTL;      // k steps per group; columns whose sums are open at a time
 #pragma unroll 1
-    for (int k0 = 0; k0 < K; k0 += 8 * KS) {
+    for (int k0 = kb; k0 < k1; k0 += 8 * KS) {
         uint32_t ah[KS][MT][4], al[KS][MT][4];
 #pragma unroll
         for (int s = 0; s < KS; ++s)
