@@ -11,7 +11,7 @@ namespace {
 // K1: per chunk-head, state-independent part: g, P, W<-, U~ (and M for the backward).  X is never formed, X K^T and T diag(gamma) X are each a product with K and one
 // with Q, their coefficients applied to the result or to T.  One set of planes holds T, T diag(gamma / |k|) and
 // T diag(lambda gamma / |q|) in turn, over what the inverse needed; at d_k = d_v = 64 three CTAs fit an SM.
-// 1024 chunks of 64 x 64: 72 us with tf32 halves and two CTAs, 50 so (d_k 128, d_v 64: 119 and 64), bound by the latency of its
+// 1024 chunks of 64 x 64: 72 us with tf32 halves and two CTAs, 50 so (d_k 128, d_v 64: 119 and 60), bound by the latency of its
 // chain of small steps.
 template <int DK, int DV>
 struct PrepPlanes {
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
 // h, dW<- and dT M^T in turn; M takes Delta's place, dT that of dO, dDelta and V.  So two CTAs fit an SM at d_k = d_v = 64: one
 // computes while the other loads or waits at a barrier, and a warp's 32 x 16 tile reads 1.5 operand pieces per 16 x 16 x 16
 // product, half of what 16 x 16 tiles of 16 warps would.  B4 T1024 H16 d_k = d_v = 64: 208 us with tf32 halves, 150 with 16
-// warps and one CTA, 122 so.
+// warps and one CTA, 122 so, 115 with triangular operands read from or to their diagonal only.
 template <int DK, int DV>
 struct BwdPlanes {
     typedef Planes<C, DK, 1> TQ;
