@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
         float a[2][2][4], o[1][2][4];
         zero(a); zero(o);
         mWQ.p = reinterpret_cast<IO*>(smb + bf * L::TA2::kBytes);
-        pmm<false, true, 2, 2, typename L::TA2, typename L::TS, C>(a, mWQ, mS, wm, wn, DK);
+        pmm<false, true, 4, 2, 2, typename L::TA2, typename L::TS, C>(a, mWQ, mS, wm, wn, DK);
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
         {
             float s[MU][2][4];
             zero(s);
-            pmm<true, true>(s, mK, mDs, si, wn, C);
+            pmm<true, true, 4>(s, mK, mDs, si, wn, C);
             const float gc = sgC[bf];
             each2(hst, s, si, wn, [&](int i, int j, float& x, float& y, float dx, float dy) {
                 x = fmaf(gc, x, dx); y = fmaf(gc, y, dy);
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
             });
         }
         // o = diag(gamma) Q h + P Delta
-        pmm<false, true>(o, mP, mD, wm, wn, wm + 16);
+        pmm<false, true, 4>(o, mP, mD, wm, wn, wm + 16);
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
         {
             float a[1][2][4], c[1][2][4];
             zero(a); zero(c);
-            pmm<false, true>(a, mK, mS, wm, wn, DK);
+            pmm<false, true, 4>(a, mK, mS, wm, wn, DK);
             each(a, wm, wn, [&](int r, int, float& x, float& y) { x *= sgk[bf][r]; y *= sgk[bf][r]; });
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
                 s += __shfl_xor_sync(0xffffffffu, s, 2);
                 if (t == 0) skd[warp >> 2][wm + 8 * h + g] = s;
             }
-            pmm<true, true>(c, mP, mO, wm, wn, C, wm);
+            pmm<true, true, 4>(c, mP, mO, wm, wn, C, wm);
             each2(a, c, wm, wn, [&](int s, int j, float x, float y, float u, float v) {
                 x += u; y += v;
                 mdD.st2(s, j, -x, -y);
@@ -377,8 +377,8 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
         {
             float s[MU][2][4];
             zero(s);
-            pmm<true, true>(s, mQ, mOs, si, wn, C);
-            pmm<true, true>(s, mW, mdD, si, wn, C);
+            pmm<true, true, 4>(s, mQ, mOs, si, wn, C);
+            pmm<true, true, 4>(s, mW, mdD, si, wn, C);
             const float gc = sgC[bf];
             each2(dst, s, si, wn, [&](int i, int j, float& x, float& y, float dx, float dy) {
                 x = fmaf(gc, x, dx); y = fmaf(gc, y, dy);
