@@ -128,11 +128,12 @@ __global__ void __launch_bounds__(NT, PrepPlanes<DK, DV>::kCtas) k_prep(Ptrs p) 
 }
 
 // ---------------------------------------------------------------------------------------------
-// K2, K3: the state chains.  One CTA per (sequence, DS-column slice of d_v).  Every warp takes a 16 x 16 tile of the 64 x DS products and DK/4 x 16 of
-// the state, which it keeps in fp32 in its registers (planes of it are what the others read).  A chunk is two phases and two
-// barriers; the tiles of one phase arrive while the other is worked on, those of the first two phases ahead.  Slices of 32
-// columns and d_k = 64 let two CTAs share an SM.  B4 T1024 H16 d_k = d_v = 64: 73 and 85 us with tf32 halves, 45 and 54 so (3 us a
-// chunk, of which the tensor unit works a quarter: the rest is the latency of two dependent products and two barriers).
+// K2, K3: the state chains.  One CTA per (sequence, DS-column slice of d_v).  Every warp takes a 16 x 16 tile of the 64 x DS
+// products and DK/4 x 16 of the state, which it keeps in fp32 in its registers (planes of it are what the others read).  A
+// chunk is two phases and two barriers; the tiles of one phase arrive while the other is worked on, those of the first two
+// phases ahead.  Slices of 32 columns and d_k = 64 let two CTAs share an SM.  B4 T1024 H16 d_k = d_v = 64: 73 and 85 us with
+// tf32 halves, 45 and 54 so (3 us a chunk, of which the tensor unit works a quarter: the rest is the latency of two dependent
+// products and two barriers).
 template <int DK, int DS>
 struct ChainPlanes {
     typedef Planes<C, DK, 1> TA;
