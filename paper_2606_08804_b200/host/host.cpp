@@ -82,14 +82,14 @@ struct NoGil {                                     // other threads may run whil
     ~NoGil() { PyEval_RestoreThread(s); }
 };
 
+// What torch throws keeps its Python type: torch.OutOfMemoryError of an allocation, IndexError, TypeError, or the exception that
+// a saved-tensor hook raised (non-reentrant checkpointing ends its recomputation with one).
 template <class F> PyObject* guarded(F f) {
     try {
         return f();
     } catch (const Raised&) {
-    } catch (const c10::Error& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {
+        torch::translate_exception_to_python(std::current_exception());
     }
     return nullptr;
 }
