@@ -37,8 +37,9 @@
  *   - Supported shapes: chunk = 64, any T >= 1, dk and dv in {64, 128}.  A sequence length that is not a
  *     multiple of the chunk is completed, inside the library, with tokens that leave the recurrence
  *     untouched (beta = 0, alpha = 1); tensors are never read or written beyond their T rows.
- *     bf16 with dk = dv = 128 runs on the tensor cores (tcgen05); fp32, and bf16 with another head
- *     dimension, run on fp32-accurate kernels (qdelta_chunk_path tells which).
+ *     bf16 with dk = dv = 128 runs on the tensor cores (tcgen05), with B H Tp < 2^30 where Tp is T rounded up
+ *     to 128; fp32, and bf16 with another head dimension, run on fp32-accurate kernels (qdelta_chunk_path
+ *     tells which), with B H Tp < 2^35.
  */
 #ifndef QDELTA_H_
 #define QDELTA_H_
@@ -52,7 +53,7 @@ extern "C" {
 typedef enum {
     QD_OK = 0,
     QD_ERR_INVALID_ARG = 1,   /* null required pointer, non-positive size, misaligned pointer, unknown flag */
-    QD_ERR_UNSUPPORTED = 2,   /* (dk, dv, chunk, dtype) outside the supported set */
+    QD_ERR_UNSUPPORTED = 2,   /* (dk, dv, chunk, dtype) outside the supported set, or a size beyond it */
     QD_ERR_WORKSPACE = 3,     /* workspace null or smaller than qdelta_chunk_workspace_bytes */
     QD_ERR_CUDA = 4,          /* a CUDA runtime call (launch, attribute) failed */
     QD_ERR_TIMEOUT = 5,       /* device side: a bounded wait expired (see qdelta_workspace_status) */

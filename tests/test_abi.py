@@ -113,3 +113,24 @@ def test_binding_rejects_cpu_tensors(lib):
     q = torch.zeros(1, 64, 1, 64)
     with pytest.raises(binding.QdeltaError):
         binding.chunk_fwd(q, q, q, torch.zeros(1, 64, 1), workspace=torch.zeros(1 << 20, dtype=torch.uint8))
+
+
+def _codes(lib, s):
+    """(path, backward workspace bytes, what forward, backward and static forward answer with a workspace of no size)"""
+    fake, r = 0x1000, ctypes.byref(s)      # never dereferenced: the shape or the workspace is refused first
+    return (lib.qdelta_chunk_path(r), lib.qdelta_chunk_workspace_bytes(r, 1),
+            lib.qdelta_chunk_fwd(r, fake, fake, fake, fake, None, None, None, fake, None, fake, 0, 0, None),
+            lib.qdelta_chunk_bwd(r, *[fake] * 4, None, None, None, fake, None, *[fake] * 4, None, None, None, fake, 0, 0, None),
+            lib.qdelta_chunk_fwd_static(r, fake, fake, fake, fake, None, None, None, fake, None, None, None))
+
+
+@pytest.mark.parametrize("B,T,H", [(1, 1 << 30, 1), (1 << 10, 1 << 10, 1 << 10), (1 << 14, 1, 1 << 9)])
+def test_shape_that_no_kernel_serves_is_refused(lib, B, T, H):
+    # bf16 128 x 128: row coordinates of the tcgen05 kernels' tensor maps are 32-bit, 2 B H Tp < 2^31, and no other kernels take it
+    from paper_2606_08804_b200.binding import QdShape
+    assert _codes(lib, QdShape(B, T, H, 128, 128, 64, 1)) == (-1, 0, 2, 2, 2)
+    path, nbytes, *codes = _codes(lib, QdShape(B, T - 128, H, 128, 128, 64, 1) if T > 128 else QdShape(B - 1, T, H, 128, 128, 64, 1))
+    assert path == 1 and nbytes > 0 and codes == [3, 3, 6]
+    # the other shapes of that size have theirs
+    for dk, dv, dtype in ((128, 64, 1), (64, 128, 1), (64, 64, 1), (128, 128, 0)):
+        assert _codes(lib, QdShape(B, T, H, dk, dv, 64, dtype))[0] == 0
