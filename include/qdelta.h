@@ -34,7 +34,7 @@
  *     Conditions found on the device (a bounded wait that ran out) are written to the first
  *     32-bit word of the workspace and can be read with qdelta_workspace_status after the
  *     caller has synchronised the stream.
- *   - Supported shapes: chunk = 64, any T >= 1, dk and dv in {64, 128}.  A sequence length that is not a
+ *   - Supported shapes: chunk = 64, T from 1 to 2^31 - 128, dk and dv in {64, 128}.  A sequence length that is not a
  *     multiple of the chunk is completed, inside the library, with tokens that leave the recurrence
  *     untouched (beta = 0, alpha = 1); tensors are never read or written beyond their T rows.
  *     bf16 with dk = dv = 128 runs on the tensor cores (tcgen05), with B H Tp < 2^30 where Tp is T rounded up

@@ -38,6 +38,7 @@ int check_shape(const qd_shape* s) {
     if (s->dtype != QD_F32 && s->dtype != QD_BF16) return QD_ERR_UNSUPPORTED;
     if (s->chunk != kChunk) return QD_ERR_UNSUPPORTED;
     if ((s->dk != 64 && s->dk != 128) || (s->dv != 64 && s->dv != 128)) return QD_ERR_UNSUPPORTED;
+    if (s->T > 0x7fffffff - 127) return QD_ERR_UNSUPPORTED;          // T is rounded up to 64 or 128 in 32 bits
     if ((long long)s->B * s->H * ((s->T + 127) / 128 * 2) > 0x7fffffffLL / 4) return QD_ERR_UNSUPPORTED;
     // bf16 128 x 128 has the tcgen05 kernels alone: split_bf16.cu has none for it
     if (s->dtype == QD_BF16 && s->dk == 128 && s->dv == 128 && !tc_supported(*s)) return QD_ERR_UNSUPPORTED;

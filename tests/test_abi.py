@@ -134,3 +134,16 @@ def test_shape_that_no_kernel_serves_is_refused(lib, B, T, H):
     # the other shapes of that size have theirs
     for dk, dv, dtype in ((128, 64, 1), (64, 128, 1), (64, 64, 1), (128, 128, 0)):
         assert _codes(lib, QdShape(B, T, H, dk, dv, 64, dtype))[0] == 0
+
+
+@pytest.mark.parametrize("dk,dv,dtype", [(64, 64, 1), (128, 64, 1), (128, 128, 1), (64, 64, 0)])
+def test_sequence_length_that_does_not_round_up_in_32_bits_is_refused(lib, dk, dv, dtype):
+    from paper_2606_08804_b200.binding import QdShape
+    top = (1 << 31) - 128                               # the last length whose next multiple of 128 is an int
+    for T in (top + 1, top + 65, (1 << 31) - 1):
+        assert _codes(lib, QdShape(1, T, 1, dk, dv, 64, dtype)) == (-1, 0, 2, 2, 2)
+    path, nbytes, *codes = _codes(lib, QdShape(1, top, 1, dk, dv, 64, dtype))
+    if (dk, dv, dtype) == (128, 128, 1):
+        assert (path, nbytes, codes) == (-1, 0, [2, 2, 2])
+    else:
+        assert path == 0 and top * (dk + dv) * 2 < nbytes < 1 << 45 and codes == [3, 3, 6]
