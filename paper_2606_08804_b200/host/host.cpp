@@ -62,13 +62,19 @@ std::string text(c10::IntArrayRef s) {
     for (size_t i = 0; i < s.size(); ++i) r += (i ? ", " : "") + std::to_string(s[i]);
     return r + (s.size() == 1 ? ",)" : ")");
 }
+// what a kernel that is given this tensor's address would trip over; empty if nothing
+std::string complaint(const at::Tensor& t, at::ScalarType dt, c10::IntArrayRef shape, const char* name, bool any_dtype = false) {
+    if (!t.is_cuda() || !t.is_contiguous()) return name + std::string(" must be a contiguous CUDA tensor");
+    if (!any_dtype && t.scalar_type() != dt)
+        return name + std::string(" must have dtype torch.") + torch::getTHPDtype(dt)->name + ", got torch." + torch::getTHPDtype(t.scalar_type())->name;
+    if (t.sizes() != shape) return name + std::string(" must have shape ") + text(shape) + ", got " + text(t.sizes());
+    return {};
+}
 // device pointer of a contiguous CUDA tensor of the given type and shape; nullptr for an absent one
 void* ptr(const at::Tensor* t, at::ScalarType dt, c10::IntArrayRef shape, const char* name, bool any_dtype = false) {
     if (!t) return nullptr;
-    if (!t->is_cuda() || !t->is_contiguous()) fail("%s must be a contiguous CUDA tensor", name);
-    if (!any_dtype && t->scalar_type() != dt)
-        fail("%s must have dtype torch.%s, got torch.%s", name, torch::getTHPDtype(dt)->name, torch::getTHPDtype(t->scalar_type())->name);
-    if (t->sizes() != shape) fail("%s must have shape %s, got %s", name, text(shape).c_str(), text(t->sizes()).c_str());
+    const std::string c = complaint(*t, dt, shape, name, any_dtype);
+    if (!c.empty()) fail("%s", c.c_str());
     return t->data_ptr();
 }
 at::Tensor empty(c10::IntArrayRef shape, at::ScalarType dt, c10::Device dev) {
@@ -299,15 +305,36 @@ struct ChunkNode : torch::autograd::Function<ChunkNode> {
         }
         return {o, hT};
     }
+    // a QdeltaError from a thread of the autograd engine, which does not hold the interpreter
+    [[noreturn]] static void raise(const std::string& what) {
+        pybind11::gil_scoped_acquire gil;
+        PyErr_SetString(g_error, what.c_str());
+        python_error e;
+        e.persist();
+        throw std::move(e);
+    }
     static variable_list backward(AutogradContext* ctx, variable_list g) {
         const variable_list in = ctx->get_saved_variables();
         const at::Tensor &q = in[0], &v = in[2], &beta = in[3], &alpha = in[4], &lam = in[5], &h0 = in[6], &ws = in[7];
+        if (q.dim() != 4 || v.dim() != 4) raise("q and v must have four dimensions");
         const int64_t B = q.size(0), T = q.size(1), H = q.size(2), dk = q.size(3), dv = v.size(3);
         const at::ScalarType dt = q.scalar_type();
         const c10::Device dev = q.device();
         const qd_shape s{(int)B, (int)T, (int)H, (int)dk, (int)dv, kChunk, dt == at::kFloat ? QD_F32 : QD_BF16};
         const at::Tensor dO = g[0].defined() ? g[0].contiguous() : at::zeros_like(v);
         const at::Tensor dhT = g[1].defined() ? g[1].contiguous().to(at::kFloat) : at::Tensor();
+        // Saved-tensor hooks may hand back other tensors than were saved, tensor hooks other gradients: none of them goes to a
+        // kernel unseen.
+        auto seen = [&](const at::Tensor& t, at::ScalarType type, c10::IntArrayRef shape, const char* name) {
+            if (!t.defined()) return;
+            const std::string c = complaint(t, type, shape, name);
+            if (!c.empty()) raise(c);
+        };
+        if (dt != at::kFloat && dt != at::kBFloat16) raise("q must be fp32 or bf16");
+        seen(q, dt, {B, T, H, dk}, "q"); seen(in[1], dt, {B, T, H, dk}, "k"); seen(v, dt, {B, T, H, dv}, "v");
+        seen(beta, dt, {B, T, H}, "beta"); seen(alpha, dt, {B, T, H}, "alpha"); seen(lam, dt, {B, T, H}, "lam");
+        seen(h0, at::kFloat, {B, H, dk, dv}, "h0"); seen(ws, at::kByte, {ws.numel()}, "the saved workspace");
+        seen(dO, dt, {B, T, H, dv}, "dO"); seen(dhT, at::kFloat, {B, H, dk, dv}, "dhT");
         auto make = [&](c10::IntArrayRef shape, at::ScalarType t) { return at::Tensor(at::detail::empty_cuda(shape, t, dev, std::nullopt)); };
         at::Tensor gq = make({B, T, H, dk}, dt), gk = make({B, T, H, dk}, dt), gv = make({B, T, H, dv}, dt), gh;
         // gradients of the gates come in fp32; one conversion takes all of them to the gates' type
@@ -322,13 +349,7 @@ struct ChunkNode : torch::autograd::Function<ChunkNode> {
         const int rc = qdelta_chunk_bwd(&s, p(q), p(in[1]), p(v), p(beta), p(alpha), p(lam), (const float*)p(h0), p(dO),
                                         (const float*)p(dhT), p(gq), p(gk), p(gv), db, da, dl, (float*)p(gh), ws.data_ptr(),
                                         (size_t)ws.numel(), flags, stream());
-        if (rc != QD_OK) {
-            pybind11::gil_scoped_acquire gil;
-            PyErr_Format(g_error, "qdelta_chunk_bwd failed: %s (%d)", qdelta_status_string(rc), rc);
-            python_error e;
-            e.persist();
-            throw std::move(e);
-        }
+        if (rc != QD_OK) raise("qdelta_chunk_bwd failed: " + std::string(qdelta_status_string(rc)) + " (" + std::to_string(rc) + ")");
         if (dt != at::kFloat) gates = gates.to(dt);
         return {gq, gk, gv, gates.select(0, 0), alpha.defined() ? gates.select(0, 1) : at::Tensor(),
                 lam.defined() ? gates.select(0, n - 1) : at::Tensor(), gh, at::Tensor(), at::Tensor()};

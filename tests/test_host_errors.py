@@ -66,3 +66,33 @@ def test_checkpointed_call_recomputes_its_forward():
     o, _ = checkpoint(qa.qdelta_chunk, *t, use_reentrant=False)
     for x, y in zip(torch.autograd.grad(o.float().sum(), t), want):
         assert torch.equal(x, y)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("change,says", [
+    (lambda x: x.cpu(), "contiguous CUDA tensor"),
+    (lambda x: x.cpu() if x.dtype == torch.uint8 else x, "contiguous CUDA tensor"),        # the workspace
+    (lambda x: x.float() if x.dim() == 4 else x, "dtype"),
+    (lambda x: x[:, :1].contiguous() if x.dim() == 3 else x, "shape"),
+    (lambda x: x.transpose(1, 2).contiguous().transpose(1, 2) if x.dim() == 4 else x, "contiguous CUDA tensor"),
+])
+def test_saved_tensors_that_come_back_changed_are_refused(change, says):
+    from paper_2606_08804_b200 import autograd as qa
+    from paper_2606_08804_b200 import binding as qd
+    t = _inputs(130, 2, requires_grad=True)
+    with torch.autograd.graph.saved_tensors_hooks(lambda x: x, change):
+        o, _ = qa.qdelta_chunk(*t)
+    with pytest.raises(qd.QdeltaError, match=says):
+        o.float().sum().backward()
+    torch.cuda.synchronize()
+
+
+@pytest.mark.gpu
+def test_saved_tensors_kept_on_the_host_give_the_same_gradients():
+    from paper_2606_08804_b200 import autograd as qa
+    t = _inputs(130, 2, requires_grad=True)
+    want = torch.autograd.grad(qa.qdelta_chunk(*t)[0].float().sum(), t)
+    with torch.autograd.graph.save_on_cpu():
+        o, _ = qa.qdelta_chunk(*t)
+    for x, y in zip(torch.autograd.grad(o.float().sum(), t), want):
+        assert torch.equal(x, y)
