@@ -118,9 +118,6 @@ __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.b
 template <int N>
 __device__ __forceinline__ void tma_store_wait_read_n() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
-}
 
 // ---- tensor memory -----------------------------------------------------------------------------
 // One full warp allocates `ncols` (power of two >= 32) TMEM columns; the base address lands in *slot.
@@ -265,28 +262,6 @@ __device__ __forceinline__ void umma_product(uint32_t d_tmem, uint32_t a_saddr, 
     }
 }
 
-// D[tmem] (+)= A[tmem] * B[smem]: the A operand (M = 128 rows on the 128 lanes, bf16 pairs packed two per
-// 32-bit column: column c of lane m holds A[m][2c], A[m][2c+1]) is read from tensor memory.
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, bool accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
-        : "memory");
-}
-template <bool B_MN>
-__device__ __forceinline__ void umma_product_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_saddr, uint32_t b_blk, int N,
-                                                int K, bool accumulate, bool a_neg = false) {
-    const uint32_t idesc = make_idesc(128, N, false, B_MN, a_neg);
-    const uint64_t b0 = B_MN ? desc_mnmajor(b_saddr, b_blk) : desc_kmajor(b_saddr);
-#pragma unroll
-    for (int k = 0; k < K; k += 16) {
-        const uint32_t bo = B_MN ? (uint32_t)k * 128u : (uint32_t)(k >> 6) * b_blk + (uint32_t)(k & 63) * 2u;
-        umma_ts(d_tmem, a_tmem + (uint32_t)(k >> 1), b0 + (uint64_t)(bo >> 4), idesc, accumulate || k > 0);
-    }
-}
-
 // ---- the same, issued by a whole converged warp ---------------------------------------------------------------------
 // One lane issues (`issue` is nonzero in one lane only), but the code around it stays warp-uniform, so that descriptors and
 // their increments live in uniform registers.  From a branch that a single lane takes, every instruction's operands are
@@ -322,6 +297,8 @@ __device__ __forceinline__ void umma_product_w(uint32_t d_tmem, uint32_t a_saddr
               "r"((uint32_t)(accumulate || k > 0)), "r"(issue) : "memory");
     }
 }
+// D[tmem] (+)= A[tmem] * B[smem]: the A operand (M = 128 rows on the 128 lanes, bf16 pairs packed two per
+// 32-bit column: column c of lane m holds A[m][2c], A[m][2c+1]) is read from tensor memory.
 template <bool B_MN>
 __device__ __forceinline__ void umma_product_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_saddr, uint32_t b_blk, int N, int K,
                                                   bool accumulate, uint32_t issue, bool a_neg = false) {
