@@ -10,6 +10,9 @@
 namespace qd {
 
 constexpr int kChunk = 64;        // chunk length C of the chunkwise form
+// SMs of the part that this library is compiled for.  A constant, because the size of a workspace depends on it (split_slice) and
+// is asked for without a device; with another number the rules below choose a slower split, nothing else.
+constexpr int kSMs = 148;
 
 // Byte offsets of the sections of the caller-provided workspace.  Every section starts on a
 // 256-byte boundary.  "io" sections are stored in the call's dtype.

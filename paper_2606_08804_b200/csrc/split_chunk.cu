@@ -625,9 +625,15 @@ cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {
 
 }  // namespace
 
-// d_v columns that one CTA of the state chains owns: narrow slices while they are what it takes to put a CTA on most of
-// the SMs, because a chain's time is its dependent steps; wider ones, which read W<-, Q, K and P fewer times, beyond.
-int split_slice(const qd_shape& s) { return (long long)s.B * s.H * (s.dv / 32) >= 120 ? 32 : 16; }
+// d_v columns that one CTA of the state chains owns: 16 while each CTA then has an SM of its own, because a chain's time is its
+// dependent steps; 32, which read W<-, Q, K and P half as often, beyond.  Both kernels turn there.  Training pass of 512 tokens,
+// narrow against wide, on either side of 148 narrow CTAs (d_k x d_v, sequences):
+//   fp32   64 x 64    37: 150 against 180 us   38: 237 against 219      bf16   64 x 64    37:  87 against  97   38: 123 against 118
+//         128 x 64    37: 230 against 273      38: 375 against 330            128 x 64    37: 121 against 137   38: 195 against 168
+//          64 x 128   18: 123 against 151      19: 214 against 194             64 x 128   18:  74 against  84   19: 114 against 108
+//         128 x 128   18: 177 against 215      19: 334 against 291
+// The same with 2048 tokens, and up to 800 narrow CTAs wide slices stay ahead, but for fp32 with d_k = 64 at 352 (narrow by 3 %).
+int split_slice(const qd_shape& s) { return (long long)s.B * s.H * (s.dv / 16) <= kSMs ? 16 : 32; }
 
 #define QD_BY_DIMS(fn, a, p)                                                                                  \
     ((a).s.dk == 128 ? ((a).s.dv == 128 ? fn<128, 128>(a, p) : fn<128, 64>(a, p))                                  \

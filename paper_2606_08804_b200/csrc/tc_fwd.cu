@@ -783,8 +783,10 @@ bool tc_supported(const qd_shape& s) {
            (long long)s.B * s.H * tc_padded_T(s) * 128 < 0x7fffffffLL * 64;
 }
 
-// Two CTAs per sequence while every CTA still gets an SM of its own: a saving forward chain of 32 sequences 975 -> 681 us.
-int chain_rows(uint64_t BH) { return BH <= 74 ? 64 : 128; }
+// Two CTAs per sequence while every CTA still gets an SM of its own.  Training pass of 74 sequences, two against one: 84 against
+// 88 us (512 tokens), 599 against 647 (4096); of 75: 121 against 100, 734 against 603.  The forward alone at 74: 30.0 against
+// 31.0 and 238 against 242 (two runs differ by 15), at 75: 51 against 41 and 295 against 225.
+int chain_rows(uint64_t BH) { return 2 * BH <= kSMs ? 64 : 128; }
 
 TcLayout tc_layout(const qd_shape& s) {
     TcLayout L{};

@@ -13,10 +13,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("dtype,B,H,T,dk,dv", [
-    ("f32", 4, 15, 65, 64, 64),       # 120 slices of 32 columns: the wide slices, one token in the last chunk
-    ("f32", 7, 17, 63, 64, 64),       # 119: narrow slices, one short chunk
+    ("f32", 4, 15, 65, 64, 64),       # wide slices (32 columns), one token in the last chunk
+    ("f32", 7, 17, 63, 64, 64),       # wide slices, one short chunk
     ("f32", 2, 15, 130, 128, 128),    # wide slices, both head dimensions 128
-    ("f32", 1, 3, 129, 128, 128),
+    ("f32", 1, 3, 129, 128, 128),     # narrow slices (16 columns)
     ("bf16", 4, 15, 100, 64, 64),
     ("bf16", 1, 2, 1, 64, 64),
     ("bf16", 5, 12, 70, 128, 64),
@@ -29,6 +29,17 @@ def test_split_kernels(dtype, B, H, T, dk, dv):
     _fwd_check(cfg, d)
     _bwd_check(cfg, d)
     _bwd_check(cfg, d, reuse=True)
+
+
+@pytest.mark.parametrize("H", [37, 38])      # sequences of d_v = 64: 148 narrow slices, and the first number that takes wide ones
+@pytest.mark.parametrize("dtype,dk,dv", [("f32", 64, 64), ("f32", 128, 128), ("bf16", 64, 64), ("bf16", 128, 64), ("bf16", 64, 128)])
+def test_edge_between_narrow_and_wide_slices(dtype, dk, dv, H):
+    base = gen.CONFIGS["cfg2"] if dtype == "bf16" else replace(gen.CONFIGS["cfg0"], h0=True, backward=True)
+    H = H if dv == 64 else H // 2            # 18 and 19 of d_v = 128
+    cfg = replace(base, B=1, H=H, T=129, dk=dk, dv=dv, regime="alpha_slow", seed=229)
+    d = gen.make_chunk_inputs(cfg)
+    _fwd_check(cfg, d)
+    _bwd_check(cfg, d)
 
 
 @pytest.mark.parametrize("T,dk,dv,logits", [(97, 64, 64, False), (64, 128, 64, True), (65, 64, 128, False)])
