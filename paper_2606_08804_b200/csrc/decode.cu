@@ -21,7 +21,8 @@ namespace {
 // with two barriers.  Fetching each token when its turn came, with four barriers (seven with QD_NORM_QK), took 20 us per
 // token of 256 x 16 states, 35 with normalisation; this takes 12 and 14 (of 5 at the rate of the FMA pipe).
 // Four CTAs per SM are asked for: left to itself the compiler schedules the row products for fewer registers in flight
-// (190 instead of 166 us for eight tokens), and five would spill.
+// (190 instead of 166 us for eight tokens).  At d_k = 128 that is 128 registers, of which an fp32 state leaves 8 - 16 bytes to
+// spill; five CTAs would spill 64 - 204.
 // SB16 (QD_STATE_BF16): the state is STORED in bf16 (half the bytes of the step); it is widened to fp32 when read, all S
 // tokens of the call are applied in fp32, and it is rounded to bf16 once, when written back.
 constexpr int kBlock = 8;

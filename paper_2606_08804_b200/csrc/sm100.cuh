@@ -43,9 +43,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // false on expiry; the caller records the failure and leaves.  One second is several hundred times the longest kernel
 // of this library and far inside any host-side watchdog.  The low 32 bits of the timer wrap every 4.29 s, so differences
 // below that are exact.  How often a waiting thread polls matters: polls are shared-memory traffic that competes with
-// the operand reads of the MMAs.  Measured on the chunk-backward kernel: a tight polling loop 0.347 ms, the timer read
-// every 64 polls 0.303 ms, the timer read after every poll (this loop) 0.289 ms; suspend-time hints on try_wait
-// (0.5 - 50 us) 0.292 ms and slower state chains.
+// the operand reads of the MMAs.  Measured on an earlier form of the chunk backward that took 0.289 ms with this loop, the
+// timer read after every poll: a tight polling loop 0.347 ms, the timer read every 64 polls 0.303 ms; suspend-time hints
+// on try_wait (0.5 - 50 us) 0.292 ms and slower state chains.
 __device__ __forceinline__ uint32_t global_timer_lo() {
     uint32_t t;
     asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));

@@ -11,8 +11,8 @@ namespace {
 // K1: per chunk-head, state-independent part: g, P, W<-, U~ (and M for the backward).  X is never formed, X K^T and T diag(gamma) X are each a product with K and one
 // with Q, their coefficients applied to the result or to T.  One set of planes holds T, T diag(gamma / |k|) and
 // T diag(lambda gamma / |q|) in turn, over what the inverse needed; at d_k = d_v = 64 three CTAs fit an SM.
-// 1024 chunks of 64 x 64: 72 us with tf32 halves and two CTAs, 50 so (d_k 128, d_v 64: 119 and 60), bound by the latency of its
-// chain of small steps.
+// 1024 chunks of 64 x 64: 72 us with tf32 halves and two CTAs, 46 so (d_k 128, d_v 64: 119 and 60; d_k 64, d_v 128: 55; 64 x 64
+// normalised 56), bound by the latency of its chain of small steps.
 template <int DK, int DV>
 struct PrepPlanes {
     typedef Planes<C, DK, 1> TQ;
@@ -408,7 +408,8 @@ struct BwdPlanes {
     static constexpr int kV = 2 * TQ::kBytes, kS = kV + 3 * TV::kBytes, kM = kS + (TS::kBytes > TW::kBytes ? TS::kBytes : TW::kBytes),
                          kBytes = kM + TC::kBytes;
     static_assert(TV::kBytes <= TC::kBytes && TC::kBytes <= 3 * TV::kBytes && TC::kBytes <= kM - kS && kV + 3 * TC::kBytes <= kBytes, "reused room");
-    // where two CTAs fit: 32 x 16 tiles of 8 warps; one CTA: 16 warps hide more (d 128 and 64: 202 against 207 us, normalised 217, 233)
+    // where two CTAs fit: 32 x 16 tiles of 8 warps; one CTA: 16 warps hide more (1024 chunks of d_k 128, d_v 64: 174 us against 191
+    // with 8 warps, normalised 197 against 220; d_k 64, d_v 128: 158 against 166)
     static constexpr int kCtas = kBytes <= 100 * 1024 ? 2 : 1, kThreads = kCtas == 2 ? 256 : 512;
 };
 template <int DK, int DV>

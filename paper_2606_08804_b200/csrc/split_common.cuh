@@ -316,9 +316,13 @@ inline Ptrs make_ptrs(const ChunkArgs& a) {
     return p;
 }
 
-// Small grids, where the gap between two kernels is a tenth of the time (31 -> 28 us for two sequences of 256 tokens), are
-// launched while the kernel before them drains.  Larger ones are not: CTAs that come early take the SMs that are free first
-// instead of one each, which cost 15 us on 128 chunks of 128 x 128 and 40 where two chains fit an SM.
+// Small grids, where the gap between two kernels is a tenth of the time, are launched while the kernel before them drains.
+// Larger ones are not: CTAs that come early take the SMs that are free first instead of one each.  Measured with this line at 0,
+// 16, 32, 64, 96, 128, 148 and 296 on eleven sizes of fp32 64 x 64 and 128 x 128 and bf16 64 x 64 and 128 x 64, training passes:
+// up to 64 every step gains or changes nothing (2 sequences of 256 tokens: 82 -> 74, 127 -> 120, 57 -> 50, 68 -> 60 us; grids of
+// 64, 8 sequences of 512: 109 -> 107, 170 -> 165, 70 -> 70, 88 -> 87), but for fp32 128 x 128 on 8 sequences of 1024 (262 -> 266); at
+// 128 the same sizes lose (16 sequences of 512: 109 -> 112, 176 -> 187, 72 -> 80, 89 -> 92; 64 of 1024, bf16 64 x 64: 250 -> 302)
+// except bf16 128 x 64 on 32 and 64 sequences (121 -> 118, 363 -> 358).
 template <class K, class... Args>
 cudaError_t launch(K kern, int grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
     cudaError_t e = set_max_smem_once(reinterpret_cast<const void*>(kern), smem);

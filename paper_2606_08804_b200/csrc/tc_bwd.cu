@@ -2,14 +2,15 @@
 //
 // The paper prints no backward pass; these kernels evaluate the exact gradient of the chunk
 // equations of Section 3.3.2 (see the forward kernels for the notation):
-//   k_tc_chain_bwd  one CTA per (batch, head), chunks in REVERSE order, dh^T (fp32) in registers:
+//   k_tc_chain_bwd  one CTA per (batch, head), or two that share its d_v rows (chain_rows), chunks in REVERSE order, dh^T
+//                   (fp32) in registers:
 //                     dDelta^T = dO^T P + diag-scaled (dh^T K^T)          (scale gamma_C/gamma_s per token s)
 //                     dh^T <- gamma_C dh^T + dO^T Qg - dDelta^T W<-
 //                   leaves per chunk dDelta^T and the bf16 dh^T at the chunk's exit.
-//   k_tc_chunk_bwd  one CTA per chunk: every remaining product (dP, dT, dA = -M^T dM M^T, dX, ...),
+//   k_tc_chunk_bwd  one CTA per SM, a chunk at a time: every remaining product (dP, dT, dA = -M^T dM M^T, dX, ...),
 //                   d_k/d_v-shaped results transposed (d index on the 128 TMEM lanes), 64 x 64-shaped
-//                   ones in natural orientation on lanes 0..63; row dot-products that run across lanes
-//                   use a warp-shuffle column reduction.
+//                   ones in natural orientation as 64-row instructions, 16 rows on each warp of a warpgroup;
+//                   row dot-products that run across lanes use a warp-shuffle column reduction.
 // All waits are bounded (see tc_fwd.cu).
 #include "internal.h"
 #include "sm100.cuh"
@@ -400,16 +401,17 @@ constexpr int kNbSumN = kBwdCompute + C;
 // 8 TMEM columns of this thread's lane (no wait)
 __device__ __forceinline__ void ld8(uint32_t taddr, float* v) { tmem_ld8(taddr, v); }
 
-// Two warpgroups: warpgroup w (threads 128w..128w+127) owns TMEM columns [32w, 32w+32) of every
-// 64-column accumulator; inside a warpgroup thread l owns TMEM lane l.
+// Four epilogue warpgroups: warpgroup w (threads 128w..128w+127) owns TMEM columns [16w, 16w+16) of every 64-column
+// accumulator; inside a warpgroup, warp wq owns TMEM lanes [32 wq, 32 wq + 32), i.e. rows 32 wq .. of a 128-row product and
+// rows 16 wq .. of a 64-row one.
 // HAS_LAM = false: lambda is absent and d lambda is not asked for (the gated delta rule, Eq. 3): X = K, nothing is built,
 // no column sum for d lambda.  HAS_ALPHA = false: alpha is absent and d alpha is not asked for (no forget gate; with
 // HAS_LAM = false too this is DeltaNet, Eq. 2): every decay factor is 1 and none of the sums that only feed d alpha is
 // taken.  The <true, true> instances serve every other case (an absent input then reads as lambda = 0, alpha = 1).
 // NORM (QD_NORM_QK): the Q and K tiles arrive un-normalised and are normalised in place with the factors the forward
 // left in the workspace; dq and dk are taken through the normalisation, dx = r (dx^ - x^ <x^, dx^>), which needs the
-// row sums <x^, dx^> before anything can be stored: the last epilogue then runs twice, once for the sums and once
-// for the stores.
+// row sums <x^, dx^>: dk^ and dq^ are staged in bf16 like dk and dq without NORM, and a second pass over the staged tiles, a
+// row to 16 lanes, takes the sums and rewrites them.
 template <bool HAS_LAM, bool HAS_ALPHA, bool NORM, bool GROUPED>
 __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_constant__ CUtensorMap mapQ,
                                                               const __grid_constant__ CUtensorMap mapK,
@@ -469,10 +471,10 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     // Work item `ch` is chunk n_ of sequence bh_.  GROUPED = false: sequence-major numbering.  GROUPED = true: items are
     // numbered in groups of p.group sequences, chunk-major inside a group, so that at any time the CTAs of the grid work
     // on a few chunk indices of p.group sequences instead of on ~148 consecutive chunks of one long sequence.  Measured,
-    // sequence-major against groups of 32: 0.330 / 0.316 ms on 32 sequences of 128 chunks, 0.347 / 0.320 on 16 of 256,
-    // 1.47 / 1.18 on 32 of 512, no gain on 128 sequences of 32 chunks; all sequences at a time (chunk-major) was the
-    // slowest there.  Compile-time, because the kernel's code generation is at a knife's edge: the grouped arithmetic
-    // compiled into the sequence-major path cost it 3.5 %, as a non-inlined function 14 %.
+    // sequence-major against groups of 32, this kernel: 114 / 109 us on 32 sequences of 64 chunks, 217 / 208 on 32 of 128,
+    // 223 / 206 on 16 of 256, 837 / 772 on 32 of 512.  An earlier form of the kernel gained nothing on 128 sequences of 32 chunks
+    // and lost most with all sequences at a time (chunk-major).  Compile-time, because the grouped arithmetic compiled into
+    // the sequence-major path cost that form 3.5 %, as a non-inlined function 14 %.
     auto item = [&](int ch, int& n_, int& bh_) {
         if (GROUPED) {
             const int per = p.group * p.N, grp = ch / per, r = ch - grp * per;
@@ -518,8 +520,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             tma_load_3d(sm + oK + blk * 8192, &mapK, hh_ * D + blk * 64, n_ * C, b_, &bar_qk);
         }
     };
-    // of the tiles of a chunk, those that are waited for most into L2 only, a chunk time ahead (985 -> 879 us on 512 chunks
-    // of 32 sequences together with the order of the waits; V, dO, M^T and P as well: no gain)
+    // of the tiles of a chunk, those that are waited for most into L2 only, a chunk time ahead: 761 us with it and 839 without on
+    // 32 sequences of 512 chunks (training pass 2420 and 2529), 219 and 216 on 128 of 32; V, dO, M^T and P as well: no gain
     auto prefetch_late = [&](int ch) {
         int n_, bh_; item(ch, n_, bh_);
         const int b_ = bh_ / p.H, hh_ = bh_ % p.H;

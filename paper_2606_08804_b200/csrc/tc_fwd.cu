@@ -6,9 +6,9 @@
 //                   per chunk, in bf16:  Qg = diag(gamma) Q  [token][dk],
 //                   P = Gamma o (Q K^T) causal incl. diagonal [token][64],
 //                   Wt = (T diag(gamma) X)^T  [dk][64 tokens],   Ut = (T V)^T  [dv][64 tokens].
-//   k_tc_chain_fwd  one CTA per (batch, head): walks the chunks in order with the fp32 state in
-//                   registers (thread j owns row j of h^T, i.e. column j of h), everything
-//                   transposed so that d_v = 128 is the MMA M dimension:
+//   k_tc_chain_fwd  one CTA per (batch, head), or two that share its d_v rows (chain_rows): walks the chunks
+//                   in order with the fp32 state in registers (a thread owns 32 columns of one row of h^T),
+//                   everything transposed so that d_v is the MMA M dimension:
 //                     Delta^T = Ut - h^T Wt            O^T = h^T Qg^T + Delta^T P^T
 //                     h^T <- gamma_C h^T + (Delta diag(gamma_C/gamma))^T K
 // All waits are bounded; on expiry the CTA records QD_ERR_TIMEOUT in the workspace status word,
