@@ -15,7 +15,6 @@
 #include "internal.h"
 #include "sm100.cuh"
 
-
 namespace qd {
 namespace {
 using namespace sm100;
@@ -23,18 +22,6 @@ typedef __nv_bfloat16 bf16;
 
 constexpr int C = kChunk;      // 64
 constexpr int D = 128;         // d_k = d_v
-
-__device__ __forceinline__ void load8(const unsigned char* p, float* f) {
-    const uint4 u = *reinterpret_cast<const uint4*>(p);
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { const float2 t = __bfloat1622float2(h[i]); f[2 * i] = t.x; f[2 * i + 1] = t.y; }
-}
-__device__ __forceinline__ uint4 pack8(const float* f) {
-    uint4 u;
-    u.x = pack_bf16(f[0], f[1]); u.y = pack_bf16(f[2], f[3]); u.z = pack_bf16(f[4], f[5]); u.w = pack_bf16(f[6], f[7]);
-    return u;
-}
 
 // One halving step of a column sum across the lanes of a warp: lanes whose `off` bit is set keep the upper half
 // of the N values, the others the lower half; each adds what its partner sends.
@@ -72,11 +59,6 @@ constexpr int kMmaWarp = kChainCompute / 32;
 
 // named barriers: compute threads arrive, the MMA warp waits (they run in lock-step)
 constexpr int kBarH = 1, kBarD = 2;
-__device__ __forceinline__ void nb_arrive(int id, int count) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory"); }
-__device__ __forceinline__ void nb_sync(int id, int count) {
-    __syncwarp();                                   // the lanes of a warp reach the barrier together
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
 
 // Reverse state chain.  Per chunk the dependency is
 //   dh ready -> A2 = dh^T K^T -> dDelta^T -> H-accumulator -= dDelta^T W<- -> dh update;
