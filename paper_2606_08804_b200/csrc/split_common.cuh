@@ -44,8 +44,10 @@ struct Ptrs {
 // fetch the operands.  Lane (g = lane / 4, t = lane % 4) holds, of every
 // 16 x 8 piece, rows g and g + 8, columns 2t and 2t + 1.
 // The tensor instruction truncates as it accumulates, which over a long contraction biases the sum by 1e-6 of itself; so it
-// only sums 16 terms at a time, from zero, and those sums are added with rounded fp32 additions.
-// Measured against fp64 on 1024 tokens: slowly forgetting gates, rms error of the outputs 1.2e-6 without, 2.9e-7 with, 2.6e-7 for plain fp32 FMAs.
+// only sums 16 terms at a time, from zero, the small products (lo hi, hi lo) of all of them before the large ones, and those sums
+// are added with rounded fp32 additions.  Measured against fp64 on 1024 tokens, d = 64, slowly forgetting gates, rms error of the
+// outputs: 1.2e-6 with one running sum, 3.0e-7 with the three products of 8 terms after those of the 8 before, 2.5e-7 so, 2.3e-7
+// with plain fp32 FMAs.
 __device__ __forceinline__ void add2(float& x, float& y, float a, float b) {
     asm("{\n\t.reg .b64 u, v;\n\tmov.b64 u, {%0, %1};\n\tmov.b64 v, {%2, %3};\n\tadd.rn.f32x2 u, u, v;\n\tmov.b64 {%0, %1}, u;\n\t}"
         : "+f"(x), "+f"(y) : "f"(a), "f"(b));
@@ -75,24 +77,26 @@ __device__ __forceinline__ void wmm(float (&acc)[MT][NTL][4], int m0, int n0, in
                 for (int j = 0; j < JN; ++j)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) part[i][j][e] = 0.f;
+            uint32_t bh[KS][JN][2], bl[KS][JN][2];
 #pragma unroll
-            for (int s = 0; s < KS; ++s) {
-                uint32_t bh[JN][2], bl[JN][2];
+            for (int s = 0; s < KS; ++s)
 #pragma unroll
                 for (int j = 0; j < JN; ++j)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const float x = b(k0 + 8 * s + t + 4 * e, n0 + 8 * (jb + j) + g);
-                        tf32_split(x, bh[j][e], bl[j][e]);
+                        tf32_split(x, bh[s][j][e], bl[s][j][e]);
                     }
+            auto add = [&](int s, const uint32_t (&x)[KS][MT][4], const uint32_t (&y)[KS][JN][2]) {
 #pragma unroll
-                for (int term = 0; term < 3; ++term)                         // lo hi, hi lo, hi hi
+                for (int i = 0; i < MT; ++i)
 #pragma unroll
-                    for (int i = 0; i < MT; ++i)
+                    for (int j = 0; j < JN; ++j) mma_tf32(part[i][j], x[s][i], y[s][j]);
+            };
 #pragma unroll
-                        for (int j = 0; j < JN; ++j)
-                            mma_tf32(part[i][j], term == 0 ? al[s][i] : ah[s][i], term == 1 ? bl[j] : bh[j]);
-            }
+            for (int s = 0; s < KS; ++s) { add(s, al, bh); add(s, ah, bl); }
+#pragma unroll
+            for (int s = 0; s < KS; ++s) add(s, ah, bh);
 #pragma unroll
             for (int i = 0; i < MT; ++i)
 #pragma unroll
