@@ -44,6 +44,7 @@ int check_shape(const qd_shape* s);
 // Workspace of the tensor-core path (bf16, d_k = d_v = 128).  Sections start on 1024-byte boundaries.
 struct TcLayout {
     size_t status;   // u32 status word
+    size_t next;     // u32 counter of the chunk backward's work items, zeroed by the reverse chain
     size_t g;        // fp32 [BH*T]
     size_t Qg;       // bf16 [BH*T][dk]        diag(gamma) Q
     size_t P;        // bf16 [BH*T][C]         Gamma o (Q K^T), causal incl. diagonal

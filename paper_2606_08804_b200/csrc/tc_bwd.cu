@@ -23,6 +23,18 @@ typedef __nv_bfloat16 bf16;
 constexpr int C = kChunk;      // 64
 constexpr int D = 128;         // d_k = d_v
 
+// What follows an unsuccessful first poll: mbar_wait, given up as soon as another wait of the CTA has expired (every later wait
+// then returns at once: the kernel drains).
+__device__ __forceinline__ bool wait_on(uint64_t* bar, uint32_t parity, volatile int& s_abort, unsigned* status) {
+    const uint32_t t0 = global_timer_lo();
+#pragma unroll 1
+    while (!s_abort) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if (global_timer_lo() - t0 > kWaitLimitNs) { s_abort = 1; *status = QD_ERR_TIMEOUT; }
+    }
+    return false;
+}
+
 // One halving step of a column sum across the lanes of a warp: lanes whose `off` bit is set keep the upper half
 // of the N values, the others the lower half; each adds what its partner sends.
 template <int N>
@@ -37,37 +49,50 @@ __device__ __forceinline__ void fold(float* v, int lane, int off) {
 }
 
 // =================================================================================================
+struct BwdMaps {               // boxes of 64 rows for token tiles, 128 for tiles by d_v or d_k, `rows` for the chain's two stores
+    CUtensorMap Q, K, V, dO, Mt, P, Dt, dDt, Hs, dHs, Wt, Qg, dHs_store, dDt_store, dQ, dK, dV;
+};
 struct ChainBwdParams {
     int Tp, H, N;              // Tp = 64 N rows per sequence in the workspace
-    int rows;                  // d_v rows of the state per CTA: 128, or 64 (two CTAs per sequence)
     int dhT_early;             // the kernel before this one in the stream is the library's own: dhT is older than it
     const float* rk;           // non-null (QD_NORM_QK): 1/|k_t| per workspace row, folded into the per-token scale
     const float* g;
     const float* dhT;
     float* dh0;
     unsigned* status;
+    unsigned* next;            // zeroed here for k_tc_chunk_bwd
 };
 
-// Tiles of a chunk in shared memory: K 16K | P 8K, three deep; dO 16K | Qg 16K, two deep; Wt 16K, two deep; staged for their
-// stores: dh^T 32K, dDelta^T 16K.
-constexpr int kDeepK = 3, kBytesK = 24576, kBytesQ = 32768, kBytesW = 16384;
-constexpr int kOffQ = kDeepK * kBytesK, kOffW = kOffQ + 2 * kBytesQ, kOffH = kOffW + 2 * kBytesW, kOffD = kOffH + 32768;
-constexpr int kChainSmem = kOffD + 16384 + 1024;
+// Tiles of a chain's chunk in shared memory: K 16K | P 8K, three deep; Qg 16K | dO 16K and Wt 16K, two deep; staged for their
+// stores, one deep: dh^T 32K | dDelta^T 16K; with 64 rows dO, dh^T and dDelta^T have half the size, and are staged two deep; then
+// the per-token scales.
+constexpr int kDeepK = 3, kBytesK = 24576;
+constexpr int kOffQ = kDeepK * kBytesK, kOffG = kOffQ + 2 * (32768 + 16384) + 32768 + 16384;
+constexpr int kChainSmem = kOffG + (kDeepK + 1) * 68 * 4 + 1024;
 constexpr int kChainCompute = 512;                 // 16 epilogue warps: 4 warpgroups split the accumulator columns
-constexpr int kChainThreads = kChainCompute + 96;  // + 1 MMA-issue warp, 1 warp each for TMA loads and saves
+constexpr int kChainThreads = kChainCompute + 96;  // + 1 MMA-issue warp, 1 warp each for saves and TMA loads
 constexpr int kMmaWarp = kChainCompute / 32;
 
-// named barriers: compute threads arrive, the MMA warp waits (they run in lock-step)
+// named barriers of the chain: compute threads arrive, the MMA warp waits (they run in lock-step)
 constexpr int kBarH = 1, kBarD = 2;
+
+// A barrier per buffer where one side may run ahead.  k, q, w: tiles loaded; fk, fq, fw: read by their last product; ht, dt:
+// staged (one arrival per compute warp); hf, df: read by their store (two deep: hf alone, for both); a, b: products complete.
+struct ChainBars { uint64_t k[kDeepK], fk[kDeepK], q[2], fq[2], w[2], fw[2], hf[2], df, a, b, ht[2], dt[2]; };
 
 // Reverse state chain.  Per chunk the dependency is
 //   dh ready -> A2 = dh^T K^T -> dDelta^T -> H-accumulator -= dDelta^T W<- -> dh update;
 // A1 = dO^T P and the dO^T Qg part of the H-accumulator do not depend on dh and are issued a chunk ahead (double-buffered
 // H-accumulator).  As in the forward chain, the dependent operands (dh^T, -dDelta^T) live in tensor memory and the issuing
-// warp stays converged; what bounds a chunk is the SM's TMA unit, 72 KB in at 45 and 48 KB out at 32 bytes per cycle, one
-// after the other: 3150 cycles.  With few sequences two CTAs share the d_v rows of one (`rows` = 64).
+// warp stays converged.  With few sequences two CTAs share the d_v rows of one (ROWS = 64).
+// With 128 rows what bounds a chunk is the SM's TMA unit, 72 KB in at 45 and 48 KB out at 32 bytes per cycle, one after the other:
+// 3150 cycles.  With 64 it is the sequence of hand-offs, so nothing that can be elsewhere is on it: a wait that has long been
+// satisfied costs 100 - 200 cycles, so the next chunk's scales are waited for under the last product, one barrier stands for both
+// staged tiles, the tiles are staged two deep, and a wait polls before it looks at the abort flag (2540 -> 2250 cycles a chunk;
+// 92 -> 85 us on 4 sequences of 64 chunks, backward).
 // Compute warpgroup w owns tokens [16w, 16w+16) of the 64-column accumulators and d_k columns
 // [32w, 32w+32) of dh^T; thread l of a warpgroup owns TMEM lane l = d_v index.
+template <int ROWS>
 __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_constant__ CUtensorMap mapWt,
                                                                 const __grid_constant__ CUtensorMap mapdO,
                                                                 const __grid_constant__ CUtensorMap mapQg,
@@ -78,26 +103,24 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
                                                                 ChainBwdParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* sdH = smem + kOffH;              // dh^T [128 dv][128 dk], 2 blocks of [128 lines][64]
-    unsigned char* sdD = smem + kOffD;              // dDelta^T [128 dv][64 tokens]
-    // A barrier per buffer where one side may run ahead.  bar_k, bar_q, bar_w: tiles loaded; bar_fk, bar_fq, bar_fw: read by
-    // their last product; bar_ht, bar_dt: staged (one arrival per compute warp); bar_hf, bar_df: read by their store.
-    __shared__ uint64_t bar_k[kDeepK], bar_fk[kDeepK], bar_q[2], bar_fq[2], bar_w[2], bar_fw[2], bar_ht, bar_hf, bar_dt, bar_df, bar_a, bar_b;
+    constexpr int rows = ROWS, bytesQ = 16384 + rows * 128, offW = kOffQ + 2 * bytesQ;
+    constexpr int two = rows == D ? 0 : 1, bytesS = rows * 384;       // staged tiles: two deep or not
+    unsigned char* stg = smem + offW + 2 * 16384;      // dh^T [rows dv][128 dk], 2 blocks of [rows lines][64]; dDelta^T [rows dv][64 tokens]
+    __shared__ ChainBars bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
-    // gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the load warp before it arrives on bar_k.  One deeper than
+    // gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the load warp before it arrives on bar.k.  One deeper than
     // K and P: those are dead when A2 is complete, but the epilogue reads these after that
-    __shared__ __align__(16) float sG[kDeepK + 1][68];
+    float (*sG)[68] = reinterpret_cast<float (*)[68]>(smem + kOffG);
 
     const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, l = tid & 127, wq = warp & 3;
-    const int rows = p.rows, nwq = rows / 32, nb = 4 * rows + 32;    // d_v rows of this CTA; warps of a warpgroup that have some; barrier participants
-    const int parts = D / rows, bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
+    constexpr int nwq = rows / 32, nb = 4 * rows + 32;               // warps of a warpgroup that have rows; barrier participants
+    constexpr int parts = D / rows;
+    const int bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
 
     if (tid == 0) {
-        for (int i = 0; i < kDeepK; ++i) { mbar_init(&bar_k[i], 1); mbar_init(&bar_fk[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&bar_q[i], 1); mbar_init(&bar_fq[i], 1); mbar_init(&bar_w[i], 1); mbar_init(&bar_fw[i], 1); }
-        mbar_init(&bar_ht, 4 * nwq); mbar_init(&bar_dt, 4 * nwq); mbar_init(&bar_hf, 1); mbar_init(&bar_df, 1);
-        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1);
+        uint64_t* all = bar.k;
+        for (int i = 0; i < (int)(sizeof(ChainBars) / 8); ++i) mbar_init(all + i, all + i >= bar.ht ? 4 * nwq : 1);
         mbar_init_fence();
         s_abort = 0;
     }
@@ -111,13 +134,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
     const uint32_t lane_base = (uint32_t)wq * 32;
 
     // bounded wait; once any wait has expired every later wait returns at once (the kernel drains)
-    auto wait = [&](uint64_t* bar, uint32_t parity) {
-        if (s_abort) return false;
-        if (mbar_wait(bar, parity)) return true;
-        s_abort = 1;
-        *p.status = QD_ERR_TIMEOUT;
-        return false;
-    };
+    auto wait = [&](uint64_t* br, uint32_t parity) { return mbar_try_wait(br, parity) || wait_on(br, parity, s_abort, p.status); };
     const float* gseq = p.g + (size_t)bh * p.Tp;
 
     if (warp < kMmaWarp && wq >= nwq) {
@@ -129,18 +146,13 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         // than that kernel and may be read while it drains; otherwise the predecessor may be the very kernel that wrote
         // dhT, whose writes are only guaranteed visible after the wait.
         if (!p.dhT_early) grid_dep_wait();
-        if (p.dhT) {
-            const float* src = p.dhT + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
+        const size_t at = (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) dh[i] = src[(size_t)i * D];
-        } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) dh[i] = 0.f;
-        }
+        for (int i = 0; i < 32; ++i) dh[i] = p.dhT ? p.dhT[at + (size_t)i * D] : 0.f;
         if (p.dhT_early) grid_dep_wait();  // the loads of dhT are in flight; everything below depends on earlier kernels
         grid_dep_launch();
-        auto arrive = [&](uint64_t* bar) { __syncwarp(); if ((tid & 31) == 0) mbar_arrive(bar); };
-        auto staged = [&](uint64_t* bar) { fence_proxy_async(); arrive(bar); };      // my part of a tile is in shared memory, for its store
+        auto arrive = [&](uint64_t* b) { __syncwarp(); if ((tid & 31) == 0) mbar_arrive(b); };
+        auto staged = [&](uint64_t* b) { fence_proxy_async(); arrive(b); };      // my part of a tile is in shared memory, for its store
         // dh as operand: my 32 columns are 16 packed columns of tensor memory; then as a tile for its store
         auto put_h = [&]() {
             uint32_t r[8];
@@ -154,21 +166,21 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
             tc_fence_before();
             nb_arrive(kBarH, nb);
         };
-        auto save_h = [&]() {             // 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
-#pragma unroll
-            for (int ch = 0; ch < 4; ++ch) sts128(sdH + (wg >> 1) * 16384 + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(dh + ch * 8));
-            staged(&bar_ht);
-        };
-        // A chunk's K and P may be reloaded as soon as A2 is complete, which the announcement of its dh^T sets off: so the
-        // scales of a chunk are waited for before that, not after (where the barrier could have come round)
-        wait(&bar_k[0], 0);
-        put_h();
-        save_h();
         int pending = 0;                  // barriers of the MMA warp that a warp which gives up has not been to
         int s = 0;
+        uint32_t sp = 0;
+        wait(&bar.k[0], 0);
         for (int it = 0; it < p.N; ++it) {
+            put_h();
+            const int sb = it & two;
+            unsigned char* sdH = stg + sb * bytesS;
+            if (it > two) wait(&bar.hf[sb], ((it >> two) - 1) & 1);       // the tile (two deep: both) has been read by the store before
+            // 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) sts128(sdH + (wg >> 1) * (rows * 128) + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(dh + ch * 8));
+            staged(&bar.ht[sb]);
             const float gamC = sG[it & 3][64];
-            if (!__all_sync(0xffffffffu, wait(&bar_a, it & 1))) { pending = 2 * (p.N - it); break; }
+            if (!__all_sync(0xffffffffu, wait(&bar.a, it & 1))) { pending = 2 * (p.N - it) - 1; break; }
             tc_fence_after();
             // dDelta^T = A1 + gamma_C/gamma_s A2, my 16 tokens; negated as operand
             {
@@ -189,12 +201,17 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
                 tmem_st_wait();
                 tc_fence_before();
                 nb_arrive(kBarD, nb);
-                if (it > 0) wait(&bar_df, (it - 1) & 1);
+                unsigned char* sdD = sdH + rows * 256;
+                if (!two && it > 0) wait(&bar.df, (it - 1) & 1);
                 sts128(sdD + sw128_chunk(l, wg * 2), make_uint4(r[0], r[1], r[2], r[3]));
                 sts128(sdD + sw128_chunk(l, wg * 2 + 1), make_uint4(r[4], r[5], r[6], r[7]));
-                staged(&bar_dt);
+                staged(&bar.dt[sb]);
             }
-            if (!__all_sync(0xffffffffu, wait(&bar_b, it & 1))) { pending = 2 * (p.N - it) - 1; break; }
+            // A chunk's K and P may be reloaded as soon as A2 is complete, which the announcement of its dh^T sets off: so
+            // the scales of the next chunk are waited for before that, not after (where the barrier could have come round)
+            if (++s == kDeepK) { s = 0; sp ^= 1; }
+            if (it + 1 < p.N) wait(&bar.k[s], sp);
+            if (!__all_sync(0xffffffffu, wait(&bar.b, it & 1))) { pending = 2 * (p.N - it) - 2; break; }
             tc_fence_after();
             {
                 float v[32];
@@ -203,17 +220,12 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
 #pragma unroll
                 for (int i = 0; i < 32; ++i) dh[i] = fmaf(gamC, dh[i], v[i]);
             }
-            if (++s == kDeepK) s = 0;
-            if (it + 1 < p.N) wait(&bar_k[s], ((it + 1) / kDeepK) & 1);
-            put_h();
-            if (it + 1 < p.N) { wait(&bar_hf, it & 1); save_h(); }
         }
-        // a wait has expired: keep step with the MMA warp, which comes to every one of them (odd counts: H is next)
-        for (; pending > 0; --pending) nb_sync(pending & 1 ? kBarH : kBarD, nb);
+        // a wait has expired: keep step with the MMA warp, which comes to every one of them (odd counts: D is next)
+        for (; pending > 0; --pending) nb_sync(pending & 1 ? kBarD : kBarH, nb);
         if (p.dh0 && !s_abort) {
-            float* dst = p.dh0 + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) dst[(size_t)i * D] = dh[i];
+            for (int i = 0; i < 32; ++i) p.dh0[at + (size_t)i * D] = dh[i];
         }
     } else if (warp == kMmaWarp) {
         // ---------------------------------- MMA-issue warp, converged ----------------------------------
@@ -222,61 +234,71 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         grid_dep_launch();
         const uint32_t sb = smem_u32(smem);
         // A1 = dO^T P (A, B MN-major: lines = token r), H-accumulator = dO^T Qg (B MN-major, two blocks of d_k)
-        auto ahead = [&](int it, int s) {
-            const uint32_t sq = sb + kOffQ + (it & 1) * kBytesQ;
-            wait(&bar_k[s], (it / kDeepK) & 1);
-            wait(&bar_q[it & 1], (it >> 1) & 1);
-            tc_fence_after();
-            umma_product_w<true, true>(tA1, sq, 8192, sb + s * kBytesK + 16384, 8192, C, C, false, issue);
-            umma_product_w<true, true>(tH0 + 128 * (it & 1), sq, 8192, sq + 16384, 8192, D, C, false, issue);
-            umma_commit_w(&bar_fq[it & 1], issue);
-        };
-        ahead(0, 0);
+        // stage of the ring of K and P, and the parity of its present round
         int s = 0;
+        uint32_t sp = 0;
+        auto ahead = [&](int it) {
+            const int t = it & 1;
+            const uint32_t sq = sb + kOffQ + t * bytesQ;
+            wait(&bar.k[s], sp);
+            wait(&bar.q[t], (it >> 1) & 1);
+            tc_fence_after();
+            umma_product_w<true, true>(tA1, sq + 16384, 8192, sb + s * kBytesK + 16384, 8192, C, C, false, issue);
+            umma_product_w<true, true>(tH0 + 128 * (it & 1), sq + 16384, 8192, sq, 8192, D, C, false, issue);
+            umma_commit_w(&bar.fq[t], issue);
+        };
+        ahead(0);
         for (int it = 0; it < p.N; ++it) {
             nb_sync(kBarH, nb);                         // dh^T operand (exit state of this chunk) is in place
             tc_fence_after();
             // A2 = dh^T K^T (B K-major)
             umma_product_ts_w<false>(tA2, aH, sb + s * kBytesK, 8192, C, D, false, issue);
-            umma_commit_w(&bar_a, issue);
-            umma_commit_w(&bar_fk[s], issue);
-            wait(&bar_w[it & 1], (it >> 1) & 1);
+            umma_commit_w(&bar.a, issue);
+            umma_commit_w(&bar.fk[s], issue);
+            const int t = it & 1;
+            wait(&bar.w[t], (it >> 1) & 1);
             nb_sync(kBarD, nb);                         // -dDelta^T operand is in place, A1 has been read
             tc_fence_after();
             // H-accumulator -= dDelta^T W<-   (B K-major: lines = d_k index, contraction over tokens)
-            umma_product_ts_w<false>(tH0 + 128 * (it & 1), aD, sb + kOffW + (it & 1) * kBytesW, 16384, D, C, true, issue);
-            umma_commit_w(&bar_b, issue);
-            umma_commit_w(&bar_fw[it & 1], issue);
-            if (++s == kDeepK) s = 0;
-            if (it + 1 < p.N) ahead(it + 1, s);           // in the shadow of the dh update
+            umma_product_ts_w<false>(tH0 + 128 * (it & 1), aD, sb + offW + t * 16384, 16384, D, C, true, issue);
+            umma_commit_w(&bar.b, issue);
+            umma_commit_w(&bar.fw[t], issue);
+            if (++s == kDeepK) { s = 0; sp ^= 1; }
+            if (it + 1 < p.N) ahead(it + 1);            // in the shadow of the dh update
         }
-        nb_sync(kBarH, nb);                               // final arrival of the compute warps
     } else if (warp == kMmaWarp + 1) {
         // ---------------------------------- saving warp ----------------------------------
         if ((tid & 31) == 0) {
             grid_dep_wait();
+            if (blockIdx.x == 0) *p.next = 0;
             for (int it = 0; it < p.N; ++it) {
-                const int y = (int)(((size_t)bh * p.N + (p.N - 1 - it)) * D) + v0;
-                wait(&bar_ht, it & 1);                    // gradient w.r.t. the exit state (rows = d_v, columns = d_k) is staged
+                const int y = (int)(((size_t)bh * p.N + (p.N - 1 - it)) * D) + v0, sb = it & two;
+                unsigned char *sdH = stg + sb * bytesS, *sdD = sdH + rows * 256;
+                wait(&bar.ht[sb], (it >> two) & 1);       // gradient w.r.t. the exit state (rows = d_v, columns = d_k) is staged
                 tma_store_2d(&mapdHs, sdH, 0, y);
-                tma_store_2d(&mapdHs, sdH + 16384, 64, y);
+                tma_store_2d(&mapdHs, sdH + rows * 128, 64, y);
                 tma_store_commit();
-                if (it > 0) { tma_store_wait_read_n<1>(); mbar_arrive(&bar_df); }     // dDelta^T of the chunk before has been read
-                wait(&bar_dt, it & 1);                    // dDelta^T is staged
+                if (!two && it > 0) { tma_store_wait_read_n<1>(); mbar_arrive(&bar.df); }        // dDelta^T of the chunk before has been read
+                wait(&bar.dt[sb], (it >> two) & 1);       // dDelta^T is staged
                 tma_store_2d(&mapdDt, sdD, 0, y);
                 tma_store_commit();
-                tma_store_wait_read_n<1>();
-                mbar_arrive(&bar_hf);                     // the dh^T tile has been read
+                if (!two) {
+                    tma_store_wait_read_n<1>();
+                    mbar_arrive(&bar.hf[0]);              // the dh^T tile has been read
+                } else if (it > 0) {
+                    tma_store_wait_read_n<2>();
+                    mbar_arrive(&bar.hf[sb ^ 1]);         // both tiles of the chunk before have been read
+                }
             }
             tma_store_wait_all();
         }
     } else {
         // ---------------------------------- TMA load warp ----------------------------------
         const bool lead = (tid & 31) == 0;
+        const int ln = tid & 31;
         grid_dep_wait();
         grid_dep_launch();
         // iteration `it` processes chunk n = N-1-it
-        const int ln = tid & 31;
         const float* rkseq = p.rk ? p.rk + (size_t)bh * p.Tp : nullptr;
         float g0, g1, gc, r0 = 1.f, r1 = 1.f;             // log-decays (and 1/|k|) of the next chunk to be loaded
         auto fetch_g = [&](int it) {
@@ -293,53 +315,54 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
             if (lead) {
                 const int n = p.N - 1 - it;
                 unsigned char* st = smem + s * kBytesK;
-                mbar_expect_tx(&bar_k[s], kBytesK);
-                tma_load_3d(st, &mapK, hh * D, n * C, b, &bar_k[s]);
-                tma_load_3d(st + 8192, &mapK, hh * D + 64, n * C, b, &bar_k[s]);
-                tma_load_2d(st + 16384, &mapP, 0, (int)((size_t)bh * p.Tp + (size_t)n * C), &bar_k[s]);
+                mbar_expect_tx(&bar.k[s], kBytesK);
+                tma_load_3d(st, &mapK, hh * D, n * C, b, &bar.k[s]);
+                tma_load_3d(st + 8192, &mapK, hh * D + 64, n * C, b, &bar.k[s]);
+                tma_load_2d(st + 16384, &mapP, 0, (int)((size_t)bh * p.Tp + (size_t)n * C), &bar.k[s]);
             }
             if (it + 1 < p.N) fetch_g(it + 1);
         };
         auto load_q = [&](int it) {                      // by the leading lane
             const int n = p.N - 1 - it;
-            unsigned char* st = smem + kOffQ + (it & 1) * kBytesQ;
-            uint64_t* bar = &bar_q[it & 1];
+            unsigned char* st = smem + kOffQ + (it & 1) * bytesQ;
+            uint64_t* br = &bar.q[it & 1];
             const int yt = (int)((size_t)bh * p.Tp + (size_t)n * C);
-            mbar_expect_tx(bar, 16384 + rows * 128);
-            tma_load_3d(st, &mapdO, hh * D + v0, n * C, b, bar);             // rows past the end of the sequence: zeros
-            if (rows == D) tma_load_3d(st + 8192, &mapdO, hh * D + 64, n * C, b, bar);
-            tma_load_2d(st + 16384, &mapQg, 0, yt, bar);
-            tma_load_2d(st + 16384 + 8192, &mapQg, 64, yt, bar);
+            mbar_expect_tx(br, bytesQ);
+            tma_load_3d(st + 16384, &mapdO, hh * D + v0, n * C, b, br);             // rows past the end of the sequence: zeros
+            if (rows == D) tma_load_3d(st + 16384 + 8192, &mapdO, hh * D + 64, n * C, b, br);
+            tma_load_2d(st, &mapQg, 0, yt, br);
+            tma_load_2d(st + 8192, &mapQg, 64, yt, br);
         };
         auto load_w = [&](int it) {
-            mbar_expect_tx(&bar_w[it & 1], kBytesW);
-            tma_load_2d(smem + kOffW + (it & 1) * kBytesW, &mapWt, 0, (int)(((size_t)bh * p.N + (p.N - 1 - it)) * D), &bar_w[it & 1]);
+            mbar_expect_tx(&bar.w[it & 1], 16384);
+            tma_load_2d(smem + offW + (it & 1) * 16384, &mapWt, 0, (int)(((size_t)bh * p.N + (p.N - 1 - it)) * D), &bar.w[it & 1]);
         };
         fetch_g(0);
         for (int it = 0; it < kDeepK && it < p.N; ++it) {
             load_k(it, it);
             if (lead && it < 2) { load_q(it); load_w(it); }
         }
-        int s = 0;
+        int s = 0;                                        // stage of chunk it's K and P, and the parity of its present round
+        uint32_t sp = 0;
         for (int it = 0; it < p.N; ++it) {
             bool more = it + kDeepK < p.N;
             if (lead) {
-                wait(&bar_fq[it & 1], (it >> 1) & 1);
+                wait(&bar.fq[it & 1], (it >> 1) & 1);
                 if (it + 2 < p.N && !s_abort) load_q(it + 2);
-                wait(&bar_fk[s], (it / kDeepK) & 1);
+                wait(&bar.fk[s], sp);
             }
             more = __shfl_sync(0xffffffffu, more && !s_abort, 0);     // one answer for the warp
             if (more) load_k(it + kDeepK, s);
             if (lead) {
-                wait(&bar_fw[it & 1], (it >> 1) & 1);
+                wait(&bar.fw[it & 1], (it >> 1) & 1);
                 if (it + 2 < p.N && !s_abort) load_w(it + 2);
             }
             __syncwarp();
-            if (++s == kDeepK) s = 0;
+            if (++s == kDeepK) { s = 0; sp ^= 1; }
         }
         if (lead && s_abort) {            // one more bounded chance for copies in flight
-            for (int i = 0; i < kDeepK; ++i) mbar_wait(&bar_k[i], 0);
-            for (int i = 0; i < 2; ++i) { mbar_wait(&bar_q[i], 0); mbar_wait(&bar_w[i], 0); }
+            for (int i = 0; i < kDeepK; ++i) mbar_wait(&bar.k[i], 0);
+            for (int i = 0; i < 2; ++i) { mbar_wait(&bar.q[i], 0); mbar_wait(&bar.w[i], 0); }
         }
     }
     tc_fence_before();
@@ -348,24 +371,27 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
 }
 
 // =================================================================================================
+struct ChunkBwdMaps { CUtensorMap Q, K, V, dO, Mt, P, Dt, dDt, Hs, dHs, dQ, dK, dV; };
 struct ChunkBwdParams {
     int logits;                // beta, alpha, lambda are logits of sigmoid gates; their gradients are taken w.r.t. the logits
     const float* rqk;          // QD_NORM_QK: 1/|q_t| per workspace row, then (BH*Tp further) 1/|k_t|
-    int group;                 // GROUPED instances: sequences per group of work items
+    int group;                 // sequences per group of work items
     int T, Tp, H, N, BH, total;   // T tokens per sequence, Tp = 64 N rows per sequence in the workspace; total = BH*N chunks
     const bf16 *beta, *alpha, *lam;
     const float* g;
     float *dbeta, *dalpha, *dlam;
     unsigned* status;
+    unsigned* next;            // work items taken beyond the first of every CTA; zero when the kernel begins
 };
 
-// shared-memory map of k_tc_chunk_bwd (bytes from the 1024-aligned base)
+// =================================================================================================
+// shared-memory map of a chunk's tiles (bytes from the 1024-aligned base)
 constexpr int oQ = 0, oK = 16384, oV = 32768, odO = 49152, oX = 65536, oMt = 81920, oP = 90112, oDt = 98304,
               odDt = 114688, oH = 131072, odH = 163840;                            // TMA-loaded tiles (X is built)
 constexpr int kBwdEarlyBytes = 3 * 16384 + 2 * 8192;
 // tiles built later reuse regions whose contents are dead by then
 constexpr int odPG = oV, odTb = oV + 8192, odW = 196608, oN = oDt, odXK = oDt + 8192, oStDv = odDt, oStDk = oX, oStDq = odW;
-constexpr int kBwdSmem = 196608 + 16384 + 1024;      // + the dW<-^T tile, written while dO is still an operand
+constexpr int kTileBytes = 196608 + 16384;     // with the dW<-^T tile, written while dO is still an operand
 constexpr int kNWG = 4;                       // warpgroups; each owns 64/kNWG columns of every 64-column accumulator
 constexpr int kCW = C / kNWG, kG8 = kCW / 8;    // columns per warpgroup, groups of 8 columns
 constexpr int kBwdCompute = 128 * kNWG;                 // epilogue threads
@@ -373,7 +399,7 @@ constexpr int kBwdCompute = 128 * kNWG;                 // epilogue threads
 // and the sums over rows and columns that become d beta, d lambda and d alpha
 constexpr int kBwdTail = kBwdCompute + 64, kBwdThreads = kBwdTail + C;
 constexpr int kBwdNb = kBwdCompute + 32;                 // participants of a named barrier: the epilogue threads and a waiting warp
-// named barriers of k_tc_chunk_bwd: 1 = the epilogue threads among themselves; the others are raised by the
+// named barriers: 1 = the epilogue threads among themselves; the others are raised by the
 // epilogue threads (bar.arrive) when a tile is complete and awaited by the MMA warp or the TMA warp (bar.sync); Sum: row
 // and column sums complete, awaited by the token threads; Tok: among themselves; End: everybody, the
 // TMA warp only arrives
@@ -382,6 +408,22 @@ constexpr int kNbSumN = kBwdCompute + C;
 
 // 8 TMEM columns of this thread's lane (no wait)
 __device__ __forceinline__ void ld8(uint32_t taddr, float* v) { tmem_ld8(taddr, v); }
+
+struct ChunkBars { uint64_t load, d, h, qk, st, a, b, c, m2, m3, m4, m5; };
+// What the warps tell each other; `_` arrays by parity of the chunk, so that the token threads can publish a chunk
+// ahead and take their sums a chunk late.
+struct ChunkShared {
+    float4 scf_[2][C];     // per token: {gamma beta, gamma_C / gamma, gamma, lambda}, one load in the last epilogue
+    float sbeta_[2][C], sg_[2][C], slam_[2][C], sgam_[2][C];
+    float2 srn_[2][C];     // NORM: {1/|k_t|, 1/|q_t|}
+    float sred_[2][2][4][C];   // per-warp column sums: [0] rowsum(dQ1 o Q) - <(K-> dh)_r, Delta_r>, [1] d lambda
+    float swk_[2][kBwdCompute / 32];        // per-warp sums of <(K-> dh)_r, Delta_r>
+    float scol[2][4][C];   // column sums of dP o P, dA o A by quarters of the rows
+    float srow[4][kNWG][C];   // per-row partial sums over each warpgroup's columns: rPP, d beta, t2, rAA
+    float swp[kBwdCompute / 32], stot[2];
+    int2 item[4];          // {chunk, sequence} of iterations it .. it + 2, by it mod 4; chunk < 0: no more
+};
+constexpr int kBwdSmem = kTileBytes + (int)sizeof(ChunkShared) + 1024;
 
 // Four epilogue warpgroups: warpgroup w (threads 128w..128w+127) owns TMEM columns [16w, 16w+16) of every 64-column
 // accumulator; inside a warpgroup, warp wq owns TMEM lanes [32 wq, 32 wq + 32), i.e. rows 32 wq .. of a 128-row product and
@@ -394,45 +436,36 @@ __device__ __forceinline__ void ld8(uint32_t taddr, float* v) { tmem_ld8(taddr, 
 // left in the workspace; dq and dk are taken through the normalisation, dx = r (dx^ - x^ <x^, dx^>), which needs the
 // row sums <x^, dx^>: dk^ and dq^ are staged in bf16 like dk and dq without NORM, and a second pass over the staged tiles, a
 // row to 16 lanes, takes the sums and rewrites them.
-template <bool HAS_LAM, bool HAS_ALPHA, bool NORM, bool GROUPED>
-__global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_constant__ CUtensorMap mapQ,
-                                                              const __grid_constant__ CUtensorMap mapK,
-                                                              const __grid_constant__ CUtensorMap mapV,
-                                                              const __grid_constant__ CUtensorMap mapdO,
-                                                              const __grid_constant__ CUtensorMap mapMt,
-                                                              const __grid_constant__ CUtensorMap mapP,
-                                                              const __grid_constant__ CUtensorMap mapDt,
-                                                              const __grid_constant__ CUtensorMap mapdDt,
-                                                              const __grid_constant__ CUtensorMap mapHs,
-                                                              const __grid_constant__ CUtensorMap mapdHs,
-                                                              const __grid_constant__ CUtensorMap mapdQ,
-                                                              const __grid_constant__ CUtensorMap mapdK,
-                                                              const __grid_constant__ CUtensorMap mapdV,
-                                                              ChunkBwdParams p) {
+// Work items: a chunk of a sequence.  They come in groups of p.group sequences, inside a group chunk by chunk from the first on
+// (which the reverse chain has left last, so its tiles are still in L2), the sequences of a chunk index next to each other.  Every
+// CTA takes the next one from a counter, two chunks ahead of its work.  Backward of 128 sequences of 32 chunks: 255 us; every
+// gridDim.x-th item to a CTA 264 - 270; from the last chunk on 258; groups of 32 sequences 263, all at a time 259.  Training passes
+// against items in sequence order with every gridDim.x-th to a CTA (and the reverse chain of then): 531 -> 514, one long
+// group of 32 sequences of 512 chunks 2549 -> 2464.
+template <bool HAS_LAM, bool HAS_ALPHA, bool NORM>
+__global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_constant__ ChunkBwdMaps m, ChunkBwdParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    // bar_load: V, dO, M^T, P, Delta^T; bar_d: dDelta^T; bar_h: h^T, dh^T; bar_qk: Q, K; bar_st: the staged dk, dq have been read
-    __shared__ uint64_t bar_load, bar_d, bar_h, bar_qk, bar_st, bm_a, bm_b, bm_c, bm_2, bm_3, bm_4, bm_5;
+    __shared__ ChunkBars bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort, s_latch;
-    // by parity of the chunk, so that the token threads can publish a chunk ahead and take their sums a chunk late
-    __shared__ __align__(16) float sbeta_[2][C], sg_[2][C], slam_[2][C], sgam_[2][C];
-    __shared__ float4 scf_[2][C];     // per token: {gamma beta, gamma_C / gamma, gamma, lambda}, one load in the last epilogue
-    __shared__ float2 srn_[2][C];     // NORM: {1/|k_t|, 1/|q_t|}
-    __shared__ float sred_[2][2][4][C];   // per-warp column sums: [0] rowsum(dQ1 o Q) - <(K-> dh)_r, Delta_r>, [1] d lambda
-    __shared__ float swk_[2][kBwdCompute / 32];        // per-warp sums of <(K-> dh)_r, Delta_r>
-    __shared__ float scol[2][4][C];   // column sums of dP o P, dA o A by quarters of the rows
-    __shared__ float srow[4][kNWG][C];   // per-row partial sums over each warpgroup's columns: rPP, d beta, t2, rAA
-
-    __shared__ float swp[kBwdCompute / 32], stot[2];
-
+    ChunkShared& sh = *reinterpret_cast<ChunkShared*>(sm + kTileBytes);
+    auto &sbeta_ = sh.sbeta_, &sg_ = sh.sg_, &slam_ = sh.slam_, &sgam_ = sh.sgam_;
+    auto& scf_ = sh.scf_;
+    auto& srn_ = sh.srn_;
+    auto& sred_ = sh.sred_;
+    auto& swk_ = sh.swk_;
+    auto& scol = sh.scol;
+    auto& srow = sh.srow;
+    auto& swp = sh.swp;
+    auto& stot = sh.stot;
+    volatile int2* const item = sh.item;
     const int tid = threadIdx.x, wg = tid >> 7, l = tid & 127, lane = tid & 31, wq = (tid >> 5) & 3;
     const int c0 = wg * kCW;                                      // my columns of a 64-column accumulator
 
     if (tid == 0) {
-        mbar_init(&bar_load, 1); mbar_init(&bar_d, 1); mbar_init(&bar_h, 1); mbar_init(&bar_qk, 1); mbar_init(&bar_st, 1);
-        mbar_init(&bm_a, 1); mbar_init(&bm_b, 1); mbar_init(&bm_c, 1); mbar_init(&bm_2, 1); mbar_init(&bm_3, 1); mbar_init(&bm_4, 1);
-        mbar_init(&bm_5, 1);
+        uint64_t* all = &bar.load;
+        for (int i = 0; i < (int)(sizeof(ChunkBars) / 8); ++i) mbar_init(all + i, 1);
         mbar_init_fence();
         s_abort = 0;
         s_latch = 0;
@@ -450,77 +483,67 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     // The tiles of a chunk arrive in three groups, as their regions fall free in the chunk before: V, dO, M^T, P, Delta^T,
     // dDelta^T after its last products; h^T, dh^T in the middle; Q, K, which the last epilogue
     // reads, at its end.  The first products need only the first two.
-    // Work item `ch` is chunk n_ of sequence bh_.  GROUPED = false: sequence-major numbering.  GROUPED = true: items are
-    // numbered in groups of p.group sequences, chunk-major inside a group, so that at any time the CTAs of the grid work
-    // on a few chunk indices of p.group sequences instead of on ~148 consecutive chunks of one long sequence.  Measured,
-    // sequence-major against groups of 32, this kernel: 114 / 109 us on 32 sequences of 64 chunks, 217 / 208 on 32 of 128,
-    // 223 / 206 on 16 of 256, 837 / 772 on 32 of 512.  An earlier form of the kernel gained nothing on 128 sequences of 32 chunks
-    // and lost most with all sequences at a time (chunk-major).  Compile-time, because the grouped arithmetic compiled into
-    // the sequence-major path cost that form 3.5 %, as a non-inlined function 14 %.
-    auto item = [&](int ch, int& n_, int& bh_) {
-        if (GROUPED) {
-            const int per = p.group * p.N, grp = ch / per, r = ch - grp * per;
-            const int g0 = grp * p.group, gs = min(p.group, p.BH - g0);       // the last group may be smaller
-            n_ = r / gs;
-            bh_ = g0 + r - n_ * gs;
-        } else {
-            bh_ = ch / p.N;
-            n_ = ch - bh_ * p.N;
-        }
+    struct Item { int n, bh; };                                  // chunk n of sequence bh; n < 0: none
+    auto slot = [&](int it) { return Item{item[it & 3].x, item[it & 3].y}; };
+    auto nth = [&](int i) {
+        if (i >= p.total) return Item{-1, 0};
+        const int per = p.group * p.N, grp = i / per, r = i - grp * per;
+        const int g0 = grp * p.group, gs = min(p.group, p.BH - g0);       // the last group may be smaller
+        return Item{r / gs, g0 + r % gs};
     };
-    auto issue_early = [&](int ch) {
-        int n_, bh_; item(ch, n_, bh_);
-        const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
-        const int yt = (int)((size_t)bh_ * p.Tp + (size_t)n_ * C);
-        const int yc = (int)(((size_t)bh_ * p.N + n_) * D);
-        mbar_expect_tx(&bar_d, 16384);            // on its own: the first product waits for it
-        tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_d);
-        mbar_expect_tx(&bar_load, kBwdEarlyBytes);
-        tma_load_2d(sm + oMt, &mapMt, 0, yt, &bar_load);
+    auto claim = [&]() { return nth((int)gridDim.x + (int)atomicAdd(p.next, 1u)); };      // a CTA's first item goes by its number
+    auto put = [&](int it, Item x) { item[it & 3].x = x.n; item[it & 3].y = x.bh; };
+    auto issue_dd = [&](Item x) {                 // dDelta^T on its own: the first product waits for it
+        mbar_expect_tx(&bar.d, 16384);
+        tma_load_2d(sm + odDt, &m.dDt, 0, (int)(((size_t)x.bh * p.N + x.n) * D), &bar.d);
+    };
+    auto issue_early = [&](Item x) {
+        const int b_ = x.bh / p.H, hh_ = x.bh % p.H;
+        const int yt = (int)((size_t)x.bh * p.Tp + (size_t)x.n * C);
+        const int yc = (int)(((size_t)x.bh * p.N + x.n) * D);
+        mbar_expect_tx(&bar.load, kBwdEarlyBytes);
+        tma_load_2d(sm + oMt, &m.Mt, 0, yt, &bar.load);
         for (int blk = 0; blk < 2; ++blk)         // token rows past the end of the sequence arrive as zeros
-            tma_load_3d(sm + oV + blk * 8192, &mapV, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
-        tma_load_2d(sm + oDt, &mapDt, 0, yc, &bar_load);
+            tma_load_3d(sm + oV + blk * 8192, &m.V, hh_ * D + blk * 64, x.n * C, b_, &bar.load);
+        tma_load_2d(sm + oDt, &m.Dt, 0, yc, &bar.load);
         for (int blk = 0; blk < 2; ++blk)
-            tma_load_3d(sm + odO + blk * 8192, &mapdO, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
-        tma_load_2d(sm + oP, &mapP, 0, yt, &bar_load);
+            tma_load_3d(sm + odO + blk * 8192, &m.dO, hh_ * D + blk * 64, x.n * C, b_, &bar.load);
+        tma_load_2d(sm + oP, &m.P, 0, yt, &bar.load);
     };
-    auto issue_h = [&](int ch) {
-        int n_, bh_; item(ch, n_, bh_);
-        const int yc = (int)(((size_t)bh_ * p.N + n_) * D);
-        mbar_expect_tx(&bar_h, 2 * 32768);
+    auto issue_h = [&](Item x) {                  // half of bar.h
+        const int yc = (int)(((size_t)x.bh * p.N + x.n) * D);
+        mbar_expect_tx(&bar.h, 2 * 32768);
+        for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + oH + blk * 16384, &m.Hs, blk * 64, yc, &bar.h);
+    };
+    auto issue_dh = [&](Item x) {                 // the other half
+        const int yc = (int)(((size_t)x.bh * p.N + x.n) * D);
+        for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + odH + blk * 16384, &m.dHs, blk * 64, yc, &bar.h);
+    };
+    auto issue_qk = [&](Item x) {
+        const int b_ = x.bh / p.H, hh_ = x.bh % p.H;
+        mbar_expect_tx(&bar.qk, 2 * 16384);
         for (int blk = 0; blk < 2; ++blk) {
-            tma_load_2d(sm + oH + blk * 16384, &mapHs, blk * 64, yc, &bar_h);
-            tma_load_2d(sm + odH + blk * 16384, &mapdHs, blk * 64, yc, &bar_h);
+            tma_load_3d(sm + oQ + blk * 8192, &m.Q, hh_ * D + blk * 64, x.n * C, b_, &bar.qk);
+            tma_load_3d(sm + oK + blk * 8192, &m.K, hh_ * D + blk * 64, x.n * C, b_, &bar.qk);
         }
     };
-    auto issue_qk = [&](int ch) {
-        int n_, bh_; item(ch, n_, bh_);
-        const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
-        mbar_expect_tx(&bar_qk, 2 * 16384);
+    // of the tiles of a chunk, those that are waited for most into L2 only, a chunk time ahead
+    auto prefetch_late = [&](Item x) {
+        const int b_ = x.bh / p.H, hh_ = x.bh % p.H;
+        const int yc = (int)(((size_t)x.bh * p.N + x.n) * D);
         for (int blk = 0; blk < 2; ++blk) {
-            tma_load_3d(sm + oQ + blk * 8192, &mapQ, hh_ * D + blk * 64, n_ * C, b_, &bar_qk);
-            tma_load_3d(sm + oK + blk * 8192, &mapK, hh_ * D + blk * 64, n_ * C, b_, &bar_qk);
+            tma_prefetch_3d(&m.Q, hh_ * D + blk * 64, x.n * C, b_);
+            tma_prefetch_3d(&m.K, hh_ * D + blk * 64, x.n * C, b_);
+            tma_prefetch_2d(&m.Hs, blk * 64, yc);
+            tma_prefetch_2d(&m.dHs, blk * 64, yc);
         }
-    };
-    // of the tiles of a chunk, those that are waited for most into L2 only, a chunk time ahead: 761 us with it and 839 without on
-    // 32 sequences of 512 chunks (training pass 2420 and 2529), 219 and 216 on 128 of 32; V, dO, M^T and P as well: no gain
-    auto prefetch_late = [&](int ch) {
-        int n_, bh_; item(ch, n_, bh_);
-        const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
-        const int yc = (int)(((size_t)bh_ * p.N + n_) * D);
-        for (int blk = 0; blk < 2; ++blk) {
-            tma_prefetch_3d(&mapQ, hh_ * D + blk * 64, n_ * C, b_);
-            tma_prefetch_3d(&mapK, hh_ * D + blk * 64, n_ * C, b_);
-            tma_prefetch_2d(&mapHs, blk * 64, yc);
-            tma_prefetch_2d(&mapdHs, blk * 64, yc);
-        }
-        tma_prefetch_2d(&mapDt, 0, yc);
-        tma_prefetch_2d(&mapdDt, 0, yc);
+        tma_prefetch_2d(&m.Dt, 0, yc);
+        tma_prefetch_2d(&m.dDt, 0, yc);
     };
     // bounded wait; once any wait has expired every later wait returns at once and the kernel drains: all
     // threads still pass every barrier, results are garbage, the status word says so
     auto wait = [&](uint64_t* bar, uint32_t parity) {
-        if (s_abort) return;
+        if (mbar_try_wait(bar, parity) || s_abort) return;
         if (!mbar_wait(bar, parity)) { s_abort = 1; *p.status = QD_ERR_TIMEOUT; }
     };
     const uint32_t aQ = smem_u32(sm + oQ), aK = smem_u32(sm + oK), aV = smem_u32(sm + oV), adO = smem_u32(sm + odO),
@@ -538,41 +561,42 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         const uint32_t issue = elect_lane();
         const uint32_t tbu = uniform(tb);
         const uint32_t T0 = tbu, T1 = tbu + 64, T2 = tbu + 128, T3 = tbu + 192, T4 = tbu + 256, T5 = tbu + 320, T6 = tbu + 384, T7 = tbu + 448;
+        __syncthreads();                                                 // the first item is known
         grid_dep_wait();
         __syncthreads();                                                 // the first chunk's coefficients have been published
-        for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
+        for (int it = 0; (int)uniform((uint32_t)slot(it).n) >= 0; ++it) {
             const uint32_t ph = it & 1;
             if (__any_sync(0xffffffffu, s_latch)) break;
-            wait(&bar_d, ph);
-            wait(&bar_h, ph);
+            wait(&bar.d, ph);
+            wait(&bar.h, ph);
             __syncwarp();
             tc_fence_after();
             umma_product_w<true, true>(T3, aH, 16384, adDt, 8192, C, D, false, issue, true);     // -h dDelta^T      [i][r] = dW<-^T
-            umma_commit_w(&bm_a, issue);
-            wait(&bar_load, ph);
+            umma_commit_w(&bar.a, issue);
+            wait(&bar.load, ph);
             umma_product_w<false, false>(T6, adDt, 16384, aMt, 8192, C, C, false, issue);        // dDelta^T M       [j][s]
             umma_product_w<false, true, 64>(T2, aV, 8192, adDt, 8192, C, D, false, issue);       // V dDelta^T       [s][r]
-            umma_commit_w(&bm_b, issue);                // from here on no product reads V or dDelta^T any more
+            umma_commit_w(&bar.b, issue);                // from here on no product reads V or dDelta^T any more
             umma_product_w<false, true, 64>(T1, adO, 8192, aDt, 8192, C, D, false, issue);       // dO Delta^T       [r][s]
-            umma_commit_w(&bm_c, issue);
+            umma_commit_w(&bar.c, issue);
             umma_product_w<true, false>(T4, aH, 16384, adO, 8192, C, D, false, issue);           // h dO^T           [i][r]
-            wait(&bar_qk, ph);
+            wait(&bar.qk, ph);
             nb_sync(kNbDW, kBwdNb);                                      // the dW<-^T tile is complete
             nb_sync(kNbX, kBwdNb);                                       // X has been built
             tc_fence_after();
             // the product that the dependent chain waits for goes first, those that are needed late after it
             umma_product_w<false, true, 64>(T3, aXe, 8192, adW, 8192, C, D, false, issue);       // X dW<-^T         [s][r]
-            umma_commit_w(&bm_2, issue);
+            umma_commit_w(&bar.m2, issue);
             umma_product_w<false, false, 64>(T0, aXe, 8192, aK, 8192, C, D, false, issue);       // X K^T            [r][i]
             umma_product_w<true, true>(T5, adH, 16384, aDt, 8192, C, D, false, issue);           // dh Delta^T       [i][s]
             nb_sync(kNbDTb, kBwdNb);
             tc_fence_after();
             umma_product_w<true, true, 64>(T3, adTb, 8192, aMt, 8192, C, C, false, issue);       // N~ = dT diag(beta) M^T   [r][u]
-            umma_commit_w(&bm_3, issue);                // from here on nobody reads h, dh or Delta^T
+            umma_commit_w(&bar.m3, issue);                // from here on nobody reads h, dh or Delta^T
             nb_sync(kNbN, kBwdNb);                                       // N~ is a tile, and so is dP o Gamma
             tc_fence_after();
             umma_product_w<false, true, 64>(T2, aMt, 8192, aN, 8192, C, C, false, issue, true);  // dA = -M^T N~     [r][s]
-            umma_commit_w(&bm_4, issue);
+            umma_commit_w(&bar.m4, issue);
             umma_product_w<true, true>(T1, aQ, 8192, adPG, 8192, C, C, false, issue);            // (dPG^T Q)^T      [i][s]
             umma_product_w<true, false>(T3, aK, 8192, adPG, 8192, C, C, false, issue);           // (dPG K)^T        [i][r]
             nb_sync(kNbDV, kBwdNb);                                      // T6 has been read
@@ -582,60 +606,49 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             tc_fence_after();
             umma_product_w<true, false>(T7, aK, 8192, adXK, 8192, C, C, false, issue);           // (dXK K)^T        [i][r]
             umma_product_w<true, true>(T1, aXe, 8192, adXK, 8192, C, C, true, issue);            // + (dXK^T X)^T    [i][s]
-            umma_commit_w(&bm_5, issue);
+            umma_commit_w(&bar.m5, issue);
             nb_sync(kNbEnd, kBwdThreads);                                // every read of this chunk's tiles and accumulators is done
         }
     } else if (tid >= kBwdNb && tid < kBwdTail) {
         // =============================== TMA warp ===============================
         const bool lead = lane == 0;
-        if (lead && (int)blockIdx.x < p.total) {
+        if (lead) put(0, nth((int)blockIdx.x));
+        __syncthreads();                                                 // the first item is known
+        if (lead) {
             // first chunk: everything that the reverse chain (the kernel before this one) does not write is fetched
             // before waiting for it -- inputs, and tiles of kernels that had finished before the reverse chain began
-            const int ch = blockIdx.x;
-            int n_, bh_; item(ch, n_, bh_);
-            const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
-            const int yc = (int)(((size_t)bh_ * p.N + n_) * D), yt = (int)((size_t)bh_ * p.Tp + (size_t)n_ * C);
-            issue_qk(ch);
-            mbar_expect_tx(&bar_load, kBwdEarlyBytes);
-            for (int blk = 0; blk < 2; ++blk) {
-                tma_load_3d(sm + oV + blk * 8192, &mapV, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
-                tma_load_3d(sm + odO + blk * 8192, &mapdO, hh_ * D + blk * 64, n_ * C, b_, &bar_load);
-            }
-            tma_load_2d(sm + oMt, &mapMt, 0, yt, &bar_load);
-            tma_load_2d(sm + oP, &mapP, 0, yt, &bar_load);
-            tma_load_2d(sm + oDt, &mapDt, 0, yc, &bar_load);
-            mbar_expect_tx_only(&bar_h, 32768);
-            for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + oH + blk * 16384, &mapHs, blk * 64, yc, &bar_h);
+            const Item x = slot(0);
+            issue_qk(x);
+            issue_early(x);
+            issue_h(x);
             grid_dep_wait();
-            mbar_expect_tx(&bar_h, 32768);
-            for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + odH + blk * 16384, &mapdHs, blk * 64, yc, &bar_h);
-            mbar_expect_tx(&bar_d, 16384);
-            tma_load_2d(sm + odDt, &mapdDt, 0, yc, &bar_d);
-            mbar_arrive(&bar_st);                                        // nothing is staged yet
+            issue_dh(x);
+            issue_dd(x);
+            put(1, claim());
+            mbar_arrive(&bar.st);                                        // nothing is staged yet
         }
-        grid_dep_wait();
         __syncthreads();                                                 // the first chunk's coefficients have been published
-        for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
-            int n, bh; item(ch_id, n, bh);
-            const int b = bh / p.H, hh = bh % p.H;
-            const int next_id = ch_id + gridDim.x;
-            const bool more = next_id < p.total;
+        for (int it = 0; slot(it).n >= 0; ++it) {
+            const Item cur = slot(it), next = slot(it + 1);
+            const int n = cur.n, b = cur.bh / p.H, hh = cur.bh % p.H;
+            const bool more = next.n >= 0;
             const uint32_t ph = it & 1;
             if (__any_sync(0xffffffffu, s_latch)) break;
-            if (lead && more) prefetch_late(next_id);
             if (lead) {
-                wait(&bm_3, ph);                                         // from here on nobody reads h or dh
-                if (more && !s_abort) issue_h(next_id);
+                if (more) prefetch_late(next);
+                put(it + 2, more ? claim() : next);
+                wait(&bar.m3, ph);                                       // from here on nobody reads h or dh
+                if (more && !s_abort) { issue_h(next); issue_dh(next); }
             }
             nb_sync(kNbDVt, kBwdNb);                                     // the dv staging tile is complete
             if (lead) {
-                tma_store_3d(&mapdV, sm + oStDv, hh * D, n * C, b);          // rows past the end of the sequence are skipped
-                tma_store_3d(&mapdV, sm + oStDv + 8192, hh * D + 64, n * C, b);
+                tma_store_3d(&m.dV, sm + oStDv, hh * D, n * C, b);          // rows past the end of the sequence are skipped
+                tma_store_3d(&m.dV, sm + oStDv + 8192, hh * D + 64, n * C, b);
                 tma_store_commit();
                 tma_store_wait_read();
-                wait(&bm_5, ph);                                         // from here on nobody reads anything but Q, K
+                wait(&bar.m5, ph);                                         // from here on nobody reads anything but Q, K
                 fence_proxy_async();
-                if (more && !s_abort) issue_early(next_id);
+                if (more && !s_abort) { issue_dd(next); issue_early(next); }
             }
             nb_sync(kNbOut, kBwdNb);                                     // the dk and dq staging tiles are complete
             // s_latch is read by everyone right after the barrier and not written again before the next one;
@@ -644,17 +657,17 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             __syncwarp();
             nb_arrive(kNbEnd, kBwdThreads);                              // nobody waits for the copies to be issued
             if (lead) {
-                tma_store_3d(&mapdK, sm + oStDk, hh * D, n * C, b);
-                tma_store_3d(&mapdK, sm + oStDk + 8192, hh * D + 64, n * C, b);
-                tma_store_3d(&mapdQ, sm + oStDq, hh * D, n * C, b);
-                tma_store_3d(&mapdQ, sm + oStDq + 8192, hh * D + 64, n * C, b);
+                tma_store_3d(&m.dK, sm + oStDk, hh * D, n * C, b);
+                tma_store_3d(&m.dK, sm + oStDk + 8192, hh * D + 64, n * C, b);
+                tma_store_3d(&m.dQ, sm + oStDq, hh * D, n * C, b);
+                tma_store_3d(&m.dQ, sm + oStDq + 8192, hh * D + 64, n * C, b);
                 tma_store_commit();
                 fence_proxy_async();                                     // the epilogue's reads of Q precede the copy into its region
-                if (more && !s_abort) issue_qk(next_id);
+                if (more && !s_abort) issue_qk(next);
             }
             if (lead) {
                 tma_store_wait_read();                                   // the staging tiles have been read by the stores
-                mbar_arrive(&bar_st);
+                mbar_arrive(&bar.st);
             }
             __syncwarp();
         }
@@ -666,8 +679,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         bf16 zb = __float2bfloat16_rn(0.f), zl = zb, za = zb;                // as stored, converted a chunk later: nothing waits for the loads
         float cg = 0.f, cgC = 0.f, rq = 1.f, rk = 1.f;
         bool tok = false;
-        auto fetch = [&](int ch) {
-            int n_, bh_; item(ch, n_, bh_);
+        auto fetch = [&](Item x) {
+            const int n_ = x.n, bh_ = x.bh;
             const int b_ = bh_ / p.H, hh_ = bh_ % p.H;
             tok = n_ * C + r < p.T;                               // tokens past the end of the sequence: beta = 0, alpha = 1
             const size_t cr = ((size_t)b_ * p.T + (size_t)n_ * C + r) * p.H + hh_, wr = (size_t)bh_ * p.Tp + (size_t)n_ * C;
@@ -690,13 +703,14 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             scf_[par][r] = make_float4(gm * be, __expf(cgC - cg), gm, lm);
             if (NORM) srn_[par][r] = make_float2(rk, rq);
         };
-        if ((int)blockIdx.x < p.total) { fetch(blockIdx.x); publish(0); }
-        grid_dep_wait();                    // coefficients and log-decays are older than the reverse chain; the results below are not
+        __syncthreads();                                                 // the first item is known
+        if (slot(0).n >= 0) { fetch(slot(0)); publish(0); }
+        grid_dep_wait();
         __syncthreads();
         // what the sums at the end of a chunk need of it, taken up a chunk later
         float dg_pre = 0.f, dhh = 0.f, be0 = 0.f, lm0 = 0.f, al0 = 1.f, gmC = 1.f;
-        auto finish = [&](int ch, int par) {
-            int n, bh; item(ch, n, bh);
+        auto finish = [&](Item x, int par) {
+            const int n = x.n, bh = x.bh;
             const size_t at = ((size_t)(bh / p.H) * p.T + (size_t)n * C + r) * p.H + bh % p.H;
             const bool in = n * C + r < p.T;
             float dg = dg_pre, dl = 0.f;
@@ -726,17 +740,17 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
                 if (in && p.dalpha) p.dalpha[at] = p.logits ? dg * (1.f - al0) : dg / al0;
             }
         };
-        int prev = -1;
+        Item prev{-1, 0};
         uint32_t last_ph = 0;
-        for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
-            int n, bh; item(ch_id, n, bh);
-            const int next_id = ch_id + gridDim.x;
+        for (int it = 0; slot(it).n >= 0; ++it) {
+            const Item cur = slot(it), next = slot(it + 1);
+            const int n = cur.n, bh = cur.bh;
             const uint32_t ph = it & 1;
-            if (__any_sync(0xffffffffu, s_latch)) { prev = -1; break; }
-            if (prev >= 0) finish(prev, ph ^ 1);
+            if (__any_sync(0xffffffffu, s_latch)) { prev.n = -1; break; }
+            if (prev.n >= 0) finish(prev, ph ^ 1);
             const float gm = sgam_[ph][C - 1];
             be0 = be; lm0 = lm; al0 = al; gmC = gm;
-            if (next_id < p.total) fetch(next_id);
+            if (next.n >= 0) fetch(next);
             nb_sync(kNbSum, kNbSumN);                                    // row sums and scratch are complete
             float rPP = 0.f, t2 = 0.f, rAA = 0.f, dbt = 0.f;
 #pragma unroll
@@ -755,12 +769,12 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
 #pragma unroll
                 for (int w = 0; w < kBwdCompute / 32; ++w) dhh += swp[w];
             }
-            if (next_id < p.total) publish(ph ^ 1);
+            if (next.n >= 0) publish(ph ^ 1);
             nb_sync(kNbEnd, kBwdThreads);                                // every read of this chunk's tiles and accumulators is done
-            prev = ch_id;
+            prev = cur;
             last_ph = ph;
         }
-        if (prev >= 0) finish(prev, last_ph);
+        if (prev.n >= 0) finish(prev, last_ph);
     } else {
     // ======================================== epilogue threads ========================================
     auto csync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(kNbC), "r"(kBwdCompute) : "memory"); };   // warps arrive converged
@@ -771,17 +785,18 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     uint32_t foff[2];
 #pragma unroll
     for (int g = 0; g < 2; ++g) foff[g] = (wq >> 1) * 8192 + sw128_chunk(c0 + 8 * g + (lane & 7), (wq & 1) * 4 + (lane >> 3));
+    __syncthreads();                    // the first item is known
     grid_dep_wait();
     __syncthreads();                    // the first chunk's coefficients have been published
 
-    for (int ch_id = blockIdx.x, it = 0; ch_id < p.total; ch_id += gridDim.x, ++it) {
+    for (int it = 0; slot(it).n >= 0; ++it) {
     const uint32_t ph = it & 1;
     if (s_latch) break;
     const float *sbeta = sbeta_[ph], *slam = slam_[ph], *sg = sg_[ph], *sgam = sgam_[ph];
     const float4* scf = scf_[ph];
     const float2* srn = srn_[ph];
     // ---- partial <dh,h>_F, under the first products ---------------------------------------------------
-    wait(&bar_h, ph);
+    wait(&bar.h, ph);
     float dhh_part = 0.f;
     if (want_da)
 #pragma unroll
@@ -803,8 +818,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         if (lane == 0) swp[tid >> 5] = dhh_part;
     }
     // ---- dW<-^T = -h dDelta^T: row i = l as an operand tile (region of its own: dO is still being read) -----
-    wait(&bar_st, ph);                                    // the staged dk, dq of the chunk before lie over X and this tile
-    wait(&bm_a, ph);
+    wait(&bar.st, ph);                                    // the staged dk, dq of the chunk before lie over X and this tile
+    wait(&bar.a, ph);
     tc_fence_after();
 #pragma unroll
     for (int g8 = 0; g8 < kG8; ++g8) {
@@ -816,8 +831,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     fence_proxy_async();
     tc_fence_before();
     nb_arrive(kNbDW, kBwdNb);
-    wait(&bar_load, ph);
-    wait(&bar_qk, ph);
+    wait(&bar.load, ph);
+    wait(&bar.qk, ph);
     // ---- X = K + lambda Q (the products that do not read X are already running) ------------------------
     if (has_lam || NORM) {
         constexpr int kPer = 16 / (kBwdCompute / 64);     // 16-byte chunks of a row per thread
@@ -871,8 +886,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         }
     }
     // ---- dT^T row s, columns r;  M[r][s] = line s of Mt ------------------------------------------------
-    wait(&bm_b, ph);
-    wait(&bm_2, ph);
+    wait(&bar.b, ph);
+    wait(&bar.m2, ph);
     tc_fence_after();
     {
         float a[8], bq[8], db[2] = {}, mb[2] = {};
@@ -904,7 +919,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         if (my_row) { srow[1][wg][mine] = d; srow[2][wg][mine] = t2; }
     }
     // ---- dP, under N~: causal mask, dP o P (row and column sums), dP o Gamma as an operand tile ----------
-    wait(&bm_c, ph);
+    wait(&bar.c, ph);
     tc_fence_after();
     {
         float v[8], rPP[2] = {}, cP[4] = {};
@@ -935,7 +950,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         }
     }
     // ---- N~ = dT diag(beta) M^T, copied out as an operand tile --------------------------------------
-    wait(&bm_3, ph);
+    wait(&bar.m3, ph);
     tc_fence_after();
     {
         float v[8];
@@ -972,7 +987,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     nb_arrive(kNbDV, kBwdNb);
     nb_arrive(kNbDVt, kBwdNb);
     // ---- dA = -M^T N~ -----------------------------------------------------------------------------
-    wait(&bm_4, ph);
+    wait(&bar.m4, ph);
     tc_fence_after();
     {
         float da[8], xk[8], dbr[2] = {}, cA[4] = {};
@@ -1007,7 +1022,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         }
     }
     nb_arrive(kNbSum, kNbSumN);
-    wait(&bm_5, ph);
+    wait(&bar.m5, ph);
     tc_fence_after();
     // The last epilogue: dk and dq, transposed, into their staging tiles, and the column sums (over the d_k index i, i.e.
     // down the fragments and across eight lanes) that d lambda and the decay gradient need.
@@ -1112,7 +1127,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     }  // epilogue threads
     tc_fence_before();
     __syncthreads();
-    if (tid == kBwdCompute && s_abort) { mbar_wait(&bar_load, 0); mbar_wait(&bar_d, 0); mbar_wait(&bar_h, 0); mbar_wait(&bar_qk, 0); }   // one more bounded chance for copies in flight
+    if (tid == kBwdCompute && s_abort) { mbar_wait(&bar.load, 0); mbar_wait(&bar.d, 0); mbar_wait(&bar.h, 0); mbar_wait(&bar.qk, 0); }   // one more bounded chance for copies in flight
     if (tid < 32) tmem_dealloc(tb, 512);
 }
 
@@ -1137,15 +1152,16 @@ cudaError_t tc_chain_bwd(const ChunkArgs& a) {
         return cudaErrorInvalidValue;
     ChainBwdParams p{};
     p.Tp = Tp; p.H = s.H; p.N = (int)N;
-    p.rows = rows;
     p.dhT_early = a.own_predecessor ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.g = (const float*)(a.ws + a.TL.g);
     p.dhT = a.dhT; p.dh0 = a.dh0;
     p.status = (unsigned*)(a.ws + a.TL.status);
-    cudaError_t e = set_smem(k_tc_chain_bwd, kChainSmem);
+    p.next = (unsigned*)(a.ws + a.TL.next);
+    const auto kern = rows == D ? k_tc_chain_bwd<D> : k_tc_chain_bwd<D / 2>;
+    cudaError_t e = set_smem(kern, kChainSmem);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(k_tc_chain_bwd, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream,
+    return launch_overlapped(kern, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream,
                              mWt, mdO, mQg, mK, mP, mdHs, mdDt, p);
 }
 
@@ -1153,54 +1169,48 @@ cudaError_t tc_chunk_bwd(const ChunkArgs& a) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
     const uint64_t BH = (uint64_t)s.B * s.H, N = Tp / kChunk;
-    CUtensorMap mQ, mK, mV, mdO, mMt, mP, mDt, mdDt, mHs, mdHs, mdQ, mdK, mdV;
-    if (!make_tmap_tokens(&mdQ, a.dq, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_tokens(&mdK, a.dk, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_tokens(&mdV, a.dv, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_tokens(&mQ, a.q, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_tokens(&mV, a.v, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_tokens(&mdO, a.dO, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_bf16_2d(&mMt, a.ws + a.TL.Mt, 64, BH * Tp, 128, 64) ||
-        !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, BH * Tp, 128, 64) ||
-        !make_tmap_bf16_2d(&mDt, a.ws + a.TL.Dt, 64, BH * N * D, 128, 128) ||
-        !make_tmap_bf16_2d(&mdDt, a.ws + a.TL.dDt, 64, BH * N * D, 128, 128) ||
-        !make_tmap_bf16_2d(&mHs, a.ws + a.TL.hsT, D, BH * N * D, D * 2, 128) ||
-        !make_tmap_bf16_2d(&mdHs, a.ws + a.TL.dhsT, D, BH * N * D, D * 2, 128))
+    ChunkBwdMaps m;
+    if (!make_tmap_tokens(&m.dQ, a.dq, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_tokens(&m.dK, a.dk, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_tokens(&m.dV, a.dv, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_tokens(&m.Q, a.q, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_tokens(&m.K, a.k, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_tokens(&m.V, a.v, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_tokens(&m.dO, a.dO, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_bf16_2d(&m.Mt, a.ws + a.TL.Mt, 64, BH * Tp, 128, 64) ||
+        !make_tmap_bf16_2d(&m.P, a.ws + a.TL.P, 64, BH * Tp, 128, 64) ||
+        !make_tmap_bf16_2d(&m.Dt, a.ws + a.TL.Dt, 64, BH * N * D, 128, 128) ||
+        !make_tmap_bf16_2d(&m.dDt, a.ws + a.TL.dDt, 64, BH * N * D, 128, 128) ||
+        !make_tmap_bf16_2d(&m.Hs, a.ws + a.TL.hsT, D, BH * N * D, D * 2, 128) ||
+        !make_tmap_bf16_2d(&m.dHs, a.ws + a.TL.dhsT, D, BH * N * D, D * 2, 128))
         return cudaErrorInvalidValue;
     ChunkBwdParams p{};
     p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = (int)N; p.BH = (int)BH; p.total = (int)(BH * N);
+    p.group = (int)std::min<uint64_t>(BH, 64);
     p.beta = (const bf16*)a.beta; p.alpha = (const bf16*)a.alpha; p.lam = (const bf16*)a.lam;
     p.g = (const float*)(a.ws + a.TL.g);
     p.dbeta = a.dbeta; p.dalpha = a.dalpha; p.dlam = a.dlam;
     p.logits = a.logits ? 1 : 0;
     p.rqk = a.norm ? (const float*)(a.ws + a.TL.rqk) : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
+    p.next = (unsigned*)(a.ws + a.TL.next);
     // the instance without lambda / without the forget gate needs the input AND its gradient to be absent
     const bool lam = a.lam || a.dlam, alpha = a.alpha || a.dalpha;
-    const bool grouped = N >= 64;         // long sequences: work items in groups of 32 sequences (see the kernel)
-    p.group = 32;
-    using Kern = decltype(&k_tc_chunk_bwd<true, true, false, false>);
-    static const Kern table[16] = {
-        k_tc_chunk_bwd<false, false, false, false>, k_tc_chunk_bwd<false, false, false, true>,
-        k_tc_chunk_bwd<false, false, true, false>,  k_tc_chunk_bwd<false, false, true, true>,
-        k_tc_chunk_bwd<false, true, false, false>,  k_tc_chunk_bwd<false, true, false, true>,
-        k_tc_chunk_bwd<false, true, true, false>,   k_tc_chunk_bwd<false, true, true, true>,
-        k_tc_chunk_bwd<true, false, false, false>,  k_tc_chunk_bwd<true, false, false, true>,
-        k_tc_chunk_bwd<true, false, true, false>,   k_tc_chunk_bwd<true, false, true, true>,
-        k_tc_chunk_bwd<true, true, false, false>,   k_tc_chunk_bwd<true, true, false, true>,
-        k_tc_chunk_bwd<true, true, true, false>,    k_tc_chunk_bwd<true, true, true, true>,
+    using Kern = decltype(&k_tc_chunk_bwd<true, true, false>);
+    static const Kern table[8] = {
+        k_tc_chunk_bwd<false, false, false>, k_tc_chunk_bwd<false, false, true>, k_tc_chunk_bwd<false, true, false>,
+        k_tc_chunk_bwd<false, true, true>,   k_tc_chunk_bwd<true, false, false>, k_tc_chunk_bwd<true, false, true>,
+        k_tc_chunk_bwd<true, true, false>,   k_tc_chunk_bwd<true, true, true>,
     };
-    const Kern kern = table[(lam ? 8 : 0) + (alpha ? 4 : 0) + (a.norm ? 2 : 0) + (grouped ? 1 : 0)];
+    const Kern kern = table[(lam ? 4 : 0) + (alpha ? 2 : 0) + (a.norm ? 1 : 0)];
     cudaError_t e = set_smem(kern, kBwdSmem);
     if (e != cudaSuccess) return e;
-    // persistent: one CTA per SM walks the work items with stride gridDim.x
+    // persistent: one CTA per SM
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<uint64_t>(BH * N, (uint64_t)sms);
-    return launch_overlapped(kern, dim3(grid), dim3(kBwdThreads), kBwdSmem, a.stream, mQ, mK, mV, mdO, mMt, mP,
-                             mDt, mdDt, mHs, mdHs, mdQ, mdK, mdV, p);
+    return launch_overlapped(kern, dim3(grid), dim3(kBwdThreads), kBwdSmem, a.stream, m, p);
 }
 
 }  // namespace qd

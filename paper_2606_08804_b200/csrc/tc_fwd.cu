@@ -777,6 +777,7 @@ TcLayout tc_layout(const qd_shape& s) {
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = (off + bytes + 1023) & ~(size_t)1023; return o; };
     L.status = take(256);
+    L.next = L.status + 128;
     L.g = take(BH * T * 4);
     L.Qg = take(BH * T * s.dk * 2);
     L.P = take(BH * T * kChunk * 2);

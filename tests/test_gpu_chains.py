@@ -17,3 +17,23 @@ def test_chain_split(B, H, T):
     _fwd_check(cfg, d, save=True)
     _bwd_check(cfg, d, reuse=True)
     _bwd_check(cfg, d)
+
+
+@pytest.mark.parametrize("B,H,T", [(1, 64, 65), (5, 13, 65), (3, 43, 129)])
+def test_chunk_order(B, H, T):
+    """Work items of the chunk backward: one group of 64 sequences, a second one of one, three; taken from a counter, so a second
+    backward over the same forward has to find it at zero again."""
+    import torch
+
+    from gpu_util import dev_inputs
+    from paper_2606_08804_b200 import binding as qd
+
+    cfg = replace(gen.CONFIGS["cfg2"], B=B, H=H, T=T, regime="trained_like", seed=331)
+    d = gen.make_chunk_inputs(cfg)
+    _bwd_check(cfg, d, reuse=True)
+    t = dev_inputs(d, cfg.dtype)
+    a = [t[n] for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")]
+    _, _, ws = qd.chunk_fwd(*a, save_for_bwd=True)
+    first, second = (qd.chunk_bwd(*a, t["dO"], t["dhT"], workspace=ws, reuse_fwd=True) for _ in range(2))
+    for n, x in first.items():
+        assert x is None or torch.equal(x, second[n]), n
