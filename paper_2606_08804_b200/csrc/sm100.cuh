@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/qdelta.h"
+
 namespace qd {
 namespace sm100 {
 
@@ -61,6 +63,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
         if (polls == 0) t0 = now;
         else if (now - t0 > limit_ns) return false;
     }
+}
+
+// What follows an unsuccessful first poll: mbar_wait, given up as soon as another wait of the CTA has expired (every later wait
+// then returns at once: the kernel drains).
+__device__ __forceinline__ bool wait_on(uint64_t* bar, uint32_t parity, volatile int& s_abort, unsigned* status) {
+    const uint32_t t0 = global_timer_lo();
+#pragma unroll 1
+    while (!s_abort) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if (global_timer_lo() - t0 > kWaitLimitNs) { s_abort = 1; *status = QD_ERR_TIMEOUT; }
+    }
+    return false;
 }
 
 // ---- programmatic dependent launch ------------------------------------------------------------------------------

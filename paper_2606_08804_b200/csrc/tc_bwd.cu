@@ -23,18 +23,6 @@ typedef __nv_bfloat16 bf16;
 constexpr int C = kChunk;      // 64
 constexpr int D = 128;         // d_k = d_v
 
-// What follows an unsuccessful first poll: mbar_wait, given up as soon as another wait of the CTA has expired (every later wait
-// then returns at once: the kernel drains).
-__device__ __forceinline__ bool wait_on(uint64_t* bar, uint32_t parity, volatile int& s_abort, unsigned* status) {
-    const uint32_t t0 = global_timer_lo();
-#pragma unroll 1
-    while (!s_abort) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (global_timer_lo() - t0 > kWaitLimitNs) { s_abort = 1; *status = QD_ERR_TIMEOUT; }
-    }
-    return false;
-}
-
 // One halving step of a column sum across the lanes of a warp: lanes whose `off` bit is set keep the upper half
 // of the N values, the others the lower half; each adds what its partner sends.
 template <int N>

@@ -1,7 +1,7 @@
 // Tensor-core (tcgen05 / TMEM / TMA) chunkwise forward for bf16, d_k = d_v = 128, chunk 64.
 //
 // Two kernels, following Section 3.3.2:
-//   k_tc_prep       one CTA per PAIR of chunks (128 tokens): g, X = K + diag(lambda) Q, the Gram
+//   k_tc_prep       one CTA per chunk, four to an SM: g, X = K + diag(lambda) Q, the Gram
 //                   blocks X K^T and Q K^T, the UT-transform inverse, and the WY factors.  It leaves,
 //                   per chunk, in bf16:  Qg = diag(gamma) Q  [token][dk],
 //                   P = Gamma o (Q K^T) causal incl. diagonal [token][64],
@@ -28,7 +28,7 @@ constexpr int D = 128;         // d_k = d_v
 // =================================================================================================
 struct PrepParams {
     float* rqk;                // non-null: L2-normalise q and k here; [0, BH*Tp) <- 1/|q_t|, [BH*Tp, 2 BH*Tp) <- 1/|k_t|
-    int T, Tp, H, N, BH;       // T tokens per sequence; the workspace holds Tp = 64 N >= T rows per sequence (N even)
+    int T, Tp, H, N, BH;       // T tokens per sequence; the workspace holds Tp = 64 N >= T rows per sequence
     const bf16 *beta, *alpha, *lam;
     float* g;
     bf16* Qg;
@@ -36,23 +36,23 @@ struct PrepParams {
     unsigned* status;
 };
 
-// 96 KB: Q (later X, in place) | K (later A in fp32, then the T tiles, then P) | V; at the end the first and the
-// last 32 KB stage U~^T and W~^T for their TMA stores.  Two CTAs fit on one SM.
-constexpr int kPrepSmem = 3 * 32768 + 1024;
-constexpr int kPrepThreads = 256;
+// 48 KB: K (then A in fp32, then the T tiles, then P) | Q (then V, then W~^T) | X (then U~^T).  Four CTAs fit on one SM.
+constexpr int kPrepSmem = 3 * 16384 + 1024;
+constexpr int kPrepCompute = 128, kPrepThreads = kPrepCompute + 32;       // + a warp that issues every copy and every product
 
 // The 64 x 64 matrices of the inverse are kept transposed, [column i][row r], so that a column is contiguous; groups of
-// four rows are permuted by column so that the fragment loads of a 16 x 8 or 8 x 8 piece, the epilogue's stores (rows
-// across the lanes) and 16-byte accesses along a column all spread over the banks.
-__device__ __forceinline__ int at_off(int i, int r) { return i * C + (r ^ (((i & 3) << 3) | (i & 4))); }
+// four rows are permuted by column so that the fragment loads of a 16 x 8 or 8 x 8 piece, the epilogue's stores (fragments: eight
+// rows, every second column) and 16-byte accesses along a column all spread over the banks.
+__device__ __forceinline__ int at_swizzle(int i) { return (((i ^ (i >> 2)) & 1) << 3) | ((i & 2) << 3) | (i & 4); }
+__device__ __forceinline__ int at_off(int i, int r) { return i * C + (r ^ at_swizzle(i)); }
 
-// acc (16 x 16) += X Y over k = 0..15: X(m, k) = a[at_off(am + m, ak + k)], Y(k, n) = b[at_off(bk + k, bn + n)] with am, ak, bk, bn
-// multiples of 8, fp32-accurate (three tf32 products).
+// acc (16 x 16) += X Y over k = 0..15: X(m, k) = a[at_off(am + m, ak + k)], Y(k, n) = b[at_off(bk + k, bn + n)] with am, ak, bk
+// multiples of 8, bn of 16, fp32-accurate (three tf32 products).
 __device__ __forceinline__ void mm16(float (&acc)[2][4], const float* a, int am, int ak, const float* b, int bk, int bn) {
     const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
     const float *a0 = a + (am + g) * C + t + (g & 4), *a1 = a + (am + g) * C + t + (4 - (g & 4));    // columns t, t + 4 of a step
-    const int am8 = (g & 3) << 3;
-    const float *b0 = b + (bk + t) * C + (bn ^ (t << 3)) + g, *b1 = b + (bk + t + 4) * C + (bn ^ (t << 3)) + (g ^ 4);
+    const int am8 = at_swizzle(g) & 24;
+    const float *b0 = b + (bk + t) * C + (bn ^ (t << 3)) + g, *b1 = b + (bk + t + 4) * C + (bn ^ (t << 3) ^ 8) + (g ^ 4);
     const int b8 = (t & 1) ? -8 : 8;                                                                   // column + 8 of Y
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
@@ -61,7 +61,7 @@ __device__ __forceinline__ void mm16(float (&acc)[2][4], const float* a, int am,
         tf32_split(a0[ac], ah[0], al[0]); tf32_split(a0[ac + 8 * C], ah[1], al[1]);
         tf32_split(a1[ac], ah[2], al[2]); tf32_split(a1[ac + 8 * C], ah[3], al[3]);
         tf32_split(b0[8 * s * C], bh[0][0], bl[0][0]); tf32_split(b1[8 * s * C], bh[0][1], bl[0][1]);
-        tf32_split(b0[8 * s * C + b8], bh[1][0], bl[1][0]); tf32_split(b1[8 * s * C + b8], bh[1][1], bl[1][1]);
+        tf32_split(b0[8 * s * C + b8], bh[1][0], bl[1][0]); tf32_split(b1[8 * s * C - b8], bh[1][1], bl[1][1]);
 #pragma unroll
         for (int j = 0; j < 2; ++j) mma_tf32(acc[j], al, bh[j]);
 #pragma unroll
@@ -78,16 +78,17 @@ __device__ __forceinline__ void put16(const float (&acc)[2][4], float sign, floa
         for (int h = 0; h < 2; ++h)
             *reinterpret_cast<float2*>(d + at_off(dm + g + 8 * h, dn + 8 * j + 2 * t)) = make_float2(sign * acc[j][2 * h], sign * acc[j][2 * h + 1]);
 }
-// M_c = (I + A_c)^-1 of two chunks, in place, both transposed (at_off): A^T comes strictly upper triangular in this view,
-// M^T leaves with its zeros and ones.  Block-wise: the 16 x 16 diagonal blocks by right-looking substitution, a column in
-// the registers of a lane, two blocks per warp; then blocks joined twice, M21^T = -M11^T (A21^T M22^T), on the warp-level
-// tensor instruction, zero blocks left out.  A column walked over all 64 rows in registers takes 63 dependent steps whose
-// broadcast loads of A are bound by shared-memory wavefronts: 7300 cycles of a CTA's 28000, against 4600 - 5300 of 24400 for this.
-__device__ __forceinline__ void invert_pair(float* sA) {
+// the four warps that do the arithmetic of a chunk among themselves
+__device__ __forceinline__ void psync() { asm volatile("bar.sync 1, %0;" ::"n"(kPrepCompute) : "memory"); }
+// M = (I + A)^-1, in place, both transposed (at_off): A^T comes strictly upper triangular in this view, M^T leaves with its zeros
+// and ones.  Block-wise: the 16 x 16 diagonal blocks by right-looking substitution, a column in the registers of a lane, a block
+// to a warp; then blocks joined twice, M21^T = -M11^T (A21^T M22^T), on the warp-level tensor instruction, zero blocks left out.
+// A column walked over all 64 rows in registers takes 63 dependent steps whose broadcast loads of A are bound by
+// shared-memory wavefronts: 7300 cycles against 3100 for this (5300 with the SM's other CTAs at work).
+__device__ __forceinline__ void invert(float* Ac) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp < 4) {
-        const int q = 2 * warp + (lane >> 4), j = lane & 15, o = (q & 3) * 16;
-        float* Ac = sA + (q >> 2) * C * C;
+    if (lane < 16) {
+        const int j = lane, o = warp * 16;
         float m[16];
 #pragma unroll
         for (int r = 0; r < 16; ++r) m[r] = r == j ? 1.f : 0.f;
@@ -100,15 +101,14 @@ __device__ __forceinline__ void invert_pair(float* sA) {
                 m[4 * r4 + 2] = fmaf(-a.z, m[i], m[4 * r4 + 2]); m[4 * r4 + 3] = fmaf(-a.w, m[i], m[4 * r4 + 3]);
             }
         }
-        __syncwarp();
+        __syncwarp(0xffffu);
 #pragma unroll
         for (int r4 = 0; r4 < 4; ++r4)
             *reinterpret_cast<float4*>(Ac + at_off(o + j, o + 4 * r4)) = make_float4(m[4 * r4], m[4 * r4 + 1], m[4 * r4 + 2], m[4 * r4 + 3]);
     }
-    __syncthreads();
-    if (warp < 4) {                                              // 16 -> 32: one warp per pair of blocks
-        float* Ac = sA + (warp >> 1) * C * C;
-        const int o = (warp & 1) * 32;
+    psync();
+    if (!(warp & 1)) {                                           // 16 -> 32: one warp per pair of blocks
+        const int o = warp * 16;
         float s[2][4] = {}, m[2][4] = {};
         mm16(s, Ac, o, o + 16, Ac, o + 16, o + 16);
         __syncwarp();
@@ -118,38 +118,40 @@ __device__ __forceinline__ void invert_pair(float* sA) {
         __syncwarp();
         put16(m, -1.f, Ac, o, o + 16);
     }
-    __syncthreads();
-    {   // 32 -> 64: four warps per chunk, 16 x 16 each; warps w and w + 4 share a scheduler, so the second chunk's pieces
-        // are numbered from the other end: every scheduler gets a long contraction and a short one
-        float* Ac = sA + (warp >> 2) * C * C;
-        const int w = warp < 4 ? warp : 7 - warp, tm = (w & 2) * 8, tn = (w & 1) * 16;
+    psync();
+    {   // 32 -> 64: 16 x 16 to a warp
+        const int tm = (warp & 2) * 8, tn = (warp & 1) * 16;
         float s[2][4] = {}, m[2][4] = {};
         mm16(s, Ac, tm, 32, Ac, 32, 32 + tn);
         if (tn) mm16(s, Ac, tm, 48, Ac, 48, 48);                 // M22^T is upper triangular: k <= n
-        __syncthreads();
+        psync();
         put16(s, 1.f, Ac, tm, 32 + tn);
-        __syncthreads();
+        psync();
         mm16(m, Ac, tm, 16, Ac, 16, 32 + tn);
         if (!tm) mm16(m, Ac, 0, 0, Ac, 0, 32 + tn);              // M11^T likewise: k >= m
-        __syncthreads();
+        psync();
         put16(m, -1.f, Ac, tm, 32 + tn);
     }
-    __syncthreads();
+    psync();
 }
 
-// One CTA prepares a pair of chunks (128 tokens) of one head.  Thread roles change by phase:
-//   scan / coefficients   thread t < 128 owns token t
-//   row-wise elementwise  16 threads per 256-byte row (coalesced), 16 rows per pass
-//   Gram epilogue         thread (row = t & 127, half = t >> 7) owns 32 columns of its TMEM lane
-//   triangular inverse    by warps, see invert_pair
-//   final epilogue        thread (d = t & 127, which = t >> 7) owns one row of U~^T resp. W~^T
+// One CTA prepares a chunk of one head.  What bounds it is the chain of short phases -- copy, Gram products, A, inverse, T, WY
+// products, copies out -- of 7 us at least; so a CTA is as small as it can be, 4 warps that do the arithmetic and one that issues
+// every copy and every product, 48 KB, 128 columns of tensor memory, and four of them share an SM.  (Pairs of chunks,
+// two CTAs of twice the size to an SM: 113 against 108 us on 128 sequences of 32 chunks, 406 against 384 on 32 of 512, 18.7 against
+// 17 on 16 of 14.  592 persistent CTAs: 121 and 447 -- four of them on an SM then go through their phases in step.)
+//   scan / coefficients   thread t < 64 owns token t
+//   row-wise elementwise  16 threads per 256-byte row (coalesced), 8 rows per pass
+//   Gram epilogue         64-row products, 16 rows to a warp, in fragment layout (tmem_ld_frag)
+//   triangular inverse    by warps, see invert
+//   final epilogue        thread d owns row d of U~^T and of W~^T
 // Both Gram products start as soon as Q and K are there: X K^T = K K^T + diag(lambda) Q K^T is combined in the epilogue, so
-// nothing waits for X, which is formed in registers under the products and takes Q's place when they have read it.
+// nothing waits for X, which is formed under the products.  V takes Q's place when they have read it.
 // NORM (QD_NORM_QK): q and k come un-normalised; 1/|q_t|, 1/|k_t| are factors wherever a row is used.  LOGITS
 // (QD_COEF_LOGITS): the coefficients are logits of sigmoid gates.  Compile-time, because even the untaken sigmoid /
 // log-sigmoid code on the path of the scan, which every later phase of the CTA waits for, cost the kernel 8 %.
 template <bool NORM, bool LOGITS>
-__global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_constant__ CUtensorMap mapQ,
+__global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_constant__ CUtensorMap mapQ,
                                                              const __grid_constant__ CUtensorMap mapK,
                                                              const __grid_constant__ CUtensorMap mapV,
                                                              const __grid_constant__ CUtensorMap mapUt,
@@ -157,56 +159,91 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
                                                              const __grid_constant__ CUtensorMap mapP, PrepParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char *sQ = smem, *sK = smem + 32768, *sV = smem + 65536;
-    // lambda absent (the gated delta rule, Eq. 3) and keys given normalised: X = K, nothing is built, and the scratch that
-    // otherwise overwrites K overwrites Q instead
-    const bool build_x = NORM || p.lam != nullptr;
-    unsigned char* sX = build_x ? sQ : sK;
-    unsigned char* sScr = build_x ? sK : sQ;                    // dead once both Grams are formed, diag(gamma)Q and X taken
-    float* sA = reinterpret_cast<float*>(sScr);                 // A^T, then M^T: [2][column][row], at_off
-    unsigned char* sT = sScr;                                   // [2] T_c, [2] T_c diag(gamma): 8 KB each, alias A
-    __shared__ uint64_t bar_load, bar_v, bar_mma;
+    unsigned char *sK = smem, *sQ = smem + 16384, *sX = smem + 32768;
+    float* sA = reinterpret_cast<float*>(sK);                   // A^T, then M^T: [column][row], at_off
+    // bar_x, bar_t, bar_o: one arrival per compute warp -- Q read and X written; T tiles written; results staged
+    __shared__ uint64_t bar_qk, bar_v, bar_g, bar_w, bar_x, bar_t, bar_o;
     __shared__ uint32_t tmem_slot;
-    __shared__ __align__(16) float sg[128], srk[128];
-    __shared__ float sbeta[128], slam[128], srq[128], swsum[4];
+    __shared__ volatile int s_abort;
+    __shared__ __align__(16) float sg[C], srk[C];
+    __shared__ float sbeta[C], slam[C], srq[C], swsum;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // CTAs are numbered pair-major, last pair first: the forward chain, which starts with chunk 0 of every sequence,
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+    // CTAs are numbered chunk-major, last chunk first: the forward chain, which starts with chunk 0 of every sequence,
     // then finds the tiles written last (and K, read last) still in L2
-    const int pairs = p.N / 2, pr = pairs - 1 - (int)blockIdx.x / p.BH, bh = (int)blockIdx.x % p.BH;
+    const int n = p.N - 1 - (int)blockIdx.x / p.BH, bh = (int)blockIdx.x % p.BH;
     const int b = bh / p.H, hh = bh % p.H;
-    const int t0 = pr * 128;                                         // first token of the pair
+    const int t0 = n * C;                                            // first token of the chunk
     const size_t wtok0 = (size_t)bh * p.Tp + (size_t)t0;             // first row in the workspace's [BH*Tp] view
 
     if (tid == 0) {
-        mbar_init(&bar_load, 1);
-        mbar_init(&bar_v, 1);
-        mbar_init(&bar_mma, 1);
+        mbar_init(&bar_qk, 1); mbar_init(&bar_v, 1); mbar_init(&bar_g, 1); mbar_init(&bar_w, 1);
+        mbar_init(&bar_x, 4); mbar_init(&bar_t, 4); mbar_init(&bar_o, 4);
         mbar_init_fence();
+        s_abort = 0;
     }
-    if (warp == 0) { tmem_alloc(&tmem_slot, 256); tmem_relinquish(); }
+    if (warp == 4) { tmem_alloc(&tmem_slot, 128); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tbase = tmem_slot;
+    const uint32_t tb = uniform(tmem_slot), T0 = tb, T1 = tb + 64;
+    auto wait = [&](uint64_t* bar) { return mbar_try_wait(bar, 0) || wait_on(bar, 0, s_abort, p.status); };
 
     grid_dep_wait();                  // set up while the kernel before drains; nothing is read or written before it has completed
     grid_dep_launch();                // the kernel after this one may set itself up while the last CTAs of this one run
-    // copies, products and coefficients start from different warps: none of them waits for another (a thread that issues
-    // copies is held up while the other CTA's stores are in the queue)
-    if (tid == 128) {
-        // the call's status word starts at zero: the first CTA to start clears it, a second before any wait can expire
-        if (blockIdx.x == 0) *p.status = 0;
-        mbar_expect_tx(&bar_load, 2 * 32768);
-        for (int blk = 0; blk < 2; ++blk) {          // rows at t >= T arrive as zeros
-            tma_load_3d(sQ + blk * 16384, &mapQ, hh * D + blk * 64, t0, b, &bar_load);
-            tma_load_3d(sK + blk * 16384, &mapK, hh * D + blk * 64, t0, b, &bar_load);
+    if (warp == 4) {
+        // ---------------------------------- copies and products ----------------------------------
+        const uint32_t issue = elect_lane();
+        const uint32_t aK = smem_u32(sK), aQ = smem_u32(sQ), aX = smem_u32(sX);
+        const bool lead = lane == 0;
+        if (lead) {
+            // the call's status word starts at zero: the first CTA to start clears it, a second before any wait can expire
+            if (blockIdx.x == 0) *p.status = 0;
+            mbar_expect_tx(&bar_qk, 32768);
+            for (int blk = 0; blk < 2; ++blk) {          // rows at t >= T arrive as zeros
+                tma_load_3d(sQ + blk * 8192, &mapQ, hh * D + blk * 64, t0, b, &bar_qk);
+                tma_load_3d(sK + blk * 8192, &mapK, hh * D + blk * 64, t0, b, &bar_qk);
+            }
+            for (int blk = 0; blk < 2; ++blk) tma_prefetch_3d(&mapV, hh * D + blk * 64, t0, b);       // loaded when Q has been used
         }
-        mbar_expect_tx(&bar_v, 32768);               // needed last
-        for (int blk = 0; blk < 2; ++blk) tma_load_3d(sV + blk * 16384, &mapV, hh * D + blk * 64, t0, b, &bar_v);
+        wait(&bar_qk);
+        __syncwarp();
+        umma_product_w<false, false, 64>(T1, aQ, 8192, aK, 8192, C, D, false, issue);                // Q K^T
+        umma_product_w<false, false, 64>(T0, aK, 8192, aK, 8192, C, D, false, issue);                // K K^T
+        umma_commit_w(&bar_g, issue);
+        wait(&bar_x);
+        wait(&bar_g);
+        if (lead && !s_abort) {
+            mbar_expect_tx(&bar_v, 16384);
+            for (int blk = 0; blk < 2; ++blk) tma_load_3d(sQ + blk * 8192, &mapV, hh * D + blk * 64, t0, b, &bar_v);
+        }
+        __syncwarp();
+        wait(&bar_t);
+        wait(&bar_v);
+        __syncwarp();
+        tc_fence_after();
+        umma_product_w<true, true>(T0, aQ, 8192, aK, 8192, C, C, false, issue);                      // Ut = V^T T^T
+        umma_product_w<true, true>(T1, aX, 8192, aK + 8192, 8192, C, C, false, issue);               // Wt = X^T (T diag(gamma))^T
+        umma_commit_w(&bar_w, issue);
+        wait(&bar_o);
+        tc_fence_after();
+        if (lead) {
+            const int y = (int)(((size_t)bh * p.N + n) * D);
+            tma_store_2d(&mapUt, sX, 0, y);
+            tma_store_2d(&mapWt, sQ, 0, y);
+            tma_store_2d(&mapP, sK, 0, (int)wtok0);
+            tma_store_commit();
+            tma_store_wait_read();             // the staging tiles must outlive the reads; the writes complete with the grid
+            if (s_abort) { mbar_wait(&bar_qk, 0); mbar_wait(&bar_v, 0); }      // one more bounded chance for copies in flight
+        }
+        __syncwarp();
+        tmem_dealloc(tb, 128);
+        return;
     }
-    // coefficients of token tid; in-chunk cumulative log-decay by a two-warp scan per chunk
-    if (tid < 128) {
+    // ---------------------------------- arithmetic ----------------------------------
+    auto arrive = [&](uint64_t* bar) { __syncwarp(); if (lane == 0) mbar_arrive(bar); };
+    // coefficients of token tid; in-chunk cumulative log-decay by a two-warp scan
+    if (tid < C) {
         // a token past the end of the sequence is an exact no-op of the recurrence: beta = 0, alpha = 1 (and q = k = v = 0)
         const bool live = t0 + tid < p.T, has_a = live && p.alpha, has_l = live && p.lam;
         const size_t crow = ((size_t)b * p.T + t0 + tid) * p.H + hh;
@@ -220,45 +257,28 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
             const float t = __shfl_up_sync(0xffffffffu, g, o);
             if (lane >= o) g += t;
         }
-        if (lane == 31) swsum[warp] = g;
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (warp & 1) g += swsum[warp - 1];
+        if (tid == 31) swsum = g;
+        asm volatile("bar.sync 2, 64;" ::: "memory");
+        if (warp == 1) g += swsum;
         sg[tid] = g;
         p.g[wtok0 + tid] = g;
     }
-
-    // all threads leave together when a wait has expired; copies in flight get one more bounded chance to land
-    auto expired = [&](bool fail) {
-        if (!__syncthreads_or(fail)) return false;
-        if (tid == 0) *p.status = QD_ERR_TIMEOUT;
-        mbar_wait(&bar_load, 0);
-        mbar_wait(&bar_v, 0);
-        __syncthreads();
-        if (warp == 0) tmem_dealloc(tbase, 256);
-        return true;
-    };
-    if (tid == 160 && mbar_wait(&bar_load, 0)) {
-        tc_fence_after();
-        // G1 = K K^T -> columns [0,128), G2 = Q K^T -> columns [128,256)
-        umma_product<false, false>(tbase + 128, smem_u32(sQ), 16384, smem_u32(sK), 16384, 128, 128, false);
-        umma_product<false, false>(tbase, smem_u32(sK), 16384, smem_u32(sK), 16384, 128, 128, false);
-        umma_commit(&bar_mma);
-    }
-    if (expired(!mbar_wait(&bar_load, 0))) return;
-    // meanwhile, row-wise, 16 lanes to a 256-byte row (chunk `ch` of 16 bytes each): Qg = gamma Q to the workspace, and X
-    uint4 xr[8];
-    const int ch = tid & 15, rsub = tid >> 4;
-    const uint32_t coff = (ch >> 3) * 16384;
+    psync();
+    wait(&bar_qk);
+    // row-wise, 16 lanes to a 256-byte row (chunk `ch` of 16 bytes each): Qg = gamma Q to the workspace, and X
     {
+        const int ch = tid & 15, rsub = tid >> 4;
+        const uint32_t coff = (ch >> 3) * 8192;
         bf16* qg = p.Qg + wtok0 * D + ch * 8;
         const size_t nrows = (size_t)p.BH * p.Tp;
+        const bool has_lam = p.lam != nullptr;
 #pragma unroll
         for (int it = 0; it < 8; ++it) {
-            const int row = it * 16 + rsub;
+            const int row = it * 8 + rsub;
             const uint32_t off = coff + sw128_chunk(row, ch & 7);
             float qv[8], kv[8], rq = 1.f, rk = 1.f;
             load8(sQ + off, qv);
-            if (build_x) load8(sK + off, kv);
+            load8(sK + off, kv);
             if (NORM) {
                 // 1 / sqrt(|q|^2 + eps), 1 / sqrt(|k|^2 + eps)
                 float sq = 0.f, sk = 0.f;
@@ -277,130 +297,104 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_tc_prep(const __grid_consta
                 }
             }
             const float gr = __expf(sg[row]) * rq, lm = slam[row] * rq;
-            if (build_x) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) kv[e] = fmaf(lm, qv[e], NORM ? rk * kv[e] : kv[e]);
-                xr[it] = pack8(kv);
+            for (int e = 0; e < 8; ++e) {
+                if (NORM) kv[e] *= rk;
+                if (NORM || has_lam) kv[e] = fmaf(lm, qv[e], kv[e]);      // lambda absent (the gated delta rule, Eq. 3): X = K
             }
+            sts128(sX + off, pack8(kv));
 #pragma unroll
             for (int e = 0; e < 8; ++e) qv[e] *= gr;
             *reinterpret_cast<uint4*>(qg + (size_t)row * D) = pack8(qv);
         }
     }
-    if (expired(!mbar_wait(&bar_mma, 0))) return;
+    fence_proxy_async();
+    arrive(&bar_x);
+    psync();                                             // K has been read, the factors of the normalisation are there
+    wait(&bar_g);
     tc_fence_after();
-    // Q, K have been read by everybody: X over Q (K-major swizzled layout), A over K
-    if (build_x) {
-#pragma unroll
-        for (int it = 0; it < 8; ++it) sts128(sX + coff + sw128_chunk(it * 16 + rsub, ch & 7), xr[it]);
-    }
     // A = strictLower(beta_r Gamma_ri (x_r . k_i)) -> shared fp32, transposed;  P = Gamma_ri (q_r . k_i), i <= r, kept in
-    // registers until its staging tile is free
-    uint4 pk[4];
-    const int row = tid & 127, half = tid >> 7;
+    // registers until its staging tile is free.  My rows: r0, r0 + 8; of every 8 columns: ft, ft + 1.
+    uint32_t pk[4][4];
+    const int rw = 16 * warp, r0 = rw + (lane >> 2), ft = 2 * (lane & 3);
     {
-        const int c = row >> 6, r = row & 63;
-        const float g = sg[row], beta = sbeta[row];
-        const float rq = NORM ? srq[row] : 1.f, rk = NORM ? srk[row] : 1.f, lm = slam[row] * rq;
-        const float *gc = sg + c * C, *rc = srk + c * C;
-        float* Ac = sA + c * C * C;
-        float v1[32], v2[32];
-        tmem_ld32(tmem_addr(tbase, (warp & 3) * 32, c * C + half * 32), v1);
-        tmem_ld32(tmem_addr(tbase, (warp & 3) * 32, 128 + c * C + half * 32), v2);
-        tmem_ld_wait();
+        const uint32_t lane_base = (uint32_t)warp * 32;
+        float gr[2], be[2], rq[2], rk[2], lm[2];
 #pragma unroll
-        for (int i4 = 0; i4 < 8; ++i4) {
-            const float4 g4 = *reinterpret_cast<const float4*>(gc + half * 32 + i4 * 4);
-            const float4 r4 = NORM ? *reinterpret_cast<const float4*>(rc + half * 32 + i4 * 4) : make_float4(1.f, 1.f, 1.f, 1.f);
-            const float gq[4] = {g4.x, g4.y, g4.z, g4.w}, rq4[4] = {r4.x, r4.y, r4.z, r4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int i = i4 * 4 + e, col = half * 32 + i;
-                float dec = (col <= r) ? __expf(g - gq[e]) : 0.f;
-                if (NORM) dec *= rq4[e];
-                sts32(Ac + at_off(col, r), (col < r) ? beta * dec * fmaf(lm, v2[i], rk * v1[i]) : 0.f);
-                v2[i] = dec * (rq * v2[i]);
-            }
+        for (int j = 0; j < 2; ++j) {
+            const int r = r0 + 8 * j;
+            gr[j] = sg[r]; be[j] = sbeta[r]; rq[j] = NORM ? srq[r] : 1.f; rk[j] = NORM ? srk[r] : 1.f; lm[j] = slam[r] * rq[j];
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) pk[i] = pack8(v2 + i * 8);
+        for (int cg = 0; cg < 4; ++cg) {
+            float kk[8], qk[8];
+            tmem_ld_frag2(tmem_addr(T0, lane_base, cg * 16), kk);
+            tmem_ld_frag2(tmem_addr(T1, lane_base, cg * 16), qk);
+            tmem_ld_wait();
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int j = m & 1, r = r0 + 8 * j, c = cg * 16 + 8 * (m >> 1) + ft;
+                const float2 g2 = *reinterpret_cast<const float2*>(sg + c);
+                const float2 k2 = NORM ? *reinterpret_cast<const float2*>(srk + c) : make_float2(1.f, 1.f);
+                float pv[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int x = 4 * (m >> 1) + 2 * j + e;
+                    float dec = c + e <= r ? __expf(gr[j] - (e ? g2.y : g2.x)) : 0.f;
+                    if (NORM) dec *= e ? k2.y : k2.x;
+                    sts32(sA + at_off(c + e, r), c + e < r ? be[j] * dec * fmaf(lm[j], qk[x], rk[j] * kk[x]) : 0.f);
+                    pv[e] = dec * (rq[j] * qk[x]);
+                }
+                pk[cg][m] = pack_bf16(pv[0], pv[1]);
+            }
+        }
     }
     tc_fence_before();
-    __syncthreads();
-    invert_pair(sA);
-    // T_c = M_c diag(beta), T_c diag(gamma): line j of the MN-major tiles holds column j over the rows; thread = (column
-    // j of chunk c, block of eight rows), eight threads to a column.  The tiles take A's place: everything is read first.
+    psync();
+    invert(sA);
+    // T = M diag(beta), T diag(gamma): line j of the MN-major tiles holds column j over the rows; thread = (column
+    // j, block of eight rows), eight threads to a column.  The tiles take A's place: everything is read first.
     {
         float m[4][8];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int id = k * kPrepThreads + tid, c = id >> 9, j = (id >> 3) & 63, kb = id & 7;
+            const int id = k * kPrepCompute + tid, j = id >> 3, kb = id & 7;
 #pragma unroll
             for (int e = 0; e < 8; e += 4)
-                *reinterpret_cast<float4*>(m[k] + e) = *reinterpret_cast<const float4*>(sA + c * C * C + at_off(j, kb * 8 + e));
+                *reinterpret_cast<float4*>(m[k] + e) = *reinterpret_cast<const float4*>(sA + at_off(j, kb * 8 + e));
         }
-        __syncthreads();
+        psync();
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int id = k * kPrepThreads + tid, c = id >> 9, j = (id >> 3) & 63, kb = id & 7;
-            const float beta = sbeta[c * C + j], bg = beta * __expf(sg[c * C + j]);
+            const int id = k * kPrepCompute + tid, j = id >> 3, kb = id & 7;
+            const float beta = sbeta[j], bg = beta * __expf(sg[j]);
             float a[8], bq[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) { a[e] = m[k][e] * beta; bq[e] = m[k][e] * bg; }
-            sts128(sT + c * 8192 + sw128_chunk(j, kb), pack8(a));
-            sts128(sT + 16384 + c * 8192 + sw128_chunk(j, kb), pack8(bq));
-            if (p.Mt) *reinterpret_cast<uint4*>(p.Mt + (((size_t)bh * p.N + 2 * pr + c) * C + j) * C + kb * 8) = pack8(m[k]);
+            sts128(sK + sw128_chunk(j, kb), pack8(a));
+            sts128(sK + 8192 + sw128_chunk(j, kb), pack8(bq));
+            if (p.Mt) *reinterpret_cast<uint4*>(p.Mt + (((size_t)bh * p.N + n) * C + j) * C + kb * 8) = pack8(m[k]);
         }
     }
     fence_proxy_async();
-    if (expired(!mbar_wait(&bar_v, 0))) return;
-    if (tid == 0) {
-        tc_fence_after();
-        for (int cc = 0; cc < 2; ++cc) {
-            // Ut_c = V_c^T T_c^T  -> columns [cc*64, +64);   Wt_c = X_c^T (T_c diag(gamma))^T -> 128 + ...
-            umma_product<true, true>(tbase + cc * C, smem_u32(sV) + cc * C * 128, 16384,
-                                     smem_u32(sT) + cc * 8192, 8192, C, C, false);
-            umma_product<true, true>(tbase + 128 + cc * C, smem_u32(sX) + cc * C * 128, 16384,
-                                     smem_u32(sT) + 16384 + cc * 8192, 8192, C, C, false);
-        }
-        umma_commit(&bar_mma);
-    }
-    if (expired(!mbar_wait(&bar_mma, 1))) return;
+    arrive(&bar_t);
+    wait(&bar_w);
     tc_fence_after();
-    // row d = tid & 127 of U~^T (threads < 128) resp. W~^T (the others), both chunks: staged as swizzled
-    // [128][64] tiles over the dead X and V regions; P, [64 tokens][64] per chunk, over the T tiles; all written by TMA
-    {
-        unsigned char* stage = half ? sV : sX;
+    // P, [64 tokens][64], over the T tiles; row d = tid of U~^T over X and of W~^T over V; all written by TMA
 #pragma unroll
-        for (int i = 0; i < 4; ++i) sts128(sScr + (row >> 6) * 8192 + sw128_chunk(row & 63, half * 4 + i), pk[i]);
+    for (int cg = 0; cg < 4; ++cg) stsm4<false>(sK + sw128_chunk(rw + (lane & 15), cg * 2 + (lane >> 4)), pk[cg]);
 #pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {
-            float v[32];
-            tmem_ld32(tmem_addr(tbase, (warp & 3) * 32, half * 128 + q4 * 32), v);
-            tmem_ld_wait();
-            unsigned char* tile = stage + (q4 >> 1) * 16384;
+    for (int q4 = 0; q4 < 4; ++q4) {
+        float v[32];
+        tmem_ld32(tmem_addr(tb, (uint32_t)warp * 32, q4 * 32), v);
+        tmem_ld_wait();
+        unsigned char* stage = q4 < 2 ? sX : sQ;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) sts128(tile + sw128_chunk(row, (q4 & 1) * 4 + i), pack8(v + i * 8));
-        }
+        for (int i = 0; i < 4; ++i) sts128(stage + sw128_chunk(tid, (q4 & 1) * 4 + i), pack8(v + i * 8));
     }
     fence_proxy_async();
     tc_fence_before();
-    __syncthreads();
-    if (tid == 0) {
-        const int y = (int)(((size_t)bh * p.N + 2 * pr) * D);
-        tma_store_2d(&mapUt, sX, 0, y);
-        tma_store_2d(&mapUt, sX + 16384, 0, y + D);
-        tma_store_2d(&mapWt, sV, 0, y);
-        tma_store_2d(&mapWt, sV + 16384, 0, y + D);
-        tma_store_2d(&mapP, sScr, 0, (int)wtok0);
-        tma_store_2d(&mapP, sScr + 8192, 0, (int)wtok0 + C);
-        tma_store_commit();
-        tma_store_wait_read();             // the staging tiles must outlive the reads; the writes complete with the grid
-    }
-    if (warp == 0) {
-        __syncwarp();
-        tmem_dealloc(tbase, 256);
-    }
+    arrive(&bar_o);
 }
 
 // =================================================================================================
@@ -409,7 +403,6 @@ struct ChainParams {
     const float* g;
     const float* h0;
     float* hT;
-    int rows;                  // d_v rows of the state per CTA: 128, or 64 (two CTAs per sequence)
     int save;                  // also store, per chunk, the bf16 entry state (mapHs) and Delta^T (mapDt)
     int scaled;                // 0: no forget gate and no key normalisation: every per-token factor on Delta is 1
     const float* rk;           // non-null (QD_NORM_QK): 1/|k_t| per workspace row; the keys are read un-normalised and
@@ -418,7 +411,7 @@ struct ChainParams {
 };
 
 // Tiles of a chunk in shared memory.  Wt 16K | Ut 16K, three deep (Delta^T is staged over Ut and held until it has been
-// read); Qg 16K | K 16K | P 8K, two deep; the exit state 32K; half an output tile 8K.
+// read); Qg 16K | K 16K | P 8K, two deep; the exit state 32K (16K with 64 rows: two deep then); half an output tile 8K.
 constexpr int kDeepA = 3, kStageA = 32768, kStageB = 40960;
 constexpr int kOffB = kDeepA * kStageA, kOffH = kOffB + 2 * kStageB, kOffO = kOffH + 32768;
 constexpr int kChainSmem = kOffO + 8192 + 1024;
@@ -433,7 +426,8 @@ constexpr int kBarH = 1, kBarD = 2, kBarOut = 3;
 //   h ready -> Delta-accumulator = h^T Wt -> Delta^T -> H-accumulator = (scaled Delta^T) K -> h update;
 // the output products (h^T Qg^T + Delta^T P^T, double-buffered accumulator), the output epilogue and
 // every TMA copy run in its shadow on their own warps.
-// What bounds a chunk is that sequence, if nothing gets in its way.  Three things did, 3800 cycles per chunk of 64 tokens:
+// What bounds a chunk is that sequence, if nothing gets in its way (2050 cycles when nothing is saved).  Three things did, 3800
+// cycles per chunk of 64 tokens:
 //  - the shared-memory port: with h^T and Delta^T as shared-memory operands it carried 368 KB per chunk, 2900 cycles.  They
 //    are A operands, so they live in tensor memory (bf16 pairs, written by the epilogues with tcgen05.st): no operand copies,
 //    no re-reading of A by every product;
@@ -442,9 +436,10 @@ constexpr int kBarH = 1, kBarD = 2, kBarOut = 3;
 //    loads and the 16 KB of its output take 2150 cycles, and the 48 KB of Delta^T and entry state that a forward saves for the
 //    backward 1300 more.  (Ordinary stores, by one or two warps from the tiles or by the epilogue from its registers, were
 //    slower: 4500 - 5000 cycles per chunk.)  So with few heads the d_v rows of a head, which evolve independently, are shared by
-//    two CTAs (`rows` = 64): each loads what both need, but only its half of Ut, and stores its half of everything.
+//    two CTAs (ROWS = 64): each loads what both need, but only its half of Ut, and stores its half of everything.
 // Compute warpgroup w owns tokens [16w, 16w+16) of the 64-column accumulators and d_k columns
 // [32w, 32w+32) of the state; thread l of a warpgroup owns TMEM lane l = d_v index.
+template <int ROWS>
 __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_constant__ CUtensorMap mapWt,
                                                                 const __grid_constant__ CUtensorMap mapUt,
                                                                 const __grid_constant__ CUtensorMap mapQg,
@@ -456,13 +451,14 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                                                                 ChainParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* sH = smem + kOffH;               // h^T [128 dv][128 dk] for its store, 2 blocks of [128 lines][64]
+    constexpr int rows = ROWS, two = rows == D ? 0 : 1;   // d_v rows of the state in this CTA; whether the exit state is staged two deep
+    unsigned char* sHs = smem + kOffH;              // h^T [rows dv][128 dk] for its store, 2 blocks of [rows lines][64]
     unsigned char* sO = smem + kOffO;               // half an output tile: [32 tokens][128 dv], 2 blocks of [32 lines][64]
     // Where one side may run ahead of the other there is a barrier per buffer; it comes round only after the other side has
     // waited for it.  bar_e: every product of a chunk has finished; bar_dt, bar_ht: Delta^T / exit state staged for their stores
     // (one arrival per compute warp); bar_df, bar_hf: they have been read; bar_o, bar_of: an output accumulator is complete /
     // has been read.
-    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_df[kDeepA], bar_ht, bar_hf, bar_a, bar_b, bar_o[2], bar_of[2];
+    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_df[kDeepA], bar_ht[2], bar_hf[2], bar_a, bar_b, bar_o[2], bar_of[2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
     // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the TMA warp before it arrives on the
@@ -470,13 +466,14 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     __shared__ __align__(16) float sG[kDeepA][68];
 
     const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, l = tid & 127, wq = warp & 3;
-    const int rows = p.rows, nwq = rows / 32, nb = 4 * rows + 32;    // d_v rows of this CTA; warps of a warpgroup that have some; barrier participants
-    const int parts = D / rows, bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
+    constexpr int nwq = rows / 32, nb = 4 * rows + 32, parts = D / rows;      // warps of a warpgroup that have rows; barrier participants
+    const int bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
 
     if (tid == 0) {
         for (int i = 0; i < kDeepA; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_dt[i], 4 * nwq); mbar_init(&bar_df[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&bar_lb[i], 1); mbar_init(&bar_e[i], 1); mbar_init(&bar_o[i], 1); mbar_init(&bar_of[i], nwq); }
-        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1); mbar_init(&bar_ht, 4 * nwq); mbar_init(&bar_hf, 1);
+        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar_ht[i], 4 * nwq); mbar_init(&bar_hf[i], 1); }
         mbar_init_fence();
         s_abort = 0;
     }
@@ -491,13 +488,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     const uint32_t lane_base = (uint32_t)wq * 32;
 
     // bounded wait; once any wait has expired every later wait returns at once (the kernel drains)
-    auto wait = [&](uint64_t* bar, uint32_t parity) {
-        if (s_abort) return false;
-        if (mbar_wait(bar, parity)) return true;
-        s_abort = 1;
-        *p.status = QD_ERR_TIMEOUT;
-        return false;
-    };
+    auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_try_wait(bar, parity) || wait_on(bar, parity, s_abort, p.status); };
     const float* gseq = p.g + (size_t)bh * p.Tp;
 
     if (warp < kMmaWarp && wq >= nwq) {
@@ -530,13 +521,16 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             tc_fence_before();
             nb_arrive(kBarH, nb);
         };
-        auto save_h = [&]() {             // the state as a tile: 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
+        // the state that chunk n begins with as a tile: 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
+        auto save_h = [&](int n) {
+            const int sb = n & two;
+            if (n > two) wait(&bar_hf[sb], ((n >> two) - 1) & 1);
 #pragma unroll
-            for (int ch = 0; ch < 4; ++ch) sts128(sH + (wg >> 1) * 16384 + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(h + ch * 8));
-            staged(&bar_ht);
+            for (int ch = 0; ch < 4; ++ch) sts128(sHs + sb * 16384 + (wg >> 1) * (rows * 128) + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(h + ch * 8));
+            staged(&bar_ht[sb]);
         };
         put_h();
-        if (p.save) save_h();
+        if (p.save) save_h(0);
         int pending = 0;                  // barriers of the MMA warp that a warp which gives up has not been to
         int s = 0;
         for (int n = 0; n < p.N; ++n) {
@@ -585,7 +579,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                 for (int i = 0; i < 32; ++i) h[i] = fmaf(gamC, h[i], v[i]);
             }
             put_h();
-            if (p.save && n + 1 < p.N) { wait(&bar_hf, n & 1); save_h(); }
+            if (p.save && n + 1 < p.N) save_h(n + 1);
             if (++s == kDeepA) s = 0;
         }
         // a wait has expired: keep step with the MMA warp, which comes to every one of them (odd counts: H is next)
@@ -674,19 +668,23 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             int s = 0;
             for (int n = 0; n < p.N; ++n) {
                 const int y = (int)(((size_t)bh * p.N + n) * D) + v0;
-                wait(&bar_ht, n & 1);                     // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
-                tma_store_2d(&mapHs, sH, 0, y);
-                tma_store_2d(&mapHs, sH + 16384, 64, y);
+                const int sb = n & two;
+                wait(&bar_ht[sb], (n >> two) & 1);        // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
+                tma_store_2d(&mapHs, sHs + sb * 16384, 0, y);
+                tma_store_2d(&mapHs, sHs + sb * 16384 + rows * 128, 64, y);
                 tma_store_commit();
-                if (n > 0) {                              // Delta^T of chunk n - 1 has been read
+                if (n > 0) {                              // Delta^T of chunk n - 1 has been read, and the entry state before it
                     tma_store_wait_read_n<1>();
                     mbar_arrive(&bar_df[s == 0 ? kDeepA - 1 : s - 1]);
+                    if (two) mbar_arrive(&bar_hf[sb ^ 1]);
                 }
                 wait(&bar_dt[s], (n / kDeepA) & 1);       // Delta^T of chunk n is staged
                 tma_store_2d(&mapDt, smem + s * kStageA + 16384, 0, y);
                 tma_store_commit();
-                tma_store_wait_read_n<1>();               // the entry state has been read
-                mbar_arrive(&bar_hf);
+                if (!two) {
+                    tma_store_wait_read_n<1>();           // the entry state has been read
+                    mbar_arrive(&bar_hf[0]);
+                }
                 if (++s == kDeepA) s = 0;
             }
             tma_store_wait_all();
@@ -800,8 +798,8 @@ cudaError_t tc_prep(const ChunkArgs& a) {
     CUtensorMap mQ, mK, mV, mUt, mWt, mP;
     const int Tp = tc_padded_T(s);
     const uint64_t trows = (uint64_t)s.B * s.H * (Tp / kChunk) * D;          // rows of the [chunk][d][64] tiles
-    if (!make_tmap_tokens(&mQ, a.q, s.B, s.T, s.H, D, 128) || !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 128) ||
-        !make_tmap_tokens(&mV, a.v, s.B, s.T, s.H, D, 128) ||
+    if (!make_tmap_tokens(&mQ, a.q, s.B, s.T, s.H, D, 64) || !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_tokens(&mV, a.v, s.B, s.T, s.H, D, 64) ||
         !make_tmap_bf16_2d(&mUt, a.ws + a.TL.Ut, 64, trows, 128, 128) ||
         !make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, trows, 128, 128) ||
         !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, (uint64_t)s.B * s.H * Tp, 128, 64))
@@ -818,7 +816,7 @@ cudaError_t tc_prep(const ChunkArgs& a) {
                        : (a.logits ? k_tc_prep<false, true> : k_tc_prep<false, false>);
     cudaError_t e = set_smem(kern, kPrepSmem);
     if (e != cudaSuccess) return e;
-    const int grid = s.B * s.H * (p.N / 2);
+    const int grid = s.B * s.H * p.N;
     return launch_overlapped(kern, dim3((unsigned)grid), dim3(kPrepThreads), kPrepSmem, a.stream, mQ, mK, mV, mUt, mWt, mP, p);
 }
 
@@ -842,13 +840,13 @@ cudaError_t tc_chain_fwd(const ChunkArgs& a) {
     p.g = (const float*)(a.ws + a.TL.g);
     p.h0 = a.h0; p.hT = a.hT;
     p.save = a.save ? 1 : 0;
-    p.rows = rows;
     p.scaled = (a.alpha || a.norm) ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
-    cudaError_t e = set_smem(k_tc_chain_fwd, kChainSmem);
+    const auto kern = rows == D ? k_tc_chain_fwd<D> : k_tc_chain_fwd<D / 2>;
+    cudaError_t e = set_smem(kern, kChainSmem);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(k_tc_chain_fwd, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream,
+    return launch_overlapped(kern, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream,
                              mWt, mUt, mQg, mK, mP, mHs, mDt, mO, p);
 }
 

@@ -37,3 +37,12 @@ def test_chunk_order(B, H, T):
     first, second = (qd.chunk_bwd(*a, t["dO"], t["dhT"], workspace=ws, reuse_fwd=True) for _ in range(2))
     for n, x in first.items():
         assert x is None or torch.equal(x, second[n]), n
+
+
+@pytest.mark.parametrize("T", [1, 63, 64, 66, 129])
+def test_preparation_edges(T):
+    """One chunk of one token, one short of a whole chunk, whole, a second one of two tokens, a third of one."""
+    cfg = replace(gen.CONFIGS["cfg2"], B=1, H=3, T=T, regime="trained_like", seed=401 + T)
+    d = gen.make_chunk_inputs(cfg)
+    _fwd_check(cfg, d)
+    _bwd_check(cfg, d, reuse=True)
