@@ -46,13 +46,14 @@ struct Planes {
         }
         return v;
     }
-    // a bf16 tile on its way from global memory (rows `stride` elements apart, rows >= live read as zeros), asynchronously
+    // a bf16 tile on its way from global memory (rows `stride` elements apart, rows >= live read as zeros), asynchronously, by TH
+    // threads, of which this is number `me`
     template <int TH>
-    __device__ __forceinline__ void fetch(const __nv_bfloat16* src, size_t stride, int live) const {
+    __device__ __forceinline__ void fetch(const __nv_bfloat16* src, size_t stride, int live, int me = threadIdx.x) const {
         static_assert(NP == 1, "stored in bf16");
         constexpr int kChunks = W / 8, kTotal = ROWS * kChunks;
 #pragma unroll
-        for (int id = threadIdx.x; id < kTotal; id += TH) {
+        for (int id = me; id < kTotal; id += TH) {
             const int row = id / kChunks, c = id % kChunks * 8;
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sm100::smem_u32(p + row * LD + c)),
                          "l"(src + (row < live ? (size_t)row * stride : 0) + c), "r"(row < live ? 16 : 0) : "memory");

@@ -132,8 +132,10 @@ __global__ void __launch_bounds__(NT, PrepPlanes<DK, DV>::kCtas) k_prep(Ptrs p) 
 // products and DK/4 x 16 of the state, which it keeps in fp32 in its registers (planes of it are what the others read).  A
 // chunk is two phases and two barriers; the tiles of one phase arrive while the other is worked on, those of the first two
 // phases ahead.  Slices of 32 columns and d_k = 64 let two CTAs share an SM.  B4 T1024 H16 d_k = d_v = 64: 73 and 85 us with
-// tf32 halves, 45 and 54 so (3 us a chunk, of which the tensor unit works a quarter: the rest is the latency of two dependent
-// products and two barriers).
+// tf32 halves, 45 and 54 with everybody loading, 42 and 49 so (2.5 us a chunk, of which the tensor unit works a third: the rest is
+// the latency of two dependent products and two barriers).  LOADERS: the copies have warps of their own, while a CTA has
+// an SM to itself; beyond that two CTAs share one, whose registers the extra warps would not leave room for (128 sequences of 1024
+// tokens, 256 CTAs: forward and backward 435 us without, 457 with).
 template <int DK, int DS>
 struct ChainPlanes {
     typedef Planes<C, DK, 1> TA;
@@ -145,10 +147,8 @@ struct ChainPlanes {
     static constexpr int kThreads = 8 * DS, kFwd = 2 * TA2::kBytes + TA::kBytes + TP::kBytes + TS::kBytes + 2 * TD::kBytes,
                          kBwd = 2 * (TA::kBytes + TP::kBytes + TO::kBytes) + 2 * TA::kBytes + TS::kBytes + 2 * TD::kBytes;
 };
-template <int N> __device__ __forceinline__ void fetch_wait_but() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int DK, int DS>
-__global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
+template <int DK, int DS, bool LOADERS>
+__global__ void __launch_bounds__(8 * DS + (LOADERS ? kLoaders : 0)) k_chain_fwd(Ptrs p, int DV) {
     extern __shared__ __align__(16) unsigned char smb[];
     typedef ChainPlanes<DK, DS> L;
     typedef __nv_bfloat16 IO;
@@ -163,16 +163,19 @@ __global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
     const int tid = threadIdx.x, warp = tid >> 5, g = (tid & 31) >> 2, t = tid & 3;
     const int wm = (warp & 4 ? 3 - (warp & 3) : warp & 3) * 16, wn = (warp >> 2) * 16, si = (warp & 3) * 16 * MU;
     const size_t nrows = (size_t)p.B * H * p.Tp, row0 = (size_t)b * p.T * H + hh, wrow0 = (size_t)bh * p.Tp;
+    constexpr int NL = LOADERS ? kLoaders : TH;
+    const int me = LOADERS ? tid - TH : tid;               // who loads: extra warps, or everybody; me < 0: not this one
+    const bool loads = !LOADERS || tid >= TH, works = !LOADERS || tid < TH;
     sm100::grid_dep_wait();            // launched while the kernel before it drains
     sm100::grid_dep_launch();
     auto fetch1 = [&](int n) {         // W<- and Q, read in the first phase of chunk n
         const typename L::TA w(smb + (n & 1) * L::TA2::kBytes), q(smb + (n & 1) * L::TA2::kBytes + L::TA::kBytes);
-        w.template fetch<TH>((const IO*)p.W + (wrow0 + (size_t)n * C) * DK, DK, C);
-        q.template fetch<TH>((const IO*)p.q + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C));
+        w.template fetch<NL>((const IO*)p.W + (wrow0 + (size_t)n * C) * DK, DK, C, me);
+        q.template fetch<NL>((const IO*)p.q + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C), me);
     };
     auto fetch2 = [&](int n) {         // K and P, read in the second
-        mK.template fetch<TH>((const IO*)p.k + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C));
-        mP.template fetch<TH>((const IO*)p.P + (wrow0 + (size_t)n * C) * C, C, C);
+        mK.template fetch<NL>((const IO*)p.k + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C), me);
+        mP.template fetch<NL>((const IO*)p.P + (wrow0 + (size_t)n * C) * C, C, C, me);
     };
     uint32_t u[2][2];                  // U~ at this thread's elements
     auto fetch_u = [&](int n) {
@@ -183,31 +186,39 @@ __global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
                 u[h][j] = *reinterpret_cast<const uint32_t*>((const IO*)p.U + (wrow0 + (size_t)n * C + wm + 8 * h + g) * DV + j0 + wn + 8 * j + 2 * t);
     };
     ChainCoef cf;
-    fetch1(0);
+    if (loads) {
+        fetch1(0);
+        cf.get(p, wrow0, nrows, me);
+    }
     fetch_commit();
-    cf.get(p, wrow0, nrows);
-    fetch_u(0);
+    if (works) fetch_u(0);
     float hst[MU][2][4];
     zero(hst);
     auto state_at = [&](float* base, int i, int j) { return reinterpret_cast<float2*>(base + (size_t)i * DV + j0 + j); };
-    if (p.h0) each(hst, si, wn, [&](int i, int j, float& x, float& y) {
+    if (p.h0 && works) each(hst, si, wn, [&](int i, int j, float& x, float& y) {
         const float2 v = *state_at(const_cast<float*>(p.h0) + (size_t)bh * DK * DV, i, j);
         x = v.x; y = v.y;
     });
-    each(hst, si, wn, [&](int i, int j, float x, float y) {
+    if (works) each(hst, si, wn, [&](int i, int j, float x, float y) {
         mS.st2(i, j, x, y);
         if (p.save) *state_at(p.hs + (size_t)bh * p.N * DK * DV, i, j) = make_float2(x, y);
     });
-    cf.put(sgq[0], sgk[0], sgC);
+    if (loads) cf.put(sgq[0], sgk[0], sgC, me);
     for (int n = 0; n < p.N; ++n) {
         const int bf = n & 1, live = min(C, p.T - n * C);
         const bool more = n + 1 < p.N;
         fetch_wait();
         __syncthreads();
-        fetch2(n);
+        if (loads) fetch2(n);
         fetch_commit();
-        if (more) { fetch1(n + 1); cf.get(p, wrow0 + (size_t)(n + 1) * C, nrows); }
+        if (more && loads) { fetch1(n + 1); cf.get(p, wrow0 + (size_t)(n + 1) * C, nrows, me); }
         fetch_commit();
+        if (LOADERS && loads) {
+            fetch_wait_but<1>();
+            __syncthreads();
+            if (more) cf.put(sgq[bf ^ 1], sgk[bf ^ 1], sgC + (bf ^ 1), me);
+            continue;
+        }
         // Delta = U~ - W<- h, and Q h, the inter-chunk part of the output
         float a[2][2][4], o[1][2][4];
         zero(a); zero(o);
@@ -249,13 +260,13 @@ __global__ void __launch_bounds__(8 * DS) k_chain_fwd(Ptrs p, int DV) {
                 if (r < live) st2((IO*)p.o + (row0 + (size_t)(n * C + r) * H) * DV + j0 + wn + 8 * j + 2 * t,
                                   fmaf(f, a[1][j][2 * h], o[0][j][2 * h]), fmaf(f, a[1][j][2 * h + 1], o[0][j][2 * h + 1]));
             }
-        if (more) cf.put(sgq[bf ^ 1], sgk[bf ^ 1], sgC + (bf ^ 1));
+        if (!LOADERS && more) cf.put(sgq[bf ^ 1], sgk[bf ^ 1], sgC + (bf ^ 1));
     }
-    if (p.hT) each(hst, si, wn, [&](int i, int j, float x, float y) { *state_at(p.hT + (size_t)bh * DK * DV, i, j) = make_float2(x, y); });
+    if (p.hT && works) each(hst, si, wn, [&](int i, int j, float x, float y) { *state_at(p.hT + (size_t)bh * DK * DV, i, j) = make_float2(x, y); });
 }
 
-template <int DK, int DS>
-__global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
+template <int DK, int DS, bool LOADERS>
+__global__ void __launch_bounds__(8 * DS + (LOADERS ? kLoaders : 0)) k_chain_bwd(Ptrs p, int DV) {
     extern __shared__ __align__(16) unsigned char smb[];
     typedef ChainPlanes<DK, DS> L;
     typedef __nv_bfloat16 IO;
@@ -268,6 +279,9 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
     const int tid = threadIdx.x, warp = tid >> 5, g = (tid & 31) >> 2, t = tid & 3;
     const int wm = (warp & 4 ? 3 - (warp & 3) : warp & 3) * 16, wn = (warp >> 2) * 16, si = (warp & 3) * 16 * MU;
     const size_t nrows = (size_t)p.B * H * p.Tp, BHN = (size_t)p.B * H * p.N, row0 = (size_t)b * p.T * H + hh, wrow0 = (size_t)bh * p.Tp;
+    constexpr int NL = LOADERS ? kLoaders : TH;
+    const int me = LOADERS ? tid - TH : tid;               // who loads: extra warps, or everybody; me < 0: not this one
+    const bool loads = !LOADERS || tid >= TH, works = !LOADERS || tid < TH;
     sm100::grid_dep_wait();            // launched while the kernel before it drains
     sm100::grid_dep_launch();
     auto fetch1 = [&](int n) {         // K, P and dO, read in the first phase of chunk n
@@ -276,13 +290,13 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
         const typename L::TP pm(s + L::TA::kBytes);
         const typename L::TO o(s + L::TA::kBytes + L::TP::kBytes);
         const int live = min(C, p.T - n * C);
-        k.template fetch<TH>((const IO*)p.k + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, live);
-        pm.template fetch<TH>((const IO*)p.P + (wrow0 + (size_t)n * C) * C, C, C);
-        o.template fetch<TH>((const IO*)p.dO + (row0 + (size_t)n * C * H) * DV + j0, (size_t)H * DV, live);
+        k.template fetch<NL>((const IO*)p.k + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, live, me);
+        pm.template fetch<NL>((const IO*)p.P + (wrow0 + (size_t)n * C) * C, C, C, me);
+        o.template fetch<NL>((const IO*)p.dO + (row0 + (size_t)n * C * H) * DV + j0, (size_t)H * DV, live, me);
     };
     auto fetch2 = [&](int n) {         // Q and W<-, read in the second
-        mQ.template fetch<TH>((const IO*)p.q + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C));
-        mW.template fetch<TH>((const IO*)p.W + (wrow0 + (size_t)n * C) * DK, DK, C);
+        mQ.template fetch<NL>((const IO*)p.q + (row0 + (size_t)n * C * H) * DK, (size_t)H * DK, min(C, p.T - n * C), me);
+        mW.template fetch<NL>((const IO*)p.W + (wrow0 + (size_t)n * C) * DK, DK, C, me);
     };
     uint32_t d[2][2];                  // Delta and the entry state at this thread's elements
     float2 hin[MU][2][2];
@@ -298,26 +312,34 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
             }
     };
     ChainCoef cf;
-    fetch1(p.N - 1);
+    if (loads) {
+        fetch1(p.N - 1);
+        cf.get(p, wrow0 + (size_t)(p.N - 1) * C, nrows, me);
+    }
     fetch_commit();
-    cf.get(p, wrow0 + (size_t)(p.N - 1) * C, nrows);
-    fetch_d(p.N - 1);
+    if (works) fetch_d(p.N - 1);
     float dst[MU][2][4];
     zero(dst);
-    if (p.dhT) each(dst, si, wn, [&](int i, int j, float& x, float& y) {
+    if (p.dhT && works) each(dst, si, wn, [&](int i, int j, float& x, float& y) {
         const float2 v = *state_at(const_cast<float*>(p.dhT) + (size_t)bh * DK * DV, i, j);
         x = v.x; y = v.y;
     });
-    each(dst, si, wn, [&](int i, int j, float x, float y) { mS.st2(i, j, x, y); });
-    cf.put(sgq[(p.N - 1) & 1], sgk[(p.N - 1) & 1], sgC + ((p.N - 1) & 1));
+    if (works) each(dst, si, wn, [&](int i, int j, float x, float y) { mS.st2(i, j, x, y); });
+    if (loads) cf.put(sgq[(p.N - 1) & 1], sgk[(p.N - 1) & 1], sgC + ((p.N - 1) & 1), me);
     for (int n = p.N - 1; n >= 0; --n) {
         const int bf = n & 1;
         fetch_wait();
         __syncthreads();
-        fetch2(n);
+        if (loads) fetch2(n);
         fetch_commit();
-        if (n > 0) { fetch1(n - 1); cf.get(p, wrow0 + (size_t)(n - 1) * C, nrows); }
+        if (n > 0 && loads) { fetch1(n - 1); cf.get(p, wrow0 + (size_t)(n - 1) * C, nrows, me); }
         fetch_commit();
+        if (LOADERS && loads) {
+            fetch_wait_but<1>();
+            __syncthreads();
+            if (n > 0) cf.put(sgq[bf ^ 1], sgk[bf ^ 1], sgC + (bf ^ 1), me);
+            continue;
+        }
         const typename L::TA mK(smb + bf * kSet);
         const typename L::TP mP(smb + bf * kSet + L::TA::kBytes);
         const typename L::TO mO(smb + bf * kSet + L::TA::kBytes + L::TP::kBytes);
@@ -386,9 +408,9 @@ __global__ void __launch_bounds__(8 * DS) k_chain_bwd(Ptrs p, int DV) {
                 mS.st2(i, j, x, y);
             });
         }
-        if (n > 0) cf.put(sgq[bf ^ 1], sgk[bf ^ 1], sgC + (bf ^ 1));
+        if (!LOADERS && n > 0) cf.put(sgq[bf ^ 1], sgk[bf ^ 1], sgC + (bf ^ 1));
     }
-    if (p.dh0) each(dst, si, wn, [&](int i, int j, float x, float y) { *state_at(p.dh0 + (size_t)bh * DK * DV, i, j) = make_float2(x, y); });
+    if (p.dh0 && works) each(dst, si, wn, [&](int i, int j, float x, float y) { *state_at(p.dh0 + (size_t)bh * DK * DV, i, j) = make_float2(x, y); });
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -662,12 +684,16 @@ cudaError_t prep_for(const ChunkArgs& a, const Ptrs& p) {
 template <int DK, int DS>
 cudaError_t chain_fwd_for(const ChunkArgs& a, const Ptrs& p) {
     typedef ChainPlanes<DK, DS> L;
-    return launch(k_chain_fwd<DK, DS>, a.s.B * a.s.H * (a.s.dv / DS), L::kThreads, L::kFwd, a.stream, p, a.s.dv);
+    const int grid = a.s.B * a.s.H * (a.s.dv / DS);
+    if (grid <= kSMs) return launch(k_chain_fwd<DK, DS, true>, grid, L::kThreads + kLoaders, L::kFwd, a.stream, p, a.s.dv);
+    return launch(k_chain_fwd<DK, DS, false>, grid, L::kThreads, L::kFwd, a.stream, p, a.s.dv);
 }
 template <int DK, int DS>
 cudaError_t chain_bwd_for(const ChunkArgs& a, const Ptrs& p) {
     typedef ChainPlanes<DK, DS> L;
-    return launch(k_chain_bwd<DK, DS>, a.s.B * a.s.H * (a.s.dv / DS), L::kThreads, L::kBwd, a.stream, p, a.s.dv);
+    const int grid = a.s.B * a.s.H * (a.s.dv / DS);
+    if (grid <= kSMs) return launch(k_chain_bwd<DK, DS, true>, grid, L::kThreads + kLoaders, L::kBwd, a.stream, p, a.s.dv);
+    return launch(k_chain_bwd<DK, DS, false>, grid, L::kThreads, L::kBwd, a.stream, p, a.s.dv);
 }
 template <int DK, int DV>
 cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {

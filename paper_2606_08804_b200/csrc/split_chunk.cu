@@ -54,6 +54,19 @@ __device__ __forceinline__ void load_tile(float* dst, const float* src, size_t s
     t.put(dst);
 }
 
+// The same asynchronously, by the threads that load (number `me` of kLoaders).
+template <int ROWS, int W, int LD>
+__device__ __forceinline__ void fetch_tile(float* dst, const float* src, size_t stride, int live, int me) {
+    constexpr int kChunks = W / 4, kTotal = ROWS * kChunks;
+#pragma unroll 8
+    for (int id = me; id < kTotal; id += kLoaders) {
+        const int row = id / kChunks, c = id % kChunks * 4;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sm100::smem_u32(dst + row * LD + c)),
+                     "l"(src + (row < live ? (size_t)row * stride : 0) + c), "r"(row < live ? 16 : 0) : "memory");
+    }
+}
+__device__ __forceinline__ void fetched() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------------------------
 // K1: per chunk-head, state-independent part: g, P, W<-, U~ (and M for the backward).
 template <int DK, int DV>
@@ -163,48 +176,55 @@ __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
 
 // ---------------------------------------------------------------------------------------------
 // K2: forward state chain.  One CTA per (sequence, DS-column slice of d_v); columns of the state evolve independently,
-// the chunks of a sequence are walked in order.  The next chunk's tiles are fetched into registers while the present
-// chunk is worked on: a chunk costs its two dependent products and three barriers, not its loads.
+// the chunks of a sequence are walked in order.  A chunk costs its two dependent products and two barriers, not its loads: four
+// warps do nothing else than copy, K and P while Delta is made, the next W<-, Q and U~ while the state is updated.
 template <int DK, int DS>
-__global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
+__global__ void __launch_bounds__(NT + kLoaders) k_chain_fwd(Ptrs p, int DV) {
     extern __shared__ float sm[];
     constexpr int LA = DK + 4, LB = DK + 8, LS = DS + 8, NS = DS / 8;
     float *sW = sm, *sQ = sW + C * LA, *sK = sQ + C * LA, *sP = sK + C * LB, *sU = sP + C * LDC, *sD = sU + C * LS,
           *sDs = sD + C * LS, *sh = sDs + C * LS;                     // sh: the state slice [DK][DS]
-    __shared__ float sgq[C], sgk[C], sgC;
+    __shared__ float sgq_[2][C], sgk_[2][C], sgC_[2];                 // by parity of the chunk
     const int H = p.H, nsl = DV / DS, j0 = (blockIdx.x % nsl) * DS, bh = blockIdx.x / nsl, b = bh / H, hh = bh % H;
     const int tid = threadIdx.x, warp = tid >> 5;
     sm100::grid_dep_wait();            // launched while the kernel before it drains
     sm100::grid_dep_launch();
+    const size_t nrows = (size_t)p.B * H * p.Tp;
+    if (tid >= NT) {
+        const int me = tid - NT;
+        auto fetch1 = [&](int n) {     // read in the first phase of chunk n
+            const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
+            fetch_tile<C, DK, LA>(sW, (const float*)p.W + wrow0 * DK, DK, C, me);
+            fetch_tile<C, DK, LA>(sQ, (const float*)p.q + row0 * DK, (size_t)H * DK, min(C, p.T - n * C), me);
+            fetch_tile<C, DS, LS>(sU, (const float*)p.U + wrow0 * DV + j0, DV, C, me);
+        };
+        auto fetch2 = [&](int n) {     // read in the second
+            const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
+            fetch_tile<C, DK, LB>(sK, (const float*)p.k + row0 * DK, (size_t)H * DK, min(C, p.T - n * C), me);
+            fetch_tile<C, C, LDC>(sP, (const float*)p.P + wrow0 * C, C, C, me);
+        };
+        ChainCoef cf;
+        fetch1(0);
+        cf.get(p, (size_t)bh * p.Tp, nrows, me);
+        for (int n = 0; n < p.N; ++n) {
+            cf.put(sgq_[n & 1], sgk_[n & 1], sgC_ + (n & 1), me);
+            fetched();
+            __syncthreads();           // W<-, Q, U~ and the factors are there; K and P have been read
+            fetch2(n);
+            fetched();
+            __syncthreads();           // K and P are there; W<-, Q and U~ have been read
+            if (n + 1 < p.N) { fetch1(n + 1); cf.get(p, (size_t)bh * p.Tp + (size_t)(n + 1) * C, nrows, me); }
+        }
+        return;
+    }
     for (int e = tid; e < DK * DS; e += NT)
         sh[(e / DS) * LS + e % DS] = p.h0 ? p.h0[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] : 0.f;
-    Tile<C, DK, LA> tw, tq;
-    Tile<C, DK, LB> tk;
-    Tile<C, C, LDC> tp;
-    Tile<C, DS, LS> tu;
-    float g = 0.f, gC = 0.f, rq = 1.f, rk = 1.f;
-    const size_t nrows = (size_t)p.B * H * p.Tp;
-    auto fetch = [&](int n) {
-        const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
-        const int live = min(C, p.T - n * C);
-        tw.get((const float*)p.W + wrow0 * DK, DK, C);
-        tq.get((const float*)p.q + row0 * DK, (size_t)H * DK, live);
-        tk.get((const float*)p.k + row0 * DK, (size_t)H * DK, live);
-        tp.get((const float*)p.P + wrow0 * C, C, C);
-        tu.get((const float*)p.U + wrow0 * DV + j0, DV, C);
-        if (tid < C) {
-            g = p.g[wrow0 + tid]; gC = p.g[wrow0 + C - 1];
-            if (p.rqk) { rq = p.rqk[wrow0 + tid]; rk = p.rqk[nrows + wrow0 + tid]; }
-        }
-    };
-    fetch(0);
     for (int n = 0; n < p.N; ++n) {
         const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
         const int live = min(C, p.T - n * C);
-        tw.put(sW); tq.put(sQ); tk.put(sK); tp.put(sP); tu.put(sU);
-        if (tid < C) { sgq[tid] = expf(g) * rq; sgk[tid] = expf(gC - g) * rk; if (tid == 0) sgC = expf(gC); }
+        const float *sgq = sgq_[n & 1], *sgk = sgk_[n & 1];
         __syncthreads();
-        if (n + 1 < p.N) fetch(n + 1);
+        const float gC = sgC_[n & 1];
         if (p.save) {
             float* dst = p.hs + ((size_t)bh * p.N + n) * DK * DV + j0;
             for (int e = tid * 4; e < DK * DS; e += NT * 4)
@@ -248,14 +268,15 @@ __global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
                                    [&](int r, int j) { return sDs[r * LS + j]; });
             each(ha, i0, 0, [&](int i, int j, float x, float y) {
                 float* d = sh + i * LS + j;
-                st2(d, fmaf(sgC, d[0], x), fmaf(sgC, d[1], y));
+                st2(d, fmaf(gC, d[0], x), fmaf(gC, d[1], y));
             });
         }
-        __syncthreads();
     }
-    if (p.hT)
+    if (p.hT) {
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");        // the state is complete
         for (int e = tid; e < DK * DS; e += NT)
             p.hT[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] = sh[(e / DS) * LS + e % DS];
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -263,45 +284,51 @@ __global__ void __launch_bounds__(NT) k_chain_fwd(Ptrs p, int DV) {
 //   dDelta = P^T dO + K-> dh ;   dh_in = gamma_C dh + (diag(gamma) Q)^T dO - W<-^T dDelta
 // and leaves per chunk: dh (exit), dDelta, and two scalar partial sums the decay gradient needs.
 template <int DK, int DS>
-__global__ void __launch_bounds__(NT) k_chain_bwd(Ptrs p, int DV) {
+__global__ void __launch_bounds__(NT + kLoaders) k_chain_bwd(Ptrs p, int DV) {
     extern __shared__ float sm[];
     constexpr int LA = DK + 4, LB = DK + 8, LP = C + 8, LS = DS + 8, NS = DS / 8;
     float *sK = sm, *sQ = sK + C * LA, *sW = sQ + C * LB, *sP = sW + C * LB, *sO = sP + C * LP, *sOs = sO + C * LS,
           *sD = sOs + C * LS, *sdD = sD + C * LS, *sdh = sdD + C * LS;
-    __shared__ float sgq[C], sgk[C], sgC, sred[NT / 32], skd[C];
+    __shared__ float sgq_[2][C], sgk_[2][C], sgC_[2], sred[NT / 32], skd[C];          // the first three by parity of the chunk
     const int H = p.H, nsl = DV / DS, sl = blockIdx.x % nsl, j0 = sl * DS, bh = blockIdx.x / nsl, b = bh / H, hh = bh % H;
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t nrows = (size_t)p.B * H * p.Tp, BHN = (size_t)p.B * H * p.N;
     sm100::grid_dep_wait();            // launched while the kernel before it drains
     sm100::grid_dep_launch();
+    if (tid >= NT) {
+        const int me = tid - NT;
+        auto fetch1 = [&](int n) {     // read in the first two phases of chunk n
+            const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
+            const int live = min(C, p.T - n * C);
+            fetch_tile<C, DS, LS>(sO, (const float*)p.dO + row0 * DV + j0, (size_t)H * DV, live, me);
+            fetch_tile<C, DS, LS>(sD, (const float*)p.D + wrow0 * DV + j0, DV, C, me);
+            fetch_tile<C, DK, LA>(sK, (const float*)p.k + row0 * DK, (size_t)H * DK, live, me);
+            fetch_tile<C, DK, LB>(sQ, (const float*)p.q + row0 * DK, (size_t)H * DK, live, me);
+            fetch_tile<C, C, LP>(sP, (const float*)p.P + wrow0 * C, C, C, me);
+        };
+        ChainCoef cf;
+        fetch1(p.N - 1);
+        cf.get(p, (size_t)bh * p.Tp + (size_t)(p.N - 1) * C, nrows, me);
+        for (int n = p.N - 1; n >= 0; --n) {
+            const size_t wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
+            cf.put(sgq_[n & 1], sgk_[n & 1], sgC_ + (n & 1), me);
+            fetched();
+            __syncthreads();           // all but W<- is there; W<- has been read
+            fetch_tile<C, DK, LB>(sW, (const float*)p.W + wrow0 * DK, DK, C, me);
+            __syncthreads();
+            fetched();
+            __syncthreads();           // W<- is there; the others have been read
+            if (n > 0) { fetch1(n - 1); cf.get(p, wrow0 - C, nrows, me); }
+        }
+        return;
+    }
     for (int e = tid; e < DK * DS; e += NT)
         sdh[(e / DS) * LS + e % DS] = p.dhT ? p.dhT[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] : 0.f;
-    Tile<C, DK, LA> tk;
-    Tile<C, DK, LB> tq, tw;
-    Tile<C, C, LP> tp;
-    Tile<C, DS, LS> to, td;
-    float g = 0.f, gC = 0.f, rq = 1.f, rk = 1.f;
-    auto fetch = [&](int n) {
-        const size_t row0 = ((size_t)b * p.T + (size_t)n * C) * H + hh, wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
-        const int live = min(C, p.T - n * C);
-        tk.get((const float*)p.k + row0 * DK, (size_t)H * DK, live);
-        tq.get((const float*)p.q + row0 * DK, (size_t)H * DK, live);
-        tw.get((const float*)p.W + wrow0 * DK, DK, C);
-        tp.get((const float*)p.P + wrow0 * C, C, C);
-        to.get((const float*)p.dO + row0 * DV + j0, (size_t)H * DV, live);
-        td.get((const float*)p.D + wrow0 * DV + j0, DV, C);
-        if (tid < C) {
-            g = p.g[wrow0 + tid]; gC = p.g[wrow0 + C - 1];
-            if (p.rqk) { rq = p.rqk[wrow0 + tid]; rk = p.rqk[nrows + wrow0 + tid]; }
-        }
-    };
-    fetch(p.N - 1);
     for (int n = p.N - 1; n >= 0; --n) {
         const size_t wrow0 = (size_t)bh * p.Tp + (size_t)n * C;
-        tk.put(sK); tq.put(sQ); tw.put(sW); tp.put(sP); to.put(sO); td.put(sD);
-        if (tid < C) { sgq[tid] = expf(g) * rq; sgk[tid] = expf(gC - g) * rk; if (tid == 0) sgC = expf(gC); }
+        const float *sgq = sgq_[n & 1], *sgk = sgk_[n & 1];
         __syncthreads();
-        if (n > 0) fetch(n - 1);
+        const float gC = sgC_[n & 1];
         // keep dh of this chunk's exit state; partial <dh, h_entry>_F over this slice
         {
             float* dst = p.dhs + ((size_t)bh * p.N + n) * DK * DV + j0;
@@ -360,16 +387,17 @@ __global__ void __launch_bounds__(NT) k_chain_bwd(Ptrs p, int DV) {
                                    [&](int r, int j) { return sdD[r * LS + j]; });
             each(ha, i0, 0, [&](int i, int j, float x, float y) {
                 float* d = sdh + i * LS + j;
-                st2(d, fmaf(sgC, d[0], x), fmaf(sgC, d[1], y));
+                st2(d, fmaf(gC, d[0], x), fmaf(gC, d[1], y));
             });
         } else if (tid < C) {
             p.kdhd[(size_t)sl * nrows + wrow0 + tid] = skd[tid];
         }
-        __syncthreads();
     }
-    if (p.dh0)
+    if (p.dh0) {
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");        // the gradient is complete
         for (int e = tid; e < DK * DS; e += NT)
             p.dh0[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] = sdh[(e / DS) * LS + e % DS];
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -611,12 +639,12 @@ cudaError_t prep_for(const ChunkArgs& a, const Ptrs& p) {
 template <int DK, int DS>
 cudaError_t chain_fwd_for(const ChunkArgs& a, const Ptrs& p) {
     constexpr size_t smem = sizeof(float) * (2 * C * (DK + 4) + C * (DK + 8) + C * LDC + (3 * C + DK) * (DS + 8));
-    return launch(k_chain_fwd<DK, DS>, a.s.B * a.s.H * (a.s.dv / DS), NT, smem, a.stream, p, a.s.dv);
+    return launch(k_chain_fwd<DK, DS>, a.s.B * a.s.H * (a.s.dv / DS), NT + kLoaders, smem, a.stream, p, a.s.dv);
 }
 template <int DK, int DS>
 cudaError_t chain_bwd_for(const ChunkArgs& a, const Ptrs& p) {
     constexpr size_t smem = sizeof(float) * (C * (DK + 4) + 2 * C * (DK + 8) + C * (C + 8) + (4 * C + DK) * (DS + 8));
-    return launch(k_chain_bwd<DK, DS>, a.s.B * a.s.H * (a.s.dv / DS), NT, smem, a.stream, p, a.s.dv);
+    return launch(k_chain_bwd<DK, DS>, a.s.B * a.s.H * (a.s.dv / DS), NT + kLoaders, smem, a.stream, p, a.s.dv);
 }
 template <int DK, int DV>
 cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {
@@ -632,7 +660,7 @@ cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {
 //         128 x 64    37: 230 against 273      38: 375 against 330            128 x 64    37: 121 against 137   38: 195 against 168
 //          64 x 128   18: 123 against 151      19: 214 against 194             64 x 128   18:  74 against  84   19: 114 against 108
 //         128 x 128   18: 177 against 215      19: 334 against 291
-// The same with 2048 tokens, and up to 800 narrow CTAs wide slices stay ahead, but for fp32 with d_k = 64 at 352 (narrow by 3 %).
+// (measured before the copies had warps of their own, which narrow slices gain more from).  The same with 2048 tokens, and up to 800 narrow CTAs wide slices stay ahead, but for fp32 with d_k = 64 at 352 (narrow by 3 %).
 int split_slice(const qd_shape& s) { return (long long)s.B * s.H * (s.dv / 16) <= kSMs ? 16 : 32; }
 
 #define QD_BY_DIMS(fn, a, p)                                                                                  \

@@ -237,18 +237,27 @@ __device__ __forceinline__ void scan64(float x, float* sg) {
     asm volatile("bar.sync 1, 64;" ::: "memory");
 }
 
-// decay factors of a chunk's tokens, thread t < 64 token t: fetched a chunk ahead, written before the barrier that ends the present one
+// Copies of the state chains: by four extra warps, which issue them while the others compute.  Issued by the warps that compute, the
+// copies and the decay factors of a chunk were 800 - 1100 of its 3500 - 4500 cycles.  Forward and backward, before and with them:
+// fp32 16 sequences of 512 tokens, 128 x 128 170 -> 161 us, 8 of 1024, 64 x 128 183 -> 161, 128 of 1024, 64 x 64 947 -> 901; bf16 64 x 64,
+// 64 of 1024 247 -> 240, 8 of 1024 102 -> 91, 2 of 4096 287 -> 246.  A warp's share of the output moved to further warps as well: 2 %
+// more on narrow slices, 2 % less on wide ones.
+constexpr int kLoaders = 128;
+template <int N> __device__ __forceinline__ void fetch_wait_but() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+// decay factors of a chunk's tokens, thread `me` < 64 token `me`: fetched a chunk ahead, written before the barrier that ends the present one
 struct ChainCoef {
     float g = 0.f, gC = 0.f, rq = 1.f, rk = 1.f;
-    __device__ __forceinline__ void get(const Ptrs& p, size_t wrow0, size_t nrows) {
-        if (threadIdx.x >= C) return;
-        g = p.g[wrow0 + threadIdx.x]; gC = p.g[wrow0 + C - 1];
-        if (p.rqk) { rq = p.rqk[wrow0 + threadIdx.x]; rk = p.rqk[nrows + wrow0 + threadIdx.x]; }
+    __device__ __forceinline__ void get(const Ptrs& p, size_t wrow0, size_t nrows, int me = threadIdx.x) {
+        if (me >= C) return;
+        g = p.g[wrow0 + me]; gC = p.g[wrow0 + C - 1];
+        if (p.rqk) { rq = p.rqk[wrow0 + me]; rk = p.rqk[nrows + wrow0 + me]; }
     }
-    __device__ __forceinline__ void put(float* gq, float* gk, float* gc) const {
-        if (threadIdx.x >= C) return;
-        gq[threadIdx.x] = expf(g) * rq; gk[threadIdx.x] = expf(gC - g) * rk;
-        if (threadIdx.x == 0) *gc = expf(gC);
+    __device__ __forceinline__ void put(float* gq, float* gk, float* gc, int me = threadIdx.x) const {
+        if (me >= C) return;
+        gq[me] = expf(g) * rq; gk[me] = expf(gC - g) * rk;
+        if (me == 0) *gc = expf(gC);
     }
 };
 // Per token, from the row sums (prow: dP o P, t1, t2, d beta, d lambda) and the column sums (cP: dP o P, cA: dA o A; db1: dT o M,

@@ -21,6 +21,9 @@ pytestmark = pytest.mark.gpu
     ("bf16", 1, 2, 1, 64, 64),
     ("bf16", 5, 12, 70, 128, 64),
     ("bf16", 3, 10, 127, 64, 128),
+    ("bf16", 2, 37, 65, 64, 64),      # 148 CTAs of the state chains: copies by warps of their own
+    ("bf16", 3, 25, 65, 64, 64),      # 150: by everybody
+    ("bf16", 3, 25, 130, 128, 64),
 ])
 def test_split_kernels(dtype, B, H, T, dk, dv):
     base = gen.CONFIGS["cfg2"] if dtype == "bf16" else replace(gen.CONFIGS["cfg0"], h0=True, backward=True)
