@@ -3,7 +3,7 @@
 //   o = h_new^T q = alpha h^T q + (k.q) delta .
 // A CTA owns DVS columns of one state (columns evolve independently); every thread keeps its part of the slice in
 // registers between the only read and the only write of the state, all loads are issued before the first use.
-// One token is bound by HBM traffic: 80.4 us for 4096 states of 128 x 128 in fp32, 1.02 of the measured copy bandwidth (48
+// One token is bound by HBM traffic: 80.4 us for 4096 states of 128 x 128 in fp32, 1.02 of the measured copy bandwidth (44 - 46
 // of 41 us at that bandwidth with a bf16 state, whose rows are read 16 bytes per thread like those of an fp32 one).
 #include "internal.h"
 #include "sm100.cuh"
@@ -25,9 +25,16 @@ namespace {
 // spill; five CTAs would spill 64 - 204.
 // SB16 (QD_STATE_BF16): the state is STORED in bf16 (half the bytes of the step); it is widened to fp32 when read, all S
 // tokens of the call are applied in fp32, and it is rounded to bf16 once, when written back.
+// ONE (bf16 state, a single token): the state is needed once more only to be updated, so it stays as it was read, is widened each
+// time and written back as it is updated: 32 registers instead of 64, and five CTAs to an SM instead of four, which with 16 KB each
+// are too little on its way to keep HBM busy (256 x 16 states 47.7 -> 44.0 us, 100 x 8 12.2 -> 11.1; six CTAs, which spill 70 bytes,
+// 49.5).  With an fp32 state it would gain nothing (30 x 16 states 11.8 -> 12.4).
+// VEC: the rows of a thread are neighbours, so that its parts of x, q and k are read four at a time (8 tokens of 256 x 16 states 156 ->
+// 150 us, of 48 x 16 36.2 -> 35.0).  Rows a whole group apart where the tokens are normalised, which leaves fewer registers (4 tokens of
+// 48 x 16 states 25.7 us so, 26.1 with neighbours).
 constexpr int kBlock = 8;
-template <typename IO, int DK, int DVS, int NT, bool LOGITS, bool NORM, bool SB16>      // flags, compile-time
-__global__ void __launch_bounds__(NT, 4) k_decode(int S, int H, int dv, const IO* __restrict__ q, const IO* __restrict__ k,
+template <typename IO, int DK, int DVS, int NT, bool LOGITS, bool NORM, bool SB16, bool ONE>      // flags, compile-time
+__global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H, int dv, const IO* __restrict__ q, const IO* __restrict__ k,
                                                      const IO* __restrict__ v, const IO* __restrict__ beta,
                                                      const IO* __restrict__ alpha, const IO* __restrict__ lam,
                                                      void* __restrict__ state_, IO* __restrict__ o) {
@@ -35,6 +42,7 @@ __global__ void __launch_bounds__(NT, 4) k_decode(int S, int H, int dv, const IO
     constexpr int CT = DVS / NC, RP = NT / CT, NP = DK / RP;
     static_assert(NT % CT == 0 && DK % RP == 0, "bad decode tiling");
     constexpr int TOKEN = 3 * DK + DVS;
+    constexpr bool VEC = SB16 || !NORM;
     extern __shared__ __align__(16) float stok[];                // per token: x [DK], q [DK], k [DK], v [DVS]
     __shared__ __align__(16) float redx[2][RP][DVS], redq[2][RP][DVS];
     __shared__ __align__(16) float sdelta[2][DVS];
@@ -43,12 +51,13 @@ __global__ void __launch_bounds__(NT, 4) k_decode(int S, int H, int dv, const IO
     const int b = bh / H, hh = bh % H;
     const int ct = tid % CT, rg = tid / CT, lane = tid & 31;
 
-    uint4* base = reinterpret_cast<uint4*>(static_cast<unsigned char*>(state_) + (((size_t)bh * DK + rg) * dv + j0) * (SB16 ? 2 : 4)) + ct;
-    const size_t rstride = (size_t)RP * dv / NC;
+    uint4* base = reinterpret_cast<uint4*>(static_cast<unsigned char*>(state_) + (((size_t)bh * DK + (VEC ? rg * NP : rg)) * dv + j0) * (SB16 ? 2 : 4)) + ct;
+    const size_t rstride = (size_t)(VEC ? 1 : RP) * dv / NC;
     // launched while the kernel before it drains (2 us less per step): nothing is read before that kernel has completed
     sm100::grid_dep_wait();
     sm100::grid_dep_launch();
-    float h[NP][NC];
+    constexpr bool KEEP = !ONE;                                  // the state in fp32 from token to token
+    float h[KEEP ? NP : 1][NC];
     uint4 raw[NP];
 #pragma unroll
     for (int pz = 0; pz < NP; ++pz) raw[pz] = __ldcs(base + pz * rstride);
@@ -109,21 +118,40 @@ __global__ void __launch_bounds__(NT, 4) k_decode(int S, int H, int dv, const IO
         __syncthreads();
     };
     stage(0);
-#pragma unroll
-    for (int pz = 0; pz < NP; ++pz) {
-        const uint32_t w[4] = {raw[pz].x, raw[pz].y, raw[pz].z, raw[pz].w};
+    auto four = [&](const float* v, int p4) {
+        if (VEC) return *reinterpret_cast<const float4*>(v + rg * NP + p4);
+        return make_float4(v[p4 * RP + rg], v[(p4 + 1) * RP + rg], v[(p4 + 2) * RP + rg], v[(p4 + 3) * RP + rg]);
+    };
+    auto widen = [&](const uint4& r, float (&d)[NC]) {
+        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             if (SB16) {
-                h[pz][(2 * e) % NC] = __uint_as_float(w[e] << 16);
-                h[pz][(2 * e + 1) % NC] = __uint_as_float(w[e] & 0xffff0000u);
+                d[(2 * e) % NC] = __uint_as_float(w[e] << 16);
+                d[(2 * e + 1) % NC] = __uint_as_float(w[e] & 0xffff0000u);
             } else {
-                h[pz][e] = __uint_as_float(w[e]);
+                d[e] = __uint_as_float(w[e]);
             }
         }
-    }
+    };
+    auto write = [&](int pz, const float (&d)[NC]) {
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (SB16) {
+                const __nv_bfloat162 t = __floats2bfloat162_rn(d[(2 * e) % NC], d[(2 * e + 1) % NC]);
+                w[e] = *reinterpret_cast<const uint32_t*>(&t);
+            } else {
+                w[e] = __float_as_uint(d[e]);
+            }
+        }
+        __stcs(base + pz * rstride, make_uint4(w[0], w[1], w[2], w[3]));
+    };
+    if (KEEP)
+#pragma unroll
+        for (int pz = 0; pz < NP; ++pz) widen(raw[pz], h[pz % (KEEP ? NP : 1)]);
     for (int s0 = 0;;) {
-        const int nb = min(kBlock, S - s0);
+        const int nb = ONE ? 1 : min(kBlock, S - s0);
 #pragma unroll 1
         for (int s = 0; s < nb; ++s) {
             const float *tx = stok + s * TOKEN, *tq = tx + DK, *tk = tq + DK;
@@ -133,10 +161,18 @@ __global__ void __launch_bounds__(NT, 4) k_decode(int S, int H, int dv, const IO
 #pragma unroll
             for (int e = 0; e < NC; ++e) { ax[e] = 0.f; aq[e] = 0.f; }
 #pragma unroll
-            for (int pz = 0; pz < NP; ++pz) {
-                const float xi = tx[pz * RP + rg], qi = tq[pz * RP + rg];
+            for (int p4 = 0; p4 < NP; p4 += 4) {
+                if (!KEEP) asm volatile("" ::: "memory");                // four rows at a time
+                const float4 x4 = four(tx, p4), q4 = four(tq, p4);
+                const float xi[4] = {x4.x, x4.y, x4.z, x4.w}, qi[4] = {q4.x, q4.y, q4.z, q4.w};
 #pragma unroll
-                for (int e = 0; e < NC; ++e) { ax[e] = fmaf(h[pz][e], xi, ax[e]); aq[e] = fmaf(h[pz][e], qi, aq[e]); }
+                for (int z = 0; z < 4; ++z) {
+                    float one[NC];
+                    if (!KEEP) widen(raw[p4 + z], one);
+                    const float (&hr)[NC] = KEEP ? h[(p4 + z) % (KEEP ? NP : 1)] : one;
+#pragma unroll
+                    for (int e = 0; e < NC; ++e) { ax[e] = fmaf(hr[e], xi[z], ax[e]); aq[e] = fmaf(hr[e], qi[z], aq[e]); }
+                }
             }
 #pragma unroll
             for (int e = 0; e < NC; e += 4) {
@@ -154,6 +190,9 @@ __global__ void __launch_bounds__(NT, 4) k_decode(int S, int H, int dv, const IO
                 st(o, row * dv + j0 + tid, fmaf(al, rq, scoef[s][2] * dl));
             }
             __syncthreads();
+            if (!KEEP)                                                   // widened anew, instead of being kept widened
+#pragma unroll
+                for (int pz = 0; pz < NP; ++pz) asm volatile("" : "+r"(raw[pz].x), "+r"(raw[pz].y), "+r"(raw[pz].z), "+r"(raw[pz].w));
             float dl[NC];
 #pragma unroll
             for (int e = 0; e < NC; e += 4) {
@@ -161,31 +200,29 @@ __global__ void __launch_bounds__(NT, 4) k_decode(int S, int H, int dv, const IO
                 dl[e] = t.x; dl[e + 1] = t.y; dl[e + 2] = t.z; dl[e + 3] = t.w;
             }
 #pragma unroll
-            for (int pz = 0; pz < NP; ++pz) {
-                const float ki = tk[pz * RP + rg];
+            for (int p4 = 0; p4 < NP; p4 += 4) {
+                if (!KEEP) asm volatile("" ::: "memory");                // four rows at a time
+                const float4 k4 = four(tk, p4);
+                const float ki[4] = {k4.x, k4.y, k4.z, k4.w};
 #pragma unroll
-                for (int e = 0; e < NC; ++e) h[pz][e] = fmaf(al, h[pz][e], ki * dl[e]);
+                for (int z = 0; z < 4; ++z) {
+                    float one[NC];
+                    if (!KEEP) widen(raw[p4 + z], one);
+                    float (&hr)[NC] = KEEP ? h[(p4 + z) % (KEEP ? NP : 1)] : one;
+#pragma unroll
+                    for (int e = 0; e < NC; ++e) hr[e] = fmaf(al, hr[e], ki[z] * dl[e]);
+                    if (!KEEP) write(p4 + z, hr);
+                }
             }
         }
         s0 += kBlock;
-        if (s0 >= S) break;
+        if (ONE || s0 >= S) break;
         __syncthreads();                                                 // the staged tokens are rewritten
         stage(s0);
     }
+    if (KEEP)
 #pragma unroll
-    for (int pz = 0; pz < NP; ++pz) {
-        uint32_t w[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (SB16) {
-                const __nv_bfloat162 t = __floats2bfloat162_rn(h[pz][(2 * e) % NC], h[pz][(2 * e + 1) % NC]);
-                w[e] = *reinterpret_cast<const uint32_t*>(&t);
-            } else {
-                w[e] = __float_as_uint(h[pz][e]);
-            }
-        }
-        __stcs(base + pz * rstride, make_uint4(w[0], w[1], w[2], w[3]));
-    }
+        for (int pz = 0; pz < NP; ++pz) write(pz, h[pz % (KEEP ? NP : 1)]);
 }
 
 template <typename IO, int DK>
@@ -194,11 +231,13 @@ cudaError_t launch(int B, int S, int H, int dv, const void* q, const void* k, co
                          cudaStream_t stream) {
     constexpr int DVS = 64, NT = 128;
     dim3 grid((unsigned)(dv / DVS) * (unsigned)(B * H));
-    auto kern = logits ? (norm ? k_decode<IO, DK, DVS, NT, true, true, false> : k_decode<IO, DK, DVS, NT, true, false, false>)
-                       : (norm ? k_decode<IO, DK, DVS, NT, false, true, false> : k_decode<IO, DK, DVS, NT, false, false, false>);
-    if (sb16)
-        kern = logits ? (norm ? k_decode<IO, DK, DVS, NT, true, true, true> : k_decode<IO, DK, DVS, NT, true, false, true>)
-                      : (norm ? k_decode<IO, DK, DVS, NT, false, true, true> : k_decode<IO, DK, DVS, NT, false, false, true>);
+    using Kern = decltype(&k_decode<IO, DK, DVS, NT, false, false, false, false>);
+#define QD_GATES(SB16, ONE)                                                                                                  \
+    {k_decode<IO, DK, DVS, NT, false, false, SB16, ONE>, k_decode<IO, DK, DVS, NT, false, true, SB16, ONE>,                  \
+     k_decode<IO, DK, DVS, NT, true, false, SB16, ONE>, k_decode<IO, DK, DVS, NT, true, true, SB16, ONE>}
+    static const Kern table[3][4] = {QD_GATES(false, false), QD_GATES(true, false), QD_GATES(true, true)};
+#undef QD_GATES
+    const Kern kern = table[sb16 ? (S == 1 ? 2 : 1) : 0][(logits ? 2 : 0) + (norm ? 1 : 0)];
     return launch_overlapped(kern, grid, dim3(NT), (S < kBlock ? S : kBlock) * (3 * DK + DVS) * sizeof(float), stream, S, H, dv,
                              (const IO*)q, (const IO*)k, (const IO*)v, (const IO*)beta, (const IO*)alpha, (const IO*)lam, state, (IO*)o);
 }

@@ -233,3 +233,23 @@ def test_decode_with_bf16_state_storage(S):
     assert state.intact()
     assert worst_r <= 2e-2 and gu.rel_err(state.t.float(), ref_r) <= 2e-2, (worst_r,)
     assert worst_x <= 2e-2 and gu.rel_err(state.t.float(), ref_x) <= 2e-2, (worst_x,)
+
+
+@pytest.mark.parametrize("dk,dv,S,raw", [(128, 128, 1, False), (128, 128, 1, True), (64, 64, 1, True), (64, 128, 1, False), (128, 64, 2, True)])
+def test_bf16_state_is_the_fp32_one_rounded(dk, dv, S, raw):
+    """A bf16 state of one token is widened where it is used, of several tokens kept widened; either way the call is the one on the
+    widened state, rounded once.  Sums over d_k = 128 products in fp32 may come in another order: 128 x 2^-24 of the largest, after
+    which a bf16 result may fall to its neighbour, 2^-7 of itself."""
+    from paper_2606_08804_b200 import binding as qd
+    g = torch.Generator(device="cuda").manual_seed(17 + dk + dv + S)
+    rnd = lambda *shape: torch.randn(*shape, device="cuda", generator=g)
+    B, H, bf = 3, 5, torch.bfloat16
+    t = [rnd(B, S, H, d).to(bf) * (1.0 if raw else d ** -0.5) for d in (dk, dk, dv)]
+    t += [x.to(bf) if raw else torch.sigmoid(x).to(bf) for x in (rnd(B, S, H), rnd(B, S, H), rnd(B, S, H))]
+    state = (rnd(B, H, dk, dv) * 0.1).to(bf)
+    wide = state.float()
+    o = qd.recurrent_steps(*t, state, logits=raw, norm_qk=raw)
+    ow = qd.recurrent_steps(*t, wide, logits=raw, norm_qk=raw)
+    for got, want in ((o, ow.float()), (state, wide)):
+        tol = 2.0 ** -7 * want.abs() + 128 * 2.0 ** -24 * want.abs().max()
+        assert ((got.float() - want).abs() <= tol).all()
