@@ -63,8 +63,9 @@ struct TcLayout {
 TcLayout tc_layout(const qd_shape& s);
 bool tc_supported(const qd_shape& s);
 int chain_rows(uint64_t BH);      // d_v rows of a state that one CTA of the state chains owns: 128 or 64
-// Rows per sequence in the tensor-core workspace: T rounded up to a whole number of chunk PAIRS (the preparation kernel
-// takes two chunks at a time).  The rows past T behave as tokens with beta = 0, alpha = 1, q = k = v = 0, which leave the
+// Rows per sequence in the tensor-core workspace: T rounded up to a multiple of 128, of which ceil(T / 64) chunks are walked (so that
+// the sizes of a workspace, and what a call with a given one accepts, stay as they were when chunks were prepared in pairs).  The rows
+// past T of the last chunk behave as tokens with beta = 0, alpha = 1, q = k = v = 0, which leave the
 // recurrence of Section 3.3.1 untouched; TMA supplies the zeros and drops the stores.
 inline int split_padded_T(const qd_shape& s) { return (s.T + kChunk - 1) / kChunk * kChunk; }   // fp32 path: whole chunks
 inline int tc_padded_T(const qd_shape& s) { return (s.T + 2 * kChunk - 1) / (2 * kChunk) * (2 * kChunk); }

@@ -41,7 +41,7 @@ struct BwdMaps {               // boxes of 64 rows for token tiles, 128 for tile
     CUtensorMap Q, K, V, dO, Mt, P, Dt, dDt, Hs, dHs, Wt, Qg, dHs_store, dDt_store, dQ, dK, dV;
 };
 struct ChainBwdParams {
-    int Tp, H, N;              // Tp = 64 N rows per sequence in the workspace
+    int Tp, H, N, Ns;          // N chunks per sequence; Tp = 64 Ns >= 64 N rows per sequence in the workspace
     int dhT_early;             // the kernel before this one in the stream is the library's own: dhT is older than it
     const float* rk;           // non-null (QD_NORM_QK): 1/|k_t| per workspace row, folded into the per-token scale
     const float* g;
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
             grid_dep_wait();
             if (blockIdx.x == 0) *p.next = 0;
             for (int it = 0; it < p.N; ++it) {
-                const int y = (int)(((size_t)bh * p.N + (p.N - 1 - it)) * D) + v0, sb = it & two;
+                const int y = (int)(((size_t)bh * p.Ns + (p.N - 1 - it)) * D) + v0, sb = it & two;
                 unsigned char *sdH = stg + sb * bytesS, *sdD = sdH + rows * 256;
                 wait(&bar.ht[sb], (it >> two) & 1);       // gradient w.r.t. the exit state (rows = d_v, columns = d_k) is staged
                 tma_store_2d(&mapdHs, sdH, 0, y);
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         };
         auto load_w = [&](int it) {
             mbar_expect_tx(&bar.w[it & 1], 16384);
-            tma_load_2d(smem + offW + (it & 1) * 16384, &mapWt, 0, (int)(((size_t)bh * p.N + (p.N - 1 - it)) * D), &bar.w[it & 1]);
+            tma_load_2d(smem + offW + (it & 1) * 16384, &mapWt, 0, (int)(((size_t)bh * p.Ns + (p.N - 1 - it)) * D), &bar.w[it & 1]);
         };
         fetch_g(0);
         for (int it = 0; it < kDeepK && it < p.N; ++it) {
@@ -364,7 +364,7 @@ struct ChunkBwdParams {
     int logits;                // beta, alpha, lambda are logits of sigmoid gates; their gradients are taken w.r.t. the logits
     const float* rqk;          // QD_NORM_QK: 1/|q_t| per workspace row, then (BH*Tp further) 1/|k_t|
     int group;                 // sequences per group of work items
-    int T, Tp, H, N, BH, total;   // T tokens per sequence, Tp = 64 N rows per sequence in the workspace; total = BH*N chunks
+    int T, Tp, H, N, Ns, BH, total;   // T tokens in N chunks per sequence, Tp = 64 Ns >= 64 N rows per sequence in the workspace; total = BH*N
     const bf16 *beta, *alpha, *lam;
     const float* g;
     float *dbeta, *dalpha, *dlam;
@@ -483,12 +483,12 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     auto put = [&](int it, Item x) { item[it & 3].x = x.n; item[it & 3].y = x.bh; };
     auto issue_dd = [&](Item x) {                 // dDelta^T on its own: the first product waits for it
         mbar_expect_tx(&bar.d, 16384);
-        tma_load_2d(sm + odDt, &m.dDt, 0, (int)(((size_t)x.bh * p.N + x.n) * D), &bar.d);
+        tma_load_2d(sm + odDt, &m.dDt, 0, (int)(((size_t)x.bh * p.Ns + x.n) * D), &bar.d);
     };
     auto issue_early = [&](Item x) {
         const int b_ = x.bh / p.H, hh_ = x.bh % p.H;
         const int yt = (int)((size_t)x.bh * p.Tp + (size_t)x.n * C);
-        const int yc = (int)(((size_t)x.bh * p.N + x.n) * D);
+        const int yc = (int)(((size_t)x.bh * p.Ns + x.n) * D);
         mbar_expect_tx(&bar.load, kBwdEarlyBytes);
         tma_load_2d(sm + oMt, &m.Mt, 0, yt, &bar.load);
         for (int blk = 0; blk < 2; ++blk)         // token rows past the end of the sequence arrive as zeros
@@ -499,12 +499,12 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         tma_load_2d(sm + oP, &m.P, 0, yt, &bar.load);
     };
     auto issue_h = [&](Item x) {                  // half of bar.h
-        const int yc = (int)(((size_t)x.bh * p.N + x.n) * D);
+        const int yc = (int)(((size_t)x.bh * p.Ns + x.n) * D);
         mbar_expect_tx(&bar.h, 2 * 32768);
         for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + oH + blk * 16384, &m.Hs, blk * 64, yc, &bar.h);
     };
     auto issue_dh = [&](Item x) {                 // the other half
-        const int yc = (int)(((size_t)x.bh * p.N + x.n) * D);
+        const int yc = (int)(((size_t)x.bh * p.Ns + x.n) * D);
         for (int blk = 0; blk < 2; ++blk) tma_load_2d(sm + odH + blk * 16384, &m.dHs, blk * 64, yc, &bar.h);
     };
     auto issue_qk = [&](Item x) {
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     // of the tiles of a chunk, those that are waited for most into L2 only, a chunk time ahead
     auto prefetch_late = [&](Item x) {
         const int b_ = x.bh / p.H, hh_ = x.bh % p.H;
-        const int yc = (int)(((size_t)x.bh * p.N + x.n) * D);
+        const int yc = (int)(((size_t)x.bh * p.Ns + x.n) * D);
         for (int blk = 0; blk < 2; ++blk) {
             tma_prefetch_3d(&m.Q, hh_ * D + blk * 64, x.n * C, b_);
             tma_prefetch_3d(&m.K, hh_ * D + blk * 64, x.n * C, b_);
@@ -1127,19 +1127,19 @@ cudaError_t set_smem(K kern, size_t bytes) { return set_max_smem_once(reinterpre
 cudaError_t tc_chain_bwd(const ChunkArgs& a) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
-    const uint64_t BH = (uint64_t)s.B * s.H, N = Tp / kChunk;
+    const uint64_t BH = (uint64_t)s.B * s.H, Ns = Tp / kChunk, N = (s.T + kChunk - 1) / kChunk;
     const int rows = chain_rows(BH);
     CUtensorMap mWt, mdO, mQg, mK, mP, mdHs, mdDt;
-    if (!make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, BH * N * D, 128, 128) ||
+    if (!make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, BH * Ns * D, 128, 128) ||
         !make_tmap_tokens(&mdO, a.dO, s.B, s.T, s.H, D, 64) ||
         !make_tmap_bf16_2d(&mQg, a.ws + a.TL.Qg, D, BH * Tp, D * 2, 64) ||
         !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 64) ||
         !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, BH * Tp, 128, 64) ||
-        !make_tmap_bf16_2d(&mdHs, a.ws + a.TL.dhsT, D, BH * N * D, D * 2, rows) ||
-        !make_tmap_bf16_2d(&mdDt, a.ws + a.TL.dDt, 64, BH * N * D, 128, rows))
+        !make_tmap_bf16_2d(&mdHs, a.ws + a.TL.dhsT, D, BH * Ns * D, D * 2, rows) ||
+        !make_tmap_bf16_2d(&mdDt, a.ws + a.TL.dDt, 64, BH * Ns * D, 128, rows))
         return cudaErrorInvalidValue;
     ChainBwdParams p{};
-    p.Tp = Tp; p.H = s.H; p.N = (int)N;
+    p.Tp = Tp; p.H = s.H; p.N = (int)N; p.Ns = (int)Ns;
     p.dhT_early = a.own_predecessor ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.g = (const float*)(a.ws + a.TL.g);
@@ -1156,7 +1156,7 @@ cudaError_t tc_chain_bwd(const ChunkArgs& a) {
 cudaError_t tc_chunk_bwd(const ChunkArgs& a) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
-    const uint64_t BH = (uint64_t)s.B * s.H, N = Tp / kChunk;
+    const uint64_t BH = (uint64_t)s.B * s.H, Ns = Tp / kChunk, N = (s.T + kChunk - 1) / kChunk;
     ChunkBwdMaps m;
     if (!make_tmap_tokens(&m.dQ, a.dq, s.B, s.T, s.H, D, 64) ||
         !make_tmap_tokens(&m.dK, a.dk, s.B, s.T, s.H, D, 64) ||
@@ -1167,13 +1167,13 @@ cudaError_t tc_chunk_bwd(const ChunkArgs& a) {
         !make_tmap_tokens(&m.dO, a.dO, s.B, s.T, s.H, D, 64) ||
         !make_tmap_bf16_2d(&m.Mt, a.ws + a.TL.Mt, 64, BH * Tp, 128, 64) ||
         !make_tmap_bf16_2d(&m.P, a.ws + a.TL.P, 64, BH * Tp, 128, 64) ||
-        !make_tmap_bf16_2d(&m.Dt, a.ws + a.TL.Dt, 64, BH * N * D, 128, 128) ||
-        !make_tmap_bf16_2d(&m.dDt, a.ws + a.TL.dDt, 64, BH * N * D, 128, 128) ||
-        !make_tmap_bf16_2d(&m.Hs, a.ws + a.TL.hsT, D, BH * N * D, D * 2, 128) ||
-        !make_tmap_bf16_2d(&m.dHs, a.ws + a.TL.dhsT, D, BH * N * D, D * 2, 128))
+        !make_tmap_bf16_2d(&m.Dt, a.ws + a.TL.Dt, 64, BH * Ns * D, 128, 128) ||
+        !make_tmap_bf16_2d(&m.dDt, a.ws + a.TL.dDt, 64, BH * Ns * D, 128, 128) ||
+        !make_tmap_bf16_2d(&m.Hs, a.ws + a.TL.hsT, D, BH * Ns * D, D * 2, 128) ||
+        !make_tmap_bf16_2d(&m.dHs, a.ws + a.TL.dhsT, D, BH * Ns * D, D * 2, 128))
         return cudaErrorInvalidValue;
     ChunkBwdParams p{};
-    p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = (int)N; p.BH = (int)BH; p.total = (int)(BH * N);
+    p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = (int)N; p.Ns = (int)Ns; p.BH = (int)BH; p.total = (int)(BH * N);
     p.group = (int)std::min<uint64_t>(BH, 64);
     p.beta = (const bf16*)a.beta; p.alpha = (const bf16*)a.alpha; p.lam = (const bf16*)a.lam;
     p.g = (const float*)(a.ws + a.TL.g);

@@ -28,7 +28,7 @@ constexpr int D = 128;         // d_k = d_v
 // =================================================================================================
 struct PrepParams {
     float* rqk;                // non-null: L2-normalise q and k here; [0, BH*Tp) <- 1/|q_t|, [BH*Tp, 2 BH*Tp) <- 1/|k_t|
-    int T, Tp, H, N, BH;       // T tokens per sequence; the workspace holds Tp = 64 N >= T rows per sequence
+    int T, Tp, H, N, Ns, BH;   // T tokens in N chunks per sequence; the workspace holds Tp = 64 Ns >= 64 N rows per sequence
     const bf16 *beta, *alpha, *lam;
     float* g;
     bf16* Qg;
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
         wait(&bar_o);
         tc_fence_after();
         if (lead) {
-            const int y = (int)(((size_t)bh * p.N + n) * D);
+            const int y = (int)(((size_t)bh * p.Ns + n) * D);
             tma_store_2d(&mapUt, sX, 0, y);
             tma_store_2d(&mapWt, sQ, 0, y);
             tma_store_2d(&mapP, sK, 0, (int)wtok0);
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
             for (int e = 0; e < 8; ++e) { a[e] = m[k][e] * beta; bq[e] = m[k][e] * bg; }
             sts128(sK + sw128_chunk(j, kb), pack8(a));
             sts128(sK + 8192 + sw128_chunk(j, kb), pack8(bq));
-            if (p.Mt) *reinterpret_cast<uint4*>(p.Mt + (((size_t)bh * p.N + n) * C + j) * C + kb * 8) = pack8(m[k]);
+            if (p.Mt) *reinterpret_cast<uint4*>(p.Mt + (((size_t)bh * p.Ns + n) * C + j) * C + kb * 8) = pack8(m[k]);
         }
     }
     fence_proxy_async();
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
 
 // =================================================================================================
 struct ChainParams {
-    int Tp, H, N;              // Tp = 64 N rows per sequence in the workspace
+    int Tp, H, N, Ns;          // N chunks per sequence; Tp = 64 Ns >= 64 N rows per sequence in the workspace
     const float* g;
     const float* h0;
     float* hT;
@@ -667,7 +667,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             grid_dep_wait();
             int s = 0;
             for (int n = 0; n < p.N; ++n) {
-                const int y = (int)(((size_t)bh * p.N + n) * D) + v0;
+                const int y = (int)(((size_t)bh * p.Ns + n) * D) + v0;
                 const int sb = n & two;
                 wait(&bar_ht[sb], (n >> two) & 1);        // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
                 tma_store_2d(&mapHs, sHs + sb * 16384, 0, y);
@@ -709,7 +709,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             if (ln == 0) sG[s][64] = __expf(gc);
             __syncwarp();
             if (lead) {
-                const int yc = (int)(((size_t)bh * p.N + n) * D);
+                const int yc = (int)(((size_t)bh * p.Ns + n) * D);
                 mbar_expect_tx(&bar_la[s], 16384 + rows * 128);
                 tma_load_2d(smem + s * kStageA, &mapWt, 0, yc, &bar_la[s]);
                 tma_load_2d(smem + s * kStageA + 16384, &mapUt, 0, yc + v0, &bar_la[s]);
@@ -805,7 +805,7 @@ cudaError_t tc_prep(const ChunkArgs& a) {
         !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, (uint64_t)s.B * s.H * Tp, 128, 64))
         return cudaErrorInvalidValue;
     PrepParams p{};
-    p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = Tp / kChunk; p.BH = s.B * s.H;
+    p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = (s.T + kChunk - 1) / kChunk; p.Ns = Tp / kChunk; p.BH = s.B * s.H;
     p.rqk = a.norm ? (float*)(a.ws + a.TL.rqk) : nullptr;
     p.beta = (const bf16*)a.beta; p.alpha = (const bf16*)a.alpha; p.lam = (const bf16*)a.lam;
     p.g = (float*)(a.ws + a.TL.g);
@@ -823,20 +823,20 @@ cudaError_t tc_prep(const ChunkArgs& a) {
 cudaError_t tc_chain_fwd(const ChunkArgs& a) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
-    const uint64_t BH = (uint64_t)s.B * s.H, N = Tp / kChunk;
+    const uint64_t BH = (uint64_t)s.B * s.H, Ns = Tp / kChunk, N = (s.T + kChunk - 1) / kChunk;
     const int rows = chain_rows(BH);
     CUtensorMap mWt, mUt, mQg, mK, mP, mHs, mDt, mO;
-    if (!make_tmap_bf16_2d(&mHs, a.ws + a.TL.hsT, D, BH * N * D, D * 2, rows) ||
-        !make_tmap_bf16_2d(&mDt, a.ws + a.TL.Dt, 64, BH * N * D, 128, rows) ||
+    if (!make_tmap_bf16_2d(&mHs, a.ws + a.TL.hsT, D, BH * Ns * D, D * 2, rows) ||
+        !make_tmap_bf16_2d(&mDt, a.ws + a.TL.Dt, 64, BH * Ns * D, 128, rows) ||
         !make_tmap_tokens(&mO, a.o, s.B, s.T, s.H, D, 32) ||
-        !make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, BH * N * D, 128, 128) ||
-        !make_tmap_bf16_2d(&mUt, a.ws + a.TL.Ut, 64, BH * N * D, 128, rows) ||
+        !make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, BH * Ns * D, 128, 128) ||
+        !make_tmap_bf16_2d(&mUt, a.ws + a.TL.Ut, 64, BH * Ns * D, 128, rows) ||
         !make_tmap_bf16_2d(&mQg, a.ws + a.TL.Qg, D, BH * Tp, D * 2, 64) ||
         !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 64) ||
         !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, BH * Tp, 128, 64))
         return cudaErrorInvalidValue;
     ChainParams p{};
-    p.Tp = Tp; p.H = s.H; p.N = (int)N;
+    p.Tp = Tp; p.H = s.H; p.N = (int)N; p.Ns = (int)Ns;
     p.g = (const float*)(a.ws + a.TL.g);
     p.h0 = a.h0; p.hT = a.hT;
     p.save = a.save ? 1 : 0;
