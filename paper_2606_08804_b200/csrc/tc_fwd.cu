@@ -403,7 +403,6 @@ struct ChainParams {
     const float* g;
     const float* h0;
     float* hT;
-    int save;                  // also store, per chunk, the bf16 entry state (mapHs) and Delta^T (mapDt)
     int scaled;                // 0: no forget gate and no key normalisation: every per-token factor on Delta is 1
     const float* rk;           // non-null (QD_NORM_QK): 1/|k_t| per workspace row; the keys are read un-normalised and
                                // the factor is folded into the per-token scale of Delta
@@ -437,9 +436,11 @@ constexpr int kBarH = 1, kBarD = 2, kBarOut = 3;
 //    backward 1300 more.  (Ordinary stores, by one or two warps from the tiles or by the epilogue from its registers, were
 //    slower: 4500 - 5000 cycles per chunk.)  So with few heads the d_v rows of a head, which evolve independently, are shared by
 //    two CTAs (ROWS = 64): each loads what both need, but only its half of Ut, and stores its half of everything.
+// SAVE: also store, per chunk, the bf16 entry state (mapHs) and Delta^T (mapDt).  Compile-time: with a flag prompts of 4 sequences
+// of 64 chunks took 80.2 us, so 77.3.
 // Compute warpgroup w owns tokens [16w, 16w+16) of the 64-column accumulators and d_k columns
 // [32w, 32w+32) of the state; thread l of a warpgroup owns TMEM lane l = d_v index.
-template <int ROWS>
+template <int ROWS, bool SAVE>
 __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_constant__ CUtensorMap mapWt,
                                                                 const __grid_constant__ CUtensorMap mapUt,
                                                                 const __grid_constant__ CUtensorMap mapQg,
@@ -530,7 +531,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             staged(&bar_ht[sb]);
         };
         put_h();
-        if (p.save) save_h(0);
+        if (SAVE) save_h(0);
         int pending = 0;                  // barriers of the MMA warp that a warp which gives up has not been to
         int s = 0;
         for (int n = 0; n < p.N; ++n) {
@@ -562,7 +563,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                 tmem_st_wait();
                 tc_fence_before();
                 nb_arrive(kBarD, nb);
-                if (p.save) {
+                if (SAVE) {
                     sts128(ut + sw128_chunk(l, wg * 2), make_uint4(r[0], r[1], r[2], r[3]));
                     sts128(ut + sw128_chunk(l, wg * 2 + 1), make_uint4(r[4], r[5], r[6], r[7]));
                     staged(&bar_dt[s]);
@@ -579,7 +580,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                 for (int i = 0; i < 32; ++i) h[i] = fmaf(gamC, h[i], v[i]);
             }
             put_h();
-            if (p.save && n + 1 < p.N) save_h(n + 1);
+            if (SAVE && n + 1 < p.N) save_h(n + 1);
             if (++s == kDeepA) s = 0;
         }
         // a wait has expired: keep step with the MMA warp, which comes to every one of them (odd counts: H is next)
@@ -663,7 +664,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     } else if (warp == kMmaWarp + 1) {
         // ---------------------------------- saving warp ----------------------------------
         // apart from the loads, which would otherwise wait for what these wait for
-        if ((tid & 31) == 0 && p.save) {
+        if ((tid & 31) == 0 && SAVE) {
             grid_dep_wait();
             int s = 0;
             for (int n = 0; n < p.N; ++n) {
@@ -738,7 +739,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             if (lead) {
                 wait(&bar_e[n & 1], (n >> 1) & 1);        // every product of chunk n has finished: refill its buffers
                 if (n + 2 < p.N && !s_abort) load_b(n + 2);
-                if (more && p.save) wait(&bar_df[s], (n / kDeepA) & 1);
+                if (more && SAVE) wait(&bar_df[s], (n / kDeepA) & 1);
             }
             more = __shfl_sync(0xffffffffu, more && !s_abort, 0);     // one answer for the warp
             if (more) load_a(n + kDeepA, s);
@@ -839,11 +840,11 @@ cudaError_t tc_chain_fwd(const ChunkArgs& a) {
     p.Tp = Tp; p.H = s.H; p.N = (int)N; p.Ns = (int)Ns;
     p.g = (const float*)(a.ws + a.TL.g);
     p.h0 = a.h0; p.hT = a.hT;
-    p.save = a.save ? 1 : 0;
     p.scaled = (a.alpha || a.norm) ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
-    const auto kern = rows == D ? k_tc_chain_fwd<D> : k_tc_chain_fwd<D / 2>;
+    const auto kern = rows == D ? (a.save ? k_tc_chain_fwd<D, true> : k_tc_chain_fwd<D, false>)
+                              : (a.save ? k_tc_chain_fwd<D / 2, true> : k_tc_chain_fwd<D / 2, false>);
     cudaError_t e = set_smem(kern, kChainSmem);
     if (e != cudaSuccess) return e;
     return launch_overlapped(kern, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream,
