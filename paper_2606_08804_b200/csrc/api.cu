@@ -85,6 +85,14 @@ template <class F> static cudaError_t timed(int stage, cudaStream_t s, F f) {
     return f();
 }
 
+// The two kernels of the forward, beside each other in parts where that is faster; one after the other when they are timed.
+static cudaError_t tc_forward(const ChunkArgs& a) {
+    const int parts = g_profile ? 1 : tc_fwd_parts(a);
+    if (parts > 1) return tc_fwd(a, parts);
+    const cudaError_t e = timed(ST_PREP, a.stream, [&] { return tc_prep(a); });
+    return e != cudaSuccess ? e : timed(ST_CHAIN_FWD, a.stream, [&] { return tc_chain_fwd(a); });
+}
+
 }  // namespace qd
 
 using namespace qd;
@@ -132,8 +140,7 @@ int qdelta_chunk_fwd(const qd_shape* shape, const void* q, const void* k, const 
     a.stream = (cudaStream_t)stream;
     if (tc_supported(*shape)) {
         a.TL = tc_layout(*shape);
-        if (timed(ST_PREP, a.stream, [&] { return tc_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
-        if (timed(ST_CHAIN_FWD, a.stream, [&] { return tc_chain_fwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
+        if (tc_forward(a) != cudaSuccess) return QD_ERR_CUDA;
         return QD_OK;
     }
     if (timed(ST_PREP, a.stream, [&] { return split_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
@@ -178,8 +185,7 @@ int qdelta_chunk_bwd(const qd_shape* shape, const void* q, const void* k, const 
             // the reverse chain overwrites afterwards
             a.o = a.ws + a.TL.dDt;
             a.hT = nullptr;
-            if (timed(ST_PREP, a.stream, [&] { return tc_prep(a); }) != cudaSuccess) return QD_ERR_CUDA;
-            if (timed(ST_CHAIN_FWD, a.stream, [&] { return tc_chain_fwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
+            if (tc_forward(a) != cudaSuccess) return QD_ERR_CUDA;
             a.own_predecessor = true;      // the reverse chain follows this library's forward chain in the stream
         }
         if (timed(ST_CHAIN_BWD, a.stream, [&] { return tc_chain_bwd(a); }) != cudaSuccess) return QD_ERR_CUDA;

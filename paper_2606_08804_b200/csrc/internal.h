@@ -117,6 +117,8 @@ cudaError_t split_chunk_bwd(const ChunkArgs& a);   // dq, dk, dv, dbeta, dalpha,
 // tcgen05 path
 cudaError_t tc_prep(const ChunkArgs& a);
 cudaError_t tc_chain_fwd(const ChunkArgs& a);
+int tc_fwd_parts(const ChunkArgs& a);                        // in how many parts tc_fwd takes a sequence; 1: tc_prep and tc_chain_fwd
+cudaError_t tc_fwd(const ChunkArgs& a, int parts);
 cudaError_t tc_chain_bwd(const ChunkArgs& a);
 cudaError_t tc_chunk_bwd(const ChunkArgs& a);
 

@@ -11,6 +11,7 @@
 //                   everything transposed so that d_v is the MMA M dimension:
 //                     Delta^T = Ut - h^T Wt            O^T = h^T Qg^T + Delta^T P^T
 //                     h^T <- gamma_C h^T + (Delta diag(gamma_C/gamma))^T K
+// With few long sequences the two run beside each other, part by part (tc_fwd_parts).
 // All waits are bounded; on expiry the CTA records QD_ERR_TIMEOUT in the workspace status word,
 // releases its tensor memory and returns.
 #include "internal.h"
@@ -28,7 +29,9 @@ constexpr int D = 128;         // d_k = d_v
 // =================================================================================================
 struct PrepParams {
     float* rqk;                // non-null: L2-normalise q and k here; [0, BH*Tp) <- 1/|q_t|, [BH*Tp, 2 BH*Tp) <- 1/|k_t|
-    int T, Tp, H, N, Ns, BH;   // T tokens in N chunks per sequence; the workspace holds Tp = 64 Ns >= 64 N rows per sequence
+    int T, Tp, H, N, Ns, BH;   // T tokens per sequence, of which the N chunks from n0 on; the workspace holds Tp = 64 Ns rows per sequence
+    int n0;
+    int beside;                // 1: runs beside the forward chain launched before it (see tc_fwd_parts), so it waits for that at its end
     const bf16 *beta, *alpha, *lam;
     float* g;
     bf16* Qg;
@@ -171,7 +174,7 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
     const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     // CTAs are numbered chunk-major, last chunk first: the forward chain, which starts with chunk 0 of every sequence,
     // then finds the tiles written last (and K, read last) still in L2
-    const int n = p.N - 1 - (int)blockIdx.x / p.BH, bh = (int)blockIdx.x % p.BH;
+    const int n = p.n0 + p.N - 1 - (int)blockIdx.x / p.BH, bh = (int)blockIdx.x % p.BH;
     const int b = bh / p.H, hh = bh % p.H;
     const int t0 = n * C;                                            // first token of the chunk
     const size_t wtok0 = (size_t)bh * p.Tp + (size_t)t0;             // first row in the workspace's [BH*Tp] view
@@ -189,7 +192,7 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
     const uint32_t tb = uniform(tmem_slot), T0 = tb, T1 = tb + 64;
     auto wait = [&](uint64_t* bar) { return mbar_try_wait(bar, 0) || wait_on(bar, 0, s_abort, p.status); };
 
-    grid_dep_wait();                  // set up while the kernel before drains; nothing is read or written before it has completed
+    if (!p.beside) grid_dep_wait();   // set up while the kernel before drains; nothing is read or written before it has completed
     grid_dep_launch();                // the kernel after this one may set itself up while the last CTAs of this one run
     if (warp == 4) {
         // ---------------------------------- copies and products ----------------------------------
@@ -198,7 +201,7 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
         const bool lead = lane == 0;
         if (lead) {
             // the call's status word starts at zero: the first CTA to start clears it, a second before any wait can expire
-            if (blockIdx.x == 0) *p.status = 0;
+            if (blockIdx.x == 0 && !p.beside) *p.status = 0;
             mbar_expect_tx(&bar_qk, 32768);
             for (int blk = 0; blk < 2; ++blk) {          // rows at t >= T arrive as zeros
                 tma_load_3d(sQ + blk * 8192, &mapQ, hh * D + blk * 64, t0, b, &bar_qk);
@@ -238,6 +241,7 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
         }
         __syncwarp();
         tmem_dealloc(tb, 128);
+        if (blockIdx.x == 0) grid_dep_wait();            // when this kernel has completed, so has the one before it
         return;
     }
     // ---------------------------------- arithmetic ----------------------------------
@@ -399,7 +403,9 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
 
 // =================================================================================================
 struct ChainParams {
-    int Tp, H, N, Ns;          // N chunks per sequence; Tp = 64 Ns >= 64 N rows per sequence in the workspace
+    int Tp, H, N, Ns;          // N chunks of a sequence, from n0 on; Tp = 64 Ns rows per sequence in the workspace
+    int n0;
+    int h0_late;               // 1: h0 is what the chain of the chunks before has left
     const float* g;
     const float* h0;
     float* hT;
@@ -490,17 +496,20 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
 
     // bounded wait; once any wait has expired every later wait returns at once (the kernel drains)
     auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_try_wait(bar, parity) || wait_on(bar, parity, s_abort, p.status); };
-    const float* gseq = p.g + (size_t)bh * p.Tp;
+    const int tok0 = p.n0 * C;                                       // first token; rows and tiles of the workspace start at
+    const size_t row0 = (size_t)bh * p.Tp + tok0, tile0 = (size_t)bh * p.Ns + p.n0;
+    const float* gseq = p.g + row0;
 
     if (warp < kMmaWarp && wq >= nwq) {
         // lanes without a row: straight to the end
     } else if (warp < kOutWarp) {
         // ---------------------------------- compute warps ----------------------------------
         float h[32];      // h^T[j = l][32 wg .. 32 wg + 31], fp32
+        if (p.h0_late) grid_dep_wait();
         if (p.h0) {
             const float* src = p.h0 + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) h[i] = src[(size_t)i * D];
+            for (int i = 0; i < 32; ++i) h[i] = __ldcg(src + (size_t)i * D);      // not from L1: it may be new
         } else {
 #pragma unroll
             for (int i = 0; i < 32; ++i) h[i] = 0.f;
@@ -620,8 +629,8 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                 fence_proxy_async();
                 nb_sync(kBarOut, rows);
                 if (first) {                              // rows past the end of the sequence are skipped
-                    tma_store_3d(&mapO, sO, hh * D + v0, n * C + half * 32, b);
-                    if (rows == D) tma_store_3d(&mapO, sO + 4096, hh * D + 64, n * C + half * 32, b);
+                    tma_store_3d(&mapO, sO, hh * D + v0, tok0 + n * C + half * 32, b);
+                    if (rows == D) tma_store_3d(&mapO, sO + 4096, hh * D + 64, tok0 + n * C + half * 32, b);
                     tma_store_commit();
                 }
             }
@@ -668,7 +677,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             grid_dep_wait();
             int s = 0;
             for (int n = 0; n < p.N; ++n) {
-                const int y = (int)(((size_t)bh * p.Ns + n) * D) + v0;
+                const int y = (int)((tile0 + n) * D) + v0;
                 const int sb = n & two;
                 wait(&bar_ht[sb], (n >> two) & 1);        // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
                 tma_store_2d(&mapHs, sHs + sb * 16384, 0, y);
@@ -696,7 +705,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         grid_dep_wait();                  // the tiles and the log-decays read below are written by the prep kernel
         grid_dep_launch();
         const int ln = tid & 31;
-        const float* rkseq = p.rk ? p.rk + (size_t)bh * p.Tp : nullptr;
+        const float* rkseq = p.rk ? p.rk + row0 : nullptr;
         // log-decays (and 1/|k|) of the next chunk to be loaded, fetched ahead
         float g0, g1, gc, r0 = 1.f, r1 = 1.f;
         auto fetch_g = [&](int n) {
@@ -710,7 +719,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             if (ln == 0) sG[s][64] = __expf(gc);
             __syncwarp();
             if (lead) {
-                const int yc = (int)(((size_t)bh * p.Ns + n) * D);
+                const int yc = (int)((tile0 + n) * D);
                 mbar_expect_tx(&bar_la[s], 16384 + rows * 128);
                 tma_load_2d(smem + s * kStageA, &mapWt, 0, yc, &bar_la[s]);
                 tma_load_2d(smem + s * kStageA + 16384, &mapUt, 0, yc + v0, &bar_la[s]);
@@ -720,12 +729,12 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         auto load_b = [&](int n) {                       // by the leading lane
             unsigned char* st = smem + kOffB + (n & 1) * kStageB;
             uint64_t* bar = &bar_lb[n & 1];
-            const int yt = (int)((size_t)bh * p.Tp + (size_t)n * C);
+            const int yt = (int)(row0 + (size_t)n * C);
             mbar_expect_tx(bar, kStageB);
             tma_load_2d(st, &mapQg, 0, yt, bar);
             tma_load_2d(st + 8192, &mapQg, 64, yt, bar);
-            tma_load_3d(st + 16384, &mapK, hh * D, n * C, b, bar);
-            tma_load_3d(st + 16384 + 8192, &mapK, hh * D + 64, n * C, b, bar);
+            tma_load_3d(st + 16384, &mapK, hh * D, tok0 + n * C, b, bar);
+            tma_load_3d(st + 16384 + 8192, &mapK, hh * D + 64, tok0 + n * C, b, bar);
             tma_load_2d(st + 32768, &mapP, 0, yt, bar);
         };
         fetch_g(0);
@@ -794,18 +803,23 @@ TcLayout tc_layout(const qd_shape& s) {
     return L;
 }
 
-cudaError_t tc_prep(const ChunkArgs& a) {
+namespace {
+
+struct PrepCall { CUtensorMap mQ, mK, mV, mUt, mWt, mP; PrepParams p; };
+struct ChainCall { CUtensorMap mWt, mUt, mQg, mK, mP, mHs, mDt, mO; ChainParams p; };
+
+bool setup(const ChunkArgs& a, PrepCall& c) {
     const qd_shape& s = a.s;
-    CUtensorMap mQ, mK, mV, mUt, mWt, mP;
     const int Tp = tc_padded_T(s);
     const uint64_t trows = (uint64_t)s.B * s.H * (Tp / kChunk) * D;          // rows of the [chunk][d][64] tiles
-    if (!make_tmap_tokens(&mQ, a.q, s.B, s.T, s.H, D, 64) || !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_tokens(&mV, a.v, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_bf16_2d(&mUt, a.ws + a.TL.Ut, 64, trows, 128, 128) ||
-        !make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, trows, 128, 128) ||
-        !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, (uint64_t)s.B * s.H * Tp, 128, 64))
-        return cudaErrorInvalidValue;
-    PrepParams p{};
+    if (!make_tmap_tokens(&c.mQ, a.q, s.B, s.T, s.H, D, 64) || !make_tmap_tokens(&c.mK, a.k, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_tokens(&c.mV, a.v, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_bf16_2d(&c.mUt, a.ws + a.TL.Ut, 64, trows, 128, 128) ||
+        !make_tmap_bf16_2d(&c.mWt, a.ws + a.TL.Wt, 64, trows, 128, 128) ||
+        !make_tmap_bf16_2d(&c.mP, a.ws + a.TL.P, 64, (uint64_t)s.B * s.H * Tp, 128, 64))
+        return false;
+    PrepParams& p = c.p;
+    p = PrepParams{};
     p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = (s.T + kChunk - 1) / kChunk; p.Ns = Tp / kChunk; p.BH = s.B * s.H;
     p.rqk = a.norm ? (float*)(a.ws + a.TL.rqk) : nullptr;
     p.beta = (const bf16*)a.beta; p.alpha = (const bf16*)a.alpha; p.lam = (const bf16*)a.lam;
@@ -813,42 +827,102 @@ cudaError_t tc_prep(const ChunkArgs& a) {
     p.Qg = (bf16*)(a.ws + a.TL.Qg);
     p.Mt = a.save ? (bf16*)(a.ws + a.TL.Mt) : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
+    return true;
+}
+cudaError_t launch(const ChunkArgs& a, const PrepCall& c) {
     auto kern = a.norm ? (a.logits ? k_tc_prep<true, true> : k_tc_prep<true, false>)
                        : (a.logits ? k_tc_prep<false, true> : k_tc_prep<false, false>);
     cudaError_t e = set_smem(kern, kPrepSmem);
     if (e != cudaSuccess) return e;
-    const int grid = s.B * s.H * p.N;
-    return launch_overlapped(kern, dim3((unsigned)grid), dim3(kPrepThreads), kPrepSmem, a.stream, mQ, mK, mV, mUt, mWt, mP, p);
+    return launch_overlapped(kern, dim3((unsigned)(c.p.BH * c.p.N)), dim3(kPrepThreads), kPrepSmem, a.stream, c.mQ, c.mK, c.mV, c.mUt,
+                             c.mWt, c.mP, c.p);
 }
 
-cudaError_t tc_chain_fwd(const ChunkArgs& a) {
+bool setup(const ChunkArgs& a, ChainCall& c) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
     const uint64_t BH = (uint64_t)s.B * s.H, Ns = Tp / kChunk, N = (s.T + kChunk - 1) / kChunk;
     const int rows = chain_rows(BH);
-    CUtensorMap mWt, mUt, mQg, mK, mP, mHs, mDt, mO;
-    if (!make_tmap_bf16_2d(&mHs, a.ws + a.TL.hsT, D, BH * Ns * D, D * 2, rows) ||
-        !make_tmap_bf16_2d(&mDt, a.ws + a.TL.Dt, 64, BH * Ns * D, 128, rows) ||
-        !make_tmap_tokens(&mO, a.o, s.B, s.T, s.H, D, 32) ||
-        !make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, BH * Ns * D, 128, 128) ||
-        !make_tmap_bf16_2d(&mUt, a.ws + a.TL.Ut, 64, BH * Ns * D, 128, rows) ||
-        !make_tmap_bf16_2d(&mQg, a.ws + a.TL.Qg, D, BH * Tp, D * 2, 64) ||
-        !make_tmap_tokens(&mK, a.k, s.B, s.T, s.H, D, 64) ||
-        !make_tmap_bf16_2d(&mP, a.ws + a.TL.P, 64, BH * Tp, 128, 64))
-        return cudaErrorInvalidValue;
-    ChainParams p{};
+    if (!make_tmap_bf16_2d(&c.mHs, a.ws + a.TL.hsT, D, BH * Ns * D, D * 2, rows) ||
+        !make_tmap_bf16_2d(&c.mDt, a.ws + a.TL.Dt, 64, BH * Ns * D, 128, rows) ||
+        !make_tmap_tokens(&c.mO, a.o, s.B, s.T, s.H, D, 32) ||
+        !make_tmap_bf16_2d(&c.mWt, a.ws + a.TL.Wt, 64, BH * Ns * D, 128, 128) ||
+        !make_tmap_bf16_2d(&c.mUt, a.ws + a.TL.Ut, 64, BH * Ns * D, 128, rows) ||
+        !make_tmap_bf16_2d(&c.mQg, a.ws + a.TL.Qg, D, BH * Tp, D * 2, 64) ||
+        !make_tmap_tokens(&c.mK, a.k, s.B, s.T, s.H, D, 64) ||
+        !make_tmap_bf16_2d(&c.mP, a.ws + a.TL.P, 64, BH * Tp, 128, 64))
+        return false;
+    ChainParams& p = c.p;
+    p = ChainParams{};
     p.Tp = Tp; p.H = s.H; p.N = (int)N; p.Ns = (int)Ns;
     p.g = (const float*)(a.ws + a.TL.g);
     p.h0 = a.h0; p.hT = a.hT;
     p.scaled = (a.alpha || a.norm) ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
+    return true;
+}
+cudaError_t launch(const ChunkArgs& a, const ChainCall& c) {
+    const uint64_t BH = (uint64_t)a.s.B * a.s.H;
+    const int rows = chain_rows(BH);
     const auto kern = rows == D ? (a.save ? k_tc_chain_fwd<D, true> : k_tc_chain_fwd<D, false>)
-                              : (a.save ? k_tc_chain_fwd<D / 2, true> : k_tc_chain_fwd<D / 2, false>);
+                                : (a.save ? k_tc_chain_fwd<D / 2, true> : k_tc_chain_fwd<D / 2, false>);
     cudaError_t e = set_smem(kern, kChainSmem);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(kern, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream,
-                             mWt, mUt, mQg, mK, mP, mHs, mDt, mO, p);
+    return launch_overlapped(kern, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream, c.mWt, c.mUt, c.mQg,
+                             c.mK, c.mP, c.mHs, c.mDt, c.mO, c.p);
+}
+
+}  // namespace
+
+cudaError_t tc_prep(const ChunkArgs& a) {
+    PrepCall c;
+    return setup(a, c) ? launch(a, c) : cudaErrorInvalidValue;
+}
+
+cudaError_t tc_chain_fwd(const ChunkArgs& a) {
+    ChainCall c;
+    return setup(a, c) ? launch(a, c) : cudaErrorInvalidValue;
+}
+
+// With few sequences the forward chain, two CTAs to a sequence, leaves SMs idle for as long as its dependent chunks take.  A
+// sequence is then taken in parts, and the preparation of a part runs beside the chain of the part before it:
+//     prep 0, chain 0, prep 1, chain 1, ...
+// in one stream, by programmatic launch alone.  prep i + 1 may start when every CTA of chain i has begun its work, which it does
+// when prep i has completed (and so everything before that); it reads inputs and writes the workspace rows of its own chunks, so
+// it need not wait.  Its first CTA waits for chain i before it leaves, so when prep i + 1 has completed chain i has too, and
+// chain i + 1, which waits for prep i + 1, finds the state that chain i left: in h_T, or without one in the section that the
+// reverse chain fills later.  The state is passed on in fp32, so the results are those of one part, bit for bit.
+// Where: with up to 40 sequences (68 SMs idle), from 64 chunks and 1.7 loads of the GPU with preparations (1024 chunks) on.  One
+// part against two, us, without and with saves: 16 sequences of 64 chunks 97.7 / 91.3, 121 / 113; 32 of 64 122.8 / 117.4,
+// 148.8 / 133.4; 40 of 64 134.7 / 131.5, 160.6 / 151.4; but 44 of 64 141.6 / 142.2, 48 of 64 147.6 / 151.5, 64 of 256 728 / 741; 8 of 64 82.2 /
+// 82.2; 40 of 32 72.7 / 75.5.  A part costs 2 - 8 us, so three of them only from 256 chunks on: 32 of 512 965 / 792 / 755 for
+// one, two, three (1103 / 948 / 923), 16 of 512 714 / 644 / 621, 40 of 256 543 / 484 / 484; 32 of 64 122.8 / 117.4 / 120.9.
+int tc_fwd_parts(const ChunkArgs& a) {
+    const long long BH = (long long)a.s.B * a.s.H, N = (a.s.T + kChunk - 1) / kChunk;
+    if (BH > 40 || N < 64 || BH * N < 1024 || !(a.hT || a.save)) return 1;
+    return N < 256 ? 2 : 3;
+}
+
+cudaError_t tc_fwd(const ChunkArgs& a, int parts) {
+    PrepCall pc;
+    ChainCall cc;
+    if (!setup(a, pc) || !setup(a, cc)) return cudaErrorInvalidValue;
+    const int N = pc.p.N;
+    float* carry = a.hT ? a.hT : (float*)(a.ws + a.TL.dhsT);             // [BH][D][D]; dhsT has as much from two chunks on
+    for (int i = 0; i < parts; ++i) {
+        const int n0 = (int)((long long)N * i / parts), n1 = (int)((long long)N * (i + 1) / parts);
+        const bool last = i + 1 == parts;
+        pc.p.n0 = cc.p.n0 = n0;
+        pc.p.N = cc.p.N = n1 - n0;
+        pc.p.beside = cc.p.h0_late = i > 0;
+        if (i > 0) cc.p.h0 = carry;
+        cc.p.hT = last ? a.hT : carry;
+        cudaError_t e = launch(a, pc);
+        if (e == cudaSuccess) e = launch(a, cc);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace qd

@@ -46,3 +46,47 @@ def test_preparation_edges(T):
     d = gen.make_chunk_inputs(cfg)
     _fwd_check(cfg, d)
     _bwd_check(cfg, d, reuse=True)
+
+
+@pytest.mark.parametrize("B,H,T", [(1, 16, 64 * 64), (2, 20, 64 * 64 + 1), (1, 4, 64 * 256), (1, 1, 64 * 1024 - 63)])
+def test_forward_in_parts(B, H, T):
+    """Long, few sequences are taken in two or three parts, unless the kernels are timed one by one: the same bits either way, with
+    the state passed on through h_T and (none asked for) through the workspace, replayed from a graph, and close to the oracle."""
+    import torch
+
+    from gpu_util import dev_inputs
+    from paper_2606_08804_b200 import binding as qd
+
+    cfg = replace(gen.CONFIGS["cfg2"], B=B, H=H, T=T, regime="trained_like", seed=347)
+    d = gen.make_chunk_inputs(cfg)
+    _fwd_check(cfg, d, pairs=[(0, 0), (B - 1, H - 1)])
+    t = dev_inputs(d, cfg.dtype)
+    a = [t[n] for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")]
+    results = []
+
+    def call(logits, norm, save, hT):
+        o, h, ws = qd.chunk_fwd(*a, save_for_bwd=save, want_hT=hT, logits=logits, norm_qk=norm)
+        g = qd.chunk_bwd(*a, t["dO"], t["dhT"], workspace=ws, reuse_fwd=True, logits=logits, norm_qk=norm) if save else {}
+        r = qd.chunk_bwd(*a, t["dO"], t["dhT"], logits=logits, norm_qk=norm) if save else {}
+        assert qd.workspace_status(ws) == 0
+        return [x for x in (o, h, *g.values(), *r.values()) if x is not None]
+
+    cases = [(False, False, False, True), (False, False, True, True), (False, False, True, False), (True, True, True, True)]
+    for timed in (False, True):
+        qd.profile_enable(timed)
+        results.append([call(*c) for c in cases])
+    qd.profile_enable(False)
+    qd.profile_read(reset=True)
+    for c, x, y in zip(cases, *results):
+        assert len(x) == len(y) and all(torch.equal(i, j) for i, j in zip(x, y)), c
+
+    o, hT, ws = qd.chunk_fwd(*a, save_for_bwd=True)
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        qd.chunk_fwd(*a, save_for_bwd=True, workspace=ws, o=o, hT=hT)
+    o.zero_(), hT.zero_()
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(o, results[0][1][0]) and torch.equal(hT, results[0][1][1])
