@@ -92,6 +92,12 @@ static cudaError_t tc_forward(const ChunkArgs& a) {
     const cudaError_t e = timed(ST_PREP, a.stream, [&] { return tc_prep(a); });
     return e != cudaSuccess ? e : timed(ST_CHAIN_FWD, a.stream, [&] { return tc_chain_fwd(a); });
 }
+// The two of the backward, likewise.
+static cudaError_t tc_backward(const ChunkArgs& a) {
+    if (!g_profile && tc_bwd_halves(a)) return tc_bwd(a);
+    const cudaError_t e = timed(ST_CHAIN_BWD, a.stream, [&] { return tc_chain_bwd(a); });
+    return e != cudaSuccess ? e : timed(ST_CHUNK_BWD, a.stream, [&] { return tc_chunk_bwd(a); });
+}
 
 }  // namespace qd
 
@@ -188,9 +194,7 @@ int qdelta_chunk_bwd(const qd_shape* shape, const void* q, const void* k, const 
             if (tc_forward(a) != cudaSuccess) return QD_ERR_CUDA;
             a.own_predecessor = true;      // the reverse chain follows this library's forward chain in the stream
         }
-        if (timed(ST_CHAIN_BWD, a.stream, [&] { return tc_chain_bwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
-        if (timed(ST_CHUNK_BWD, a.stream, [&] { return tc_chunk_bwd(a); }) != cudaSuccess) return QD_ERR_CUDA;
-        return QD_OK;
+        return tc_backward(a) == cudaSuccess ? QD_OK : QD_ERR_CUDA;
     }
     if (!(flags & QD_BWD_REUSE_FWD)) {
         // recompute the forward intermediates (outputs of the forward itself are not rewritten:

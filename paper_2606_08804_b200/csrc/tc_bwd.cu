@@ -41,14 +41,15 @@ struct BwdMaps {               // boxes of 64 rows for token tiles, 128 for tile
     CUtensorMap Q, K, V, dO, Mt, P, Dt, dDt, Hs, dHs, Wt, Qg, dHs_store, dDt_store, dQ, dK, dV;
 };
 struct ChainBwdParams {
-    int Tp, H, N, Ns;          // N chunks per sequence; Tp = 64 Ns >= 64 N rows per sequence in the workspace
+    int Tp, H, N, Ns;          // N chunks of a sequence, from n0 on; Tp = 64 Ns rows per sequence in the workspace
+    int n0;
     int dhT_early;             // the kernel before this one in the stream is the library's own: dhT is older than it
     const float* rk;           // non-null (QD_NORM_QK): 1/|k_t| per workspace row, folded into the per-token scale
     const float* g;
     const float* dhT;
     float* dh0;
     unsigned* status;
-    unsigned* next;            // zeroed here for k_tc_chunk_bwd
+    unsigned* next;            // two counters, zeroed here for k_tc_chunk_bwd; null: they are already
 };
 
 // Tiles of a chain's chunk in shared memory: K 16K | P 8K, three deep; Qg 16K | dO 16K and Wt 16K, two deep; staged for their
@@ -123,7 +124,9 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
 
     // bounded wait; once any wait has expired every later wait returns at once (the kernel drains)
     auto wait = [&](uint64_t* br, uint32_t parity) { return mbar_try_wait(br, parity) || wait_on(br, parity, s_abort, p.status); };
-    const float* gseq = p.g + (size_t)bh * p.Tp;
+    const int tok0 = p.n0 * C;                                       // first token; rows and tiles of the workspace start at
+    const size_t row0 = (size_t)bh * p.Tp + tok0, tile0 = (size_t)bh * p.Ns + p.n0;
+    const float* gseq = p.g + row0;
 
     if (warp < kMmaWarp && wq >= nwq) {
         // lanes without a row: straight to the end
@@ -136,7 +139,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         if (!p.dhT_early) grid_dep_wait();
         const size_t at = (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) dh[i] = p.dhT ? p.dhT[at + (size_t)i * D] : 0.f;
+        for (int i = 0; i < 32; ++i) dh[i] = p.dhT ? __ldcg(p.dhT + at + (size_t)i * D) : 0.f;      // not from L1: it may be new
         if (p.dhT_early) grid_dep_wait();  // the loads of dhT are in flight; everything below depends on earlier kernels
         grid_dep_launch();
         auto arrive = [&](uint64_t* b) { __syncwarp(); if ((tid & 31) == 0) mbar_arrive(b); };
@@ -258,9 +261,9 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         // ---------------------------------- saving warp ----------------------------------
         if ((tid & 31) == 0) {
             grid_dep_wait();
-            if (blockIdx.x == 0) *p.next = 0;
+            if (blockIdx.x == 0 && p.next) p.next[0] = p.next[1] = 0;
             for (int it = 0; it < p.N; ++it) {
-                const int y = (int)(((size_t)bh * p.Ns + (p.N - 1 - it)) * D) + v0, sb = it & two;
+                const int y = (int)((tile0 + (p.N - 1 - it)) * D) + v0, sb = it & two;
                 unsigned char *sdH = stg + sb * bytesS, *sdD = sdH + rows * 256;
                 wait(&bar.ht[sb], (it >> two) & 1);       // gradient w.r.t. the exit state (rows = d_v, columns = d_k) is staged
                 tma_store_2d(&mapdHs, sdH, 0, y);
@@ -287,7 +290,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         grid_dep_wait();
         grid_dep_launch();
         // iteration `it` processes chunk n = N-1-it
-        const float* rkseq = p.rk ? p.rk + (size_t)bh * p.Tp : nullptr;
+        const float* rkseq = p.rk ? p.rk + row0 : nullptr;
         float g0, g1, gc, r0 = 1.f, r1 = 1.f;             // log-decays (and 1/|k|) of the next chunk to be loaded
         auto fetch_g = [&](int it) {
             const size_t at = (size_t)(p.N - 1 - it) * C;
@@ -304,9 +307,9 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
                 const int n = p.N - 1 - it;
                 unsigned char* st = smem + s * kBytesK;
                 mbar_expect_tx(&bar.k[s], kBytesK);
-                tma_load_3d(st, &mapK, hh * D, n * C, b, &bar.k[s]);
-                tma_load_3d(st + 8192, &mapK, hh * D + 64, n * C, b, &bar.k[s]);
-                tma_load_2d(st + 16384, &mapP, 0, (int)((size_t)bh * p.Tp + (size_t)n * C), &bar.k[s]);
+                tma_load_3d(st, &mapK, hh * D, tok0 + n * C, b, &bar.k[s]);
+                tma_load_3d(st + 8192, &mapK, hh * D + 64, tok0 + n * C, b, &bar.k[s]);
+                tma_load_2d(st + 16384, &mapP, 0, (int)(row0 + (size_t)n * C), &bar.k[s]);
             }
             if (it + 1 < p.N) fetch_g(it + 1);
         };
@@ -314,16 +317,16 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
             const int n = p.N - 1 - it;
             unsigned char* st = smem + kOffQ + (it & 1) * bytesQ;
             uint64_t* br = &bar.q[it & 1];
-            const int yt = (int)((size_t)bh * p.Tp + (size_t)n * C);
+            const int yt = (int)(row0 + (size_t)n * C);
             mbar_expect_tx(br, bytesQ);
-            tma_load_3d(st + 16384, &mapdO, hh * D + v0, n * C, b, br);             // rows past the end of the sequence: zeros
-            if (rows == D) tma_load_3d(st + 16384 + 8192, &mapdO, hh * D + 64, n * C, b, br);
+            tma_load_3d(st + 16384, &mapdO, hh * D + v0, tok0 + n * C, b, br);             // rows past the end of the sequence: zeros
+            if (rows == D) tma_load_3d(st + 16384 + 8192, &mapdO, hh * D + 64, tok0 + n * C, b, br);
             tma_load_2d(st, &mapQg, 0, yt, br);
             tma_load_2d(st + 8192, &mapQg, 64, yt, br);
         };
         auto load_w = [&](int it) {
             mbar_expect_tx(&bar.w[it & 1], 16384);
-            tma_load_2d(smem + offW + (it & 1) * 16384, &mapWt, 0, (int)(((size_t)bh * p.Ns + (p.N - 1 - it)) * D), &bar.w[it & 1]);
+            tma_load_2d(smem + offW + (it & 1) * 16384, &mapWt, 0, (int)((tile0 + (p.N - 1 - it)) * D), &bar.w[it & 1]);
         };
         fetch_g(0);
         for (int it = 0; it < kDeepK && it < p.N; ++it) {
@@ -364,7 +367,9 @@ struct ChunkBwdParams {
     int logits;                // beta, alpha, lambda are logits of sigmoid gates; their gradients are taken w.r.t. the logits
     const float* rqk;          // QD_NORM_QK: 1/|q_t| per workspace row, then (BH*Tp further) 1/|k_t|
     int group;                 // sequences per group of work items
-    int T, Tp, H, N, Ns, BH, total;   // T tokens in N chunks per sequence, Tp = 64 Ns >= 64 N rows per sequence in the workspace; total = BH*N
+    int T, Tp, H, N, Ns, BH, total;   // T tokens per sequence, of which the N chunks from n0 on; Tp = 64 Ns rows per sequence in the workspace; total = BH*N
+    int n0;
+    int beside;                // 1: runs beside the reverse chain launched before it (tc_bwd), so it waits for that at its end
     const bf16 *beta, *alpha, *lam;
     const float* g;
     float *dbeta, *dalpha, *dlam;
@@ -477,7 +482,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         if (i >= p.total) return Item{-1, 0};
         const int per = p.group * p.N, grp = i / per, r = i - grp * per;
         const int g0 = grp * p.group, gs = min(p.group, p.BH - g0);       // the last group may be smaller
-        return Item{r / gs, g0 + r % gs};
+        return Item{p.n0 + r / gs, g0 + r % gs};
     };
     auto claim = [&]() { return nth((int)gridDim.x + (int)atomicAdd(p.next, 1u)); };      // a CTA's first item goes by its number
     auto put = [&](int it, Item x) { item[it & 3].x = x.n; item[it & 3].y = x.bh; };
@@ -550,7 +555,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         const uint32_t tbu = uniform(tb);
         const uint32_t T0 = tbu, T1 = tbu + 64, T2 = tbu + 128, T3 = tbu + 192, T4 = tbu + 256, T5 = tbu + 320, T6 = tbu + 384, T7 = tbu + 448;
         __syncthreads();                                                 // the first item is known
-        grid_dep_wait();
+        if (!p.beside) grid_dep_wait();
         __syncthreads();                                                 // the first chunk's coefficients have been published
         for (int it = 0; (int)uniform((uint32_t)slot(it).n) >= 0; ++it) {
             const uint32_t ph = it & 1;
@@ -609,7 +614,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             issue_qk(x);
             issue_early(x);
             issue_h(x);
-            grid_dep_wait();
+            if (!p.beside) grid_dep_wait();
             issue_dh(x);
             issue_dd(x);
             put(1, claim());
@@ -693,7 +698,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         };
         __syncthreads();                                                 // the first item is known
         if (slot(0).n >= 0) { fetch(slot(0)); publish(0); }
-        grid_dep_wait();
+        if (!p.beside) grid_dep_wait();
         __syncthreads();
         // what the sums at the end of a chunk need of it, taken up a chunk later
         float dg_pre = 0.f, dhh = 0.f, be0 = 0.f, lm0 = 0.f, al0 = 1.f, gmC = 1.f;
@@ -774,7 +779,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
 #pragma unroll
     for (int g = 0; g < 2; ++g) foff[g] = (wq >> 1) * 8192 + sw128_chunk(c0 + 8 * g + (lane & 7), (wq & 1) * 4 + (lane >> 3));
     __syncthreads();                    // the first item is known
-    grid_dep_wait();
+    if (!p.beside) grid_dep_wait();
     __syncthreads();                    // the first chunk's coefficients have been published
 
     for (int it = 0; slot(it).n >= 0; ++it) {
@@ -1117,6 +1122,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     __syncthreads();
     if (tid == kBwdCompute && s_abort) { mbar_wait(&bar.load, 0); mbar_wait(&bar.d, 0); mbar_wait(&bar.h, 0); mbar_wait(&bar.qk, 0); }   // one more bounded chance for copies in flight
     if (tid < 32) tmem_dealloc(tb, 512);
+    if (tid == 0 && blockIdx.x == 0) grid_dep_wait();            // when this kernel has completed, so has the one before it
 }
 
 template <class K>
@@ -1124,10 +1130,13 @@ cudaError_t set_smem(K kern, size_t bytes) { return set_max_smem_once(reinterpre
 
 }  // namespace
 
-cudaError_t tc_chain_bwd(const ChunkArgs& a) {
+namespace {
+
+// Chunks [n0, n1) of every sequence; what comes after them is in dhT, what goes before them to dh0.
+cudaError_t chain_bwd(const ChunkArgs& a, int n0, int n1, const float* dhT, float* dh0) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
-    const uint64_t BH = (uint64_t)s.B * s.H, Ns = Tp / kChunk, N = (s.T + kChunk - 1) / kChunk;
+    const uint64_t BH = (uint64_t)s.B * s.H, Ns = Tp / kChunk;
     const int rows = chain_rows(BH);
     CUtensorMap mWt, mdO, mQg, mK, mP, mdHs, mdDt;
     if (!make_tmap_bf16_2d(&mWt, a.ws + a.TL.Wt, 64, BH * Ns * D, 128, 128) ||
@@ -1139,13 +1148,14 @@ cudaError_t tc_chain_bwd(const ChunkArgs& a) {
         !make_tmap_bf16_2d(&mdDt, a.ws + a.TL.dDt, 64, BH * Ns * D, 128, rows))
         return cudaErrorInvalidValue;
     ChainBwdParams p{};
-    p.Tp = Tp; p.H = s.H; p.N = (int)N; p.Ns = (int)Ns;
-    p.dhT_early = a.own_predecessor ? 1 : 0;
+    const bool first = dhT == a.dhT;
+    p.Tp = Tp; p.H = s.H; p.N = n1 - n0; p.n0 = n0; p.Ns = (int)Ns;
+    p.dhT_early = first && a.own_predecessor ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.g = (const float*)(a.ws + a.TL.g);
-    p.dhT = a.dhT; p.dh0 = a.dh0;
+    p.dhT = dhT; p.dh0 = dh0;
     p.status = (unsigned*)(a.ws + a.TL.status);
-    p.next = (unsigned*)(a.ws + a.TL.next);
+    p.next = first ? (unsigned*)(a.ws + a.TL.next) : nullptr;
     const auto kern = rows == D ? k_tc_chain_bwd<D> : k_tc_chain_bwd<D / 2>;
     cudaError_t e = set_smem(kern, kChainSmem);
     if (e != cudaSuccess) return e;
@@ -1153,10 +1163,10 @@ cudaError_t tc_chain_bwd(const ChunkArgs& a) {
                              mWt, mdO, mQg, mK, mP, mdHs, mdDt, p);
 }
 
-cudaError_t tc_chunk_bwd(const ChunkArgs& a) {
+cudaError_t chunk_bwd(const ChunkArgs& a, int n0, int n1, bool beside, int counter) {
     const qd_shape& s = a.s;
     const int Tp = tc_padded_T(s);
-    const uint64_t BH = (uint64_t)s.B * s.H, Ns = Tp / kChunk, N = (s.T + kChunk - 1) / kChunk;
+    const uint64_t BH = (uint64_t)s.B * s.H, Ns = Tp / kChunk, N = n1 - n0;
     ChunkBwdMaps m;
     if (!make_tmap_tokens(&m.dQ, a.dq, s.B, s.T, s.H, D, 64) ||
         !make_tmap_tokens(&m.dK, a.dk, s.B, s.T, s.H, D, 64) ||
@@ -1173,7 +1183,7 @@ cudaError_t tc_chunk_bwd(const ChunkArgs& a) {
         !make_tmap_bf16_2d(&m.dHs, a.ws + a.TL.dhsT, D, BH * Ns * D, D * 2, 128))
         return cudaErrorInvalidValue;
     ChunkBwdParams p{};
-    p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = (int)N; p.Ns = (int)Ns; p.BH = (int)BH; p.total = (int)(BH * N);
+    p.T = s.T; p.Tp = Tp; p.H = s.H; p.N = (int)N; p.n0 = n0; p.beside = beside; p.Ns = (int)Ns; p.BH = (int)BH; p.total = (int)(BH * N);
     p.group = (int)std::min<uint64_t>(BH, 64);
     p.beta = (const bf16*)a.beta; p.alpha = (const bf16*)a.alpha; p.lam = (const bf16*)a.lam;
     p.g = (const float*)(a.ws + a.TL.g);
@@ -1181,7 +1191,7 @@ cudaError_t tc_chunk_bwd(const ChunkArgs& a) {
     p.logits = a.logits ? 1 : 0;
     p.rqk = a.norm ? (const float*)(a.ws + a.TL.rqk) : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
-    p.next = (unsigned*)(a.ws + a.TL.next);
+    p.next = (unsigned*)(a.ws + a.TL.next) + counter;
     // the instance without lambda / without the forget gate needs the input AND its gradient to be absent
     const bool lam = a.lam || a.dlam, alpha = a.alpha || a.dalpha;
     using Kern = decltype(&k_tc_chunk_bwd<true, true, false>);
@@ -1199,6 +1209,41 @@ cudaError_t tc_chunk_bwd(const ChunkArgs& a) {
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<uint64_t>(BH * N, (uint64_t)sms);
     return launch_overlapped(kern, dim3(grid), dim3(kBwdThreads), kBwdSmem, a.stream, m, p);
+}
+
+int chunks(const ChunkArgs& a) { return (a.s.T + kChunk - 1) / kChunk; }
+
+}  // namespace
+
+cudaError_t tc_chain_bwd(const ChunkArgs& a) { return chain_bwd(a, 0, chunks(a), a.dhT, a.dh0); }
+cudaError_t tc_chunk_bwd(const ChunkArgs& a) { return chunk_bwd(a, 0, chunks(a), false, 0); }
+
+// With few long sequences the reverse chain leaves SMs idle, as the forward chain does (tc_fwd_parts).  Its chunks are then taken
+// in two parts, and those of the first, the later ones of every sequence, are differentiated beside the chain of the second:
+//     chain [n, N), chain [0, n), chunks [n, N), chunks [0, n)
+// in one stream, by programmatic launch alone.  The third kernel may start when every CTA of the second has begun its work, which it
+// does when the first has completed; it touches the rows of its own chunks, so it need not wait, and what remains of its work
+// when the second kernel leaves its SMs is taken by further CTAs.  Its first CTA waits for the second kernel before it leaves, so the
+// fourth, which waits for the third, comes after all.  dh passes on in fp32, through U~'s section, which no kernel of the
+// backward reads; results are those of one part, bit for bit.
+// Where the line n lies: the fewer sequences, the more SMs for the third kernel and the more it is given: n = N (20 + sequences) / 88.
+// Backward, us, one part / halves / this: 32 sequences of 512 chunks 1332 / 1191 / 1160, 16 of 512 854 / 728 / 709, 8 of 128 179 / 169 /
+// 166, 40 of 128 389 / 384 / 374.  Where it is used: 48 of 256 899 / 856, but 48 of 128 446 / 443, 64 of 256 1159 / 1164; 40 of 96
+// 292 / 285, 32 of 96 247 / 243, 24 of 64 136 / 133, 4 of 64 80.3 / 78.2; but 40 of 64 196 / 201, 32 of 32 85.6 / 90.9, 16 of 32
+// 63.9 / 64.3, 2 of 64 72.9 / 77.1.
+bool tc_bwd_halves(const ChunkArgs& a) {
+    const long long BH = (long long)a.s.B * a.s.H, N = chunks(a);
+    return BH <= 48 && N >= 64 && N >= 3 * BH && BH * N >= 256;
+}
+
+cudaError_t tc_bwd(const ChunkArgs& a) {
+    const int N = chunks(a), n = (int)((long long)N * (20 + a.s.B * a.s.H) / 88);
+    float* carry = (float*)(a.ws + a.TL.Ut);                 // [BH][D][D], from four chunks on
+    cudaError_t e = chain_bwd(a, n, N, a.dhT, carry);
+    if (e == cudaSuccess) e = chain_bwd(a, 0, n, carry, a.dh0);
+    if (e == cudaSuccess) e = chunk_bwd(a, n, N, true, 0);
+    if (e == cudaSuccess) e = chunk_bwd(a, 0, n, false, 1);
+    return e;
 }
 
 }  // namespace qd

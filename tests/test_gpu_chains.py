@@ -48,10 +48,11 @@ def test_preparation_edges(T):
     _bwd_check(cfg, d, reuse=True)
 
 
-@pytest.mark.parametrize("B,H,T", [(1, 16, 64 * 64), (2, 20, 64 * 64 + 1), (1, 4, 64 * 256), (1, 1, 64 * 1024 - 63)])
-def test_forward_in_parts(B, H, T):
-    """Long, few sequences are taken in two or three parts, unless the kernels are timed one by one: the same bits either way, with
-    the state passed on through h_T and (none asked for) through the workspace, replayed from a graph, and close to the oracle."""
+@pytest.mark.parametrize("B,H,T", [(1, 16, 64 * 64), (2, 20, 64 * 64 + 1), (1, 4, 64 * 256), (1, 1, 64 * 1024 - 63), (1, 40, 64 * 120 - 1), (2, 2, 64 * 64)])
+def test_in_parts(B, H, T):
+    """Long, few sequences are taken in two or three parts forward and in two backward (the second case forward, the last backward
+    alone), unless the kernels are timed one by one: the same bits either way, with the state passed on through h_T and (none asked
+    for) through the workspace, replayed from a graph, and close to the oracle."""
     import torch
 
     from gpu_util import dev_inputs
@@ -60,6 +61,7 @@ def test_forward_in_parts(B, H, T):
     cfg = replace(gen.CONFIGS["cfg2"], B=B, H=H, T=T, regime="trained_like", seed=347)
     d = gen.make_chunk_inputs(cfg)
     _fwd_check(cfg, d, pairs=[(0, 0), (B - 1, H - 1)])
+    _bwd_check(cfg, d, pairs=[(0, 0), (B - 1, H - 1)], reuse=True)
     t = dev_inputs(d, cfg.dtype)
     a = [t[n] for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")]
     results = []
@@ -85,8 +87,10 @@ def test_forward_in_parts(B, H, T):
     side.wait_stream(torch.cuda.current_stream())
     with torch.cuda.graph(graph, stream=side):
         qd.chunk_fwd(*a, save_for_bwd=True, workspace=ws, o=o, hT=hT)
+        g = qd.chunk_bwd(*a, t["dO"], t["dhT"], workspace=ws, reuse_fwd=True)
     o.zero_(), hT.zero_()
     for _ in range(2):
         graph.replay()
     torch.cuda.synchronize()
-    assert torch.equal(o, results[0][1][0]) and torch.equal(hT, results[0][1][1])
+    for x, y in zip((o, hT, *g.values()), results[0][1]):
+        assert torch.equal(x, y)
