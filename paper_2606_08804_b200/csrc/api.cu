@@ -94,7 +94,8 @@ static cudaError_t tc_forward(const ChunkArgs& a) {
 }
 // The two of the backward, likewise.
 static cudaError_t tc_backward(const ChunkArgs& a) {
-    if (!g_profile && tc_bwd_halves(a)) return tc_bwd(a);
+    const int parts = g_profile ? 1 : tc_bwd_parts(a);
+    if (parts > 1) return tc_bwd(a, parts);
     const cudaError_t e = timed(ST_CHAIN_BWD, a.stream, [&] { return tc_chain_bwd(a); });
     return e != cudaSuccess ? e : timed(ST_CHUNK_BWD, a.stream, [&] { return tc_chunk_bwd(a); });
 }

@@ -44,7 +44,7 @@ int check_shape(const qd_shape* s);
 // Workspace of the tensor-core path (bf16, d_k = d_v = 128).  Sections start on 1024-byte boundaries.
 struct TcLayout {
     size_t status;   // u32 status word
-    size_t next;     // two u32 counters of the chunk backward's work items, zeroed by the reverse chain
+    size_t next;     // three u32 counters of the chunk backward's work items, zeroed by the reverse chain
     size_t g;        // fp32 [BH*T]
     size_t Qg;       // bf16 [BH*T][dk]        diag(gamma) Q
     size_t P;        // bf16 [BH*T][C]         Gamma o (Q K^T), causal incl. diagonal
@@ -121,8 +121,8 @@ int tc_fwd_parts(const ChunkArgs& a);                        // in how many part
 cudaError_t tc_fwd(const ChunkArgs& a, int parts);
 cudaError_t tc_chain_bwd(const ChunkArgs& a);
 cudaError_t tc_chunk_bwd(const ChunkArgs& a);
-bool tc_bwd_halves(const ChunkArgs& a);                      // whether tc_bwd stands in for tc_chain_bwd and tc_chunk_bwd
-cudaError_t tc_bwd(const ChunkArgs& a);
+int tc_bwd_parts(const ChunkArgs& a);                        // likewise: 1: tc_chain_bwd and tc_chunk_bwd
+cudaError_t tc_bwd(const ChunkArgs& a, int parts);
 
 // S consecutive tokens of every sequence; qdelta_recurrent_step is S = 1
 cudaError_t decode_steps(int B, int S, int H, int dk, int dv, int dtype, const void* q, const void* k, const void* v,

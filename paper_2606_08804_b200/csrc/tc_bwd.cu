@@ -49,7 +49,7 @@ struct ChainBwdParams {
     const float* dhT;
     float* dh0;
     unsigned* status;
-    unsigned* next;            // two counters, zeroed here for k_tc_chunk_bwd; null: they are already
+    unsigned* next;            // three counters, zeroed here for k_tc_chunk_bwd; null: they are already
 };
 
 // Tiles of a chain's chunk in shared memory: K 16K | P 8K, three deep; Qg 16K | dO 16K and Wt 16K, two deep; staged for their
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         // ---------------------------------- saving warp ----------------------------------
         if ((tid & 31) == 0) {
             grid_dep_wait();
-            if (blockIdx.x == 0 && p.next) p.next[0] = p.next[1] = 0;
+            if (blockIdx.x == 0 && p.next) p.next[0] = p.next[1] = p.next[2] = 0;
             for (int it = 0; it < p.N; ++it) {
                 const int y = (int)((tile0 + (p.N - 1 - it)) * D) + v0, sb = it & two;
                 unsigned char *sdH = stg + sb * bytesS, *sdD = sdH + rows * 256;
@@ -1219,31 +1219,46 @@ cudaError_t tc_chain_bwd(const ChunkArgs& a) { return chain_bwd(a, 0, chunks(a),
 cudaError_t tc_chunk_bwd(const ChunkArgs& a) { return chunk_bwd(a, 0, chunks(a), false, 0); }
 
 // With few long sequences the reverse chain leaves SMs idle, as the forward chain does (tc_fwd_parts).  Its chunks are then taken
-// in two parts, and those of the first, the later ones of every sequence, are differentiated beside the chain of the second:
+// in two parts or three, and those of a part, the later ones of every sequence first, are differentiated beside the chain of the next:
 //     chain [n, N), chain [0, n), chunks [n, N), chunks [0, n)
-// in one stream, by programmatic launch alone.  The third kernel may start when every CTA of the second has begun its work, which it
-// does when the first has completed; it touches the rows of its own chunks, so it need not wait, and what remains of its work
-// when the second kernel leaves its SMs is taken by further CTAs.  Its first CTA waits for the second kernel before it leaves, so the
-// fourth, which waits for the third, comes after all.  dh passes on in fp32, through U~'s section, which no kernel of the
-// backward reads; results are those of one part, bit for bit.
-// Where the line n lies: the fewer sequences, the more SMs for the third kernel and the more it is given: n = N (20 + sequences) / 88.
-// Backward, us, one part / halves / this: 32 sequences of 512 chunks 1332 / 1191 / 1160, 16 of 512 854 / 728 / 709, 8 of 128 179 / 169 /
-// 166, 40 of 128 389 / 384 / 374.  Where it is used: 48 of 256 899 / 856, but 48 of 128 446 / 443, 64 of 256 1159 / 1164; 40 of 96
-// 292 / 285, 32 of 96 247 / 243, 24 of 64 136 / 133, 4 of 64 80.3 / 78.2; but 40 of 64 196 / 201, 32 of 32 85.6 / 90.9, 16 of 32
-// 63.9 / 64.3, 2 of 64 72.9 / 77.1.
-bool tc_bwd_halves(const ChunkArgs& a) {
+//     chain [n2, N), chain [n1, n2), chunks [n2, N), chain [0, n1), chunks [n1, n2), chunks [0, n1)
+// in one stream, by programmatic launch alone.  Chunks that stand after a chain that they do not depend on may start when every CTA
+// of that chain has begun its work, which it does when all before it has completed; they touch the rows of their own chunks, so
+// they need not wait, and what remains of their work when the chain leaves its SMs is taken by further CTAs.  Their first CTA
+// waits for the chain before it leaves, so whatever is launched next and waits for them comes after the chain too.
+// dh passes on in fp32, through U~'s section, which no kernel of the backward reads (a CTA of the chain has read its part of it
+// when it writes it); results are those of one part, bit for bit.
+// Where the line n lies: the fewer sequences, the more SMs for the chunks beside a chain and the more they are given:
+// n = N (20 + sequences) / 88.  Backward, us, one part / halves / this: 32 sequences of 512 chunks 1332 / 1191 / 1160, 16 of 512
+// 854 / 728 / 709, 8 of 128 179 / 169 / 166, 40 of 128 389 / 384 / 374.  Where it is used: 48 of 256 899 / 856, but 48 of 128 446 / 443, 64
+// of 256 1159 / 1164; 40 of 96 292 / 285, 32 of 96 247 / 243, 24 of 64 136 / 133, 4 of 64 80.3 / 78.2; but 40 of 64 196 / 201, 32 of 32
+// 85.6 / 90.9, 16 of 32 63.9 / 64.3, 2 of 64 72.9 / 77.1.
+// Three parts let the first chain, beside which nothing runs, be a third to a half as long, for one more pair of launches: n1 = N sequences
+// / 56 (34 at most), n2 = n1 + 5 N / 16, near the best of a sweep over both.  Two parts / three: 32 sequences of 512 chunks 1117 / 1074, 16 of
+// 512 731 / 694, 12 of 1024 1258 / 1210, 12 of 256 334 / 329, 12 of 171 233 / 228, 16 of 128 196 / 192, 32 of 128 288 / 281, 36 of 128
+// 312 / 309; but 32 of 112 257 / 256, 12 of 128 178.6 / 180.2, 40 of 140 369 / 370, 40 of 256 645 / 642, and the sweep had 8 of 512
+// 596 / 604, 48 of 256 853 / 862.
+int tc_bwd_parts(const ChunkArgs& a) {
     const long long BH = (long long)a.s.B * a.s.H, N = chunks(a);
-    return BH <= 48 && N >= 64 && N >= 3 * BH && BH * N >= 256;
+    if (BH > 48 || N < 64 || N < 3 * BH || BH * N < 256) return 1;
+    return BH >= 12 && BH <= 36 && N >= 128 && BH * N >= 2048 ? 3 : 2;
 }
 
-cudaError_t tc_bwd(const ChunkArgs& a) {
-    const int N = chunks(a), n = (int)((long long)N * (20 + a.s.B * a.s.H) / 88);
+cudaError_t tc_bwd(const ChunkArgs& a, int parts) {
+    const int N = chunks(a), BH = a.s.B * a.s.H;
     float* carry = (float*)(a.ws + a.TL.Ut);                 // [BH][D][D], from four chunks on
-    cudaError_t e = chain_bwd(a, n, N, a.dhT, carry);
-    if (e == cudaSuccess) e = chain_bwd(a, 0, n, carry, a.dh0);
-    if (e == cudaSuccess) e = chunk_bwd(a, n, N, true, 0);
-    if (e == cudaSuccess) e = chunk_bwd(a, 0, n, false, 1);
-    return e;
+    const int lo = parts == 2 ? (int)((long long)N * (20 + BH) / 88) : (int)((long long)N * std::min(BH, 34) / 56);
+    const int hi = parts == 2 ? lo : lo + (int)((long long)N * 5 / 16);
+    cudaError_t e = chain_bwd(a, hi, N, a.dhT, carry);
+    int n1 = N;                                              // the chunks from here on are differentiated; chains have come to n0
+    for (int i = 0, n0 = hi; i + 1 < parts; ++i) {
+        const int to = i + 2 == parts ? 0 : lo;
+        if (e == cudaSuccess) e = chain_bwd(a, to, n0, carry, to ? carry : a.dh0);
+        if (e == cudaSuccess) e = chunk_bwd(a, n0, n1, true, i);
+        n1 = n0;
+        n0 = to;
+    }
+    return e == cudaSuccess ? chunk_bwd(a, 0, n1, false, parts - 1) : e;
 }
 
 }  // namespace qd

@@ -48,10 +48,9 @@ def test_preparation_edges(T):
     _bwd_check(cfg, d, reuse=True)
 
 
-@pytest.mark.parametrize("B,H,T", [(1, 16, 64 * 64), (2, 20, 64 * 64 + 1), (1, 4, 64 * 256), (1, 1, 64 * 1024 - 63), (1, 40, 64 * 120 - 1), (2, 2, 64 * 64)])
+@pytest.mark.parametrize("B,H,T", [(1, 16, 64 * 64), (2, 20, 64 * 64 + 1), (1, 4, 64 * 256), (1, 1, 64 * 1024 - 63), (1, 40, 64 * 120 - 1), (2, 2, 64 * 64), (2, 8, 64 * 128 - 5), (1, 36, 64 * 128)])
 def test_in_parts(B, H, T):
-    """Long, few sequences are taken in two or three parts forward and in two backward (the second case forward, the last backward
-    alone), unless the kernels are timed one by one: the same bits either way, with the state passed on through h_T and (none asked
+    """Long, few sequences are taken in two or three parts (the second case forward, the sixth backward alone), unless the kernels are timed one by one: the same bits either way, with the state passed on through h_T and (none asked
     for) through the workspace, replayed from a graph, and close to the oracle."""
     import torch
 
