@@ -29,9 +29,11 @@ namespace {
 // time and written back as it is updated: 32 registers instead of 64, and five CTAs to an SM instead of four, which with 16 KB each
 // are too little on its way to keep HBM busy (256 x 16 states 47.7 -> 44.0 us, 100 x 8 12.2 -> 11.1; six CTAs, which spill 70 bytes,
 // 49.5).  With an fp32 state it would gain nothing (30 x 16 states 11.8 -> 12.4).
-// VEC: the rows of a thread are neighbours, so that its parts of x, q and k are read four at a time (8 tokens of 256 x 16 states 156 ->
-// 150 us, of 48 x 16 36.2 -> 35.0).  Rows a whole group apart where the tokens are normalised, which leaves fewer registers (4 tokens of
-// 48 x 16 states 25.7 us so, 26.1 with neighbours).
+// VEC: a thread has groups of four rows that are neighbours, so that its parts of x, q and k are read four at a time while what a CTA
+// loads at a time stays close together.  One token of 149 x 8 states 18.45 us with rows a whole group apart, 18.9 with all rows
+// of a thread next to each other, 18.3 so; 8 tokens of 256 x 16 153 / 148 / 146.5, of a bf16 state 155 / 152 / 150.6.  Rows a
+// whole group apart where the tokens of an fp32 state are normalised, which leaves fewer registers.  The rule does not look at S,
+// since the order of the sums follows the rows.
 constexpr int kBlock = 8;
 template <typename IO, int DK, int DVS, int NT, bool LOGITS, bool NORM, bool SB16, bool ONE>      // flags, compile-time
 __global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H, int dv, const IO* __restrict__ q, const IO* __restrict__ k,
@@ -51,8 +53,9 @@ __global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H
     const int b = bh / H, hh = bh % H;
     const int ct = tid % CT, rg = tid / CT, lane = tid & 31;
 
-    uint4* base = reinterpret_cast<uint4*>(static_cast<unsigned char*>(state_) + (((size_t)bh * DK + (VEC ? rg * NP : rg)) * dv + j0) * (SB16 ? 2 : 4)) + ct;
-    const size_t rstride = (size_t)(VEC ? 1 : RP) * dv / NC;
+    uint4* base = reinterpret_cast<uint4*>(static_cast<unsigned char*>(state_) + (((size_t)bh * DK + (VEC ? rg * 4 : rg)) * dv + j0) * (SB16 ? 2 : 4)) + ct;
+    const size_t rowq = (size_t)dv / NC;
+    auto at = [&](int pz) { return base + (VEC ? (pz >> 2) * 4 * RP + (pz & 3) : pz * RP) * rowq; };
     // launched while the kernel before it drains (2 us less per step): nothing is read before that kernel has completed
     sm100::grid_dep_wait();
     sm100::grid_dep_launch();
@@ -60,7 +63,7 @@ __global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H
     float h[KEEP ? NP : 1][NC];
     uint4 raw[NP];
 #pragma unroll
-    for (int pz = 0; pz < NP; ++pz) raw[pz] = __ldcs(base + pz * rstride);
+    for (int pz = 0; pz < NP; ++pz) raw[pz] = __ldcs(at(pz));
     auto stage = [&](int s0) {
         const int nb = min(kBlock, S - s0);
         for (int s = tid >> 5; s < nb; s += NT / 32) {
@@ -119,7 +122,7 @@ __global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H
     };
     stage(0);
     auto four = [&](const float* v, int p4) {
-        if (VEC) return *reinterpret_cast<const float4*>(v + rg * NP + p4);
+        if (VEC) return *reinterpret_cast<const float4*>(v + rg * 4 + p4 * RP);
         return make_float4(v[p4 * RP + rg], v[(p4 + 1) * RP + rg], v[(p4 + 2) * RP + rg], v[(p4 + 3) * RP + rg]);
     };
     auto widen = [&](const uint4& r, float (&d)[NC]) {
@@ -145,7 +148,7 @@ __global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H
                 w[e] = __float_as_uint(d[e]);
             }
         }
-        __stcs(base + pz * rstride, make_uint4(w[0], w[1], w[2], w[3]));
+        __stcs(at(pz), make_uint4(w[0], w[1], w[2], w[3]));
     };
     if (KEEP)
 #pragma unroll
