@@ -25,24 +25,26 @@ namespace {
 // spill; five CTAs would spill 64 - 204.
 // SB16 (QD_STATE_BF16): the state is STORED in bf16 (half the bytes of the step); it is widened to fp32 when read, all S
 // tokens of the call are applied in fp32, and it is rounded to bf16 once, when written back.
-// ONE (bf16 state, a single token): the state is needed once more only to be updated, so it stays as it was read, is widened each
-// time and written back as it is updated: 32 registers instead of 64, and five CTAs to an SM instead of four, which with 16 KB each
-// are too little on its way to keep HBM busy (256 x 16 states 47.7 -> 44.0 us, 100 x 8 12.2 -> 11.1; six CTAs, which spill 70 bytes,
-// 49.5).  With an fp32 state it would gain nothing (30 x 16 states 11.8 -> 12.4).
+// ONE (bf16 state, a single token), KEEP false: the state is needed once more only to be updated, so it stays as it was read, is
+// widened each time and written back as it is updated: 32 registers instead of 64, and five CTAs to an SM instead of four, which with
+// 16 KB each are too little on its way to keep HBM busy (256 x 16 states 47.7 -> 44.0 us, 100 x 8 12.2 -> 11.1; six CTAs, which spill
+// 70 bytes, 49.5).  With an fp32 state it would gain nothing (30 x 16 states 11.8 -> 12.4).  It is one_token_kept's choice at d_k = 128:
+// for one CTA it takes longer.  At d_k = 64 it gains at any number of CTAs (4 of them 1.72 -> 1.60 us).
 // VEC: a thread has groups of four rows that are neighbours, so that its parts of x, q and k are read four at a time while what a CTA
 // loads at a time stays close together.  One token of 149 x 8 states 18.45 us with rows a whole group apart, 18.9 with all rows
 // of a thread next to each other, 18.3 so; 8 tokens of 256 x 16 153 / 148 / 146.5, of a bf16 state 155 / 152 / 150.6.  Rows a
 // whole group apart where the tokens of an fp32 state are normalised, which leaves fewer registers.  The rule does not look at S,
 // since the order of the sums follows the rows.
 constexpr int kBlock = 8;
-template <typename IO, int DK, int DVS, int NT, bool LOGITS, bool NORM, bool SB16, bool ONE>      // flags, compile-time
-__global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H, int dv, const IO* __restrict__ q, const IO* __restrict__ k,
+template <typename IO, int DK, int DVS, int NT, bool LOGITS, bool NORM, bool SB16, bool ONE, bool KEEP>      // flags, compile-time
+__global__ void __launch_bounds__(NT, KEEP ? 4 : 5) k_decode(int S, int H, int dv, const IO* __restrict__ q, const IO* __restrict__ k,
                                                      const IO* __restrict__ v, const IO* __restrict__ beta,
                                                      const IO* __restrict__ alpha, const IO* __restrict__ lam,
                                                      void* __restrict__ state_, IO* __restrict__ o) {
     constexpr int NC = SB16 ? 8 : 4;                             // columns per thread: 16 bytes of a state row
     constexpr int CT = DVS / NC, RP = NT / CT, NP = DK / RP;
-    static_assert(NT % CT == 0 && DK % RP == 0, "bad decode tiling");
+    static_assert(NT % CT == 0 && DK % RP == 0 && NP % 4 == 0, "bad decode tiling");
+    static_assert(KEEP || ONE, "several tokens need the state in fp32 from token to token");
     constexpr int TOKEN = 3 * DK + DVS;
     constexpr bool VEC = SB16 || !NORM;
     extern __shared__ __align__(16) float stok[];                // per token: x [DK], q [DK], k [DK], v [DVS]
@@ -59,8 +61,7 @@ __global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H
     // launched while the kernel before it drains (2 us less per step): nothing is read before that kernel has completed
     sm100::grid_dep_wait();
     sm100::grid_dep_launch();
-    constexpr bool KEEP = !ONE;                                  // the state in fp32 from token to token
-    float h[KEEP ? NP : 1][NC];
+    float h[KEEP ? NP : 1][NC];                                  // the state in fp32
     uint4 raw[NP];
 #pragma unroll
     for (int pz = 0; pz < NP; ++pz) raw[pz] = __ldcs(at(pz));
@@ -228,19 +229,31 @@ __global__ void __launch_bounds__(NT, SB16 && ONE ? 5 : 4) k_decode(int S, int H
         for (int pz = 0; pz < NP; ++pz) write(pz, h[pz % (KEEP ? NP : 1)]);
 }
 
+// One token on a bf16 state with d_k = 128: whether the widened state is kept, which lets four CTAs share an SM, or widened twice,
+// which lets five.  Kept where five would bring nothing: they do when more than four to an SM are wanted, and when two launches,
+// the second of which begins while the first drains, fit on the GPU five to an SM but not four.  Widened twice / kept, us per call
+// of many: 8 CTAs 2.23 / 1.95, 290 2.86 / 2.59, but 300 3.22 / 3.45, 350 3.32 / 3.51; then 400 4.20 / 3.59, 592 4.41 / 3.69, but 608 4.33 /
+// 5.00.  Normalised tokens 290 3.20 / 3.10, 350 3.67 / 4.12, 592 4.85 / 4.20; fp32 tokens 592 4.70 / 3.69.
+bool one_token_kept(unsigned ctas) {
+    const bool two_want_five = 2 * ctas > 4 * kSMs && 2 * ctas <= 5 * kSMs;
+    return ctas <= 4 * kSMs && !two_want_five;
+}
+
 template <typename IO, int DK>
 cudaError_t launch(int B, int S, int H, int dv, const void* q, const void* k, const void* v, const void* beta,
                          const void* alpha, const void* lam, void* state, void* o, bool logits, bool norm, bool sb16,
                          cudaStream_t stream) {
     constexpr int DVS = 64, NT = 128;
     dim3 grid((unsigned)(dv / DVS) * (unsigned)(B * H));
-    using Kern = decltype(&k_decode<IO, DK, DVS, NT, false, false, false, false>);
-#define QD_GATES(SB16, ONE)                                                                                                  \
-    {k_decode<IO, DK, DVS, NT, false, false, SB16, ONE>, k_decode<IO, DK, DVS, NT, false, true, SB16, ONE>,                  \
-     k_decode<IO, DK, DVS, NT, true, false, SB16, ONE>, k_decode<IO, DK, DVS, NT, true, true, SB16, ONE>}
-    static const Kern table[3][4] = {QD_GATES(false, false), QD_GATES(true, false), QD_GATES(true, true)};
+    using Kern = decltype(&k_decode<IO, DK, DVS, NT, false, false, false, false, true>);
+#define QD_GATES(...)                                                                                                        \
+    {k_decode<IO, DK, DVS, NT, false, false, __VA_ARGS__>, k_decode<IO, DK, DVS, NT, false, true, __VA_ARGS__>,              \
+     k_decode<IO, DK, DVS, NT, true, false, __VA_ARGS__>, k_decode<IO, DK, DVS, NT, true, true, __VA_ARGS__>}
+    static const Kern table[4][4] = {QD_GATES(false, false, true), QD_GATES(true, false, true), QD_GATES(true, true, false),
+                                     QD_GATES(true, true, DK == 128)};
 #undef QD_GATES
-    const Kern kern = table[sb16 ? (S == 1 ? 2 : 1) : 0][(logits ? 2 : 0) + (norm ? 1 : 0)];
+    const int form = !sb16 ? 0 : S > 1 ? 1 : DK == 128 && one_token_kept(grid.x) ? 3 : 2;
+    const Kern kern = table[form][(logits ? 2 : 0) + (norm ? 1 : 0)];
     return launch_overlapped(kern, grid, dim3(NT), (S < kBlock ? S : kBlock) * (3 * DK + DVS) * sizeof(float), stream, S, H, dv,
                              (const IO*)q, (const IO*)k, (const IO*)v, (const IO*)beta, (const IO*)alpha, (const IO*)lam, state, (IO*)o);
 }

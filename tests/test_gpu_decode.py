@@ -253,3 +253,23 @@ def test_bf16_state_is_the_fp32_one_rounded(dk, dv, S, raw):
     for got, want in ((o, ow.float()), (state, wide)):
         tol = 2.0 ** -7 * want.abs() + 128 * 2.0 ** -24 * want.abs().max()
         assert ((got.float() - want).abs() <= tol).all()
+
+
+@pytest.mark.parametrize("dt", ["bf16", "f32"])
+@pytest.mark.parametrize("raw", [False, True])
+@pytest.mark.parametrize("dv,parts", [(128, (148, 149)), (64, (296, 297, 370, 371, 592, 593))])
+def test_one_token_on_bf16_states_does_not_look_at_their_number(dt, dv, parts, raw):
+    """d_k = 128: the widened state is kept or widened twice, by the number of 64-column slices (kept up to 296 and from 371 to 592).
+    One call over all states gives the bits of calls over some of them each."""
+    from paper_2606_08804_b200 import binding as qd
+    g = torch.Generator(device="cuda").manual_seed(41 + dv)
+    rnd = lambda *shape: torch.randn(*shape, device="cuda", generator=g)
+    B, io = sum(parts), {"bf16": torch.bfloat16, "f32": torch.float32}[dt]
+    t = [rnd(B, 1, 1, d) * (1.0 if raw else d ** -0.5) for d in (128, 128, dv)]
+    t += [x if raw else torch.sigmoid(x) for x in (rnd(B, 1, 1), rnd(B, 1, 1), rnd(B, 1, 1))]
+    t = [x.to(io) for x in t]
+    state = (rnd(B, 1, 128, dv) * 0.1).to(torch.bfloat16)
+    states = [s.clone() for s in state.split(parts)]
+    o = qd.recurrent_steps(*t, state, logits=raw, norm_qk=raw)
+    os = [qd.recurrent_steps(*x, s, logits=raw, norm_qk=raw) for *x, s in zip(*(x.split(parts) for x in t), states)]
+    assert torch.equal(o, torch.cat(os)) and torch.equal(state, torch.cat(states))
