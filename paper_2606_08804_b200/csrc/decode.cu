@@ -33,8 +33,9 @@ namespace {
 // VEC: a thread has groups of four rows that are neighbours, so that its parts of x, q and k are read four at a time while what a CTA
 // loads at a time stays close together.  One token of 149 x 8 states 18.45 us with rows a whole group apart, 18.9 with all rows
 // of a thread next to each other, 18.3 so; 8 tokens of 256 x 16 153 / 148 / 146.5, of a bf16 state 155 / 152 / 150.6.  Rows a
-// whole group apart where the tokens of an fp32 state are normalised, which leaves fewer registers.  The rule does not look at S,
-// since the order of the sums follows the rows.
+// whole group apart where the tokens of an fp32 state are normalised, which leaves fewer registers, and for several fp32 tokens on
+// a bf16 state with d_k = 128 (3 tokens of 256 x 16 states 80.5 in groups of four, 75.7 so; 4 tokens 100.2 and 92.4).  The order of the
+// sums follows the rows, so the rule looks neither at the number of states nor, with an fp32 state, at S.
 constexpr int kBlock = 8;
 template <typename IO, int DK, int DVS, int NT, bool LOGITS, bool NORM, bool SB16, bool ONE, bool KEEP>      // flags, compile-time
 __global__ void __launch_bounds__(NT, KEEP ? 4 : 5) k_decode(int S, int H, int dv, const IO* __restrict__ q, const IO* __restrict__ k,
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(NT, KEEP ? 4 : 5) k_decode(int S, int H, int d
     static_assert(NT % CT == 0 && DK % RP == 0 && NP % 4 == 0, "bad decode tiling");
     static_assert(KEEP || ONE, "several tokens need the state in fp32 from token to token");
     constexpr int TOKEN = 3 * DK + DVS;
-    constexpr bool VEC = SB16 || !NORM;
+    constexpr bool VEC = SB16 ? ONE || NORM || DK == 64 || sizeof(IO) == 2 : !NORM;
     extern __shared__ __align__(16) float stok[];                // per token: x [DK], q [DK], k [DK], v [DVS]
     __shared__ __align__(16) float redx[2][RP][DVS], redq[2][RP][DVS];
     __shared__ __align__(16) float sdelta[2][DVS];
@@ -57,7 +58,8 @@ __global__ void __launch_bounds__(NT, KEEP ? 4 : 5) k_decode(int S, int H, int d
 
     uint4* base = reinterpret_cast<uint4*>(static_cast<unsigned char*>(state_) + (((size_t)bh * DK + (VEC ? rg * 4 : rg)) * dv + j0) * (SB16 ? 2 : 4)) + ct;
     const size_t rowq = (size_t)dv / NC;
-    auto at = [&](int pz) { return base + (VEC ? (pz >> 2) * 4 * RP + (pz & 3) : pz * RP) * rowq; };
+    const size_t rstride = (size_t)RP * dv / NC;
+    auto at = [&](int pz) { return VEC ? base + ((pz >> 2) * 4 * RP + (pz & 3)) * rowq : base + pz * rstride; };
     // launched while the kernel before it drains (2 us less per step): nothing is read before that kernel has completed
     sm100::grid_dep_wait();
     sm100::grid_dep_launch();
@@ -122,9 +124,17 @@ __global__ void __launch_bounds__(NT, KEEP ? 4 : 5) k_decode(int S, int H, int d
         __syncthreads();
     };
     stage(0);
-    auto four = [&](const float* v, int p4) {
-        if (VEC) return *reinterpret_cast<const float4*>(v + rg * 4 + p4 * RP);
-        return make_float4(v[p4 * RP + rg], v[(p4 + 1) * RP + rg], v[(p4 + 2) * RP + rg], v[(p4 + 3) * RP + rg]);
+    // What a staged vector has for G rows of this thread, from the p-th on.  Rows a whole group apart are read one at a time, where
+    // d_k = 128 leaves an fp32 state registers four (8 normalised tokens of 256 x 16 states 170.9 -> 169.2 us; at d_k = 64 57.2 -> 57.5).
+    constexpr int G = VEC || (DK == 128 && !SB16) ? 4 : 1;
+    auto rows = [&](const float* t, int p, float (&r)[G]) {
+        if constexpr (VEC) {
+            const float4 f = *reinterpret_cast<const float4*>(t + rg * 4 + p * RP);
+            r[0] = f.x; r[1] = f.y; r[2] = f.z; r[3] = f.w;
+        } else {
+#pragma unroll
+            for (int z = 0; z < G; ++z) r[z] = t[(p + z) * RP + rg];
+        }
     };
     auto widen = [&](const uint4& r, float (&d)[NC]) {
         const uint32_t w[4] = {r.x, r.y, r.z, r.w};
@@ -165,15 +175,16 @@ __global__ void __launch_bounds__(NT, KEEP ? 4 : 5) k_decode(int S, int H, int d
 #pragma unroll
             for (int e = 0; e < NC; ++e) { ax[e] = 0.f; aq[e] = 0.f; }
 #pragma unroll
-            for (int p4 = 0; p4 < NP; p4 += 4) {
-                if (!KEEP) asm volatile("" ::: "memory");                // four rows at a time
-                const float4 x4 = four(tx, p4), q4 = four(tq, p4);
-                const float xi[4] = {x4.x, x4.y, x4.z, x4.w}, qi[4] = {q4.x, q4.y, q4.z, q4.w};
+            for (int p = 0; p < NP; p += G) {
+                if (!KEEP) asm volatile("" ::: "memory");                // G rows at a time
+                float xi[G], qi[G];
+                rows(tx, p, xi);
+                rows(tq, p, qi);
 #pragma unroll
-                for (int z = 0; z < 4; ++z) {
+                for (int z = 0; z < G; ++z) {
                     float one[NC];
-                    if (!KEEP) widen(raw[p4 + z], one);
-                    const float (&hr)[NC] = KEEP ? h[(p4 + z) % (KEEP ? NP : 1)] : one;
+                    if (!KEEP) widen(raw[p + z], one);
+                    const float (&hr)[NC] = KEEP ? h[(p + z) % (KEEP ? NP : 1)] : one;
 #pragma unroll
                     for (int e = 0; e < NC; ++e) { ax[e] = fmaf(hr[e], xi[z], ax[e]); aq[e] = fmaf(hr[e], qi[z], aq[e]); }
                 }
@@ -204,18 +215,18 @@ __global__ void __launch_bounds__(NT, KEEP ? 4 : 5) k_decode(int S, int H, int d
                 dl[e] = t.x; dl[e + 1] = t.y; dl[e + 2] = t.z; dl[e + 3] = t.w;
             }
 #pragma unroll
-            for (int p4 = 0; p4 < NP; p4 += 4) {
-                if (!KEEP) asm volatile("" ::: "memory");                // four rows at a time
-                const float4 k4 = four(tk, p4);
-                const float ki[4] = {k4.x, k4.y, k4.z, k4.w};
+            for (int p = 0; p < NP; p += G) {
+                if (!KEEP) asm volatile("" ::: "memory");                // G rows at a time
+                float ki[G];
+                rows(tk, p, ki);
 #pragma unroll
-                for (int z = 0; z < 4; ++z) {
+                for (int z = 0; z < G; ++z) {
                     float one[NC];
-                    if (!KEEP) widen(raw[p4 + z], one);
-                    float (&hr)[NC] = KEEP ? h[(p4 + z) % (KEEP ? NP : 1)] : one;
+                    if (!KEEP) widen(raw[p + z], one);
+                    float (&hr)[NC] = KEEP ? h[(p + z) % (KEEP ? NP : 1)] : one;
 #pragma unroll
                     for (int e = 0; e < NC; ++e) hr[e] = fmaf(al, hr[e], ki[z] * dl[e]);
-                    if (!KEEP) write(p4 + z, hr);
+                    if (!KEEP) write(p + z, hr);
                 }
             }
         }
