@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(NT, KEEP ? 4 : 5) k_decode(int S, int H, int d
     };
     stage(0);
     // What a staged vector has for G rows of this thread, from the p-th on.  Rows a whole group apart are read one at a time, where
-    // d_k = 128 leaves an fp32 state registers four (8 normalised tokens of 256 x 16 states 170.9 -> 169.2 us; at d_k = 64 57.2 -> 57.5).
+    // d_k = 128 leaves an fp32 state registers four (8 normalised tokens of 256 x 16 states 170.9 -> 169.2 us; at d_k = 64 57.6 -> 58.2).
     constexpr int G = VEC || (DK == 128 && !SB16) ? 4 : 1;
     auto rows = [&](const float* t, int p, float (&r)[G]) {
         if constexpr (VEC) {

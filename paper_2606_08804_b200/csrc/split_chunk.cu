@@ -71,7 +71,7 @@ __device__ __forceinline__ void fetched() { asm volatile("cp.async.wait_all;" ::
 // K1: per chunk-head, state-independent part: g, P, W<-, U~ (and M for the backward).
 template <int DK, int DV>
 __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     constexpr int LK = DK + kPad, LV = DV + kPad;
     float *sQ = sm, *sK = sQ + C * LK, *sV = sK + C * LK, *sA = sV + C * LV, *sM = sA + C * LDC;
     __shared__ __align__(16) float sg[C];
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(NT) k_prep(Ptrs p) {
 // warps do nothing else than copy, K and P while Delta is made, the next W<-, Q and U~ while the state is updated.
 template <int DK, int DS>
 __global__ void __launch_bounds__(NT + kLoaders) k_chain_fwd(Ptrs p, int DV) {
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     constexpr int LA = DK + 4, LB = DK + 8, LS = DS + 8, NS = DS / 8;
     float *sW = sm, *sQ = sW + C * LA, *sK = sQ + C * LA, *sP = sK + C * LB, *sU = sP + C * LDC, *sD = sU + C * LS,
           *sDs = sD + C * LS, *sh = sDs + C * LS;                     // sh: the state slice [DK][DS]
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(NT + kLoaders) k_chain_fwd(Ptrs p, int DV) {
 // and leaves per chunk: dh (exit), dDelta, and two scalar partial sums the decay gradient needs.
 template <int DK, int DS>
 __global__ void __launch_bounds__(NT + kLoaders) k_chain_bwd(Ptrs p, int DV) {
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     constexpr int LA = DK + 4, LB = DK + 8, LP = C + 8, LS = DS + 8, NS = DS / 8;
     float *sK = sm, *sQ = sK + C * LA, *sW = sQ + C * LB, *sP = sW + C * LB, *sO = sP + C * LP, *sOs = sO + C * LS,
           *sD = sOs + C * LS, *sdD = sD + C * LS, *sdh = sdD + C * LS;
@@ -412,7 +412,7 @@ struct BwdSmem {
 };
 template <int DK, int DV>
 __global__ void __launch_bounds__(NT) k_chunk_bwd(Ptrs p) {
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     constexpr int LT = BwdSmem<DK, DV>::LT, LH = DV + kPad, kSlot = BwdSmem<DK, DV>::kSlot, NK = DK / 32;
     static_assert(DK * LH <= 2 * kSlot, "a state fits two slots");
     float *s0 = sm, *s1 = s0 + kSlot, *s2 = s1 + kSlot, *s3 = s2 + kSlot;
