@@ -608,6 +608,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         for (int e = 0; e < 8; ++e)
             xoff[e] = (uint32_t)e * 128u + (((((uint32_t)l & 63u) >> 3) ^ (uint32_t)e) << 4) + ((uint32_t)l & 7u) * 2u;
         unsigned char* stg = sO + (l >> 6) * 4096;
+        grid_dep_wait();                  // the chain before may take longer than a wait has (tc_fwd_parts)
         for (int n = 0; n < p.N; ++n) {
             const int ob = n & 1;
             wait(&bar_o[ob], (n >> 1) & 1);

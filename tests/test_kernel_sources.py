@@ -18,3 +18,17 @@ def test_dynamic_shared_memory_is_aligned(name):
         assert ("extern __shared__" in line) == bool(m), line
         if m and int(m.group(1) or 0) < 16:
             assert re.search(r"\(uintptr_t\)%s \+ 1023\) & ~\(uintptr_t\)1023" % m.group(2), lines[i + 1]), (name, i + 1, line)
+
+
+@pytest.mark.parametrize("name,kernel", [("tc_fwd.cu", "k_tc_chain_fwd"), ("tc_bwd.cu", "k_tc_chain_bwd"), ("tc_bwd.cu", "k_tc_chunk_bwd")])
+def test_bounded_waits_begin_after_the_kernel_before(name, kernel):
+    """A CTA may start while the kernel before it runs, for as long as that takes; the time limit of a wait inside the CTA is meant for the
+    CTA's own work, so every role of its warps waits for that kernel before its first bounded wait."""
+    src = open(os.path.join(CSRC, name)).read()
+    body = src[re.search(r"__global__ [^;{]*\b%s\(" % kernel, src).end():]
+    body = body[:body.index("\n}\n")]
+    roles = re.split(r"\n *// (?:-{10,}|={10,}) (.+?) (?:-{10,}|={10,})\n", body)
+    assert len(roles) >= 9, kernel
+    for role, text in zip(roles[1::2], roles[2::2]):
+        first = re.search(r"\bwait\(&", text)
+        assert first is None or 0 <= text.find("grid_dep_wait()") < first.start(), (kernel, role)
