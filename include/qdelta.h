@@ -97,6 +97,12 @@ typedef struct CUstream_st *qd_stream;   /* a cudaStream_t */
  * 1 = tensor-core kernels, 0 = fp32-accurate kernels, -1 = invalid or unsupported shape. */
 int qdelta_chunk_path(const qd_shape *shape);
 
+/* In how many parts a chunkwise call takes every sequence of `shape` (likewise a query for tests and benchmarks): the
+ * backward (backward != 0), or a forward that returns hT or saves for the backward; -1 = invalid or unsupported shape.  With few
+ * long sequences the tensor-core kernels take them in 2 or 3 parts and work on one part beside another; the results are the bits of one
+ * part.  1 while the timing aid (qdelta_profile_enable) is on. */
+int qdelta_chunk_parts(const qd_shape *shape, int backward);
+
 /* Bytes of device workspace the chunkwise calls need for this shape (0 on invalid shape).
  * for_backward != 0: the size qdelta_chunk_bwd (and a QD_FWD_SAVE_FOR_BWD forward) needs. */
 size_t qdelta_chunk_workspace_bytes(const qd_shape *shape, int for_backward);

@@ -19,7 +19,7 @@ QD_FWD_SAVE_FOR_BWD, QD_BWD_REUSE_FWD, QD_COEF_LOGITS, QD_NORM_QK, QD_STATE_BF16
 EXPORTS = ("qdelta_chunk_workspace_bytes", "qdelta_chunk_fwd", "qdelta_chunk_bwd",
            "qdelta_recurrent_step", "qdelta_workspace_status", "qdelta_status_string",
            "qdelta_profile_enable", "qdelta_profile_stage_count", "qdelta_profile_stage_name",
-           "qdelta_profile_read", "qdelta_chunk_fwd_static", "qdelta_chunk_path",
+           "qdelta_profile_read", "qdelta_chunk_fwd_static", "qdelta_chunk_path", "qdelta_chunk_parts",
            "qdelta_recurrent_steps")
 
 
@@ -65,6 +65,8 @@ def load():
     lib.qdelta_chunk_workspace_bytes.argtypes = [ctypes.POINTER(QdShape), i]
     lib.qdelta_chunk_path.restype = i
     lib.qdelta_chunk_path.argtypes = [ctypes.POINTER(QdShape)]
+    lib.qdelta_chunk_parts.restype = i
+    lib.qdelta_chunk_parts.argtypes = [ctypes.POINTER(QdShape), i]
     lib.qdelta_chunk_fwd.restype = i
     lib.qdelta_chunk_fwd.argtypes = [ctypes.POINTER(QdShape)] + [vp] * 9 + [vp, sz, u, vp]
     lib.qdelta_chunk_bwd.restype = i
@@ -158,6 +160,14 @@ def chunk_path(shape: QdShape) -> str:
     if r < 0:
         raise QdeltaError("unsupported or invalid shape for the chunkwise kernels")
     return "tensor_core" if r == 1 else "fp32"
+
+
+def chunk_parts(shape: QdShape, backward: bool) -> int:
+    """In how many parts a call takes every sequence: the backward, or a forward that returns hT or saves."""
+    r = load().qdelta_chunk_parts(ctypes.byref(shape), 1 if backward else 0)
+    if r < 0:
+        raise QdeltaError("unsupported or invalid shape for the chunkwise kernels")
+    return r
 
 
 def alloc_workspace(shape: QdShape, for_backward: bool, device) -> torch.Tensor:

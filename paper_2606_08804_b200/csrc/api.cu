@@ -85,16 +85,20 @@ template <class F> static cudaError_t timed(int stage, cudaStream_t s, F f) {
     return f();
 }
 
-// The two kernels of the forward, beside each other in parts where that is faster; one after the other when they are timed.
+// Kernels are timed one by one, so in one part.
+static int fwd_parts(const ChunkArgs& a) { return g_profile ? 1 : tc_fwd_parts(a); }
+static int bwd_parts(const ChunkArgs& a) { return g_profile ? 1 : tc_bwd_parts(a); }
+
+// The two kernels of the forward, beside each other in parts where that is faster.
 static cudaError_t tc_forward(const ChunkArgs& a) {
-    const int parts = g_profile ? 1 : tc_fwd_parts(a);
+    const int parts = fwd_parts(a);
     if (parts > 1) return tc_fwd(a, parts);
     const cudaError_t e = timed(ST_PREP, a.stream, [&] { return tc_prep(a); });
     return e != cudaSuccess ? e : timed(ST_CHAIN_FWD, a.stream, [&] { return tc_chain_fwd(a); });
 }
 // The two of the backward, likewise.
 static cudaError_t tc_backward(const ChunkArgs& a) {
-    const int parts = g_profile ? 1 : tc_bwd_parts(a);
+    const int parts = bwd_parts(a);
     if (parts > 1) return tc_bwd(a, parts);
     const cudaError_t e = timed(ST_CHAIN_BWD, a.stream, [&] { return tc_chain_bwd(a); });
     return e != cudaSuccess ? e : timed(ST_CHUNK_BWD, a.stream, [&] { return tc_chunk_bwd(a); });
@@ -120,6 +124,15 @@ size_t qdelta_chunk_workspace_bytes(const qd_shape* shape, int for_backward) {
 int qdelta_chunk_path(const qd_shape* shape) {
     if (check_shape(shape) != QD_OK) return -1;
     return tc_supported(*shape) ? 1 : 0;
+}
+
+int qdelta_chunk_parts(const qd_shape* shape, int backward) {
+    if (check_shape(shape) != QD_OK) return -1;
+    if (!tc_supported(*shape)) return 1;
+    ChunkArgs a{};
+    a.s = *shape;
+    a.save = true;
+    return backward ? bwd_parts(a) : fwd_parts(a);
 }
 
 int qdelta_chunk_fwd(const qd_shape* shape, const void* q, const void* k, const void* v, const void* beta,

@@ -77,6 +77,27 @@ def test_workspace_size_and_shape_validation(lib):
             chunk_workspace_bytes(bad, False)
 
 
+@pytest.mark.parametrize("seqs,chunks,fwd,bwd", [
+    (1, 1023, 1, 2), (1, 1024, 3, 2), (1, 255, 1, 1), (1, 256, 1, 2), (4, 63, 1, 1), (4, 64, 1, 2), (16, 63, 1, 1), (16, 64, 2, 2),
+    (4, 255, 1, 2), (4, 256, 3, 2), (5, 255, 2, 2), (11, 187, 2, 2), (12, 171, 2, 3), (12, 170, 2, 2), (16, 127, 2, 2), (16, 128, 2, 3),
+    (36, 128, 2, 3), (37, 128, 2, 2), (40, 119, 2, 1), (40, 120, 2, 2), (41, 512, 1, 2), (48, 143, 1, 1), (48, 144, 1, 2), (49, 512, 1, 1),
+    (32, 512, 3, 3), (128, 32, 1, 1)])
+def test_parts(lib, seqs, chunks, fwd, bwd):
+    """On either side of every bound of the rules; the last chunk of one token; the timing aid takes one part."""
+    from paper_2606_08804_b200 import binding as qd
+    for T in (64 * chunks, 64 * chunks - 63):
+        s = qd.QdShape(seqs, T, 1, 128, 128, 64, 1)
+        assert (qd.chunk_parts(s, False), qd.chunk_parts(s, True)) == (fwd, bwd)
+        qd.profile_enable(True)
+        try:
+            assert (qd.chunk_parts(s, False), qd.chunk_parts(s, True)) == (1, 1)
+        finally:
+            qd.profile_enable(False)
+    other = qd.QdShape(seqs, 64 * chunks, 1, 64, 128, 64, 1)
+    assert (qd.chunk_parts(other, False), qd.chunk_parts(other, True)) == (1, 1)
+    assert lib.qdelta_chunk_parts(ctypes.byref(qd.QdShape(seqs, 64 * chunks, 1, 96, 128, 64, 1)), 1) == -1
+
+
 def test_host_side_argument_errors_enqueue_nothing(lib):
     from paper_2606_08804_b200.binding import QdShape
     s = QdShape(1, 64, 1, 64, 64, 64, 0)

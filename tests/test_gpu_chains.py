@@ -48,10 +48,12 @@ def test_preparation_edges(T):
     _bwd_check(cfg, d, reuse=True)
 
 
-@pytest.mark.parametrize("B,H,T", [(1, 16, 64 * 64), (2, 20, 64 * 64 + 1), (1, 4, 64 * 256), (1, 1, 64 * 1024 - 63), (1, 40, 64 * 120 - 1), (2, 2, 64 * 64), (2, 8, 64 * 128 - 5), (1, 36, 64 * 128)])
-def test_in_parts(B, H, T):
-    """Long, few sequences are taken in two or three parts (the second case forward, the sixth backward alone), unless the kernels are timed one by one: the same bits either way, with the state passed on through h_T and (none asked
-    for) through the workspace, replayed from a graph, and close to the oracle."""
+@pytest.mark.parametrize("B,H,T,parts", [(1, 16, 64 * 64, (2, 2)), (2, 20, 64 * 64 + 1, (2, 1)), (1, 4, 64 * 256, (3, 2)),
+                                         (1, 1, 64 * 1024 - 63, (3, 2)), (1, 40, 64 * 120 - 1, (2, 2)), (2, 2, 64 * 64, (1, 2)),
+                                         (2, 8, 64 * 128 - 5, (2, 3)), (1, 36, 64 * 128, (2, 3)), (1, 32, 64 * 256 + 1, (3, 3))])
+def test_in_parts(B, H, T, parts):
+    """Long, few sequences are taken in `parts` (forward, backward), unless the kernels are timed one by one: the same bits either way,
+    with the state passed on through h_T and (none asked for) through the workspace, replayed from a graph, and close to the oracle."""
     import torch
 
     from gpu_util import dev_inputs
@@ -63,7 +65,7 @@ def test_in_parts(B, H, T):
     _bwd_check(cfg, d, pairs=[(0, 0), (B - 1, H - 1)], reuse=True)
     t = dev_inputs(d, cfg.dtype)
     a = [t[n] for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")]
-    results = []
+    shape = qd.make_shape(t["q"], t["v"], 64)
 
     def call(logits, norm, save, hT):
         o, h, ws = qd.chunk_fwd(*a, save_for_bwd=save, want_hT=hT, logits=logits, norm_qk=norm)
@@ -73,12 +75,9 @@ def test_in_parts(B, H, T):
         return [x for x in (o, h, *g.values(), *r.values()) if x is not None]
 
     cases = [(False, False, False, True), (False, False, True, True), (False, False, True, False), (True, True, True, True)]
-    for timed in (False, True):
-        qd.profile_enable(timed)
-        results.append([call(*c) for c in cases])
-    qd.profile_enable(False)
-    qd.profile_read(reset=True)
-    for c, x, y in zip(cases, *results):
+    assert (qd.chunk_parts(shape, False), qd.chunk_parts(shape, True)) == parts
+    results = [call(*c) for c in cases]
+    for c, x, y in zip(cases, results, _in_one_part(shape, lambda: [call(*c) for c in cases])):
         assert len(x) == len(y) and all(torch.equal(i, j) for i, j in zip(x, y)), c
 
     o, hT, ws = qd.chunk_fwd(*a, save_for_bwd=True)
@@ -91,5 +90,18 @@ def test_in_parts(B, H, T):
     for _ in range(2):
         graph.replay()
     torch.cuda.synchronize()
-    for x, y in zip((o, hT, *g.values()), results[0][1]):
+    for x, y in zip((o, hT, *g.values()), results[1]):
         assert torch.equal(x, y)
+
+
+def _in_one_part(shape, f):
+    """f() with the kernels timed one by one, which takes one part."""
+    from paper_2606_08804_b200 import binding as qd
+
+    qd.profile_enable(True)
+    try:
+        assert (qd.chunk_parts(shape, False), qd.chunk_parts(shape, True)) == (1, 1)
+        return f()
+    finally:
+        qd.profile_enable(False)
+        qd.profile_read(reset=True)
