@@ -105,3 +105,85 @@ def _in_one_part(shape, f):
     finally:
         qd.profile_enable(False)
         qd.profile_read(reset=True)
+
+
+@pytest.mark.parametrize("without", ["h0", "dhT", "dh0", "h0 dhT dh0", "alpha", "lam", "alpha lam", "alpha lam h0 dhT dh0"])
+@pytest.mark.parametrize("B,H,T", [(1, 16, 64 * 128 - 5), (3, 4, 64 * 256)])
+def test_in_parts_without(B, H, T, without):
+    """Inputs that a call may leave out, and dh0 not asked for, in two and three parts: the bits of one part; and h_T in h0's place."""
+    import torch
+
+    from gpu_util import dev_inputs
+    from paper_2606_08804_b200 import binding as qd
+
+    cfg = replace(gen.CONFIGS["cfg2"], B=B, H=H, T=T, regime="alpha_slow", seed=353)
+    d = gen.make_chunk_inputs(cfg)
+    for n in without.split():
+        d[n] = None
+    t = dev_inputs(d, cfg.dtype)
+    a = [t[n] for n in ("q", "k", "v", "beta", "alpha", "lam")]
+    shape, want = qd.make_shape(t["q"], t["v"], 64), "dh0" not in without.split()
+    assert (qd.chunk_parts(shape, False), qd.chunk_parts(shape, True)) == (2 if T < 64 * 255 else 3, 3)
+
+    def call():
+        r = []
+        for save in (False, True):
+            o, hT, ws = qd.chunk_fwd(*a, t["h0"], save_for_bwd=save)
+            r += [o, hT]
+        for kw in (dict(workspace=ws, reuse_fwd=True), {}):
+            # gradients of coefficients that are absent, on request
+            out = {n: torch.full((B, T, H), float("nan"), device="cuda") for n, x in (("dalpha", t["alpha"]), ("dlam", t["lam"])) if x is None}
+            for o in ({}, out) if out else ({},):
+                g = qd.chunk_bwd(*a, t["h0"], t["dO"], t["dhT"], want_dh0=want, out=dict(o), **kw)
+                assert (g["dh0"] is not None) == want
+                r += [x for x in g.values() if x is not None]
+        if t["h0"] is not None:
+            state = t["h0"].clone()
+            o, _, ws = qd.chunk_fwd(*a, state, hT=state)
+            r += [o, state]
+        assert qd.workspace_status(ws) == 0
+        return r
+
+    x, y = call(), _in_one_part(shape, call)
+    assert len(x) == len(y) and all(torch.equal(i, j) for i, j in zip(x, y))
+
+
+@pytest.mark.parametrize("B,H,T", [(1, 16, 64 * 128), (1, 4, 64 * 256 - 1)])
+def test_in_parts_between_other_kernels(B, H, T):
+    """Kernels that write the inputs right before the calls, and overwrite them and the outputs' copies right after, in one stream: the
+    preparation and the chunk backward of a part, which do not wait for the chain before them, are ordered with both."""
+    import torch
+
+    from gpu_util import dev_inputs
+    from paper_2606_08804_b200 import binding as qd
+
+    cfg = replace(gen.CONFIGS["cfg2"], B=B, H=H, T=T, regime="trained_like", seed=359)
+    t = dev_inputs(gen.make_chunk_inputs(cfg), cfg.dtype)
+    names = ("q", "k", "v", "beta", "alpha", "lam", "h0", "dO", "dhT")
+    shape = qd.make_shape(t["q"], t["v"], 64)
+    assert qd.chunk_parts(shape, True) > 1
+
+    def pair(x, ws, o, hT, g):
+        qd.chunk_fwd(*(x[n] for n in names[:7]), save_for_bwd=True, workspace=ws, o=o, hT=hT)
+        qd.chunk_bwd(*(x[n] for n in names[:7]), x["dO"], x["dhT"], workspace=ws, reuse_fwd=True, out=g)
+
+    want = [None, None, {}]
+    want[0], want[1], ws = qd.chunk_fwd(*(t[n] for n in names[:7]), save_for_bwd=True)
+    want[2] = qd.chunk_bwd(*(t[n] for n in names[:7]), t["dO"], t["dhT"], workspace=ws, reuse_fwd=True)
+    o, hT, g = torch.empty_like(want[0]), torch.empty_like(want[1]), {n: torch.empty_like(x) for n, x in want[2].items()}
+    outs = [o, hT, *g.values()]
+    x = {n: torch.full_like(t[n], float("nan")) for n in names}
+    copies = [[] for _ in range(3)]
+    for c in copies:
+        for n in names:
+            x[n].copy_(t[n])                              # the producers
+        pair(x, ws, o, hT, g)
+        for n in names:
+            x[n].fill_(float("nan"))                      # the next user of the buffers
+        for y in outs:
+            c.append(y.clone())
+            y.fill_(float("nan"))
+    torch.cuda.synchronize()
+    assert qd.workspace_status(ws) == 0
+    for c in copies:
+        assert all(torch.equal(i, j) for i, j in zip(c, [want[0], want[1], *want[2].values()]))
