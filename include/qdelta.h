@@ -22,9 +22,10 @@
  *     never allocates, frees or synchronises; all work is enqueued on `stream`.
  *   - Ordering: a call reads its inputs only after everything enqueued on `stream` before the call has
  *     completed, and everything enqueued on `stream` after the call sees its outputs complete -- ordinary
- *     stream order.  (Internally the kernels of one call overlap their set-up with the tail of the kernel
- *     before them; none of them touches caller data, or workspace contents it depends on, before that
- *     kernel has completed.)  Work on OTHER streams needs events as usual.
+ *     stream order.  (Internally kernels overlap: the first of a call touches nothing before everything older has
+ *     completed; a later one may work while the one before it runs, on inputs, outputs and parts of the workspace that
+ *     that one does not write, and does not read where the later one writes; the last completes after all others.)
+ *     Work on OTHER streams needs events as usual.
  *   - Inputs are read-only.  Outputs are fully overwritten.  q,k,v,o,dO,dq,dk,dv, the
  *     states and the workspace must be 16-byte aligned; coefficient tensors (and the decode step's o)
  *     need only the alignment of their element type.

@@ -75,7 +75,7 @@ inline int tc_padded_T(const qd_shape& s) { return (s.T + 2 * kChunk - 1) / (2 *
 cudaError_t set_max_smem_once(const void* kernel, size_t bytes);
 
 // Launch with the programmatic-stream-serialization attribute: the kernel may begin before the previous kernel of the
-// stream has finished and orders itself with grid_dep_wait() (see sm100.cuh).
+// stream has finished; what it may touch before grid_dep_wait() returns stands in sm100.cuh.
 template <class... KArgs, class... Args>
 cudaError_t launch_overlapped(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args&&... args) {
     cudaLaunchConfig_t cfg{};

@@ -80,9 +80,13 @@ __device__ __forceinline__ bool wait_on(uint64_t* bar, uint32_t parity, volatile
 // ---- programmatic dependent launch ------------------------------------------------------------------------------
 // A kernel launched with cudaLaunchAttributeProgrammaticStreamSerialization may begin while the kernel before it in
 // the stream is still running.  grid_dep_wait() returns once that kernel has completed and its writes are visible
-// (at once if the launch had no such relation); everything before it may only touch data that is older than the
-// preceding kernel.  grid_dep_launch() lets the kernel after this one begin; the kernels here call it right after
-// their own wait, so a kernel that has begun can rely on everything up to its predecessor's predecessor.
+// (at once if the launch had no such relation); what a kernel touches before it, neither that kernel nor one that may
+// run beside that kernel writes.  grid_dep_launch() lets the kernel after this one begin.  Most kernels here call it right after
+// their own wait; a kernel behind one of those can rely on everything up to its predecessor's predecessor.
+// The preparation and the chunk backward of a part (`beside`) do not wait before they work: the kernel before them is a state
+// chain that they do not depend on, and they touch rows of their own chunks and what is older than that chain.  Their first
+// CTA waits for it at its end, so that whoever waits for them comes after the chain too.  Before that wait a kernel behind a
+// `beside` one may rely on NOTHING of that chain: only on what is older than it.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
