@@ -74,11 +74,11 @@ def stage_bytes_per_token_head(dk, dv, C):
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch: NOT measured by this run (a profiler cannot run inside the
-# timed program); constants from the ncu capture summarised in profiles/tc_kernels_fullsize_counters_cfg2.md (full-size
-# cfg2).  Other workloads: not captured.
+# timed program); constants from an ncu capture of the full-size cfg2, one launch of each kernel.  Other workloads: not
+# captured.
 NCU_TRAFFIC_BYTES = {"cfg2": {"prep": 419.0e6, "chain_fwd": 534.8e6, "chain_bwd": 468.9e6, "chunk_bwd": 922.6e6}}
-NCU_TRAFFIC_SOURCE = "constant from profiles/tc_kernels_fullsize_counters_cfg2.md (ncu, one launch each); not measured by this run"
-# which pass of the path a kernel belongs to (its share of the algorithmic bytes of SURVEY section 8(d))
+NCU_TRAFFIC_SOURCE = "constant from an ncu capture of this workload (one launch of each kernel); not measured by this run"
+# which pass of the path a kernel belongs to
 STAGE_PASS = {"prep": "fwd", "chain_fwd": "fwd", "chain_bwd": "bwd", "chunk_bwd": "bwd"}
 
 
@@ -252,7 +252,11 @@ def extra_workload(torch, qd, gen, cfg, pk, pk_kind, backward, steps, regions, d
     stage_ms = {n: v[0] / v[1] for n, v in qd.profile_read(reset=True).items() if v[1] > 0}
     rl = path_roofline(cfg, pk, fwd=True, bwd=backward)
     ms = st["ms_per_step_median"]
-    out = {"workload": workload_name(cfg, backward), "ms_per_step": ms, "tokens_per_s": cfg.B * cfg.T / (ms * 1e-3),
+    # the stage times are those of one part, whatever the timed steps take
+    parts = {"forward": qd.chunk_parts(w.shape, False)}
+    if backward:
+        parts["backward"] = qd.chunk_parts(w.shape, True)
+    out = {"workload": workload_name(cfg, backward), "parts_of_timed_step": parts, "ms_per_step": ms, "tokens_per_s": cfg.B * cfg.T / (ms * 1e-3),
            "roofline_ms": rl["roofline_ms"], "frac": rl["roofline_ms"] / ms, "frac_nominal": rl["roofline_ms_nominal"] / ms,
            "peak_kind": "of " + pk_kind, "regions": st, "stage_ms_per_launch": stage_ms}
     if drop:
@@ -455,7 +459,9 @@ def run_ours(args, cfg):
                 "stage_floor": {n: {"bytes_per_launch": sb[n] * th, "ms_at_peak": sb[n] * th / (pk["hbm_gbs"] * 1e6),
                                     "achieved_gbs_of_staged_bytes": sb[n] * th / (stage_ms[n] * 1e-3) / 1e9}
                                 for n in stage_ms}}
-    launches = int(sum(v[1] for v in stages.values()))
+    # two kernels per part; the pass that timed the kernels took one part
+    parts = {"forward": qd.chunk_parts(w.shape, False), "backward": qd.chunk_parts(w.shape, True)}
+    launches = args.steps * 2 * sum(parts.values())
 
     extras = {}
     if rank == 0 and world == 1 and not args.no_extras:
@@ -492,7 +498,9 @@ def run_ours(args, cfg):
                                  "stream, max over ranks" % (len(times), args.steps),
                        "clock_sampling": "nvidia-smi during the timed regions and 1 s more of the same step loop",
                        "kernel_timing": "per-kernel CUDA events in a separate pass over K steps (events between "
-                                        "launches would serialise the overlapped launches of the timed regions)",
+                                        "launches would serialise the overlapped launches of the timed regions), every "
+                                        "sequence in one part",
+                       "parts_of_timed_step": parts,
                        "tokens_per_step": tokens_step, "parallelism": "batch sharded over %d rank(s), no collective" % world},
             "clocks": clocks, "regions": regions,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,

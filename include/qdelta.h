@@ -177,6 +177,8 @@ int qdelta_workspace_status(const void *workspace, int *status_out, qd_stream st
  * the entry points enqueue is bracketed by two CUDA events recorded on the caller's stream;
  * qdelta_profile_read waits for the recorded events, adds their elapsed times to per-stage totals and
  * returns the total milliseconds and number of launches of `stage` (reset != 0 clears that total).
+ * Timed so, kernels run one after the other and take every sequence in one part (qdelta_chunk_parts): where a call
+ * otherwise works on one part beside another, its stages add up to more than the call takes.
  * Stages are numbered 0 .. qdelta_profile_stage_count()-1; qdelta_profile_stage_name names them.
  * Events are created on first use and reused.  Not thread-safe; off by default.
  */

@@ -93,7 +93,7 @@ def load():
 
 
 def profile_enable(on: bool) -> None:
-    """Turn the library's per-kernel CUDA-event timing on or off."""
+    """Turn the library's per-kernel CUDA-event timing on or off.  Kernels then run one by one, every sequence in one part."""
     load().qdelta_profile_enable(1 if on else 0)
 
 
