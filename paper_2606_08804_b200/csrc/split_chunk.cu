@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(NT + kLoaders) k_chain_fwd(Ptrs p, int DV) {
         }
     }
     if (p.hT) {
-    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");        // the state is complete
+        asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");    // the state is complete
         for (int e = tid; e < DK * DS; e += NT)
             p.hT[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] = sh[(e / DS) * LS + e % DS];
     }
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(NT + kLoaders) k_chain_bwd(Ptrs p, int DV) {
         }
     }
     if (p.dh0) {
-    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");        // the gradient is complete
+        asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");    // the gradient is complete
         for (int e = tid; e < DK * DS; e += NT)
             p.dh0[((size_t)bh * DK + e / DS) * DV + j0 + e % DS] = sdh[(e / DS) * LS + e % DS];
     }
@@ -656,11 +656,12 @@ cudaError_t chunk_bwd_for(const ChunkArgs& a, const Ptrs& p) {
 // d_v columns that one CTA of the state chains owns: 16 while each CTA then has an SM of its own, because a chain's time is its
 // dependent steps; 32, which read W<-, Q, K and P half as often, beyond.  Both kernels turn there.  Training pass of 512 tokens,
 // narrow against wide, on either side of 148 narrow CTAs (d_k x d_v, sequences):
-//   fp32   64 x 64    37: 150 against 180 us   38: 237 against 219      bf16   64 x 64    37:  87 against  97   38: 123 against 118
-//         128 x 64    37: 230 against 273      38: 375 against 330            128 x 64    37: 121 against 137   38: 195 against 168
-//          64 x 128   18: 123 against 151      19: 214 against 194             64 x 128   18:  74 against  84   19: 114 against 108
-//         128 x 128   18: 177 against 215      19: 334 against 291
-// (measured before the copies had warps of their own, which narrow slices gain more from).  The same with 2048 tokens, and up to 800 narrow CTAs wide slices stay ahead, but for fp32 with d_k = 64 at 352 (narrow by 3 %).
+//   fp32   64 x 64    37: 145 against 169 us   38: 226 against 202      bf16   64 x 64    37:  83 against  96   38: 124 against 116
+//         128 x 64    37: 219 against 262      38: 354 against 318            128 x 64    37: 112 against 132   38: 193 against 163
+//          64 x 128   18: 117 against 139      19: 207 against 181             64 x 128   18:  70 against  82   19: 112 against 105
+//         128 x 128   18: 164 against 199      19: 310 against 272
+// With 2048 tokens both sides are further apart (fp32 128 x 128 661 against 792, 1046 against 866); between 160 and 800 narrow CTAs wide
+// slices stay ahead, least with fp32 at 300 to 400 of them (1.3 - 3.5 %).
 int split_slice(const qd_shape& s) { return (long long)s.B * s.H * (s.dv / 16) <= kSMs ? 16 : 32; }
 
 #define QD_BY_DIMS(fn, a, p)                                                                                  \

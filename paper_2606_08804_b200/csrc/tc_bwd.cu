@@ -37,9 +37,6 @@ __device__ __forceinline__ void fold(float* v, int lane, int off) {
 }
 
 // =================================================================================================
-struct BwdMaps {               // boxes of 64 rows for token tiles, 128 for tiles by d_v or d_k, `rows` for the chain's two stores
-    CUtensorMap Q, K, V, dO, Mt, P, Dt, dDt, Hs, dHs, Wt, Qg, dHs_store, dDt_store, dQ, dK, dV;
-};
 struct ChainBwdParams {
     int Tp, H, N, Ns;          // N chunks of a sequence, from n0 on; Tp = 64 Ns rows per sequence in the workspace
     int n0;
@@ -398,9 +395,6 @@ constexpr int kBwdNb = kBwdCompute + 32;                 // participants of a na
 // TMA warp only arrives
 constexpr int kNbC = 1, kNbX = 2, kNbDW = 3, kNbDTb = 4, kNbN = 5, kNbDXK = 6, kNbOut = 7, kNbDV = 8, kNbDVt = 10, kNbSum = 11, kNbTok = 12, kNbEnd = 13;
 constexpr int kNbSumN = kBwdCompute + C;
-
-// 8 TMEM columns of this thread's lane (no wait)
-__device__ __forceinline__ void ld8(uint32_t taddr, float* v) { tmem_ld8(taddr, v); }
 
 struct ChunkBars { uint64_t load, d, h, qk, st, a, b, c, m2, m3, m4, m5; };
 // What the warps tell each other; `_` arrays by parity of the chunk, so that the token threads can publish a chunk
@@ -817,7 +811,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
 #pragma unroll
     for (int g8 = 0; g8 < kG8; ++g8) {
         float dw[8];
-        ld8(my(T3) + g8 * 8, dw);
+        tmem_ld8(my(T3) + g8 * 8, dw);
         tmem_ld_wait();
         sts128(sm + odW + sw128_chunk(l, wg * kG8 + g8), pack8(dw));
     }
@@ -1120,7 +1114,9 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     }  // epilogue threads
     tc_fence_before();
     __syncthreads();
-    if (tid == kBwdCompute && s_abort) { mbar_wait(&bar.load, 0); mbar_wait(&bar.d, 0); mbar_wait(&bar.h, 0); mbar_wait(&bar.qk, 0); }   // one more bounded chance for copies in flight
+    if (tid == kBwdCompute && s_abort) {                         // one more bounded chance for copies in flight
+        mbar_wait(&bar.load, 0); mbar_wait(&bar.d, 0); mbar_wait(&bar.h, 0); mbar_wait(&bar.qk, 0);
+    }
     if (tid < 32) tmem_dealloc(tb, 512);
     if (tid == 0 && blockIdx.x == 0) grid_dep_wait();            // when this kernel has completed, so has the one before it
 }
