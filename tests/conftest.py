@@ -26,6 +26,18 @@ def pytest_collection_modifyitems(config, items):
             item.add_marker(skip)
 
 
+@pytest.fixture(scope="module", autouse=True)
+def _memory_given_back():
+    """Every module begins with nothing in torch's pool: a test that limits the memory would find room there that another test left."""
+    yield
+    import gc
+
+    import torch
+    if torch.cuda.is_available():
+        gc.collect()
+        torch.cuda.empty_cache()
+
+
 def pytest_sessionfinish(session, exitstatus):
     """With QD_PARITY_LOG=<file>: dump the error figures the GPU parity tests collected (max-normalised, rms-relative,
     worst sequence) as JSON."""
