@@ -3,8 +3,9 @@
 //   o = h_new^T q = alpha h^T q + (k.q) delta .
 // A CTA owns DVS columns of one state (columns evolve independently); every thread keeps its part of the slice in
 // registers between the only read and the only write of the state, all loads are issued before the first use.
-// One token is bound by HBM traffic: 80.4 us for 4096 states of 128 x 128 in fp32, 1.02 of the measured copy bandwidth (44 - 46
-// of 41 us at that bandwidth with a bf16 state, whose rows are read 16 bytes per thread like those of an fp32 one).
+// One token is bound by HBM traffic: 80.5 us for 4096 states of 128 x 128 in fp32, 1.04 of the measured copy bandwidth (44 on the same
+// tokens again and again, 46.7 on new ones, of 42 us at that bandwidth with a bf16 state, whose rows are read 16 bytes per thread
+// like those of an fp32 one).
 #include "internal.h"
 #include "sm100.cuh"
 
