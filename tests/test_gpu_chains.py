@@ -187,3 +187,49 @@ def test_in_parts_between_other_kernels(B, H, T):
     assert qd.workspace_status(ws) == 0
     for c in copies:
         assert all(torch.equal(i, j) for i, j in zip(c, [want[0], want[1], *want[2].values()]))
+
+
+def test_in_parts_on_two_streams():
+    """Two calls in parts at a time, each on its own stream, thread and workspace, with a decode on a third: the bits of one after the other."""
+    import threading
+
+    import torch
+
+    from gpu_util import dev_inputs
+    from paper_2606_08804_b200 import binding as qd
+
+    work = []
+    for H, T, seed in ((16, 64 * 128 - 5, 367), (4, 64 * 256, 373)):
+        t = dev_inputs(gen.make_chunk_inputs(replace(gen.CONFIGS["cfg2"], B=1, H=H, T=T, regime="trained_like", seed=seed)), "bf16")
+        a = [t[n] for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")]
+        ws = qd.alloc_workspace(qd.make_shape(t["q"], t["v"], 64), True, "cuda")
+        assert qd.chunk_parts(qd.make_shape(t["q"], t["v"], 64), True) > 1
+
+        def pair(a=a, t=t, ws=ws):
+            o, hT, _ = qd.chunk_fwd(*a, save_for_bwd=True, workspace=ws)
+            return [o, hT, *qd.chunk_bwd(*a, t["dO"], t["dhT"], workspace=ws, reuse_fwd=True).values()]
+
+        work.append(pair)
+    x = [y[:, 0].contiguous() for y in a[:6]]
+    work.append(lambda: [qd.recurrent_step(*x, t["h0"].clone())])
+    want = [f() for f in work]
+    torch.cuda.synchronize()
+    got, errors = [[] for _ in work], []
+
+    def run(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(6):
+                    got[i].append(work[i]())
+                torch.cuda.current_stream().synchronize()
+        except Exception as e:          # noqa: BLE001 -- told to the test below
+            errors.append(e)
+
+    threads = [threading.Thread(target=run, args=(i,)) for i in range(len(work))]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not errors, errors
+    for w, rounds in zip(want, got):
+        assert len(rounds) == 6 and all(torch.equal(p, q) for r in rounds for p, q in zip(r, w))
