@@ -189,6 +189,21 @@ __device__ __forceinline__ void tmem_ld_frag2(uint32_t taddr, float* v) {       
     asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld_frag4(uint32_t taddr, float* v) {            // 32 columns
+    uint32_t* r = reinterpret_cast<uint32_t*>(v);
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr) : "memory");
+}
+// Store bf16 pairs in the same layout, 16 lanes x 4 N packed columns: the packed pair of columns 2 (t % 4) and 2 (t % 4) + 1 of every 8, of
+// row t / 4 (r[2 g]) and row t / 4 + 8 (r[2 g + 1])
+__device__ __forceinline__ void tmem_st_frag2(uint32_t taddr, const uint32_t* r) {   // 16 columns
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x2.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void tmem_st_frag4(uint32_t taddr, const uint32_t* r) {   // 32 columns
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+}
 // Four 8 x 8 bf16 matrices; lane l passes the address of row l % 8 of matrix l / 8.  T: transposed, register m of thread t
 // holds elements (row 2 (t % 4) + {0, 1}, column t / 4) of matrix m instead of (row t / 4, columns 2 (t % 4) + {0, 1})
 template <bool T>
@@ -311,11 +326,11 @@ __device__ __forceinline__ void umma_product_w(uint32_t d_tmem, uint32_t a_saddr
     }
 }
 // D[tmem] (+)= A[tmem] * B[smem]: the A operand (M = 128 rows on the 128 lanes, bf16 pairs packed two per
-// 32-bit column: column c of lane m holds A[m][2c], A[m][2c+1]) is read from tensor memory.
-template <bool B_MN>
+// 32-bit column: column c of lane m holds A[m][2c], A[m][2c+1]) is read from tensor memory.  M = 64: A's rows on the lanes of the product's.
+template <bool B_MN, int M = 128>
 __device__ __forceinline__ void umma_product_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_saddr, uint32_t b_blk, int N, int K,
                                                   bool accumulate, uint32_t issue, bool a_neg = false) {
-    const uint32_t idesc = make_idesc(128, N, false, B_MN, a_neg);
+    const uint32_t idesc = make_idesc(M, N, false, B_MN, a_neg);
     const uint64_t b0 = B_MN ? desc_mnmajor(b_saddr, b_blk) : desc_kmajor(b_saddr);
 #pragma unroll
     for (int k = 0; k < K; k += 16) {

@@ -6,9 +6,8 @@
 //                   per chunk, in bf16:  Qg = diag(gamma) Q  [token][dk],
 //                   P = Gamma o (Q K^T) causal incl. diagonal [token][64],
 //                   Wt = (T diag(gamma) X)^T  [dk][64 tokens],   Ut = (T V)^T  [dv][64 tokens].
-//   k_tc_chain_fwd  one CTA per (batch, head), or two that share its d_v rows (chain_rows): walks the chunks
-//                   in order with the fp32 state in registers (a thread owns 32 columns of one row of h^T),
-//                   everything transposed so that d_v is the MMA M dimension:
+//   k_tc_chain_fwd  one CTA per (batch, head), or two that share its d_v rows (chain_rows; k_tc_chain_fwd_half): walks the
+//                   chunks in order with the fp32 state in registers, everything transposed so that d_v is the MMA M dimension:
 //                     Delta^T = Ut - h^T Wt            O^T = h^T Qg^T + Delta^T P^T
 //                     h^T <- gamma_C h^T + (Delta diag(gamma_C/gamma))^T K
 // With few long sequences the two run beside each other, part by part (tc_fwd_parts).
@@ -420,6 +419,8 @@ struct ChainParams {
     const float* g;
     const float* h0;
     float* hT;
+    int T;                     // tokens per sequence
+    bf16* o;                   // [B][T][H][D], as mapO
     int scaled;                // 0: no forget gate and no key normalisation: every per-token factor on Delta is 1
     const float* rk;           // non-null (QD_NORM_QK): 1/|k_t| per workspace row; the keys are read un-normalised and
                                // the factor is folded into the per-token scale of Delta
@@ -427,7 +428,7 @@ struct ChainParams {
 };
 
 // Tiles of a chunk in shared memory.  Wt 16K | Ut 16K, three deep (Delta^T is staged over Ut and held until it has been
-// read); Qg 16K | K 16K | P 8K, two deep; the exit state 32K (16K with 64 rows: two deep then); half an output tile 8K.
+// read); Qg 16K | K 16K | P 8K, two deep; the exit state 32K; half an output tile 8K.
 constexpr int kDeepA = 3, kStageA = 32768, kStageB = 40960;
 constexpr int kOffB = kDeepA * kStageA, kOffH = kOffB + 2 * kStageB, kOffO = kOffH + 32768;
 constexpr int kChainSmem = kOffO + 8192 + 1024;
@@ -452,12 +453,12 @@ constexpr int kBarH = 1, kBarD = 2, kBarOut = 3;
 //    loads and the 16 KB of its output take 2150 cycles, and the 48 KB of Delta^T and entry state that a forward saves for the
 //    backward 1300 more.  (Ordinary stores, by one or two warps from the tiles or by the epilogue from its registers, were
 //    slower: 4500 - 5000 cycles per chunk.)  So with few heads the d_v rows of a head, which evolve independently, are shared by
-//    two CTAs (ROWS = 64): each loads what both need, but only its half of Ut, and stores its half of everything.
+//    two CTAs (k_tc_chain_fwd_half): each loads what both need, but only its half of Ut, and stores its half of everything.
 // SAVE: also store, per chunk, the bf16 entry state (mapHs) and Delta^T (mapDt).  Compile-time: with a flag prompts of 4 sequences
 // of 64 chunks took 80.2 us, so 77.3.
 // Compute warpgroup w owns tokens [16w, 16w+16) of the 64-column accumulators and d_k columns
 // [32w, 32w+32) of the state; thread l of a warpgroup owns TMEM lane l = d_v index.
-template <int ROWS, bool SAVE>
+template <bool SAVE>
 __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_constant__ CUtensorMap mapWt,
                                                                 const __grid_constant__ CUtensorMap mapUt,
                                                                 const __grid_constant__ CUtensorMap mapQg,
@@ -469,14 +470,13 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                                                                 ChainParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    constexpr int rows = ROWS, two = rows == D ? 0 : 1;   // d_v rows of the state in this CTA; whether the exit state is staged two deep
-    unsigned char* sHs = smem + kOffH;              // h^T [rows dv][128 dk] for its store, 2 blocks of [rows lines][64]
+    unsigned char* sHs = smem + kOffH;              // h^T [128 dv][128 dk] for its store, 2 blocks of [128 lines][64]
     unsigned char* sO = smem + kOffO;               // half an output tile: [32 tokens][128 dv], 2 blocks of [32 lines][64]
     // Where one side may run ahead of the other there is a barrier per buffer; it comes round only after the other side has
     // waited for it.  bar_e: every product of a chunk has finished; bar_dt, bar_ht: Delta^T / exit state staged for their stores
     // (one arrival per compute warp); bar_df, bar_hf: they have been read; bar_o, bar_of: an output accumulator is complete /
     // has been read.
-    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_df[kDeepA], bar_ht[2], bar_hf[2], bar_a, bar_b, bar_o[2], bar_of[2];
+    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_df[kDeepA], bar_ht, bar_hf, bar_a, bar_b, bar_o[2], bar_of[2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
     // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the TMA warp before it arrives on the
@@ -484,14 +484,14 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     __shared__ __align__(16) float sG[kDeepA][68];
 
     const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, l = tid & 127, wq = warp & 3;
-    constexpr int nwq = rows / 32, nb = 4 * rows + 32, parts = D / rows;      // warps of a warpgroup that have rows; barrier participants
-    const int bh = blockIdx.x / parts, v0 = (blockIdx.x % parts) * rows, b = bh / p.H, hh = bh % p.H;
+    constexpr int nb = kChainCompute + 32;                            // participants of a named barrier
+    const int bh = blockIdx.x, b = bh / p.H, hh = bh % p.H;
 
     if (tid == 0) {
-        for (int i = 0; i < kDeepA; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_dt[i], 4 * nwq); mbar_init(&bar_df[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&bar_lb[i], 1); mbar_init(&bar_e[i], 1); mbar_init(&bar_o[i], 1); mbar_init(&bar_of[i], nwq); }
+        for (int i = 0; i < kDeepA; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_dt[i], 16); mbar_init(&bar_df[i], 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar_lb[i], 1); mbar_init(&bar_e[i], 1); mbar_init(&bar_o[i], 1); mbar_init(&bar_of[i], 4); }
         mbar_init(&bar_a, 1); mbar_init(&bar_b, 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(&bar_ht[i], 4 * nwq); mbar_init(&bar_hf[i], 1); }
+        mbar_init(&bar_ht, 16); mbar_init(&bar_hf, 1);
         mbar_init_fence();
         s_abort = 0;
     }
@@ -511,14 +511,12 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     const size_t row0 = (size_t)bh * p.Tp + tok0, tile0 = (size_t)bh * p.Ns + p.n0;
     const float* gseq = p.g + row0;
 
-    if (warp < kMmaWarp && wq >= nwq) {
-        // lanes without a row: straight to the end
-    } else if (warp < kOutWarp) {
+    if (warp < kOutWarp) {
         // ---------------------------------- compute warps ----------------------------------
         float h[32];      // h^T[j = l][32 wg .. 32 wg + 31], fp32
         if (p.h0_late) grid_dep_wait();
         if (p.h0) {
-            const float* src = p.h0 + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
+            const float* src = p.h0 + (size_t)bh * D * D + (size_t)(32 * wg) * D + l;
 #pragma unroll
             for (int i = 0; i < 32; ++i) h[i] = __ldcg(src + (size_t)i * D);      // not from L1: it may be new
         } else {
@@ -544,11 +542,10 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         };
         // the state that chunk n begins with as a tile: 64-column block wg >> 1, 16-byte chunks 4 (wg & 1) ..
         auto save_h = [&](int n) {
-            const int sb = n & two;
-            if (n > two) wait(&bar_hf[sb], ((n >> two) - 1) & 1);
+            if (n > 0) wait(&bar_hf, (n - 1) & 1);
 #pragma unroll
-            for (int ch = 0; ch < 4; ++ch) sts128(sHs + sb * 16384 + (wg >> 1) * (rows * 128) + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(h + ch * 8));
-            staged(&bar_ht[sb]);
+            for (int ch = 0; ch < 4; ++ch) sts128(sHs + (wg >> 1) * 16384 + sw128_chunk(l, (wg & 1) * 4 + ch), pack8(h + ch * 8));
+            staged(&bar_ht);
         };
         put_h();
         if (SAVE) save_h(0);
@@ -606,7 +603,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         // a wait has expired: keep step with the MMA warp, which comes to every one of them (odd counts: H is next)
         for (; pending > 0; --pending) nb_sync(pending & 1 ? kBarH : kBarD, nb);
         if (p.hT && !s_abort) {
-            float* dst = p.hT + (size_t)bh * D * D + (size_t)(32 * wg) * D + v0 + l;
+            float* dst = p.hT + (size_t)bh * D * D + (size_t)(32 * wg) * D + l;
 #pragma unroll
             for (int i = 0; i < 32; ++i) dst[(size_t)i * D] = h[i];
         }
@@ -635,14 +632,14 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                     if ((tid & 31) == 0) mbar_arrive(&bar_of[ob]);
                 }
                 if (first) tma_store_wait_read_n<0>();    // the half tile before has been read
-                nb_sync(kBarOut, rows);
+                nb_sync(kBarOut, 128);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) sts16(stg + (i >> 3) * 1024 + xoff[i & 7], __float2bfloat16_rn(v[i]));
                 fence_proxy_async();
-                nb_sync(kBarOut, rows);
+                nb_sync(kBarOut, 128);
                 if (first) {                              // rows past the end of the sequence are skipped
-                    tma_store_3d(&mapO, sO, hh * D + v0, tok0 + n * C + half * 32, b);
-                    if (rows == D) tma_store_3d(&mapO, sO + 4096, hh * D + 64, tok0 + n * C + half * 32, b);
+                    tma_store_3d(&mapO, sO, hh * D, tok0 + n * C + half * 32, b);
+                    tma_store_3d(&mapO, sO + 4096, hh * D + 64, tok0 + n * C + half * 32, b);
                     tma_store_commit();
                 }
             }
@@ -689,24 +686,20 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             grid_dep_wait();
             int s = 0;
             for (int n = 0; n < p.N; ++n) {
-                const int y = (int)((tile0 + n) * D) + v0;
-                const int sb = n & two;
-                wait(&bar_ht[sb], (n >> two) & 1);        // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
-                tma_store_2d(&mapHs, sHs + sb * 16384, 0, y);
-                tma_store_2d(&mapHs, sHs + sb * 16384 + rows * 128, 64, y);
+                const int y = (int)((tile0 + n) * D);
+                wait(&bar_ht, n & 1);                     // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
+                tma_store_2d(&mapHs, sHs, 0, y);
+                tma_store_2d(&mapHs, sHs + 16384, 64, y);
                 tma_store_commit();
-                if (n > 0) {                              // Delta^T of chunk n - 1 has been read, and the entry state before it
+                if (n > 0) {                              // Delta^T of chunk n - 1 has been read
                     tma_store_wait_read_n<1>();
                     mbar_arrive(&bar_df[s == 0 ? kDeepA - 1 : s - 1]);
-                    if (two) mbar_arrive(&bar_hf[sb ^ 1]);
                 }
                 wait(&bar_dt[s], (n / kDeepA) & 1);       // Delta^T of chunk n is staged
                 tma_store_2d(&mapDt, smem + s * kStageA + 16384, 0, y);
                 tma_store_commit();
-                if (!two) {
-                    tma_store_wait_read_n<1>();           // the entry state has been read
-                    mbar_arrive(&bar_hf[0]);
-                }
+                tma_store_wait_read_n<1>();               // the entry state has been read
+                mbar_arrive(&bar_hf);
                 if (++s == kDeepA) s = 0;
             }
             tma_store_wait_all();
@@ -732,9 +725,9 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             __syncwarp();
             if (lead) {
                 const int yc = (int)((tile0 + n) * D);
-                mbar_expect_tx(&bar_la[s], 16384 + rows * 128);
+                mbar_expect_tx(&bar_la[s], 32768);
                 tma_load_2d(smem + s * kStageA, &mapWt, 0, yc, &bar_la[s]);
-                tma_load_2d(smem + s * kStageA + 16384, &mapUt, 0, yc + v0, &bar_la[s]);
+                tma_load_2d(smem + s * kStageA + 16384, &mapUt, 0, yc, &bar_la[s]);
             }
             if (n + 1 < p.N) fetch_g(n + 1);
         };
@@ -769,6 +762,331 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         if (lead && s_abort) {            // one more bounded chance for copies in flight
             for (int i = 0; i < kDeepA; ++i) mbar_wait(&bar_la[i], 0);
             for (int i = 0; i < 2; ++i) mbar_wait(&bar_lb[i], 0);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (tid < 32) tmem_dealloc(tbase, 512);
+}
+
+// Tiles of a chunk for 64 of the 128 d_v rows, all three deep: Wt 16K | Ut 8K; Qg 16K | K 16K | P 8K.  Then what goes out, one deep: the
+// entry state 16K (2 blocks of [64 dv][64]) | Delta^T 8K | the output 8K ([64 tokens][64 dv]).
+constexpr int kHalfDeep = 3, kHalfStageA = 24576, kHalfStageB = 40960;
+constexpr int kHalfOffB = kHalfDeep * kHalfStageA, kHalfOffS = kHalfOffB + kHalfDeep * kHalfStageB, kHalfOffO = kHalfOffS + 24576;
+constexpr int kHalfSmem = kHalfOffO + 8192 + 1024;
+constexpr int kHalfThreads = kChainCompute + 128 + 128;      // + the output warpgroup, 1 warp each to issue MMAs, load, relay and save
+constexpr int kBarA = 4, kBarB = 5;                          // the relay warp arrives, the compute warps wait
+
+// The chain of 64 d_v rows, two CTAs to a sequence.  What bounds a chunk is the sequence of hand-offs alone: 772 cycles of the two
+// products that depend on one another and twice the way from an accumulator to the next operand.  So that way is kept short:
+//  - 64-row products put 16 rows on each of a warpgroup's four warps, so all four schedulers of the SM share the epilogues (as the
+//    lower half of 128 rows they ran on two), and in fragment layout every thread has half as many elements; tiles are read and
+//    staged by ldmatrix / stmatrix instead of element by element;
+//  - the compute warps do not poll the products' barriers: a relay warp does, and raises a named barrier, at which they sleep;
+//  - what does not depend on h is fetched, and waited for, under the product before: Ut and the scales by the compute warps, tiles
+//    and the output accumulator by the MMA warp;
+//  - tiles are three deep (the first group two deep: 1.30 times the time of a prompt of 8 x 128 chunks, the second 1.12 times), which
+//    leaves room for one staged copy of what goes out.
+// Entry state and Delta^T go out by TMA: stored by the compute warps from their fragments in 64-byte pieces, or by others in whole
+// rows from the staged tiles, they delay every shared-memory access and wait of the SM (16 of 64: 104 us either way against 94).
+// The output, a quarter of that, goes in whole rows of 128 bytes: the TMA unit, 64 KB in and 24 KB out a chunk, is what bounds a
+// forward with saves, about 2100 cycles a chunk.
+// us, as 64 of k_tc_chain_fwd's 128 rows before and so, prompts and forwards with saves: 4 sequences of 16 chunks 27.3 / 24.5, 31.9 / 26.7;
+// 16 of 64 92.4 / 81.6, 113 / 94.3; 8 of 128 155 / 134, 198 / 156; 32 of 64 117 / 113, 133 / 124; 74 of 64 204 / 194, 243 / 228.
+template <bool SAVE>
+__global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid_constant__ CUtensorMap mapWt,
+                                                                    const __grid_constant__ CUtensorMap mapUt,
+                                                                    const __grid_constant__ CUtensorMap mapQg,
+                                                                    const __grid_constant__ CUtensorMap mapK,
+                                                                    const __grid_constant__ CUtensorMap mapP,
+                                                                    const __grid_constant__ CUtensorMap mapHs,
+                                                                    const __grid_constant__ CUtensorMap mapDt, ChainParams p) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    // bar_la, bar_lb: tiles loaded; bar_e: every product of a chunk has finished; bar_a, bar_b: products complete; bar_o, bar_of: an output
+    // accumulator is complete / has been read; bar_ht, bar_dt: entry state / Delta^T staged (one arrival per compute warp); bar_hf, bar_df: read
+    __shared__ uint64_t bar_la[kHalfDeep], bar_lb[kHalfDeep], bar_e[kHalfDeep], bar_a, bar_b, bar_o[2], bar_of[2], bar_ht, bar_dt, bar_hf, bar_df;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int s_abort;
+    __shared__ __align__(16) float sG[kHalfDeep][68];        // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C
+
+    const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, wq = warp & 3, lane = tid & 31;
+    constexpr int nb = kChainCompute + 32;                   // participants of a named barrier
+    const int bh = blockIdx.x >> 1, v0 = (blockIdx.x & 1) * 64, b = bh / p.H, hh = bh % p.H;
+
+    if (tid == 0) {
+        for (int i = 0; i < kHalfDeep; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_lb[i], 1); mbar_init(&bar_e[i], 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar_o[i], 1); mbar_init(&bar_of[i], 4); }
+        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1);
+        mbar_init(&bar_ht, 16); mbar_init(&bar_dt, 16); mbar_init(&bar_hf, 1); mbar_init(&bar_df, 1);
+        mbar_init_fence();
+        s_abort = 0;
+    }
+    if (tid < 32) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = uniform(tmem_slot);
+    // accumulators: Delta 64 columns, H 128, O 2 x 64; operands, two bf16 per column: h^T 64, Delta^T 32, scaled Delta^T 32
+    const uint32_t tD = tbase, tH = tbase + 64, tO0 = tbase + 192, aH = tbase + 320, aD = tbase + 384;
+    const uint32_t aDs = p.scaled ? tbase + 416 : aD;        // all factors 1: the scaled copy is Delta itself
+    const uint32_t lane_base = (uint32_t)wq * 32;
+
+    // bounded wait; once any wait has expired every later wait returns at once: every warp still comes to every barrier, the results
+    // are garbage, the status word says so
+    auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_try_wait(bar, parity) || wait_on(bar, parity, s_abort, p.status); };
+    const int tok0 = p.n0 * C;                               // first token; rows and tiles of the workspace start at
+    const size_t row0 = (size_t)bh * p.Tp + tok0, tile0 = (size_t)bh * p.Ns + p.n0;
+
+    if (warp < kOutWarp) {
+        // ---------------------------------- compute warps ----------------------------------
+        // fragments: rows r0, r0 + 8 of the CTA's 64; of every 8 columns two, ft and ft + 1
+        const int ft = 2 * (lane & 3), r0 = 16 * wq + (lane >> 2);
+        float h[16];          // h^T: [4 (8 d_k columns from 32 wg on)][2 (row)][2 (column)]
+        const size_t hat = (size_t)bh * D * D + (size_t)(32 * wg + ft) * D + v0 + r0;
+        auto at = [](int x) { return (size_t)(8 * (x >> 2) + (x & 1)) * D + 8 * ((x >> 1) & 1); };
+        if (p.h0_late) grid_dep_wait();
+#pragma unroll
+        for (int x = 0; x < 16; ++x) h[x] = p.h0 ? __ldcg(p.h0 + hat + at(x)) : 0.f;        // not from L1: it may be new
+        grid_dep_wait();                  // the loads of h0 (an input) are in flight; everything below depends on the prep kernel
+        grid_dep_launch();
+        const int rl = lane & 15, cl = lane >> 4;             // the row and the 16-byte chunk that this lane addresses for stsm4, ldsm4
+        unsigned char *sHs = smem + kHalfOffS + (wg >> 1) * 8192, *sDt = smem + kHalfOffS + 16384;
+        auto staged = [&](uint64_t* bar) { fence_proxy_async(); __syncwarp(); if (lane == 0) mbar_arrive(bar); };
+        // the state as operand, and staged as the entry state of chunk n
+        auto put_h = [&](int n) {
+            uint32_t r[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) r[i] = pack_bf16(h[2 * i], h[2 * i + 1]);
+            tmem_st_frag4(tmem_addr(aH, lane_base, wg * 16), r);
+            tmem_st_wait();
+            tc_fence_before();
+            nb_arrive(kBarH, nb);
+            if (SAVE && n < p.N) {
+                if (n > 0) wait(&bar_hf, (n - 1) & 1);
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 2; ++i) stsm4<false>(sHs + sw128_chunk(16 * wq + rl, (wg & 1) * 4 + 2 * i + cl), r + 4 * i);
+                staged(&bar_ht);
+            }
+        };
+        put_h(0);
+        int s = 0;
+        uint32_t sp = 0;
+        uint32_t u[4];                    // Ut of the chunk, [2 (8 tokens)][2 (row)], and its scales
+        float2 f0, f1;
+        float gamN;
+        auto fetch = [&]() {
+            wait(&bar_la[s], sp);
+            __syncwarp();
+            ldsm4<false>(smem + s * kHalfStageA + 16384 + sw128_chunk(16 * wq + rl, 2 * wg + cl), u);
+            f0 = *reinterpret_cast<const float2*>(&sG[s][16 * wg + ft]);
+            f1 = *reinterpret_cast<const float2*>(&sG[s][16 * wg + 8 + ft]);
+            gamN = sG[s][64];
+            if (++s == kHalfDeep) { s = 0; sp ^= 1; }
+        };
+        fetch();
+        for (int n = 0; n < p.N; ++n) {
+            const float gamC = gamN;
+            nb_sync(kBarA, nb);
+            tc_fence_after();
+            // Delta^T = Ut - acc, my 16 tokens, as operands: plain, and scaled by gamma_C/gamma_r
+            {
+                float v[8];
+                tmem_ld_frag2(tmem_addr(tD, lane_base, wg * 16), v);
+                tmem_ld_wait();
+                uint32_t r[4], rs[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float2 f = m < 2 ? f0 : f1;
+                    const float x = __uint_as_float(u[m] << 16) - v[2 * m], y = __uint_as_float(u[m] & 0xffff0000u) - v[2 * m + 1];
+                    r[m] = pack_bf16(x, y);
+                    rs[m] = pack_bf16(x * f.x, y * f.y);
+                }
+                if (p.scaled) tmem_st_frag2(tmem_addr(aDs, lane_base, wg * 8), rs);
+                tmem_st_frag2(tmem_addr(aD, lane_base, wg * 8), r);
+                tmem_st_wait();
+                tc_fence_before();
+                nb_arrive(kBarD, nb);
+                if (SAVE) {
+                    if (n > 0) wait(&bar_df, (n - 1) & 1);
+                    __syncwarp();
+                    stsm4<false>(sDt + sw128_chunk(16 * wq + rl, 2 * wg + cl), r);
+                    staged(&bar_dt);
+                }
+            }
+            if (n + 1 < p.N) fetch();     // under the product
+            // h^T <- gamma_C h^T + acc (my 32 d_k columns), refresh the operand
+            nb_sync(kBarB, nb);
+            tc_fence_after();
+            {
+                float v[16];
+                tmem_ld_frag4(tmem_addr(tH, lane_base, wg * 32), v);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 16; ++i) h[i] = fmaf(gamC, h[i], v[i]);
+            }
+            put_h(n + 1);
+        }
+        if (p.hT && !s_abort) {
+#pragma unroll
+            for (int x = 0; x < 16; ++x) p.hT[hat + at(x)] = h[x];
+        }
+    } else if (warp < kMmaWarp) {
+        // ---------------------------------- output warps ----------------------------------
+        // O^T of a chunk, 16 rows to a warp -> token-major tile -> 16 tokens to a warp
+        unsigned char* sO = smem + kHalfOffO;
+        const size_t pitch = (size_t)p.H * D;
+        bf16* o = p.o + (size_t)b * p.T * pitch + (size_t)hh * D + v0 + 8 * (lane & 7);
+        grid_dep_wait();                  // the chain before may take longer than a wait has (tc_fwd_parts)
+        for (int n = 0; n < p.N; ++n) {
+            const int ob = n & 1;
+            wait(&bar_o[ob], (n >> 1) & 1);
+            __syncwarp();
+            tc_fence_after();
+            float v[2][16];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) tmem_ld_frag4(tmem_addr(tO0 + 64 * ob, lane_base, 32 * i), v[i]);
+            tmem_ld_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_of[ob]);          // the accumulator may be written again
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint32_t r[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) r[m] = pack_bf16(v[i >> 1][8 * (i & 1) + 2 * m], v[i >> 1][8 * (i & 1) + 2 * m + 1]);
+                stsm4<true>(sO + sw128_chunk(16 * i + 8 * (lane >> 4) + (lane & 7), 2 * wq + ((lane >> 3) & 1)), r);
+            }
+            nb_sync(kBarOut, 128);
+            uint4 x[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const uint4*>(sO + sw128_chunk(16 * wq + 4 * i + (lane >> 3), lane & 7));
+            nb_sync(kBarOut, 128);                            // the tile may be written again
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int t = tok0 + n * C + 16 * wq + 4 * i + (lane >> 3);
+                if (t < p.T) *reinterpret_cast<uint4*>(o + t * pitch) = x[i];      // rows past the end of the sequence are skipped
+            }
+        }
+    } else if (warp == kMmaWarp) {
+        // ---------------------------------- MMA-issue warp, converged ----------------------------------
+        const uint32_t issue = elect_lane();
+        grid_dep_wait();
+        grid_dep_launch();
+        int s = 0;
+        uint32_t sp = 0;
+        wait(&bar_la[0], 0);
+        for (int n = 0; n < p.N; ++n) {
+            const int ob = n & 1, st = s;
+            const uint32_t stA = smem_u32(smem) + s * kHalfStageA, stB = smem_u32(smem) + kHalfOffB + s * kHalfStageB;
+            const uint32_t tO = tO0 + 64 * ob;
+            nb_sync(kBarH, nb);                               // h^T operand of chunk n is in place
+            tc_fence_after();
+            // Delta-accumulator = h^T Wt (B: MN-major, lines = d_k)
+            umma_product_ts_w<true, 64>(tD, aH, stA, 8192, C, D, false, issue);
+            umma_commit_w(&bar_a, issue);
+            // O-accumulator = h^T Qg^T (B: K-major); it reads the operand that the h update rewrites, so the commit
+            // behind the H product below (which releases that update) must cover it
+            wait(&bar_lb[s], sp);
+            umma_product_ts_w<false, 64>(tO, aH, stB, 8192, C, D, false, issue);
+            if (++s == kHalfDeep) { s = 0; sp ^= 1; }
+            if (n + 1 < p.N) {                                // what the next chunk needs besides h^T, while there is time
+                wait(&bar_la[s], sp);
+                if (n > 0) wait(&bar_of[ob ^ 1], ((n - 1) >> 1) & 1);
+            }
+            nb_sync(kBarD, nb);                               // Delta^T operands of chunk n are in place
+            tc_fence_after();
+            // H-accumulator = scaled Delta^T K (B: MN-major, lines = tokens)
+            umma_product_ts_w<true, 64>(tH, aDs, stB + 16384, 8192, D, C, false, issue);
+            umma_commit_w(&bar_b, issue);
+            // O-accumulator += Delta^T P^T (B: K-major [r][s])
+            umma_product_ts_w<false, 64>(tO, aD, stB + 32768, 8192, C, C, true, issue);
+            umma_commit_w(&bar_o[ob], issue);
+            umma_commit_w(&bar_e[st], issue);
+        }
+        nb_sync(kBarH, nb);                                   // final arrival of the compute warps
+    } else if (warp == kMmaWarp + 1) {
+        // ---------------------------------- TMA load warp ----------------------------------
+        const bool lead = lane == 0;
+        grid_dep_wait();                  // the tiles and the log-decays read below are written by the prep kernel
+        grid_dep_launch();
+        const float *gseq = p.g + row0, *rkseq = p.rk ? p.rk + row0 : nullptr;
+        // log-decays (and 1/|k|) of the next chunk to be loaded, fetched ahead
+        float g0, g1, gc, k0 = 1.f, k1 = 1.f;
+        auto fetch_g = [&](int n) {
+            const float* gn = gseq + (size_t)n * C;
+            g0 = gn[lane]; g1 = gn[32 + lane]; gc = gn[C - 1];
+            if (rkseq) { k0 = rkseq[(size_t)n * C + lane]; k1 = rkseq[(size_t)n * C + 32 + lane]; }
+        };
+        auto load = [&](int n, int s) {                       // by the whole warp
+            sG[s][lane] = __expf(gc - g0) * k0;
+            sG[s][32 + lane] = __expf(gc - g1) * k1;
+            if (lane == 0) sG[s][64] = __expf(gc);
+            __syncwarp();
+            if (lead) {
+                const int yc = (int)((tile0 + n) * D), yt = (int)(row0 + (size_t)n * C);
+                unsigned char *sa = smem + s * kHalfStageA, *sb = smem + kHalfOffB + s * kHalfStageB;
+                mbar_expect_tx(&bar_la[s], kHalfStageA);
+                tma_load_2d(sa, &mapWt, 0, yc, &bar_la[s]);
+                tma_load_2d(sa + 16384, &mapUt, 0, yc + v0, &bar_la[s]);
+                mbar_expect_tx(&bar_lb[s], kHalfStageB);
+                tma_load_2d(sb, &mapQg, 0, yt, &bar_lb[s]);
+                tma_load_2d(sb + 8192, &mapQg, 64, yt, &bar_lb[s]);
+                tma_load_3d(sb + 16384, &mapK, hh * D, tok0 + n * C, b, &bar_lb[s]);
+                tma_load_3d(sb + 16384 + 8192, &mapK, hh * D + 64, tok0 + n * C, b, &bar_lb[s]);
+                tma_load_2d(sb + 32768, &mapP, 0, yt, &bar_lb[s]);
+            }
+            if (n + 1 < p.N) fetch_g(n + 1);
+        };
+        fetch_g(0);
+        for (int n = 0; n < kHalfDeep && n < p.N; ++n) load(n, n);
+        int s = 0;
+        uint32_t sp = 0;
+        for (int n = 0; n + kHalfDeep < p.N; ++n) {
+            wait(&bar_e[s], sp);                              // every product of chunk n has finished: refill its buffers
+            if (!__all_sync(0xffffffffu, !s_abort)) break;    // one answer for the warp
+            load(n + kHalfDeep, s);
+            if (++s == kHalfDeep) { s = 0; sp ^= 1; }
+        }
+        if (lead && s_abort)              // one more bounded chance for copies in flight
+            for (int i = 0; i < kHalfDeep; ++i) { mbar_wait(&bar_la[i], 0); mbar_wait(&bar_lb[i], 0); }
+    } else if (warp == kMmaWarp + 2) {
+        // ---------------------------------- relay warp ----------------------------------
+        auto relay = [&](uint64_t* bar, uint32_t parity, int id) {
+            wait(bar, parity);
+            tc_fence_after();
+            tc_fence_before();
+            __syncwarp();
+            nb_arrive(id, nb);
+        };
+        grid_dep_wait();
+        for (int n = 0; n < p.N; ++n) {
+            relay(&bar_a, n & 1, kBarA);
+            relay(&bar_b, n & 1, kBarB);
+        }
+    } else {
+        // ---------------------------------- saving warp ----------------------------------
+        if (lane == 0 && SAVE) {
+            unsigned char *sHs = smem + kHalfOffS, *sDt = sHs + 16384;
+            grid_dep_wait();
+            for (int n = 0; n < p.N; ++n) {
+                const int y = (int)((tile0 + n) * D) + v0;
+                wait(&bar_ht, n & 1);                         // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
+                tma_store_2d(&mapHs, sHs, 0, y);
+                tma_store_2d(&mapHs, sHs + 8192, 64, y);
+                tma_store_commit();
+                if (n > 0) {                                  // Delta^T of chunk n - 1 has been read
+                    tma_store_wait_read_n<1>();
+                    mbar_arrive(&bar_df);
+                }
+                wait(&bar_dt, n & 1);                         // Delta^T of chunk n is staged
+                tma_store_2d(&mapDt, sDt, 0, y);
+                tma_store_commit();
+                tma_store_wait_read_n<1>();                   // the entry state has been read
+                mbar_arrive(&bar_hf);
+            }
+            tma_store_wait_all();
         }
     }
     tc_fence_before();
@@ -869,6 +1187,7 @@ bool setup(const ChunkArgs& a, ChainCall& c) {
     p.Tp = Tp; p.H = s.H; p.N = (int)N; p.Ns = (int)Ns;
     p.g = (const float*)(a.ws + a.TL.g);
     p.h0 = a.h0; p.hT = a.hT;
+    p.T = s.T; p.o = (bf16*)a.o;
     p.scaled = (a.alpha || a.norm) ? 1 : 0;
     p.rk = a.norm ? (const float*)(a.ws + a.TL.rqk) + BH * Tp : nullptr;
     p.status = (unsigned*)(a.ws + a.TL.status);
@@ -877,11 +1196,17 @@ bool setup(const ChunkArgs& a, ChainCall& c) {
 cudaError_t launch(const ChunkArgs& a, const ChainCall& c) {
     const uint64_t BH = (uint64_t)a.s.B * a.s.H;
     const int rows = chain_rows(BH);
-    const auto kern = rows == D ? (a.save ? k_tc_chain_fwd<D, true> : k_tc_chain_fwd<D, false>)
-                                : (a.save ? k_tc_chain_fwd<D / 2, true> : k_tc_chain_fwd<D / 2, false>);
+    if (rows != D) {
+        const auto half = a.save ? k_tc_chain_fwd_half<true> : k_tc_chain_fwd_half<false>;
+        cudaError_t e = set_smem(half, kHalfSmem);
+        if (e != cudaSuccess) return e;
+        return launch_overlapped(half, dim3((unsigned)(2 * BH)), dim3(kHalfThreads), kHalfSmem, a.stream, c.mWt, c.mUt, c.mQg, c.mK, c.mP,
+                                 c.mHs, c.mDt, c.p);
+    }
+    const auto kern = a.save ? k_tc_chain_fwd<true> : k_tc_chain_fwd<false>;
     cudaError_t e = set_smem(kern, kChainSmem);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(kern, dim3((unsigned)(BH * (D / rows))), dim3(kChainThreads), kChainSmem, a.stream, c.mWt, c.mUt, c.mQg,
+    return launch_overlapped(kern, dim3((unsigned)BH), dim3(kChainThreads), kChainSmem, a.stream, c.mWt, c.mUt, c.mQg,
                              c.mK, c.mP, c.mHs, c.mDt, c.mO, c.p);
 }
 

@@ -48,6 +48,29 @@ def test_preparation_edges(T):
     _bwd_check(cfg, d, reuse=True)
 
 
+@pytest.mark.parametrize("T", [64 * 2, 64 * 3, 64 * 3 + 1, 64 * 4 - 1, 64 * 6 + 17])
+@pytest.mark.parametrize("without", ["", "alpha lam", "h0"])
+def test_half_chain_edges(T, without):
+    """Two CTAs to a sequence, their tiles three deep: as many chunks as that, one fewer, one more, twice around; without a forget gate (one
+    copy of Delta^T instead of two); and a prompt has the bits of a forward with saves."""
+    import torch
+
+    from gpu_util import dev_inputs
+    from paper_2606_08804_b200 import binding as qd
+
+    cfg = replace(gen.CONFIGS["cfg2"], B=2, H=3, T=T, regime="trained_like", seed=419 + T)
+    d = gen.make_chunk_inputs(cfg)
+    for n in without.split():
+        d[n] = None
+    _fwd_check(cfg, d, save=True)
+    _bwd_check(cfg, d, reuse=True)
+    t = dev_inputs(d, cfg.dtype)
+    a = [t[n] for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")]
+    for norm in (False, True):
+        (o, hT, _), (p, hP, _) = (qd.chunk_fwd(*a, save_for_bwd=s, norm_qk=norm) for s in (True, False))
+        assert torch.equal(o, p) and torch.equal(hT, hP)
+
+
 @pytest.mark.parametrize("B,H,T,parts", [(1, 16, 64 * 64, (2, 2)), (2, 20, 64 * 64 + 1, (2, 1)), (1, 4, 64 * 256, (3, 2)),
                                          (1, 1, 64 * 1024 - 63, (3, 2)), (1, 40, 64 * 120 - 1, (2, 2)), (2, 2, 64 * 64, (1, 2)),
                                          (2, 8, 64 * 128 - 5, (2, 3)), (1, 36, 64 * 128, (2, 3)), (1, 32, 64 * 256 + 1, (3, 3))])

@@ -20,7 +20,7 @@ def test_dynamic_shared_memory_is_aligned(name):
             assert re.search(r"\(uintptr_t\)%s \+ 1023\) & ~\(uintptr_t\)1023" % m.group(2), lines[i + 1]), (name, i + 1, line)
 
 
-@pytest.mark.parametrize("name,kernel", [("tc_fwd.cu", "k_tc_chain_fwd"), ("tc_bwd.cu", "k_tc_chain_bwd"), ("tc_bwd.cu", "k_tc_chunk_bwd")])
+@pytest.mark.parametrize("name,kernel", [("tc_fwd.cu", "k_tc_chain_fwd"), ("tc_fwd.cu", "k_tc_chain_fwd_half"), ("tc_bwd.cu", "k_tc_chain_bwd"), ("tc_bwd.cu", "k_tc_chunk_bwd")])
 def test_bounded_waits_begin_after_the_kernel_before(name, kernel):
     """A CTA may start while the kernel before it runs, for as long as that takes; the time limit of a wait inside the CTA is meant for the
     CTA's own work, so every role of its warps waits for that kernel before its first bounded wait."""
