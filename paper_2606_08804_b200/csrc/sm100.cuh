@@ -60,6 +60,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
     }
 }
 
+// For what has been issued and completes by itself (copies, products), whatever else has expired.
+__device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity) { return mbar_wait(bar, parity); }
+
 // What follows an unsuccessful first poll: mbar_wait, given up as soon as another wait of the CTA has expired (every later wait
 // then returns at once: the kernel drains).
 __device__ __forceinline__ bool wait_on(uint64_t* bar, uint32_t parity, volatile int& s_abort, unsigned* status) {

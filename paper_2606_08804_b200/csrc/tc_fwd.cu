@@ -833,7 +833,16 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
     const uint32_t lane_base = (uint32_t)wq * 32;
 
     // bounded wait; once any wait has expired every later wait returns at once: every warp still comes to every barrier, the results
-    // are garbage, the status word says so
+    // are garbage, the status word says so.
+    // The named barriers come in the order H, A, D, B, H, ...  Whoever arrives without waiting (bar.arrive) must not come to the same
+    // barrier again before its phase is over: the second arrival would stand for that of a warp still to come, and that warp would
+    // then wait for good.  It cannot, because the relay warp raises A of a chunk only when the MMA warp has passed H, and B when it has passed D:
+    //  - a compute warp comes to D again behind the next A, so after the MMA warp has passed the next H and with it this D; to H
+    //    again behind A and B of the chunk, so after the MMA warp has passed this H;
+    //  - the relay warp comes to A (B) again after the MMA warp has passed the next H (D), to which every compute warp
+    //    came from behind this A (B).
+    // That a product is complete says that the MMA warp has passed the barrier before it, so the relay warp waits for the products of a
+    // chunk whether a wait has expired or not: the MMA warp, which waits for nothing else by then, issues them all the same.
     auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_try_wait(bar, parity) || wait_on(bar, parity, s_abort, p.status); };
     const int tok0 = p.n0 * C;                               // first token; rows and tiles of the workspace start at
     const size_t row0 = (size_t)bh * p.Tp + tok0, tile0 = (size_t)bh * p.Ns + p.n0;
@@ -1054,7 +1063,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
     } else if (warp == kMmaWarp + 2) {
         // ---------------------------------- relay warp ----------------------------------
         auto relay = [&](uint64_t* bar, uint32_t parity, int id) {
-            wait(bar, parity);
+            if (!wait(bar, parity)) mbar_drain(bar, parity);
             tc_fence_after();
             tc_fence_before();
             __syncwarp();
