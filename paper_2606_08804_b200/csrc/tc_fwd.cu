@@ -1012,7 +1012,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
             // O-accumulator += Delta^T P^T (B: K-major [r][s])
             umma_product_ts_w<false, 64>(tO, aD, stB + 32768, 8192, C, C, true, issue);
             umma_commit_w(&bar_o[ob], issue);
-            umma_commit_w(&bar_e[st], issue);
+            if (n + kHalfDeep < p.N) umma_commit_w(&bar_e[st], issue);      // the load warp waits for these: nothing arrives in a CTA that has left
         }
         nb_sync(kBarH, nb);                                   // final arrival of the compute warps
     } else if (warp == kMmaWarp + 1) {

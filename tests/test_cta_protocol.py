@@ -112,12 +112,25 @@ def programs(tmp_path_factory):
     return get
 
 
-# what is looked at (emu::kinds)
-KERNELS = [("tc_fwd.cu", "full", "b"), ("tc_fwd.cu", "half", "b"), ("tc_bwd.cu", "chain", "b")]
+ALL = [("tc_fwd.cu", "prep"), ("tc_fwd.cu", "full"), ("tc_fwd.cu", "half"), ("tc_bwd.cu", "chain"), ("tc_bwd.cu", "chunk")]
 
 
-@pytest.mark.parametrize("name,kernel,kinds", KERNELS)
-@pytest.mark.parametrize("expire,lose", [(0, 0), (0.0005, 0), (0.05, 0), (0.005, 0.02)], ids=["sound", "rare", "early", "lost load"])
-def test_any_order_of_warps(programs, name, kernel, kinds, expire, lose):
-    r = subprocess.run([programs(name), kernel, "200" if expire else "100", str(expire), str(lose), kinds], capture_output=True, text=True, timeout=600)
+def _run(exe, kernel, runs, expire, lose, kinds):
+    r = subprocess.run([exe, kernel, str(runs), str(expire), str(lose), kinds], capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("name,kernel", ALL)
+def test_any_order_of_warps(programs, name, kernel):
+    """No wait expires, and the CTA leaves with everything done."""
+    _run(programs(name), kernel, 100, 0, 0, "bct")
+
+
+# what is looked at (emu::kinds)
+EXPIRED = [("tc_fwd.cu", "full", "b"), ("tc_fwd.cu", "half", "b"), ("tc_bwd.cu", "chain", "b")]
+
+
+@pytest.mark.parametrize("name,kernel,kinds", EXPIRED)
+@pytest.mark.parametrize("expire,lose", [(0.0005, 0), (0.05, 0), (0.005, 0.02)], ids=["rare", "early", "lost load"])
+def test_expired_waits(programs, name, kernel, kinds, expire, lose):
+    _run(programs(name), kernel, 200, expire, lose, kinds)
