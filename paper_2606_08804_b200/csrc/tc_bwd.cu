@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ChunkBars bar;
     __shared__ uint32_t tmem_slot;
-    __shared__ volatile int s_abort, s_latch;
+    __shared__ volatile int s_abort, s_latch[2];                  // s_latch[it % 2]: a wait had expired before iteration it
     ChunkShared& sh = *reinterpret_cast<ChunkShared*>(sm + kTileBytes);
     auto &sbeta_ = sh.sbeta_, &sg_ = sh.sg_, &slam_ = sh.slam_, &sgam_ = sh.sgam_;
     auto& scf_ = sh.scf_;
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         for (int i = 0; i < (int)(sizeof(ChunkBars) / 8); ++i) mbar_init(all + i, 1);
         mbar_init_fence();
         s_abort = 0;
-        s_latch = 0;
+        s_latch[0] = s_latch[1] = 0;
     }
     if (tid < 32) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
         __syncthreads();                                                 // the first chunk's coefficients have been published
         for (int it = 0; (int)uniform((uint32_t)slot(it).n) >= 0; ++it) {
             const uint32_t ph = it & 1;
-            if (__any_sync(0xffffffffu, s_latch)) break;
+            if (__any_sync(0xffffffffu, s_latch[ph])) break;
             wait(&bar.d, ph);
             wait(&bar.h, ph);
             __syncwarp();
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             const int n = cur.n, b = cur.bh / p.H, hh = cur.bh % p.H;
             const bool more = next.n >= 0;
             const uint32_t ph = it & 1;
-            if (__any_sync(0xffffffffu, s_latch)) break;
+            if (__any_sync(0xffffffffu, s_latch[ph])) break;
             if (lead) {
                 if (more) prefetch_late(next);
                 put(it + 2, more ? claim() : next);
@@ -638,9 +638,10 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
                 if (more && !s_abort) { issue_dd(next); issue_early(next); }
             }
             nb_sync(kNbOut, kBwdNb);                                     // the dk and dq staging tiles are complete
-            // s_latch is read by everyone right after the barrier and not written again before the next one;
-            // an expiry that this read misses is seen one chunk later (waits return at once meanwhile)
-            if (lead) s_latch = s_abort;
+            // Everybody has to leave in the same iteration.  This one's latch may not have been read by every warp yet: once a wait has
+            // expired the epilogue comes here without the others.  The next one's was read before the End barrier that the epilogue has passed
+            // since.  An expiry that this misses is seen one chunk later (waits return at once meanwhile).
+            if (lead) s_latch[ph ^ 1] = s_abort;
             __syncwarp();
             nb_arrive(kNbEnd, kBwdThreads);                              // nobody waits for the copies to be issued
             if (lead) {
@@ -733,7 +734,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             const Item cur = slot(it), next = slot(it + 1);
             const int n = cur.n, bh = cur.bh;
             const uint32_t ph = it & 1;
-            if (__any_sync(0xffffffffu, s_latch)) { prev.n = -1; break; }
+            if (__any_sync(0xffffffffu, s_latch[ph])) { prev.n = -1; break; }
             if (prev.n >= 0) finish(prev, ph ^ 1);
             const float gm = sgam_[ph][C - 1];
             be0 = be; lm0 = lm; al0 = al; gmC = gm;
@@ -778,7 +779,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
 
     for (int it = 0; slot(it).n >= 0; ++it) {
     const uint32_t ph = it & 1;
-    if (s_latch) break;
+    if (s_latch[ph]) break;
     const float *sbeta = sbeta_[ph], *slam = slam_[ph], *sg = sg_[ph], *sgam = sgam_[ph];
     const float4* scf = scf_[ph];
     const float2* srn = srn_[ph];
