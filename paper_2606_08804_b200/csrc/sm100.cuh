@@ -62,6 +62,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
 
 // For what has been issued and completes by itself (copies, products), whatever else has expired.
 __device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity) { return mbar_wait(bar, parity); }
+// The last loads of a ring: load i went to barrier i mod depth, `loads` have been issued.
+__device__ __forceinline__ void mbar_drain_ring(uint64_t* bars, int depth, int loads) {
+    for (int i = 0; i < depth && i < loads; ++i) mbar_drain(&bars[i], (uint32_t)((loads - 1 - i) / depth) & 1);
+}
 
 // What follows an unsuccessful first poll: mbar_wait, given up as soon as another wait of the CTA has expired (every later wait
 // then returns at once: the kernel drains).

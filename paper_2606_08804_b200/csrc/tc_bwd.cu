@@ -63,8 +63,9 @@ constexpr int kMmaWarp = kChainCompute / 32;
 constexpr int kBarH = 1, kBarD = 2;
 
 // A barrier per buffer where one side may run ahead.  k, q, w: tiles loaded; fk, fq, fw: read by their last product; ht, dt:
-// staged (one arrival per compute warp); hf, df: read by their store (two deep: hf alone, for both); a, b: products complete.
-struct ChainBars { uint64_t k[kDeepK], fk[kDeepK], q[2], fq[2], w[2], fw[2], hf[2], df, a, b, ht[2], dt[2]; };
+// staged (one arrival per compute warp); hf, df: read by their store (two deep: hf alone, for both); a, b: products complete;
+// end: all of them, after a wait has expired.
+struct ChainBars { uint64_t k[kDeepK], fk[kDeepK], q[2], fq[2], w[2], fw[2], hf[2], df, a, b, end, ht[2], dt[2]; };
 
 // Reverse state chain.  Per chunk the dependency is
 //   dh ready -> A2 = dh^T K^T -> dDelta^T -> H-accumulator -= dDelta^T W<- -> dh update;
@@ -95,6 +96,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
     __shared__ ChainBars bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
+    __shared__ int s_loads[3];                         // issued in all: K and P; Qg and dO; Wt
     // gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the load warp before it arrives on bar.k.  One deeper than
     // K and P: those are dead when A2 is complete, but the epilogue reads these after that
     float (*sG)[68] = reinterpret_cast<float (*)[68]>(smem + kOffG);
@@ -332,29 +334,32 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
         }
         int s = 0;                                        // stage of chunk it's K and P, and the parity of its present round
         uint32_t sp = 0;
+        int nk = min(kDeepK, p.N), nq = min(2, p.N), nw = nq;
         for (int it = 0; it < p.N; ++it) {
             bool more = it + kDeepK < p.N;
             if (lead) {
                 wait(&bar.fq[it & 1], (it >> 1) & 1);
-                if (it + 2 < p.N && !s_abort) load_q(it + 2);
+                if (it + 2 < p.N && !s_abort) { load_q(it + 2); nq = it + 3; }
                 wait(&bar.fk[s], sp);
             }
             more = __shfl_sync(0xffffffffu, more && !s_abort, 0);     // one answer for the warp
-            if (more) load_k(it + kDeepK, s);
+            if (more) { load_k(it + kDeepK, s); nk = it + kDeepK + 1; }
             if (lead) {
                 wait(&bar.fw[it & 1], (it >> 1) & 1);
-                if (it + 2 < p.N && !s_abort) load_w(it + 2);
+                if (it + 2 < p.N && !s_abort) { load_w(it + 2); nw = it + 3; }
             }
             __syncwarp();
             if (++s == kDeepK) { s = 0; sp ^= 1; }
         }
-        if (lead && s_abort) {            // one more bounded chance for copies in flight
-            for (int i = 0; i < kDeepK; ++i) mbar_wait(&bar.k[i], 0);
-            for (int i = 0; i < 2; ++i) { mbar_wait(&bar.q[i], 0); mbar_wait(&bar.w[i], 0); }
-        }
+        if (lead) { s_loads[0] = nk; s_loads[1] = nq; s_loads[2] = nw; }
     }
     tc_fence_before();
     __syncthreads();
+    if (s_abort) {                        // a wait has expired, so what is in flight has not been waited for
+        if ((tid >> 5) == kMmaWarp) { umma_commit_w(&bar.end, elect_lane()); mbar_drain(&bar.end, 0); }
+        if (tid == (kMmaWarp + 2) * 32) { mbar_drain_ring(bar.k, kDeepK, s_loads[0]); mbar_drain_ring(bar.q, 2, s_loads[1]); mbar_drain_ring(bar.w, 2, s_loads[2]); }
+        __syncthreads();
+    }
     if (tid < 32) tmem_dealloc(tbase, 512);
 }
 
@@ -396,7 +401,7 @@ constexpr int kBwdNb = kBwdCompute + 32;                 // participants of a na
 constexpr int kNbC = 1, kNbX = 2, kNbDW = 3, kNbDTb = 4, kNbN = 5, kNbDXK = 6, kNbOut = 7, kNbDV = 8, kNbDVt = 10, kNbSum = 11, kNbTok = 12, kNbEnd = 13;
 constexpr int kNbSumN = kBwdCompute + C;
 
-struct ChunkBars { uint64_t load, d, h, qk, st, a, b, c, m2, m3, m4, m5; };
+struct ChunkBars { uint64_t load, d, h, qk, st, a, b, c, m2, m3, m4, m5, end; };
 // What the warps tell each other; `_` arrays by parity of the chunk, so that the token threads can publish a chunk
 // ahead and take their sums a chunk late.
 struct ChunkShared {
@@ -436,6 +441,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     __shared__ ChunkBars bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort, s_latch[2];                  // s_latch[it % 2]: a wait had expired before iteration it
+    __shared__ int s_loads[3];                                    // issued in all: bar.load and bar.d, bar.h, bar.qk
     ChunkShared& sh = *reinterpret_cast<ChunkShared*>(sm + kTileBytes);
     auto &sbeta_ = sh.sbeta_, &sg_ = sh.sg_, &slam_ = sh.slam_, &sgam_ = sh.sgam_;
     auto& scf_ = sh.scf_;
@@ -615,6 +621,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             mbar_arrive(&bar.st);                                        // nothing is staged yet
         }
         __syncthreads();                                                 // the first chunk's coefficients have been published
+        int ne = 1, nh = 1, nqk = 1;
         for (int it = 0; slot(it).n >= 0; ++it) {
             const Item cur = slot(it), next = slot(it + 1);
             const int n = cur.n, b = cur.bh / p.H, hh = cur.bh % p.H;
@@ -625,7 +632,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
                 if (more) prefetch_late(next);
                 put(it + 2, more ? claim() : next);
                 wait(&bar.m3, ph);                                       // from here on nobody reads h or dh
-                if (more && !s_abort) { issue_h(next); issue_dh(next); }
+                if (more && !s_abort) { issue_h(next); issue_dh(next); ++nh; }
             }
             nb_sync(kNbDVt, kBwdNb);                                     // the dv staging tile is complete
             if (lead) {
@@ -635,7 +642,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
                 tma_store_wait_read();
                 wait(&bar.m5, ph);                                         // from here on nobody reads anything but Q, K
                 fence_proxy_async();
-                if (more && !s_abort) { issue_dd(next); issue_early(next); }
+                if (more && !s_abort) { issue_dd(next); issue_early(next); ++ne; }
             }
             nb_sync(kNbOut, kBwdNb);                                     // the dk and dq staging tiles are complete
             // Everybody has to leave in the same iteration.  This one's latch may not have been read by every warp yet: once a wait has
@@ -651,7 +658,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
                 tma_store_3d(&m.dQ, sm + oStDq + 8192, hh * D + 64, n * C, b);
                 tma_store_commit();
                 fence_proxy_async();                                     // the epilogue's reads of Q precede the copy into its region
-                if (more && !s_abort) issue_qk(next);
+                if (more && !s_abort) { issue_qk(next); ++nqk; }
             }
             if (lead) {
                 tma_store_wait_read();                                   // the staging tiles have been read by the stores
@@ -659,7 +666,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             }
             __syncwarp();
         }
-        if (lead) tma_store_wait_all();
+        if (lead) { s_loads[0] = ne; s_loads[1] = nh; s_loads[2] = nqk; tma_store_wait_all(); }
     } else if (tid >= kBwdTail) {
         // =============================== token threads ===============================
         // thread r owns token r of the chunk
@@ -1115,8 +1122,13 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     }  // epilogue threads
     tc_fence_before();
     __syncthreads();
-    if (tid == kBwdCompute && s_abort) {                         // one more bounded chance for copies in flight
-        mbar_wait(&bar.load, 0); mbar_wait(&bar.d, 0); mbar_wait(&bar.h, 0); mbar_wait(&bar.qk, 0);
+    if (s_abort) {                        // a wait has expired, so what is in flight has not been waited for
+        if ((tid >> 5) == kBwdCompute / 32) { umma_commit_w(&bar.end, elect_lane()); mbar_drain(&bar.end, 0); }
+        if (tid == kBwdNb) {
+            mbar_drain_ring(&bar.load, 1, s_loads[0]); mbar_drain_ring(&bar.d, 1, s_loads[0]);
+            mbar_drain_ring(&bar.h, 1, s_loads[1]); mbar_drain_ring(&bar.qk, 1, s_loads[2]);
+        }
+        __syncthreads();
     }
     if (tid < 32) tmem_dealloc(tb, 512);
     if (tid == 0 && blockIdx.x == 0) grid_dep_wait();            // when this kernel has completed, so has the one before it

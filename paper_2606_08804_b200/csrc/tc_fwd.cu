@@ -11,8 +11,8 @@
 //                     Delta^T = Ut - h^T Wt            O^T = h^T Qg^T + Delta^T P^T
 //                     h^T <- gamma_C h^T + (Delta diag(gamma_C/gamma))^T K
 // With few long sequences the two run beside each other, part by part (tc_fwd_parts).
-// All waits are bounded; on expiry the CTA records QD_ERR_TIMEOUT in the workspace status word,
-// releases its tensor memory and returns.
+// All waits are bounded; on expiry the CTA records QD_ERR_TIMEOUT in the workspace status word, lets what it has in flight
+// come to an end (mbar_drain), releases its tensor memory and returns.
 #include "internal.h"
 #include "sm100.cuh"
 #include "tf32.cuh"
@@ -476,9 +476,10 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     // waited for it.  bar_e: every product of a chunk has finished; bar_dt, bar_ht: Delta^T / exit state staged for their stores
     // (one arrival per compute warp); bar_df, bar_hf: they have been read; bar_o, bar_of: an output accumulator is complete /
     // has been read.
-    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_df[kDeepA], bar_ht, bar_hf, bar_a, bar_b, bar_o[2], bar_of[2];
+    __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_df[kDeepA], bar_ht, bar_hf, bar_a, bar_b, bar_o[2], bar_of[2], bar_end;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
+    __shared__ int s_loads[2];                      // issued in all: Wt and Ut; Qg, K and P
     // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the TMA warp before it arrives on the
     // stage's load barrier, so no epilogue thread waits for a global load
     __shared__ __align__(16) float sG[kDeepA][68];
@@ -490,7 +491,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     if (tid == 0) {
         for (int i = 0; i < kDeepA; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_dt[i], 16); mbar_init(&bar_df[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&bar_lb[i], 1); mbar_init(&bar_e[i], 1); mbar_init(&bar_o[i], 1); mbar_init(&bar_of[i], 4); }
-        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1);
+        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1); mbar_init(&bar_end, 1);
         mbar_init(&bar_ht, 16); mbar_init(&bar_hf, 1);
         mbar_init_fence();
         s_abort = 0;
@@ -747,25 +748,27 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             load_a(n, n);
             if (lead && n < 2) load_b(n);
         }
-        int s = 0;
+        int s = 0, na = min(kDeepA, p.N), nb = min(2, p.N);
         for (int n = 0; n < p.N; ++n) {
             bool more = n + kDeepA < p.N;
             if (lead) {
                 wait(&bar_e[n & 1], (n >> 1) & 1);        // every product of chunk n has finished: refill its buffers
-                if (n + 2 < p.N && !s_abort) load_b(n + 2);
+                if (n + 2 < p.N && !s_abort) { load_b(n + 2); nb = n + 3; }
                 if (more && SAVE) wait(&bar_df[s], (n / kDeepA) & 1);
             }
             more = __shfl_sync(0xffffffffu, more && !s_abort, 0);     // one answer for the warp
-            if (more) load_a(n + kDeepA, s);
+            if (more) { load_a(n + kDeepA, s); na = n + kDeepA + 1; }
             if (++s == kDeepA) s = 0;
         }
-        if (lead && s_abort) {            // one more bounded chance for copies in flight
-            for (int i = 0; i < kDeepA; ++i) mbar_wait(&bar_la[i], 0);
-            for (int i = 0; i < 2; ++i) mbar_wait(&bar_lb[i], 0);
-        }
+        if (lead) { s_loads[0] = na; s_loads[1] = nb; }
     }
     tc_fence_before();
     __syncthreads();
+    if (s_abort) {                        // a wait has expired, so what is in flight has not been waited for
+        if ((tid >> 5) == kMmaWarp) { umma_commit_w(&bar_end, elect_lane()); mbar_drain(&bar_end, 0); }
+        if (tid == (kMmaWarp + 2) * 32) { mbar_drain_ring(bar_la, kDeepA, s_loads[0]); mbar_drain_ring(bar_lb, 2, s_loads[1]); }
+        __syncthreads();
+    }
     if (tid < 32) tmem_dealloc(tbase, 512);
 }
 
@@ -805,9 +808,10 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     // bar_la, bar_lb: tiles loaded; bar_e: every product of a chunk has finished; bar_a, bar_b: products complete; bar_o, bar_of: an output
     // accumulator is complete / has been read; bar_ht, bar_dt: entry state / Delta^T staged (one arrival per compute warp); bar_hf, bar_df: read
-    __shared__ uint64_t bar_la[kHalfDeep], bar_lb[kHalfDeep], bar_e[kHalfDeep], bar_a, bar_b, bar_o[2], bar_of[2], bar_ht, bar_dt, bar_hf, bar_df;
+    __shared__ uint64_t bar_la[kHalfDeep], bar_lb[kHalfDeep], bar_e[kHalfDeep], bar_a, bar_b, bar_o[2], bar_of[2], bar_ht, bar_dt, bar_hf, bar_df, bar_end;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
+    __shared__ int s_loads;                                  // chunks whose tiles are loaded or on their way
     __shared__ __align__(16) float sG[kHalfDeep][68];        // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C
 
     const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, wq = warp & 3, lane = tid & 31;
@@ -817,7 +821,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
     if (tid == 0) {
         for (int i = 0; i < kHalfDeep; ++i) { mbar_init(&bar_la[i], 1); mbar_init(&bar_lb[i], 1); mbar_init(&bar_e[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&bar_o[i], 1); mbar_init(&bar_of[i], 4); }
-        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1);
+        mbar_init(&bar_a, 1); mbar_init(&bar_b, 1); mbar_init(&bar_end, 1);
         mbar_init(&bar_ht, 16); mbar_init(&bar_dt, 16); mbar_init(&bar_hf, 1); mbar_init(&bar_df, 1);
         mbar_init_fence();
         s_abort = 0;
@@ -1049,17 +1053,17 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
             if (n + 1 < p.N) fetch_g(n + 1);
         };
         fetch_g(0);
-        for (int n = 0; n < kHalfDeep && n < p.N; ++n) load(n, n);
+        int loads = 0;
+        for (; loads < kHalfDeep && loads < p.N; ++loads) load(loads, loads);
         int s = 0;
         uint32_t sp = 0;
-        for (int n = 0; n + kHalfDeep < p.N; ++n) {
-            wait(&bar_e[s], sp);                              // every product of chunk n has finished: refill its buffers
+        for (; loads < p.N; ++loads) {
+            wait(&bar_e[s], sp);                              // every product of the chunk three before has finished: refill its buffers
             if (!__all_sync(0xffffffffu, !s_abort)) break;    // one answer for the warp
-            load(n + kHalfDeep, s);
+            load(loads, s);
             if (++s == kHalfDeep) { s = 0; sp ^= 1; }
         }
-        if (lead && s_abort)              // one more bounded chance for copies in flight
-            for (int i = 0; i < kHalfDeep; ++i) { mbar_wait(&bar_la[i], 0); mbar_wait(&bar_lb[i], 0); }
+        if (lead) s_loads = loads;
     } else if (warp == kMmaWarp + 2) {
         // ---------------------------------- relay warp ----------------------------------
         auto relay = [&](uint64_t* bar, uint32_t parity, int id) {
@@ -1100,6 +1104,12 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
     }
     tc_fence_before();
     __syncthreads();
+    if (s_abort) {                        // a wait has expired, so what is in flight has not been waited for
+        // (from tid: with `warp` kept to here the compute warps get four registers less, 16 x 64 chunks 80.8 -> 83.6 us)
+        if ((tid >> 5) == kMmaWarp) { umma_commit_w(&bar_end, elect_lane()); mbar_drain(&bar_end, 0); }
+        if (tid == (kMmaWarp + 1) * 32) { mbar_drain_ring(bar_la, kHalfDeep, s_loads); mbar_drain_ring(bar_lb, kHalfDeep, s_loads); }
+        __syncthreads();
+    }
     if (tid < 32) tmem_dealloc(tbase, 512);
 }
 

@@ -127,7 +127,7 @@ def test_any_order_of_warps(programs, name, kernel):
 
 
 # what is looked at (emu::kinds)
-EXPIRED = [("tc_fwd.cu", "full", "b"), ("tc_fwd.cu", "half", "b"), ("tc_bwd.cu", "chain", "b"), ("tc_bwd.cu", "chunk", "b")]
+EXPIRED = [("tc_fwd.cu", "full", "bct"), ("tc_fwd.cu", "half", "bct"), ("tc_bwd.cu", "chain", "bct"), ("tc_bwd.cu", "chunk", "bct")]
 
 
 @pytest.mark.parametrize("name,kernel,kinds", EXPIRED)
