@@ -231,7 +231,8 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
         umma_commit_w(&bar_g, issue);
         wait(&bar_x);
         wait(&bar_g);
-        if (lead && !s_abort) {
+        const bool has_v = lead && !s_abort;
+        if (has_v) {
             mbar_expect_tx(&bar_v, 16384);
             for (int blk = 0; blk < 2; ++blk) tma_load_3d(sQ + blk * 8192, &mapV, hh * D + blk * 64, t0, b, &bar_v);
         }
@@ -252,8 +253,11 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
             tma_store_2d(&mapP, sK, 0, (int)wtok0);
             tma_store_commit();
             tma_store_wait_read();             // the staging tiles must outlive the reads; the writes complete with the grid
-            if (s_abort) { mbar_wait(&bar_qk, 0); mbar_wait(&bar_v, 0); }      // one more bounded chance for copies in flight
         }
+        __syncwarp();
+        // A wait has expired: the other warps may still be at their work, which they come to the end of by now without waiting, and what is
+        // in flight has not been waited for
+        if (s_abort) { mbar_drain(&bar_o, 0); mbar_drain(&bar_w, 0); mbar_drain(&bar_qk, 0); if (has_v) mbar_drain(&bar_v, 0); }
         __syncwarp();
         tmem_dealloc(tb, 128);
         if (blockIdx.x == 0) grid_dep_wait();            // when this kernel has completed, so has the one before it

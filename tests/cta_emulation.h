@@ -62,8 +62,6 @@ struct Cta {
 };
 inline Cta* c;
 inline bool c_expired;             // of the last run
-inline std::string kinds = "bct";  // what is looked at: barriers, what has to have completed, tensor memory
-inline bool checks(char kind) { return kinds.find(kind) != std::string::npos; }
 inline dim3 block, blockDim_, gridDim_;
 alignas(1024) inline unsigned char smem[256 * 1024];
 
@@ -178,16 +176,16 @@ inline std::string run(const Scenario& s, int threads, dim3 blk, dim3 grid, std:
         if (!cta.error.empty()) return cta.error;
     }
     for (auto& b : cta.named) if (b.second.arrived) return "arrivals left over at named barrier " + std::to_string(b.first);
-    if (checks('c')) for (const Load& l : cta.loads) if (!l.lost) return "leaves with a load in flight";
-    if (checks('c')) for (const Op& o : cta.tensor) return o.commit ? "leaves with the arrival of a commit to come" : "leaves with a product in flight";
+    for (const Load& l : cta.loads) if (!l.lost) return "leaves with a load in flight";
+    for (const Op& o : cta.tensor) return o.commit ? "leaves with the arrival of a commit to come" : "leaves with a product in flight";
     for (int i = 0; i < n; ++i) if (cta.warps[i].uncommitted || !cta.warps[i].groups.empty()) return "leaves with a store that is still reading";
-    if (checks('t') && (cta.tmem || !cta.tmem_ever)) return "tensor memory not released";
+    if (cta.tmem || !cta.tmem_ever) return "tensor memory not released";
     return "";
 }
 
 inline void touch_tmem(const char* what) {
     yield();
-    if (!c->tmem && checks('t')) fail(std::string(what) + " of tensor memory that is not allocated");
+    if (!c->tmem) fail(std::string(what) + " of tensor memory that is not allocated");
 }
 
 }  // namespace emu
@@ -279,7 +277,7 @@ inline void tmem_alloc(uint32_t* slot, uint32_t) { *slot = 0; emu::c->tmem = emu
 inline void tmem_relinquish() {}
 inline void tmem_dealloc(uint32_t, uint32_t) {
     emu::touch_tmem("release");
-    for (const emu::Op& o : emu::c->tensor) if (!o.commit && emu::checks('c')) emu::fail("tensor memory released under a product");
+    for (const emu::Op& o : emu::c->tensor) if (!o.commit) emu::fail("tensor memory released under a product");
     emu::c->tmem = false;
 }
 inline void tmem_ld_wait() {}

@@ -21,7 +21,6 @@ int main(int argc, char** argv) {
     const std::string name = argv[1];
     const int runs = atoi(argv[2]);
     const double expire = atof(argv[3]), lose = atof(argv[4]);
-    emu::kinds = argv[5];
     int aborted = 0;
     for (int i = 0; i < runs; ++i) {
         emu::Scenario s{(unsigned)i, expire, lose, true};
@@ -115,22 +114,19 @@ def programs(tmp_path_factory):
 ALL = [("tc_fwd.cu", "prep"), ("tc_fwd.cu", "full"), ("tc_fwd.cu", "half"), ("tc_bwd.cu", "chain"), ("tc_bwd.cu", "chunk")]
 
 
-def _run(exe, kernel, runs, expire, lose, kinds):
-    r = subprocess.run([exe, kernel, str(runs), str(expire), str(lose), kinds], capture_output=True, text=True, timeout=600)
+def _run(exe, kernel, runs, expire, lose):
+    r = subprocess.run([exe, kernel, str(runs), str(expire), str(lose)], capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout + r.stderr
 
 
 @pytest.mark.parametrize("name,kernel", ALL)
 def test_any_order_of_warps(programs, name, kernel):
     """No wait expires, and the CTA leaves with everything done."""
-    _run(programs(name), kernel, 100, 0, 0, "bct")
+    _run(programs(name), kernel, 100, 0, 0)
 
 
-# what is looked at (emu::kinds)
-EXPIRED = [("tc_fwd.cu", "full", "bct"), ("tc_fwd.cu", "half", "bct"), ("tc_bwd.cu", "chain", "bct"), ("tc_bwd.cu", "chunk", "bct")]
-
-
-@pytest.mark.parametrize("name,kernel,kinds", EXPIRED)
+@pytest.mark.parametrize("name,kernel", ALL)
 @pytest.mark.parametrize("expire,lose", [(0.0005, 0), (0.05, 0), (0.005, 0.02)], ids=["rare", "early", "lost load"])
-def test_expired_waits(programs, name, kernel, kinds, expire, lose):
-    _run(programs(name), kernel, 200, expire, lose, kinds)
+def test_expired_waits(programs, name, kernel, expire, lose):
+    """Waits expire at any place, copies are lost: the kernel comes to its end all the same, and leaves as cleanly."""
+    _run(programs(name), kernel, 200, expire, lose)
