@@ -179,8 +179,9 @@ __global__ void __launch_bounds__(kPrepThreads, 4) k_tc_prep(const __grid_consta
     const size_t wtok0 = (size_t)bh * p.Tp + (size_t)t0;             // first row in the workspace's [BH*Tp] view
 
     // What a CTA reads is on its way before anything else is set up: with the SM's other CTAs at work a third of its time went by until
-    // Q and K had come.  Prompts of 128 sequences of 32 chunks 164.0 -> 161.4 us, of 4 of 16 24.5 -> 23.8.  (Nothing is read or written
-    // before the kernel before this one has completed.)
+    // Q and K had come.  Prompts of 128 sequences of 32 chunks 164.0 -> 161.4 us, of 4 of 16 24.5 -> 23.8.  Nothing is read or written
+    // before the kernel before this one has completed, unless this one runs beside it: then it reads inputs, which are older than
+    // that chain, and writes rows that the chain does not touch.
     // A token past the end of the sequence is an exact no-op of the recurrence: beta = 0, alpha = 1 (and q = k = v = 0).
     const bf16 zero = __ushort_as_bfloat16(0);
     const bool live = tid < C && t0 + tid < p.T, has_a = live && p.alpha, has_l = live && p.lam;
@@ -1070,6 +1071,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
         if (lead) s_loads = loads;
     } else if (warp == kMmaWarp + 2) {
         // ---------------------------------- relay warp ----------------------------------
+        grid_dep_wait();
         auto relay = [&](uint64_t* bar, uint32_t parity, int id) {
             if (!wait(bar, parity)) mbar_drain(bar, parity);
             tc_fence_after();
@@ -1077,7 +1079,6 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
             __syncwarp();
             nb_arrive(id, nb);
         };
-        grid_dep_wait();
         for (int n = 0; n < p.N; ++n) {
             relay(&bar_a, n & 1, kBarA);
             relay(&bar_b, n & 1, kBarB);

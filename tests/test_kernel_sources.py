@@ -20,15 +20,25 @@ def test_dynamic_shared_memory_is_aligned(name):
             assert re.search(r"\(uintptr_t\)%s \+ 1023\) & ~\(uintptr_t\)1023" % m.group(2), lines[i + 1]), (name, i + 1, line)
 
 
-@pytest.mark.parametrize("name,kernel", [("tc_fwd.cu", "k_tc_chain_fwd"), ("tc_fwd.cu", "k_tc_chain_fwd_half"), ("tc_bwd.cu", "k_tc_chain_bwd"), ("tc_bwd.cu", "k_tc_chunk_bwd")])
-def test_bounded_waits_begin_after_the_kernel_before(name, kernel):
+@pytest.mark.parametrize("name,kernel,waiting", [("tc_fwd.cu", "k_tc_chain_fwd", 5), ("tc_fwd.cu", "k_tc_chain_fwd_half", 6),
+                                                 ("tc_bwd.cu", "k_tc_chain_bwd", 4), ("tc_bwd.cu", "k_tc_chunk_bwd", 3)])
+def test_bounded_waits_begin_after_the_kernel_before(name, kernel, waiting):
     """A CTA may start while the kernel before it runs, for as long as that takes; the time limit of a wait inside the CTA is meant for the
-    CTA's own work, so every role of its warps waits for that kernel before its first bounded wait."""
+    CTA's own work, so every role of its warps waits for that kernel before its first bounded wait: always, or whatever a flag says, or
+    (p.beside, see sm100.cuh) unless the launch depends on nothing of it."""
     src = open(os.path.join(CSRC, name)).read()
     body = src[re.search(r"__global__ [^;{]*\b%s\(" % kernel, src).end():]
     body = body[:body.index("\n}\n")]
     roles = re.split(r"\n *// (?:-{10,}|={10,}) (.+?) (?:-{10,}|={10,})\n", body)
     assert len(roles) >= 9, kernel
+    found = 0
     for role, text in zip(roles[1::2], roles[2::2]):
-        first = re.search(r"\bwait\(&", text)
-        assert first is None or 0 <= text.find("grid_dep_wait()") < first.start(), (kernel, role)
+        first = re.search(r"\bwait\(", text)
+        if first is None:
+            continue
+        found += 1
+        before = text[:first.start()]
+        flags = re.findall(r"^ *if \((!?)p\.(\w+)\) grid_dep_wait\(\);", before, re.M)
+        assert re.search(r"^ *grid_dep_wait\(\);", before, re.M) or ("!", "beside") in flags or \
+            any(("!", f) in flags and ("", f) in flags for _, f in flags), (kernel, role)
+    assert found == waiting, (kernel, found)
