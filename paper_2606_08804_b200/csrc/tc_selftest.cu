@@ -182,7 +182,21 @@ __global__ void __launch_bounds__(128) k_selftest_frag(const __grid_constant__ C
     const uint32_t tbase = uniform(tmem_slot), aA = tbase + 128;
     const int RA = A_MN ? a.K : M, CA = A_MN ? M : a.K, RB = B_MN ? a.K : a.N, CB = B_MN ? a.N : a.K;
     const uint32_t a_blk = (uint32_t)RA * 128u, b_blk = (uint32_t)RB * 128u;
-    if (a.a_tmem) {            // A is [128][K]: thread = row
+    const int fr = lane >> 2, fc = 2 * (lane & 3);      // fragments: rows fr, fr + 8, of every 8 columns fc, fc + 1
+    if (a.a_tmem && M == 64) { // A is [64][K]: 16 rows to a warp, in fragments of 16 (K = 64) or 32 columns
+        const __nv_bfloat16* row = a.A + (size_t)(16 * warp + fr) * a.K + fc;
+        for (int c = 0; c < a.K; c += a.K / 4) {
+            uint32_t r[8];
+            for (int i = 0; i < a.K / 16; ++i) {
+                const __nv_bfloat16* x = row + (size_t)(8 * (i & 1)) * a.K + c + 8 * (i >> 1);
+                r[i] = pack_bf16(__bfloat162float(x[0]), __bfloat162float(x[1]));
+            }
+            if (a.K == 64) tmem_st_frag2(tmem_addr(aA, warp * 32, c / 2), r);
+            else tmem_st_frag4(tmem_addr(aA, warp * 32, c / 2), r);
+        }
+        tmem_st_wait();
+        tc_fence_before();
+    } else if (a.a_tmem) {     // A is [128][K]: thread = row
         for (int c8 = 0; c8 < a.K / 16; ++c8) {
             uint32_t r[8];
             for (int j = 0; j < 8; ++j)
@@ -204,7 +218,7 @@ __global__ void __launch_bounds__(128) k_selftest_frag(const __grid_constant__ C
         const uint32_t issue = elect_lane();
         tc_fence_after();
         for (int pass = 0; pass < 2; ++pass) {
-            if (a.a_tmem) umma_product_ts_w<B_MN>(tbase, aA, smem_u32(sB), b_blk, a.N, a.K, pass > 0, issue, a.neg != 0);
+            if (a.a_tmem) umma_product_ts_w<B_MN, M>(tbase, aA, smem_u32(sB), b_blk, a.N, a.K, pass > 0, issue, a.neg != 0);
             else umma_product_w<A_MN, B_MN, M>(tbase, smem_u32(sA), a_blk, smem_u32(sB), b_blk, a.N, a.K, pass > 0, issue, a.neg != 0);
         }
         umma_commit_w(&bar_mma, issue);
@@ -219,19 +233,19 @@ __global__ void __launch_bounds__(128) k_selftest_frag(const __grid_constant__ C
             a.D[(size_t)r * a.N + c] = v[0];
             a.D[(size_t)r * a.N + c + 1] = v[1];
         };
-        const int fr = lane >> 2, fc = 2 * (lane & 3);
         uint32_t r[4], back[4];
         if (M == 64) {
             for (int cg = 0; cg < a.N / 16; ++cg) {
-                float v[8];
-                tmem_ld_frag2(tmem_addr(tbase, warp * 32, cg * 16), v);
+                float v[16];
+                if (a.a_tmem) tmem_ld_frag4(tmem_addr(tbase, warp * 32, (cg >> 1) * 32), v);
+                else tmem_ld_frag2(tmem_addr(tbase, warp * 32, cg * 16), v);
                 tmem_ld_wait();
                 for (int m = 0; m < 4; ++m) {
-                    const float* x = v + 4 * (m >> 1) + 2 * (m & 1);
+                    const float* x = v + (a.a_tmem ? 8 * (cg & 1) : 0) + 4 * (m >> 1) + 2 * (m & 1);
                     put(16 * warp + fr + 8 * (m & 1), cg * 16 + 8 * (m >> 1) + fc, x);
                     r[m] = pack_bf16(x[0], x[1]);
                 }
-                unsigned char* at = sT + sw128_chunk(16 * warp + (lane & 15), 2 * cg + (lane >> 4));
+                unsigned char* at = sT + (cg >> 2) * 8192 + sw128_chunk(16 * warp + (lane & 15), 2 * (cg & 3) + (lane >> 4));
                 stsm4<false>(at, r);
                 __syncwarp();
                 ldsm4<false>(at, back);
@@ -278,8 +292,8 @@ extern "C" int qdelta_selftest_frag(const void* A, const void* B, float* D, void
                                     int a_tmem, int neg, unsigned* status, qd_stream stream) {
     using namespace qd;
     if (!A || !B || !D || !tile || !status) return QD_ERR_INVALID_ARG;
-    if ((M != 64 && M != 128) || (N != 64 && N != 128) || (K != 64 && K != 128) || (M == 64 && N != 64)) return QD_ERR_UNSUPPORTED;
-    if (a_tmem && (M != 128 || a_mn)) return QD_ERR_UNSUPPORTED;
+    if ((M != 64 && M != 128) || (N != 64 && N != 128) || (K != 64 && K != 128) || (M == 64 && N != 64 && !a_tmem)) return QD_ERR_UNSUPPORTED;
+    if (a_tmem && a_mn) return QD_ERR_UNSUPPORTED;
     FragArgs a{(const __nv_bfloat16*)A, (const __nv_bfloat16*)B, D, (__nv_bfloat16*)tile, N, K, a_tmem, neg, status};
     const int RA = a_mn ? K : M, CA = a_mn ? M : K, RB = b_mn ? K : N, CB = b_mn ? N : K;
     CUtensorMap mA, mB;

@@ -38,7 +38,7 @@ def test_umma_product(N, K, a_mn, b_mn, by_threads):
 
 _FRAG = [(128, N, K, a_mn, b_mn, 0) for N in (64, 128) for K in (64, 128) for a_mn in (0, 1) for b_mn in (0, 1)]
 _FRAG += [(64, 64, K, a_mn, b_mn, 0) for K in (64, 128) for a_mn in (0, 1) for b_mn in (0, 1)]
-_FRAG += [(128, N, K, 0, b_mn, 1) for N in (64, 128) for K in (64, 128) for b_mn in (0, 1)]
+_FRAG += [(M, N, K, 0, b_mn, 1) for M in (128, 64) for N in (64, 128) for K in (64, 128) for b_mn in (0, 1)]
 
 
 @pytest.mark.parametrize("M,N,K,a_mn,b_mn,a_tmem", _FRAG)
