@@ -52,10 +52,12 @@ def test_preparation_edges(T):
 @pytest.mark.parametrize("without", ["", "alpha lam", "h0"])
 def test_half_chain_edges(T, without):
     """Two CTAs to a sequence, their tiles three deep: as many chunks as that, one fewer, one more, twice around; without a forget gate (one
-    copy of Delta^T instead of two); and a prompt has the bits of a forward with saves."""
+    copy of Delta^T instead of two); normalised in the kernels too; and a prompt has the bits of a forward with saves."""
     import torch
 
+    import gpu_util as gu
     from gpu_util import dev_inputs
+    from oracle import recurrence as orc
     from paper_2606_08804_b200 import binding as qd
 
     cfg = replace(gen.CONFIGS["cfg2"], B=2, H=3, T=T, regime="trained_like", seed=419 + T)
@@ -69,6 +71,35 @@ def test_half_chain_edges(T, without):
     for norm in (False, True):
         (o, hT, _), (p, hP, _) = (qd.chunk_fwd(*a, save_for_bwd=s, norm_qk=norm) for s in (True, False))
         assert torch.equal(o, p) and torch.equal(hT, hP)
+        if norm:
+            ro, rh = orc.forward_fused(*(d[n] for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")), norm_qk=True)
+            gu.check("half chain norm", "o", o, ro, cfg.dtype)
+            gu.check("half chain norm", "hT", hT, rh, cfg.dtype, state=True)
+
+
+@pytest.mark.parametrize("T", [64, 64 * 3 + 1, 64 * 7 - 1])
+@pytest.mark.parametrize("norm", [False, True])
+def test_half_and_whole_chain_have_the_same_bits(T, norm):
+    """74 sequences take two CTAs each, 75 one: what the first 74 of 75 come to does not depend on it, prompts, saves and gradients."""
+    import torch
+
+    from gpu_util import dev_inputs
+    from paper_2606_08804_b200 import binding as qd
+
+    cfg = replace(gen.CONFIGS["cfg2"], B=75, H=1, T=T, regime="trained_like", seed=617 + T)
+    t = dev_inputs(gen.make_chunk_inputs(cfg), cfg.dtype)
+
+    def run(B):
+        a = [t[n][:B].contiguous() for n in ("q", "k", "v", "beta", "alpha", "lam", "h0")]
+        p, hP, _ = qd.chunk_fwd(*a, save_for_bwd=False, norm_qk=norm)
+        o, hT, ws = qd.chunk_fwd(*a, save_for_bwd=True, norm_qk=norm)
+        g = qd.chunk_bwd(*a, t["dO"][:B].contiguous(), t["dhT"][:B].contiguous(), workspace=ws, reuse_fwd=True, want_dh0=True, norm_qk=norm)
+        assert qd.workspace_status(ws) == 0
+        return [p, hP, o, hT] + [x for x in g.values() if x is not None]
+    half, whole = run(74), run(75)
+    assert len(half) == len(whole) > 10
+    for x, y in zip(half, whole):
+        assert torch.equal(x, y[:74])
 
 
 @pytest.mark.parametrize("B,H,T,parts", [(1, 16, 64 * 64, (2, 2)), (2, 20, 64 * 64 + 1, (2, 1)), (1, 4, 64 * 256, (3, 2)),
