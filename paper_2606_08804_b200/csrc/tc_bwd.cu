@@ -12,6 +12,7 @@
 //                   ones in natural orientation as 64-row instructions, 16 rows on each warp of a warpgroup;
 //                   row dot-products that run across lanes use a warp-shuffle column reduction.
 // All waits are bounded (see tc_fwd.cu).
+#include "chain.cuh"
 #include "internal.h"
 #include "sm100.cuh"
 
@@ -125,7 +126,6 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
     auto wait = [&](uint64_t* br, uint32_t parity) { return mbar_try_wait(br, parity) || wait_on(br, parity, s_abort, p.status); };
     const int tok0 = p.n0 * C;                                       // first token; rows and tiles of the workspace start at
     const size_t row0 = (size_t)bh * p.Tp + tok0, tile0 = (size_t)bh * p.Ns + p.n0;
-    const float* gseq = p.g + row0;
 
     if (warp < kMmaWarp && wq >= nwq) {
         // lanes without a row: straight to the end
@@ -285,22 +285,12 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
     } else {
         // ---------------------------------- TMA load warp ----------------------------------
         const bool lead = (tid & 31) == 0;
-        const int ln = tid & 31;
         grid_dep_wait();
         grid_dep_launch();
         // iteration `it` processes chunk n = N-1-it
-        const float* rkseq = p.rk ? p.rk + row0 : nullptr;
-        float g0, g1, gc, r0 = 1.f, r1 = 1.f;             // log-decays (and 1/|k|) of the next chunk to be loaded
-        auto fetch_g = [&](int it) {
-            const size_t at = (size_t)(p.N - 1 - it) * C;
-            g0 = gseq[at + ln]; g1 = gseq[at + 32 + ln]; gc = gseq[at + C - 1];
-            if (rkseq) { r0 = rkseq[at + ln]; r1 = rkseq[at + 32 + ln]; }
-        };
+        TokenScales ts(p.g, p.rk, row0, tid & 31);
         auto load_k = [&](int it, int s) {               // by the whole warp
-            float* sg = sG[it & 3];
-            sg[ln] = __expf(gc - g0) * r0;
-            sg[32 + ln] = __expf(gc - g1) * r1;
-            if (ln == 0) sg[64] = __expf(gc);
+            ts.put(sG[it & 3]);
             __syncwarp();
             if (lead) {
                 const int n = p.N - 1 - it;
@@ -310,7 +300,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
                 tma_load_3d(st + 8192, &mapK, hh * D + 64, tok0 + n * C, b, &bar.k[s]);
                 tma_load_2d(st + 16384, &mapP, 0, (int)(row0 + (size_t)n * C), &bar.k[s]);
             }
-            if (it + 1 < p.N) fetch_g(it + 1);
+            if (it + 1 < p.N) ts.fetch(p.N - 2 - it);
         };
         auto load_q = [&](int it) {                      // by the leading lane
             const int n = p.N - 1 - it;
@@ -327,7 +317,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
             mbar_expect_tx(&bar.w[it & 1], 16384);
             tma_load_2d(smem + offW + (it & 1) * 16384, &mapWt, 0, (int)((tile0 + (p.N - 1 - it)) * D), &bar.w[it & 1]);
         };
-        fetch_g(0);
+        ts.fetch(p.N - 1);
         for (int it = 0; it < kDeepK && it < p.N; ++it) {
             load_k(it, it);
             if (lead && it < 2) { load_q(it); load_w(it); }

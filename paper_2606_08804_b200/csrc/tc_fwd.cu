@@ -13,6 +13,7 @@
 // With few long sequences the two run beside each other, part by part (tc_fwd_parts).
 // All waits are bounded; on expiry the CTA records QD_ERR_TIMEOUT in the workspace status word, lets what it has in flight
 // come to an end (mbar_drain), releases its tensor memory and returns.
+#include "chain.cuh"
 #include "internal.h"
 #include "sm100.cuh"
 #include "tf32.cuh"
@@ -444,6 +445,32 @@ constexpr int kOutWarp = kChainCompute / 32, kMmaWarp = kOutWarp + 4;
 // named barriers: compute threads arrive, the MMA warp waits (they run in lock-step); kBarOut: the output warpgroup among itself
 constexpr int kBarH = 1, kBarD = 2, kBarOut = 3;
 
+// What the saving warp of a forward chain does, one lane of it: entry state of every chunk (two 64-column blocks, `block` bytes apart) and
+// Delta^T, in the order in which they are staged; the state's tile is one deep, Delta^T's DEEP, `stage` bytes apart.
+template <int DEEP, class Wait>
+__device__ __forceinline__ void save_chunks(const CUtensorMap* mapHs, const CUtensorMap* mapDt, size_t row, int N, const unsigned char* sHs, int block,
+                                            const unsigned char* sDt, int stage, uint64_t* ht, uint64_t* hf, uint64_t* dt, uint64_t* df, Wait wait) {
+    int s = 0;
+    for (int n = 0; n < N; ++n) {
+        const int y = (int)(row + (size_t)n * D);
+        wait(ht, n & 1);                                  // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
+        tma_store_2d(mapHs, sHs, 0, y);
+        tma_store_2d(mapHs, sHs + block, 64, y);
+        tma_store_commit();
+        if (n > 0) {                                      // Delta^T of chunk n - 1 has been read
+            tma_store_wait_read_n<1>();
+            mbar_arrive(df + (s == 0 ? DEEP - 1 : s - 1));
+        }
+        wait(dt + s, (n / DEEP) & 1);                     // Delta^T of chunk n is staged
+        tma_store_2d(mapDt, sDt + s * stage, 0, y);
+        tma_store_commit();
+        tma_store_wait_read_n<1>();                       // the entry state has been read
+        mbar_arrive(hf);
+        if (++s == DEEP) s = 0;
+    }
+    tma_store_wait_all();
+}
+
 // Forward state chain.  The only true dependency per chunk is
 //   h ready -> Delta-accumulator = h^T Wt -> Delta^T -> H-accumulator = (scaled Delta^T) K -> h update;
 // the output products (h^T Qg^T + Delta^T P^T, double-buffered accumulator), the output epilogue and
@@ -515,7 +542,6 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_try_wait(bar, parity) || wait_on(bar, parity, s_abort, p.status); };
     const int tok0 = p.n0 * C;                                       // first token; rows and tiles of the workspace start at
     const size_t row0 = (size_t)bh * p.Tp + tok0, tile0 = (size_t)bh * p.Ns + p.n0;
-    const float* gseq = p.g + row0;
 
     if (warp < kOutWarp) {
         // ---------------------------------- compute warps ----------------------------------
@@ -690,44 +716,16 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
         // apart from the loads, which would otherwise wait for what these wait for
         if ((tid & 31) == 0 && SAVE) {
             grid_dep_wait();
-            int s = 0;
-            for (int n = 0; n < p.N; ++n) {
-                const int y = (int)((tile0 + n) * D);
-                wait(&bar_ht, n & 1);                     // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
-                tma_store_2d(&mapHs, sHs, 0, y);
-                tma_store_2d(&mapHs, sHs + 16384, 64, y);
-                tma_store_commit();
-                if (n > 0) {                              // Delta^T of chunk n - 1 has been read
-                    tma_store_wait_read_n<1>();
-                    mbar_arrive(&bar_df[s == 0 ? kDeepA - 1 : s - 1]);
-                }
-                wait(&bar_dt[s], (n / kDeepA) & 1);       // Delta^T of chunk n is staged
-                tma_store_2d(&mapDt, smem + s * kStageA + 16384, 0, y);
-                tma_store_commit();
-                tma_store_wait_read_n<1>();               // the entry state has been read
-                mbar_arrive(&bar_hf);
-                if (++s == kDeepA) s = 0;
-            }
-            tma_store_wait_all();
+            save_chunks<kDeepA>(&mapHs, &mapDt, tile0 * D, p.N, sHs, 16384, smem + 16384, kStageA, &bar_ht, &bar_hf, bar_dt, bar_df, wait);
         }
     } else {
         // ---------------------------------- TMA load warp ----------------------------------
         const bool lead = (tid & 31) == 0;
         grid_dep_wait();                  // the tiles and the log-decays read below are written by the prep kernel
         grid_dep_launch();
-        const int ln = tid & 31;
-        const float* rkseq = p.rk ? p.rk + row0 : nullptr;
-        // log-decays (and 1/|k|) of the next chunk to be loaded, fetched ahead
-        float g0, g1, gc, r0 = 1.f, r1 = 1.f;
-        auto fetch_g = [&](int n) {
-            const float* gn = gseq + (size_t)n * C;
-            g0 = gn[ln]; g1 = gn[32 + ln]; gc = gn[C - 1];
-            if (rkseq) { r0 = rkseq[(size_t)n * C + ln]; r1 = rkseq[(size_t)n * C + 32 + ln]; }
-        };
+        TokenScales ts(p.g, p.rk, row0, tid & 31);
         auto load_a = [&](int n, int s) {                // by the whole warp
-            sG[s][ln] = __expf(gc - g0) * r0;
-            sG[s][32 + ln] = __expf(gc - g1) * r1;
-            if (ln == 0) sG[s][64] = __expf(gc);
+            ts.put(sG[s]);
             __syncwarp();
             if (lead) {
                 const int yc = (int)((tile0 + n) * D);
@@ -735,7 +733,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
                 tma_load_2d(smem + s * kStageA, &mapWt, 0, yc, &bar_la[s]);
                 tma_load_2d(smem + s * kStageA + 16384, &mapUt, 0, yc, &bar_la[s]);
             }
-            if (n + 1 < p.N) fetch_g(n + 1);
+            if (n + 1 < p.N) ts.fetch(n + 1);
         };
         auto load_b = [&](int n) {                       // by the leading lane
             unsigned char* st = smem + kOffB + (n & 1) * kStageB;
@@ -748,7 +746,7 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             tma_load_3d(st + 16384 + 8192, &mapK, hh * D + 64, tok0 + n * C, b, bar);
             tma_load_2d(st + 32768, &mapP, 0, yt, bar);
         };
-        fetch_g(0);
+        ts.fetch(0);
         for (int n = 0; n < kDeepA && n < p.N; ++n) {
             load_a(n, n);
             if (lead && n < 2) load_b(n);
@@ -1029,18 +1027,9 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
         const bool lead = lane == 0;
         grid_dep_wait();                  // the tiles and the log-decays read below are written by the prep kernel
         grid_dep_launch();
-        const float *gseq = p.g + row0, *rkseq = p.rk ? p.rk + row0 : nullptr;
-        // log-decays (and 1/|k|) of the next chunk to be loaded, fetched ahead
-        float g0, g1, gc, k0 = 1.f, k1 = 1.f;
-        auto fetch_g = [&](int n) {
-            const float* gn = gseq + (size_t)n * C;
-            g0 = gn[lane]; g1 = gn[32 + lane]; gc = gn[C - 1];
-            if (rkseq) { k0 = rkseq[(size_t)n * C + lane]; k1 = rkseq[(size_t)n * C + 32 + lane]; }
-        };
+        TokenScales ts(p.g, p.rk, row0, lane);
         auto load = [&](int n, int s) {                       // by the whole warp
-            sG[s][lane] = __expf(gc - g0) * k0;
-            sG[s][32 + lane] = __expf(gc - g1) * k1;
-            if (lane == 0) sG[s][64] = __expf(gc);
+            ts.put(sG[s]);
             __syncwarp();
             if (lead) {
                 const int yc = (int)((tile0 + n) * D), yt = (int)(row0 + (size_t)n * C);
@@ -1055,9 +1044,9 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
                 tma_load_3d(sb + 16384 + 8192, &mapK, hh * D + 64, tok0 + n * C, b, &bar_lb[s]);
                 tma_load_2d(sb + 32768, &mapP, 0, yt, &bar_lb[s]);
             }
-            if (n + 1 < p.N) fetch_g(n + 1);
+            if (n + 1 < p.N) ts.fetch(n + 1);
         };
-        fetch_g(0);
+        ts.fetch(0);
         int loads = 0;
         for (; loads < kHalfDeep && loads < p.N; ++loads) load(loads, loads);
         int s = 0;
@@ -1086,25 +1075,8 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
     } else {
         // ---------------------------------- saving warp ----------------------------------
         if (lane == 0 && SAVE) {
-            unsigned char *sHs = smem + kHalfOffS, *sDt = sHs + 16384;
             grid_dep_wait();
-            for (int n = 0; n < p.N; ++n) {
-                const int y = (int)((tile0 + n) * D) + v0;
-                wait(&bar_ht, n & 1);                         // entry state of chunk n (rows = d_v index, columns = d_k index) is staged
-                tma_store_2d(&mapHs, sHs, 0, y);
-                tma_store_2d(&mapHs, sHs + 8192, 64, y);
-                tma_store_commit();
-                if (n > 0) {                                  // Delta^T of chunk n - 1 has been read
-                    tma_store_wait_read_n<1>();
-                    mbar_arrive(&bar_df);
-                }
-                wait(&bar_dt, n & 1);                         // Delta^T of chunk n is staged
-                tma_store_2d(&mapDt, sDt, 0, y);
-                tma_store_commit();
-                tma_store_wait_read_n<1>();                   // the entry state has been read
-                mbar_arrive(&bar_hf);
-            }
-            tma_store_wait_all();
+            save_chunks<1>(&mapHs, &mapDt, tile0 * D + v0, p.N, smem + kHalfOffS, 8192, smem + kHalfOffS + 16384, 0, &bar_ht, &bar_hf, &bar_dt, &bar_df, wait);
         }
     }
     tc_fence_before();
@@ -1199,7 +1171,7 @@ bool setup(const ChunkArgs& a, ChainCall& c) {
     const int rows = chain_rows(BH);
     if (!make_tmap_bf16_2d(&c.mHs, a.ws + a.TL.hsT, D, BH * Ns * D, D * 2, rows) ||
         !make_tmap_bf16_2d(&c.mDt, a.ws + a.TL.Dt, 64, BH * Ns * D, 128, rows) ||
-        !make_tmap_tokens(&c.mO, a.o, s.B, s.T, s.H, D, 32) ||
+        (rows == D && !make_tmap_tokens(&c.mO, a.o, s.B, s.T, s.H, D, 32)) ||
         !make_tmap_bf16_2d(&c.mWt, a.ws + a.TL.Wt, 64, BH * Ns * D, 128, 128) ||
         !make_tmap_bf16_2d(&c.mUt, a.ws + a.TL.Ut, 64, BH * Ns * D, 128, rows) ||
         !make_tmap_bf16_2d(&c.mQg, a.ws + a.TL.Qg, D, BH * Tp, D * 2, 64) ||
