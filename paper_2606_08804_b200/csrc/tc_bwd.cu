@@ -65,7 +65,7 @@ constexpr int kBarH = 1, kBarD = 2;
 
 // A barrier per buffer where one side may run ahead.  k, q, w: tiles loaded; fk, fq, fw: read by their last product; ht, dt:
 // staged (one arrival per compute warp); hf, df: read by their store (two deep: hf alone, for both); a, b: products complete;
-// end: all of them, after a wait has expired.
+// end: all of them.
 struct ChainBars { uint64_t k[kDeepK], fk[kDeepK], q[2], fq[2], w[2], fw[2], hf[2], df, a, b, end, ht[2], dt[2]; };
 
 // Reverse state chain.  Per chunk the dependency is
@@ -97,7 +97,6 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
     __shared__ ChainBars bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
-    __shared__ int s_loads[3];                         // issued in all: K and P; Qg and dO; Wt
     // gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the load warp before it arrives on bar.k.  One deeper than
     // K and P: those are dead when A2 is complete, but the epilogue reads these after that
     float (*sG)[68] = reinterpret_cast<float (*)[68]>(smem + kOffG);
@@ -256,6 +255,8 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
             if (++s == kDeepK) { s = 0; sp ^= 1; }
             if (it + 1 < p.N) ahead(it + 1);            // in the shadow of the dh update
         }
+        umma_commit_w(&bar.end, issue);                 // leaves when its products have come to their end, whatever has expired
+        mbar_drain(&bar.end, 0);
     } else if (warp == kMmaWarp + 1) {
         // ---------------------------------- saving warp ----------------------------------
         if ((tid & 31) == 0) {
@@ -341,15 +342,11 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_bwd(const __grid_con
             __syncwarp();
             if (++s == kDeepK) { s = 0; sp ^= 1; }
         }
-        if (lead) { s_loads[0] = nk; s_loads[1] = nq; s_loads[2] = nw; }
+        // unless a wait has expired the products have been waited for, and so have the loads
+        if (lead && s_abort) { mbar_drain_ring(bar.k, kDeepK, nk); mbar_drain_ring(bar.q, 2, nq); mbar_drain_ring(bar.w, 2, nw); }
     }
     tc_fence_before();
     __syncthreads();
-    if (s_abort) {                        // a wait has expired, so what is in flight has not been waited for
-        if ((tid >> 5) == kMmaWarp) { umma_commit_w(&bar.end, elect_lane()); mbar_drain(&bar.end, 0); }
-        if (tid == (kMmaWarp + 2) * 32) { mbar_drain_ring(bar.k, kDeepK, s_loads[0]); mbar_drain_ring(bar.q, 2, s_loads[1]); mbar_drain_ring(bar.w, 2, s_loads[2]); }
-        __syncthreads();
-    }
     if (tid < 32) tmem_dealloc(tbase, 512);
 }
 
@@ -431,7 +428,6 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     __shared__ ChunkBars bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort, s_latch[2];                  // s_latch[it % 2]: a wait had expired before iteration it
-    __shared__ int s_loads[3];                                    // issued in all: bar.load and bar.d, bar.h, bar.qk
     ChunkShared& sh = *reinterpret_cast<ChunkShared*>(sm + kTileBytes);
     auto &sbeta_ = sh.sbeta_, &sg_ = sh.sg_, &slam_ = sh.slam_, &sgam_ = sh.sgam_;
     auto& scf_ = sh.scf_;
@@ -592,6 +588,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             umma_commit_w(&bar.m5, issue);
             nb_sync(kNbEnd, kBwdThreads);                                // every read of this chunk's tiles and accumulators is done
         }
+        umma_commit_w(&bar.end, issue);                                  // leaves when its products have come to their end, whatever has expired
+        mbar_drain(&bar.end, 0);
     } else if (tid >= kBwdNb && tid < kBwdTail) {
         // =============================== TMA warp ===============================
         const bool lead = lane == 0;
@@ -656,7 +654,10 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
             }
             __syncwarp();
         }
-        if (lead) { s_loads[0] = ne; s_loads[1] = nh; s_loads[2] = nqk; tma_store_wait_all(); }
+        if (lead && s_abort) {        // otherwise the products have been waited for, and so have the loads
+            mbar_drain_ring(&bar.load, 1, ne); mbar_drain_ring(&bar.d, 1, ne); mbar_drain_ring(&bar.h, 1, nh); mbar_drain_ring(&bar.qk, 1, nqk);
+        }
+        if (lead) tma_store_wait_all();
     } else if (tid >= kBwdTail) {
         // =============================== token threads ===============================
         // thread r owns token r of the chunk
@@ -1112,14 +1113,6 @@ __global__ void __launch_bounds__(kBwdThreads) k_tc_chunk_bwd(const __grid_const
     }  // epilogue threads
     tc_fence_before();
     __syncthreads();
-    if (s_abort) {                        // a wait has expired, so what is in flight has not been waited for
-        if ((tid >> 5) == kBwdCompute / 32) { umma_commit_w(&bar.end, elect_lane()); mbar_drain(&bar.end, 0); }
-        if (tid == kBwdNb) {
-            mbar_drain_ring(&bar.load, 1, s_loads[0]); mbar_drain_ring(&bar.d, 1, s_loads[0]);
-            mbar_drain_ring(&bar.h, 1, s_loads[1]); mbar_drain_ring(&bar.qk, 1, s_loads[2]);
-        }
-        __syncthreads();
-    }
     if (tid < 32) tmem_dealloc(tb, 512);
     if (tid == 0 && blockIdx.x == 0) grid_dep_wait();            // when this kernel has completed, so has the one before it
 }

@@ -511,7 +511,6 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
     __shared__ uint64_t bar_la[kDeepA], bar_lb[2], bar_e[2], bar_dt[kDeepA], bar_df[kDeepA], bar_ht, bar_hf, bar_a, bar_b, bar_o[2], bar_of[2], bar_end;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
-    __shared__ int s_loads[2];                      // issued in all: Wt and Ut; Qg, K and P
     // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C; written by the TMA warp before it arrives on the
     // stage's load barrier, so no epilogue thread waits for a global load
     __shared__ __align__(16) float sG[kDeepA][68];
@@ -711,6 +710,8 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             if (++s == kDeepA) s = 0;
         }
         nb_sync(kBarH, nb);                               // final arrival of the compute warps
+        umma_commit_w(&bar_end, issue);                   // leaves when its products have come to their end, whatever has expired
+        mbar_drain(&bar_end, 0);
     } else if (warp == kMmaWarp + 1) {
         // ---------------------------------- saving warp ----------------------------------
         // apart from the loads, which would otherwise wait for what these wait for
@@ -763,15 +764,11 @@ __global__ void __launch_bounds__(kChainThreads) k_tc_chain_fwd(const __grid_con
             if (more) { load_a(n + kDeepA, s); na = n + kDeepA + 1; }
             if (++s == kDeepA) s = 0;
         }
-        if (lead) { s_loads[0] = na; s_loads[1] = nb; }
+        // unless a wait has expired the products have been waited for, and so have the loads
+        if (lead && s_abort) { mbar_drain_ring(bar_la, kDeepA, na); mbar_drain_ring(bar_lb, 2, nb); }
     }
     tc_fence_before();
     __syncthreads();
-    if (s_abort) {                        // a wait has expired, so what is in flight has not been waited for
-        if ((tid >> 5) == kMmaWarp) { umma_commit_w(&bar_end, elect_lane()); mbar_drain(&bar_end, 0); }
-        if (tid == (kMmaWarp + 2) * 32) { mbar_drain_ring(bar_la, kDeepA, s_loads[0]); mbar_drain_ring(bar_lb, 2, s_loads[1]); }
-        __syncthreads();
-    }
     if (tid < 32) tmem_dealloc(tbase, 512);
 }
 
@@ -814,7 +811,6 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
     __shared__ uint64_t bar_la[kHalfDeep], bar_lb[kHalfDeep], bar_e[kHalfDeep], bar_a, bar_b, bar_o[2], bar_of[2], bar_ht, bar_dt, bar_hf, bar_df, bar_end;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
-    __shared__ int s_loads;                                  // chunks whose tiles are loaded or on their way
     __shared__ __align__(16) float sG[kHalfDeep][68];        // per stage: gamma_C / gamma_t for the 64 tokens, then gamma_C
 
     const int tid = threadIdx.x, warp = warp_index(), wg = warp >> 2, wq = warp & 3, lane = tid & 31;
@@ -1022,6 +1018,8 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
             if (n + kHalfDeep < p.N) umma_commit_w(&bar_e[st], issue);      // the load warp waits for these: nothing arrives in a CTA that has left
         }
         nb_sync(kBarH, nb);                                   // final arrival of the compute warps
+        umma_commit_w(&bar_end, issue);                       // leaves when its products have come to their end, whatever has expired
+        mbar_drain(&bar_end, 0);
     } else if (warp == kMmaWarp + 1) {
         // ---------------------------------- TMA load warp ----------------------------------
         const bool lead = lane == 0;
@@ -1057,7 +1055,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
             load(loads, s);
             if (++s == kHalfDeep) { s = 0; sp ^= 1; }
         }
-        if (lead) s_loads = loads;
+        if (lead) { mbar_drain_ring(bar_la, kHalfDeep, loads); mbar_drain_ring(bar_lb, kHalfDeep, loads); }      // leaves when its loads have come
     } else if (warp == kMmaWarp + 2) {
         // ---------------------------------- relay warp ----------------------------------
         grid_dep_wait();
@@ -1081,12 +1079,6 @@ __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid
     }
     tc_fence_before();
     __syncthreads();
-    if (s_abort) {                        // a wait has expired, so what is in flight has not been waited for
-        // (from tid: with `warp` kept to here the compute warps get four registers less, 16 x 64 chunks 80.8 -> 83.6 us)
-        if ((tid >> 5) == kMmaWarp) { umma_commit_w(&bar_end, elect_lane()); mbar_drain(&bar_end, 0); }
-        if (tid == (kMmaWarp + 1) * 32) { mbar_drain_ring(bar_la, kHalfDeep, s_loads); mbar_drain_ring(bar_lb, kHalfDeep, s_loads); }
-        __syncthreads();
-    }
     if (tid < 32) tmem_dealloc(tbase, 512);
 }
 
