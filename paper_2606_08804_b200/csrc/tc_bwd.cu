@@ -73,11 +73,12 @@ struct ChainBars { uint64_t k[kDeepK], fk[kDeepK], q[2], fq[2], w[2], fw[2], hf[
 // A1 = dO^T P and the dO^T Qg part of the H-accumulator do not depend on dh and are issued a chunk ahead (double-buffered
 // H-accumulator).  As in the forward chain, the dependent operands (dh^T, -dDelta^T) live in tensor memory and the issuing
 // warp stays converged.  With few sequences two CTAs share the d_v rows of one (ROWS = 64).
-// With 128 rows what bounds a chunk is the SM's TMA unit, 72 KB in at 45 and 48 KB out at 32 bytes per cycle, one after the other:
-// 3150 cycles.  With 64 it is the sequence of hand-offs, so nothing that can be elsewhere is on it: a wait that has long been
+// With 128 rows what bounds a chunk is HBM if there are many sequences; with few (2500 cycles) the SM's TMA unit, which is busy for
+// 2200 of them: 72 KB in at 98 - 113 bytes per cycle and 48 KB out at 32, which add up.  With 64 it is the sequence of hand-offs (1930
+// cycles with 1 - 32 sequences, of which TMA 1310 - 1370), so nothing that can be elsewhere is on it: a wait that has long been
 // satisfied costs 100 - 200 cycles, so the next chunk's scales are waited for under the last product, one barrier stands for both
-// staged tiles, the tiles are staged two deep, and a wait polls before it looks at the abort flag (2540 -> 2250 cycles a chunk;
-// 92 -> 85 us on 4 sequences of 64 chunks, backward).
+// staged tiles, the tiles are staged two deep, and a wait polls before it looks at the abort flag (4 sequences of 64 chunks, backward,
+// 92 -> 85 us when that was done).
 // Compute warpgroup w owns tokens [16w, 16w+16) of the 64-column accumulators and d_k columns
 // [32w, 32w+32) of dh^T; thread l of a warpgroup owns TMEM lane l = d_v index.
 template <int ROWS>

@@ -475,19 +475,20 @@ __device__ __forceinline__ void save_chunks(const CUtensorMap* mapHs, const CUte
 //   h ready -> Delta-accumulator = h^T Wt -> Delta^T -> H-accumulator = (scaled Delta^T) K -> h update;
 // the output products (h^T Qg^T + Delta^T P^T, double-buffered accumulator), the output epilogue and
 // every TMA copy run in its shadow on their own warps.
-// What bounds a chunk is that sequence, if nothing gets in its way (2050 cycles when nothing is saved).  Three things did, 3800
-// cycles per chunk of 64 tokens:
+// With many sequences HBM bounds it: 75 of 256 chunks move 6.2 TB/s with saves.  With few, a chunk takes 2210 cycles when nothing is
+// saved and 3330 with saves.  Three things were in the way of that sequence:
 //  - the shared-memory port: with h^T and Delta^T as shared-memory operands it carried 368 KB per chunk, 2900 cycles.  They
 //    are A operands, so they live in tensor memory (bf16 pairs, written by the epilogues with tcgen05.st): no operand copies,
 //    no re-reading of A by every product;
 //  - the issue of 24 products from a branch taken by one lane, 80 - 130 cycles each: the MMA warp stays converged;
-//  - TMA, whose loads run at 45 and stores at 32 bytes per cycle and SM, one after the other (measured): the 72 KB that a chunk
-//    loads and the 16 KB of its output take 2150 cycles, and the 48 KB of Delta^T and entry state that a forward saves for the
-//    backward 1300 more.  (Ordinary stores, by one or two warps from the tiles or by the epilogue from its registers, were
-//    slower: 4500 - 5000 cycles per chunk.)  So with few heads the d_v rows of a head, which evolve independently, are shared by
-//    two CTAs (k_tc_chain_fwd_half): each loads what both need, but only its half of Ut, and stores its half of everything.
-// SAVE: also store, per chunk, the bf16 entry state (mapHs) and Delta^T (mapDt).  Compile-time: with a flag prompts of 4 sequences
-// of 64 chunks took 80.2 us, so 77.3.
+//  - the TMA unit: from L2 it brings 98 - 113 bytes per cycle and SM (boxes of 8 and 16 KB), but takes out 32, and the two add up
+//    (64 KB in 580 - 670 cycles, 64 KB out 2050, both 2570).  The 72 KB that a chunk loads and the 16 KB of its output are about 1200
+//    cycles; the 48 KB of Delta^T and entry state that a forward saves for the backward make it 2750.  (Ordinary stores, by one or two warps from
+//    the tiles or by the epilogue from its registers, were slower: 4500 - 5000 cycles per chunk.)  So with few heads the d_v rows of a
+//    head, which evolve independently, are shared by two CTAs (k_tc_chain_fwd_half): each loads what both need, but only its half of
+//    Ut, and stores its half of everything.
+// SAVE: also store, per chunk, the bf16 entry state (mapHs) and Delta^T (mapDt).  Compile-time for the half chain's sake (4 sequences of
+// 64 chunks with saves 76.6 us, with a flag 80.3); this kernel is indifferent (128 of 32: 160.8 / 161.1, with saves 202.2 / 202.0).
 // Compute warpgroup w owns tokens [16w, 16w+16) of the 64-column accumulators and d_k columns
 // [32w, 32w+32) of the state; thread l of a warpgroup owns TMEM lane l = d_v index.
 template <bool SAVE>
@@ -780,8 +781,9 @@ constexpr int kHalfSmem = kHalfOffO + 8192 + 1024;
 constexpr int kHalfThreads = kChainCompute + 128 + 128;      // + the output warpgroup, 1 warp each to issue MMAs, load, relay and save
 constexpr int kBarA = 4, kBarB = 5;                          // the relay warp arrives, the compute warps wait
 
-// The chain of 64 d_v rows, two CTAs to a sequence.  What bounds a chunk is the sequence of hand-offs alone: 772 cycles of the two
-// products that depend on one another and twice the way from an accumulator to the next operand.  So that way is kept short:
+// The chain of 64 d_v rows, two CTAs to a sequence.  What bounds a chunk is the sequence of hand-offs: 772 cycles of the two
+// products that depend on one another and twice the way from an accumulator to the next operand, 1560 - 1760 cycles in all with 1 - 32
+// sequences, 1840 - 2090 with saves.  So that way is kept short:
 //  - 64-row products put 16 rows on each of a warpgroup's four warps, so all four schedulers of the SM share the epilogues (as the
 //    lower half of 128 rows they ran on two), and in fragment layout every thread has half as many elements; tiles are read and
 //    staged by ldmatrix / stmatrix instead of element by element;
@@ -792,10 +794,11 @@ constexpr int kBarA = 4, kBarB = 5;                          // the relay warp a
 //    leaves room for one staged copy of what goes out.
 // Entry state and Delta^T go out by TMA: stored by the compute warps from their fragments in 64-byte pieces, or by others in whole
 // rows from the staged tiles, they delay every shared-memory access and wait of the SM (16 of 64: 104 us either way against 94).
-// The output, a quarter of that, goes in whole rows of 128 bytes: the TMA unit, 64 KB in and 24 KB out a chunk, is what bounds a
-// forward with saves, about 2100 cycles a chunk.
-// us, as 64 of k_tc_chain_fwd's 128 rows before and so, prompts and forwards with saves: 4 sequences of 16 chunks 27.3 / 24.5, 31.9 / 26.7;
-// 16 of 64 92.4 / 81.6, 113 / 94.3; 8 of 128 155 / 134, 198 / 156; 32 of 64 117 / 113, 133 / 124; 74 of 64 204 / 194, 243 / 228.
+// The output, a quarter of that, goes in whole rows of 128 bytes by ordinary stores.  The TMA unit, 64 KB in and 24 KB out a chunk with saves,
+// is busy for 1310 - 1370 cycles of it, 580 - 670 without.
+// us, as 64 of k_tc_chain_fwd's 128 rows and so, prompts and forwards with saves, both in turn on one box: 4 sequences of 16 chunks
+// 27.2 / 24.2, 31.6 / 26.3; 4 of 64 77.6 / 65.0, 99.0 / 77.1; 16 of 64 91.5 / 81.0, 112 / 92.9; 8 of 128 155 / 133.6, 196.5 / 155.7; 32 of 64 115.3 /
+// 111.3, 131.3 / 121.3; 72 of 16 54.1 / 54.2, 62.1 / 61.2.  With more sequences HBM takes over (64 of 256: 2120 and 2940 cycles a chunk).
 template <bool SAVE>
 __global__ void __launch_bounds__(kHalfThreads) k_tc_chain_fwd_half(const __grid_constant__ CUtensorMap mapWt,
                                                                     const __grid_constant__ CUtensorMap mapUt,
@@ -1092,9 +1095,9 @@ bool tc_supported(const qd_shape& s) {
            (long long)s.B * s.H * tc_padded_T(s) * 128 < 0x7fffffffLL * 64;
 }
 
-// Two CTAs per sequence while every CTA still gets an SM of its own.  Training pass of 74 sequences, two against one: 84 against
-// 88 us (512 tokens), 599 against 647 (4096); of 75: 121 against 100, 734 against 603.  The forward alone at 74: 30.0 against
-// 31.0 and 238 against 242 (two runs differ by 15), at 75: 51 against 41 and 295 against 225.
+// Two CTAs per sequence while every CTA still gets an SM of its own.  us, two against one, prompt / with saves / backward: 74
+// sequences of 8 chunks 29.7 31.4 / 32.5 36.9 / 45.1 48.8, of 64 203 209 / 230 249 / 298 313; 75 of 8 42.2 35.3 / 46.0 41.7 / 59.2 53.5,
+// of 64 245 199 / 284 236 / 351 299.
 int chain_rows(uint64_t BH) { return 2 * BH <= kSMs ? 64 : 128; }
 
 TcLayout tc_layout(const qd_shape& s) {
@@ -1218,11 +1221,14 @@ cudaError_t tc_chain_fwd(const ChunkArgs& a) {
 // it need not wait.  Its first CTA waits for chain i before it leaves, so when prep i + 1 has completed chain i has too, and
 // chain i + 1, which waits for prep i + 1, finds the state that chain i left: in h_T, or without one in the section that the
 // reverse chain fills later.  The state is passed on in fp32, so the results are those of one part, bit for bit.
-// Where: with up to 40 sequences (68 SMs idle), from 64 chunks and 1.7 loads of the GPU with preparations (1024 chunks) on.  One
-// part against two, us, without and with saves: 16 sequences of 64 chunks 97.7 / 91.3, 121 / 113; 32 of 64 122.8 / 117.4,
-// 148.8 / 133.4; 40 of 64 134.7 / 131.5, 160.6 / 151.4; but 44 of 64 141.6 / 142.2, 48 of 64 147.6 / 151.5, 64 of 256 728 / 741; 8 of 64 82.2 /
-// 82.2; 40 of 32 72.7 / 75.5.  A part costs 2 - 8 us, so three of them only from 256 chunks on: 32 of 512 965 / 792 / 755 for
-// one, two, three (1103 / 948 / 923), 16 of 512 714 / 644 / 621, 40 of 256 543 / 484 / 484; 32 of 64 122.8 / 117.4 / 120.9.
+// Where: with up to 40 sequences (68 SMs idle), from 64 chunks and 1.7 loads of the GPU with preparations (1024 chunks) on.  One, two, three
+// parts, us, prompts; with saves: 16 sequences of 64 chunks 88.8 / 82.8 / 84.3; 98.8 / 93.3 / 96.4.  32 of 64 116.7 / 111.7 / 113.3; 128.4 / 121.3 /
+// 122.9.  40 of 64 129.3 / 126.0 / 130.9; 143.9 / 139.4 / 146.3.  8 of 128 140.5 / 133.9 / 133.9; 161.5 / 155.7 / 157.4.  But 8 of 64 71.0 / 70.6; 83.4 /
+// 83.7.  40 of 32 69.3 / 71.4; 76.8 / 78.6.  44 of 64 136.7 / 137.1; 155.0 / 152.6.  48 of 64 143.0 / 146.1; 162.1 / 163.9.  64 of 256 744 / 757;
+// 859 / 867.  (From 128 chunks on 41 to 48 sequences would gain 2 - 5 %: 48 of 128 287 / 281; 326 / 316, 48 of 256 593 / 576; 672 / 646.)  Three of them
+// from 256 chunks on: 32 of 512 877 / 779 / 749; 990 / 891 / 854.  16 of 512 637 / 578 / 564; 715 / 659 / 646.  40 of 256 521 / 489 / 487; 585 / 545 /
+// 542.  4 of 256 246 / 239 / 240; 287 / 280 / 284.  With 128 chunks the third part gives 0 - 2 % (32 sequences 221 / 201 / 200, 40 247 / 235 / 239).
+// The parts are equal.  A third of 32 x 512 chunks takes the chain about 190 us, and the preparation beside it, on 84 SMs, 240 - 250.
 int tc_fwd_parts(const ChunkArgs& a) {
     const long long BH = (long long)a.s.B * a.s.H, N = (a.s.T + kChunk - 1) / kChunk;
     if (BH > 40 || N < 64 || BH * N < 1024 || !(a.hT || a.save)) return 1;
